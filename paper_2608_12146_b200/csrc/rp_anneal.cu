@@ -61,7 +61,7 @@ k_anneal_level(const AnnealArgs A)
     char *sm_static = sm_blob + A.bl.bytes;
     int *scratch = (int *)(sm_static + A.sl.bytes);
     // Per-cell caches of the proposal keys (attention cost of the cell, cost and attention part of its
-    // row-shard).  With one cell per row-shard (every DP slot its own shard) they equal the row-shard
+    // row-shard).  Where cell and row-shard have the same index (DP slot d is shard d) they equal the row-shard
     // arrays of the blob; ALIAS then uses those arrays themselves and keeps no copy (chosen where the
     // shared memory saved lets one more chain be resident per SM).
     i64 *attkey = (i64 *)(scratch + 2 * slice_pad);
@@ -498,7 +498,7 @@ int rp_anneal_smem_bytes(const rp_ctx *c, int *threads, size_t *bytes)
     const size_t b_alias = b - sizeof(i64) * 3 * (size_t)dm.K;
     const int minb = rp_coop_chains_per_sm(dm);
     const size_t room = 227 * 1024;
-    const bool alias = (dm.G == dm.D) && (room / (b + 1024) < (size_t)minb) && (room / (b_alias + 1024) > room / (b + 1024));
+    const bool alias = dm.own_shard && (room / (b + 1024) < (size_t)minb) && (room / (b_alias + 1024) > room / (b + 1024));
     *threads = nt;
     *bytes = alias ? b_alias : b;
     return alias ? 2 : 0;

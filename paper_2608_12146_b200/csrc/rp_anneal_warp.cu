@@ -156,8 +156,8 @@ __device__ __forceinline__ void rp_warp_staged_commit(int lane, int nchunks, boo
     }
 }
 
-// ID: every DP slot is its own shard, so a cell is a row-shard and the per-cell proposal keys are
-// the row-shard arrays of the blob themselves.
+// ID: DP slot d is shard d, so a cell is the row-shard of the same index and the per-cell proposal
+// keys are the row-shard arrays of the blob themselves.
 template <bool ID>
 __global__ void __launch_bounds__(32, WARP_CHAINS_PER_SM)
 k_anneal_warp(const AnnealArgs A, const RpWarpLayout wl)
@@ -497,7 +497,7 @@ bool rp_uses_warp_chains(const rp_ctx *c)
     if (!vec) return false;
     if (c->knob_chain_kernel == 1) return false;
     if (c->knob_chain_kernel != 2 && rp_uses_wpc(dm) && c->Ppop <= WARP_MIN_CHAINS) return false;
-    const RpWarpLayout wl = rp_warp_layout(dm, c->bl, c->sl, dm.G == dm.D);
+    const RpWarpLayout wl = rp_warp_layout(dm, c->bl, c->sl, dm.own_shard);
     return wl.bytes <= 100 * 1024;
 }
 
@@ -514,7 +514,7 @@ static int launch_warp(rp_ctx *c, const AnnealArgs &A, const RpWarpLayout &wl)
 
 int rp_launch_anneal_warp(rp_ctx *c, AnnealArgs &A)
 {
-    const bool identity = (c->dm.G == c->dm.D);
+    const bool identity = c->dm.own_shard;
     const RpWarpLayout wl = rp_warp_layout(c->dm, c->bl, c->sl, identity);
     A.smem_bytes = (unsigned)wl.bytes;
     if (identity) RP_TRY(launch_warp<true>(c, A, wl));

@@ -238,6 +238,8 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
     dm.N = N; dm.L = L; dm.E = E; dm.k = cfg->top_k; dm.C = cfg->token_cap; dm.D = D; dm.P = P; dm.G = G;
     dm.H = E / P; dm.S = cfg->n_stages;
     dm.R = 0; dm.K = 0; dm.RG = 0; dm.LP = L * P; dm.slices = 0;
+    dm.own_shard = (G == D);
+    for (int d = 0; d < D; ++d) if (edp[d] != d) dm.own_shard = 0;       // a permutation has G == D as well
     dm.asum = 0; dm.bsum = 0;
     for (int s = 0; s < RP_MAX_STAGES; ++s) { dm.ahat[s] = 0; dm.bhat[s] = 0; }
     for (int s = 0; s < dm.S; ++s) {

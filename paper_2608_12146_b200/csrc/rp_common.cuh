@@ -41,6 +41,7 @@ struct RpDims {
     int N, L, E, k, C, D, P, G, H, S;   // H = E / P experts per rank, S = attention stages
     int R, K, RG, LP;                   // rows, cells R*D, row-shards R*G, L*P (set after packing)
     int slices;                         // rank loads kept as shared slices (set after packing; see AnnealArgs)
+    int own_shard;                      // DP slot d is shard d: a cell and its row-shard have the same index
     i64 ahat[RP_MAX_STAGES], bhat[RP_MAX_STAGES];
     i64 asum, bsum;                     // sums over stages (attention key of a cell)
     i64 SC;                             // 2^8 * C^2

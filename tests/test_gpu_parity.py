@@ -425,6 +425,30 @@ def test_warp_per_chain_kernel_on_small_windows(spec):
         rp.rp_destroy(ctx)
 
 
+PERMUTED_CASES = [
+    # name, N, L, E, k, C, D, P, min_rows, pop, knob: one DP slot per shard, but slot d is not shard d
+    ("perm_on_chip", 96, 5, 16, 2, 4096, 4, 4, 3, 20, 0),
+    ("perm_warp", 120, 20, 32, 2, 4096, 4, 32, 3, 24, 2),
+    ("perm_128_threads", 1100, 16, 64, 2, 8192, 64, 64, 8, 8, 1),      # 512 cells: the form without per-cell key caches is in reach
+]
+
+
+@pytest.mark.parametrize("spec", PERMUTED_CASES, ids=[e[0] for e in PERMUTED_CASES])
+def test_permuted_shards(spec):
+    """As many shards as DP slots, in another order: a cell and its row-shard then differ in index,
+    on each chain kernel."""
+    name, N, L, E, k, C, D, P, min_rows, pop, kernel = spec
+    edp = [(d + 1) % D for d in range(D)]
+    w = make_window(custom_spec(name, N, L, E, k, C, D, P, pop, 400, data_seed=len(name) * 13 + N))
+    ref = oracle_front(w, edp, min_rows)
+    ctx = load(w, pop=pop, edp=edp, min_rows=min_rows)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", kernel)
+    check_front(w, ctx, ref)
+    _, stats = check_anneal(w, ctx, ref, edp, pop, 4, 60, t_ratio=0.6, check_members=2)
+    assert stats.accepted > 0
+    rp.rp_destroy(ctx)
+
+
 @pytest.mark.parametrize("spec", [BARRIER_CASES[0], BARRIER_CASES[2], WARP_CHAIN_CASES[0]],
                          ids=["warp_per_candidate", "cooperative", "warp_per_chain"])
 def test_a_wait_that_runs_out_is_reported_and_the_context_survives(spec):
