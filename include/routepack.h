@@ -300,17 +300,17 @@ typedef enum {
  *     gives up after that many microseconds (default 2 s + 50 us per step of a level).
  *   RP_KNOB_STALL_ONE_CHAIN: chain 0 waits once more, after its copies have landed, on a barrier
  *     phase that nothing completes: the wait runs out and rp_anneal returns RP_ERR_TIMEOUT.
- *   RP_KNOB_LAUNCH_PER_LEVEL: how rp_anneal launches windows whose chains can all be resident at
- *     once (rank loads on chip, at most 256 members).  0 or 2 = one launch for all levels (lowest
+ *   RP_KNOB_LAUNCH_PER_LEVEL (set before rp_pack_rows): how rp_anneal launches windows whose chains can
+ *     all be resident at once with their rank loads on chip.  0 or 2 = one launch for all levels (lowest
  *     latency of a single plan); 1 = one launch per level (two windows planned at once on two
  *     streams then share the GPU, which two launches of the first kind cannot).
  *   RP_KNOB_RANK_LOAD_SLICES (set before rp_pack_rows): how windows with L*P > 512 keep the rank
  *     loads of the population.  0 or 1 = shared slices with copy-on-write (the default), 2 = one
  *     private cell per member, copied whole when resampling replaces the member.
- *   RP_KNOB_CHAIN_KERNEL: which chain kernel windows use whose rank loads live in the slice pool
- *     (not on chip).  0 = one warp per chain, except for windows with L*P <= 512 and at most 592
- *     members, which finish sooner with several warps per chain; 1 = always several warps per
- *     chain; 2 = always one warp per chain. */
+ *   RP_KNOB_CHAIN_KERNEL: which chain kernel runs the levels.  0 = chosen by the window (one layer of the rank
+ *     loads per lane wherever a row fits a warp's registers, whole or compressed; else one warp per chain, or
+ *     several warps per chain); 1 = always several warps per chain; 2 = one warp per chain with whole
+ *     rows staged in shared memory, where the rank loads live in the slice pool. */
 typedef enum { RP_KNOB_BARRIER_WORKSPACE = 1, RP_KNOB_WAIT_POLLS = 2, RP_KNOB_STALL_ONE_CHAIN = 3,
                RP_KNOB_RANK_LOAD_SLICES = 4, RP_KNOB_LAUNCH_PER_LEVEL = 5, RP_KNOB_CHAIN_KERNEL = 6 } rp_knob;
 int rp_debug_set_knob(rp_ctx *ctx, int knob, int64_t value);
@@ -342,7 +342,8 @@ int rp_debug_philox(const uint32_t *ctr, const uint32_t key[2], uint32_t *out, i
 int rp_debug_l2_read_rate(int64_t bytes, int32_t reps, double *gb_per_s);
 /* Which chain kernel rp_anneal runs for this context (valid after rp_pack_rows; inspection only):
  * 0 = warp per candidate (k_anneal_wpc), 1 = 128 threads per chain (k_anneal_level), 2 = warp per
- * chain (k_anneal_warp). */
+ * chain (k_anneal_warp), 3 = one layer per lane (k_anneal_row; windows whose rows it would compress decide
+ * between 2 and 3 in the first rp_anneal call). */
 int rp_debug_chain_kernel(rp_ctx *ctx, int32_t *which);
 /* Number of kernels this library has launched in this process so far. */
 int64_t rp_debug_launch_count(void);

@@ -339,7 +339,7 @@ def rp_debug_l2_read_rate(nbytes: int = 32 << 20, reps: int = 50) -> float:
     return float(out.value)
 
 
-CHAIN_KERNELS = ("k_anneal_wpc", "k_anneal_level", "k_anneal_warp")
+CHAIN_KERNELS = ("k_anneal_wpc", "k_anneal_level", "k_anneal_warp", "k_anneal_row")
 
 
 def rp_debug_chain_kernel(ctx: Context) -> str:

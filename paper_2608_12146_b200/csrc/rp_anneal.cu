@@ -408,8 +408,29 @@ void rp_decide_layouts(rp_ctx *c)
     } else {
         dm.slices = rp_slice_mode(dm, c->knob_slices);
     }
+    // The one-layer-per-lane kernel where the window allows it: all levels in one launch when every
+    // chain's rank loads fit on chip at once, else with the rank loads as slices.  (With one launch per level asked
+    // for, windows whose rank loads the warp-per-candidate kernel keeps on chip stay with that kernel.)
+    c->row_mode = 0;
+    if (c->knob_chain_kernel == 0 && c->knob_slices == 0) {
+        if (c->knob_level_launches != 1 && rp_row_fits_chip(c, c->bl, c->sl)) c->row_mode = 1;
+        else if (rp_row_kind(dm) && (dm.slices || c->knob_level_launches != 1)) { c->row_mode = 2; dm.slices = 1; }
+    }
     if (dm.slices) rp_make_layouts(dm, &c->bl, &c->sl);
 }
+
+bool rp_row_compressed(const rp_ctx *c) { return c->row_mode == 2 && rp_row_kind(c->dm) == 2; }
+
+// Compressed rows: at most one row-shard in 64 of the members counted may need its loads added up anew (a
+// scored candidate names two, and adding one up costs about what ten candidates cost; a window that fails
+// this runs the warp-per-chain kernel on whole rows).
+bool rp_may_use_row(const rp_ctx *c)
+{
+    if (!c->row_mode || c->knob_chain_kernel != 0) return false;
+    if (c->row_mode == 1) return c->knob_level_launches != 1;
+    return !rp_row_compressed(c) || c->row_undecided < 0 || (long long)c->row_undecided * 64 <= (long long)c->row_counted * c->dm.RG;
+}
+bool rp_uses_row(const rp_ctx *c) { return rp_may_use_row(c) && !(rp_row_compressed(c) && c->row_undecided < 0); }
 
 // Slice bookkeeping between two levels: holders of every slice among the members that start the
 // next level (member m starts from the terminal table of anc[m]), then the list of free slices,
@@ -520,6 +541,8 @@ static u32 host_philox_x(u32 c0, u32 c1, u32 c2, u32 c3, u32 k0, u32 k1)
 
 int rp_launch_anneal_wpc_all(rp_ctx *c, const AnnealArgs &A, int *done);
 int rp_launch_anneal_warp(rp_ctx *c, AnnealArgs &A);
+int rp_launch_anneal_row(rp_ctx *c, AnnealArgs &A);
+int rp_launch_anneal_row_all(rp_ctx *c, const AnnealArgs &A, int *done);
 
 static void fill_args(rp_ctx *c, int level, int n_levels, const rp_anneal_params *prm, u64 rho_q32, u64 guide_q32, AnnealArgs &A)
 {
@@ -591,9 +614,15 @@ int rp_launch_anneal_all(rp_ctx *c, int n_levels, const rp_anneal_params *prm, u
     // one another needs all of them resident at once, so two such launches do not share the SMs: a
     // caller that plans several windows at once on separate streams asks for one launch per level.
     const bool wanted = c->knob_level_launches != 1;
-    if (!use_wpc(c->dm) || !wanted || !c->d_levels) return RP_OK;
+    if (!wanted || !c->d_levels) return RP_OK;
     AnnealArgs A;
     fill_args(c, 0, n_levels, prm, rho_q32, guide_q32, A);
+    if (rp_uses_row(c)) {
+        if (c->row_mode != 1) return RP_OK;
+        RP_TRY(rp_launch_anneal_row_all(c, A, done));
+        return *done ? RP_OK : RP_ERR_STATE;
+    }
+    if (!use_wpc(c->dm)) return RP_OK;
     return rp_launch_anneal_wpc_all(c, A, done);
 }
 
@@ -602,6 +631,7 @@ int rp_launch_anneal_level(rp_ctx *c, int level, int n_levels, const rp_anneal_p
     AnnealArgs A;
     fill_args(c, level, n_levels, prm, rho_q32, guide_q32, A);
     if (rp_uses_slices(c->dm)) RP_TRY(rp_launch_slice_gc(c));
+    if (rp_uses_row(c)) return rp_launch_anneal_row(c, A);
     if (rp_uses_warp_chains(c)) return rp_launch_anneal_warp(c, A);
     if (use_wpc(c->dm)) return rp_launch_anneal_wpc(c, A);
     int nt; size_t smem;

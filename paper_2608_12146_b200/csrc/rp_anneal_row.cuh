@@ -1,0 +1,37 @@
+// What the one-layer-per-lane chain kernel is given beside AnnealArgs (rp_anneal_row.cu).
+#pragma once
+#include "rp_anneal.cuh"
+
+#define ROW_MAX_WARPS 8          // chains of a CTA in the launch that runs all levels, at most
+#define ROW_THREADS 256          // its threads
+
+struct RowArgs {
+    const int *qr;               // [N][rlp] demand rows: cpl 16-byte chunks per layer
+    const int2 *tf;              // [N] length, and the demand on the layers' fixed ranks summed over the layers
+    int *Wr;                     // rank-load slices in the same form
+    const i64 *F_src;            // [P_pop][RG] slack of a row-shard: sum of its busiest loads less sum of its samples' tf.y; the level's start, its end, both buffers
+    i64 *F_dst, *F_buf;
+    int rlp, cpl, comp;
+    int off_tab, off_leF, off_chain;                                       // shared memory of the CTA
+    int off_F, off_book, off_wtab, off_spare, off_top, off_cell, off_snap, off_recs, off_W;   // of one chain
+    int chain_bytes, smem_bytes, cw, recs;
+};
+
+// Bounded wait of one thread until a counter that the other CTAs of the launch add to has reached
+// `target`; false when the time allowed ran out or another chain has raised the time-out word.
+__device__ __forceinline__ bool rp_wait_count(const int *ctr, int target, const AnnealArgs &A)
+{
+    u64 t0;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    for (unsigned it = 0;; ++it) {
+        int v;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+        if (v >= target) return true;
+        if ((it & 15u) == 15u) {
+            if (__ldcg(&A.status[RP_SW_TIMEOUT])) return false;
+            u64 t1;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+            if (t1 - t0 > A.bar_timeout_ns) return false;
+        }
+    }
+}

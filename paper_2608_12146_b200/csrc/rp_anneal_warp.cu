@@ -512,6 +512,8 @@ static int launch_warp(rp_ctx *c, const AnnealArgs &A, const RpWarpLayout &wl)
     return RP_OK;
 }
 
+int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A);
+
 int rp_launch_anneal_warp(rp_ctx *c, AnnealArgs &A)
 {
     const bool identity = c->dm.own_shard;
@@ -519,6 +521,12 @@ int rp_launch_anneal_warp(rp_ctx *c, AnnealArgs &A)
     A.smem_bytes = (unsigned)wl.bytes;
     if (identity) RP_TRY(launch_warp<true>(c, A, wl));
     else RP_TRY(launch_warp<false>(c, A, wl));
+    ++g_rp_launches;
+    return rp_launch_level_end(c, A);
+}
+
+int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A)
+{
     // workspace of the barrier: cumulative weights and the replayed layout on chip where they fit
     size_t ws = 2 * std::max((size_t)c->Ppop * 8, (size_t)c->dm.N * 2);
     ws = std::min(std::max(ws, (size_t)16 * 1024), (size_t)200 * 1024);
@@ -527,7 +535,7 @@ int rp_launch_anneal_warp(rp_ctx *c, AnnealArgs &A)
     B.smem_bytes = (unsigned)ws;
     RP_CUDA(cudaFuncSetAttribute(k_level_end, cudaFuncAttributeMaxDynamicSharedMemorySize, WARP_SMEM_OPTIN));
     k_level_end<<<1, LEVEL_END_THREADS, ws, c->stream>>>(B);
-    g_rp_launches += 2;
+    ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
 }

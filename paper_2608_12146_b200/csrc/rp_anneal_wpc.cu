@@ -22,6 +22,7 @@
 #include <string.h>
 
 #include "rp_level_end.cuh"
+#include "rp_anneal_row.cuh"
 
 struct CandS {                  // a feasible proposal and the cell statistics it would leave behind
     MoveS m;
@@ -84,25 +85,6 @@ __device__ __forceinline__ void rp_finish_level_async(const AnnealArgs &A, int t
     if (!is_last_a) return;
     __threadfence();
     rp_level_end(A, tid, nt, ws, rp_le_ws_bytes(A, ws_bytes));
-}
-
-// Bounded wait of one thread until a counter that the other CTAs of the launch add to has reached
-// `target`; false when the time allowed ran out or another chain has raised the time-out word.
-__device__ __forceinline__ bool rp_wait_count(const int *ctr, int target, const AnnealArgs &A)
-{
-    u64 t0;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-    for (unsigned it = 0;; ++it) {
-        int v;
-        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-        if (v >= target) return true;
-        if ((it & 15u) == 15u) {
-            if (__ldcg(&A.status[RP_SW_TIMEOUT])) return false;
-            u64 t1;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-            if (t1 - t0 > A.bar_timeout_ns) return false;
-        }
-    }
 }
 
 template <int NW, bool WS, int CH, bool PERSIST>
@@ -727,7 +709,7 @@ size_t rp_wpc_smem_bytes(const RpDims &dm, const RpBlob &bl, const RpStatic &sl,
                16 + ((sizeof(unsigned short) * dm.N + 15) & ~(size_t)15);
     const size_t wbytes = sizeof(int) * ((((size_t)dm.RG * dm.LP) + 3) & ~(size_t)3);
     const size_t per_cta = (size_t)220 * 1024 / (16 / nw);
-    *w_in_smem = (b + wbytes <= per_cta);
+    *w_in_smem = !dm.slices && (b + wbytes <= per_cta);         // (a population laid out as slices stays one)
     if (*w_in_smem) b += wbytes;
     else b += 16 + (size_t)dm.RG * 5;            // spare slices and ownership flags
     return (b + 15) & ~(size_t)15;

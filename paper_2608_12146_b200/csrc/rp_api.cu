@@ -154,6 +154,7 @@ static void free_population(rp_ctx *c)
     c->d_W = nullptr; c->d_wloc = nullptr; c->d_wloc_next = nullptr; c->d_le_scratch = nullptr;
     c->d_wref = nullptr; c->d_wcount = nullptr; c->d_wfree = nullptr; c->d_wfree_head = nullptr;
     c->d_cand_layout = nullptr; c->d_inc_slot = nullptr;
+    c->d_tf = nullptr; c->d_qr = nullptr; c->d_Wr = nullptr; c->d_rowF = nullptr; c->d_undecided = nullptr;
     c->d_sync = nullptr;
     c->d_anc = nullptr; c->d_anc_next = nullptr; c->d_done = nullptr; c->d_term = nullptr; c->d_best = nullptr; c->d_best_step = nullptr;
     c->d_best_nlog = nullptr; c->d_digest = nullptr; c->d_F = nullptr;
@@ -282,6 +283,7 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
             slab.take(&c->d_pi, (size_t)L * E);
             slab.take(&c->d_inv, (size_t)L * E);
             slab.take(&c->d_rank_load, (size_t)L * P);
+            slab.take(&c->d_top, (size_t)L * 3);
             slab.take(&c->d_q, (size_t)N * L * P);
             slab.take(&c->d_sort_keys, (size_t)2 * n_pow2);
             slab.take(&c->d_seed_layout, N);
@@ -485,6 +487,13 @@ extern "C" int rp_pack_rows(rp_ctx *c, int32_t *n_rows, int32_t *certified)
 
 // Buffers of a population of c->Ppop members for the row count in c->dm, every member a copy of the
 // length-only seed (evaluated once into slot 0, which all slots descend from); the seed is the incumbent.
+// Members 0 .. n-1 have just been scored into the current buffer (the others descend from them): what the
+// one-layer-per-lane kernel keeps beside the scores is worked out when it is about to run.
+static void forget_rows(rp_ctx *c, int n)
+{
+    c->rows_current = 0; c->full_stale = 0; c->row_undecided = -1; c->row_members = n;
+}
+
 static int build_population(rp_ctx *c)
 {
     RpDims &dm = c->dm;
@@ -513,7 +522,16 @@ static int build_population(rp_ctx *c)
                 slab.take(&c->d_wfree_head, 2);
             }
             slab.take(&c->d_inc_slot, 1);
-            if (rp_uses_wpc(c->dm)) slab.take(&c->d_cand_layout, P * (size_t)c->dm.N);
+            if (rp_uses_wpc(c->dm) || c->row_mode == 1) slab.take(&c->d_cand_layout, P * (size_t)c->dm.N);
+            if (c->row_mode) {
+                slab.take(&c->d_tf, 2 * (size_t)dm.N);
+                slab.take(&c->d_rowF, 2 * P * (size_t)dm.RG);
+                slab.take(&c->d_undecided, 1);
+                if (rp_row_separate(c)) {
+                    slab.take(&c->d_qr, (size_t)dm.N * rp_row_ints(c));
+                    slab.take(&c->d_Wr, 2 * P * (size_t)dm.RG * rp_row_ints(c));
+                }
+            }
             slab.take(&c->d_anc, P);
             slab.take(&c->d_anc_next, P);
             slab.take(&c->d_done, 1);
@@ -523,7 +541,7 @@ static int build_population(rp_ctx *c)
             slab.take(&c->d_best_step, 2 * P);
             slab.take(&c->d_best_nlog, 2 * P);
             slab.take(&c->d_digest, 2 * P);
-            slab.take(&c->d_F, P);
+            slab.take(&c->d_F, 2 * P);                   // (two sets like the reports, see rp_anneal_row.cu)
             if (pass == 0) { RP_TRY(dev_alloc(c, &c->d_pop_slab, slab.off)); slab.base = c->d_pop_slab; }
         }
     }
@@ -546,6 +564,8 @@ static int build_population(rp_ctx *c)
         ++g_rp_launches;
         RP_CUDA(cudaGetLastError());
     }
+    c->rows_made = 0;
+    forget_rows(c, 1);
     stage_mark(c, RP_EV_SEED_1, c->stream);
     return RP_OK;
 }
@@ -635,6 +655,7 @@ static int install_population(rp_ctx *c, const int *lay, int n_distinct = 0)
         k_descend_cyclic<<<(int)((P + 255) / 256), 256, 0, c->stream>>>((int)P, (int)ne, c->d_anc, c->d_wloc, c->d_wloc_next);
         ++g_rp_launches;
     }
+    forget_rows(c, (int)ne);
     if (st == RP_OK) st = rp_launch_pick_best(c, c->d_eval_score, lay, (int)ne, best);
     cudaError_t e = cudaSuccess;
     if (st == RP_OK) e = cudaMemcpyAsync(c->d_seed_score, best, sizeof(i64) * 3, cudaMemcpyDeviceToDevice, c->stream);
@@ -900,6 +921,22 @@ __global__ void k_reset_anneal(i64 *__restrict__ counters, int *__restrict__ sta
     for (int y = x; y < n_sync; y += blockDim.x) sync[y] = 0;
 }
 
+// The population's rank loads in full form again, scored from its layouts: every member owns rank-load cell m.
+static int rebuild_rank_loads(rp_ctx *c)
+{
+    const size_t P = (size_t)c->Ppop;
+    RP_TRY(ensure_eval_scratch(c, P, false));
+    k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, c->dm.N, c->d_eval_cells, nullptr);
+    RP_TRY(rp_launch_eval(c, c->d_eval_cells, (int)P, c->d_W, c->buf[1 - c->cur].blob, c->d_eval_score, nullptr));
+    c->cur = 1 - c->cur;
+    k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_wloc, (int)P, 0);
+    k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_wloc_next, (int)P, 0);
+    k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_anc, (int)P, 0);
+    g_rp_launches += 4;
+    RP_CUDA(cudaGetLastError());
+    return RP_OK;
+}
+
 extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *stats)
 {
     if (!c || !p) return RP_ERR_ARG;
@@ -943,7 +980,24 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     int st = RP_OK;
     // One launch for all levels where every chain can be resident at once, else one launch per level.
     int all_in_one = 0;
-    if (rp_uses_wpc(c->dm) && c->knob_level_launches != 1) st = rp_upload_levels(c, NL);
+    // Which kernel: the one-layer-per-lane kernel where the window allows it; compressed rows must decide nearly
+    // every row-shard of the members as they were scored.
+    if (rp_may_use_row(c)) {
+        if (!c->rows_made) { RP_TRY(rp_launch_make_rows(c)); c->rows_made = 1; }
+        if (!c->rows_current) { RP_TRY(rp_launch_member_rows(c, c->row_members)); c->rows_current = 1; }
+        if (rp_row_compressed(c) && c->row_undecided < 0) {
+            int *u = (int *)(c->h_pin + 60);
+            RP_CUDA(cudaMemcpyAsync(u, c->d_undecided, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+            RP_CUDA(cudaStreamSynchronize(c->stream));
+            c->row_undecided = *u;
+        }
+    }
+    const bool row = rp_uses_row(c);
+    if (!row && c->full_stale) st = rebuild_rank_loads(c);
+    if (!row) c->rows_current = 0;
+    c->row_members = c->Ppop;                  // after a level every member has a state of its own
+    c->full_stale = row && rp_row_separate(c);
+    if (st == RP_OK && (rp_uses_wpc(c->dm) || (row && c->row_mode == 1)) && c->knob_level_launches != 1) st = rp_upload_levels(c, NL);
     if (stats) cudaEventRecord(ev[0], c->stream);
     if (st == RP_OK) st = rp_launch_anneal_all(c, NL, p, rho_q32, guide_q32, &all_in_one);
     if (all_in_one) c->cur = (c->cur + NL) & 1;       // the kernel has left both ancestor tables and both cell tables current
@@ -982,7 +1036,7 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     if (stats) {
         stats->proposed = cn[0]; stats->feasible = cn[1]; stats->accepted = cn[2]; stats->improved = cn[3];
         stats->move_bytes = cn[4]; stats->gather_bytes = cn[5]; stats->staging_bytes = cn[6];
-        stats->kernel_launches = all_in_one ? 1 : (int64_t)NL * ((rp_uses_slices(c->dm) ? 3 : 1) + (rp_uses_warp_chains(c) ? 1 : 0));
+        stats->kernel_launches = all_in_one ? 1 : (int64_t)NL * ((rp_uses_slices(c->dm) ? 3 : 1) + (row || rp_uses_warp_chains(c) ? 1 : 0));
         stats->ms_chains = ms_chains;
     }
     c->best_verdict = best_verdict(c, sw);
@@ -1147,6 +1201,18 @@ extern "C" int rp_debug_dump(rp_ctx *c, int what, int32_t index, void *buf, int6
             break;
         }
         case RP_DUMP_W:
+            if (c->full_stale) {               // kept as other rows during annealing: added up from the member's layout
+                need = sizeof(int) * (size_t)dm.RG * dm.LP;
+                if ((st = dev_alloc(c, (int **)&tmp, (size_t)dm.RG * dm.LP)) != RP_OK) return st;
+                if ((st = ensure_eval_scratch(c, 1, false)) == RP_OK) {
+                    k_gather_cells<<<1, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc + index, dm.N, c->d_eval_cells, nullptr);
+                    ++g_rp_launches;
+                    st = rp_launch_eval(c, c->d_eval_cells, 1, (int *)tmp, nullptr, c->d_eval_score, nullptr);
+                }
+                if (st != RP_OK) { dev_free(c, tmp); return st; }
+                src = tmp;
+                break;
+            }
             if (rp_uses_slices(dm)) {          // the member's slices, gathered through its table
                 need = sizeof(int) * (size_t)dm.RG * dm.LP;
                 if ((st = dev_alloc(c, (int **)&tmp, (size_t)dm.RG * dm.LP)) != RP_OK) return st;
@@ -1237,7 +1303,8 @@ extern "C" int rp_debug_chain_kernel(rp_ctx *c, int32_t *which)
 {
     if (!c || !which) return RP_ERR_ARG;
     if (c->stage < 3) return RP_ERR_STATE;
-    *which = rp_uses_warp_chains(c) ? 2 : (rp_uses_wpc(c->dm) ? 0 : 1);
+    // (compressed rows: decided by the first rp_anneal call)
+    *which = rp_uses_row(c) ? 3 : rp_uses_warp_chains(c) ? 2 : (rp_uses_wpc(c->dm) ? 0 : 1);
     return RP_OK;
 }
 

@@ -134,6 +134,20 @@ struct rp_ctx {
     int *d_wcount;             // [2*P_pop*RG] the same while it is being counted; zero between two counts
     int *d_wfree;              // [2*P_pop*RG] slices nobody holds, handed out in this order during the level
     int *d_wfree_head;         // [2] next free-list entry to hand out, entries in the list
+    // One-layer-per-lane chain kernel (rp_anneal_row.cu)
+    int row_mode;              // 0 = not for this window, 1 = one launch for all levels (rank loads on chip), 2 = one launch per level
+    int rows_current;          // the row-shard sums (and rows kept apart) describe the population
+    int full_stale;            // that kernel ran on rows kept apart: d_W no longer describes the population
+    int row_undecided;         // compressed rows: row-shards of the evaluated members that they do not decide, -1 = not read back yet
+    int row_members;           // members with a scored state of their own (0 .. n-1 of the current buffer)
+    int row_counted;           // members row_undecided was counted over
+    int rows_made;             // d_tf and d_qr are filled
+    int *d_top;                // [L][3] ranks of each layer by decreasing aggregate load
+    int *d_tf;                 // [N][2] length, demand on the fixed ranks
+    int *d_qr;                 // [N][row] demand rows in row form, where they are kept apart
+    int *d_Wr;                 // [2*P_pop*RG][row] rank-load slices in row form, where they are kept apart
+    i64 *d_rowF;               // [2][P_pop][RG] demand on the fixed ranks of every row-shard, per population buffer
+    int *d_undecided;          // [1]
     RpBlob bl;
     RpStatic sl;
     char *d_static;            // static tables block
@@ -248,6 +262,15 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
                      int *n_distinct, i64 *dist);
 bool rp_uses_wpc(const RpDims &dm);
 bool rp_uses_warp_chains(const rp_ctx *c);
+bool rp_may_use_row(const rp_ctx *c);
+bool rp_uses_row(const rp_ctx *c);
+bool rp_row_compressed(const rp_ctx *c);
+bool rp_row_fits_chip(const rp_ctx *c, const RpBlob &bl, const RpStatic &sl);
+int rp_row_kind(const RpDims &dm);
+bool rp_row_separate(const rp_ctx *c);
+size_t rp_row_ints(const rp_ctx *c);
+int rp_launch_make_rows(rp_ctx *c);
+int rp_launch_member_rows(rp_ctx *c, int n);
 int rp_launch_anneal_level(rp_ctx *c, int level, int n_levels, const rp_anneal_params *prm, u64 rho_q32, u64 guide_q32);
 int rp_launch_anneal_all(rp_ctx *c, int n_levels, const rp_anneal_params *prm, u64 rho_q32, u64 guide_q32, int *done);
 int rp_upload_levels(rp_ctx *c, int n_levels);

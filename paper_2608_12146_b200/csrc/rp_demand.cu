@@ -287,7 +287,7 @@ int rp_launch_check_reduce(rp_ctx *c)
 // with the smallest (load, id) among ranks holding fewer than H experts.
 __global__ void __launch_bounds__(1024)
 k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *__restrict__ pi, int *__restrict__ inv,
-      i64 *__restrict__ rank_load)
+      i64 *__restrict__ rank_load, int *__restrict__ top)
 {
     extern __shared__ unsigned char smraw[];
     i64 *load = (i64 *)smraw;                 // [E]
@@ -346,7 +346,20 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *__restrict__ pi, int *__rest
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) { const int p = lane + 32 * u; if (p < dm.P) rank_load[(size_t)l * dm.P + p] = Gr[u]; }
+        for (int u = 0; u < 4; ++u) { const int p = lane + 32 * u; if (p < dm.P) rank_load[(size_t)l * dm.P + p] = Gr[u]; else Gr[u] = -1; }
+        // the three busiest ranks (ties: lower rank), for the chain kernel's fixed ranks and compressed rows
+        for (int x = 0; x < 3; ++x) {
+            i64 best = -1;
+            int bp = 0x7fffffff;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) if (Gr[u] > best) { best = Gr[u]; bp = lane + 32 * u; }
+            const u32 hi = (u32)((u64)(best + 1) >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+            const u32 lo = hi == mh ? (u32)(best + 1) : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+            const int mp = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? bp : 0x7fffffff);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) if (lane + 32 * u == mp) Gr[u] = -1;
+            if (lane == 0) top[3 * l + x] = mp < dm.P ? mp : 0;
+        }
     } else if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         int width = 1;                               // lanes that hold ranks, rounded up to a power of two
@@ -380,7 +393,7 @@ int rp_launch_lpt(rp_ctx *c)
     const RpDims &dm = c->dm;
     size_t smem = sizeof(i64) * (dm.E + dm.P) + sizeof(int) * (dm.E + dm.P);
     int threads = dm.E < 32 ? 32 : (dm.E > 1024 ? 1024 : ((dm.E + 31) / 32) * 32);
-    k_lpt<<<dm.L, threads, smem, c->stream>>>(c->d_Lagg, dm, c->d_pi, c->d_inv, c->d_rank_load);
+    k_lpt<<<dm.L, threads, smem, c->stream>>>(c->d_Lagg, dm, c->d_pi, c->d_inv, c->d_rank_load, c->d_top);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;

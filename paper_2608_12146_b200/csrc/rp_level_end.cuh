@@ -81,9 +81,10 @@ __device__ __forceinline__ void le_weights(const i64 (&e)[U], i64 emin, u64 M, u
 }
 
 // Inclusive prefix sums F[j] of the weights, U consecutive members per thread and round.
-template <int U>
-__device__ __forceinline__ void le_prefix_weights(int P, const i64 *term, u64 cq, int tid, int nt, i64 emin, u64 M, u64 *F,
-                                                  u64 *rsum, u64 *carry_s, bool have_e = false, i64 e_mine = 0)
+// energy(j) gives the terminal energy of member j.
+template <int U, class Energy>
+__device__ __forceinline__ void le_prefix_weights_of(int P, Energy energy, u64 cq, int tid, int nt, i64 emin, u64 M, u64 *F,
+                                                     u64 *rsum, u64 *carry_s)
 {
     const int lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
     for (int base = 0; base < P; base += nt * U) {
@@ -93,9 +94,7 @@ __device__ __forceinline__ void le_prefix_weights(int P, const i64 *term, u64 cq
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int j = j0 + u;
-            if (U == 1 && have_e) e[u] = (j < P) ? e_mine : emin;       // member tid's energy is still in a register
-            else e[u] = (j < P) ? rp_energy(LE_LD(term[3 * (size_t)j]), LE_LD(term[3 * (size_t)j + 1]), LE_LD(term[3 * (size_t)j + 2]))
-                                : emin;
+            e[u] = (j < P) ? energy(j) : emin;
         }
         le_weights<U>(e, emin, M, cq, w);
         u64 v = 0;
@@ -118,6 +117,16 @@ __device__ __forceinline__ void le_prefix_weights(int P, const i64 *term, u64 cq
         if (tid == nt - 1) *carry_s = upto;
         __syncthreads();
     }
+}
+
+// The same from the terminal scores; have_e: member tid's energy is still in a register.
+template <int U>
+__device__ __forceinline__ void le_prefix_weights(int P, const i64 *term, u64 cq, int tid, int nt, i64 emin, u64 M, u64 *F,
+                                                  u64 *rsum, u64 *carry_s, bool have_e = false, i64 e_mine = 0)
+{
+    le_prefix_weights_of<U>(P, [&](int j) {
+        return U == 1 && have_e ? e_mine : rp_energy(LE_LD(term[3 * (size_t)j]), LE_LD(term[3 * (size_t)j + 1]), LE_LD(term[3 * (size_t)j + 2]));
+    }, cq, tid, nt, emin, M, F, rsum, carry_s);
 }
 
 // Lane holding the lexicographically smallest (v0, v1, v2) among the lanes with j != INT_MAX

@@ -449,6 +449,71 @@ def test_permuted_shards(spec):
     rp.rp_destroy(ctx)
 
 
+ROW_CASES = [
+    # name, N, L, E, k, C, D, P, edp, min_rows, pop: one launch for all levels up to 1184 members, else one per level
+    ("row_one_chunk", 70, 32, 8, 2, 4096, 3, 4, None, 3, 21),              # a lane per layer, exactly 32 layers
+    ("row_33_layers", 66, 33, 16, 2, 4096, 2, 8, [1, 0], 4, 9),            # two layers per lane, a permuted shard map
+    ("row_65_layers", 61, 65, 8, 1, 4096, 2, 4, [0, 0], 4, 5),             # four layers per lane
+    ("row_8_chunks", 90, 20, 64, 2, 4096, 4, 32, [0, 1, 1, 0], 3, 160),    # L*P > 512: starts from slices, two chains per CTA
+    ("row_padded", 57, 5, 10, 2, 4096, 3, 5, [0, 1, 1], 3, 310),           # rows padded to whole chunks, four chains per CTA
+    ("row_8_per_cta", 40, 3, 8, 2, 4096, 2, 8, None, 3, 601),              # no warp left for the step records
+    ("row_levels", 60, 24, 32, 2, 4096, 3, 16, [0, 0, 1], 3, 1190),        # one launch per level, four chunks per lane
+    ("row_levels_pad", 45, 6, 6, 2, 4096, 2, 3, None, 3, 1201),            # the same with padded rows
+    ("row_levels_64", 48, 64, 8, 2, 4096, 2, 4, None, 3, 1185),            # the same, two layers per lane
+]
+
+
+@pytest.mark.parametrize("spec", ROW_CASES, ids=[e[0] for e in ROW_CASES])
+def test_one_layer_per_lane_kernel(spec):
+    """The chain kernel most windows use, at the edges of its lanes, chunks, chains per CTA and launch
+    forms; then the same population annealed on by another kernel and by this one again, so that the
+    rank loads change form and back."""
+    name, N, L, E, k, C, D, P, edp, min_rows, pop = spec
+    w = make_window(custom_spec(name, N, L, E, k, C, D, P, pop, 400, data_seed=len(name) * 23 + N))
+    s = w.spec
+    ref = oracle_front(w, edp, min_rows)
+    ctx = load(w, pop=pop, edp=edp, min_rows=min_rows)
+    check_front(w, ctx, ref)
+    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row"
+    want, stats = check_anneal(w, ctx, ref, edp, pop, 3, 40, t_ratio=0.5, check_members=2)
+    assert stats.accepted > 0
+    for knob in (1, 0):
+        rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", knob)
+        want = oracle.anneal(w.lengths, ref["q"], want["final_pop"], ref["R"], s.token_cap, D, n_levels=2, steps=33, t0=1e-4,
+                             t_ratio=0.5, p_reloc=0.5, p_guide=0.3, seed=s.anneal_seed, edp_of_dp=edp, alpha=s.alpha,
+                             beta=s.beta, n_threads=8)
+        rp.rp_anneal(ctx, n_levels=2, steps_per_level=33, t0=1e-4, t_ratio=0.5, p_reloc=0.5, p_guide=0.3)
+        assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (2, pop, 3), np.int64) == want["term"]).all()
+        assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == want["final_pop"]).all()
+        G = 1 + (max(edp) if edp is not None else D - 1)
+        ev = oracle.eval_layouts(w.lengths, ref["q"], want["final_pop"][pop - 1], ref["R"], s.token_cap, D, edp, s.alpha, s.beta)
+        assert (rp.rp_debug_dump(ctx, "W", (ref["R"], G, L, P), np.int32, index=pop - 1) == ev["W"][0]).all()
+    rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("spec", [ROW_CASES[0], ROW_CASES[6]], ids=["one_launch", "launch_per_level"])
+def test_a_wait_of_the_one_layer_per_lane_kernel_that_runs_out(spec):
+    """Its bounded waits, cut short while one chain waits for something that never comes: a time-out
+    status, a context that is refused until it is packed again and then anneals as the oracle does."""
+    name, N, L, E, k, C, D, P, edp, min_rows, pop = spec
+    w = make_window(custom_spec(name, N, L, E, k, C, D, P, pop, 400, data_seed=len(name) * 23 + N))
+    s = w.spec
+    ref = oracle_front(w, edp, min_rows)
+    ctx = load(w, pop=pop, edp=edp, min_rows=min_rows)
+    check_front(w, ctx, ref)
+    rp.rp_debug_set_knob(ctx, "WAIT_POLLS", 10000)
+    rp.rp_debug_set_knob(ctx, "STALL_ONE_CHAIN", 1)
+    for status in (-8, -7):
+        with pytest.raises(rp.RpError) as e:
+            rp.rp_anneal(ctx, n_levels=3, steps_per_level=20, t0=s.t0, t_ratio=0.6, p_reloc=s.p_reloc, p_guide=s.p_guide)
+        assert e.value.status == status
+    rp.rp_debug_set_knob(ctx, "STALL_ONE_CHAIN", 0)
+    rp.rp_debug_set_knob(ctx, "WAIT_POLLS", 0)
+    assert rp.rp_pack_rows(ctx) == (ref["R"], ref["cert"])
+    check_anneal(w, ctx, ref, edp, pop, 3, 20, t_ratio=0.6, check_members=1)
+    rp.rp_destroy(ctx)
+
+
 @pytest.mark.parametrize("spec", [BARRIER_CASES[0], BARRIER_CASES[2], WARP_CHAIN_CASES[0]],
                          ids=["warp_per_candidate", "cooperative", "warp_per_chain"])
 def test_a_wait_that_runs_out_is_reported_and_the_context_survives(spec):
