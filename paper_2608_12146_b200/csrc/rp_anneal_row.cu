@@ -61,47 +61,58 @@ __device__ __forceinline__ int4 add4(const int4 &a, const int4 &b) { return make
 
 // Busiest loads of the layers in `who` (bit x: layer x + first) of row-shard rg once sample mi has left it
 // (sgn = -1) or joined it (+1) and mi2 (>= 0: a swap) the other way round, added up from the samples that sit
-// there; lane x receives layer x + first, the other lanes keep `mine`.  Four layers per pass over the assignment.
-__device__ __noinline__ int rp_row_exact_max(const RpDims &dm, const int *__restrict__ q, const unsigned short *cells,
-                                             const unsigned short *rg_of, int rg, unsigned who, int first, int mi, int mi2, int sgn, int mine)
+// there; lane x receives layer x + first, the other lanes keep `mine`.  The samples are first collected in `list`
+// (its last entry is the counter), then sixteen of their counts are in flight at a time, a rank per lane: nearly always a
+// single layer is asked for, of a row-shard of a hundred short samples.  Kept small: a form with the collection
+// unrolled took 110000 cycles a call on wide and slowed the other chains of the SM threefold (instruction fetches).
+#define ROW_LIST 256
+__device__ __noinline__ int rp_row_exact_max(int N, int P, int LP, const int *__restrict__ q, const unsigned short *cells,
+                                             const unsigned short *rg_of, int *list, int rg, unsigned who, int first, int mi, int mi2,
+                                             int sgn, int mine)
 {
-    const int lane = threadIdx.x & 31, n4 = dm.N >> 2;
-    const uint2 *c4 = (const uint2 *)cells;
-    while (who) {
-        int ly[4], at[4], best[4] = { 0, 0, 0, 0 };
-#pragma unroll
-        for (int x = 0; x < 4; ++x) { at[x] = who ? __ffs(who) - 1 : -1; ly[x] = at[x] < 0 ? 0 : at[x] + first; who &= who - 1; }
-        for (int p0 = 0; p0 < dm.P; p0 += 32) {
-            const bool on = p0 + lane < dm.P;
-            const int *col = q + (on ? p0 + lane : 0);
-            int acc[4] = { 0, 0, 0, 0 };
-            auto add = [&](int i, int f) {
-                const int *row = col + (size_t)i * dm.LP;
-#pragma unroll
-                for (int x = 0; x < 4; ++x) if (at[x] >= 0) acc[x] += f * __ldg(row + ly[x] * dm.P);
-            };
-            for (int b = 0; b < n4; b += 256) {
-                uint2 v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) { const int x = b + 32 * u + lane; v[u] = x < n4 ? __ldcg(c4 + x) : make_uint2(~0u, ~0u); }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const unsigned cc[4] = { v[u].x & 0xffffu, v[u].x >> 16, v[u].y & 0xffffu, v[u].y >> 16 };
+    const int lane = threadIdx.x & 31;
+    int *count = list + ROW_LIST;
+#pragma unroll 1
+    for (; who; who &= who - 1) {
+        const int at = __ffs(who) - 1;
+        const int *layer = q + (size_t)(at + first) * P;
+        int best = 0;
+#pragma unroll 1
+        for (int p0 = 0; p0 < P; p0 += 32) {
+            const bool on = p0 + lane < P;
+            const int *col = layer + (on ? p0 + lane : 0);
+            int acc = sgn * __ldg(col + (size_t)mi * LP), seg = (N + 3) & ~3;
+            if (mi2 >= 0) acc -= sgn * __ldg(col + (size_t)mi2 * LP);
+#pragma unroll 1
+            for (int b = 0; b < N; b += seg) {
+                __syncwarp();
+                if (lane == 0) *count = 0;
+                __syncwarp();
+                const int e = min(b + seg, N);
+#pragma unroll 8
+                for (int i = b + 4 * lane; i < e; i += 128) {
+                    const uint2 v = __ldcg((const uint2 *)(cells + i));            // (the blob is padded to 16 bytes)
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
-                        unsigned here = __ballot_sync(0xffffffffu, cc[h] != 0xffffu && (int)rg_of[cc[h] == 0xffffu ? 0 : cc[h]] == rg);
-                        for (; here; here &= here - 1) add(4 * (b + 32 * u + __ffs(here) - 1) + h, 1);
+                        const unsigned c = ((h & 2 ? v.y : v.x) >> (16 * (h & 1))) & 0xffffu;
+                        if (i + h < e && (int)rg_of[c] == rg) { const int x = atomicAdd(count, 1); if (x < ROW_LIST) list[x] = i + h; }
                     }
                 }
+                __syncwarp();
+                const int n = *count;
+                if (n > ROW_LIST) { seg = ROW_LIST; b = -seg; continue; }          // too many at once: again, a piece at a time
+#pragma unroll 1
+                for (int x0 = 0; x0 < n; x0 += 16) {
+                    int v[16];
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) v[x] = x0 + x < n ? __ldg(col + (size_t)list[x0 + x] * LP) : 0;
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) acc += v[x];
+                }
             }
-            for (int i = n4 << 2; i < dm.N; ++i) if (rg_of[__ldcg(cells + i)] == rg) add(i, 1);
-            add(mi, sgn);
-            if (mi2 >= 0) add(mi2, -sgn);
-#pragma unroll
-            for (int x = 0; x < 4; ++x) best[x] = max(best[x], (int)__reduce_max_sync(0xffffffffu, on ? acc[x] : 0));
+            best = max(best, (int)__reduce_max_sync(0xffffffffu, on ? acc : 0));
         }
-#pragma unroll
-        for (int x = 0; x < 4; ++x) if (lane == at[x]) mine = best[x];
+        if (lane == at) mine = best;
     }
     return mine;
 }
@@ -167,9 +178,14 @@ __device__ __forceinline__ i64 row_energy(i64 s0, i64 s1, i64 s2)       // rp_en
     return s0 + (i64)((u64)s1 / 1000000ull) + (i64)((u64)s2 / 1000000000ull);
 }
 
+// Resident chains the register budget is set for.  Heavy (one chunk per lane) at 12 / 14 / 16 / 19 / 24 chains: 96 / 87.5 /
+// 90 / 100 / 112 ms a plan (spills from 19 on); wide (two) at 12 / 14 / 16 / 19: 10.8 / 11.9 / 11.9 / 16.0 ms; four chunks need the
+// registers of 12.
+#define ROW_CHAINS_PER_SM(LPL, CPL) ((LPL) * (CPL) == 1 ? 14 : 12)
+
 // LPL layers per lane, CPL 16-byte chunks per layer (X.cpl <= CPL of them in use).
 template <int LPL, int CPL, bool CHIP, bool COMP>
-__global__ void __launch_bounds__(CHIP ? ROW_THREADS : 32, CHIP ? 1 : (LPL * CPL > 2 ? 12 : 16))
+__global__ void __launch_bounds__(CHIP ? ROW_THREADS : 32, CHIP ? 1 : ROW_CHAINS_PER_SM(LPL, CPL))
 k_anneal_row(const AnnealArgs A, const RowArgs X)
 {
     constexpr int NCH = LPL * CPL;
@@ -458,7 +474,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
 #pragma unroll
                                 for (int s = 0; s < 2; ++s) {
                                     const unsigned who = __ballot_sync(0xffffffffu, (over >> (2 * y + s)) & 1u);
-                                    if (who) mx[y][s] = rp_row_exact_max(dm, A.q, cells, rg_of, s ? r2 : r1, who, 32 * y, wi, wi2, s ? 1 : -1, mx[y][s]);
+                                    if (who) mx[y][s] = rp_row_exact_max(dm.N, dm.P, dm.LP, A.q, cells, rg_of, (int *)(ch.base + X.off_list), s ? r2 : r1, who, 32 * y, wi, wi2, s ? 1 : -1, mx[y][s]);
                                 }
                         }
                         if (sum32) {
@@ -948,6 +964,7 @@ static void chain_layout(const RpDims &dm, const RpBlob &bl, const RpStatic &sl,
     X.recs = chip && cw < ROW_THREADS / 32 ? std::min(steps, 256) : 0;
     X.off_recs = (int)c;  c += (size_t)2 * X.recs * sizeof(StepRec);
     c = (c + 15) & ~(size_t)15;
+    X.off_list = (int)c;  c += X.comp ? (size_t)4 * (ROW_LIST + 1) : 0;
     X.off_W = (int)c;     c += chip ? (size_t)4 * dm.RG * X.rlp : 0;
     X.chain_bytes = (int)((c + 15) & ~(size_t)15);
     X.smem_bytes = X.off_chain + X.chain_bytes * cw;

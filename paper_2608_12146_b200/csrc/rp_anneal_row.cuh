@@ -13,7 +13,7 @@ struct RowArgs {
     i64 *F_dst, *F_buf;
     int rlp, cpl, comp;
     int off_tab, off_leF, off_chain;                                       // shared memory of the CTA
-    int off_F, off_book, off_wtab, off_spare, off_top, off_cell, off_snap, off_recs, off_W;   // of one chain
+    int off_F, off_book, off_wtab, off_spare, off_top, off_cell, off_snap, off_recs, off_list, off_W;   // of one chain
     int chain_bytes, smem_bytes, cw, recs;
 };
 

@@ -149,7 +149,8 @@ static int copy_out(rp_ctx *c, void *dst, const void *src, size_t bytes)
 
 static void free_population(rp_ctx *c)
 {
-    dev_free(c, c->d_pop_slab); c->d_pop_slab = nullptr;           // every buffer below is a piece of it
+    dev_free(c, c->d_pop_slab); c->d_pop_slab = nullptr;           // every buffer below but d_W is a piece of it
+    dev_free(c, c->d_W); c->W_cells = 0;
     c->buf[0].blob = nullptr; c->buf[1].blob = nullptr;
     c->d_W = nullptr; c->d_wloc = nullptr; c->d_wloc_next = nullptr; c->d_le_scratch = nullptr;
     c->d_wref = nullptr; c->d_wcount = nullptr; c->d_wfree = nullptr; c->d_wfree_head = nullptr;
@@ -460,6 +461,21 @@ __global__ void k_init_population(int P, int N, int *__restrict__ anc, int *__re
 
 static int build_population(rp_ctx *c);
 
+// Rank-load cells in full form, at least `cells` of them (keep: with what the present ones hold).  A population that
+// is annealed on rows kept apart (padded or compressed) needs only as many as it is scored with: one for the seed
+// instead of two per member (wide: 14.5 GB).
+static int need_rank_loads(rp_ctx *c, size_t cells, bool keep)
+{
+    if (cells <= c->W_cells) return RP_OK;
+    const size_t wn = (size_t)c->dm.RG * c->dm.LP;
+    int *W = nullptr;
+    RP_TRY(dev_alloc(c, &W, cells * wn));
+    if (keep && c->W_cells) RP_CUDA(cudaMemcpyAsync(W, c->d_W, sizeof(int) * wn * c->W_cells, cudaMemcpyDeviceToDevice, c->stream));
+    dev_free(c, c->d_W);
+    c->d_W = W; c->W_cells = cells;
+    return RP_OK;
+}
+
 extern "C" int rp_pack_rows(rp_ctx *c, int32_t *n_rows, int32_t *certified)
 {
     if (!c) return RP_ERR_ARG;
@@ -504,14 +520,14 @@ static int build_population(rp_ctx *c)
 
     // population buffers
     free_population(c); free_eval(c);
-    const size_t P = (size_t)c->Ppop, wn = (size_t)dm.RG * dm.LP;
+    const size_t P = (size_t)c->Ppop;
+    RP_TRY(need_rank_loads(c, c->row_mode && rp_row_separate(c) ? 1 : 2 * P, false));
     {
         RpSlab slab = { nullptr, 0 };
         for (int pass = 0; pass < 2; ++pass) {
             slab.off = 0;
             slab.take(&c->buf[0].blob, P * (size_t)c->bl.bytes);
             slab.take(&c->buf[1].blob, P * (size_t)c->bl.bytes);
-            slab.take(&c->d_W, 2 * P * wn);
             slab.take(&c->d_wloc, P);
             slab.take(&c->d_wloc_next, P);
             slab.take(&c->d_le_scratch, 6 * P);
@@ -643,6 +659,7 @@ static int install_population(rp_ctx *c, const int *lay, int n_distinct = 0)
     i64 *best = nullptr;
     RP_TRY(dev_alloc(c, &best, 3));
     int st = ensure_eval_scratch(c, ne, false);
+    if (st == RP_OK) st = need_rank_loads(c, ne, false);
     if (st == RP_OK) st = rp_launch_cells_from_layouts(c, lay, (int)ne, c->d_eval_cells);
     c->cur = 0;
     if (st == RP_OK) st = rp_launch_eval(c, c->d_eval_cells, (int)ne, c->d_W, c->buf[0].blob, c->d_eval_score, nullptr);
@@ -716,6 +733,7 @@ extern "C" int rp_pair_population(rp_ctx *c, int32_t choice_width, int32_t *n_ch
     RP_TRY(dev_alloc(c, &lay, P * dm.N));
     int st = dev_alloc(c, &out, P * dm.N);
     if (st == RP_OK) st = dev_alloc(c, &cnt, 1);
+    if (st == RP_OK) st = need_rank_loads(c, P, true);          // the pairing's rank loads
     const int batch = (int)(P - 1 < 1024 ? P - 1 : 1024);          // members paired per launch (bounds the scratch)
     if (st == RP_OK && batch > 0) st = dev_alloc(c, &prof, (size_t)batch * dm.K * dm.LP);
     cudaError_t e = cudaSuccess;
@@ -837,6 +855,7 @@ extern "C" int rp_init_population(rp_ctx *c, int32_t n_candidates, int32_t choic
         if ((st = dev_alloc(c, &d_order, M)) != RP_OK) break;
         if ((st = dev_alloc(c, &d_nd, 1)) != RP_OK) break;
         if ((st = dev_alloc(c, &dist, (size_t)M * M)) != RP_OK) break;
+        if ((st = need_rank_loads(c, M, true)) != RP_OK) break;
         const int batch = M - 1 < 1024 ? M - 1 : 1024;
         if ((st = dev_alloc(c, &prof, (size_t)batch * dm.K * dm.LP)) != RP_OK) break;
         // trials 2 .. M-1; candidates 0 and 1 start as the length-only seed
@@ -993,7 +1012,8 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
         }
     }
     const bool row = rp_uses_row(c);
-    if (!row && c->full_stale) st = rebuild_rank_loads(c);
+    if (!row) st = need_rank_loads(c, 2 * P, true);
+    if (st == RP_OK && !row && c->full_stale) st = rebuild_rank_loads(c);
     if (!row) c->rows_current = 0;
     c->row_members = c->Ppop;                  // after a level every member has a state of its own
     c->full_stale = row && rp_row_separate(c);

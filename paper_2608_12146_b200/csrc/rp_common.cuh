@@ -127,6 +127,7 @@ struct rp_ctx {
     // population
     RpPopBuf buf[2];
     int *d_W;                  // [2*P_pop][RG][LP] rank-load cells; a member's W sits in the cell wloc says
+    size_t W_cells;            // cells there are (fewer where the population is annealed on rows kept apart)
     int *d_wloc;               // [P_pop] cell of each member's current W (read through d_anc)
     int *d_wloc_next;          // [P_pop] cell each member works in during the next level
     int *d_le_scratch;         // [6*P_pop] ints for the level barrier's cell bookkeeping
