@@ -428,6 +428,7 @@ static int ensure_eval_scratch(rp_ctx *c, size_t n, bool want_W)
         RP_TRY(dev_alloc(c, &c->d_eval_Esum, n * dm.RG));
         RP_TRY(dev_alloc(c, &c->d_eval_tickets, n));
         RP_CUDA(cudaMemsetAsync(c->d_eval_tickets, 0, sizeof(int) * n, c->stream));
+        RP_CUDA(cudaMemsetAsync(c->d_eval_Esum, 0, sizeof(i64) * n * dm.RG, c->stream));
         c->eval_cap = n;
     }
     if (want_W && (int)n > c->eval_W_n) {

@@ -1,12 +1,21 @@
 // Full evaluation of layouts (K4): cell statistics, per-row-shard rank loads W, expert and
 // attention costs, shard work and the score tuple (Sections 3.4-3.5 of the paper).
 //
-// One CTA per layout.  Samples are bucketed by row-shard in shared memory; each warp then
-// owns whole row-shards and adds up the q rows of its members with coalesced loads (q is
-// shared by all layouts and stays L2-resident), so W is produced without atomics and is
-// written at most once.  Algorithmic bytes per layout: N*2 (assignment) + N*L*P*4 (q rows,
-// L2-served) read, R*G*L*P*4 written when W is kept.
+// The work is the sum of the q rows of every row-shard's samples: N*L*P*4 bytes per layout, served by L2
+// (q is shared by all layouts).  Two forms:
+//  * few layouts (k_eval_few: the seed, the incumbent, diagnostics, small batches), bound by latency: a cluster of
+//    CTAs per row-shard, each over its share of the samples, sixteen 16-byte loads in flight per lane; the CTAs'
+//    sums meet through distributed shared memory;
+//  * many layouts (k_eval), bound by L2: a CTA per layout and range of row-shards groups the samples by row-shard
+//    once and a warp sums the rows of a row-shard.
+// In both the CTA that finishes a layout last (atomic ticket) scores it.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "rp_score.cuh"
+
+namespace cg = cooperative_groups;
 
 #define EVAL_THREADS 256
 
@@ -30,98 +39,182 @@ int rp_launch_cells_from_layouts(rp_ctx *c, const int *layouts, int n, unsigned 
     return RP_OK;
 }
 
-// grid = (layouts, splits): the CTAs of a layout share its row-shards (8 per CTA, one per warp);
-// the CTA that finishes last (atomic ticket) gathers the row-shard sums and scores the layout.
-// DEEP: eight members' loads in flight per pass (few layouts: latency matters); otherwise two
-// (many layouts: the CTAs in flight hide the latency and registers are better spent on occupancy).
-template <bool DEEP>
-__global__ void __launch_bounds__(EVAL_THREADS)
-k_eval(const unsigned short *__restrict__ cells, const int *__restrict__ t, const int *__restrict__ q,
-       const int *__restrict__ edp, const int *__restrict__ dp_list, const int *__restrict__ dp_off,
-       RpDims dm, RpBlob bl, int *__restrict__ W_out, char *__restrict__ blob_out,
-       i64 *__restrict__ score_out, double *__restrict__ f64_out, i64 *__restrict__ Esum_g,
-       int *__restrict__ tickets)
-{
-    extern __shared__ __align__(16) unsigned char smraw[];
-    // layout: Q[K] u64 | Esum[RG] | Afx[RG] | U[G] | T[K] | cnt[K] | off[RG+1] | cur[RG] | members[N] | cell_of[N]
-    u64 *Q = (u64 *)smraw;
-    i64 *Esum = (i64 *)(Q + dm.K);
-    i64 *Afx = Esum + dm.RG;
-    i64 *U = Afx + dm.RG;
-    int *T = (int *)(U + dm.G);
-    int *cnt = T + dm.K;
-    int *off = cnt + dm.K;
-    int *cur = off + dm.RG + 1;
-    int *members = cur + dm.RG;
-    unsigned short *cell_of = (unsigned short *)(members + dm.N);
-    __shared__ int last_s;
-    RpSmemState st = { cell_of, T, Q, cnt, Esum, Afx, U };
+// What a launch scores and where its results go.
+struct EvalArgs {
+    RpDims dm;
+    RpBlob bl;
+    const unsigned short *cells;                  // [n][N]
+    const int *t, *q, *edp, *dp_list, *dp_off;
+    int *W_out;                                   // [n][RG][LP], nullable
+    char *blob_out;                               // [n] chain-state blobs (see RpBlob), nullable
+    i64 *score_out;                               // [n][3], nullable
+    double *f64_out;                              // [n][3], nullable
+    i64 *Esum;                                    // [n][RG] row-shard sums handed to the finishing CTA; zero between launches
+    int *tickets;                                 // [n] arrival counters; zero between launches
+};
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = EVAL_THREADS / 32;
-    const int lay = blockIdx.x;
-    const unsigned short *src = cells + (size_t)lay * dm.N;
-    for (int i = tid; i < dm.N; i += EVAL_THREADS) cell_of[i] = src[i];
-    for (int c = tid; c < dm.K; c += EVAL_THREADS) { T[c] = 0; Q[c] = 0; cnt[c] = 0; }
-    for (int x = tid; x <= dm.RG; x += EVAL_THREADS) { off[x] = 0; if (x < dm.RG) cur[x] = 0; }
+// Shared memory of the finishing CTA.
+struct EvalFinish { u64 *Q; i64 *Esum, *Afx, *U; int *T, *cnt; unsigned short *cell_of; };
+__host__ __device__ static inline size_t eval_finish_bytes(const RpDims &dm)
+{
+    return (sizeof(u64) * dm.K + sizeof(i64) * (2 * (size_t)dm.RG + dm.G) + sizeof(int) * 2 * (size_t)dm.K + 2 * (size_t)dm.N + 15) & ~(size_t)15;
+}
+__device__ __forceinline__ EvalFinish eval_finish_views(const RpDims &dm, unsigned char *sm)
+{
+    EvalFinish f;
+    f.Q = (u64 *)sm;
+    f.Esum = (i64 *)(f.Q + dm.K);
+    f.Afx = f.Esum + dm.RG;
+    f.U = f.Afx + dm.RG;
+    f.T = (int *)(f.U + dm.G);
+    f.cnt = f.T + dm.K;
+    f.cell_of = (unsigned short *)(f.cnt + dm.K);
+    return f;
+}
+
+// Scores layout `lay` once its row-shard sums are complete.  All threads of one CTA call; cell_of is in place.
+__device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const EvalFinish &f, int tid)
+{
+    const RpDims &dm = A.dm;
+    const int lane = tid & 31;
+    i64 *eg = A.Esum + (size_t)lay * dm.RG;
+    for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS) { f.Esum[rg] = __ldcg(eg + rg); eg[rg] = 0; }
+    for (int c = tid; c < dm.K; c += EVAL_THREADS) { f.T[c] = 0; f.Q[c] = 0; f.cnt[c] = 0; }
     __syncthreads();
-    rp_accumulate_cells(dm, st, t, tid, EVAL_THREADS);
-    for (int i = tid; i < dm.N; i += EVAL_THREADS) atomicAdd(&off[rp_rowshard(dm, edp, cell_of[i]) + 1], 1);
+    RpSmemState st = { f.cell_of, f.T, f.Q, f.cnt, f.Esum, f.Afx, f.U };
+    rp_accumulate_cells(dm, st, A.t, tid, EVAL_THREADS);
     __syncthreads();
-    if (tid == 0) for (int x = 0; x < dm.RG; ++x) off[x + 1] += off[x];
+    for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS)
+        f.Afx[rg] = rp_attention(dm, st, A.dp_list, A.dp_off, rg / dm.G, rg % dm.G, -1, 0, 0, -1, 0, 0);
     __syncthreads();
-    for (int i = tid; i < dm.N; i += EVAL_THREADS) {
-        int rg = rp_rowshard(dm, edp, cell_of[i]);
-        members[off[rg] + atomicAdd(&cur[rg], 1)] = i;
+    for (int g = tid; g < dm.G; g += EVAL_THREADS) {
+        i64 u = 0;
+        for (int r = 0; r < dm.R; ++r) u += f.Afx[r * dm.G + g] + dm.EC * f.Esum[r * dm.G + g];
+        f.U[g] = u;
     }
     __syncthreads();
-    i64 *esum_lay = Esum_g + (size_t)lay * dm.RG;
+    char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
+    if (tid < 32) {
+        i64 s0 = 0, s1 = 0, s2 = 0;
+        for (int g = lane; g < dm.G; g += 32) { const i64 u = f.U[g]; s1 += u; s0 = u > s0 ? u : s0; }
+        for (int rg = lane; rg < dm.RG; rg += 32) { const i64 J = f.Afx[rg] + dm.EC * f.Esum[rg]; s2 = J > s2 ? J : s2; }
+        for (int o = 16; o; o >>= 1) {
+            const i64 a = __shfl_xor_sync(0xffffffffu, s0, o), c = __shfl_xor_sync(0xffffffffu, s2, o);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            s0 = a > s0 ? a : s0; s2 = c > s2 ? c : s2;
+        }
+        if (lane == 0) {
+            const i64 sc[3] = { s0, s1, s2 };
+            for (int x = 0; x < 3; ++x) {
+                if (A.score_out) A.score_out[(size_t)lay * 3 + x] = sc[x];
+                if (A.f64_out) A.f64_out[(size_t)lay * 3 + x] = (double)sc[x] / (double)dm.SC;
+            }
+            if (b) { i64 *S = (i64 *)(b + A.bl.off_S); S[0] = s0; S[1] = s1; S[2] = s2; S[3] = rp_energy(s0, s1, s2); }
+        }
+    }
+    if (!b) return;
+    for (int c = tid; c < dm.K; c += EVAL_THREADS) {
+        ((u64 *)(b + A.bl.off_Q))[c] = f.Q[c];
+        ((int *)(b + A.bl.off_T))[c] = f.T[c];
+        ((int *)(b + A.bl.off_cnt))[c] = f.cnt[c];
+    }
+    for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS) {
+        ((i64 *)(b + A.bl.off_Esum))[rg] = f.Esum[rg];
+        ((i64 *)(b + A.bl.off_Afx))[rg] = f.Afx[rg];
+        ((i64 *)(b + A.bl.off_Jfx))[rg] = f.Afx[rg] + dm.EC * f.Esum[rg];
+        if (A.bl.off_wtab >= 0)        // W_out holds layout `lay` as RG consecutive slices of the pool
+            ((int *)(b + A.bl.off_wtab))[rg] = lay * dm.RG + rg;
+    }
+    for (int g = tid; g < dm.G; g += EVAL_THREADS) ((i64 *)(b + A.bl.off_U))[g] = f.U[g];
+    for (int i = tid; i < dm.N; i += EVAL_THREADS) ((unsigned short *)(b + A.bl.off_cell))[i] = f.cell_of[i];
+}
+
+__device__ __forceinline__ void eval_load_cells(const EvalArgs &A, int lay, unsigned short *cell_of, int tid)
+{
+    const unsigned short *src = A.cells + (size_t)lay * A.dm.N;
+#pragma unroll 4
+    for (int i = tid; i < A.dm.N; i += EVAL_THREADS) cell_of[i] = __ldg(src + i);
+}
+
+// Sum of one 16-byte column of the listed samples' rows, U loads in flight.
+template <int U>
+__device__ __forceinline__ int4 eval_sum_column(const int4 *__restrict__ col, size_t row4, const int *list, int m0, int m1)
+{
+    int4 a = make_int4(0, 0, 0, 0);
+    for (int mb = m0; mb < m1; mb += U) {
+        int4 v[U];
+#pragma unroll
+        for (int e = 0; e < U; ++e) v[e] = mb + e < m1 ? __ldg(col + (size_t)list[mb + e] * row4) : make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int e = 0; e < U; ++e) { a.x += v[e].x; a.y += v[e].y; a.z += v[e].z; a.w += v[e].w; }
+    }
+    return a;
+}
+
+// Rows of whole 16-byte chunks with at most 32 chunks per layer: a warp takes whole layers, chunk by lane.
+__host__ __device__ static inline bool eval_vec(const RpDims &dm) { return (dm.P & 3) == 0 && dm.P <= 128; }
+__device__ __forceinline__ int eval_layer_max(int m, int lane, int cpl)      // maximum over the cpl lanes of a layer, in its first lane
+{
+    if ((cpl & (cpl - 1)) == 0) { for (int o = cpl >> 1; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o)); }
+    else { const int own = m; for (int o = 1; o < cpl; ++o) m = max(m, __shfl_down_sync(0xffffffffu, own, o)); }
+    return m;
+}
+
+// grid = (layouts, splits): the CTAs of a layout share its row-shards (one per warp at a time).
+__global__ void __launch_bounds__(EVAL_THREADS, 5)
+k_eval(const EvalArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const RpDims &dm = A.dm;
+    const EvalFinish f = eval_finish_views(dm, smraw);
+    int *off = (int *)(smraw + eval_finish_bytes(dm));                  // [RG+1]
+    int *cur = off + dm.RG + 1;                                         // [RG]
+    int *members = cur + dm.RG;                                         // [N]
+    __shared__ int last_s, wsum[EVAL_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = EVAL_THREADS / 32;
+    const int lay = blockIdx.x;
+    eval_load_cells(A, lay, f.cell_of, tid);
+    for (int x = tid; x <= dm.RG; x += EVAL_THREADS) off[x] = 0;
+    __syncthreads();
+    for (int i = tid; i < dm.N; i += EVAL_THREADS) atomicAdd(&off[rp_rowshard(dm, A.edp, f.cell_of[i])], 1);
+    __syncthreads();
+    {   // exclusive prefix sums: a thread takes consecutive row-shards
+        const int chunk = (dm.RG + EVAL_THREADS - 1) / EVAL_THREADS, x0 = min(dm.RG, tid * chunk), x1 = min(dm.RG, x0 + chunk);
+        int sum = 0;
+        for (int x = x0; x < x1; ++x) sum += off[x];
+        int v = sum;
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += y; }
+        if (lane == 31) wsum[warp] = v;
+        __syncthreads();
+        int run = v - sum;
+        for (int w = 0; w < warp; ++w) run += wsum[w];
+        for (int x = x0; x < x1; ++x) { const int c = off[x]; off[x] = run; cur[x] = run; run += c; }
+        if (tid == EVAL_THREADS - 1) off[dm.RG] = dm.N;
+    }
+    __syncthreads();
+    for (int i = tid; i < dm.N; i += EVAL_THREADS) members[atomicAdd(&cur[rp_rowshard(dm, A.edp, f.cell_of[i])], 1)] = i;
+    __syncthreads();
+    i64 *esum_lay = A.Esum + (size_t)lay * dm.RG;
+    const int cpl = dm.P >> 2, lps = eval_vec(dm) ? 32 / cpl : 1, used = lps * cpl, rc = dm.LP >> 2;
     for (int rg = blockIdx.y * nwarps + warp; rg < dm.RG; rg += gridDim.y * nwarps) {
         const int m0 = off[rg], m1 = off[rg + 1];
-        int *wout = W_out ? W_out + ((size_t)lay * dm.RG + rg) * dm.LP : nullptr;
+        int *wout = A.W_out ? A.W_out + ((size_t)lay * dm.RG + rg) * dm.LP : nullptr;
         i64 es;
-        if (dm.P <= 32 && (dm.P & (dm.P - 1)) == 0) {
-            // four strips of 32 columns at a time: four independent loads per member in flight, the
-            // busiest rank of a layer by segmented shuffles over the coalesced column order
+        if (eval_vec(dm)) {
             es = 0;
-            for (int x0 = 0; x0 < dm.LP; x0 += 128) {
-                int acc[4] = { 0, 0, 0, 0 };
-                if constexpr (DEEP) {
-                    for (int mb = m0; mb < m1; mb += 8) {      // eight members' loads in flight before any is added
-                        int v[8][4];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const bool on = mb + e < m1;
-                            const int *row = q + (size_t)(on ? members[mb + e] : 0) * dm.LP + x0 + lane;
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) v[e][u] = (on && x0 + 32 * u + lane < dm.LP) ? __ldg(row + 32 * u) : 0;
-                        }
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) acc[u] += v[e][u];
-                    }
-                } else {
-#pragma unroll 2
-                    for (int m = m0; m < m1; ++m) {
-                        const int *row = q + (size_t)members[m] * dm.LP + x0 + lane;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) if (x0 + 32 * u + lane < dm.LP) acc[u] += __ldg(row + 32 * u);
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int x = x0 + 32 * u + lane;
-                    int v = (x < dm.LP) ? acc[u] : 0;
-                    if (wout && x < dm.LP) wout[x] = v;
-                    for (int o = dm.P >> 1; o; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-                    if ((lane & (dm.P - 1)) == 0 && x < dm.LP) es += v;
-                }
+            for (int c0 = 0; c0 < rc; c0 += used) {
+                const int c = c0 + lane;
+                const bool on = lane < used && c < rc;
+                const int4 a = eval_sum_column<8>((const int4 *)A.q + (on ? c : 0), rc, members, m0, m1);
+                if (wout && on) ((int4 *)wout)[c] = a;
+                const int m = eval_layer_max(on ? max(max(a.x, a.y), max(a.z, a.w)) : 0, lane, cpl);
+                if (on && lane % cpl == 0) es += m;
             }
             for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
         } else {
             es = rp_warp_layer_max_sum(dm, lane, [&](int x) {
                 int s = 0;
-                for (int m = m0; m < m1; ++m) s += __ldg(q + (size_t)members[m] * dm.LP + x);
+                for (int m = m0; m < m1; ++m) s += __ldg(A.q + (size_t)members[m] * dm.LP + x);
                 if (wout) wout[x] = s;
                 return s;
             });
@@ -131,80 +224,130 @@ k_eval(const unsigned short *__restrict__ cells, const int *__restrict__ t, cons
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-        const int ticket = atomicAdd(&tickets[lay], 1);
-        last_s = (ticket == (int)gridDim.y - 1);
-        if (last_s) tickets[lay] = 0;                 // ready for the next launch
+        last_s = (atomicAdd(&A.tickets[lay], 1) == (int)gridDim.y - 1);
+        if (last_s) A.tickets[lay] = 0;                   // ready for the next launch
     }
     __syncthreads();
     if (!last_s) return;
     __threadfence();
-    for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS) Esum[rg] = ((volatile i64 *)esum_lay)[rg];
+    eval_finish(A, lay, f, tid);
+}
+
+// grid = (MS, row-shards, layouts), clusters of MS CTAs along x: CTA x of a row-shard takes the samples of
+// range x, then the layers of range x of the summed row.
+__global__ void __launch_bounds__(EVAL_THREADS)
+k_eval_few(const EvalArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const RpDims &dm = A.dm;
+    const cg::cluster_group cl = cg::this_cluster();
+    const int MS = gridDim.x, ms = blockIdx.x, rg = blockIdx.y, lay = blockIdx.z;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = EVAL_THREADS / 32;
+    int *part = (int *)smraw;                                           // [LP] this CTA's share of the sum
+    int *list = part + dm.LP;                                           // [N / MS + 1] its samples
+    __shared__ int n_s, last_s;
+    __shared__ u64 es_s;
+    const unsigned short *cells = A.cells + (size_t)lay * dm.N;
+    if (tid == 0) { n_s = 0; es_s = 0; }
     __syncthreads();
-    i64 sc[3];
-    rp_rows_to_score(dm, st, dp_list, dp_off, tid, EVAL_THREADS, sc);
-    if (blob_out) {      // the chain-state blob of this layout (see RpBlob)
-        char *b = blob_out + (size_t)lay * bl.bytes;
-        for (int c = tid; c < dm.K; c += EVAL_THREADS) {
-            ((u64 *)(b + bl.off_Q))[c] = Q[c];
-            ((int *)(b + bl.off_T))[c] = T[c];
-            ((int *)(b + bl.off_cnt))[c] = cnt[c];
-        }
-        for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS) {
-            ((i64 *)(b + bl.off_Esum))[rg] = Esum[rg];
-            ((i64 *)(b + bl.off_Afx))[rg] = Afx[rg];
-            ((i64 *)(b + bl.off_Jfx))[rg] = Afx[rg] + dm.EC * Esum[rg];
-        }
-        for (int g = tid; g < dm.G; g += EVAL_THREADS) ((i64 *)(b + bl.off_U))[g] = U[g];
-        if (bl.off_wtab >= 0)          // W_out holds layout `lay` as RG consecutive slices of the pool
-            for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS) ((int *)(b + bl.off_wtab))[rg] = lay * dm.RG + rg;
-        for (int i = tid; i < dm.N; i += EVAL_THREADS) ((unsigned short *)(b + bl.off_cell))[i] = cell_of[i];
-        if (tid == 0) {
-            i64 *S = (i64 *)(b + bl.off_S);
-            S[0] = sc[0]; S[1] = sc[1]; S[2] = sc[2]; S[3] = rp_energy(sc[0], sc[1], sc[2]);
-        }
+    const int row = rg / dm.G, g = rg % dm.G;
+    const int i0 = (int)((long long)dm.N * ms / MS), i1 = (int)((long long)dm.N * (ms + 1) / MS);
+#pragma unroll 8
+    for (int i = i0 + tid; i < i1; i += EVAL_THREADS) {
+        const int c = __ldg(cells + i);
+        if (c / dm.D == row && __ldg(A.edp + c % dm.D) == g) list[atomicAdd(&n_s, 1)] = i;
     }
+    __syncthreads();
+    const int cpl = dm.P >> 2, rc = dm.LP >> 2, n = n_s;
+    for (int c0 = 32 * warp; c0 < rc; c0 += 32 * nwarps) {
+        const int c = c0 + lane;
+        const int4 a = eval_sum_column<16>((const int4 *)A.q + (c < rc ? c : 0), rc, list, 0, n);
+        if (c < rc) ((int4 *)part)[c] = a;
+    }
+    cl.sync();
+    const int l0 = dm.L * ms / MS, l1 = dm.L * (ms + 1) / MS, lps = 32 / cpl, used = lps * cpl;
+    int4 *wout = A.W_out ? (int4 *)(A.W_out + ((size_t)lay * dm.RG + rg) * dm.LP) : nullptr;
+    i64 es = 0;
+    for (int c0 = l0 * cpl + warp * used; c0 < l1 * cpl; c0 += nwarps * used) {
+        const int c = c0 + lane;
+        const bool on = lane < used && c < l1 * cpl;
+        int4 a = make_int4(0, 0, 0, 0);
+        if (on)
+            for (int x = 0; x < MS; ++x) {
+                const int4 v = ((const int4 *)cl.map_shared_rank(part, x))[c];
+                a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+            }
+        if (wout && on) wout[c] = a;
+        const int m = eval_layer_max(on ? max(max(a.x, a.y), max(a.z, a.w)) : 0, lane, cpl);
+        if (on && lane % cpl == 0) es += m;
+    }
+    for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
+    if (lane == 0 && es) atomicAdd(&es_s, (u64)es);
+    cl.sync();                                            // nobody reads another CTA's shared memory from here on
     if (tid == 0) {
-        for (int x = 0; x < 3; ++x) {
-            if (score_out) score_out[(size_t)lay * 3 + x] = sc[x];
-            if (f64_out) f64_out[(size_t)lay * 3 + x] = (double)sc[x] / (double)dm.SC;
-        }
+        if (es_s) atomicAdd((u64 *)(A.Esum + (size_t)lay * dm.RG + rg), es_s);
+        __threadfence();
+        last_s = (atomicAdd(&A.tickets[lay], 1) == (int)(gridDim.x * gridDim.y) - 1);
+        if (last_s) A.tickets[lay] = 0;
     }
+    if (wout) __threadfence();
+    __syncthreads();
+    if (!last_s) return;
+    __threadfence();
+    const EvalFinish f = eval_finish_views(dm, smraw);
+    eval_load_cells(A, lay, f.cell_of, tid);
+    eval_finish(A, lay, f, tid);
 }
 
 static size_t eval_smem_bytes(const RpDims &dm)
 {
-    size_t b = sizeof(u64) * dm.K + sizeof(i64) * (2 * (size_t)dm.RG + dm.G);
-    b += sizeof(int) * (2 * (size_t)dm.K + 2 * (size_t)dm.RG + 1 + dm.N);
-    b += sizeof(unsigned short) * dm.N;
-    return (b + 15) & ~(size_t)15;
+    return (eval_finish_bytes(dm) + sizeof(int) * (2 * (size_t)dm.RG + 1 + dm.N) + 15) & ~(size_t)15;
 }
 
-int rp_launch_eval(rp_ctx *c, const unsigned short *cells, int n, int *W_out, char *blob_out,
-                   i64 *score_out, double *f64_out)
+#define EVAL_SMEM_MAX (220 * 1024)
+
+// One launch either way; the scratch (Esum, tickets) is zero before and after it.
+static int eval_launch(rp_ctx *c, const unsigned short *cells, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out,
+                       i64 *Esum, int *tickets)
 {
     const RpDims &dm = c->dm;
-    size_t smem = eval_smem_bytes(dm);
-    if (smem > 220 * 1024) return RP_ERR_RANGE;
-    if (smem > 32 * 1024) {
-        RP_CUDA(cudaFuncSetAttribute(k_eval<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        RP_CUDA(cudaFuncSetAttribute(k_eval<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = eval_smem_bytes(dm);
+    if (smem > EVAL_SMEM_MAX) return RP_ERR_RANGE;
+    EvalArgs A;
+    A.dm = dm; A.bl = c->bl; A.cells = cells; A.t = c->d_t; A.q = c->d_q; A.edp = c->d_edp; A.dp_list = c->d_dp_list; A.dp_off = c->d_dp_off;
+    A.W_out = W_out; A.blob_out = blob_out; A.score_out = score_out; A.f64_out = f64_out; A.Esum = Esum; A.tickets = tickets;
+    // A cluster per row-shard scans the assignment once per row-shard, a CTA per layout groups it once: the first
+    // form up to about sixteen waves of its CTAs.
+    if (eval_vec(dm) && (long long)n * dm.RG <= 16 * 148 * 8 && n < 65536 && dm.RG < 65536 && dm.LP <= 16384) {
+        int MS = 1;
+        while (MS < 8 && (long long)n * dm.RG * MS < 148 * 4 && dm.N >= 64 * MS) MS *= 2;
+        const size_t sm = std::max(eval_finish_bytes(dm), sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2));
+        if (sm > EVAL_SMEM_MAX) return RP_ERR_RANGE;
+        if (sm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_few, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(MS, dm.RG, n); cfg.blockDim = dim3(EVAL_THREADS);
+        cfg.dynamicSmemBytes = sm; cfg.stream = c->stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = MS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        cfg.attrs = at; cfg.numAttrs = 1;
+        RP_CUDA(cudaLaunchKernelEx(&cfg, k_eval_few, A));
+    } else {
+        if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
+        // every SM holds five CTAs: split the layouts' row-shards until they are filled
+        int splits = (5 * 148 + n - 1) / n;
+        const int max_splits = (dm.RG + EVAL_THREADS / 32 - 1) / (EVAL_THREADS / 32);
+        splits = std::max(1, std::min(splits, max_splits));
+        k_eval<<<dim3(n, splits), EVAL_THREADS, smem, c->stream>>>(A);
     }
-    // few layouts: split each one's row-shards over several CTAs so the GPU is not left idle
-    int splits = (2 * 148 + n - 1) / n;
-    const int max_splits = (dm.RG + EVAL_THREADS / 32 - 1) / (EVAL_THREADS / 32);
-    if (splits > max_splits) splits = max_splits;
-    if (splits < 1) splits = 1;
-    if ((long long)n * splits <= 2 * 148)
-        k_eval<true><<<dim3(n, splits), EVAL_THREADS, smem, c->stream>>>(cells, c->d_t, c->d_q, c->d_edp, c->d_dp_list, c->d_dp_off,
-                                                                        dm, c->bl, W_out, blob_out, score_out, f64_out,
-                                                                        c->d_eval_Esum, c->d_eval_tickets);
-    else
-        k_eval<false><<<dim3(n, splits), EVAL_THREADS, smem, c->stream>>>(cells, c->d_t, c->d_q, c->d_edp, c->d_dp_list, c->d_dp_off,
-                                                                         dm, c->bl, W_out, blob_out, score_out, f64_out,
-                                                                         c->d_eval_Esum, c->d_eval_tickets);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
+}
+
+int rp_launch_eval(rp_ctx *c, const unsigned short *cells, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out)
+{
+    return eval_launch(c, cells, n, W_out, blob_out, score_out, f64_out, c->d_eval_Esum, c->d_eval_tickets);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -265,34 +408,39 @@ int rp_launch_build_static(rp_ctx *c)
 // ---------------------------------------------------------------------------------------------
 struct RpDiagDev { double cv_identity, cv_placed; i64 s_ep, t_ep, n_ep; i64 afx_sum, s0; };
 
-// One thread per layer, each with plain sequential IEEE sums (no fused multiply-add), then
-// thread 0 averages the layers in order.
-__global__ void k_diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, RpDims dm,
-                          RpDiagDev *__restrict__ out)
+// One warp per layer: the lanes fetch the rank loads, one lane adds them up with plain sequential IEEE sums (no fused
+// multiply-add); then thread 0 averages the layers in order.
+#define DIAG_THREADS 1024
+__global__ void __launch_bounds__(DIAG_THREADS)
+k_diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, RpDims dm, RpDiagDev *__restrict__ out)
 {
-    extern __shared__ double cvs[];          // [2][L]
-    const int l = threadIdx.x;
-    if (l < dm.L) {
-        for (int which = 0; which < 2; ++which) {
-            double mean = 0.0;
-            for (int p = 0; p < dm.P; ++p) {
-                i64 g = 0;
-                if (which) g = rank_load[(size_t)l * dm.P + p];
-                else for (int n = 0; n < dm.H; ++n) g += Lagg[(size_t)l * dm.E + p * dm.H + n];
-                mean = __dadd_rn(mean, (double)g);
+    extern __shared__ double cvs[];          // [2][L], then one row of rank loads per warp
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double *G = cvs + 2 * dm.L + (size_t)warp * dm.P;
+    for (int x = warp; x < 2 * dm.L; x += DIAG_THREADS / 32) {
+        const int l = x >> 1, which = x & 1;
+        for (int p = lane; p < dm.P; p += 32) {
+            i64 g = 0;
+            if (which) g = __ldg(rank_load + (size_t)l * dm.P + p);
+            else {
+#pragma unroll 4
+                for (int n = 0; n < dm.H; ++n) g += __ldg(Lagg + (size_t)l * dm.E + p * dm.H + n);
             }
+            G[p] = (double)g;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            double mean = 0.0, var = 0.0;
+            for (int p = 0; p < dm.P; ++p) mean = __dadd_rn(mean, G[p]);
             mean = __ddiv_rn(mean, (double)dm.P);
-            double var = 0.0;
             for (int p = 0; p < dm.P; ++p) {
-                i64 g = 0;
-                if (which) g = rank_load[(size_t)l * dm.P + p];
-                else for (int n = 0; n < dm.H; ++n) g += Lagg[(size_t)l * dm.E + p * dm.H + n];
-                const double d = __dsub_rn((double)g, mean);
+                const double d = __dsub_rn(G[p], mean);
                 var = __dadd_rn(var, __dmul_rn(d, d));
             }
             var = __ddiv_rn(var, (double)dm.P);
             cvs[which * dm.L + l] = (mean > 0.0) ? __ddiv_rn(__dsqrt_rn(var), mean) : 0.0;
         }
+        __syncwarp();
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -375,22 +523,16 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
         k_layouts_to_cells<<<(dm.N + 255) / 256, 256, 0, c->stream>>>(dl, dm.N, dm.K, (unsigned short *)(buf + off_cells),
                                                                      c->d_status);
         ++g_rp_launches;
-        const size_t smem = eval_smem_bytes(dm);
-        if (smem > 220 * 1024) { st = RP_ERR_RANGE; break; }
-        if (smem > 32 * 1024) {
-            e = cudaFuncSetAttribute(k_eval<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        st = eval_launch(c, (const unsigned short *)(buf + off_cells), 1, (int *)(buf + off_W), buf + off_blob, nullptr, nullptr,
+                         (i64 *)(buf + off_es), (int *)(buf + off_tk));
+        if (st != RP_OK) break;
+        RpDiagDev *res = (RpDiagDev *)(buf + off_res);
+        const size_t cv_smem = sizeof(double) * (2 * (size_t)dm.L + (DIAG_THREADS / 32) * (size_t)dm.P);
+        if (cv_smem > 32 * 1024) {
+            e = cudaFuncSetAttribute(k_diag_cv, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX);
             if (e != cudaSuccess) break;
         }
-        int splits = 2 * 148;
-        const int max_splits = (dm.RG + EVAL_THREADS / 32 - 1) / (EVAL_THREADS / 32);
-        if (splits > max_splits) splits = max_splits;
-        k_eval<true><<<dim3(1, splits), EVAL_THREADS, smem, c->stream>>>((const unsigned short *)(buf + off_cells), c->d_t, c->d_q,
-                                                                  c->d_edp, c->d_dp_list, c->d_dp_off, dm, c->bl,
-                                                                  (int *)(buf + off_W), buf + off_blob, nullptr, nullptr,
-                                                                  (i64 *)(buf + off_es), (int *)(buf + off_tk));
-        ++g_rp_launches;
-        RpDiagDev *res = (RpDiagDev *)(buf + off_res);
-        k_diag_cv<<<1, ((dm.L + 31) / 32) * 32, sizeof(double) * 2 * dm.L, c->stream>>>(c->d_Lagg, c->d_rank_load, dm, res);
+        k_diag_cv<<<1, DIAG_THREADS, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, dm, res);
         ++g_rp_launches;
         k_diag_peaks<<<148, 256, 0, c->stream>>>((const int *)(buf + off_W), buf + off_blob, c->bl, dm, res);
         ++g_rp_launches;
@@ -463,24 +605,15 @@ extern "C" int rp_eval_layouts_noalloc(rp_ctx *c, const int32_t *layouts, int32_
         g_noalloc_addr[cur] = p;
     }
     RpNoAllocScratch *sc = (RpNoAllocScratch *)g_noalloc_addr[cur];
-    // the array keeps what the previous call left: the arrival counters must start at zero
+    // the array keeps what the previous call left: the arrival counters and the row-shard sums must start at zero
     RP_CUDA(cudaMemsetAsync(sc->tickets, 0, sizeof(int) * n, c->stream));
+    RP_CUDA(cudaMemsetAsync(sc->esum, 0, sizeof(i64) * (size_t)n * dm.RG, c->stream));
     RP_CUDA(cudaMemsetAsync(c->d_status + RP_SW_BAD_LAYOUT, 0, sizeof(int), c->stream));
     const long long total = (long long)n * dm.N;
     k_layouts_to_cells<<<(int)((total + 255) / 256), 256, 0, c->stream>>>(layouts, total, dm.K, sc->cells, c->d_status);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
-    if (smem > 32 * 1024)
-        RP_CUDA(cudaFuncSetAttribute(k_eval<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int splits = (2 * 148 + n - 1) / n;
-    const int max_splits = (dm.RG + EVAL_THREADS / 32 - 1) / (EVAL_THREADS / 32);
-    if (splits > max_splits) splits = max_splits;
-    if (splits < 1) splits = 1;
-    k_eval<false><<<dim3(n, splits), EVAL_THREADS, smem, c->stream>>>(sc->cells, c->d_t, c->d_q, c->d_edp, c->d_dp_list, c->d_dp_off,
-                                                              dm, c->bl, nullptr, nullptr, (i64 *)score_fx, score_f64, sc->esum,
-                                                              sc->tickets);
-    ++g_rp_launches;
-    RP_CUDA(cudaGetLastError());
+    RP_TRY(eval_launch(c, sc->cells, n, nullptr, nullptr, (i64 *)score_fx, score_f64, sc->esum, sc->tickets));
     int bad = 0;
     RP_CUDA(cudaMemcpyAsync(&bad, c->d_status + RP_SW_BAD_LAYOUT, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     RP_CUDA(cudaStreamSynchronize(c->stream));

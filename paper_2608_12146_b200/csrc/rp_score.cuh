@@ -84,29 +84,3 @@ __device__ __forceinline__ void rp_accumulate_cells(const RpDims &dm, const RpSm
         atomicAdd(&st.cnt[c], 1);
     }
 }
-
-// Afx for every row-shard, then U[g] and the score tuple (Eq. lexicographic-score).
-// Needs Esum, T, Q in shared memory; all threads call; result valid in thread 0 after return.
-__device__ __forceinline__ void rp_rows_to_score(const RpDims &dm, const RpSmemState &st,
-                                                 const int *__restrict__ dp_list, const int *__restrict__ dp_off,
-                                                 int tid, int nt, i64 out[3])
-{
-    for (int rg = tid; rg < dm.RG; rg += nt)
-        st.Afx[rg] = rp_attention(dm, st, dp_list, dp_off, rg / dm.G, rg % dm.G, -1, 0, 0, -1, 0, 0);
-    __syncthreads();
-    for (int g = tid; g < dm.G; g += nt) {
-        i64 u = 0;
-        for (int r = 0; r < dm.R; ++r) u += st.Afx[r * dm.G + g] + dm.EC * st.Esum[r * dm.G + g];
-        st.U[g] = u;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        i64 s0 = 0, s1 = 0, s2 = 0;
-        for (int g = 0; g < dm.G; ++g) { s1 += st.U[g]; s0 = st.U[g] > s0 ? st.U[g] : s0; }
-        for (int rg = 0; rg < dm.RG; ++rg) {
-            i64 J = st.Afx[rg] + dm.EC * st.Esum[rg];
-            s2 = J > s2 ? J : s2;
-        }
-        out[0] = s0; out[1] = s1; out[2] = s2;
-    }
-}
