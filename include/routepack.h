@@ -204,8 +204,8 @@ int rp_eval_population(rp_ctx *ctx, const int32_t *layouts, int32_t n, int64_t *
  * framework has already handed all free device memory to its own pool, or from a section
  * where an allocation would stall the whole device (cudaMalloc and cudaFree synchronise it).
  * The paper has no counterpart; this is a deployment variant of the full evaluation.
- * It calls no cudaMalloc/cudaFree or any allocating routine: its working memory (16-bit cell
- * ids, row-shard sums, arrival counters; about 1.3 MiB) is a fixed array inside the library
+ * It calls no cudaMalloc/cudaFree or any allocating routine: its working memory (samples grouped by
+ * row-shard, row-shard sums, arrival counters; about 1.4 MiB) is a fixed array inside the library
  * image, present on every GPU that loads the library until the process exits.
  *   layouts [n][N] int32, score_fx [n][3] int64 (nullable), score_f64 [n][3] double
  *   (nullable): all three must be DEVICE pointers (a host array would need a staging buffer).

@@ -1,7 +1,6 @@
 // Fixed-row population annealing (Algorithm 3 of the paper): the per-level chain kernel
 // (K5: GuidedProposal, feasibility, IncrementalScore, Metropolis), the level barrier
-// (K6 incumbent update + K7 Boltzmann weights and systematic resampling) and the final
-// validation (K8).
+// (K6 incumbent update + K7 Boltzmann weights and systematic resampling).
 //
 // Mapping.  One CTA runs one chain for all K steps of a level.  The chain's small state
 // (assignment, cell statistics, per-row-shard costs, shard work) lives in shared memory.
@@ -594,14 +593,17 @@ int rp_upload_levels(rp_ctx *c, int n_levels)
         RP_TRY(dev_alloc(c, &d, (size_t)n_levels));
         c->d_levels = d; c->levels_dev_cap = n_levels;
     }
-    RpLevelDev *h = (RpLevelDev *)malloc(sizeof(RpLevelDev) * n_levels);
+    // through the pinned mail area where they fit (nothing in it is in use: the placement has been handed over or is
+    // kept in the first half), a piece at a time otherwise
+    const size_t bytes = sizeof(RpLevelDev) * n_levels;
+    RpLevelDev *h = bytes <= RP_MAIL_BYTES / 2 ? (RpLevelDev *)(rp_mail(c) + RP_MAIL_BYTES / 2) : (RpLevelDev *)malloc(bytes);
     const u32 k0 = (u32)c->cfg.seed, k1 = (u32)(c->cfg.seed >> 32);
     for (int n = 0; n < n_levels; ++n) {
         h[n].tau = c->h_levels[n].tau; h[n].cq = c->h_levels[n].cq;
         h[n].resample_x = host_philox_x(0u, (u32)n, 0u, 3u, k0, k1); h[n].pad = 0;
     }
-    const cudaError_t e = cudaMemcpyAsync(c->d_levels, h, sizeof(RpLevelDev) * n_levels, cudaMemcpyHostToDevice, c->stream);
-    free(h);            // pageable source: staged before the call returned
+    const cudaError_t e = cudaMemcpyAsync(c->d_levels, h, bytes, cudaMemcpyHostToDevice, c->stream);
+    if (bytes > RP_MAIL_BYTES / 2) free(h);            // pageable source: staged before the call returned
     if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
     return RP_OK;
 }
@@ -654,41 +656,6 @@ int rp_launch_anneal_level(rp_ctx *c, int level, int n_levels, const rp_anneal_p
     else { if (alias) { COOP_PICK(false, true) } else { COOP_PICK(false, false) } }
 #undef COOP_PICK
 #undef COOP_LAUNCH
-    ++g_rp_launches;
-    RP_CUDA(cudaGetLastError());
-    return RP_OK;
-}
-
-// ---------------------------------------------------------------------------------------------
-// Validate(x*): every sample in a real cell, no empty cell, no cell over the token cap.
-// (Score consistency and non-regression are checked by the caller from a full rescoring.)
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024)
-k_validate(const int *__restrict__ layout, const int *__restrict__ t, RpDims dm, int *__restrict__ fill,
-           int *__restrict__ cnt, int *__restrict__ status)
-{
-    const int tid = threadIdx.x;
-    for (int c = tid; c < dm.K; c += 1024) { fill[c] = 0; cnt[c] = 0; }
-    __syncthreads();
-    int bad = 0;
-    for (int i = tid; i < dm.N; i += 1024) {
-        int c = layout[i];
-        if (c < 0 || c >= dm.K) { bad |= 1; continue; }
-        atomicAdd(&fill[c], t[i]);
-        atomicAdd(&cnt[c], 1);
-    }
-    __syncthreads();
-    for (int c = tid; c < dm.K; c += 1024) {
-        if (cnt[c] < 1) bad |= 2;
-        if (fill[c] > dm.C) bad |= 4;
-    }
-    if (bad) atomicOr(&status[RP_SW_VALIDATE], bad);
-}
-
-int rp_launch_validate(rp_ctx *c)
-{
-    int *fill = (int *)c->d_sort_keys;                 // scratch: 2*K ints fit (K <= N)
-    k_validate<<<1, 1024, 0, c->stream>>>(c->d_inc_layout, c->d_t, c->dm, fill, fill + c->dm.K, c->d_status);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;

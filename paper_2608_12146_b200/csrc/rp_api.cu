@@ -58,17 +58,11 @@ int rp_get_pool(int device, cudaMemPool_t *out)
     return RP_OK;
 }
 
-extern "C" int rp_release_cached_memory(void)
-{
-    for (int d = 0; d < RP_MAX_DEVICES; ++d)
-        if (g_pool_ready[d]) RP_CUDA(cudaMemPoolTrimTo(g_pools[d], 0));
-    return RP_OK;
-}
-
-// Pinned staging blocks (512 bytes) for reading scalars back without a synchronous pageable copy;
-// recycled across contexts because pinning memory is slow.
+// Pinned blocks the kernels write scalars, placements and layouts to; recycled across contexts because pinning memory is
+// slow.  At most RP_PIN_KEEP idle ones are kept; rp_release_cached_memory() gives those back too.
 #include <mutex>
 #include <vector>
+#define RP_PIN_KEEP 16
 static std::mutex g_pin_mutex;
 static std::vector<void *> g_pin_free;
 static void *pin_take()
@@ -78,19 +72,22 @@ static void *pin_take()
         if (!g_pin_free.empty()) { void *p = g_pin_free.back(); g_pin_free.pop_back(); return p; }
     }
     void *p = nullptr;
-    if (cudaHostAlloc(&p, 512, cudaHostAllocDefault) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (cudaHostAlloc(&p, 512 + RP_MAIL_BYTES, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     return p;
 }
 static void pin_give(void *p)
 {
     if (!p) return;
-    std::lock_guard<std::mutex> lk(g_pin_mutex);
-    g_pin_free.push_back(p);
+    {
+        std::lock_guard<std::mutex> lk(g_pin_mutex);
+        if (g_pin_free.size() < RP_PIN_KEEP) { g_pin_free.push_back(p); return; }
+    }
+    cudaFreeHost(p);
 }
 
-// A side stream with two events, recycled across contexts of a device like the pinned blocks:
+// A side stream with four events, recycled across contexts of a device like the pinned blocks:
 // packing needs only the lengths, so it runs beside the check / placement / projection kernels.
-struct RpSide { int device; cudaStream_t stream; cudaEvent_t fork, join; };
+struct RpSide { int device; cudaStream_t stream; cudaEvent_t fork, join, t0, t1; };      // t0, t1: rp_anneal's device time
 static std::vector<RpSide *> g_side_free;
 static RpSide *side_take(int device)
 {
@@ -107,7 +104,8 @@ static RpSide *side_take(int device)
     s->device = device;
     if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreate(&s->t0) != cudaSuccess || cudaEventCreate(&s->t1) != cudaSuccess) {
         cudaGetLastError();
         delete s;
         return nullptr;
@@ -122,6 +120,16 @@ static void side_give(RpSide *s)
 }
 
 
+extern "C" int rp_release_cached_memory(void)
+{
+    for (int d = 0; d < RP_MAX_DEVICES; ++d)
+        if (g_pool_ready[d]) RP_CUDA(cudaMemPoolTrimTo(g_pools[d], 0));
+    std::lock_guard<std::mutex> lk(g_pin_mutex);
+    for (void *p : g_pin_free) cudaFreeHost(p);
+    g_pin_free.clear();
+    return RP_OK;
+}
+
 // Optional stage timing: one flag for the process (a context only exists once rp_window_load has
 // already queued the front end), events per context.
 static int g_stage_timing = 0;
@@ -132,7 +140,7 @@ static void stage_mark(rp_ctx *c, int which, cudaStream_t stream)
     else cudaGetLastError();
 }
 
-static bool is_device_ptr(const void *p)
+bool rp_is_device_ptr(const void *p)
 {
     cudaPointerAttributes at;
     cudaError_t e = cudaPointerGetAttributes(&at, p);
@@ -176,10 +184,10 @@ static void free_trace(rp_ctx *c)
 
 static void free_eval(rp_ctx *c)
 {
-    dev_free(c, c->d_eval_score); dev_free(c, c->d_eval_f64); dev_free(c, c->d_eval_W);
-    dev_free(c, c->d_eval_cells); dev_free(c, c->d_eval_Esum); dev_free(c, c->d_eval_tickets);
-    c->d_eval_score = nullptr; c->d_eval_f64 = nullptr; c->d_eval_W = nullptr;
-    c->d_eval_cells = nullptr; c->d_eval_Esum = nullptr; c->d_eval_tickets = nullptr;
+    dev_free(c, c->d_eval_slab); dev_free(c, c->d_eval_W);
+    c->d_eval_slab = nullptr; c->d_eval_W = nullptr;
+    c->d_eval_score = nullptr; c->d_eval_f64 = nullptr; c->d_eval_list = nullptr; c->d_eval_off = nullptr;
+    c->d_eval_Esum = nullptr; c->d_eval_tickets = nullptr;
     c->eval_cap = 0; c->eval_W_n = 0;
 }
 
@@ -188,7 +196,7 @@ extern "C" void rp_destroy(rp_ctx *c)
     if (!c) return;
     cudaStreamSynchronize(c->stream);
     free_population(c); free_trace(c); free_eval(c);
-    dev_free(c, c->own_t); dev_free(c, c->own_a); dev_free(c, c->d_load_slab); dev_free(c, c->d_static); dev_free(c, c->d_levels);
+    dev_free(c, c->own_t); dev_free(c, c->own_a); dev_free(c, c->d_load_slab); dev_free(c, c->d_levels);
     pin_give(c->h_pin);
     for (int x = 0; x < RP_STAGE_EVENTS; ++x) if (c->ev_stage[x]) cudaEventDestroy(c->ev_stage[x]);
     side_give((RpSide *)c->side);
@@ -199,15 +207,6 @@ extern "C" void rp_destroy(rp_ctx *c)
 static int reset_status(rp_ctx *c)
 {
     RP_CUDA(cudaMemsetAsync(c->d_status, 0, sizeof(int) * RP_SW_COUNT, c->stream));
-    return RP_OK;
-}
-
-static int read_status(rp_ctx *c, int out[RP_SW_COUNT])
-{
-    int *stage = (int *)(c->h_pin + 56);
-    RP_CUDA(cudaMemcpyAsync(stage, c->d_status, sizeof(int) * RP_SW_COUNT, cudaMemcpyDeviceToHost, c->stream));
-    RP_CUDA(cudaStreamSynchronize(c->stream));
-    memcpy(out, stage, sizeof(int) * RP_SW_COUNT);
     return RP_OK;
 }
 
@@ -258,13 +257,13 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
     const size_t n_a = (size_t)N * L * E;
     int st = RP_OK;
     do {
-        if (is_device_ptr(lengths)) c->d_t = lengths;
+        if (rp_is_device_ptr(lengths)) c->d_t = lengths;
         else {
             if ((st = dev_alloc(c, &c->own_t, N)) != RP_OK) break;
             if (cudaMemcpyAsync(c->own_t, lengths, sizeof(int) * N, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) { st = RP_ERR_CUDA; break; }
             c->d_t = c->own_t;
         }
-        if (is_device_ptr(demand)) c->d_a = demand;
+        if (rp_is_device_ptr(demand)) c->d_a = demand;
         else {
             if ((st = dev_alloc(c, &c->own_a, n_a)) != RP_OK) break;
             if (cudaMemcpyAsync(c->own_a, demand, sizeof(int) * n_a, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) { st = RP_ERR_CUDA; break; }
@@ -275,11 +274,13 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
         while (n_pow2 < N) n_pow2 <<= 1;
         const size_t n_tab = (size_t)2 * D + G + 1;
         RpSlab slab = { nullptr, 0 };
+        size_t n_zero = 0;
         for (int pass = 0; pass < 2 && st == RP_OK; ++pass) {
             slab.off = 0;
-            slab.take(&c->d_Lagg, (size_t)L * E);
+            slab.take(&c->d_Lagg, (size_t)L * E);                 // (these three start at zero: one memset)
             slab.take(&c->d_status, RP_SW_COUNT);
             slab.take(&c->d_counters, 8);
+            if (pass == 0) n_zero = slab.off;
             slab.take(&c->d_edp, n_tab);
             slab.take(&c->d_pi, (size_t)L * E);
             slab.take(&c->d_inv, (size_t)L * E);
@@ -289,12 +290,9 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
             slab.take(&c->d_sort_keys, (size_t)2 * n_pow2);
             slab.take(&c->d_seed_layout, N);
             slab.take(&c->d_order, N);
-            slab.take(&c->d_pack_out, 4);
             slab.take(&c->d_inc_layout, N);
             slab.take(&c->d_inc_score, 3);
             slab.take(&c->d_seed_score, 3);
-            slab.take(&c->d_best_score, 3);
-            slab.take(&c->d_best_f64, 3);
             if (pass == 0) { st = dev_alloc(c, &c->d_load_slab, slab.off); slab.base = c->d_load_slab; }
         }
         if (st != RP_OK) break;
@@ -302,18 +300,17 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
         c->d_dp_off = c->d_dp_list + D;
         // input checks + aggregate expert load + token total in one pass over the demand tensor,
         // put in flight before the rest of the set-up
-        if (cudaMemsetAsync(c->d_counters, 0, sizeof(i64) * 8, c->stream) != cudaSuccess) { st = RP_ERR_CUDA; break; }
-        if ((st = reset_status(c)) != RP_OK) break;
+        if (cudaMemsetAsync(c->d_load_slab, 0, n_zero, c->stream) != cudaSuccess) { st = RP_ERR_CUDA; break; }
         stage_mark(c, RP_EV_K1_0, c->stream);
         if ((st = rp_launch_check_reduce(c)) != RP_OK) break;
         stage_mark(c, RP_EV_K1_1, c->stream);
-        // the EDP tables: one copy (pageable source: staged before the call returns)
-        int *tab = (int *)malloc(sizeof(int) * n_tab);
+        // the EDP tables: one copy out of the pinned block (its mail area is idle until the placement is written)
+        int *tab = n_tab * sizeof(int) <= RP_MAIL_BYTES / 2 ? (int *)(rp_mail(c) + RP_MAIL_BYTES / 2) : (int *)malloc(sizeof(int) * n_tab);
         memcpy(tab, edp, sizeof(int) * D);
         memcpy(tab + D, list, sizeof(int) * D);
         memcpy(tab + 2 * D, off, sizeof(int) * (G + 1));
         const cudaError_t e = cudaMemcpyAsync(c->d_edp, tab, sizeof(int) * n_tab, cudaMemcpyHostToDevice, c->stream);
-        free(tab);
+        if (n_tab * sizeof(int) > RP_MAIL_BYTES / 2) free(tab);            // pageable source: staged before the call returns
         if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; st = RP_ERR_CUDA; break; }
     } while (0);
     free(edp); free(off); free(list);
@@ -341,14 +338,11 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
     stage_mark(c, RP_EV_K3_1, c->stream);
     if (forked) RP_CUDA(cudaStreamWaitEvent(c->stream, side->join, 0));
     else c->eager_pack = (rp_launch_pack(c, 0) == RP_OK);
-    if (c->eager_pack)
-        RP_CUDA(cudaMemcpyAsync(c->h_pin + 10, c->d_pack_out, sizeof(int) * 4, cudaMemcpyDeviceToHost, c->stream));
 
-    // verdict of the checks and the token total ride back in the pinned block
-    RP_CUDA(cudaMemcpyAsync(c->h_pin + 8, c->d_counters + 7, sizeof(i64), cudaMemcpyDeviceToHost, c->stream));
-    int sw[RP_SW_COUNT];
-    RP_TRY(read_status(c, sw));
-    if (sw[RP_SW_BAD_SAMPLE]) return RP_ERR_CONSERVATION;
+    // the kernels have left the verdict of the checks, the token total and the packing result in the pinned block
+    RP_CUDA(cudaStreamSynchronize(c->stream));
+    if (!c->eager_place) return RP_ERR_CUDA;              // nothing reported
+    if (((const int *)(c->h_pin + 56))[RP_SW_BAD_SAMPLE]) return RP_ERR_CONSERVATION;
     memcpy(c->pack_out, c->h_pin + 10, sizeof(int) * 4);
 
     // fixed-point range of the score: s1 <= (2^8*C*L*k + (asum+bsum)*C) * sum t  must stay below 2^62
@@ -404,11 +398,18 @@ extern "C" int rp_place_experts(rp_ctx *c, int32_t *pi, int64_t *rank_load)
         RP_TRY(rp_launch_lpt(c));
         RP_TRY(rp_launch_project(c));
     }
+    const bool waited = c->eager_place;       // rp_window_load has waited for the kernels
     c->eager_place = 0;               // a repeated call recomputes
-    RP_TRY(copy_out(c, pi, c->d_pi, sizeof(int) * (size_t)dm.L * dm.E));
-    RP_TRY(copy_out(c, rank_load, c->d_rank_load, sizeof(i64) * (size_t)dm.L * dm.P));
-    // Outputs are complete when the call returns (nothing to wait for when none was asked for).
-    if (pi || rank_load) RP_CUDA(cudaStreamSynchronize(c->stream));
+    // Outputs are complete when the call returns (nothing to wait for when none was asked for): the placement is in the
+    // pinned block, or copied when it is wanted on the device or does not fit there.
+    const size_t np = sizeof(int) * (size_t)dm.L * dm.E, nl = sizeof(i64) * (size_t)dm.L * dm.P;
+    const bool mail = rp_mail_pi(c) != nullptr;
+    const bool pi_host = pi && mail && !rp_is_device_ptr(pi), load_host = rank_load && mail && !rp_is_device_ptr(rank_load);
+    if (pi && !pi_host) RP_TRY(copy_out(c, pi, c->d_pi, np));
+    if (rank_load && !load_host) RP_TRY(copy_out(c, rank_load, c->d_rank_load, nl));
+    if ((pi && !pi_host) || (rank_load && !load_host) || ((pi || rank_load) && !waited)) RP_CUDA(cudaStreamSynchronize(c->stream));
+    if (pi_host) memcpy(pi, rp_mail_pi(c), np);
+    if (load_host) memcpy(rank_load, rp_mail_rank_load(c), nl);
     if (c->stage < 2) c->stage = 2;
     return RP_OK;
 }
@@ -417,18 +418,24 @@ static int ensure_eval_scratch(rp_ctx *c, size_t n, bool want_W)
 {
     const RpDims &dm = c->dm;
     if (n > c->eval_cap) {
-        dev_free(c, c->d_eval_score); dev_free(c, c->d_eval_f64); dev_free(c, c->d_eval_cells);
-        dev_free(c, c->d_eval_Esum); dev_free(c, c->d_eval_tickets);
-        c->d_eval_score = nullptr; c->d_eval_f64 = nullptr; c->d_eval_cells = nullptr;
-        c->d_eval_Esum = nullptr; c->d_eval_tickets = nullptr;
+        dev_free(c, c->d_eval_slab);
+        c->d_eval_slab = nullptr;
         c->eval_cap = 0;
-        RP_TRY(dev_alloc(c, &c->d_eval_score, n * 3));
-        RP_TRY(dev_alloc(c, &c->d_eval_f64, n * 3));
-        RP_TRY(dev_alloc(c, &c->d_eval_cells, n * dm.N));
-        RP_TRY(dev_alloc(c, &c->d_eval_Esum, n * dm.RG));
-        RP_TRY(dev_alloc(c, &c->d_eval_tickets, n));
-        RP_CUDA(cudaMemsetAsync(c->d_eval_tickets, 0, sizeof(int) * n, c->stream));
-        RP_CUDA(cudaMemsetAsync(c->d_eval_Esum, 0, sizeof(i64) * n * dm.RG, c->stream));
+        RpSlab slab = { nullptr, 0 };
+        size_t n_zero = 0;
+        for (int pass = 0; pass < 2; ++pass) {
+            slab.off = 0;
+            slab.take(&c->d_eval_Esum, n * dm.RG);            // (these two start at zero)
+            slab.take(&c->d_eval_tickets, n);
+            if (pass == 0) n_zero = slab.off;
+            slab.take(&c->d_eval_score, n * 3);
+            slab.take(&c->d_eval_f64, n * 3);
+            // (fewer layouts than this may take the other form: its lists are the longest at the largest such n)
+            slab.take(&c->d_eval_list, n * dm.N);
+            slab.take(&c->d_eval_off, n * (dm.RG + 1));
+            if (pass == 0) { RP_TRY(dev_alloc(c, &c->d_eval_slab, slab.off)); slab.base = c->d_eval_slab; }
+        }
+        RP_CUDA(cudaMemsetAsync(c->d_eval_slab, 0, n_zero, c->stream));
         c->eval_cap = n;
     }
     if (want_W && (int)n > c->eval_W_n) {
@@ -444,20 +451,6 @@ __global__ void k_iota(int *out, int n, int first)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x < n) out[x] = first + x;
-}
-
-// Population bookkeeping of a fresh seed in one launch: every member descends from slot 0, whose
-// rank loads sit in cell 0 and are copied into a cell of the member's own (P + m) at level 0; the
-// seed is the incumbent.
-__global__ void k_init_population(int P, int N, int *__restrict__ anc, int *__restrict__ wloc, int *__restrict__ wloc_next,
-                                  int *__restrict__ done, const int *__restrict__ seed_layout, int *__restrict__ inc_layout,
-                                  const i64 *__restrict__ inc_score, i64 *__restrict__ seed_score)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x < P) { anc[x] = 0; wloc[x] = 0; wloc_next[x] = P + x; }
-    if (x < N) inc_layout[x] = seed_layout[x];
-    if (x < 3) seed_score[x] = inc_score[x];
-    if (x == 0) *done = 0;
 }
 
 static int build_population(rp_ctx *c);
@@ -486,7 +479,6 @@ extern "C" int rp_pack_rows(rp_ctx *c, int32_t *n_rows, int32_t *certified)
     int *po = c->pack_out;
     if (!c->eager_pack) {
         RP_TRY(rp_launch_pack(c, 0));
-        RP_CUDA(cudaMemcpyAsync(c->h_pin + 10, c->d_pack_out, sizeof(int) * 4, cudaMemcpyDeviceToHost, c->stream));
         RP_CUDA(cudaStreamSynchronize(c->stream));
         memcpy(c->pack_out, c->h_pin + 10, sizeof(int) * 4);
     }
@@ -539,11 +531,16 @@ static int build_population(rp_ctx *c)
                 slab.take(&c->d_wfree_head, 2);
             }
             slab.take(&c->d_inc_slot, 1);
+            slab.take(&c->d_undecided, 1);
+            slab.take(&c->d_static, (size_t)c->sl.bytes);
+            slab.take(&c->d_one_Esum, (size_t)dm.RG);
+            slab.take(&c->d_one_ticket, 1);
+            slab.take(&c->d_one_list, rp_eval_list_len(dm, 1));
+            slab.take(&c->d_one_off, rp_eval_off_len(dm, 1));
             if (rp_uses_wpc(c->dm) || c->row_mode == 1) slab.take(&c->d_cand_layout, P * (size_t)c->dm.N);
             if (c->row_mode) {
                 slab.take(&c->d_tf, 2 * (size_t)dm.N);
                 slab.take(&c->d_rowF, 2 * P * (size_t)dm.RG);
-                slab.take(&c->d_undecided, 1);
                 if (rp_row_separate(c)) {
                     slab.take(&c->d_qr, (size_t)dm.N * rp_row_ints(c));
                     slab.take(&c->d_Wr, 2 * P * (size_t)dm.RG * rp_row_ints(c));
@@ -563,39 +560,23 @@ static int build_population(rp_ctx *c)
         }
     }
     c->cur = 0;
-    if (c->d_wcount) RP_CUDA(cudaMemsetAsync(c->d_wcount, 0, sizeof(int) * 2 * P * (size_t)dm.RG, c->stream));
     // every member starts as the length-only seed: evaluate it once into slot 0 and let all
     // slots descend from slot 0
-    dev_free(c, c->d_static); c->d_static = nullptr;
-    RP_TRY(dev_alloc(c, &c->d_static, (size_t)c->sl.bytes));
     stage_mark(c, RP_EV_SEED_0, c->stream);
-    RP_TRY(rp_launch_build_static(c));
-    RP_TRY(ensure_eval_scratch(c, 1, false));
-    RP_TRY(rp_launch_cells_from_layouts(c, c->d_seed_layout, 1, c->d_eval_cells));
-    RP_TRY(rp_launch_eval(c, c->d_eval_cells, 1, c->d_W, c->buf[0].blob, c->d_inc_score, nullptr));
-    {
-        const size_t n = P > (size_t)dm.N ? P : (size_t)dm.N;
-        k_init_population<<<(int)((n + 255) / 256), 256, 0, c->stream>>>((int)P, dm.N, c->d_anc, c->d_wloc, c->d_wloc_next, c->d_done,
-                                                                          c->d_seed_layout, c->d_inc_layout, c->d_inc_score,
-                                                                          c->d_seed_score);
-        ++g_rp_launches;
-        RP_CUDA(cudaGetLastError());
-    }
+    RP_TRY(rp_launch_setup_population(c));
+    c->log_clean = 1;
+    RP_TRY(rp_launch_eval_seed(c));
     c->rows_made = 0;
     forget_rows(c, 1);
     stage_mark(c, RP_EV_SEED_1, c->stream);
     return RP_OK;
 }
 
-__global__ void k_gather_cells(const char *__restrict__ blobs, RpBlob bl, const int *__restrict__ anc, int N,
-                               unsigned short *__restrict__ dst16, int *__restrict__ dst32)
+__global__ void k_gather_cells(const char *__restrict__ blobs, RpBlob bl, const int *__restrict__ anc, int N, int *__restrict__ dst)
 {
     const int j = blockIdx.x;
     const unsigned short *s = (const unsigned short *)(blobs + (size_t)anc[j] * bl.bytes + bl.off_cell);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        if (dst16) dst16[(size_t)j * N + i] = s[i];
-        if (dst32) dst32[(size_t)j * N + i] = s[i];
-    }
+    for (int i = threadIdx.x; i < N; i += blockDim.x) dst[(size_t)j * N + i] = s[i];
 }
 
 extern "C" int rp_eval_population(rp_ctx *c, const int32_t *layouts, int32_t n, int64_t *score_fx, double *score_f64)
@@ -607,32 +588,33 @@ extern "C" int rp_eval_population(rp_ctx *c, const int32_t *layouts, int32_t n, 
     if (n < 1) return RP_ERR_ARG;
     const bool keepW = layouts && n <= 64;
     RP_TRY(ensure_eval_scratch(c, (size_t)n, keepW));
-    if (layouts) {
-        const int *dl = layouts;
-        int *tmp = nullptr;
-        if (!is_device_ptr(layouts)) {
-            RP_TRY(dev_alloc(c, &tmp, (size_t)n * dm.N));
-            cudaError_t e = cudaMemcpyAsync(tmp, layouts, sizeof(int) * (size_t)n * dm.N, cudaMemcpyHostToDevice, c->stream);
-            if (e != cudaSuccess) { dev_free(c, tmp); g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
-            dl = tmp;
-        }
-        RP_TRY(reset_status(c));
-        int st = rp_launch_cells_from_layouts(c, dl, n, c->d_eval_cells);
-        int sw[RP_SW_COUNT];
-        if (st == RP_OK) st = read_status(c, sw);
-        dev_free(c, tmp);
-        RP_TRY(st);
-        if (sw[RP_SW_BAD_LAYOUT]) return RP_ERR_ARG;
-    } else {
-        k_gather_cells<<<n, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, c->d_eval_cells, nullptr);
-        ++g_rp_launches;
-    RP_CUDA(cudaGetLastError());
+    const int *dl = layouts;
+    int *tmp = nullptr;
+    if (layouts && !rp_is_device_ptr(layouts)) {
+        RP_TRY(dev_alloc(c, &tmp, (size_t)n * dm.N));
+        cudaError_t e = cudaMemcpyAsync(tmp, layouts, sizeof(int) * (size_t)n * dm.N, cudaMemcpyHostToDevice, c->stream);
+        if (e != cudaSuccess) { dev_free(c, tmp); g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+        dl = tmp;
     }
-    RP_TRY(rp_launch_eval(c, c->d_eval_cells, n, keepW ? c->d_eval_W : nullptr, nullptr, c->d_eval_score,
-                          c->d_eval_f64));
-    RP_TRY(copy_out(c, score_fx, c->d_eval_score, sizeof(i64) * 3 * (size_t)n));
-    RP_TRY(copy_out(c, score_f64, c->d_eval_f64, sizeof(double) * 3 * (size_t)n));
+    // Results straight to where they are wanted: device outputs, or the second half of the pinned mail area.
+    const size_t nf = sizeof(i64) * 3 * (size_t)n;
+    const bool mail = 2 * nf <= RP_MAIL_BYTES / 2;
+    char *half = rp_mail(c) + RP_MAIL_BYTES / 2;
+    const bool fx_dev = score_fx && rp_is_device_ptr(score_fx), f64_dev = score_f64 && rp_is_device_ptr(score_f64);
+    i64 *fx = fx_dev ? (i64 *)score_fx : mail ? (i64 *)half : c->d_eval_score;
+    double *fd = f64_dev ? score_f64 : mail ? (double *)(half + nf) : c->d_eval_f64;
+    int *bad = rp_pin_bad(c);
+    *bad = 0;
+    if (mail) c->best_ready = 0;               // (the incumbent's layout was there)
+    int st = rp_launch_eval(c, dl, layouts ? nullptr : c->d_anc, n, keepW ? c->d_eval_W : nullptr, nullptr, fx, fd);
+    if (st == RP_OK && score_fx && !fx_dev && !mail) st = copy_out(c, score_fx, fx, nf);
+    if (st == RP_OK && score_f64 && !f64_dev && !mail) st = copy_out(c, score_f64, fd, nf);
+    dev_free(c, tmp);
+    RP_TRY(st);
     RP_CUDA(cudaStreamSynchronize(c->stream));
+    if (*bad) return RP_ERR_ARG;
+    if (score_fx && !fx_dev && mail) memcpy(score_fx, fx, nf);
+    if (score_f64 && !f64_dev && mail) memcpy(score_f64, fd, nf);
     return RP_OK;
 }
 
@@ -661,9 +643,8 @@ static int install_population(rp_ctx *c, const int *lay, int n_distinct = 0)
     RP_TRY(dev_alloc(c, &best, 3));
     int st = ensure_eval_scratch(c, ne, false);
     if (st == RP_OK) st = need_rank_loads(c, ne, false);
-    if (st == RP_OK) st = rp_launch_cells_from_layouts(c, lay, (int)ne, c->d_eval_cells);
     c->cur = 0;
-    if (st == RP_OK) st = rp_launch_eval(c, c->d_eval_cells, (int)ne, c->d_W, c->buf[0].blob, c->d_eval_score, nullptr);
+    if (st == RP_OK) st = rp_launch_eval(c, lay, nullptr, (int)ne, c->d_W, c->buf[0].blob, c->d_eval_score, nullptr);
     if (st == RP_OK && ne == P) {
         k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_wloc, (int)P, 0);
         k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_wloc_next, (int)P, 0);
@@ -739,7 +720,7 @@ extern "C" int rp_pair_population(rp_ctx *c, int32_t choice_width, int32_t *n_ch
     if (st == RP_OK && batch > 0) st = dev_alloc(c, &prof, (size_t)batch * dm.K * dm.LP);
     cudaError_t e = cudaSuccess;
     if (st == RP_OK) {
-        k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, nullptr, lay);
+        k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, lay);
         ++g_rp_launches;
         e = cudaMemcpyAsync(out, lay, sizeof(int) * dm.N, cudaMemcpyDeviceToDevice, c->stream);     // member 0 stays
         if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(int), c->stream);
@@ -781,13 +762,12 @@ extern "C" int rp_select_population(rp_ctx *c, int32_t n_proj, int64_t eta_q16, 
     if (st == RP_OK) st = dev_alloc(c, &d_nd, 1);
     if (st == RP_OK) st = dev_alloc(c, &c->d_sel_dist, P * P);
     if (st == RP_OK) {
-        k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, nullptr, lay);
+        k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, lay);
         ++g_rp_launches;
         // exact scores of the members as they stand
         st = ensure_eval_scratch(c, P, false);
     }
-    if (st == RP_OK) st = rp_launch_cells_from_layouts(c, lay, (int)P, c->d_eval_cells);
-    if (st == RP_OK) st = rp_launch_eval(c, c->d_eval_cells, (int)P, nullptr, nullptr, c->d_eval_score, nullptr);
+    if (st == RP_OK) st = rp_launch_eval(c, lay, nullptr, (int)P, nullptr, nullptr, c->d_eval_score, nullptr);
     if (st == RP_OK) st = rp_launch_select(c, lay, out, c->d_eval_score, n_proj, eta_q16, d_order, d_nd, c->d_sel_dist);
     if (st == RP_OK) st = install_population(c, out);
     int *h = (int *)malloc(sizeof(int) * (P + 1));
@@ -869,8 +849,7 @@ extern "C" int rp_init_population(rp_ctx *c, int32_t n_candidates, int32_t choic
         if (st != RP_OK) break;
         // x_paired: the pairing of the seed only if it scores lower
         if ((st = ensure_eval_scratch(c, (size_t)M, false)) != RP_OK) break;
-        if ((st = rp_launch_cells_from_layouts(c, out + dm.N, 1, c->d_eval_cells)) != RP_OK) break;
-        if ((st = rp_launch_eval(c, c->d_eval_cells, 1, nullptr, nullptr, c->d_eval_score, nullptr)) != RP_OK) break;
+        if ((st = rp_launch_eval(c, out + dm.N, nullptr, 1, nullptr, nullptr, c->d_eval_score, nullptr)) != RP_OK) break;
         k_keep_better_of_seed<<<1, 256, 0, c->stream>>>(c->d_seed_layout, c->d_seed_score, out + dm.N, c->d_eval_score, dm.N);
         ++g_rp_launches;
         // all candidates scored and installed, then the selection over them
@@ -946,13 +925,12 @@ static int rebuild_rank_loads(rp_ctx *c)
 {
     const size_t P = (size_t)c->Ppop;
     RP_TRY(ensure_eval_scratch(c, P, false));
-    k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, c->dm.N, c->d_eval_cells, nullptr);
-    RP_TRY(rp_launch_eval(c, c->d_eval_cells, (int)P, c->d_W, c->buf[1 - c->cur].blob, c->d_eval_score, nullptr));
+    RP_TRY(rp_launch_eval(c, nullptr, c->d_anc, (int)P, c->d_W, c->buf[1 - c->cur].blob, c->d_eval_score, nullptr));
     c->cur = 1 - c->cur;
     k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_wloc, (int)P, 0);
     k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_wloc_next, (int)P, 0);
     k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_anc, (int)P, 0);
-    g_rp_launches += 4;
+    g_rp_launches += 3;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
 }
@@ -972,8 +950,8 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     make_schedule(p, c->h_levels);
     const u64 rho_q32 = (u64)floor(p->p_reloc * 4294967296.0);
     const u64 guide_q32 = (u64)floor(p->p_guide * 4294967296.0);
-    // accepted-move log
-    if (c->log_cap < p->steps_per_level) {
+    // accepted-move log (not kept by the launch that runs all levels with one layer per lane)
+    if (c->log_cap < p->steps_per_level && !(rp_may_use_row(c) && c->row_mode == 1)) {
         dev_free(c, c->d_log); c->d_log = nullptr; c->log_cap = 0;
         RP_TRY(dev_alloc(c, &c->d_log, P * (size_t)p->steps_per_level));
         c->log_cap = p->steps_per_level;
@@ -989,13 +967,18 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
         RP_TRY(dev_alloc(c, &c->d_tr_anc, (size_t)(NL > 1 ? NL - 1 : 1) * P));
         c->trace_levels = NL;
     }
-    // counters and status words to zero, incumbent slot to -1 (the incumbent is in d_inc_layout)
-    k_reset_anneal<<<1, 256, 0, c->stream>>>(c->d_counters, c->d_status, c->d_inc_slot, c->d_done, c->d_sync, c->Ppop + 1);
-    ++g_rp_launches;
-    RP_CUDA(cudaGetLastError());
+    // counters and status words to zero, incumbent slot to -1 (the incumbent is in d_inc_layout): done by the
+    // set-up of a fresh population
+    if (!c->log_clean) {
+        k_reset_anneal<<<1, 256, 0, c->stream>>>(c->d_counters, c->d_status, c->d_inc_slot, c->d_done, c->d_sync, c->Ppop + 1);
+        ++g_rp_launches;
+        RP_CUDA(cudaGetLastError());
+    }
+    c->log_clean = 0;
 
-    cudaEvent_t ev[2] = { nullptr, nullptr };
-    if (stats) for (int x = 0; x < 2; ++x) RP_CUDA(cudaEventCreate(&ev[x]));
+    RpSide *side = (RpSide *)c->side;
+    cudaEvent_t ev[2] = { side ? side->t0 : nullptr, side ? side->t1 : nullptr };
+    if (stats && !side) for (int x = 0; x < 2; ++x) RP_CUDA(cudaEventCreate(&ev[x]));
     float ms_chains = 0.f;
     int st = RP_OK;
     // One launch for all levels where every chain can be resident at once, else one launch per level.
@@ -1033,15 +1016,13 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     // rp_best finds them done
     c->best_ready = 0;
     if (st == RP_OK) st = launch_best_check(c);
-    // one synchronisation: the counters and the status words ride back in the pinned block
-    i64 *cn = c->h_pin;                       // [8] counters
-    int *sw = (int *)(c->h_pin + 56);         // status words
-    cudaError_t e = cudaMemcpyAsync(cn, c->d_counters, sizeof(i64) * 8, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sw, c->d_status, sizeof(int) * RP_SW_COUNT, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    // one synchronisation: the incumbent's check has left the counters and the status words in the pinned block
+    const i64 *cn = c->h_pin;                       // [8] counters
+    const int *sw = (const int *)(c->h_pin + 56);   // status words
+    cudaError_t e = cudaStreamSynchronize(c->stream);
     if (stats) {
         if (e == cudaSuccess) cudaEventElapsedTime(&ms_chains, ev[0], ev[1]);
-        for (int x = 0; x < 2; ++x) cudaEventDestroy(ev[x]);
+        if (!side) for (int x = 0; x < 2; ++x) cudaEventDestroy(ev[x]);
     }
     if (st == RP_OK && e != cudaSuccess) { g_rp_last_cuda_error = (int)e; st = RP_ERR_CUDA; }
     RP_TRY(st);
@@ -1067,18 +1048,13 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
 }
 
 // Validate(x*) on the device: coverage / capacity / non-empty cells, and a full rescoring of the
-// incumbent; the three score tuples the verdict needs are queued into the pinned block.
+// incumbent, in one launch that leaves its results in the pinned block.
 static int launch_best_check(rp_ctx *c)
 {
     stage_mark(c, RP_EV_BEST_0, c->stream);
-    RP_TRY(rp_launch_validate(c));
-    RP_TRY(ensure_eval_scratch(c, 1, false));
-    RP_TRY(rp_launch_cells_from_layouts(c, c->d_inc_layout, 1, c->d_eval_cells));
-    RP_TRY(rp_launch_eval(c, c->d_eval_cells, 1, nullptr, nullptr, c->d_best_score, c->d_best_f64));
+    *rp_pin_bad(c) = 0;
+    RP_TRY(rp_launch_eval_incumbent(c));
     stage_mark(c, RP_EV_BEST_1, c->stream);
-    RP_CUDA(cudaMemcpyAsync(c->h_pin + 16, c->d_inc_score, sizeof(i64) * 3, cudaMemcpyDeviceToHost, c->stream));
-    RP_CUDA(cudaMemcpyAsync(c->h_pin + 19, c->d_best_score, sizeof(i64) * 3, cudaMemcpyDeviceToHost, c->stream));
-    RP_CUDA(cudaMemcpyAsync(c->h_pin + 22, c->d_seed_score, sizeof(i64) * 3, cudaMemcpyDeviceToHost, c->stream));
     return RP_OK;
 }
 
@@ -1086,7 +1062,7 @@ static int launch_best_check(rp_ctx *c)
 static int best_verdict(const rp_ctx *c, const int *sw)
 {
     const i64 *inc = c->h_pin + 16, *full = c->h_pin + 19, *seed = c->h_pin + 22;
-    bool ok = !sw[RP_SW_VALIDATE] && !sw[RP_SW_BAD_LAYOUT];
+    bool ok = !sw[RP_SW_VALIDATE] && !*(const int *)(c->h_pin + 30);
     ok = ok && inc[0] == full[0] && inc[1] == full[1] && inc[2] == full[2];
     // non-regression: not worse than the best member of the initial population
     const bool worse = (seed[0] != inc[0]) ? (seed[0] < inc[0]) : (seed[1] != inc[1]) ? (seed[1] < inc[1]) : (seed[2] < inc[2]);
@@ -1099,18 +1075,24 @@ extern "C" int rp_best(rp_ctx *c, int32_t *cell_of_sample, int64_t *score_fx, do
     if (!c) return RP_ERR_ARG;
     if (c->stage < 3) return RP_ERR_STATE;
     const RpDims &dm = c->dm;
-    int *sw = (int *)(c->h_pin + 56);
+    const int *sw = (const int *)(c->h_pin + 56);
     const bool fresh = !c->best_ready;          // rp_anneal validates its incumbent before it returns
     if (fresh) {
         RP_TRY(reset_status(c));
         RP_TRY(launch_best_check(c));
-        RP_CUDA(cudaMemcpyAsync(sw, c->d_status, sizeof(int) * RP_SW_COUNT, cudaMemcpyDeviceToHost, c->stream));
     }
-    RP_TRY(copy_out(c, cell_of_sample, c->d_inc_layout, sizeof(int) * (size_t)dm.N));
-    RP_TRY(copy_out(c, score_fx, c->d_inc_score, sizeof(i64) * 3));
-    RP_TRY(copy_out(c, score_f64, c->d_best_f64, sizeof(double) * 3));
-    // Outputs are complete when the call returns.
-    if (fresh || cell_of_sample || score_fx || score_f64) RP_CUDA(cudaStreamSynchronize(c->stream));
+    // Outputs are complete when the call returns: the results are in the pinned block (the layout too when it fits).
+    const int *lay = rp_mail_layout(c);
+    const bool lay_host = cell_of_sample && lay && !rp_is_device_ptr(cell_of_sample);
+    const bool fx_host = score_fx && !rp_is_device_ptr(score_fx), f64_host = score_f64 && !rp_is_device_ptr(score_f64);
+    if (cell_of_sample && !lay_host) RP_TRY(copy_out(c, cell_of_sample, c->d_inc_layout, sizeof(int) * (size_t)dm.N));
+    if (fresh) RP_CUDA(cudaStreamSynchronize(c->stream));
+    if (score_fx && !fx_host) RP_TRY(copy_out(c, score_fx, c->h_pin + 16, sizeof(i64) * 3));
+    if (score_f64 && !f64_host) RP_TRY(copy_out(c, score_f64, c->h_pin + 25, sizeof(double) * 3));
+    if ((cell_of_sample && !lay_host) || (score_fx && !fx_host) || (score_f64 && !f64_host)) RP_CUDA(cudaStreamSynchronize(c->stream));
+    if (lay_host) memcpy(cell_of_sample, lay, sizeof(int) * (size_t)dm.N);
+    if (fx_host) memcpy(score_fx, c->h_pin + 16, sizeof(i64) * 3);
+    if (f64_host) memcpy(score_f64, c->h_pin + 25, sizeof(double) * 3);
     if (fresh) { c->best_verdict = best_verdict(c, sw); c->best_ready = 1; }
     return c->best_verdict;
 }
@@ -1216,7 +1198,7 @@ extern "C" int rp_debug_dump(rp_ctx *c, int what, int32_t index, void *buf, int6
         case RP_DUMP_POPULATION: {
             need = sizeof(int) * P * dm.N;
             if ((st = dev_alloc(c, (int **)&tmp, P * dm.N)) != RP_OK) return st;
-            k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, nullptr, (int *)tmp);
+            k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, (int *)tmp);
             ++g_rp_launches;
             src = tmp;
             break;
@@ -1226,9 +1208,7 @@ extern "C" int rp_debug_dump(rp_ctx *c, int what, int32_t index, void *buf, int6
                 need = sizeof(int) * (size_t)dm.RG * dm.LP;
                 if ((st = dev_alloc(c, (int **)&tmp, (size_t)dm.RG * dm.LP)) != RP_OK) return st;
                 if ((st = ensure_eval_scratch(c, 1, false)) == RP_OK) {
-                    k_gather_cells<<<1, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc + index, dm.N, c->d_eval_cells, nullptr);
-                    ++g_rp_launches;
-                    st = rp_launch_eval(c, c->d_eval_cells, 1, (int *)tmp, nullptr, c->d_eval_score, nullptr);
+                    st = rp_launch_eval(c, nullptr, c->d_anc + index, 1, (int *)tmp, nullptr, c->d_eval_score, nullptr);
                 }
                 if (st != RP_OK) { dev_free(c, tmp); return st; }
                 src = tmp;

@@ -121,7 +121,6 @@ struct rp_ctx {
     u64 *d_sort_keys;          // scratch for the length sort
     int *d_seed_layout;        // [N]
     int *d_order;              // [N] samples sorted by (-t, i)
-    int *d_pack_out;           // [4]: R*, certified, R_lb, failure flag
     int Rstar, certified;
     i64 seed_score[3];
     // population
@@ -175,8 +174,6 @@ struct rp_ctx {
     int *d_inc_slot;           // [1]
     i64 *d_sel_dist;           // [P_pop][P_pop] plan distances of the last rp_select_population (inspection hook on)
     i64 *d_inc_score;          // [3]
-    i64 *d_best_score;         // [3] full rescoring of the incumbent (validation)
-    double *d_best_f64;        // [3] the same as the real-valued objective
     void *side;                // side stream + two events borrowed for the call that packs beside the placement (see RpSide)
     int eager_place, eager_pack;   // rp_window_load already queued the placement / packing kernels behind its checks
     int pack_out[4];           // R*, certified, R_lb, failure flag as read back with the load's verdict
@@ -199,15 +196,32 @@ struct rp_ctx {
     double *d_eval_f64;        // [n][3]
     int *d_eval_W;             // W of explicitly evaluated layouts (n <= 64), for inspection
     int eval_W_n;
-    unsigned short *d_eval_cells;
-    i64 *d_eval_Esum;          // [n][RG] row-shard sums handed to the finishing CTA
+    char *d_eval_slab;         // one allocation behind the arrays here
+    unsigned short *d_eval_list;   // [n][N] samples grouped by row-shard
+    int *d_eval_off;           // [n][RG+1]
+    i64 *d_eval_Esum;          // [n][RG] row-shard sums handed to the finishing CTA, zero between launches
     int *d_eval_tickets;       // [n] arrival counters, zero between launches
     size_t eval_cap;
+    i64 *d_one_Esum; int *d_one_ticket, *d_one_off; unsigned short *d_one_list;     // the same for one layout (part of the population's slab)
     RpLevel *h_levels;         // host copy of the per-level schedule integers
     int levels_cap;
-    i64 *h_pin;                // small pinned staging block for device->host scalars (64 x 8 bytes)
+    // Pinned block the kernels write their results to (no copies): 64 x 8 bytes of scalars, then RP_MAIL_BYTES in which
+    // rp_window_load leaves the placement and the incumbent's check its layout.
+    //   [0..7] counters  [8] token total  [10,11] packing result  [16..18] cached, [19..21] full, [22..24] seed score of the
+    //   incumbent  [25..27] its real-valued objective  [30] bad-layout flag  [32..] diagnostics  [56..59] status words  [60] undecided
+    i64 *h_pin;
+    int log_clean;             // counters, status words and arrival counters are as rp_anneal wants them
     i64 *d_seed_score;         // [3] best score of the initial population
 };
+
+#define RP_MAIL_BYTES (256 * 1024)
+static inline int *rp_pin_bad(rp_ctx *c) { return (int *)(c->h_pin + 30); }
+static inline char *rp_mail(rp_ctx *c) { return (char *)(c->h_pin + 64); }
+static inline size_t rp_mail_place(const RpDims &dm) { return ((size_t)4 * dm.L * dm.E + 7) / 8 * 8 + (size_t)8 * dm.L * dm.P; }
+// Where the placement and the incumbent's layout go in the mail area; null when they do not fit.
+static inline int *rp_mail_pi(rp_ctx *c) { return rp_mail_place(c->dm) <= RP_MAIL_BYTES / 2 ? (int *)rp_mail(c) : nullptr; }
+static inline i64 *rp_mail_rank_load(rp_ctx *c) { return rp_mail_pi(c) ? (i64 *)(rp_mail(c) + ((size_t)4 * c->dm.L * c->dm.E + 7) / 8 * 8) : nullptr; }
+static inline int *rp_mail_layout(rp_ctx *c) { return (size_t)4 * c->dm.N <= RP_MAIL_BYTES / 2 ? (int *)(rp_mail(c) + RP_MAIL_BYTES / 2) : nullptr; }
 
 enum RpStatusWord { RP_SW_BAD_SAMPLE = 0, RP_SW_BAD_LAYOUT = 1, RP_SW_VALIDATE = 2, RP_SW_TIMEOUT = 3, RP_SW_POOL = 4, RP_SW_COUNT = 8 };
 
@@ -218,9 +232,13 @@ int rp_launch_check_reduce(rp_ctx *c);
 int rp_launch_lpt(rp_ctx *c);
 int rp_launch_project(rp_ctx *c);
 int rp_launch_pack(rp_ctx *c, int Rlb_hint);
-int rp_launch_eval(rp_ctx *c, const unsigned short *cells, int n, int *W_out, char *blob_out,
-                   i64 *score_out, double *f64_out);
-int rp_launch_build_static(rp_ctx *c);
+int rp_launch_eval(rp_ctx *c, const int *lay, const int *src, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out);
+int rp_launch_eval_seed(rp_ctx *c);
+int rp_launch_eval_incumbent(rp_ctx *c);
+size_t rp_eval_list_len(const RpDims &dm, int n);
+size_t rp_eval_off_len(const RpDims &dm, int n);
+int rp_launch_setup_population(rp_ctx *c);
+bool rp_is_device_ptr(const void *p);
 int rp_launch_seed_trials(rp_ctx *c, int width, int *layouts, int *ok);
 int rp_launch_edp_pair(rp_ctx *c, const int *lay_in, int *lay_out, int *prof, int first, int count, int width);
 int rp_launch_pack_on(rp_ctx *c, cudaStream_t stream);
@@ -231,7 +249,6 @@ bool rp_uses_slices(const RpDims &dm);
 int rp_slice_mode(const RpDims &dm, int knob);
 void rp_decide_layouts(rp_ctx *c);
 int rp_launch_slice_gc(rp_ctx *c);
-int rp_launch_cells_from_layouts(rp_ctx *c, const int *layouts, int n, unsigned short *cells);
 // Stream-ordered device memory from the device's pool (n elements of T; freed on the context's stream).
 template <class T>
 static inline int dev_alloc(rp_ctx *c, T **p, size_t n)
@@ -275,7 +292,6 @@ int rp_launch_member_rows(rp_ctx *c, int n);
 int rp_launch_anneal_level(rp_ctx *c, int level, int n_levels, const rp_anneal_params *prm, u64 rho_q32, u64 guide_q32);
 int rp_launch_anneal_all(rp_ctx *c, int n_levels, const rp_anneal_params *prm, u64 rho_q32, u64 guide_q32, int *done);
 int rp_upload_levels(rp_ctx *c, int n_levels);
-int rp_launch_validate(rp_ctx *c);
 int rp_anneal_smem_bytes(const rp_ctx *c, int *threads, size_t *bytes);
 
 // ---------------------------------------------------------------------------------------

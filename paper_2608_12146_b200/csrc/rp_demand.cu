@@ -225,7 +225,6 @@ static int launch_check_reduce_seq(rp_ctx *c)
 int rp_launch_check_reduce(rp_ctx *c)
 {
     const RpDims &dm = c->dm;
-    RP_CUDA(cudaMemsetAsync(c->d_Lagg, 0, sizeof(i64) * dm.L * dm.E, c->stream));
     // The sequential form where it measured faster (512-byte rows, 32 layers: one atomic per expert,
     // layer and CTA is then the smaller part of the time; on wider or fewer rows the form below wins).
     if (((size_t)c->d_a & 15) == 0 && dm.N >= 2 * 148 && dm.E == 128 && dm.L == 32) return launch_check_reduce_seq<1, 2, 16, 4>(c);
@@ -286,8 +285,9 @@ int rp_launch_check_reduce(rp_ctx *c)
 // many experts precede each one; then one warp assigns them in that order to the rank
 // with the smallest (load, id) among ranks holding fewer than H experts.
 __global__ void __launch_bounds__(1024)
-k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *__restrict__ pi, int *__restrict__ inv,
-      i64 *__restrict__ rank_load, int *__restrict__ top)
+k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
+      i64 *rank_load, int *__restrict__ top, const int *__restrict__ status, const i64 *__restrict__ t_sum,
+      i64 *__restrict__ h_pin, int *__restrict__ h_pi, i64 *__restrict__ h_load)
 {
     extern __shared__ unsigned char smraw[];
     i64 *load = (i64 *)smraw;                 // [E]
@@ -386,6 +386,14 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *__restrict__ pi, int *__rest
         }
         for (int p = lane; p < dm.P; p += 32) rank_load[(size_t)l * dm.P + p] = G[p];
     }
+    // what the host is waiting for, straight into its memory: the verdict of the checks, the token total, the placement
+    if (l == 0 && threadIdx.x < RP_SW_COUNT) ((int *)(h_pin + 56))[threadIdx.x] = status[threadIdx.x];
+    if (l == 0 && threadIdx.x == 0) h_pin[8] = *t_sum;
+    if (h_pi) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < dm.E; e += blockDim.x) h_pi[(size_t)l * dm.E + e] = pi[(size_t)l * dm.E + e];
+        for (int p = threadIdx.x; p < dm.P; p += blockDim.x) h_load[(size_t)l * dm.P + p] = rank_load[(size_t)l * dm.P + p];
+    }
 }
 
 int rp_launch_lpt(rp_ctx *c)
@@ -393,7 +401,8 @@ int rp_launch_lpt(rp_ctx *c)
     const RpDims &dm = c->dm;
     size_t smem = sizeof(i64) * (dm.E + dm.P) + sizeof(int) * (dm.E + dm.P);
     int threads = dm.E < 32 ? 32 : (dm.E > 1024 ? 1024 : ((dm.E + 31) / 32) * 32);
-    k_lpt<<<dm.L, threads, smem, c->stream>>>(c->d_Lagg, dm, c->d_pi, c->d_inv, c->d_rank_load, c->d_top);
+    k_lpt<<<dm.L, threads, smem, c->stream>>>(c->d_Lagg, dm, c->d_pi, c->d_inv, c->d_rank_load, c->d_top, c->d_status,
+                                                c->d_counters + 7, c->h_pin, rp_mail_pi(c), rp_mail_rank_load(c));
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;

@@ -6,8 +6,8 @@
 //  * few layouts (k_eval_few: the seed, the incumbent, diagnostics, small batches), bound by latency: a cluster of
 //    CTAs per row-shard, each over its share of the samples, sixteen 16-byte loads in flight per lane; the CTAs'
 //    sums meet through distributed shared memory;
-//  * many layouts (k_eval), bound by L2: a CTA per layout and range of row-shards groups the samples by row-shard
-//    once and a warp sums the rows of a row-shard.
+//  * many layouts (k_eval_group, k_eval_sum), bound by L2: the samples of a layout are grouped by row-shard once, then
+//    a warp per row-shard sums its rows, sixteen bytes per lane and eight samples in flight.
 // In both the CTA that finishes a layout last (atomic ticket) scores it.
 #include <cooperative_groups.h>
 
@@ -19,39 +19,48 @@ namespace cg = cooperative_groups;
 
 #define EVAL_THREADS 256
 
-__global__ void k_layouts_to_cells(const int *__restrict__ layouts, long long total, int K,
-                                   unsigned short *__restrict__ cells, int *__restrict__ status)
-{
-    long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= total) return;
-    int c = layouts[x];
-    if (c < 0 || c >= K) { atomicExch(&status[RP_SW_BAD_LAYOUT], 1); c = 0; }
-    cells[x] = (unsigned short)c;
-}
-
-int rp_launch_cells_from_layouts(rp_ctx *c, const int *layouts, int n, unsigned short *cells)
-{
-    long long total = (long long)n * c->dm.N;
-    int grid = (int)((total + 255) / 256);
-    k_layouts_to_cells<<<grid, 256, 0, c->stream>>>(layouts, total, c->dm.K, cells, c->d_status);
-    ++g_rp_launches;
-    RP_CUDA(cudaGetLastError());
-    return RP_OK;
-}
-
 // What a launch scores and where its results go.
 struct EvalArgs {
     RpDims dm;
     RpBlob bl;
-    const unsigned short *cells;                  // [n][N]
+    const int *lay32;                             // [n][N] layouts, or (null) the assignments of blobs[src[0..n-1]]
+    const char *blobs;
+    const int *src;
     const int *t, *q, *edp, *dp_list, *dp_off;
     int *W_out;                                   // [n][RG][LP], nullable
     char *blob_out;                               // [n] chain-state blobs (see RpBlob), nullable
-    i64 *score_out;                               // [n][3], nullable
+    i64 *score_out, *score_out2;                  // [n][3], nullable
     double *f64_out;                              // [n][3], nullable
+    int *bad;                                     // raised when a layout names a cell outside [0, K) (host memory; such a sample counts as cell 0)
     i64 *Esum;                                    // [n][RG] row-shard sums handed to the finishing CTA; zero between launches
     int *tickets;                                 // [n] arrival counters; zero between launches
+    unsigned short *list;                         // [n][N] samples grouped by row-shard (k_eval_group)
+    int *off;                                     // [n][RG+1]
+    // Validation of the incumbent: with `host` set (pinned), the finishing CTA leaves the search's counters, the status
+    // words, the incumbent's cached score, its full score, the best seed's and its layout there.
+    i64 *host;
+    const i64 *counters, *inc_score, *seed_score;
+    const int *status;
+    int *layout_host;
 };
+
+// Cell of sample i in layout lay.
+struct EvalCells { const int *a; const unsigned short *b; };
+__device__ __forceinline__ EvalCells eval_cells(const EvalArgs &A, int lay)
+{
+    EvalCells e;
+    e.a = A.lay32 ? A.lay32 + (size_t)lay * A.dm.N : nullptr;
+    e.b = A.lay32 ? nullptr : (const unsigned short *)(A.blobs + (size_t)A.src[lay] * A.bl.bytes + A.bl.off_cell);
+    return e;
+}
+__device__ __forceinline__ int eval_cell(const EvalArgs &A, const EvalCells &e, int i)
+{
+    if (!e.a) return __ldg(e.b + i);
+    const int c = __ldg(e.a + i);
+    if ((unsigned)c < (unsigned)A.dm.K) return c;
+    *A.bad = 1;
+    return 0;
+}
 
 // Shared memory of the finishing CTA.
 struct EvalFinish { u64 *Q; i64 *Esum, *Afx, *U; int *T, *cnt; unsigned short *cell_of; };
@@ -94,6 +103,15 @@ __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const Ev
     }
     __syncthreads();
     char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
+    if (A.host) {          // coverage is checked by the caller's `bad` flag: every sample sits in one cell by construction
+        int wrong = 0;
+        for (int c = tid; c < dm.K; c += EVAL_THREADS) wrong |= (f.cnt[c] < 1 ? 2 : 0) | (f.T[c] > dm.C ? 4 : 0);
+        wrong = __syncthreads_or(wrong);
+        if (tid < 8) A.host[tid] = A.counters[tid];
+        if (tid < 3) { A.host[16 + tid] = A.inc_score[tid]; A.host[22 + tid] = A.seed_score[tid]; }
+        if (tid < RP_SW_COUNT) ((int *)(A.host + 56))[tid] = A.status[tid] | (tid == RP_SW_VALIDATE && wrong ? 1 : 0);
+        if (A.layout_host) for (int i = tid; i < dm.N; i += EVAL_THREADS) A.layout_host[i] = __ldg(A.lay32 + i);
+    }
     if (tid < 32) {
         i64 s0 = 0, s1 = 0, s2 = 0;
         for (int g = lane; g < dm.G; g += 32) { const i64 u = f.U[g]; s1 += u; s0 = u > s0 ? u : s0; }
@@ -107,6 +125,7 @@ __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const Ev
             const i64 sc[3] = { s0, s1, s2 };
             for (int x = 0; x < 3; ++x) {
                 if (A.score_out) A.score_out[(size_t)lay * 3 + x] = sc[x];
+                if (A.score_out2) A.score_out2[(size_t)lay * 3 + x] = sc[x];
                 if (A.f64_out) A.f64_out[(size_t)lay * 3 + x] = (double)sc[x] / (double)dm.SC;
             }
             if (b) { i64 *S = (i64 *)(b + A.bl.off_S); S[0] = s0; S[1] = s1; S[2] = s2; S[3] = rp_energy(s0, s1, s2); }
@@ -129,11 +148,11 @@ __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const Ev
     for (int i = tid; i < dm.N; i += EVAL_THREADS) ((unsigned short *)(b + A.bl.off_cell))[i] = f.cell_of[i];
 }
 
-__device__ __forceinline__ void eval_load_cells(const EvalArgs &A, int lay, unsigned short *cell_of, int tid)
+__device__ __forceinline__ void eval_load_cells(const EvalArgs &A, int lay, unsigned short *cell_of, int tid, int nt)
 {
-    const unsigned short *src = A.cells + (size_t)lay * A.dm.N;
+    const EvalCells e = eval_cells(A, lay);
 #pragma unroll 4
-    for (int i = tid; i < A.dm.N; i += EVAL_THREADS) cell_of[i] = __ldg(src + i);
+    for (int i = tid; i < A.dm.N; i += nt) cell_of[i] = (unsigned short)eval_cell(A, e, i);
 }
 
 // Sum of one 16-byte column of the listed samples' rows, U loads in flight.
@@ -160,26 +179,31 @@ __device__ __forceinline__ int eval_layer_max(int m, int lane, int cpl)      // 
     return m;
 }
 
-// grid = (layouts, splits): the CTAs of a layout share its row-shards (one per warp at a time).
-__global__ void __launch_bounds__(EVAL_THREADS, 5)
-k_eval(const EvalArgs A)
+// Many layouts, first kernel: the samples of each layout grouped by row-shard (one CTA per layout).
+#define GROUP_THREADS 512
+__global__ void __launch_bounds__(GROUP_THREADS)
+k_eval_group(const EvalArgs A)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     const RpDims &dm = A.dm;
-    const EvalFinish f = eval_finish_views(dm, smraw);
-    int *off = (int *)(smraw + eval_finish_bytes(dm));                  // [RG+1]
-    int *cur = off + dm.RG + 1;                                         // [RG]
-    int *members = cur + dm.RG;                                         // [N]
-    __shared__ int last_s, wsum[EVAL_THREADS / 32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = EVAL_THREADS / 32;
-    const int lay = blockIdx.x;
-    eval_load_cells(A, lay, f.cell_of, tid);
-    for (int x = tid; x <= dm.RG; x += EVAL_THREADS) off[x] = 0;
+    int *off = (int *)smraw;                                            // [RG] counts, then fill pointers
+    unsigned short *rg_of = (unsigned short *)(off + dm.RG);            // [K]
+    unsigned short *rgs = rg_of + dm.K;                                 // [N]
+    __shared__ int wsum[GROUP_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lay = blockIdx.x;
+    for (int x = tid; x < dm.RG; x += GROUP_THREADS) off[x] = 0;
+    for (int c = tid; c < dm.K; c += GROUP_THREADS) rg_of[c] = (unsigned short)rp_rowshard(dm, A.edp, c);
     __syncthreads();
-    for (int i = tid; i < dm.N; i += EVAL_THREADS) atomicAdd(&off[rp_rowshard(dm, A.edp, f.cell_of[i])], 1);
+    const EvalCells e = eval_cells(A, lay);
+#pragma unroll 4
+    for (int i = tid; i < dm.N; i += GROUP_THREADS) {
+        const int rg = rg_of[eval_cell(A, e, i)];
+        rgs[i] = (unsigned short)rg;
+        atomicAdd(&off[rg], 1);
+    }
     __syncthreads();
     {   // exclusive prefix sums: a thread takes consecutive row-shards
-        const int chunk = (dm.RG + EVAL_THREADS - 1) / EVAL_THREADS, x0 = min(dm.RG, tid * chunk), x1 = min(dm.RG, x0 + chunk);
+        const int chunk = (dm.RG + GROUP_THREADS - 1) / GROUP_THREADS, x0 = min(dm.RG, tid * chunk), x1 = min(dm.RG, x0 + chunk);
         int sum = 0;
         for (int x = x0; x < x1; ++x) sum += off[x];
         int v = sum;
@@ -188,24 +212,52 @@ k_eval(const EvalArgs A)
         __syncthreads();
         int run = v - sum;
         for (int w = 0; w < warp; ++w) run += wsum[w];
-        for (int x = x0; x < x1; ++x) { const int c = off[x]; off[x] = run; cur[x] = run; run += c; }
-        if (tid == EVAL_THREADS - 1) off[dm.RG] = dm.N;
+        int *go = A.off + (size_t)lay * (dm.RG + 1);
+        for (int x = x0; x < x1; ++x) { const int c = off[x]; off[x] = run; go[x] = run; run += c; }
+        if (tid == 0) go[dm.RG] = dm.N;
     }
     __syncthreads();
-    for (int i = tid; i < dm.N; i += EVAL_THREADS) members[atomicAdd(&cur[rp_rowshard(dm, A.edp, f.cell_of[i])], 1)] = i;
-    __syncthreads();
-    i64 *esum_lay = A.Esum + (size_t)lay * dm.RG;
-    const int cpl = dm.P >> 2, lps = eval_vec(dm) ? 32 / cpl : 1, used = lps * cpl, rc = dm.LP >> 2;
-    for (int rg = blockIdx.y * nwarps + warp; rg < dm.RG; rg += gridDim.y * nwarps) {
-        const int m0 = off[rg], m1 = off[rg + 1];
+    unsigned short *list = A.list + (size_t)lay * dm.N;
+    for (int i = tid; i < dm.N; i += GROUP_THREADS) list[atomicAdd(&off[rgs[i]], 1)] = (unsigned short)i;
+}
+
+// Many layouts, second kernel: grid (row-shards / 8, layouts), a warp per row-shard.
+__global__ void __launch_bounds__(EVAL_THREADS, 5)
+k_eval_sum(const EvalArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const RpDims &dm = A.dm;
+    __shared__ int last_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lay = blockIdx.y;
+    const int rg = blockIdx.x * (EVAL_THREADS / 32) + warp;
+    if (rg < dm.RG) {
+        const int *go = A.off + (size_t)lay * (dm.RG + 1);
+        const unsigned short *list = A.list + (size_t)lay * dm.N;
+        const int m0 = __ldg(go + rg), m1 = __ldg(go + rg + 1), rc = dm.LP >> 2;
         int *wout = A.W_out ? A.W_out + ((size_t)lay * dm.RG + rg) * dm.LP : nullptr;
         i64 es;
         if (eval_vec(dm)) {
+            const int cpl = dm.P >> 2, used = (32 / cpl) * cpl;
             es = 0;
             for (int c0 = 0; c0 < rc; c0 += used) {
                 const int c = c0 + lane;
                 const bool on = lane < used && c < rc;
-                const int4 a = eval_sum_column<8>((const int4 *)A.q + (on ? c : 0), rc, members, m0, m1);
+                const int4 *col = (const int4 *)A.q + (on ? c : 0);
+                int4 a = make_int4(0, 0, 0, 0);
+                for (int mb = m0; mb < m1; mb += 32) {
+                    // the next 32 samples of the list, one per lane, handed round by shuffles; eight rows in flight
+                    const int id = mb + lane < m1 ? (int)__ldg(list + mb + lane) : 0, nm = min(32, m1 - mb);
+                    for (int x0 = 0; x0 < nm; x0 += 8) {
+                        int4 v[8];
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) {
+                            const int s = __shfl_sync(0xffffffffu, id, x0 + x);
+                            v[x] = x0 + x < nm ? __ldg(col + (size_t)s * rc) : make_int4(0, 0, 0, 0);
+                        }
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) { a.x += v[x].x; a.y += v[x].y; a.z += v[x].z; a.w += v[x].w; }
+                    }
+                }
                 if (wout && on) ((int4 *)wout)[c] = a;
                 const int m = eval_layer_max(on ? max(max(a.x, a.y), max(a.z, a.w)) : 0, lane, cpl);
                 if (on && lane % cpl == 0) es += m;
@@ -214,22 +266,24 @@ k_eval(const EvalArgs A)
         } else {
             es = rp_warp_layer_max_sum(dm, lane, [&](int x) {
                 int s = 0;
-                for (int m = m0; m < m1; ++m) s += __ldg(A.q + (size_t)members[m] * dm.LP + x);
+                for (int m = m0; m < m1; ++m) s += __ldg(A.q + (size_t)__ldg(list + m) * dm.LP + x);
                 if (wout) wout[x] = s;
                 return s;
             });
         }
-        if (lane == 0) esum_lay[rg] = es;
+        if (lane == 0) A.Esum[(size_t)lay * dm.RG + rg] = es;
     }
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-        last_s = (atomicAdd(&A.tickets[lay], 1) == (int)gridDim.y - 1);
+        last_s = (atomicAdd(&A.tickets[lay], 1) == (int)gridDim.x - 1);
         if (last_s) A.tickets[lay] = 0;                   // ready for the next launch
     }
     __syncthreads();
     if (!last_s) return;
     __threadfence();
+    const EvalFinish f = eval_finish_views(dm, smraw);
+    eval_load_cells(A, lay, f.cell_of, tid, EVAL_THREADS);
     eval_finish(A, lay, f, tid);
 }
 
@@ -247,14 +301,14 @@ k_eval_few(const EvalArgs A)
     int *list = part + dm.LP;                                           // [N / MS + 1] its samples
     __shared__ int n_s, last_s;
     __shared__ u64 es_s;
-    const unsigned short *cells = A.cells + (size_t)lay * dm.N;
+    const EvalCells cells = eval_cells(A, lay);
     if (tid == 0) { n_s = 0; es_s = 0; }
     __syncthreads();
     const int row = rg / dm.G, g = rg % dm.G;
     const int i0 = (int)((long long)dm.N * ms / MS), i1 = (int)((long long)dm.N * (ms + 1) / MS);
 #pragma unroll 8
     for (int i = i0 + tid; i < i1; i += EVAL_THREADS) {
-        const int c = __ldg(cells + i);
+        const int c = eval_cell(A, cells, i);
         if (c / dm.D == row && __ldg(A.edp + c % dm.D) == g) list[atomicAdd(&n_s, 1)] = i;
     }
     __syncthreads();
@@ -295,7 +349,7 @@ k_eval_few(const EvalArgs A)
     if (!last_s) return;
     __threadfence();
     const EvalFinish f = eval_finish_views(dm, smraw);
-    eval_load_cells(A, lay, f.cell_of, tid);
+    eval_load_cells(A, lay, f.cell_of, tid, EVAL_THREADS);
     eval_finish(A, lay, f, tid);
 }
 
@@ -306,19 +360,22 @@ static size_t eval_smem_bytes(const RpDims &dm)
 
 #define EVAL_SMEM_MAX (220 * 1024)
 
-// One launch either way; the scratch (Esum, tickets) is zero before and after it.
-static int eval_launch(rp_ctx *c, const unsigned short *cells, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out,
-                       i64 *Esum, int *tickets)
+// Whether n layouts take the few-layouts form: a cluster per row-shard scans the assignment once per row-shard, the other
+// form groups it once per layout; the first up to about sixteen waves of its CTAs.
+static bool eval_is_few(const RpDims &dm, int n)
+{
+    return eval_vec(dm) && (long long)n * dm.RG <= 16 * 148 * 8 && n < 65536 && dm.RG < 65536 && dm.LP <= 16384;
+}
+size_t rp_eval_list_len(const RpDims &dm, int n) { return eval_is_few(dm, n) ? 0 : (size_t)n * dm.N; }
+size_t rp_eval_off_len(const RpDims &dm, int n) { return eval_is_few(dm, n) ? 0 : (size_t)n * (dm.RG + 1); }
+
+// The scratch (Esum, tickets) is zero before and after a launch.
+static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
 {
     const RpDims &dm = c->dm;
-    const size_t smem = eval_smem_bytes(dm);
-    if (smem > EVAL_SMEM_MAX) return RP_ERR_RANGE;
-    EvalArgs A;
-    A.dm = dm; A.bl = c->bl; A.cells = cells; A.t = c->d_t; A.q = c->d_q; A.edp = c->d_edp; A.dp_list = c->d_dp_list; A.dp_off = c->d_dp_off;
-    A.W_out = W_out; A.blob_out = blob_out; A.score_out = score_out; A.f64_out = f64_out; A.Esum = Esum; A.tickets = tickets;
-    // A cluster per row-shard scans the assignment once per row-shard, a CTA per layout groups it once: the first
-    // form up to about sixteen waves of its CTAs.
-    if (eval_vec(dm) && (long long)n * dm.RG <= 16 * 148 * 8 && n < 65536 && dm.RG < 65536 && dm.LP <= 16384) {
+    if (eval_smem_bytes(dm) > EVAL_SMEM_MAX) return RP_ERR_RANGE;
+    A.dm = dm; A.bl = c->bl; A.t = c->d_t; A.q = c->d_q; A.edp = c->d_edp; A.dp_list = c->d_dp_list; A.dp_off = c->d_dp_off;
+    if (eval_is_few(dm, n)) {
         int MS = 1;
         while (MS < 8 && (long long)n * dm.RG * MS < 148 * 4 && dm.N >= 64 * MS) MS *= 2;
         const size_t sm = std::max(eval_finish_bytes(dm), sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2));
@@ -333,21 +390,64 @@ static int eval_launch(rp_ctx *c, const unsigned short *cells, int n, int *W_out
         cfg.attrs = at; cfg.numAttrs = 1;
         RP_CUDA(cudaLaunchKernelEx(&cfg, k_eval_few, A));
     } else {
-        if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
-        // every SM holds five CTAs: split the layouts' row-shards until they are filled
-        int splits = (5 * 148 + n - 1) / n;
-        const int max_splits = (dm.RG + EVAL_THREADS / 32 - 1) / (EVAL_THREADS / 32);
-        splits = std::max(1, std::min(splits, max_splits));
-        k_eval<<<dim3(n, splits), EVAL_THREADS, smem, c->stream>>>(A);
+        const size_t gm = sizeof(int) * (size_t)dm.RG + 2 * ((size_t)dm.K + dm.N), fm = eval_finish_bytes(dm);
+        if (gm > EVAL_SMEM_MAX || dm.N > 65535) return RP_ERR_RANGE;
+        if (gm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_group, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
+        if (fm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_sum, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
+        const int gx = (dm.RG + EVAL_THREADS / 32 - 1) / (EVAL_THREADS / 32);
+        for (int first = 0; first < n; first += 65535) {                 // (layouts along y)
+            EvalArgs B = A;
+            const int m = std::min(65535, n - first);
+            if (B.lay32) B.lay32 += (size_t)first * dm.N; else B.src += first;
+            if (B.W_out) B.W_out += (size_t)first * dm.RG * dm.LP;
+            if (B.blob_out) B.blob_out += (size_t)first * c->bl.bytes;
+            if (B.score_out) B.score_out += 3 * (size_t)first;
+            if (B.f64_out) B.f64_out += 3 * (size_t)first;
+            B.Esum += (size_t)first * dm.RG; B.tickets += first; B.list += (size_t)first * dm.N; B.off += (size_t)first * (dm.RG + 1);
+            k_eval_group<<<m, GROUP_THREADS, gm, c->stream>>>(B);
+            k_eval_sum<<<dim3(gx, m), EVAL_THREADS, fm, c->stream>>>(B);
+            ++g_rp_launches;
+        }
     }
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
 }
 
-int rp_launch_eval(rp_ctx *c, const unsigned short *cells, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out)
+// n layouts lay [n][N] (null: the assignments of the current buffer's blobs that src names) with the context's scratch.
+int rp_launch_eval(rp_ctx *c, const int *lay, const int *src, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out)
 {
-    return eval_launch(c, cells, n, W_out, blob_out, score_out, f64_out, c->d_eval_Esum, c->d_eval_tickets);
+    EvalArgs A = {};
+    A.lay32 = lay; A.blobs = c->buf[c->cur].blob; A.src = src;
+    A.W_out = W_out; A.blob_out = blob_out; A.score_out = score_out; A.f64_out = f64_out;
+    A.bad = rp_pin_bad(c);
+    A.Esum = c->d_eval_Esum; A.tickets = c->d_eval_tickets; A.list = c->d_eval_list; A.off = c->d_eval_off;
+    return eval_launch(c, A, n);
+}
+
+// One layout with the population's own scratch.
+static void eval_one(rp_ctx *c, EvalArgs &A)
+{
+    A.bad = rp_pin_bad(c);
+    A.Esum = c->d_one_Esum; A.tickets = c->d_one_ticket; A.list = c->d_one_list; A.off = c->d_one_off;
+}
+int rp_launch_eval_seed(rp_ctx *c)
+{
+    EvalArgs A = {};
+    eval_one(c, A);
+    A.lay32 = c->d_seed_layout; A.W_out = c->d_W; A.blob_out = c->buf[0].blob; A.score_out = c->d_inc_score; A.score_out2 = c->d_seed_score;
+    return eval_launch(c, A, 1);
+}
+// Validate(x*) and the full rescoring of the incumbent; the results go to the pinned block (see EvalArgs::host).
+int rp_launch_eval_incumbent(rp_ctx *c)
+{
+    EvalArgs A = {};
+    eval_one(c, A);
+    A.lay32 = c->d_inc_layout;
+    A.score_out = c->h_pin + 19; A.f64_out = (double *)(c->h_pin + 25);
+    A.host = c->h_pin; A.counters = c->d_counters; A.inc_score = c->d_inc_score; A.seed_score = c->d_seed_score; A.status = c->d_status;
+    A.layout_host = rp_mail_layout(c);
+    return eval_launch(c, A, 1);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -379,24 +479,53 @@ void rp_make_layouts(const RpDims &dm, RpBlob *bl, RpStatic *sl)
     sl->bytes = (o + 15) & ~15;
 }
 
-__global__ void k_build_static(const int *__restrict__ t, const int *__restrict__ edp, const int *__restrict__ dp_list,
-                               const int *__restrict__ dp_off, RpDims dm, RpStatic sl, char *__restrict__ blk)
+// A fresh population in one launch: the static tables; every member descends from slot 0, whose rank loads sit in cell 0 and
+// are copied into a cell of the member's own (P + m) at level 0; the seed is the incumbent; counters, scratch and the
+// slices' holder counts at zero.
+struct SetupArgs {
+    RpDims dm;
+    RpStatic sl;
+    const int *t, *edp, *dp_list, *dp_off, *seed_layout;
+    char *blk;
+    int P, *anc, *wloc, *wloc_next, *done, *inc_layout, *one_ticket, *wcount, *undecided, *inc_slot, *sync, *status;
+    i64 *one_Esum, *counters;
+};
+__global__ void __launch_bounds__(256)
+k_setup_population(const SetupArgs A)
 {
+    const RpDims &dm = A.dm;
+    const RpStatic &sl = A.sl;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    for (int d = tid; d < dm.D; d += nt) ((int *)(blk + sl.off_dpl))[d] = dp_list[d];
-    for (int g = tid; g <= dm.G; g += nt) ((int *)(blk + sl.off_dpo))[g] = dp_off[g];
-    if (sl.t_staged) for (int i = tid; i < dm.N; i += nt) ((int *)(blk + sl.off_t))[i] = t[i];
+    for (int d = tid; d < dm.D; d += nt) ((int *)(A.blk + sl.off_dpl))[d] = A.dp_list[d];
+    for (int g = tid; g <= dm.G; g += nt) ((int *)(A.blk + sl.off_dpo))[g] = A.dp_off[g];
+    if (sl.t_staged) for (int i = tid; i < dm.N; i += nt) ((int *)(A.blk + sl.off_t))[i] = A.t[i];
     for (int c = tid; c < dm.K; c += nt) {
-        const int r = c / dm.D, g = edp[c % dm.D];
-        ((unsigned short *)(blk + sl.off_rg))[c] = (unsigned short)(r * dm.G + g);
-        ((unsigned short *)(blk + sl.off_g))[c] = (unsigned short)g;
-        ((unsigned short *)(blk + sl.off_row))[c] = (unsigned short)(r * dm.D);
+        const int r = c / dm.D, g = A.edp[c % dm.D];
+        ((unsigned short *)(A.blk + sl.off_rg))[c] = (unsigned short)(r * dm.G + g);
+        ((unsigned short *)(A.blk + sl.off_g))[c] = (unsigned short)g;
+        ((unsigned short *)(A.blk + sl.off_row))[c] = (unsigned short)(r * dm.D);
     }
+    for (int m = tid; m < A.P; m += nt) { A.anc[m] = 0; A.wloc[m] = 0; A.wloc_next[m] = A.P + m; }
+    for (int i = tid; i < dm.N; i += nt) A.inc_layout[i] = A.seed_layout[i];
+    for (int x = tid; x < dm.RG; x += nt) A.one_Esum[x] = 0;
+    for (int x = tid; x <= A.P; x += nt) A.sync[x] = 0;
+    if (A.wcount) for (size_t x = tid; x < 2 * (size_t)A.P * dm.RG; x += nt) A.wcount[x] = 0;
+    if (tid < 7) A.counters[tid] = 0;                      // (the eighth is the window's token total)
+    if (tid < RP_SW_COUNT) A.status[tid] = 0;
+    if (tid == 0) { *A.done = 0; *A.one_ticket = 0; *A.undecided = 0; *A.inc_slot = -1; }
 }
 
-int rp_launch_build_static(rp_ctx *c)
+int rp_launch_setup_population(rp_ctx *c)
 {
-    k_build_static<<<4, 256, 0, c->stream>>>(c->d_t, c->d_edp, c->d_dp_list, c->d_dp_off, c->dm, c->sl, c->d_static);
+    const RpDims &dm = c->dm;
+    SetupArgs A = {};
+    A.dm = dm; A.sl = c->sl; A.t = c->d_t; A.edp = c->d_edp; A.dp_list = c->d_dp_list; A.dp_off = c->d_dp_off; A.seed_layout = c->d_seed_layout;
+    A.blk = c->d_static; A.P = c->Ppop; A.anc = c->d_anc; A.wloc = c->d_wloc; A.wloc_next = c->d_wloc_next; A.done = c->d_done;
+    A.inc_layout = c->d_inc_layout; A.one_ticket = c->d_one_ticket; A.wcount = c->d_wcount; A.undecided = c->d_undecided;
+    A.inc_slot = c->d_inc_slot; A.sync = c->d_sync; A.status = c->d_status; A.one_Esum = c->d_one_Esum; A.counters = c->d_counters;
+    const size_t most = std::max((size_t)std::max(c->Ppop + 1, dm.N), c->d_wcount ? 2 * (size_t)c->Ppop * dm.RG / 8 : 0);
+    const int grid = (int)std::min<size_t>(148 * 4, (most + 255) / 256);
+    k_setup_population<<<grid, 256, 0, c->stream>>>(A);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
@@ -406,16 +535,17 @@ int rp_launch_build_static(rp_ctx *c)
 // Load-balance diagnostics (evaluation section of the paper): coefficient of variation of the
 // aggregate rank loads, EP peak sum, tail peak, EP balance efficiency, attention and joint proxies.
 // ---------------------------------------------------------------------------------------------
-struct RpDiagDev { double cv_identity, cv_placed; i64 s_ep, t_ep, n_ep; i64 afx_sum, s0; };
+struct RpDiagDev { double cv_identity, cv_placed; i64 s_ep, t_ep, n_ep; i64 afx_sum, s0; int tickets, pad; };
 
 // One warp per layer: the lanes fetch the rank loads, one lane adds them up with plain sequential IEEE sums (no fused
 // multiply-add); then thread 0 averages the layers in order.
 #define DIAG_THREADS 1024
 __global__ void __launch_bounds__(DIAG_THREADS)
-k_diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, RpDims dm, RpDiagDev *__restrict__ out)
+k_diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, RpDims dm, RpDiagDev *__restrict__ sums, RpDiagDev *__restrict__ out)
 {
     extern __shared__ double cvs[];          // [2][L], then one row of rank loads per warp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) { sums->s_ep = 0; sums->t_ep = 0; sums->n_ep = 0; sums->tickets = 0; }      // for the kernel behind this one
     double *G = cvs + 2 * dm.L + (size_t)warp * dm.P;
     for (int x = warp; x < 2 * dm.L; x += DIAG_THREADS / 32) {
         const int l = x >> 1, which = x & 1;
@@ -453,7 +583,7 @@ k_diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, RpDim
 
 // One warp per (row, layer): lanes over ranks, loop over shards; integer results by atomics.
 __global__ void k_diag_peaks(const int *__restrict__ W, const char *__restrict__ blob, RpBlob bl, RpDims dm,
-                             RpDiagDev *__restrict__ out)
+                             RpDiagDev *__restrict__ sums, RpDiagDev *__restrict__ out)
 {
     const int lane = threadIdx.x & 31;
     const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
@@ -461,6 +591,7 @@ __global__ void k_diag_peaks(const int *__restrict__ W, const char *__restrict__
     for (int rl = wid; rl < dm.R * dm.L; rl += nw) {
         const int r = rl / dm.L, l = rl % dm.L;
         i64 peak = 0, best_sum = 0;
+#pragma unroll 4
         for (int g = 0; g < dm.G; ++g) {
             const int *w = W + (((size_t)r * dm.G + g) * dm.L + l) * dm.P;
             i64 sum = 0, mx = 0;
@@ -476,9 +607,9 @@ __global__ void k_diag_peaks(const int *__restrict__ W, const char *__restrict__
         s_ep += peak; n_ep += best_sum; t_ep = peak > t_ep ? peak : t_ep;
     }
     if (lane == 0) {
-        if (s_ep) atomicAdd((u64 *)&out->s_ep, (u64)s_ep);
-        if (n_ep) atomicAdd((u64 *)&out->n_ep, (u64)n_ep);
-        atomicMax((i64 *)&out->t_ep, t_ep);
+        if (s_ep) atomicAdd((u64 *)&sums->s_ep, (u64)s_ep);
+        if (n_ep) atomicAdd((u64 *)&sums->n_ep, (u64)n_ep);
+        if (t_ep) atomicMax((i64 *)&sums->t_ep, t_ep);
     }
     if (blockIdx.x == 0 && threadIdx.x < 32) {      // attention total and joint from the layout's blob
         const i64 *Afx = (const i64 *)(blob + bl.off_Afx);
@@ -486,6 +617,12 @@ __global__ void k_diag_peaks(const int *__restrict__ W, const char *__restrict__
         for (int x = lane; x < dm.RG; x += 32) a += Afx[x];
         for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
         if (lane == 0) { out->afx_sum = a; out->s0 = ((const i64 *)(blob + bl.off_S))[0]; }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&sums->tickets, 1) == (int)gridDim.x - 1) {
+        __threadfence();
+        out->s_ep = __ldcg(&sums->s_ep); out->n_ep = __ldcg(&sums->n_ep); out->t_ep = __ldcg(&sums->t_ep);
     }
 }
 
@@ -497,54 +634,44 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
     if (dm.L > 1024) return RP_ERR_RANGE;
     cudaMemPool_t pool;
     RP_TRY(rp_get_pool(c->device, &pool));
-    // scratch: cells, W, one blob, the result record, and the row-shard sums / ticket of the scoring kernel
+    // scratch: a copy of a host layout, W, one blob
     const size_t wn = (size_t)dm.RG * dm.LP;
-    size_t off_cells = 0, off_lay = off_cells + (((size_t)dm.N * 2 + 255) & ~(size_t)255);
-    size_t off_W = off_lay + (((size_t)dm.N * 4 + 255) & ~(size_t)255);
-    size_t off_blob = off_W + ((wn * 4 + 255) & ~(size_t)255);
-    size_t off_res = off_blob + (((size_t)c->bl.bytes + 255) & ~(size_t)255);
-    size_t off_es = off_res + 256, off_tk = off_es + (((size_t)dm.RG * 8 + 255) & ~(size_t)255);
-    size_t total = off_tk + 256;
+    const size_t off_W = ((size_t)dm.N * 4 + 255) & ~(size_t)255, off_blob = off_W + ((wn * 4 + 255) & ~(size_t)255);
+    const size_t off_res = off_blob + (((size_t)c->bl.bytes + 255) & ~(size_t)255);
+    const size_t cv_smem = sizeof(double) * (2 * (size_t)dm.L + (DIAG_THREADS / 32) * (size_t)dm.P);
     char *buf = nullptr;
-    RP_CUDA(cudaMallocFromPoolAsync((void **)&buf, total, pool, c->stream));
+    RP_CUDA(cudaMallocFromPoolAsync((void **)&buf, off_res + 256, pool, c->stream));
     int st = RP_OK;
     cudaError_t e = cudaSuccess;
     do {
-        const int *dl = c->d_inc_layout;
-        if (layout) {
-            e = cudaMemcpyAsync(buf + off_lay, layout, sizeof(int) * dm.N, cudaMemcpyDefault, c->stream);
+        const int *dl = layout ? layout : c->d_inc_layout;
+        if (layout && !rp_is_device_ptr(layout)) {
+            e = cudaMemcpyAsync(buf, layout, sizeof(int) * dm.N, cudaMemcpyDefault, c->stream);
             if (e != cudaSuccess) break;
-            dl = (const int *)(buf + off_lay);
+            dl = (const int *)buf;
         }
-        e = cudaMemsetAsync(buf + off_res, 0, 256 + (off_tk - off_es) + 256, c->stream);
-        if (e != cudaSuccess) break;
-        e = cudaMemsetAsync(c->d_status + RP_SW_BAD_LAYOUT, 0, sizeof(int), c->stream);
-        if (e != cudaSuccess) break;
-        k_layouts_to_cells<<<(dm.N + 255) / 256, 256, 0, c->stream>>>(dl, dm.N, dm.K, (unsigned short *)(buf + off_cells),
-                                                                     c->d_status);
-        ++g_rp_launches;
-        st = eval_launch(c, (const unsigned short *)(buf + off_cells), 1, (int *)(buf + off_W), buf + off_blob, nullptr, nullptr,
-                         (i64 *)(buf + off_es), (int *)(buf + off_tk));
+        int *bad = rp_pin_bad(c);
+        *bad = 0;
+        EvalArgs A = {};
+        eval_one(c, A);
+        A.lay32 = dl; A.W_out = (int *)(buf + off_W); A.blob_out = buf + off_blob;
+        st = eval_launch(c, A, 1);
         if (st != RP_OK) break;
-        RpDiagDev *res = (RpDiagDev *)(buf + off_res);
-        const size_t cv_smem = sizeof(double) * (2 * (size_t)dm.L + (DIAG_THREADS / 32) * (size_t)dm.P);
+        // the record goes to the pinned block: its sums by the last CTA of the peaks, the rest by the first
+        RpDiagDev *res = (RpDiagDev *)(buf + off_res), *host = (RpDiagDev *)(c->h_pin + 32);
         if (cv_smem > 32 * 1024) {
             e = cudaFuncSetAttribute(k_diag_cv, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX);
             if (e != cudaSuccess) break;
         }
-        k_diag_cv<<<1, DIAG_THREADS, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, dm, res);
+        k_diag_cv<<<1, DIAG_THREADS, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, dm, res, host);
         ++g_rp_launches;
-        k_diag_peaks<<<148, 256, 0, c->stream>>>((const int *)(buf + off_W), buf + off_blob, c->bl, dm, res);
+        k_diag_peaks<<<148, 256, 0, c->stream>>>((const int *)(buf + off_W), buf + off_blob, c->bl, dm, res, host);
         ++g_rp_launches;
         e = cudaGetLastError();
-        if (e != cudaSuccess) break;
-        RpDiagDev h;
-        int bad = 0;
-        e = cudaMemcpyAsync(&h, res, sizeof h, cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, c->d_status + RP_SW_BAD_LAYOUT, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) break;
-        if (bad) { st = RP_ERR_ARG; break; }
+        if (*bad) { st = RP_ERR_ARG; break; }
+        const RpDiagDev h = *host;
         out->cv_identity = h.cv_identity; out->cv_placed = h.cv_placed;
         out->s_ep = h.s_ep; out->t_ep = h.t_ep; out->n_ep = h.n_ep;
         out->eta_ep = h.s_ep > 0 ? (double)h.n_ep / ((double)dm.P * (double)h.s_ep) : 1.0;
@@ -557,8 +684,8 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
 }
 
 // ---------------------------------------------------------------------------------------------
-// Scoring layouts without allocating: the kernels above, with their scratch (16-bit cell ids,
-// row-shard sums, arrival counters) taken from a fixed array that is part of the library image
+// Scoring layouts without allocating: the kernels above, with their scratch (samples grouped by
+// row-shard, row-shard sums, arrival counters) taken from a fixed array that is part of the library image
 // instead of from the context's allocator.
 // ---------------------------------------------------------------------------------------------
 #define RP_NOALLOC_MAX_LAYOUTS 1024            // layouts per call
@@ -566,11 +693,12 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
 #define RP_NOALLOC_MAX_ROWSHARDS (1 << 15)     // n * R * G      (256 KiB of 64-bit sums)
 
 struct RpNoAllocScratch {
+    int tickets[RP_NOALLOC_MAX_LAYOUTS];           // (next to the sums: cleared together)
     i64 esum[RP_NOALLOC_MAX_ROWSHARDS];
-    int tickets[RP_NOALLOC_MAX_LAYOUTS];
-    unsigned short cells[RP_NOALLOC_MAX_CELLS];
+    int off[RP_NOALLOC_MAX_ROWSHARDS + RP_NOALLOC_MAX_LAYOUTS];
+    unsigned short list[RP_NOALLOC_MAX_CELLS];
 };
-// About 1.3 MiB on every GPU that loads the library, held until the process exits.
+// About 1.4 MiB on every GPU that loads the library, held until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(RpNoAllocScratch)];
 // Device address of the array above, per device (in host code the symbol itself is only a
 // stand-in, never a device address).
@@ -606,16 +734,13 @@ extern "C" int rp_eval_layouts_noalloc(rp_ctx *c, const int32_t *layouts, int32_
     }
     RpNoAllocScratch *sc = (RpNoAllocScratch *)g_noalloc_addr[cur];
     // the array keeps what the previous call left: the arrival counters and the row-shard sums must start at zero
-    RP_CUDA(cudaMemsetAsync(sc->tickets, 0, sizeof(int) * n, c->stream));
-    RP_CUDA(cudaMemsetAsync(sc->esum, 0, sizeof(i64) * (size_t)n * dm.RG, c->stream));
-    RP_CUDA(cudaMemsetAsync(c->d_status + RP_SW_BAD_LAYOUT, 0, sizeof(int), c->stream));
-    const long long total = (long long)n * dm.N;
-    k_layouts_to_cells<<<(int)((total + 255) / 256), 256, 0, c->stream>>>(layouts, total, dm.K, sc->cells, c->d_status);
-    ++g_rp_launches;
-    RP_CUDA(cudaGetLastError());
-    RP_TRY(eval_launch(c, sc->cells, n, nullptr, nullptr, (i64 *)score_fx, score_f64, sc->esum, sc->tickets));
-    int bad = 0;
-    RP_CUDA(cudaMemcpyAsync(&bad, c->d_status + RP_SW_BAD_LAYOUT, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    RP_CUDA(cudaMemsetAsync(sc, 0, sizeof(sc->tickets) + sizeof(i64) * (size_t)n * dm.RG, c->stream));
+    int *bad = rp_pin_bad(c);
+    *bad = 0;
+    EvalArgs A = {};
+    A.lay32 = layouts; A.score_out = (i64 *)score_fx; A.f64_out = score_f64; A.bad = bad;
+    A.Esum = sc->esum; A.tickets = sc->tickets; A.list = sc->list; A.off = sc->off;
+    RP_TRY(eval_launch(c, A, n));
     RP_CUDA(cudaStreamSynchronize(c->stream));
-    return bad ? RP_ERR_ARG : RP_OK;
+    return *bad ? RP_ERR_ARG : RP_OK;
 }

@@ -208,7 +208,7 @@ int rp_launch_pack_on(rp_ctx *c, cudaStream_t stream)
     // small windows: fewer warps make the block-wide barriers of the sort cheaper
     const int threads = n_pow2 >= PACK_THREADS ? PACK_THREADS : (n_pow2 < 256 ? 256 : n_pow2);
     k_pack_ffd<<<1, threads, smem, stream>>>(dm, c->d_t, c->cfg.min_rows, keys_g, n_pow2, fill_g,
-                                                    c->d_seed_layout, c->d_pack_out, c->d_order);
+                                                    c->d_seed_layout, (int *)(c->h_pin + 10), c->d_order);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
