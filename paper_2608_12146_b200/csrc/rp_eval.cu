@@ -6,9 +6,9 @@
 //  * few layouts (k_eval_few: the seed, the incumbent, diagnostics, small batches), bound by latency: a cluster of
 //    CTAs per row-shard, each over its share of the samples, sixteen 16-byte loads in flight per lane; the CTAs'
 //    sums meet through distributed shared memory;
-//  * many layouts (k_eval_group, k_eval_sum), bound by L2: the samples of a layout are grouped by row-shard once, then
-//    a warp per row-shard sums its rows, sixteen bytes per lane and eight samples in flight.
-// In both the CTA that finishes a layout last (atomic ticket) scores it.
+//  * many layouts (k_eval_group, k_eval_sum, k_eval_score), bound by L2: the samples of a layout are grouped by row-shard once, then
+//    a warp per row-shard sums its rows, sixteen bytes per lane and eight to twelve loads in flight.
+// In the first the CTA that finishes a layout last (atomic ticket) scores it.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -221,70 +221,108 @@ k_eval_group(const EvalArgs A)
     for (int i = tid; i < dm.N; i += GROUP_THREADS) list[atomicAdd(&off[rgs[i]], 1)] = (unsigned short)i;
 }
 
-// Many layouts, second kernel: grid (row-shards / 8, layouts), a warp per row-shard.
-__global__ void __launch_bounds__(EVAL_THREADS, 5)
-k_eval_sum(const EvalArgs A)
+// Many layouts, second kernel.  A task is NS strips of 32 chunks (whole layers) of `rpt` consecutive row-shards of one
+// layout: a warp streams through their samples, which lie one after the other in the list, with U*NS loads in flight
+// whatever row-shard they belong to, and closes a row-shard when its last sample has been added.  Bound by its
+// instructions before it is by L2: row-shards hold 8.5 samples on average on large, and loops over one row-shard, or
+// one strip, at a time took 127 to 175 us for 256 layouts (46 instructions per sample and strip; 20 per sample and three strips here).
+template <int NS, int U>
+__global__ void __launch_bounds__(EVAL_THREADS, NS == 1 ? 4 : (NS == 2 ? 3 : 2))
+k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt)
 {
-    extern __shared__ __align__(16) unsigned char smraw[];
     const RpDims &dm = A.dm;
-    __shared__ int last_s;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lay = blockIdx.y;
-    const int rg = blockIdx.x * (EVAL_THREADS / 32) + warp;
-    if (rg < dm.RG) {
-        const int *go = A.off + (size_t)lay * (dm.RG + 1);
+    const int lane = threadIdx.x & 31, RG = dm.RG, rc = dm.LP >> 2;
+    const bool vec = eval_vec(dm);
+    const int groups = (RG + rpt - 1) / rpt, per = groups * sgroups;
+    const int cpl = dm.P >> 2, used = vec ? (32 / cpl) * cpl : 32;
+    const bool sum32 = (i64)dm.L * dm.k * dm.C * ((dm.D + dm.G - 1) / dm.G) < (1ll << 31);
+    for (unsigned task = blockIdx.x * (EVAL_THREADS / 32) + (threadIdx.x >> 5); task < (unsigned)n * (unsigned)per; task += gridDim.x * (EVAL_THREADS / 32)) {
+        const int lay = (int)(task / (unsigned)per), r = (int)(task - (unsigned)lay * per), sg = r % sgroups, rg0 = r / sgroups * rpt, nr = min(rpt, RG - rg0);
+        const int *go = A.off + (size_t)lay * (RG + 1) + rg0;
         const unsigned short *list = A.list + (size_t)lay * dm.N;
-        const int m0 = __ldg(go + rg), m1 = __ldg(go + rg + 1), rc = dm.LP >> 2;
-        int *wout = A.W_out ? A.W_out + ((size_t)lay * dm.RG + rg) * dm.LP : nullptr;
-        i64 es;
-        if (eval_vec(dm)) {
-            const int cpl = dm.P >> 2, used = (32 / cpl) * cpl;
-            es = 0;
-            for (int c0 = 0; c0 < rc; c0 += used) {
-                const int c = c0 + lane;
-                const bool on = lane < used && c < rc;
-                const int4 *col = (const int4 *)A.q + (on ? c : 0);
-                int4 a = make_int4(0, 0, 0, 0);
-                for (int mb = m0; mb < m1; mb += 32) {
-                    // the next 32 samples of the list, one per lane, handed round by shuffles; eight rows in flight
-                    const int id = mb + lane < m1 ? (int)__ldg(list + mb + lane) : 0, nm = min(32, m1 - mb);
-                    for (int x0 = 0; x0 < nm; x0 += 8) {
-                        int4 v[8];
+        const int ends = __ldg(go + min(lane + 1, nr)), s0 = __ldg(go);           // lane x: where row-shard rg0 + x ends
+        if (!vec) {
+            int m0 = s0;
+            for (int x = 0; x < nr; ++x) {
+                const int m1 = __shfl_sync(0xffffffffu, ends, x);
+                int *wout = A.W_out ? A.W_out + ((size_t)lay * RG + rg0 + x) * dm.LP : nullptr;
+                const i64 es = rp_warp_layer_max_sum(dm, lane, [&](int e) {
+                    int sum = 0;
+                    for (int m = m0; m < m1; ++m) sum += __ldg(A.q + (size_t)__ldg(list + m) * dm.LP + e);
+                    if (wout) wout[e] = sum;
+                    return sum;
+                });
+                if (lane == 0) A.Esum[(size_t)lay * RG + rg0 + x] = es;
+                m0 = m1;
+            }
+            continue;
+        }
+        int4 a[NS];
+        const int4 *col[NS];                // (lanes and strips past the row's end read its first chunk and are ignored)
+        unsigned on = 0;
 #pragma unroll
-                        for (int x = 0; x < 8; ++x) {
-                            const int s = __shfl_sync(0xffffffffu, id, x0 + x);
-                            v[x] = x0 + x < nm ? __ldg(col + (size_t)s * rc) : make_int4(0, 0, 0, 0);
-                        }
+        for (int z = 0; z < NS; ++z) {
+            const int c = (sg * NS + z) * used + lane;
+            a[z] = make_int4(0, 0, 0, 0);
+            if (lane < used && c < rc) on |= 1u << z;
+            col[z] = (const int4 *)A.q + (((on >> z) & 1u) ? c : 0);
+        }
+        const int s1 = __shfl_sync(0xffffffffu, ends, nr - 1);
+        int x = 0, end = __shfl_sync(0xffffffffu, ends, 0);
+        auto close = [&]() {                // row-shard rg0 + x is complete
+            const size_t at = (size_t)lay * RG + rg0 + x;
+            int own = 0;
 #pragma unroll
-                        for (int x = 0; x < 8; ++x) { a.x += v[x].x; a.y += v[x].y; a.z += v[x].z; a.w += v[x].w; }
+            for (int z = 0; z < NS; ++z) {
+                const bool o = (on >> z) & 1u;
+                if (A.W_out && o) ((int4 *)(A.W_out + at * dm.LP))[(sg * NS + z) * used + lane] = a[z];
+                const int m = eval_layer_max(o ? max(max(a[z].x, a[z].y), max(a[z].z, a[z].w)) : 0, lane, cpl);
+                own += o && lane % cpl == 0 ? m : 0;          // (a layer's busiest load fits 31 bits, three of them 32)
+                a[z] = make_int4(0, 0, 0, 0);
+            }
+            i64 es;
+            if (sum32) es = (i64)__reduce_add_sync(0xffffffffu, (unsigned)own);
+            else { es = (i64)(unsigned)own; for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o); }
+            if (lane == 0) {
+                if (sgroups > 1) atomicAdd((u64 *)(A.Esum + at), (u64)es);
+                else A.Esum[at] = es;
+            }
+            ++x;
+            end = __shfl_sync(0xffffffffu, ends, x);
+        };
+        int next = s0 + lane < s1 ? (int)__ldg(list + s0 + lane) : 0;
+        for (int p = s0; p < s1; p += 32) {
+            const int id = next, nm = min(32, s1 - p);
+            next = p + 32 + lane < s1 ? (int)__ldg(list + p + 32 + lane) : 0;
+            for (int y = 0; y < nm; y += U) {
+                int4 v[U][NS];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {               // (past the end: sample 0, not counted)
+                    const int at = __shfl_sync(0xffffffffu, id, y + u) * rc;          // N*L*P/4 fits 31 bits
+#pragma unroll
+                    for (int z = 0; z < NS; ++z) v[u][z] = __ldg(col[z] + at);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (y + u < nm) {
+                        while (p + y + u == end) close();
+#pragma unroll
+                        for (int z = 0; z < NS; ++z) { a[z].x += v[u][z].x; a[z].y += v[u][z].y; a[z].z += v[u][z].z; a[z].w += v[u][z].w; }
                     }
                 }
-                if (wout && on) ((int4 *)wout)[c] = a;
-                const int m = eval_layer_max(on ? max(max(a.x, a.y), max(a.z, a.w)) : 0, lane, cpl);
-                if (on && lane % cpl == 0) es += m;
             }
-            for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
-        } else {
-            es = rp_warp_layer_max_sum(dm, lane, [&](int x) {
-                int s = 0;
-                for (int m = m0; m < m1; ++m) s += __ldg(A.q + (size_t)__ldg(list + m) * dm.LP + x);
-                if (wout) wout[x] = s;
-                return s;
-            });
         }
-        if (lane == 0) A.Esum[(size_t)lay * dm.RG + rg] = es;
+        while (x < nr) close();             // the last ones (no sample lies beyond s1)
     }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        last_s = (atomicAdd(&A.tickets[lay], 1) == (int)gridDim.x - 1);
-        if (last_s) A.tickets[lay] = 0;                   // ready for the next launch
-    }
-    __syncthreads();
-    if (!last_s) return;
-    __threadfence();
-    const EvalFinish f = eval_finish_views(dm, smraw);
-    eval_load_cells(A, lay, f.cell_of, tid, EVAL_THREADS);
-    eval_finish(A, lay, f, tid);
+}
+
+__global__ void __launch_bounds__(EVAL_THREADS)
+k_eval_score(const EvalArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const EvalFinish f = eval_finish_views(A.dm, smraw);
+    eval_load_cells(A, blockIdx.x, f.cell_of, threadIdx.x, EVAL_THREADS);
+    eval_finish(A, blockIdx.x, f, threadIdx.x);
 }
 
 // grid = (MS, row-shards, layouts), clusters of MS CTAs along x: CTA x of a row-shard takes the samples of
@@ -393,20 +431,28 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
         const size_t gm = sizeof(int) * (size_t)dm.RG + 2 * ((size_t)dm.K + dm.N), fm = eval_finish_bytes(dm);
         if (gm > EVAL_SMEM_MAX || dm.N > 65535) return RP_ERR_RANGE;
         if (gm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_group, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
-        if (fm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_sum, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
-        const int gx = (dm.RG + EVAL_THREADS / 32 - 1) / (EVAL_THREADS / 32);
-        for (int first = 0; first < n; first += 65535) {                 // (layouts along y)
+        if (fm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_score, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
+        const int cpl = dm.P >> 2, used = eval_vec(dm) ? 32 / cpl * cpl : 32, strips = eval_vec(dm) ? ((dm.LP >> 2) + used - 1) / used : 1;
+        const int ns = std::min(3, strips), sgroups = (strips + ns - 1) / ns, warps = ns == 1 ? 32 : (ns == 2 ? 24 : 16);     // per SM
+        for (int first = 0; first < n; first += 16384) {                 // (bounds the task numbers of a launch)
             EvalArgs B = A;
-            const int m = std::min(65535, n - first);
+            const int m = std::min(16384, n - first);
             if (B.lay32) B.lay32 += (size_t)first * dm.N; else B.src += first;
             if (B.W_out) B.W_out += (size_t)first * dm.RG * dm.LP;
             if (B.blob_out) B.blob_out += (size_t)first * c->bl.bytes;
             if (B.score_out) B.score_out += 3 * (size_t)first;
             if (B.f64_out) B.f64_out += 3 * (size_t)first;
             B.Esum += (size_t)first * dm.RG; B.tickets += first; B.list += (size_t)first * dm.N; B.off += (size_t)first * (dm.RG + 1);
+            // several tasks for each warp the SMs hold, of at most 31 row-shards
+            const int rpt = (int)std::max<long long>(1, std::min<long long>(31, (long long)m * dm.RG * sgroups / (148 * warps * 6)));
+            const long long want = ((long long)m * ((dm.RG + rpt - 1) / rpt) * sgroups + 7) / 8;
+            const int grid = (int)std::min<long long>(want, 148 * warps / 8);
             k_eval_group<<<m, GROUP_THREADS, gm, c->stream>>>(B);
-            k_eval_sum<<<dim3(gx, m), EVAL_THREADS, fm, c->stream>>>(B);
-            ++g_rp_launches;
+            if (ns == 1) k_eval_sum<1, 8><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt);
+            else if (ns == 2) k_eval_sum<2, 4><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt);
+            else k_eval_sum<3, 4><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt);
+            k_eval_score<<<m, EVAL_THREADS, fm, c->stream>>>(B);
+            g_rp_launches += 2;
         }
     }
     ++g_rp_launches;
