@@ -9,51 +9,85 @@
 
 #define PACK_THREADS 1024
 
-// First fit of the samples keys[K..N) into K cells by one warp; lane `tid` owns cells
-// [tid*B, tid*B+B).  Returns true when some sample fits nowhere.  BR >= B cells per lane are
-// kept in registers (statically indexed); the shared-memory variant handles any B.
-template <int BR>
-__device__ __forceinline__ bool first_fit_regs(const RpDims &dm, const u64 *keys, int *fill, int *cell_of, int K, int B, int tid)
+// First fit of the samples keys[K..N) into K cells by one warp, 32 samples at a time.
+//
+// Every lane looks up the lowest cell that takes its own sample, against the same state, in a tree of maxima (eight
+// children per node, two 16-byte loads a level).  Samples come longest first, so the cells found do not increase from
+// lane to lane and samples that found the same cell are neighbours: a segmented sum tells which of them still fit after
+// the ones before; these are placed.  The others (and those behind them in their group) stay for the next round, ahead
+// of new samples.  The order of placement does not matter: a sample that waits found a higher cell than every later
+// sample placed meanwhile, so it does not fit where those went, and wherever it goes in the end lies higher.  A sample
+// for which no cell is left has none in the one-by-one order either.
+// One sample at a time cost 250 cycles (524 us on wide's 4096 samples); see k_pack_ffd for now.
+#define FFD_LEVELS 4                        // 8^4 cells
+#define FFD_MAX_CELLS 4096
+__device__ __forceinline__ int max8(const int *p)
 {
-    const int b0 = tid * B;
-    int rem[BR];
-    int blockmax = -1;
-    bool failed = false;                           // some sample fitted nowhere (the rest of the pass is then moot)
-#pragma unroll
-    for (int u = 0; u < BR; ++u) {
-        rem[u] = (u < B && b0 + u < K) ? dm.C - fill[b0 + u] : -1;
-        blockmax = max(blockmax, rem[u]);
-    }
-    for (int x0 = K; x0 < dm.N; x0 += 32) {
-        // the next 32 keys, one per lane, handed out by shuffles
-        const u64 mine = (x0 + tid < dm.N) ? keys[x0 + tid] : 0;
-        const int nx = min(32, dm.N - x0);
-        const int my_len = dm.C - (int)(mine >> 32), my_id = (int)(u32)mine;
-#pragma unroll 4
-        for (int y = 0; y < nx; ++y) {
-            const int ts = __shfl_sync(0xffffffffu, my_len, y), id = __shfl_sync(0xffffffffu, my_id, y);
-            // every lane works out what it would do if the sample fell to it (first cell of its
-            // block that fits, block maximum afterwards), with no chain from cell to cell; only
-            // the ballot and the selects after it link one sample to the next
-            bool fits[BR];
-#pragma unroll
-            for (int u = 0; u < BR; ++u) fits[u] = rem[u] >= ts;
-            int first = BR;
-#pragma unroll
-            for (int u = BR - 1; u >= 0; --u) first = fits[u] ? u : first;
-            int nm = -1;
-#pragma unroll
-            for (int u = 0; u < BR; ++u) nm = max(nm, u == first ? rem[u] - ts : rem[u]);
-            const unsigned m = __ballot_sync(0xffffffffu, blockmax >= ts);
-            failed |= (m == 0);
-            const bool win = (tid == __ffs(m) - 1);
-#pragma unroll
-            for (int u = 0; u < BR; ++u) rem[u] = (win && u == first) ? rem[u] - ts : rem[u];
-            blockmax = win ? nm : blockmax;
-            if (win) cell_of[id] = b0 + first;
+    const int4 a = ((const int4 *)p)[0], b = ((const int4 *)p)[1];
+    return max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w)));
+}
+__device__ __forceinline__ int first8(const int *p, int t)              // first of eight entries that is at least t
+{
+    const int4 a = ((const int4 *)p)[0], b = ((const int4 *)p)[1];
+    const unsigned m = (a.x >= t ? 1u : 0u) | (a.y >= t ? 2u : 0u) | (a.z >= t ? 4u : 0u) | (a.w >= t ? 8u : 0u) |
+                       (b.x >= t ? 16u : 0u) | (b.y >= t ? 32u : 0u) | (b.z >= t ? 64u : 0u) | (b.w >= t ? 128u : 0u);
+    return __ffs(m) - 1;
+}
+// tree: levels from the leaves (remaining capacity, padded with -1) up; lev[x] = start of level x; depth levels, the last of at most 8 entries.
+__device__ __forceinline__ bool first_fit_rounds(const RpDims &dm, const u64 *keys, int *tree, const int *lev, int depth, int *queue,
+                                                 int *cell_of, int K, int lane)
+{
+    int len = 0, id = 0, kept = 0, next = K;
+    bool have = false;
+    for (;;) {
+        // samples left over from the last round first, then new ones
+        if (lane >= kept) {
+            const int x = next + lane - kept;
+            have = x < dm.N;
+            if (have) { const u64 key = keys[x]; len = dm.C - (int)(key >> 32); id = (int)(u32)key; }
         }
+        next += 32 - kept;
+        if (!__any_sync(0xffffffffu, have)) return false;
+        const int want = have ? len : 0x7fffffff;
+        int c = 0;
+        for (int l = depth - 1; l >= 0; --l) {
+            const int f = first8(tree + lev[l] + 8 * c, want);
+            c = 8 * c + (f < 0 ? 0 : f);
+            if (l == depth - 1 && __any_sync(0xffffffffu, have && f < 0)) return true;           // nowhere to go
+        }
+        if (!have) c = -1;
+        // length of the group before this lane
+        const int before_c = __shfl_up_sync(0xffffffffu, c, 1);
+        const bool head = lane == 0 || before_c != c;
+        const unsigned heads = __ballot_sync(0xffffffffu, head);
+        const int h = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+        int sum = have ? len : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, sum, o); if (lane - o >= h) sum += y; }
+        const int rem = have ? tree[lev[0] + c] : 0;
+        const bool fits = have && sum <= rem;                        // sums grow along a group: true up to a lane, then false
+        const unsigned ok = __ballot_sync(0xffffffffu, fits), wait = __ballot_sync(0xffffffffu, have && !fits);
+        __syncwarp();
+        if (fits) {
+            cell_of[id] = c;
+            const bool lastly = lane == 31 || ((heads >> (lane + 1)) & 1u) || !((ok >> (lane + 1)) & 1u);
+            if (lastly) tree[lev[0] + c] = rem - sum;
+        } else if (have) {
+            const int at = __popc(wait & ((1u << lane) - 1u));
+            queue[2 * at] = len; queue[2 * at + 1] = id;
+        }
+        __syncwarp();
+        // maxima above the changed cells, level by level (several lanes may write the same value)
+        for (int l = 1, n = c >> 3; l < depth; ++l, n >>= 3) {
+            const int m = fits ? max8(tree + lev[l - 1] + 8 * n) : 0;
+            __syncwarp();
+            if (fits) tree[lev[l] + n] = m;
+            __syncwarp();
+        }
+        kept = __popc(wait);
+        if (lane < kept) { len = queue[2 * lane]; id = queue[2 * lane + 1]; have = true; }
+        __syncwarp();
     }
-    return failed;
 }
 
 __device__ __forceinline__ bool first_fit_smem(const RpDims &dm, const u64 *keys, int *fill, int *cell_of, int K, int B, int tid)
@@ -84,9 +118,11 @@ __global__ void __launch_bounds__(PACK_THREADS)
 k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *__restrict__ keys_g, int n_pow2,
            int *__restrict__ fill_g, int *__restrict__ cell_of, int *__restrict__ out, int *__restrict__ order_out)
 {
-    extern __shared__ u64 keys_s[];
+    extern __shared__ __align__(16) u64 keys_s[];
     u64 *keys = keys_g ? keys_g : keys_s;
     int *fill = fill_g ? fill_g : (int *)(keys_s + (keys_g ? 0 : n_pow2));
+    __shared__ __align__(16) int tree[FFD_MAX_CELLS + FFD_MAX_CELLS / 8 + FFD_MAX_CELLS / 64 + 8];
+    __shared__ int queue[64], lev[FFD_LEVELS];
     __shared__ i64 total_s;
     __shared__ int fail_s;
     const int tid = threadIdx.x, nt = (int)blockDim.x;
@@ -162,21 +198,29 @@ k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *__restrict__
         // the K longest samples open the cells
         for (int x = tid; x < K; x += nt) {
             const u64 key = keys[x];
-            fill[x] = dm.C - (int)(key >> 32);
+            if (K > FFD_MAX_CELLS) fill[x] = dm.C - (int)(key >> 32);
+            else tree[x] = (int)(key >> 32);                         // what is left of the cell
             cell_of[(u32)key] = x;
+        }
+        int depth = 1;
+        if (K <= FFD_MAX_CELLS) {
+            int n = (K + 7) & ~7, at = 0;                             // entries of a level, padded to whole nodes
+            for (int x = K + tid; x < n; x += nt) tree[x] = -1;
+            if (tid == 0) lev[0] = 0;
+            __syncthreads();
+            for (; n > 8; ++depth) {
+                const int up = n >> 3, upn = (up + 7) & ~7;
+                for (int x = tid; x < upn; x += nt) tree[at + n + x] = x < up ? max8(tree + at + 8 * x) : -1;
+                if (tid == 0) lev[depth] = at + n;
+                at += n; n = upn;
+                __syncthreads();
+            }
         }
         __syncthreads();
         if (tid < 32) {
-            // First fit = the lowest cell whose remaining capacity takes the sample.  Each lane
-            // owns a block of B consecutive cells and keeps the largest remaining capacity of its
-            // block in a register: one ballot finds the lowest lane that can take the sample, and
-            // only that lane scans its block (held in registers when B <= 16).
-            const int B = (K + 31) / 32;
-            bool failed;
-            if (B <= 4) failed = first_fit_regs<4>(dm, keys, fill, cell_of, K, B, tid);
-            else if (B <= 8) failed = first_fit_regs<8>(dm, keys, fill, cell_of, K, B, tid);
-            else if (B <= 16) failed = first_fit_regs<16>(dm, keys, fill, cell_of, K, B, tid);
-            else failed = first_fit_smem(dm, keys, fill, cell_of, K, B, tid);
+            // First fit = the lowest cell whose remaining capacity takes the sample.
+            const bool failed = K <= FFD_MAX_CELLS ? first_fit_rounds(dm, keys, tree, lev, depth, queue, cell_of, K, tid)
+                                                   : first_fit_smem(dm, keys, fill, cell_of, K, (K + 31) / 32, tid);
             if (failed && tid == 0) fail_s = 1;
         }
         __syncthreads();
