@@ -1157,3 +1157,22 @@ def test_smallest_window_and_empty_moves():
     layout, fx, _ = rp.rp_best(ctx)
     assert (layout == want["best_layout"]).all() and (fx == want["best_score"]).all()
     rp.rp_destroy(ctx)
+
+
+# Both orders (sort in the packing CTA up to 512 samples and above 32768, counting on the whole GPU between), cells held one
+# and four a lane, keys in shared and global memory, one-token samples that fill a cell by the run.
+@pytest.mark.parametrize("N,D,min_rows,cap,longest", [
+    (33, 1, 0, 40, 40), (512, 4, 0, 64, 64), (513, 4, 0, 64, 20), (700, 7, 0, 4096, 1), (2100, 4, 256, 64, 40),
+    (2100, 5, 205, 64, 40), (2049, 2, 1024, 100, 100), (8193, 8, 120, 64, 4),
+    (9000, 8, 0, 4096, 300), (32770, 8, 0, 1 << 20, 4096)])
+def test_packing_at_the_edges_of_its_forms(N, D, min_rows, cap, longest):
+    rng = np.random.default_rng(N + D)
+    t = rng.integers(1, longest + 1, N).astype(np.int32)
+    a = np.zeros((N, 1, 2), np.int32)
+    a[np.arange(N), 0, rng.integers(0, 2, N)] = t
+    R, cert, seed = oracle.pack_ffd(t, cap, D, min_rows)
+    ctx = rp.rp_window_load(t, a, top_k=1, token_cap=cap, dp_width=D, ep_width=2, pop_size=2, min_rows=min_rows)
+    rp.rp_place_experts(ctx)
+    assert rp.rp_pack_rows(ctx) == (R, cert)
+    assert (rp.rp_debug_dump(ctx, "SEED_LAYOUT", (N,), np.int32) == seed).all()
+    rp.rp_destroy(ctx)
