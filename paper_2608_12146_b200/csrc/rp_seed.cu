@@ -2,32 +2,45 @@
 //
 // WindowShuffle keeps the window of the next `width` samples (decreasing length) in the
 // registers of `width` lanes; RandomizedBestFit ranks the cells a sample fits in by one 64-bit
-// key (remaining capacity, then sample count, then index: smaller = fuller, fewer, lower) and
-// finds the r-th smallest with r+1 warp-wide minimum passes over per-warp cell tables in
-// shared memory.  Random words: Philox(h, 0, trial, 4) for the shuffle, (h, 0, trial, 5) for
-// the fit, h = position of the sample in the emitted order.
+// key (remaining capacity, then sample count, then index: smaller = fuller, fewer, lower).
+// Random words: Philox(h, 0, trial, 4) for the shuffle, (h, 0, trial, 5) for the fit, h = position
+// of the sample in the emitted order.
+//
+// A trial is a chain of N steps, so its latency is what counts.  The warp keeps the keys of the cells sorted: the cells a
+// sample fits in are the keys from (length, 0, 0) on, the r-th of them is taken out, and its smaller new key goes in front of
+// those it passes, which move up by one.  Up to 512 cells a lane holds E consecutive keys in registers (a position is one
+// warp-wide sum of compares, the move one shuffle: 600 cycles a sample at 240 cells); beyond, the keys lie in shared memory
+// (two searches of two ballots: 1100 cycles).  Ranking by r + 1 passes over all cells took 4400.  What does not depend on the
+// fit runs 32 samples at a time: a lane draws the random words of its sample, then the shuffle emits the 32 samples.
 #include "rp_common.cuh"
 
 #define SEED_WARPS 4
 
-// Warp minimum of 64-bit keys with two reduction instructions: the smallest high word, then the
-// smallest low word among the lanes that hold it.
-__device__ __forceinline__ u64 warp_min_u64(u64 v)
+// Keys sorted in blocks of 2^lb: block x of the 32 starts at x * (2^lb + 1), so that the last keys of all blocks lie in
+// different banks.  Unused places hold ~0.
+__device__ __forceinline__ int seed_at(int x, int lb) { return x + (x >> lb); }
+
+// Number of keys below v; `top` is the last key of this lane's block.
+__device__ __forceinline__ int seed_below(const u64 *keys, int lb, u64 top, u64 v, int lane)
 {
-    const u32 hi = (u32)(v >> 32), lo = (u32)v;
-    const u32 mh = __reduce_min_sync(0xffffffffu, hi);
-    const u32 ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : 0xffffffffu);
-    return ((u64)mh << 32) | ml;
+    const int w = __popc(__ballot_sync(0xffffffffu, top < v)), B = 1 << lb;
+    if (w == 32) return 32 << lb;
+    int n = w << lb;
+    for (int e0 = 0; e0 < B; e0 += 32)
+        n += __popc(__ballot_sync(0xffffffffu, e0 + lane < B && keys[(w << lb) + w + min(e0 + lane, B - 1)] < v));
+    return n;
 }
 
+// E > 0: E keys a lane in registers (K <= 32 * E); E = 0: in shared memory, blocks of 2^lb.
+template <int E>
 __global__ void __launch_bounds__(SEED_WARPS * 32)
 k_seed_trials(const int *__restrict__ t, const int *__restrict__ order, const int *__restrict__ seed_layout, RpDims dm,
-              int width, u32 key0, u32 key1, int Ppop, int *__restrict__ layouts, int *__restrict__ ok)
+              int width, int lb, u32 key0, u32 key1, int Ppop, int *__restrict__ layouts, int *__restrict__ ok)
 {
-    extern __shared__ int sm[];
+    extern __shared__ __align__(16) u64 seed_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int *fill = sm + (size_t)warp * 2 * dm.K;        // tokens per cell
-    int *cnt = fill + dm.K;                          // samples per cell
+    const int places = (32 << lb) + 32;
+    u64 *keys = seed_smem + (size_t)warp * places;
     const int j = blockIdx.x * SEED_WARPS + warp;
     if (j >= Ppop) return;
     int *lay = layouts + (size_t)j * dm.N;
@@ -36,51 +49,96 @@ k_seed_trials(const int *__restrict__ t, const int *__restrict__ order, const in
         if (lane == 0) ok[0] = 1;
         return;
     }
-    for (int c = lane; c < dm.K; c += 32) { fill[c] = 0; cnt[c] = 0; }
+    u64 v[E ? E : 1];                                // keys of places lane * E .. + E-1, unused places ~0
+#pragma unroll
+    for (int e = 0; e < (E ? E : 1); ++e) v[e] = ~0ull;
+    if (E == 0) for (int x = lane; x < places; x += 32) keys[x] = ~0ull;
     __syncwarp();
-    int win = -1, nwin = 0, next = 0;                // lane x < nwin holds the x-th sample of the window
+    const int last = (lane << lb) + lane + (1 << lb) - 1;        // last key of this lane's block
+    int win = lane < dm.N ? order[lane] : -1;        // lane x < width: the x-th sample of the window
     bool good = true;
-    for (int h = 0; h < dm.N; ++h) {
-        while (nwin < width && next < dm.N) {        // refill (one sample per step after the start)
-            const int s_new = order[next];
-            if (lane == nwin) win = s_new;
-            ++nwin; ++next;
+    for (int h0 = 0; h0 < dm.N && good; h0 += 32) {
+        const int nb = min(32, dm.N - h0), h = h0 + lane;
+        const int ahead = width + h < dm.N ? order[width + h] : -1;      // enters the window after step h
+        // the window holds min(width, N - h) samples at step h
+        const int pos = rp_pick(rp_philox((u32)h, 0u, (u32)j, 4u, key0, key1).x, min(width, dm.N - h));
+        const u32 xf = rp_philox((u32)h, 0u, (u32)j, 5u, key0, key1).x;
+        int em = 0;                                  // the emitted sample of position h0 + lane
+#pragma unroll 4
+        for (int u = 0; u < nb; ++u) {
+            const int at = __shfl_sync(0xffffffffu, pos, u), in = __shfl_sync(0xffffffffu, ahead, u);
+            const int s = __shfl_sync(0xffffffffu, win, at), up = __shfl_down_sync(0xffffffffu, win, 1);
+            if (lane >= at) win = lane == width - 1 ? in : up;           // close the gap, order kept
+            if (lane == u) em = s;
         }
-        const uint4 xs = rp_philox((u32)h, 0u, (u32)j, 4u, key0, key1);
-        const int pos = rp_pick(xs.x, nwin);
-        const int s = __shfl_sync(0xffffffffu, win, pos);
-        const int up = __shfl_down_sync(0xffffffffu, win, 1);
-        if (lane >= pos && lane < nwin - 1) win = up;        // close the gap, order kept
-        --nwin;
-        const int ts = t[s];
-        int b;
-        if (h < dm.K) b = h;
-        else {
-            // feasible cells, ranked by (remaining capacity, count, index)
-            int nc = 0;
-            for (int c0 = 0; c0 < dm.K; c0 += 32) {
-                const int c = c0 + lane;
-                nc += __popc(__ballot_sync(0xffffffffu, c < dm.K && fill[c] + ts <= dm.C));
-            }
-            if (nc == 0) { good = false; break; }
-            const uint4 xf = rp_philox((u32)h, 0u, (u32)j, 5u, key0, key1);
-            const int r = rp_pick(xf.x, nc < width ? nc : width);
-            u64 prev = 0;                            // keys are >= 1: (.., index + 1)
-            for (int round = 0; round <= r; ++round) {
-                u64 best = ~0ull;
-                for (int c = lane; c < dm.K; c += 32) {
-                    const int f = fill[c];
-                    if (f + ts > dm.C) continue;
-                    const u64 key = ((u64)(u32)(dm.C - f) << 40) | ((u64)(u32)cnt[c] << 20) | (u64)(u32)(c + 1);
-                    if (key > prev && key < best) best = key;
+        const int len = lane < nb ? t[em] : 0;
+        int place = 0;
+        for (int u = 0; u < nb; ++u) {
+            const u64 ts = (u64)(u32)__shfl_sync(0xffffffffu, len, u) << 40;
+            const u32 x = __shfl_sync(0xffffffffu, xf, u);
+            u64 key;
+            int from;                                // place the new key comes from
+            if (E > 0) {
+                if (h0 + u < dm.K) {
+                    from = h0 + u;                   // cell h opens
+                    key = (((u64)(u32)dm.C << 40) - ts) | (1ull << 20) | (u64)(u32)(from + 1);
+                } else {
+                    int n = 0;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) n += v[e] < ts;
+                    const int p0 = __reduce_add_sync(0xffffffffu, n), nc = dm.K - p0;        // feasible cells
+                    if (nc == 0) { good = false; break; }
+                    from = p0 + rp_pick(x, nc < width ? nc : width);
+                    u64 m[E ? E : 1];                            // key number from % E of every lane by halving
+#pragma unroll
+                    for (int e = 0; e < E; ++e) m[e] = v[e];
+#pragma unroll
+                    for (int half = E / 2; half; half /= 2)
+#pragma unroll
+                        for (int e = 0; e < half; ++e) m[e] = (from & half) ? m[e + half] : m[e];
+                    key = __shfl_sync(0xffffffffu, m[0], from / (E ? E : 1)) - ts + (1ull << 20);
                 }
-                prev = warp_min_u64(best);
+                int n = 0;
+#pragma unroll
+                for (int e = 0; e < E; ++e) n += v[e] < key;
+                const int to = __reduce_add_sync(0xffffffffu, n) - lane * E, top = from - lane * E;
+                // keys to .. from-1 move up by one
+                const u64 below = __shfl_up_sync(0xffffffffu, v[E ? E - 1 : 0], 1);
+#pragma unroll
+                for (int e = E - 1; e >= 0; --e) {
+                    if (e > to && e <= top) v[e] = e ? v[e ? e - 1 : 0] : below;
+                    if (e == to) v[e] = key;
+                }
+            } else {
+                const u64 top = keys[last];
+                if (h0 + u < dm.K) {
+                    from = h0 + u;
+                    key = (((u64)(u32)dm.C << 40) - ts) | (1ull << 20) | (u64)(u32)(from + 1);
+                } else {
+                    const int p0 = seed_below(keys, lb, top, ts, lane), nc = dm.K - p0;
+                    if (nc == 0) { good = false; break; }
+                    from = p0 + rp_pick(x, nc < width ? nc : width);
+                    key = keys[seed_at(from, lb)] - ts + (1ull << 20);
+                }
+                const int to = seed_below(keys, lb, top, key, lane);
+                __syncwarp();
+                for (int hi = from; hi > to; hi -= 128) {        // from the top
+                    u64 w[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) { const int y = hi - 32 * e - lane; if (y > to) w[e] = keys[seed_at(y - 1, lb)]; }
+                    __syncwarp();
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) { const int y = hi - 32 * e - lane; if (y > to) keys[seed_at(y, lb)] = w[e]; }
+                    __syncwarp();
+                }
+                if (lane == 0) keys[seed_at(to, lb)] = key;
+                __syncwarp();
             }
-            b = (int)(prev & 0xFFFFFu) - 1;
+            if (lane == u) place = (int)(key & 0xFFFFFu) - 1;
         }
-        if (lane == 0) { fill[b] += ts; cnt[b] += 1; lay[s] = b; }
-        __syncwarp();
+        if (lane < nb && good) lay[em] = place;
     }
+    __syncwarp();
     if (!good) for (int i = lane; i < dm.N; i += 32) lay[i] = seed_layout[i];
     if (lane == 0) ok[j] = good ? 1 : 0;
 }
@@ -88,13 +146,15 @@ k_seed_trials(const int *__restrict__ t, const int *__restrict__ order, const in
 int rp_launch_seed_trials(rp_ctx *c, int width, int *layouts, int *ok)
 {
     const RpDims &dm = c->dm;
-    const size_t smem = sizeof(int) * (size_t)SEED_WARPS * 2 * dm.K;
+    int lb = 0;
+    while ((32 << lb) < dm.K) ++lb;
+    const size_t smem = lb > 4 ? sizeof(u64) * (size_t)SEED_WARPS * ((32 << lb) + 32) : 0;
     if (smem > 200 * 1024) return RP_ERR_RANGE;
-    if (smem > 32 * 1024)
-        RP_CUDA(cudaFuncSetAttribute(k_seed_trials, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_seed_trials<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    auto fn = lb > 4 ? k_seed_trials<0> : lb == 4 ? k_seed_trials<16> : lb == 3 ? k_seed_trials<8> : lb == 2 ? k_seed_trials<4> : k_seed_trials<2>;
     const int grid = (c->Ppop + SEED_WARPS - 1) / SEED_WARPS;
-    k_seed_trials<<<grid, SEED_WARPS * 32, smem, c->stream>>>(c->d_t, c->d_order, c->d_seed_layout, dm, width,
-                                                             (u32)c->cfg.seed, (u32)(c->cfg.seed >> 32), c->Ppop, layouts, ok);
+    fn<<<grid, SEED_WARPS * 32, smem, c->stream>>>(c->d_t, c->d_order, c->d_seed_layout, dm, width, lb,
+                                                  (u32)c->cfg.seed, (u32)(c->cfg.seed >> 32), c->Ppop, layouts, ok);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     return RP_OK;

@@ -1176,3 +1176,38 @@ def test_packing_at_the_edges_of_its_forms(N, D, min_rows, cap, longest):
     assert rp.rp_pack_rows(ctx) == (R, cert)
     assert (rp.rp_debug_dump(ctx, "SEED_LAYOUT", (N,), np.int32) == seed).all()
     rp.rp_destroy(ctx)
+
+
+# Cells on both sides of the numbers the sorted keys of a trial are kept for (64, 256, 512 in registers, more in shared memory),
+# several and one slot per row-shard beyond one a thread, and pair counts of the distances in 32, 16 and 8 bits, whole and in blocks.
+@pytest.mark.parametrize("N,D,min_rows,edp,longest,full", [
+    (200, 8, 8, None, 60, 0), (200, 5, 13, [0, 0, 1, 1, 1], 60, 0), (700, 8, 32, [0, 1] * 4, 60, 0), (700, 1, 257, None, 60, 0),
+    (1300, 4, 128, [0, 0, 0, 0], 60, 0), (1300, 3, 171, [0, 1, 1], 60, 0), (2300, 4, 300, [0, 0, 1, 1], 60, 0),
+    (3150, 8, 20, None, 1, 150), (3240, 10, 25, [0, 1] * 5, 1, 240)])
+def test_candidate_stages_at_the_edges_of_their_forms(N, D, min_rows, edp, longest, full):
+    rng = np.random.default_rng(N + D)
+    cap, pop, L, E, k = 600, 4, 2, 8, 2
+    t = rng.integers(1, longest + 1, N).astype(np.int32)
+    t[:full] = cap
+    a = np.stack([[rng.multinomial(k * int(ti), np.full(E, 1 / E)) for _ in range(L)] for ti in t]).astype(np.int32)
+    ref_pi, _ = oracle.lpt(oracle.aggregate(a), 2)
+    q = oracle.project(a, ref_pi, 2)
+    R, cert, seed = oracle.pack_ffd(t, cap, D, min_rows)
+    ctx = rp.rp_window_load(t, a, top_k=k, token_cap=cap, dp_width=D, ep_width=2, pop_size=pop, min_rows=min_rows, edp_of_dp=edp, seed=5)
+    rp.rp_debug_set_trace(ctx, True)
+    rp.rp_place_experts(ctx)
+    assert rp.rp_pack_rows(ctx) == (R, cert)
+    lays, ok = oracle.seed_trials(t, seed, R, cap, D, pop, 5, 5)
+    assert rp.rp_seed_population(ctx, 5) == int(ok.sum())
+    assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == lays).all()
+    pairs = oracle.edp_pair(q, lays, R, D, 4, 5, edp)
+    rp.rp_pair_population(ctx, 4)
+    assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == pairs).all()
+    sc = oracle.eval_layouts(t, q, pairs, R, cap, D, edp)["score"]
+    want = oracle.select_population(t, q, pairs, sc, R, cap, D, k, 9, 1 << 16, 5, edp, want_dist=True)
+    nd, order = rp.rp_select_population(ctx, 9, 1 << 16)
+    assert nd == want["n_distinct"] and (order == want["order"]).all()
+    dist = rp.rp_debug_dump(ctx, "SELECT_DIST", (pop, pop), np.int64)
+    reps = sorted(set(order[:nd].tolist()))
+    assert (dist[np.ix_(reps, reps)] == want["dist"][np.ix_(reps, reps)]).all()
+    rp.rp_destroy(ctx)
