@@ -17,14 +17,17 @@
 //               (distance to the nearest selected one) - ((eta_q16 * gap) >> 16), gap =
 //               floor((S0 - S0*) * 2^20 / S0*), ties by lower index.
 #include "rp_common.cuh"
+#include <algorithm>
 
 #define SEL_THREADS 256
-#define SEL_TABLE 4096
+#define SEL_WARPS (SEL_THREADS / 32)
 
 struct SelBuf {                 // per-member arrays in global memory
     int *lay;                   // [P][N] layouts
     int *canon;                 // [P][N] signatures
     u64 *hash;                  // [P]
+    u32 *lab;                   // [P][N] cell | row << 16
+    int *big;                   // [P][2] samples of the largest cell, of the largest row
     int *clist, *cstart;        // [P][N], [P][K+1] samples grouped by cell
     int *rlist, *rstart;        // [P][N], [P][R+1] samples grouped by row
     i64 *pc, *pr;               // [P] pairs together in a cell / in a row
@@ -67,7 +70,8 @@ k_sel_prepare(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const int *_
     int *ng = rcount + R + 1;                      // [G] slots per shard
     __shared__ u64 hsum;
     __shared__ i64 pcs, prs;
-    const int tid = threadIdx.x;
+    __shared__ int big_s[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int j = blockIdx.x;
     const int *lay = B.lay + (size_t)j * N;
     const char *blob = blobs + (size_t)anc[j] * bl.bytes;
@@ -80,22 +84,25 @@ k_sel_prepare(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const int *_
     for (int r = tid; r <= R; r += SEL_THREADS) rcount[r] = 0;
     for (int r = tid; r < R; r += SEL_THREADS) rname[r] = N;
     for (int g = tid; g < G; g += SEL_THREADS) ng[g] = 0;
-    for (int x = tid; x < n_proj * R; x += SEL_THREADS) ph[x] = 0;
-    if (tid == 0) { hsum = 0; pcs = 0; prs = 0; }
+    if (tid == 0) { hsum = 0; pcs = 0; prs = 0; big_s[0] = 0; big_s[1] = 0; }
     __syncthreads();
     for (int i = tid; i < N; i += SEL_THREADS) {
-        const int c = lay[i];
+        const int c = lay[i], r = c / D;
+        B.lab[(size_t)j * N + i] = (u32)c | ((u32)r << 16);
         atomicMin(&name[c], i);
         atomicAdd(&ccount[c + 1], 1);
-        atomicAdd(&rcount[c / D + 1], 1);
+        atomicAdd(&rcount[r + 1], 1);
     }
     for (int d = tid; d < D; d += SEL_THREADS) atomicAdd(&ng[g_of_cell[d]], 1);
     __syncthreads();
     for (int c = tid; c < K; c += SEL_THREADS) atomicMin(&rname[c / D], name[c]);
     {   // pairs together, from the group sizes
         i64 a = 0, b = 0;
-        for (int c = tid; c < K; c += SEL_THREADS) { const i64 n = ccount[c + 1]; a += n * (n - 1) / 2; }
-        for (int r = tid; r < R; r += SEL_THREADS) { const i64 n = rcount[r + 1]; b += n * (n - 1) / 2; }
+        int ma = 0, mb = 0;
+        for (int c = tid; c < K; c += SEL_THREADS) { const int n = ccount[c + 1]; a += (i64)n * (n - 1) / 2; ma = max(ma, n); }
+        for (int r = tid; r < R; r += SEL_THREADS) { const int n = rcount[r + 1]; b += (i64)n * (n - 1) / 2; mb = max(mb, n); }
+        ma = __reduce_max_sync(0xffffffffu, ma); mb = __reduce_max_sync(0xffffffffu, mb);
+        if (lane == 0) { atomicMax(&big_s[0], ma); atomicMax(&big_s[1], mb); }
         if (a) atomicAdd((u64 *)&pcs, (u64)a);
         if (b) atomicAdd((u64 *)&prs, (u64)b);
     }
@@ -115,11 +122,18 @@ k_sel_prepare(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const int *_
         for (int r2 = 0; r2 < R; ++r2) pos += (rname[r2] < rname[r]);
         new_r[r] = pos;
     }
-    if (tid == 0) {              // exclusive starts of the groups
+    if (warp < 2) {              // starts of the groups: prefix sums of the sizes (one place on), a warp for cells, one for rows
+        int *count = warp ? rcount : ccount;
+        const int n = warp ? R : K;
         int run = 0;
-        for (int c = 0; c <= K; ++c) { run += ccount[c]; ccount[c] = run; }
-        run = 0;
-        for (int r = 0; r <= R; ++r) { run += rcount[r]; rcount[r] = run; }
+        for (int x0 = 0; x0 <= n; x0 += 32) {
+            const int x = x0 + lane;
+            int v = x <= n ? count[x] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += y; }
+            if (x <= n) count[x] = run + v;
+            run += __shfl_sync(0xffffffffu, v, 31);
+        }
     }
     __syncthreads();
     for (int c = tid; c <= K; c += SEL_THREADS) B.cstart[(size_t)j * (K + 1) + c] = ccount[c];
@@ -141,23 +155,40 @@ k_sel_prepare(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const int *_
         B.clist[(size_t)j * N + atomicAdd(&ccount[c], 1)] = i;
         B.rlist[(size_t)j * N + atomicAdd(&rcount[c / D], 1)] = i;
     }
-    // row features -> projections
+    // row features -> projections: one warp per row, lanes over the features, eight projections summed in registers at a time
+    // (64-bit shared-memory atomics of all lanes on one row's sums took most of this kernel: 256 members of 2048 samples and 24
+    // layers 500 us, now 84)
     const i64 CD = (i64)dm.C * D;
-    for (int x = tid; x < R * F; x += SEL_THREADS) {
-        const int r = x / F, f = x % F;
-        i64 h;
-        if (f < 2) {
-            if (f == 0) { i64 s = 0; for (int d = 0; d < D; ++d) s += T[r * D + d]; h = (s << 16) / CD; }
-            else { u64 s = 0; for (int d = 0; d < D; ++d) s += Q[r * D + d]; h = (i64)((s << 16) / ((u64)CD * (u64)dm.C)); }
-        } else {
-            const int g = (f - 2) / L, l = (f - 2) % L;
-            const int *wr = W + ((size_t)r * G + g) * dm.LP + (size_t)l * P;
-            int m = 0;
-            for (int p = 0; p < P; ++p) m = max(m, wr[p]);
-            h = ((i64)m << 16) / ((i64)dm.k * dm.C * ng[g]);
+    for (int r = warp; r < R; r += SEL_WARPS) {
+        for (int k0 = 0; k0 < n_proj; k0 += 8) {
+            i64 acc[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[k] = 0;
+            for (int f = lane; f < F; f += 32) {
+                i64 h;
+                if (f < 2) {
+                    if (f == 0) { i64 s = 0; for (int d = 0; d < D; ++d) s += T[r * D + d]; h = (s << 16) / CD; }
+                    else { u64 s = 0; for (int d = 0; d < D; ++d) s += Q[r * D + d]; h = (i64)((s << 16) / ((u64)CD * (u64)dm.C)); }
+                } else {
+                    const int g = (f - 2) / L, l = (f - 2) % L;
+                    const int *wr = W + ((size_t)r * G + g) * dm.LP + (size_t)l * P;
+                    int m = 0;
+                    if (P % 4 == 0) {
+                        for (int p = 0; p < P; p += 4) { const int4 w = *(const int4 *)(wr + p); m = max(max(m, max(w.x, w.y)), max(w.z, w.w)); }
+                    } else {
+                        for (int p = 0; p < P; ++p) m = max(m, wr[p]);
+                    }
+                    h = ((i64)m << 16) / ((i64)dm.k * dm.C * ng[g]);
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) if (k0 + k < n_proj) acc[k] += sgn[(size_t)(k0 + k) * F + f] ? -h : h;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                for (int o = 16; o; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+                if (lane == 0 && k0 + k < n_proj) ph[(k0 + k) * R + r] = acc[k];
+            }
         }
-        for (int k = 0; k < n_proj; ++k)
-            atomicAdd((unsigned long long *)&ph[k * R + r], (unsigned long long)(sgn[k * F + f] ? -h : h));
     }
     __syncthreads();
     for (int x = tid; x < n_proj * R; x += SEL_THREADS) {        // sort each projection by counting
@@ -167,7 +198,7 @@ k_sel_prepare(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const int *_
         for (int r2 = 0; r2 < R; ++r2) { const i64 o = ph[k * R + r2]; pos += (o < v) || (o == v && r2 < r); }
         B.phi[((size_t)j * n_proj + k) * R + pos] = v;
     }
-    if (tid == 0) { B.hash[j] = hsum; B.pc[j] = pcs; B.pr[j] = prs; }
+    if (tid == 0) { B.hash[j] = hsum; B.pc[j] = pcs; B.pr[j] = prs; B.big[2 * j] = big_s[0]; B.big[2 * j + 1] = big_s[1]; }
 }
 
 // ---- CanonicalMap: is member j the representative of its class? ---------------------------------
@@ -181,119 +212,175 @@ k_sel_map(int N, int Ppop, const int *__restrict__ canon, const u64 *__restrict_
     __syncthreads();
     const u64 hj = hash[j];
     const i64 a0 = score[3 * (size_t)j], a1 = score[3 * (size_t)j + 1], a2 = score[3 * (size_t)j + 2];
-    for (int o = threadIdx.x; o < Ppop; o += SEL_THREADS) {
-        if (o == j || hash[o] != hj) continue;
-        bool same = true;
-        for (int i = 0; i < N && same; ++i) same = canon[(size_t)j * N + i] == canon[(size_t)o * N + i];
-        if (!same) continue;
-        const i64 b0 = score[3 * (size_t)o], b1 = score[3 * (size_t)o + 1], b2 = score[3 * (size_t)o + 2];
-        if (rp_lex_less(b0, b1, b2, a0, a1, a2) || (!rp_lex_less(a0, a1, a2, b0, b1, b2) && o < j)) beaten = 1;
+    const int lane = threadIdx.x & 31;
+    for (int o0 = threadIdx.x - lane; o0 < Ppop; o0 += SEL_THREADS) {
+        const int mine = o0 + lane;
+        for (unsigned todo = __ballot_sync(0xffffffffu, mine < Ppop && mine != j && hash[min(mine, Ppop - 1)] == hj); todo; todo &= todo - 1) {
+            const int o = o0 + __ffs(todo) - 1;        // the whole warp compares the two signatures
+            bool same = true;
+            for (int i = lane; i < N && same; i += 32) same = canon[(size_t)j * N + i] == canon[(size_t)o * N + i];
+            if (!__all_sync(0xffffffffu, same)) continue;
+            const i64 b0 = score[3 * (size_t)o], b1 = score[3 * (size_t)o + 1], b2 = score[3 * (size_t)o + 2];
+            if (rp_lex_less(b0, b1, b2, a0, a1, a2) || (!rp_lex_less(a0, a1, a2, b0, b1, b2) && o < j)) beaten = 1;
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) rep[j] = !beaten;
 }
 
 // ---- plan distances between representatives ------------------------------------------------------
-// Pairs together in both labelings: every pair of one group of a is looked up in b.
-__device__ __forceinline__ i64 sel_both(const int *__restrict__ list, const int *__restrict__ start, int n_groups,
-                                        const int *__restrict__ lb, int div_b, int tid)
+// Pairs together in a group of both plans = sum over (group of a, group of b) of C(count, 2).  Every sample adds one to the
+// count of its pair of groups in shared memory; what the atomic returns is the number of samples before it there, and these
+// sum up to C(count, 2): no pass over the table.  Clearing stores a zero at the same places.  Bound by the shared-memory
+// atomics, two a sample (cells and rows): 32640 pairs of plans of 2048 samples in 240 cells 0.27 ms; looking every pair of a
+// cell's samples up in the other plan took 4.15 ms.
+//
+// Counts are as narrow as the largest group of a allows when the whole table fits only so (8 bits up to 255 samples); where
+// no width fits, the groups of a are taken in blocks, whose samples are contiguous in a's grouped list.
+#define SEL_CHUNK 8             // plans b per work item
+struct SelTab { u32 *tab; int n, lbits, block; };      // n groups; counts of 2^lbits bits; groups of a per pass
+
+__device__ __forceinline__ SelTab sel_table(u32 *tab, size_t bytes, int n, int big)
 {
-    i64 both = 0;
-    for (int g = 0; g < n_groups; ++g) {
-        const int s = start[g], n = start[g + 1] - s;
-        const int np = n * (n - 1) / 2;
-        for (int x = tid; x < np; x += SEL_THREADS) {
-            // x-th pair (u < v) of the group
-            int v = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)x)) * 0.5f);
-            while (v * (v - 1) / 2 > x) --v;
-            while ((v + 1) * v / 2 <= x) ++v;
-            const int u = x - v * (v - 1) / 2;
-            both += (lb[list[s + u]] / div_b == lb[list[s + v]] / div_b);
-        }
-    }
-    return both;
+    SelTab t = { tab, n, 5, n };
+    const size_t bits = bytes * 8, all = (size_t)n * n;
+    if (all * 32 > bits && big <= 65535) t.lbits = 4;
+    if (t.lbits == 4 && all * 16 > bits && big <= 255) t.lbits = 3;
+    if ((all << t.lbits) > bits) t.block = (int)((bits >> t.lbits) / n);
+    return t;
 }
 
-__global__ void __launch_bounds__(SEL_THREADS)
-k_sel_dist(RpDims dm, int Ppop, int n_proj, const int *__restrict__ rep, SelBuf B, i64 *__restrict__ dist, int cells_by_table)
+__device__ __forceinline__ u32 sel_add(const SelTab &t, int x)
 {
-    const int a = blockIdx.x, b = blockIdx.y;
-    if (b <= a) { if (a == b && threadIdx.x == 0) dist[(size_t)a * Ppop + a] = 0; return; }
-    if (!rep[a] || !rep[b]) return;
-    __shared__ i64 acc[3];
-    __shared__ int tab[SEL_TABLE];                 // row-by-row contingency counts when R*R fits
-    extern __shared__ int ctab[];                  // cell-by-cell contingency counts when K*K ints fit (cells_by_table)
-    const int tid = threadIdx.x;
-    const int N = dm.N, K = dm.K, R = dm.R, D = dm.D;
-    const bool rows_by_table = R * R <= SEL_TABLE;
-    if (tid < 3) acc[tid] = 0;
-    if (rows_by_table) for (int x = tid; x < R * R; x += SEL_THREADS) tab[x] = 0;
-    if (cells_by_table) for (int x = tid; x < K * K; x += SEL_THREADS) ctab[x] = 0;
-    __syncthreads();
-    const int *la = B.lay + (size_t)a * N, *lb = B.lay + (size_t)b * N;
-    i64 bc = 0;
-    if (cells_by_table) {
-        // pairs in the same cell of both plans = sum over (cell of a, cell of b) of C(count, 2): N counts
-        // instead of one look-up per pair of a cell's samples (cells of hundreds of samples)
-        for (int i = tid; i < N; i += SEL_THREADS) atomicAdd(&ctab[la[i] * K + lb[i]], 1);
+    const int per = 5 - t.lbits, sh = (x & ((1 << per) - 1)) << t.lbits;
+    const u32 old = atomicAdd(&t.tab[x >> per], 1u << sh);
+    return (old >> sh) & (0xffffffffu >> (32 - (1 << t.lbits)));
+}
+
+__device__ __forceinline__ void sel_clear(const SelTab &t, int x) { t.tab[x >> (5 - t.lbits)] = 0; }
+
+// The same in blocks of a's groups; SH = 0 for cells, 16 for rows.
+template <typename SUM, int SH>
+__device__ __forceinline__ SUM sel_blocks(const SelTab &t, const int *list, const int *start, const u32 *la, const u32 *lb, int tid)
+{
+    SUM sum = 0;
+    for (int g0 = 0; g0 < t.n; g0 += t.block) {
+        const int x0 = start[g0], x1 = start[min(t.n, g0 + t.block)];
+        for (int pass = 0; pass < 2; ++pass) {
+            for (int x = x0 + tid; x < x1; x += SEL_THREADS) {
+                const int i = list[x];
+                const int at = ((int)((la[i] >> SH) & 0xffffu) - g0) * t.n + (int)((lb[i] >> SH) & 0xffffu);
+                if (pass == 0) sum += sel_add(t, at); else sel_clear(t, at);
+            }
+            __syncthreads();
+        }
+    }
+    return sum;
+}
+
+// SUM: 32 bits hold the pairs of up to 65535 samples.
+template <typename SUM>
+__global__ void __launch_bounds__(SEL_THREADS)
+k_sel_dist(RpDims dm, int Ppop, int n_proj, const int *__restrict__ rep, SelBuf B, i64 *__restrict__ dist, int ctab_bytes, int rtab_bytes)
+{
+    extern __shared__ __align__(16) u32 sel_tabs[];
+    __shared__ u64 acc[SEL_CHUNK][3];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int N = dm.N, K = dm.K, R = dm.R, F = 2 + dm.G * dm.L;
+    for (int x = tid; x < (ctab_bytes + rtab_bytes) / 4; x += SEL_THREADS) sel_tabs[x] = 0;
+    const int chunks = (Ppop + SEL_CHUNK - 1) / SEL_CHUNK;
+    for (size_t item = blockIdx.x; item < (size_t)chunks * Ppop; item += gridDim.x) {
+        const int a = (int)(item % Ppop), b0 = (int)(item / Ppop) * SEL_CHUNK;
+        if (b0 + SEL_CHUNK - 1 <= a || !rep[a]) continue;
+        if (tid < 3 * SEL_CHUNK) acc[tid / 3][tid % 3] = 0;
         __syncthreads();
-        for (int x = tid; x < K * K; x += SEL_THREADS) { const i64 n = ctab[x]; bc += n * (n - 1) / 2; }
-    } else {
-        bc = sel_both(B.clist + (size_t)a * N, B.cstart + (size_t)a * (K + 1), K, lb, 1, tid);
-    }
-    i64 br = 0;
-    if (rows_by_table) {
-        // pairs in the same row of both plans = sum over (row of a, row of b) of C(count, 2)
-        for (int i = tid; i < N; i += SEL_THREADS) atomicAdd(&tab[(la[i] / D) * R + lb[i] / D], 1);
+        const SelTab ct = sel_table(sel_tabs, ctab_bytes, K, B.big[2 * a]), rt = sel_table(sel_tabs + ctab_bytes / 4, rtab_bytes, R, B.big[2 * a + 1]);
+        const bool whole = ct.block == K && rt.block == R;
+        const u32 *la = B.lab + (size_t)a * N;
+        const i64 *pa = B.phi + (size_t)a * n_proj * R;
+        for (int u = 0; u < SEL_CHUNK; ++u) {
+            const int b = b0 + u;
+            if (b <= a || b >= Ppop || !rep[b]) continue;
+            const u32 *lb = B.lab + (size_t)b * N;
+            SUM bc = 0, br = 0;
+            if (whole) {
+#pragma unroll 4
+                for (int i = tid; i < N; i += SEL_THREADS) {
+                    const u32 ga = la[i], gb = lb[i];
+                    bc += sel_add(ct, (int)(ga & 0xffffu) * K + (int)(gb & 0xffffu));
+                    br += sel_add(rt, (int)(ga >> 16) * R + (int)(gb >> 16));
+                }
+                __syncthreads();
+#pragma unroll 4
+                for (int i = tid; i < N; i += SEL_THREADS) {
+                    const u32 ga = la[i], gb = lb[i];
+                    sel_clear(ct, (int)(ga & 0xffffu) * K + (int)(gb & 0xffffu));
+                    sel_clear(rt, (int)(ga >> 16) * R + (int)(gb >> 16));
+                }
+            } else {
+                bc = sel_blocks<SUM, 0>(ct, B.clist + (size_t)a * N, B.cstart + (size_t)a * (K + 1), la, lb, tid);
+                br = sel_blocks<SUM, 16>(rt, B.rlist + (size_t)a * N, B.rstart + (size_t)a * (R + 1), la, lb, tid);
+            }
+            const i64 *pb = B.phi + (size_t)b * n_proj * R;
+            if (tid - lane < n_proj * R) {                       // sketch: the warps that have part of it
+                i64 sw = 0;
+                for (int x = tid; x < n_proj * R; x += SEL_THREADS) { const i64 d = pa[x] - pb[x]; sw += d < 0 ? -d : d; }
+                for (int o = 16; o; o >>= 1) sw += __shfl_xor_sync(0xffffffffu, sw, o);
+                if (lane == 0) atomicAdd((unsigned long long *)&acc[u][2], (unsigned long long)sw);
+            }
+            if (sizeof(SUM) == 4) {
+                const u32 sc = __reduce_add_sync(0xffffffffu, (u32)bc), sr = __reduce_add_sync(0xffffffffu, (u32)br);
+                bc = sc; br = sr;
+            } else {
+                for (int o = 16; o; o >>= 1) { bc += __shfl_xor_sync(0xffffffffu, bc, o); br += __shfl_xor_sync(0xffffffffu, br, o); }
+            }
+            if (lane == 0) {
+                atomicAdd((unsigned long long *)&acc[u][0], (unsigned long long)bc);
+                atomicAdd((unsigned long long *)&acc[u][1], (unsigned long long)br);
+            }
+            __syncthreads();                                     // tables are clear again
+        }
+        const int b = b0 + tid;
+        if (tid < SEL_CHUNK && b > a && b < Ppop && rep[b]) {
+            const i64 bc = (i64)acc[tid][0], br = (i64)acc[tid][1];
+            const i64 uc = B.pc[a] + B.pc[b] - bc, ur = B.pr[a] + B.pr[b] - br;
+            i64 d = 0;
+            if (uc) d += ((i64)1 << 20) - (bc << 20) / uc;
+            if (ur) d += ((i64)1 << 20) - (br << 20) / ur;
+            d += ((i64)acc[tid][2] * 16) / ((i64)n_proj * R * F);
+            dist[(size_t)a * Ppop + b] = d;
+            dist[(size_t)b * Ppop + a] = d;
+        }
         __syncthreads();
-        for (int x = tid; x < R * R; x += SEL_THREADS) { const i64 n = tab[x]; br += n * (n - 1) / 2; }
-    } else {
-        br = sel_both(B.rlist + (size_t)a * N, B.rstart + (size_t)a * (R + 1), R, lb, D, tid);
-    }
-    i64 sw = 0;
-    const i64 *pa = B.phi + (size_t)a * n_proj * R, *pb = B.phi + (size_t)b * n_proj * R;
-    for (int x = tid; x < n_proj * R; x += SEL_THREADS) { const i64 d = pa[x] - pb[x]; sw += d < 0 ? -d : d; }
-    for (int o = 16; o; o >>= 1) {
-        bc += __shfl_xor_sync(0xffffffffu, bc, o);
-        br += __shfl_xor_sync(0xffffffffu, br, o);
-        sw += __shfl_xor_sync(0xffffffffu, sw, o);
-    }
-    if ((tid & 31) == 0) {
-        atomicAdd((unsigned long long *)&acc[0], (unsigned long long)bc);
-        atomicAdd((unsigned long long *)&acc[1], (unsigned long long)br);
-        atomicAdd((unsigned long long *)&acc[2], (unsigned long long)sw);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        const int F = 2 + dm.G * dm.L;
-        const i64 uc = B.pc[a] + B.pc[b] - acc[0], ur = B.pr[a] + B.pr[b] - acc[1];
-        i64 d = 0;
-        if (uc) d += ((i64)1 << 20) - (acc[0] << 20) / uc;
-        if (ur) d += ((i64)1 << 20) - (acc[1] << 20) / ur;
-        d += (acc[2] * 16) / ((i64)n_proj * R * F);
-        dist[(size_t)a * Ppop + b] = d;
-        dist[(size_t)b * Ppop + a] = d;
     }
 }
 
 // ---- greedy selection (one CTA) -------------------------------------------------------------------
+// One selection after the other: a step is the load of one row of distances (L2), three warp-wide minima, one barrier and the
+// same minima over the warps' results, which every warp works out for itself (256 candidates 164 us; a shuffle tree over
+// triples, a serial pass of one thread and two barriers over 32 warps took 920).
 #define GREEDY_THREADS 1024
+#define GREEDY_SMEM (160 * 1024)        // nearest distances and penalties of the candidates on chip up to this
 struct SelPick { i64 v0, v1, v2; int j; };
 
 __global__ void __launch_bounds__(GREEDY_THREADS)
 k_sel_greedy(int Ppop, const int *__restrict__ rep, const i64 *__restrict__ score, const i64 *__restrict__ dist,
-             i64 eta_q16, i64 *__restrict__ mind, i64 *__restrict__ pen, int *__restrict__ order, int *__restrict__ n_distinct)
+             i64 eta_q16, i64 *mind, i64 *pen, int *__restrict__ order, int *__restrict__ n_distinct)
 {
     __shared__ SelPick red[GREEDY_THREADS / 32];
     __shared__ SelPick pick_s;
     __shared__ int nd_s;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ u64 red_v[2][GREEDY_THREADS / 32];
+    __shared__ int red_j[2][GREEDY_THREADS / 32];
+    extern __shared__ __align__(16) i64 greedy_smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = (int)blockDim.x, nw = nt / 32;
+    if (!mind) { mind = greedy_smem; pen = mind + Ppop; }
     if (tid == 0) nd_s = 0;
     __syncthreads();
     // winner by score (lowest triple, lowest index) and the number of representatives
     SelPick best = { 0x7fffffffffffffffll, 0x7fffffffffffffffll, 0x7fffffffffffffffll, 0x7fffffff };
     int cnt = 0;
-    for (int j = tid; j < Ppop; j += GREEDY_THREADS) {
+    for (int j = tid; j < Ppop; j += nt) {
         if (!rep[j]) continue;
         ++cnt;
         const i64 s0 = score[3 * (size_t)j], s1 = score[3 * (size_t)j + 1], s2 = score[3 * (size_t)j + 2];
@@ -311,7 +398,7 @@ k_sel_greedy(int Ppop, const int *__restrict__ rep, const i64 *__restrict__ scor
         if (lane == 0) red[warp] = b;
         __syncthreads();
         if (tid == 0) {
-            for (int w = 1; w < GREEDY_THREADS / 32; ++w) {
+            for (int w = 1; w < nw; ++w) {
                 const SelPick ot = red[w];
                 if (rp_lex_less(ot.v0, ot.v1, ot.v2, b.v0, b.v1, b.v2) ||
                     (ot.v0 == b.v0 && ot.v1 == b.v1 && ot.v2 == b.v2 && ot.j < b.j)) b = ot;
@@ -324,7 +411,7 @@ k_sel_greedy(int Ppop, const int *__restrict__ rep, const i64 *__restrict__ scor
     const int nd = nd_s;
     const i64 s0 = pick_s.v0;
     int last = pick_s.j;
-    for (int j = tid; j < Ppop; j += GREEDY_THREADS) {
+    for (int j = tid; j < Ppop; j += nt) {
         i64 p = 0;
         if (rep[j] && s0 > 0) {
             const unsigned __int128 gap = ((unsigned __int128)(u64)(score[3 * (size_t)j] - s0) << 20) / (u64)s0;
@@ -336,21 +423,33 @@ k_sel_greedy(int Ppop, const int *__restrict__ rep, const i64 *__restrict__ scor
     __syncthreads();
     for (int n = 0; n < nd; ++n) {
         if (tid == 0) order[n] = last;
-        // negated objective so that the same lexicographic minimum applies: maximise v, lowest index
-        SelPick b = { 0x7fffffffffffffffll, 0, 0, 0x7fffffff };
-        for (int j = tid; j < Ppop; j += GREEDY_THREADS) {
-            if (j == last) mind[j] = -1;
+        // negated objective, as an unsigned number, so that the minimum applies: maximise distance - penalty, lowest index
+        u64 bv = ~0ull;
+        u32 bj = 0xffffffffu;
+        for (int j = tid; j < Ppop; j += nt) {
             i64 m = mind[j];
+            if (j == last) { mind[j] = -1; m = -1; }
             if (m < 0) continue;
-            const i64 d = dist[(size_t)j * Ppop + last];
+            const i64 d = dist[(size_t)last * Ppop + j];
             if (d < m) { m = d; mind[j] = m; }
-            const i64 neg = -(m - pen[j]);
-            if (neg < b.v0 || (neg == b.v0 && j < b.j)) { b.v0 = neg; b.j = j; }
+            const u64 neg = (u64)(pen[j] - m) ^ 0x8000000000000000ull;
+            if (neg < bv) { bv = neg; bj = (u32)j; }
         }
-        reduce_min(b);
-        last = pick_s.j;
+        for (int pass = 0; pass < 2; ++pass) {
+            const u32 hi = __reduce_min_sync(0xffffffffu, (u32)(bv >> 32));
+            const bool in = (u32)(bv >> 32) == hi;
+            const u32 lo = __reduce_min_sync(0xffffffffu, in ? (u32)bv : 0xffffffffu);
+            bj = __reduce_min_sync(0xffffffffu, in && (u32)bv == lo ? bj : 0xffffffffu);
+            bv = ((u64)hi << 32) | lo;
+            if (pass) break;
+            if (lane == 0) { red_v[n & 1][warp] = bv; red_j[n & 1][warp] = (int)bj; }
+            __syncthreads();
+            bv = lane < nw ? red_v[n & 1][lane] : ~0ull;
+            bj = lane < nw ? (u32)red_j[n & 1][lane] : 0xffffffffu;
+        }
+        last = (int)bj;
     }
-    for (int m = nd + tid; m < Ppop; m += GREEDY_THREADS) order[m] = order[m % nd];
+    for (int m = nd + tid; m < Ppop; m += nt) order[m] = order[m % nd];
     if (tid == 0) *n_distinct = nd;
 }
 
@@ -375,9 +474,11 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
     int *rep = nullptr;
     i64 *mind = nullptr, *pen = nullptr;
     B.canon = nullptr; B.hash = nullptr; B.clist = nullptr; B.cstart = nullptr; B.rlist = nullptr; B.rstart = nullptr;
-    B.pc = nullptr; B.pr = nullptr; B.phi = nullptr;
+    B.pc = nullptr; B.pr = nullptr; B.phi = nullptr; B.lab = nullptr; B.big = nullptr;
     int st = dev_alloc(c, &B.canon, P * dm.N);
     if (st == RP_OK) st = dev_alloc(c, &B.hash, P);
+    if (st == RP_OK) st = dev_alloc(c, &B.lab, P * dm.N);
+    if (st == RP_OK) st = dev_alloc(c, &B.big, 2 * P);
     if (st == RP_OK) st = dev_alloc(c, &B.clist, P * dm.N);
     if (st == RP_OK) st = dev_alloc(c, &B.cstart, P * (dm.K + 1));
     if (st == RP_OK) st = dev_alloc(c, &B.rlist, P * dm.N);
@@ -387,8 +488,9 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
     if (st == RP_OK) st = dev_alloc(c, &B.phi, P * n_proj * dm.R);
     if (st == RP_OK) st = dev_alloc(c, &sgn, (size_t)F * n_proj);
     if (st == RP_OK) st = dev_alloc(c, &rep, P);
-    if (st == RP_OK) st = dev_alloc(c, &mind, P);
-    if (st == RP_OK) st = dev_alloc(c, &pen, P);
+    const bool greedy_smem = 2 * sizeof(i64) * P <= GREEDY_SMEM;
+    if (st == RP_OK && !greedy_smem) st = dev_alloc(c, &mind, P);
+    if (st == RP_OK && !greedy_smem) st = dev_alloc(c, &pen, P);
     const size_t smem = sizeof(i64) * (size_t)n_proj * dm.R + sizeof(int) * ((size_t)3 * dm.K + 3 * dm.R + dm.G + 2) + 16;
     if (st == RP_OK && smem > 200 * 1024) st = RP_ERR_RANGE;
     cudaError_t e = cudaSuccess;
@@ -402,15 +504,23 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
             e = cudaMemsetAsync(dist, 0, sizeof(i64) * P * P, c->stream);
         }
         if (e == cudaSuccess) {
-            // cell-by-cell counts in shared memory where they fit twice per SM beside the row table
-            const size_t ctab_bytes = sizeof(int) * (size_t)dm.K * dm.K;
-            const int cells_by_table = ctab_bytes <= 80 * 1024;
-            if (cells_by_table && ctab_bytes > 24 * 1024)
-                e = cudaFuncSetAttribute(k_sel_dist, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+            // Tables of three CTAs per SM; larger ones are worked through in blocks.  (Prepare's limit keeps K below 18 k, so
+            // that a block has at least one group.)
+            const size_t rtab = std::min<size_t>(sizeof(int) * (size_t)dm.R * dm.R, std::max<size_t>(8 * 1024, sizeof(int) * (size_t)dm.R));
+            const size_t ctab = std::min<size_t>(sizeof(int) * (size_t)dm.K * dm.K, std::max<size_t>((72 * 1024 - rtab) / 4 * 4, sizeof(int) * (size_t)dm.K));
+            const void *fn = dm.N <= 65535 ? (const void *)k_sel_dist<u32> : (const void *)k_sel_dist<u64>;
+            if (ctab + rtab > 32 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(ctab + rtab));
+            if (e == cudaSuccess) {
+                const size_t items = P * ((P + SEL_CHUNK - 1) / SEL_CHUNK);
+                const int grid = (int)std::min<size_t>(items, (size_t)148 * 3);
+                if (dm.N <= 65535) k_sel_dist<u32><<<grid, SEL_THREADS, ctab + rtab, c->stream>>>(dm, (int)P, n_proj, rep, B, dist, (int)ctab, (int)rtab);
+                else k_sel_dist<u64><<<grid, SEL_THREADS, ctab + rtab, c->stream>>>(dm, (int)P, n_proj, rep, B, dist, (int)ctab, (int)rtab);
+            }
+            const int gt = (int)std::min<size_t>(GREEDY_THREADS, (P + 31) / 32 * 32);
+            const size_t gm = greedy_smem ? 2 * sizeof(i64) * P : 0;
+            if (e == cudaSuccess && gm > 32 * 1024) e = cudaFuncSetAttribute(k_sel_greedy, cudaFuncAttributeMaxDynamicSharedMemorySize, GREEDY_SMEM);
             if (e == cudaSuccess)
-                k_sel_dist<<<dim3((unsigned)P, (unsigned)P), SEL_THREADS, cells_by_table ? ctab_bytes : 0, c->stream>>>(
-                    dm, (int)P, n_proj, rep, B, dist, cells_by_table);
-            k_sel_greedy<<<1, GREEDY_THREADS, 0, c->stream>>>((int)P, rep, score, dist, eta_q16, mind, pen, order, n_distinct);
+                k_sel_greedy<<<1, gt, gm, c->stream>>>((int)P, rep, score, dist, eta_q16, mind, pen, order, n_distinct);
             k_sel_fill<<<(int)P, 256, 0, c->stream>>>(dm.N, order, lay, out);
             g_rp_launches += 6;
             e = cudaGetLastError();
@@ -418,7 +528,7 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
     }
     dev_free(c, B.canon); dev_free(c, B.hash); dev_free(c, B.clist); dev_free(c, B.cstart); dev_free(c, B.rlist);
     dev_free(c, B.rstart); dev_free(c, B.pc); dev_free(c, B.pr); dev_free(c, B.phi); dev_free(c, sgn); dev_free(c, rep);
-    dev_free(c, mind); dev_free(c, pen);
+    dev_free(c, mind); dev_free(c, pen); dev_free(c, B.lab); dev_free(c, B.big);
     if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
     return st;
 }
