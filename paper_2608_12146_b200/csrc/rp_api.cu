@@ -155,12 +155,12 @@ static int copy_out(rp_ctx *c, void *dst, const void *src, size_t bytes)
     return RP_OK;
 }
 
-static void free_population(rp_ctx *c)
+static void free_population(rp_ctx *c, bool keep_rank_loads = false)
 {
     dev_free(c, c->d_pop_slab); c->d_pop_slab = nullptr;           // every buffer below but d_W is a piece of it
-    dev_free(c, c->d_W); c->W_cells = 0;
+    if (!keep_rank_loads) { dev_free(c, c->d_W); c->d_W = nullptr; c->W_cells = 0; }
     c->buf[0].blob = nullptr; c->buf[1].blob = nullptr;
-    c->d_W = nullptr; c->d_wloc = nullptr; c->d_wloc_next = nullptr; c->d_le_scratch = nullptr;
+    c->d_wloc = nullptr; c->d_wloc_next = nullptr; c->d_le_scratch = nullptr;
     c->d_wref = nullptr; c->d_wcount = nullptr; c->d_wfree = nullptr; c->d_wfree_head = nullptr;
     c->d_cand_layout = nullptr; c->d_inc_slot = nullptr;
     c->d_tf = nullptr; c->d_qr = nullptr; c->d_Wr = nullptr; c->d_rowF = nullptr; c->d_undecided = nullptr;
@@ -453,7 +453,7 @@ __global__ void k_iota(int *out, int n, int first)
     if (x < n) out[x] = first + x;
 }
 
-static int build_population(rp_ctx *c);
+static int build_population(rp_ctx *c, bool candidates = false, bool same_rows = false);
 
 // Rank-load cells in full form, at least `cells` of them (keep: with what the present ones hold).  A population that
 // is annealed on rows kept apart (padded or compressed) needs only as many as it is scored with: one for the seed
@@ -463,6 +463,7 @@ static int need_rank_loads(rp_ctx *c, size_t cells, bool keep)
     if (cells <= c->W_cells) return RP_OK;
     const size_t wn = (size_t)c->dm.RG * c->dm.LP;
     int *W = nullptr;
+    if (!keep) { dev_free(c, c->d_W); c->d_W = nullptr; c->W_cells = 0; }
     RP_TRY(dev_alloc(c, &W, cells * wn));
     if (keep && c->W_cells) RP_CUDA(cudaMemcpyAsync(W, c->d_W, sizeof(int) * wn * c->W_cells, cudaMemcpyDeviceToDevice, c->stream));
     dev_free(c, c->d_W);
@@ -503,7 +504,11 @@ static void forget_rows(rp_ctx *c, int n)
     c->rows_current = 0; c->full_stale = 0; c->row_undecided = -1; c->row_members = n;
 }
 
-static int build_population(rp_ctx *c)
+// `candidates`: the population is scored and selected from, never annealed (one rank-load cell per member is enough).
+// `same_rows`: the row count is that of the population before, whose rank-load memory is kept if it is large enough.  (Giving
+// back a few hundred MB and asking for as much again while smaller buffers sit between has the pool unmap and map pages:
+// 2.4 to 15 ms in an initial population of 256 candidates, 377 MB of rank loads.)
+static int build_population(rp_ctx *c, bool candidates, bool same_rows)
 {
     RpDims &dm = c->dm;
     rp_decide_layouts(c);
@@ -512,9 +517,9 @@ static int build_population(rp_ctx *c)
     if (smem > 220 * 1024) return RP_ERR_RANGE;
 
     // population buffers
-    free_population(c); free_eval(c);
+    free_population(c, same_rows); free_eval(c);
     const size_t P = (size_t)c->Ppop;
-    RP_TRY(need_rank_loads(c, c->row_mode && rp_row_separate(c) ? 1 : 2 * P, false));
+    RP_TRY(need_rank_loads(c, c->row_mode && rp_row_separate(c) ? 1 : candidates ? P : 2 * P, false));
     {
         RpSlab slab = { nullptr, 0 };
         for (int pass = 0; pass < 2; ++pass) {
@@ -717,7 +722,7 @@ extern "C" int rp_pair_population(rp_ctx *c, int32_t choice_width, int32_t *n_ch
     if (st == RP_OK) st = dev_alloc(c, &cnt, 1);
     if (st == RP_OK) st = need_rank_loads(c, P, true);          // the pairing's rank loads
     const int batch = (int)(P - 1 < 1024 ? P - 1 : 1024);          // members paired per launch (bounds the scratch)
-    if (st == RP_OK && batch > 0) st = dev_alloc(c, &prof, (size_t)batch * dm.K * dm.LP);
+    if (st == RP_OK && batch > 0 && dm.RG != dm.K) st = dev_alloc(c, &prof, (size_t)batch * dm.K * dm.LP);   // not with one slot per row-shard
     cudaError_t e = cudaSuccess;
     if (st == RP_OK) {
         k_gather_cells<<<c->Ppop, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, lay);
@@ -826,7 +831,7 @@ extern "C" int rp_init_population(rp_ctx *c, int32_t n_candidates, int32_t choic
     cudaError_t e = cudaSuccess;
     // the candidates as a population of their own
     c->Ppop = M;
-    st = build_population(c);
+    st = build_population(c, true, true);
     do {
         if (st != RP_OK) break;
         if ((st = dev_alloc(c, &lay, (size_t)M * dm.N)) != RP_OK) break;
@@ -838,7 +843,7 @@ extern "C" int rp_init_population(rp_ctx *c, int32_t n_candidates, int32_t choic
         if ((st = dev_alloc(c, &dist, (size_t)M * M)) != RP_OK) break;
         if ((st = need_rank_loads(c, M, true)) != RP_OK) break;
         const int batch = M - 1 < 1024 ? M - 1 : 1024;
-        if ((st = dev_alloc(c, &prof, (size_t)batch * dm.K * dm.LP)) != RP_OK) break;
+        if (dm.RG != dm.K && (st = dev_alloc(c, &prof, (size_t)batch * dm.K * dm.LP)) != RP_OK) break;
         // trials 2 .. M-1; candidates 0 and 1 start as the length-only seed
         if ((st = rp_launch_seed_trials(c, choice_width, lay, ok)) != RP_OK) break;
         if ((e = cudaMemcpyAsync(lay + dm.N, c->d_seed_layout, sizeof(int) * dm.N, cudaMemcpyDeviceToDevice, c->stream)) != cudaSuccess) break;
@@ -870,7 +875,7 @@ extern "C" int rp_init_population(rp_ctx *c, int32_t n_candidates, int32_t choic
         if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) break;      // `pick` is pageable memory
         // the population proper
         c->Ppop = P;
-        if ((st = build_population(c)) != RP_OK) break;
+        if ((st = build_population(c, false, true)) != RP_OK) break;
         if ((st = install_population(c, fin, nd)) != RP_OK) break;          // rows nd.. repeat the first nd
         if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) break;
         if (n_distinct) *n_distinct = nd;
@@ -881,7 +886,7 @@ extern "C" int rp_init_population(rp_ctx *c, int32_t n_candidates, int32_t choic
     free(h);
     if (c->Ppop != P) {                      // failed half way: back to a seed population of the right size
         c->Ppop = P;
-        const int st2 = build_population(c);
+        const int st2 = build_population(c, false, true);
         if (st == RP_OK && e == cudaSuccess) st = st2;
     }
     if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
