@@ -632,7 +632,8 @@ int rp_launch_anneal_level(rp_ctx *c, int level, int n_levels, const rp_anneal_p
 {
     AnnealArgs A;
     fill_args(c, level, n_levels, prm, rho_q32, guide_q32, A);
-    if (rp_uses_slices(c->dm)) RP_TRY(rp_launch_slice_gc(c));
+    if (rp_uses_slices(c->dm) && !c->slices_listed) RP_TRY(rp_launch_slice_gc(c));
+    c->slices_listed = 0;
     if (rp_uses_row(c)) return rp_launch_anneal_row(c, A);
     if (rp_uses_warp_chains(c)) return rp_launch_anneal_warp(c, A);
     if (use_wpc(c->dm)) return rp_launch_anneal_wpc(c, A);

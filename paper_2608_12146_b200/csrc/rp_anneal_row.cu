@@ -658,6 +658,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
         A.best[3 * (rep + j)] = B0; A.best[3 * (rep + j) + 1] = B1; A.best[3 * (rep + j) + 2] = B2;
         if (!CHIP || A.lo.tr_term) { A.best_step[rep + j] = bk->best_step; A.digest[rep + j] = bk->dig; }
         if (!CHIP) A.best_nlog[j] = bk->best_nlog;
+        if (!CHIP && !A.last) { A.lo.F[j] = (u64)ch.Sc[3]; atomicMin(A.lo.F + 2 * (size_t)P, (u64)ch.Sc[3]); }
         sum_feas += n_feas; sum_acc += n_acc; sum_imp += bk->n_imp; sum_rows += n_rows;
         if (!CHIP || last) {
             atomicAdd((u64 *)&A.counters[0], (u64)A.steps * n_levels);
@@ -1117,6 +1118,7 @@ int rp_launch_anneal_row_all(rp_ctx *c, const AnnealArgs &A0, int *done)
 }
 
 int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A);
+int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A);
 
 int rp_launch_anneal_row(rp_ctx *c, AnnealArgs &A)
 {
@@ -1138,5 +1140,6 @@ int rp_launch_anneal_row(rp_ctx *c, AnnealArgs &A)
     ROW_CASE(1, 1); ROW_CASE(1, 2); ROW_CASE(1, 4); ROW_CASE(2, 1); ROW_CASE(2, 2); ROW_CASE(4, 1);
 #undef ROW_CASE
     RP_TRY(st);
+    if (!A.last && rp_row_turns(c)) return rp_launch_level_turn(c, A);
     return rp_launch_level_end(c, A);
 }

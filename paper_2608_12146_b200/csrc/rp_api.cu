@@ -560,7 +560,7 @@ static int build_population(rp_ctx *c, bool candidates, bool same_rows)
             slab.take(&c->d_best_step, 2 * P);
             slab.take(&c->d_best_nlog, 2 * P);
             slab.take(&c->d_digest, 2 * P);
-            slab.take(&c->d_F, 2 * P);                   // (two sets like the reports, see rp_anneal_row.cu)
+            slab.take(&c->d_F, 2 * P + 1);               // (two sets like the reports, see rp_anneal_row.cu; smallest energy, see rp_level_turn.cu)
             if (pass == 0) { RP_TRY(dev_alloc(c, &c->d_pop_slab, slab.off)); slab.base = c->d_pop_slab; }
         }
     }
@@ -916,12 +916,12 @@ static int launch_best_check(rp_ctx *c);
 static int best_verdict(const rp_ctx *c, const int *sw);
 
 __global__ void k_reset_anneal(i64 *__restrict__ counters, int *__restrict__ status, int *__restrict__ inc_slot,
-                               int *__restrict__ done, int *__restrict__ sync, int n_sync)
+                               int *__restrict__ done, int *__restrict__ sync, int n_sync, u64 *__restrict__ emin)
 {
     const int x = threadIdx.x;
     if (x < 8) counters[x] = 0;
     if (x < RP_SW_COUNT) status[x] = 0;
-    if (x == 0) { *inc_slot = -1; *done = 0; }
+    if (x == 0) { *inc_slot = -1; *done = 0; *emin = ~0ull >> 1; }
     for (int y = x; y < n_sync; y += blockDim.x) sync[y] = 0;
 }
 
@@ -975,11 +975,13 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     // counters and status words to zero, incumbent slot to -1 (the incumbent is in d_inc_layout): done by the
     // set-up of a fresh population
     if (!c->log_clean) {
-        k_reset_anneal<<<1, 256, 0, c->stream>>>(c->d_counters, c->d_status, c->d_inc_slot, c->d_done, c->d_sync, c->Ppop + 1);
+        k_reset_anneal<<<1, 256, 0, c->stream>>>(c->d_counters, c->d_status, c->d_inc_slot, c->d_done, c->d_sync, c->Ppop + 1,
+                                                c->d_F + 2 * (size_t)c->Ppop);
         ++g_rp_launches;
         RP_CUDA(cudaGetLastError());
     }
     c->log_clean = 0;
+    c->slices_listed = 0;
 
     RpSide *side = (RpSide *)c->side;
     cudaEvent_t ev[2] = { side ? side->t0 : nullptr, side ? side->t1 : nullptr };
@@ -1043,7 +1045,8 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     if (stats) {
         stats->proposed = cn[0]; stats->feasible = cn[1]; stats->accepted = cn[2]; stats->improved = cn[3];
         stats->move_bytes = cn[4]; stats->gather_bytes = cn[5]; stats->staging_bytes = cn[6];
-        stats->kernel_launches = all_in_one ? 1 : (int64_t)NL * ((rp_uses_slices(c->dm) ? 3 : 1) + (row || rp_uses_warp_chains(c) ? 1 : 0));
+        stats->kernel_launches = all_in_one ? 1 : row && rp_row_turns(c) ? 2 * (int64_t)NL + 2
+                               : (int64_t)NL * ((rp_uses_slices(c->dm) ? 3 : 1) + (row || rp_uses_warp_chains(c) ? 1 : 0));
         stats->ms_chains = ms_chains;
     }
     c->best_verdict = best_verdict(c, sw);

@@ -166,7 +166,8 @@ struct rp_ctx {
     u64 *d_digest;             // [P_pop]
     uint2 *d_log;              // [P_pop][log_cap] accepted moves (sample, second | reloc<<31)
     int log_cap;
-    u64 *d_F;                  // [P_pop] cumulative weights
+    u64 *d_F;                  // [P_pop] cumulative weights; the one-layer-per-lane kernel: [2*P_pop] energies and weights, then the smallest energy
+    int slices_listed;         // the level before has left holders and free slices for the next one
     i64 *d_counters;           // [4]
     // incumbent
     int *d_inc_layout;         // [N]
@@ -249,6 +250,7 @@ bool rp_uses_slices(const RpDims &dm);
 int rp_slice_mode(const RpDims &dm, int knob);
 void rp_decide_layouts(rp_ctx *c);
 int rp_launch_slice_gc(rp_ctx *c);
+bool rp_row_turns(const rp_ctx *c);
 // Stream-ordered device memory from the device's pool (n elements of T; freed on the context's stream).
 template <class T>
 static inline int dev_alloc(rp_ctx *c, T **p, size_t n)

@@ -535,6 +535,7 @@ struct SetupArgs {
     char *blk;
     int P, *anc, *wloc, *wloc_next, *done, *inc_layout, *one_ticket, *wcount, *undecided, *inc_slot, *sync, *status;
     i64 *one_Esum, *counters;
+    u64 *emin;
 };
 __global__ void __launch_bounds__(256)
 k_setup_population(const SetupArgs A)
@@ -558,7 +559,7 @@ k_setup_population(const SetupArgs A)
     if (A.wcount) for (size_t x = tid; x < 2 * (size_t)A.P * dm.RG; x += nt) A.wcount[x] = 0;
     if (tid < 7) A.counters[tid] = 0;                      // (the eighth is the window's token total)
     if (tid < RP_SW_COUNT) A.status[tid] = 0;
-    if (tid == 0) { *A.done = 0; *A.one_ticket = 0; *A.undecided = 0; *A.inc_slot = -1; }
+    if (tid == 0) { *A.done = 0; *A.one_ticket = 0; *A.undecided = 0; *A.inc_slot = -1; *A.emin = ~0ull >> 1; }
 }
 
 int rp_launch_setup_population(rp_ctx *c)
@@ -569,6 +570,7 @@ int rp_launch_setup_population(rp_ctx *c)
     A.blk = c->d_static; A.P = c->Ppop; A.anc = c->d_anc; A.wloc = c->d_wloc; A.wloc_next = c->d_wloc_next; A.done = c->d_done;
     A.inc_layout = c->d_inc_layout; A.one_ticket = c->d_one_ticket; A.wcount = c->d_wcount; A.undecided = c->d_undecided;
     A.inc_slot = c->d_inc_slot; A.sync = c->d_sync; A.status = c->d_status; A.one_Esum = c->d_one_Esum; A.counters = c->d_counters;
+    A.emin = c->d_F + 2 * (size_t)c->Ppop;
     const size_t most = std::max((size_t)std::max(c->Ppop + 1, dm.N), c->d_wcount ? 2 * (size_t)c->Ppop * dm.RG / 8 : 0);
     const int grid = (int)std::min<size_t>(148 * 4, (most + 255) / 256);
     k_setup_population<<<grid, 256, 0, c->stream>>>(A);

@@ -151,24 +151,24 @@ __device__ __forceinline__ int le_lexmin_lane(i64 v0, i64 v1, i64 v2, int j)
     return who ? __ffs(who) - 1 : -1;
 }
 
-// Called by all threads of one CTA (nt a multiple of 32, at most 1024).  `ws` is the CTA's
-// dynamic shared memory, free once the chain has been stored: the cumulative weights and the
-// replayed layout live there when they fit (global memory otherwise), which keeps the
-// dependent accesses of the binary search and of the replay off the L2 round trip.
-__device__ __forceinline__ void rp_level_end(const AnnealArgs &A, int tid, int nt, unsigned char *ws, size_t ws_bytes)
+// Shared by the incumbent's part and the resampling.
+struct LeShared {
+    i64 r0[LE_MAX_WARPS], r1[LE_MAX_WARPS], r2[LE_MAX_WARPS], rmin[LE_MAX_WARPS];
+    int rj[LE_MAX_WARPS], rn[LE_MAX_WARPS], ra[LE_MAX_WARPS];
+    u64 rsum[LE_MAX_WARPS], carry_s;
+    int win_j, win_n, win_a, do_update;
+};
+
+// Traces of the chains' reports, and the incumbent: lexicographic argmin of the trajectory-best scores.  Called by all
+// threads of one CTA (nt a multiple of 32, at most 1024); `ws` is workspace for the replayed layout and the move log.
+// ENERGY: also the smallest terminal energy (S.rmin per warp) and e_first, that of member tid.
+template <bool ENERGY>
+__device__ __forceinline__ void le_incumbent(const AnnealArgs &A, int tid, int nt, unsigned char *ws, size_t ws_bytes, LeShared &S, i64 &e_first)
 {
-    __shared__ i64 r0[LE_MAX_WARPS], r1[LE_MAX_WARPS], r2[LE_MAX_WARPS];
-    __shared__ int rj[LE_MAX_WARPS], rn[LE_MAX_WARPS], ra[LE_MAX_WARPS];
-    __shared__ u64 rsum[LE_MAX_WARPS];
-    __shared__ int win_j, win_n, win_a, do_update;
-    __shared__ i64 rmin[LE_MAX_WARPS];
-    __shared__ u64 carry_s;
     const int lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
     const int P = A.Ppop;
     const LevelOut &O = A.lo;
-    const bool F_on_chip = (size_t)P * 8 <= ws_bytes / 2;
     const bool lay_on_chip = (size_t)A.dm.N * 2 <= ws_bytes / 2;
-    u64 *F = F_on_chip ? (u64 *)ws : O.F;
     unsigned short *lay_s = (unsigned short *)(ws + ws_bytes / 2);
 
     // trace copies of the per-chain reports
@@ -184,26 +184,26 @@ __device__ __forceinline__ void rp_level_end(const AnnealArgs &A, int tid, int n
     i64 b0 = i0, b1 = i1, b2 = i2;
     int bj = 0x7fffffff, bn = 0, ba = 0;
     i64 emin = 0x7fffffffffffffffll;         // smallest terminal energy, for the weights further down
-    i64 e_first = 0;                         // energy of member tid (all there is to weigh when P <= nt)
-    const int now0 = A.w_on_chip ? A.wloc_dst[0] : 0;      // which half of the cells this level worked in (needed at the end)
 #pragma unroll 2
     for (int j = tid; j < P; j += nt) {
         const i64 s0 = LE_LD(A.best[3 * (size_t)j]), s1 = LE_LD(A.best[3 * (size_t)j + 1]), s2 = LE_LD(A.best[3 * (size_t)j + 2]);
-        const i64 t0 = LE_LD(A.term[3 * (size_t)j]), t1 = LE_LD(A.term[3 * (size_t)j + 1]), t2 = LE_LD(A.term[3 * (size_t)j + 2]);
+        const i64 t0 = ENERGY ? LE_LD(A.term[3 * (size_t)j]) : 0, t1 = ENERGY ? LE_LD(A.term[3 * (size_t)j + 1]) : 0, t2 = ENERGY ? LE_LD(A.term[3 * (size_t)j + 2]) : 0;
         if (rp_lex_less(s0, s1, s2, b0, b1, b2)) {    // ascending j: first wins
             b0 = s0; b1 = s1; b2 = s2; bj = j;
             if (!O.cand_layout) { bn = LE_LD(A.best_nlog[j]); ba = A.anc[j]; }     // what the replay needs, fetched with the rest
         }
-        const i64 e = rp_energy(t0, t1, t2);
-        if (j == tid) e_first = e;
-        emin = e < emin ? e : emin;
+        if (ENERGY) {
+            const i64 e = rp_energy(t0, t1, t2);
+            if (j == tid) e_first = e;
+            emin = e < emin ? e : emin;
+        }
     }
-    {   // warp minimum of the (non-negative) energies: smallest high word, then smallest low word among its holders
+    if (ENERGY) {   // warp minimum of the (non-negative) energies: smallest high word, then smallest low word among its holders
         const u32 hi = (u32)((u64)emin >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
         const u32 ml = __reduce_min_sync(0xffffffffu, hi == mh ? (u32)emin : 0xffffffffu);
         emin = (i64)(((u64)mh << 32) | ml);
+        if (lane == 0) S.rmin[warp] = emin;
     }
-    if (lane == 0) rmin[warp] = emin;
     if (__syncthreads_or(bj != 0x7fffffff)) {
     {
         const int src = le_lexmin_lane(b0, b1, b2, bj);         // this warp's best, handed to lane 0
@@ -212,12 +212,12 @@ __device__ __forceinline__ void rp_level_end(const AnnealArgs &A, int tid, int n
             bj = __shfl_sync(0xffffffffu, bj, src); bn = __shfl_sync(0xffffffffu, bn, src); ba = __shfl_sync(0xffffffffu, ba, src);
         }
     }
-    if (lane == 0) { r0[warp] = b0; r1[warp] = b1; r2[warp] = b2; rj[warp] = bj; rn[warp] = bn; ra[warp] = ba; }
+    if (lane == 0) { S.r0[warp] = b0; S.r1[warp] = b1; S.r2[warp] = b2; S.rj[warp] = bj; S.rn[warp] = bn; S.ra[warp] = ba; }
     __syncthreads();
     if (warp == 0) {                                            // the same over the warps' results
         const bool has = lane < nwarps;
-        b0 = has ? r0[lane] : 0; b1 = has ? r1[lane] : 0; b2 = has ? r2[lane] : 0;
-        bj = has ? rj[lane] : 0x7fffffff; bn = has ? rn[lane] : 0; ba = has ? ra[lane] : 0;
+        b0 = has ? S.r0[lane] : 0; b1 = has ? S.r1[lane] : 0; b2 = has ? S.r2[lane] : 0;
+        bj = has ? S.rj[lane] : 0x7fffffff; bn = has ? S.rn[lane] : 0; ba = has ? S.ra[lane] : 0;
         const int src = le_lexmin_lane(b0, b1, b2, bj);
         if (src >= 0) {
             b0 = __shfl_sync(0xffffffffu, b0, src); b1 = __shfl_sync(0xffffffffu, b1, src); b2 = __shfl_sync(0xffffffffu, b2, src);
@@ -225,19 +225,19 @@ __device__ __forceinline__ void rp_level_end(const AnnealArgs &A, int tid, int n
         }
     }
     if (tid == 0) {
-        win_j = bj; win_n = bn; win_a = ba;
-        do_update = rp_lex_less(b0, b1, b2, i0, i1, i2);
-        if (do_update) {
+        S.win_j = bj; S.win_n = bn; S.win_a = ba;
+        S.do_update = rp_lex_less(b0, b1, b2, i0, i1, i2);
+        if (S.do_update) {
             O.inc_score[0] = b0; O.inc_score[1] = b1; O.inc_score[2] = b2;
             if (O.cand_layout) *O.inc_slot = bj;         // the winner stored its best layout itself
         }
     }
     __syncthreads();
-    if (do_update && !O.cand_layout) {
-        const int w = win_j;
-        const unsigned short *cs = (const unsigned short *)(A.blob_src + (size_t)win_a * A.bl.bytes + A.bl.off_cell);
+    if (S.do_update && !O.cand_layout) {
+        const int w = S.win_j;
+        const unsigned short *cs = (const unsigned short *)(A.blob_src + (size_t)S.win_a * A.bl.bytes + A.bl.off_cell);
         const uint2 *lg = A.log + (size_t)w * A.log_cap;
-        const int n = win_n;
+        const int n = S.win_n;
         if (lay_on_chip) {
             // the log goes through the other half of the workspace when it fits (no dependent L2 round trips)
             uint2 *lg_s = (uint2 *)ws;
@@ -281,6 +281,23 @@ __device__ __forceinline__ void rp_level_end(const AnnealArgs &A, int tid, int n
     }     // some chain beat the incumbent
     __syncthreads();
     if (O.tr_inc && tid < 3) O.tr_inc[(size_t)A.level * 3 + tid] = O.inc_score[tid];
+}
+
+// Called by all threads of one CTA (nt a multiple of 32, at most 1024).  `ws` is the CTA's
+// dynamic shared memory, free once the chain has been stored: the cumulative weights and the
+// replayed layout live there when they fit (global memory otherwise), which keeps the
+// dependent accesses of the binary search and of the replay off the L2 round trip.
+__device__ __forceinline__ void rp_level_end(const AnnealArgs &A, int tid, int nt, unsigned char *ws, size_t ws_bytes)
+{
+    __shared__ LeShared S;
+    const int lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
+    const int P = A.Ppop;
+    const LevelOut &O = A.lo;
+    const bool F_on_chip = (size_t)P * 8 <= ws_bytes / 2;
+    u64 *F = F_on_chip ? (u64 *)ws : O.F;
+    i64 e_first = 0;                         // energy of member tid (all there is to weigh when P <= nt)
+    const int now0 = A.w_on_chip ? A.wloc_dst[0] : 0;      // which half of the cells this level worked in (needed at the end)
+    le_incumbent<true>(A, tid, nt, ws, ws_bytes, S, e_first);
 
     if (A.last) {            // the terminal states are the population as they stand
         if (O.cand_layout) {
@@ -295,13 +312,14 @@ __device__ __forceinline__ void rp_level_end(const AnnealArgs &A, int tid, int n
     }
 
     // ---- resampling -------------------------------------------------------------------------
-    for (int w = 0; w < nwarps; ++w) emin = rmin[w] < emin ? rmin[w] : emin;
-    if (tid == 0) carry_s = 0;
+    i64 emin = S.rmin[0];
+    for (int w = 1; w < nwarps; ++w) emin = S.rmin[w] < emin ? S.rmin[w] : emin;
+    if (tid == 0) S.carry_s = 0;
     __syncthreads();
     const u64 M = (u64)(emin > A.dm.SC ? emin : A.dm.SC);
-    if (P <= nt) le_prefix_weights<1>(P, A.term, A.cq, tid, nt, emin, M, F, rsum, &carry_s, true, e_first);
-    else if (P <= 2 * nt) le_prefix_weights<2>(P, A.term, A.cq, tid, nt, emin, M, F, rsum, &carry_s);
-    else le_prefix_weights<4>(P, A.term, A.cq, tid, nt, emin, M, F, rsum, &carry_s);
+    if (P <= nt) le_prefix_weights<1>(P, A.term, A.cq, tid, nt, emin, M, F, S.rsum, &S.carry_s, true, e_first);
+    else if (P <= 2 * nt) le_prefix_weights<2>(P, A.term, A.cq, tid, nt, emin, M, F, S.rsum, &S.carry_s);
+    else le_prefix_weights<4>(P, A.term, A.cq, tid, nt, emin, M, F, S.rsum, &S.carry_s);
     const u64 Ftot = F[P - 1];
     const u64 u0 = (u64)(((unsigned __int128)A.resample_x * Ftot) >> 32);
     // The cell bookkeeping further down works in shared memory when 8*P ints fit: ancestors and
@@ -392,15 +410,15 @@ __device__ __forceinline__ void rp_level_end(const AnnealArgs &A, int tid, int n
         for (int x = x0; x < x1; ++x) total += arr[x];
         int v = total;
         for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += y; }
-        if (lane == 31) rj[warp] = v;
+        if (lane == 31) S.rj[warp] = v;
         __syncthreads();
         if (warp == 0) {
-            int s2 = (lane < nwarps) ? rj[lane] : 0;
+            int s2 = (lane < nwarps) ? S.rj[lane] : 0;
             for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, s2, o); if (lane >= o) s2 += y; }
-            rj[lane] = s2;
+            S.rj[lane] = s2;
         }
         __syncthreads();
-        int rank = (warp ? rj[warp - 1] : 0) + v - total;          // exclusive rank of the chunk's first element
+        int rank = (warp ? S.rj[warp - 1] : 0) + v - total;          // exclusive rank of the chunk's first element
         for (int x = x0; x < x1; ++x) {
             const int flag = arr[x];
             if (pass) { if (flag) freelist[rank] = x; }

@@ -1,0 +1,215 @@
+// From one level of the population annealing to the next for the one-layer-per-lane kernel with one launch per level:
+// incumbent, Boltzmann weights, ancestors, holders of the rank-load slices, list of free slices, in one cooperative launch.
+//
+// The three launches this replaces (a level barrier of one CTA, the holders, the free list) are short and one behind the
+// other: what bounds them is latency, 34 us a level at 1024 members of 240 row-shards with the gaps.  Here the worker CTAs
+// share the members out, meet twice and otherwise never wait; the last CTA looks after the incumbent (whose move log is
+// replayed one move after the other) beside them.  The chains leave their energies and the smallest of them behind.
+//   1. weights of a worker's members
+//   2. all cumulative weights (every worker for itself), ancestors of its members, their slices' holders
+//   3. its piece of the slice table: holders out, counts back to zero, free slices to the list
+// 14 us a level at the same size (plans: large 3.23 -> 2.77 ms, wide 10.8 -> 9.4, ragged 1.78 -> 1.63).
+#include <algorithm>
+#include <string.h>
+
+#include "rp_level_end.cuh"
+#include "rp_anneal_row.cuh"
+
+#define TURN_THREADS 512
+#define TURN_WARPS (TURN_THREADS / 32)
+#define TURN_ROWS 8
+#define TURN_MAX_MEMBERS 16384           // cumulative weights on chip (with their padding, 136 KB)
+
+struct TurnArgs {
+    u64 *E, *weight;             // [P] energies of the terminal states, weights
+    u64 *emin;                   // the smallest energy; left at its start value for the next level
+    int *ref, *holders, *list, *head;        // slices: counts (zero between launches), holders, free ones, cursors
+    int ns;                      // slices
+    int base;                    // arrivals at the meeting point of the launches before
+};
+
+__device__ __forceinline__ bool turn_meet(const AnnealArgs &A, int target)
+{
+    __shared__ int ok;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(A.sync, 1);
+        ok = rp_wait_count(A.sync, target, A);
+    }
+    __syncthreads();
+    return ok;
+}
+
+__global__ void __launch_bounds__(TURN_THREADS)
+k_level_turn(const AnnealArgs A, const TurnArgs T)
+{
+    extern __shared__ __align__(16) unsigned char turn_smem[];
+    if (__ldcg(&A.status[RP_SW_TIMEOUT])) return;
+    __shared__ LeShared S;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int workers = (int)gridDim.x - 1, P = A.Ppop, RG = A.dm.RG;
+    if ((int)blockIdx.x == workers) {
+        i64 none;
+        le_incumbent<false>(A, tid, TURN_THREADS, turn_smem, rp_le_ws_bytes(A, A.smem_bytes), S, none);
+        return;
+    }
+    const int m0 = (int)((long long)P * blockIdx.x / workers), m1 = (int)((long long)P * (blockIdx.x + 1) / workers);
+
+    // ---- 1: weights ------------------------------------------------------------------------------
+    const i64 emin = (i64)__ldcg(T.emin);
+    const u64 M = (u64)(emin > A.dm.SC ? emin : A.dm.SC);
+    for (int m = m0 + tid; m < m1; m += TURN_THREADS) {
+        const i64 e[1] = { (i64)__ldcg(T.E + m) };
+        u64 w[1];
+        le_weights<1>(e, emin, M, A.cq, w);
+        T.weight[m] = w[0];
+    }
+    if (blockIdx.x == 0 && tid == 0) { T.head[0] = 0; T.head[1] = 0; }
+    if (!turn_meet(A, T.base + workers)) { if (tid == 0) atomicExch(&A.status[RP_SW_TIMEOUT], 1); return; }
+    if (blockIdx.x == 0 && tid == 0) *T.emin = ~0ull >> 1;
+
+    // ---- 2: cumulative weights; a thread adds up 2^lu consecutive members, place j of the table is j + (j >> lu) (no bank
+    // conflicts) ----------------------------------------------------------------------------------------
+    u64 *F = (u64 *)turn_smem;
+    int lu = 0;
+    while ((TURN_THREADS << lu) < P) ++lu;
+    {
+        const int j0 = tid << lu, j1 = min(P, j0 + (1 << lu));
+        u64 own = 0;
+        for (int j = j0; j < j1; ++j) { own += __ldcg(T.weight + j); F[j + (j >> lu)] = own; }
+        u64 v = own;
+        for (int o = 1; o < 32; o <<= 1) { const u64 x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
+        if (lane == 31) S.rsum[warp] = v;
+        __syncthreads();
+        if (warp == 0) {
+            u64 s2 = lane < TURN_WARPS ? S.rsum[lane] : 0;
+            for (int o = 1; o < 32; o <<= 1) { const u64 x = __shfl_up_sync(0xffffffffu, s2, o); if (lane >= o) s2 += x; }
+            if (lane < TURN_WARPS) S.rsum[lane] = s2;
+        }
+        __syncthreads();
+        const u64 before = (warp ? S.rsum[warp - 1] : 0) + v - own;
+        for (int j = j0; j < j1; ++j) F[j + (j >> lu)] += before;
+        __syncthreads();
+    }
+    int *anc = (int *)(F + P + (P >> lu) + 1);                   // of this worker's members
+    {
+        const u64 Ftot = F[P - 1 + ((P - 1) >> lu)];
+        const u64 u0 = (u64)(((unsigned __int128)A.resample_x * Ftot) >> 32);
+        for (int m = m0 + tid; m < m1; m += TURN_THREADS) {
+            const unsigned __int128 at = (unsigned __int128)u0 + (unsigned __int128)m * Ftot;
+            int lo = 0, hi = P - 1;
+            while (lo < hi) {                       // smallest slot with P * F > at
+                const int mid = (lo + hi) >> 1;
+                if ((unsigned __int128)P * F[mid + (mid >> lu)] > at) hi = mid; else lo = mid + 1;
+            }
+            anc[m - m0] = lo;
+            A.lo.anc_out[m] = lo;
+            if (A.lo.tr_anc) A.lo.tr_anc[(size_t)A.level * P + m] = lo;
+        }
+    }
+    __syncthreads();
+    // Holders among the members that start the next level.  Most members share most slices for some levels, and additions to one
+    // address queue up (one each: 14 k cycles at 1024 members of 240 row-shards, 60 k at 4096 of 288; now 3 to 7 k and 20 k); so a thread takes one row-shard of several members and adds a run of equal slices
+    // at once, with the slice it saw first, the one nearly all of them share, counted beside the runs.
+    {
+        const int groups = max(1, TURN_THREADS / RG), n = m1 - m0;
+        for (int x = tid; x < groups * RG; x += TURN_THREADS) {
+            const int g = x / RG, rg = x - g * RG;
+            const int a0 = n * g / groups, a1 = n * (g + 1) / groups;
+            int first = -1, n_first = 0, run = -1, n_run = 0;
+            for (int m = a0; m <= a1; m += 4) {
+                int s[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    s[u] = m + u < a1 ? __ldcg((const int *)(A.blob_dst + (size_t)anc[m + u] * A.bl.bytes + A.bl.off_wtab) + rg) : -1;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (m + u >= a1) continue;
+                    if ((unsigned)s[u] >= (unsigned)T.ns) { atomicExch(&A.status[RP_SW_POOL], 1); continue; }
+                    if (first < 0) first = s[u];
+                    if (s[u] == first) { ++n_first; continue; }
+                    if (s[u] != run) { if (n_run) atomicAdd(&T.ref[run], n_run); run = s[u]; n_run = 0; }
+                    ++n_run;
+                }
+            }
+            if (n_first) atomicAdd(&T.ref[first], n_first);
+            if (n_run) atomicAdd(&T.ref[run], n_run);
+        }
+    }
+    if (!turn_meet(A, T.base + 2 * workers)) { if (tid == 0) atomicExch(&A.status[RP_SW_TIMEOUT], 1); return; }
+
+    // ---- 3: free slices.  A warp takes 32 * TURN_ROWS slices at a time, the CTA one piece of the list for all of its warps; loads and
+    // stores of consecutive lanes are consecutive --------------------------------------------------------
+    const int per = TURN_THREADS * TURN_ROWS;
+    for (long long b0 = (long long)blockIdx.x * per; b0 < T.ns; b0 += (long long)workers * per) {
+        const int s0 = (int)b0 + warp * 32 * TURN_ROWS + lane;
+        unsigned isfree[TURN_ROWS];
+        int v[TURN_ROWS], n = 0;
+#pragma unroll
+        for (int r = 0; r < TURN_ROWS; ++r) v[r] = s0 + 32 * r < T.ns ? __ldcg(T.ref + s0 + 32 * r) : 1;
+#pragma unroll
+        for (int r = 0; r < TURN_ROWS; ++r) {
+            const int s = s0 + 32 * r;
+            if (s < T.ns) { T.holders[s] = v[r]; T.ref[s] = 0; }
+            isfree[r] = __ballot_sync(0xffffffffu, v[r] == 0);
+            n += __popc(isfree[r]);
+        }
+        __syncthreads();                             // (S.rj of the round before)
+        if (lane == 0) S.rj[warp] = n;
+        __syncthreads();
+        if (warp == 0) {
+            int w = lane < TURN_WARPS ? S.rj[lane] : 0;
+            const int mine = w;
+            for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, w, o); if (lane >= o) w += y; }
+            int base = 0;
+            if (lane == 31 && w) base = atomicAdd(&T.head[1], w);
+            base = __shfl_sync(0xffffffffu, base, 31);
+            if (lane < TURN_WARPS) S.rj[lane] = base + w - mine;
+        }
+        __syncthreads();
+        int at = S.rj[warp];
+#pragma unroll
+        for (int r = 0; r < TURN_ROWS; ++r) {
+            if (v[r] == 0) T.list[at + __popc(isfree[r] & ((1u << lane) - 1))] = s0 + 32 * r;
+            at += __popc(isfree[r]);
+        }
+    }
+}
+
+// One launch per level asked for means that a caller plans several windows at once on separate streams: a launch whose CTAs wait
+// for one another would make them wait for its SMs, so the parts then stay launches of their own, as beyond the table on chip.
+bool rp_row_turns(const rp_ctx *c) { return c->knob_level_launches != 1 && c->Ppop <= TURN_MAX_MEMBERS; }
+
+// Between level A.level of an rp_anneal call and the next one.
+int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A0)
+{
+    const int P = c->Ppop, ns = 2 * P * c->dm.RG;
+    AnnealArgs A = A0;
+    TurnArgs T;
+    T.E = c->d_F; T.weight = c->d_F + P; T.emin = c->d_F + 2 * (size_t)P;
+    T.ref = c->d_wcount; T.holders = c->d_wref; T.list = c->d_wfree; T.head = c->d_wfree_head;
+    T.ns = ns;
+    A.sync = c->d_sync;
+    // Workers: as many as have something to do (a meeting costs the more the more there are); every one resident.
+    const int workers = std::max(4, std::min(147, std::max((P + 15) / 16, (ns + 4095) / 4096)));
+    T.base = A.level * 2 * workers;                  // (the count is zero when the call starts)
+    int lu = 0;
+    while ((TURN_THREADS << lu) < P) ++lu;
+    const size_t ws_workers = sizeof(u64) * ((size_t)P + (P >> lu) + 1) + sizeof(int) * ((size_t)P / workers + 2);
+    size_t ws = std::max((size_t)16 * 1024, std::min((size_t)2 * std::max((size_t)A.log_cap * 8, (size_t)c->dm.N * 2), (size_t)160 * 1024));
+    ws = (std::max(ws, ws_workers) + 15) & ~(size_t)15;
+    A.smem_bytes = (unsigned)ws;
+    RP_CUDA(cudaFuncSetAttribute(k_level_turn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(workers + 1); cfg.blockDim = dim3(TURN_THREADS); cfg.dynamicSmemBytes = ws; cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    RP_CUDA(cudaLaunchKernelEx(&cfg, k_level_turn, A, T));
+    ++g_rp_launches;
+    c->slices_listed = 1;
+    return RP_OK;
+}

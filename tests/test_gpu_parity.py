@@ -1211,3 +1211,22 @@ def test_candidate_stages_at_the_edges_of_their_forms(N, D, min_rows, edp, longe
     reps = sorted(set(order[:nd].tolist()))
     assert (dist[np.ix_(reps, reps)] == want["dist"][np.ix_(reps, reps)]).all()
     rp.rp_destroy(ctx)
+
+
+# From level to level in one launch: fewer members than CTAs and several per thread, more row-shards than threads and a few, slices
+# in one piece and several; the same with the parts as launches of their own.
+@pytest.mark.parametrize("N,D,min_rows,edp,pop,levels", [(600, 4, 140, None, 2, 6), (600, 4, 140, None, 37, 5), (60, 2, 2, [0, 0], 1200, 5),
+                                                         (48, 2, 3, None, 5003, 3)])
+def test_between_two_levels_at_the_edges(N, D, min_rows, edp, pop, levels):
+    w = make_window(custom_spec("turn", N, 24, 32, 2, 4096, D, 16, pop, 400, data_seed=N + pop))
+    ref = oracle_front(w, edp, min_rows)
+    for knob in (0, 1):
+        ctx = load(w, pop=pop, edp=edp, min_rows=min_rows)
+        rp.rp_debug_set_knob(ctx, "LAUNCH_PER_LEVEL", knob)
+        check_front(w, ctx, ref)
+        if knob == 0:
+            assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row"
+        _, stats = check_anneal(w, ctx, ref, edp, pop, levels, 20, t_ratio=0.5, check_members=2)
+        if knob == 0:
+            assert stats.kernel_launches == 2 * levels + 2
+        rp.rp_destroy(ctx)
