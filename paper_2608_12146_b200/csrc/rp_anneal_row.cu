@@ -12,7 +12,9 @@
 //    Windows whose samples follow one routing mix have the same busiest rank nearly everywhere, and
 //    then every rejection is decided this way and what is scored is accepted (large, wide, heavy, medium of
 //    the named windows: all but 1e-4 of the rejections); with four routing mixes an eighth to a third
-//    is.  A candidate that is not rejected by its bound is scored exactly.
+//    is.  A candidate that is not rejected by its bound is scored exactly.  The bound is worked out in single precision with an
+//    allowance for its roundings: in 64-bit integers it was a third of a round's instructions (with the decision shared by two
+//    lanes: heavy 89.2 -> 81.4 ms, wide 8.22 -> 8.04, medium 0.87 -> 0.84).
 //  * Rows in registers.  A lane holds whole layers (layer = lane, lane + 32, ...) of the two slices and the two
 //    demand rows: 16-byte loads, one trip, no shuffles, no staging; the new slices are stored from the
 //    same registers.
@@ -51,6 +53,7 @@ struct ChainR {                                      // bookkeeping of the chain
 struct StepX {                   // what a lane keeps about the step it proposes for
     u32 flags, bz;
     u64 thr;
+    float thrf;                  // thr / 2^32, rounded up; infinite where every rise is accepted
     int i[4];                    // samples; for a relocation i[2], i[3] are target cells
     int c[4];                    // cell of sample i[x] (i[2], i[3] themselves for a relocation)
     int t[4], f[4];              // length of sample i[x] and its demand on the fixed ranks (0 for relocation targets)
@@ -214,6 +217,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
     const bool ident = dm.own_shard;
     const bool sum32 = (i64)L * dm.k * dm.C * ((dm.D + dm.G - 1) / dm.G) < (1ll << 31);
     const i64 aC = dm.asum * dm.C, bS = dm.bsum;
+    const float aCf = (float)aC, bSf = (float)bS, ECf = (float)dm.EC;
     const int4 *qr = (const int4 *)X.qr;
     unsigned short *cells = CHIP ? ch.cell : (unsigned short *)(A.blob_dst + (size_t)j * A.bl.bytes + A.bl.off_cell);
     const int nh16 = (A.bl.off_cell + 15) >> 4, nhw = A.bl.off_cell >> 2;     // the blob's arrays before the assignment
@@ -332,13 +336,14 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
             const int nb = min(SPEC, A.steps - kb);
             // ---- the next 32 steps, one per lane: random words, candidate cells, lengths, fixed-rank demands ----
             StepX sr;
-            sr.flags = 0; sr.bz = 0; sr.thr = 0;
+            sr.flags = 0; sr.bz = 0; sr.thr = 0; sr.thrf = 0.f;
 #pragma unroll
             for (int x = 0; x < 4; ++x) { sr.i[x] = -1; sr.c[x] = 0; sr.t[x] = 0; sr.f[x] = 0; }
             if (lane < nb) {
                 const StepRec r = (CHIP && kb + lane < X.recs) ? recs[(ln & 1) * X.recs + kb + lane] : rp_make_step_rec(A, level, tau, (u32)(kb + lane), (u32)j);
                 const bool rl = r.flags & 1u;
                 sr.flags = r.flags; sr.bz = r.bz; sr.thr = r.thr;
+                sr.thrf = r.flags & 4u ? __int_as_float(0x7f800000) : (float)r.thr * (0x1p-32f * (1.f + 0x1p-20f));
                 sr.i[0] = r.i0; sr.i[1] = r.i1; sr.i[2] = r.i2; sr.i[3] = r.i3;
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
@@ -351,11 +356,10 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
             int pos = 0;
             while (pos < nb) {
                 // ---- proposals of steps kb+pos .. kb+nb-1 against the current state, one per lane: GuidedProposal and
-                // feasibility (the rule of rp_propose), then the change of the attention costs, the accept
-                // bound, and the rejection by the fixed ranks --------------------------------------------------
+                // feasibility (the rule of rp_propose), then the rejection by the fixed ranks ----------------------------
                 bool ok = false, pass = false;
                 int mi = 0, mi2 = -1, c1 = 0, c2 = 0, rg1 = 0, rg2 = 0, ti = 0, t2 = 0, df = 0;
-                i64 dA1 = 0, dA2 = 0, bound = 0;     // accepted when the energy rises by less than `bound` (at least 1: never uphill by 0)
+                i64 dA1 = 0, dA2 = 0;                // (shards of several slots)
                 if (lane >= pos && lane < nb) {
                     const bool reloc = sr.flags & 1u;
                     const int ca = sr.c[0], cb = sr.c[1], xa = sr.c[2], xb = sr.c[3];
@@ -365,12 +369,10 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                         const u64 Ja = (u64)ch.Jfx[ra], Aa = (u64)ch.Afx[ra];
                         // bz * Ja < Aa * 2^32  <=>  floor(bz * Ja / 2^32) < Aa
                         const u64 pr = (Ja >> 32) * sr.bz + (((Ja & 0xffffffffull) * sr.bz) >> 32);
-                        i64 ka, kb_, ta, tb;
-                        if (pr < Aa) {
-                            const i64 *key = ident ? ch.Afx : ch.att;
-                            ka = key[ca]; kb_ = key[cb]; ta = key[xa]; tb = key[xb];
-                        } else { ka = (i64)Ja; kb_ = ch.Jfx[rb]; ta = ch.Jfx[rx]; tb = ch.Jfx[ry]; }
-                        src_b = kb_ > ka; dst_b = tb < ta;
+                        const bool by_a = pr < Aa, by_cell = ident || by_a;
+                        const i64 *key = by_a ? (ident ? ch.Afx : ch.att) : ch.Jfx;
+                        src_b = key[by_cell ? cb : rb] > key[by_cell ? ca : ra];
+                        dst_b = key[by_cell ? xb : ry] < key[by_cell ? xa : rx];
                     }
                     mi = src_b ? sr.i[1] : sr.i[0];
                     c1 = src_b ? cb : ca;
@@ -383,20 +385,10 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                     rg1 = ident ? c1 : rg_of[c1]; rg2 = ident ? c2 : rg_of[c2];
                     const int g1 = g_of[c1], g2 = g_of[c2];
                     const int T1 = ch.T[c1], T2 = ch.T[c2], n1 = ch.cnt[c1];
-                    const i64 S0 = ch.Sc[0], S1 = ch.Sc[1], Ecur = ch.Sc[3];
-                    const i64 k1 = ch.slack[rg1], k2 = ch.slack[rg2], J1o = ch.Jfx[rg1], J2o = ch.Jfx[rg2], U1o = ch.U[g1], U2o = ch.U[g2];
-                    const u64 M = (u64)(Ecur > dm.SC ? Ecur : dm.SC);
-                    const u64 bh = __umul64hi(sr.thr, M), bl = sr.thr * M;
-                    bound = (i64)((bh << 32) | (bl >> 32));
-                    bound = bound > 1 ? bound : 1;
-                    if ((sr.flags & 4u) || (bh >> 31)) bound = 0x7fffffffffffffffll;
+                    const i64 S0 = ch.Sc[0], Ecur = ch.Sc[3], k1 = ch.slack[rg1], k2 = ch.slack[rg2], U1o = ch.U[g1], U2o = ch.U[g2];
                     ok = c1 != c2 && T2 - t2 + ti <= dm.C && (reloc ? n1 > 1 : T1 - ti + t2 <= dm.C);
                     const bool tw = ident || rg1 != rg2;
-                    if (ident) {
-                        // aC*T + bS*Q of either cell changes by +-(t2 - ti) * (aC + bS * (t2 + ti))
-                        dA1 = (aC + bS * (t2 + ti)) * (t2 - ti);
-                        dA2 = -dA1;
-                    } else if (ok) {
+                    if (!ident && ok) {
                         const int Ta = T1 - ti + t2, Tb = T2 + ti - t2;
                         const i64 dq = (i64)t2 * t2 - (i64)ti * ti, Qa = (i64)ch.Q[c1] + dq, Qb = (i64)ch.Q[c2] - dq;
                         i64 A1 = 0, A2 = 0;
@@ -412,13 +404,20 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                         } else A1 = rp_attention(dm, st, dpl, dpo, rowbase[c1] / dm.D, g1, c1, Ta, Qa, c2, Tb, Qb);
                         dA1 = A1 - ch.Afx[rg1];
                     }
-                    // the busiest loads fall by at most what the samples put on the fixed ranks plus the slack
-                    // (both cells in one row-shard: nothing changes)
-                    const i64 dJ1 = dA1 + (tw ? dm.EC * (-df - k1) : 0), dJ2 = tw ? dA2 + dm.EC * (df - k2) : 0;
-                    const i64 J1 = J1o + dJ1, J2 = tw ? J2o + dJ2 : J1;
-                    const i64 u1 = U1o + dJ1 + (g1 == g2 ? dJ2 : 0), u2 = g1 == g2 ? u1 : U2o + dJ2;
-                    const i64 n0 = u1 > u2 ? u1 : u2;
-                    pass = ok && (n0 <= S0 || row_energy(n0, S1 + dJ1 + dJ2, J1 > J2 ? J1 : J2) - Ecur < bound);
+                    // Rejected for certain?  The busiest loads fall by at most what the samples put on the fixed ranks plus the
+                    // slack (both cells in one row-shard: nothing changes), so x below is the least by which the largest shard
+                    // cost can rise and x + 1e-6 * (J1 + J2) - 1e-9 * S2 (S2 <= S0 <= E) the least by which the energy can.  In single
+                    // precision, of differences only: a dozen roundings of 2^-24 of the magnitudes in `mag`, allowed for by
+                    // 2^-20 of them; what is not rejected here is decided by the exact score.
+                    const float k1f = sum32 ? (float)(int)k1 : (float)k1, k2f = sum32 ? (float)(int)k2 : (float)k2, dff = (float)df;
+                    const float a1 = ident ? (aCf + bSf * (float)(t2 + ti)) * (float)(t2 - ti) : (float)dA1, a2 = ident ? -a1 : (float)dA2;
+                    const float v1 = (float)(U1o - S0), v2 = (float)(U2o - S0), Mf = (float)(Ecur > dm.SC ? Ecur : dm.SC);
+                    const float J1 = a1 + (tw ? ECf * (-dff - k1f) : 0.f), J2 = tw ? a2 + ECf * (dff - k2f) : 0.f;
+                    const float u1 = v1 + J1 + (g1 == g2 ? J2 : 0.f), u2 = g1 == g2 ? u1 : v2 + J2, x = fmaxf(u1, u2);
+                    const float mag = fabsf(v1) + fabsf(v2) + fabsf(a1) + fabsf(a2) + ECf * (2.f * fabsf(dff) + k1f + k2f);
+                    const float err = 8.f + 0x1p-20f * mag;
+                    const float most = sr.thrf * Mf + 2.f;                   // accepted below (rounded up, see thrf)
+                    pass = ok && !(x > err && x + 1e-6f * (J1 + J2) - 1.001e-9f * Mf - err >= most);
                 }
                 unsigned pmask = __ballot_sync(0xffffffffu, pass);
                 int win = -1;                                   // step accepted
@@ -430,6 +429,29 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                     const unsigned rr = __shfl_sync(0xffffffffu, (unsigned)rg1 | ((unsigned)rg2 << 16), ls);
                     const int r1 = (int)(rr & 0xffffu), r2 = (int)(rr >> 16);
                     const bool touchW = r1 != r2, swap = wi2 >= 0;
+                    // What the decision needs: even lanes look at the cell that gives (1), odd lanes at the one that takes (2).  Ahead
+                    // of the rows its latency hides behind theirs; with one compressed chunk per lane, the form with the most chains
+                    // per SM, the registers count (heavy: 80.3 ms behind the rows, 88.2 ahead; one lane for both sides 84.2 to 86.5).
+                    const bool second = lane & 1;
+                    int d1, d2, wti, wt2, mc, mr, mg;
+                    i64 S0, S1, S2, Ecur, Jo, Uo, eo, wb, dA;
+                    auto look = [&]() {
+                        const unsigned dd = __shfl_sync(0xffffffffu, (unsigned)c1 | ((unsigned)c2 << 16), ls);
+                        d1 = (int)(dd & 0xffffu); d2 = (int)(dd >> 16);
+                        wti = __shfl_sync(0xffffffffu, ti, ls); wt2 = __shfl_sync(0xffffffffu, t2, ls);
+                        mc = second ? d2 : d1; mr = second ? r2 : r1; mg = g_of[mc];
+                        S0 = ch.Sc[0]; S1 = ch.Sc[1]; S2 = ch.Sc[2]; Ecur = ch.Sc[3];
+                        Jo = ch.Jfx[mr]; Uo = ch.U[mg]; eo = ch.Esum[mr];
+                        // accepted when the energy rises by less than wb (at least 1: never uphill by 0)
+                        const u64 thr = __shfl_sync(0xffffffffu, sr.thr, ls), M = (u64)(Ecur > dm.SC ? Ecur : dm.SC);
+                        const u64 bh = __umul64hi(thr, M), bl = thr * M;
+                        wb = (i64)((bh << 32) | (bl >> 32));
+                        wb = wb > 1 ? wb : 1;
+                        if ((__shfl_sync(0xffffffffu, sr.flags, ls) & 4u) || (bh >> 31)) wb = 0x7fffffffffffffffll;
+                        if (ident) { dA = (aC + bS * (wt2 + wti)) * (wt2 - wti); if (second) dA = -dA; }
+                        else { const i64 da1 = __shfl_sync(0xffffffffu, dA1, ls), da2 = __shfl_sync(0xffffffffu, dA2, ls); dA = second && touchW ? da2 : da1; }
+                    };
+                    if (!(COMP && LPL == 1)) look();
                     int4 d[NCH], w1[NCH], w2[NCH];
                     i64 E1 = 0, E2 = 0;
                     if (touchW) {
@@ -490,60 +512,42 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                             E2 = warp_sum_i64(E2);
                         }
                     }
-                    // ---- exact new score and the Metropolis decision, in the lane that proposed the step --------------
-                    i64 n0 = 0, n1 = 0, n2 = 0, J1n = 0, J2n = 0, U1n = 0, U2n = 0, e1o = 0, e2o = 0, en = 0;
-                    int fb = 0, g1 = 0, g2 = 0;
-                    bool acc = false;
-                    if (lane == ls) {
-                        const i64 S0 = ch.Sc[0], S1 = ch.Sc[1], S2 = ch.Sc[2], Ecur = ch.Sc[3];
-                        g1 = g_of[c1]; g2 = g_of[c2];
-                        const i64 J1o = ch.Jfx[rg1], J2o = ch.Jfx[rg2], U1o = ch.U[g1], U2o = ch.U[g2];
-                        e1o = ch.Esum[rg1]; e2o = ch.Esum[rg2];
-                        const i64 dJ1 = dA1 + (touchW ? dm.EC * (E1 - e1o) : 0), dJ2 = touchW ? dA2 + dm.EC * (E2 - e2o) : 0;
-                        J1n = J1o + dJ1; J2n = touchW ? J2o + dJ2 : J1n;
-                        U1n = U1o + dJ1 + (g1 == g2 ? dJ2 : 0); U2n = g1 == g2 ? U1n : U2o + dJ2;
-                        n1 = S1 + dJ1 + dJ2;
-                        {
-                            const i64 newmax = U1n > U2n ? U1n : U2n, oldmax = U1o > U2o ? U1o : U2o;
-                            n0 = newmax;
-                            if (newmax < S0) { if (oldmax < S0) n0 = S0; else fb |= 1; }
-                        }
-                        {
-                            const i64 newmax = J1n > J2n ? J1n : J2n, oldmax = J1o > J2o ? J1o : J2o;
-                            n2 = newmax;
-                            if (newmax < S2) { if (oldmax < S2) n2 = S2; else fb |= 2; }
-                        }
-                        en = row_energy(n0, n1, n2);
-                        acc = rp_lex_less(n0, n1, n2, S0, S1, S2) || en - Ecur < bound;
-                        if (!acc) fb = 0;
-                    }
-                    // where the previous maximum sat on a changed entry and fell, the maximum is searched anew (it can
-                    // only be larger than what was just used: a candidate rejected with the smaller one stays rejected)
-                    fb = __shfl_sync(0xffffffffu, fb, ls);
-                    if (fb) {
-                        const unsigned gg = __shfl_sync(0xffffffffu, (unsigned)g1 | ((unsigned)g2 << 16), ls);
+                    // ---- exact new score and the Metropolis decision: all lanes come to the same result (both cells in one
+                    // row-shard: both kinds of lanes see all of the change) --------------------------------------------
+                    if (COMP && LPL == 1) look();
+                    const i64 Em = second ? E2 : E1;
+                    const i64 dJ = dA + (touchW ? dm.EC * (Em - eo) : 0), dJo = touchW ? __shfl_xor_sync(0xffffffffu, dJ, 1) : 0;
+                    const int og = __shfl_xor_sync(0xffffffffu, mg, 1);
+                    const i64 Jn = Jo + dJ, Un = Uo + dJ + (mg == og ? dJo : 0), Jx = __shfl_xor_sync(0xffffffffu, Jn, 1), Ux = __shfl_xor_sync(0xffffffffu, Un, 1);
+                    const i64 n1 = S1 + dJ + dJo;
+                    i64 n0 = Un > Ux ? Un : Ux, n2 = Jn > Jx ? Jn : Jx;
+                    // where the previous maximum sat on a changed entry and fell, the maximum is searched anew, if the candidate is
+                    // not rejected with the smaller one already
+                    const bool fb0 = __any_sync(0xffffffffu, Uo >= S0) && n0 < S0, fb2 = __any_sync(0xffffffffu, Jo >= S2) && n2 < S2;
+                    if (!fb0 && n0 < S0) n0 = S0;
+                    if (!fb2 && n2 < S2) n2 = S2;
+                    i64 en = row_energy(n0, n1, n2);
+                    bool acc = rp_lex_less(n0, n1, n2, S0, S1, S2) || en - Ecur < wb;
+                    if (acc && (fb0 || fb2)) {
                         i64 v0 = 0, v2 = 0;
-                        if (fb & 1) {
-                            for (int g = lane; g < dm.G; g += 32) if (g != (int)(gg & 0xffffu) && g != (int)(gg >> 16)) { const i64 v = ch.U[g]; if (v > v0) v0 = v; }
+                        if (fb0) {
+                            const int ga = __shfl_sync(0xffffffffu, mg, 0), gb = __shfl_sync(0xffffffffu, mg, 1);
+                            for (int g = lane; g < dm.G; g += 32) if (g != ga && g != gb) { const i64 v = ch.U[g]; if (v > v0) v0 = v; }
                             v0 = warp_max_nonneg_i64(v0);
                         }
-                        if (fb & 2) {
+                        if (fb2) {
                             for (int rg = lane; rg < dm.RG; rg += 32) if (rg != r1 && rg != r2) { const i64 v = ch.Jfx[rg]; if (v > v2) v2 = v; }
                             v2 = warp_max_nonneg_i64(v2);
                         }
-                        if (lane == ls) {
-                            if (v0 > n0) n0 = v0;
-                            if (v2 > n2) n2 = v2;
-                            en = row_energy(n0, n1, n2);
-                            acc = rp_lex_less(n0, n1, n2, ch.Sc[0], ch.Sc[1], ch.Sc[2]) || en - ch.Sc[3] < bound;
-                        }
+                        if (v0 > n0) n0 = v0;
+                        if (v2 > n2) n2 = v2;
+                        en = row_energy(n0, n1, n2);
+                        acc = rp_lex_less(n0, n1, n2, S0, S1, S2) || en - Ecur < wb;
                     }
-                    if (!__any_sync(0xffffffffu, acc)) continue;
+                    if (!acc) continue;
                     // ---- commit -----------------------------------------------------------------------------------
                     win = ls;
                     n_acc += 1;
-                    const unsigned dd = __shfl_sync(0xffffffffu, (unsigned)c1 | ((unsigned)c2 << 16), ls);
-                    const int d1 = (int)(dd & 0xffffu), d2 = (int)(dd >> 16);
                     if (touchW) {
                         int o1 = 0, o2 = 0;
                         if (!CHIP) {
@@ -571,42 +575,39 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                             }
                     }
                     int better = 0;
-                    if (lane == ls) {
+                    const int wdf = __shfl_sync(0xffffffffu, df, ls);
+                    if (lane < 2) {
                         // (all loads before the first store: the compiler cannot tell the arrays apart)
-                        const int k = kb + ls;
-                        const i64 dq = (i64)t2 * t2 - (i64)ti * ti;
+                        const int k = kb + ls, up = second ? 1 : -1, dt = second ? wti - wt2 : wt2 - wti;
+                        const i64 dq = (i64)wt2 * wt2 - (i64)wti * wti;
                         ChainR *bk = ch.book;
-                        const int T1 = ch.T[c1], T2 = ch.T[c2], m1 = ch.cnt[c1], m2 = ch.cnt[c2], nlog = bk->nlog, n_imp = bk->n_imp;
-                        const u64 Q1 = ch.Q[c1], Q2 = ch.Q[c2], dig = bk->dig;
-                        const i64 a1 = ch.Afx[rg1], a2 = ch.Afx[rg2], k1 = ch.slack[rg1], k2 = ch.slack[rg2];
+                        const int T = ch.T[mc], m = ch.cnt[mc], nlog = bk->nlog, n_imp = bk->n_imp;
+                        const u64 Q = ch.Q[mc], dig = bk->dig;
+                        const i64 af = ch.Afx[mr], sk = ch.slack[mr], at = ident ? 0 : ch.att[mc];
                         const i64 B0 = bk->B[0], B1 = bk->B[1], B2 = bk->B[2];
-                        const i64 t1 = ident ? 0 : ch.att[c1], t3 = ident ? 0 : ch.att[c2];
-                        const u32 second = swap ? (u32)wi2 : (u32)c2;
-                        const u64 code = ((u64)(swap ? 0 : 1) << 63) ^ ((u64)(u32)k << 40) ^ ((u64)(u32)wi << 20) ^ (u64)second;
-                        cells[wi] = (unsigned short)c2;
-                        if (swap) cells[wi2] = (unsigned short)c1;
-                        else { ch.cnt[c1] = m1 - 1; ch.cnt[c2] = m2 + 1; }
-                        ch.T[c1] = T1 + t2 - ti; ch.T[c2] = T2 + ti - t2;
-                        ch.Q[c1] = Q1 + (u64)dq; ch.Q[c2] = Q2 - (u64)dq;
-                        if (!ident) { const i64 da = (aC + bS * (t2 + ti)) * (t2 - ti); ch.att[c1] = t1 + da; ch.att[c2] = t3 - da; }
-                        ch.Afx[rg1] = a1 + dA1; ch.Jfx[rg1] = J1n;
-                        if (touchW) {
-                            ch.slack[rg1] = k1 + E1 - e1o + df; ch.slack[rg2] = k2 + E2 - e2o - df;
-                            ch.Esum[rg1] = E1; ch.Esum[rg2] = E2;
-                            ch.Afx[rg2] = a2 + dA2; ch.Jfx[rg2] = J2n;
+                        const u32 other = swap ? (u32)wi2 : (u32)d2;
+                        const u64 code = ((u64)(swap ? 0 : 1) << 63) ^ ((u64)(u32)k << 40) ^ ((u64)(u32)wi << 20) ^ (u64)other;
+                        if (!second || swap) cells[second ? wi2 : wi] = (unsigned short)(second ? d1 : d2);
+                        if (!swap) ch.cnt[mc] = m + up;
+                        ch.T[mc] = T + dt;
+                        ch.Q[mc] = second ? Q - (u64)dq : Q + (u64)dq;
+                        if (!ident) { const i64 da = (aC + bS * (wt2 + wti)) * (wt2 - wti); ch.att[mc] = second ? at - da : at + da; }
+                        ch.Afx[mr] = af + dA; ch.Jfx[mr] = Jn;
+                        if (touchW) { ch.slack[mr] = sk + Em - eo + (second ? -wdf : wdf); ch.Esum[mr] = Em; }
+                        ch.U[mg] = Un;
+                        if (lane == 0) {
+                            ch.Sc[0] = n0; ch.Sc[1] = n1; ch.Sc[2] = n2; ch.Sc[3] = en;
+                            if (!CHIP && nlog < A.log_cap) A.log[(size_t)j * A.log_cap + nlog] = make_uint2((u32)wi, other | (swap ? 0u : 0x80000000u));
+                            bk->nlog = nlog + 1;
+                            bk->dig = (dig ^ code) * 0x100000001B3ull;
+                            if (rp_lex_less(n0, n1, n2, B0, B1, B2)) {
+                                bk->B[0] = n0; bk->B[1] = n1; bk->B[2] = n2;
+                                bk->best_step = k + 1; bk->best_nlog = nlog + 1;
+                                bk->n_imp = n_imp + 1;
+                                if (CHIP) better = rp_lex_less(n0, n1, n2, inc_s[0], inc_s[1], inc_s[2]) ? 1 : 0;
+                            }
+                            if (touchW) n_rows += 2;
                         }
-                        ch.U[g1] = U1n; ch.U[g2] = U2n;
-                        ch.Sc[0] = n0; ch.Sc[1] = n1; ch.Sc[2] = n2; ch.Sc[3] = en;
-                        if (!CHIP && nlog < A.log_cap) A.log[(size_t)j * A.log_cap + nlog] = make_uint2((u32)wi, second | (swap ? 0u : 0x80000000u));
-                        bk->nlog = nlog + 1;
-                        bk->dig = (dig ^ code) * 0x100000001B3ull;
-                        if (rp_lex_less(n0, n1, n2, B0, B1, B2)) {
-                            bk->B[0] = n0; bk->B[1] = n1; bk->B[2] = n2;
-                            bk->best_step = k + 1; bk->best_nlog = nlog + 1;
-                            bk->n_imp = n_imp + 1;
-                            if (CHIP) better = rp_lex_less(n0, n1, n2, inc_s[0], inc_s[1], inc_s[2]) ? 1 : 0;
-                        }
-                        if (touchW) n_rows += 2;
                     }
                     // the cached cells of the steps still to come follow the move
                     {
@@ -617,7 +618,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                             if (x < n && sr.i[x] == wi2) sr.c[x] = d1;      // (no sample is -1; wi2 != wi, their cells differ)
                         }
                     }
-                    __syncwarp();                               // the deciding lane's updates are visible
+                    __syncwarp();                               // the updates are visible
                     if (!ident && lane < 2 * dm.S) {
                         const bool b = lane >= dm.S;
                         const int c = b ? d2 : d1;
