@@ -186,6 +186,44 @@ __device__ __forceinline__ i64 row_energy(i64 s0, i64 s1, i64 s2)       // rp_en
 // registers of 12.
 #define ROW_CHAINS_PER_SM(LPL, CPL) ((LPL) * (CPL) == 1 ? 14 : 12)
 
+// The level barrier of up to 32 members by one warp, a member a lane: incumbent (inc, *win = its slot or -1), then, unless this
+// was the last level, ancestors of members m0 .. m1-1.  No CTA-wide barrier between its parts (tiny 333 -> 308 us a plan); with
+// eight members a lane one warp takes longer than eight do with their barriers (medium 913 -> 978 us).
+__device__ __forceinline__ void row_barrier_warp(const AnnealArgs &A, int P, const u64 *eL, const i64 *bestL, bool last, u64 cq, u32 resample_x,
+                                                 int m0, int m1, i64 *inc, int *win, int *anc, int lane)
+{
+    const u64 r = lane < P ? __ldcg(eL + lane) : 0x7fffffffffffffffull;
+    const i64 e[1] = { (i64)(r & ~(1ull << 63)) };
+    i64 b0 = inc[0], b1 = inc[1], b2 = inc[2];
+    int bj = 0x7fffffff;
+    if (r >> 63) {                               // its trajectory best beats the incumbent
+        b0 = __ldcg(bestL + 3 * lane); b1 = __ldcg(bestL + 3 * lane + 1); b2 = __ldcg(bestL + 3 * lane + 2);
+        bj = lane;
+    }
+    const u32 hi = (u32)((u64)e[0] >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
+    const i64 emin = (i64)(((u64)mh << 32) | __reduce_min_sync(0xffffffffu, hi == mh ? (u32)e[0] : 0xffffffffu));
+    int slot = -1;
+    if (__any_sync(0xffffffffu, bj != 0x7fffffff)) {
+        slot = le_lexmin_lane(b0, b1, b2, bj);
+        if (lane == slot) { inc[0] = b0; inc[1] = b1; inc[2] = b2; }
+    }
+    if (lane == 0) *win = slot;                  // that chain stored its trajectory-best layout in its row of cand_layout
+    if (last) return;
+    const u64 M = (u64)(emin > A.dm.SC ? emin : A.dm.SC);
+    u64 w[1];
+    le_weights<1>(e, emin, M, cq, w);
+    u64 F = lane < P ? w[0] : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const u64 x = __shfl_up_sync(0xffffffffu, F, o); if (lane >= o) F += x; }
+    const u64 Ftot = __shfl_sync(0xffffffffu, F, 31), u0 = (u64)(((unsigned __int128)resample_x * Ftot) >> 32);
+    for (int m = m0; m < m1; ++m) {
+        // slots with P * F <= at (those past the last member hold the total: never)
+        const unsigned __int128 at = (unsigned __int128)u0 + (unsigned __int128)m * Ftot;
+        const int n = __popc(__ballot_sync(0xffffffffu, (unsigned __int128)P * F <= at));
+        if (lane == 0) anc[m] = n;
+    }
+}
+
 // LPL layers per lane, CPL 16-byte chunks per layer (X.cpl <= CPL of them in use).
 template <int LPL, int CPL, bool CHIP, bool COMP>
 __global__ void __launch_bounds__(CHIP ? ROW_THREADS : 32, CHIP ? 1 : ROW_CHAINS_PER_SM(LPL, CPL))
@@ -734,6 +772,13 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
         __shared__ u64 rsum[LE_MAX_WARPS];
         __shared__ u64 carry_s;
         __shared__ int win_s;
+        const bool all_anc = blockIdx.x == 0 && A.lo.tr_anc;        // the first CTA writes the traces
+        const int m0 = all_anc ? 0 : blockIdx.x * cw, m1 = all_anc ? P : min(P, m0 + cw);
+        if (P <= 32) {
+            if (warp == 0) row_barrier_warp(A, P, eL, bestL, last, lv.cq, lv.resample_x, m0, m1, inc_s, &win_s, le_anc, lane);
+            __syncthreads();
+            if (win_s >= 0) inc_slot = win_s;
+        } else {
         // incumbent: the lowest slot among the lexicographically best trajectory-best scores, if it beats it
         i64 b0 = inc_s[0], b1 = inc_s[1], b2 = inc_s[2], emin = 0x7fffffffffffffffll, e_mine = emin;
         int bj = 0x7fffffff;
@@ -776,7 +821,6 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
         __syncthreads();
         if (win_s >= 0) inc_slot = win_s;
         // Boltzmann weights, cumulative weights, ancestors (not after the last level)
-        const bool all_anc = blockIdx.x == 0 && A.lo.tr_anc;        // the first CTA writes the traces
         if (!last) {
             const u64 M = (u64)(emin > dm.SC ? emin : dm.SC);
             auto en_of = [&](int m) { return (i64)(__ldcg(eL + m) & ~(1ull << 63)); };
@@ -785,7 +829,6 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
             else le_prefix_weights_of<4>(P, en_of, lv.cq, tid, NT, emin, M, le_F, rsum, &carry_s);
             const u64 Ftot = le_F[P - 1];
             const u64 u0 = (u64)(((unsigned __int128)lv.resample_x * Ftot) >> 32);
-            const int m0 = all_anc ? 0 : blockIdx.x * cw, m1 = all_anc ? P : min(P, m0 + cw);
             for (int m = m0 + tid; m < m1; m += NT) {
                 const unsigned __int128 at = (unsigned __int128)u0 + (unsigned __int128)m * Ftot;
                 int lo = 0, hi = P - 1;
@@ -796,6 +839,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                 le_anc[m] = lo;
             }
             __syncthreads();
+        }
         }
         // per-level traces (inspection hook), by the first CTA
         if (blockIdx.x == 0 && A.lo.tr_term) {
