@@ -215,12 +215,11 @@ def plan_once(rp, w, t_in, a_in, outs, stream, stages=None, knobs=None):
         rp.rp_debug_set_knob(ctx, k, v)
     rp.rp_place_experts(ctx, outs["pi"], outs["rank_load"])
     rp.rp_pack_rows(ctx)
-    if stages is not None:
-        stages["chain_kernel"] = rp.rp_debug_chain_kernel(ctx)
     stats = rp.rp_anneal(ctx, n_levels=s.n_levels, steps_per_level=s.steps_per_level, t0=s.t0,
                          t_ratio=s.t_ratio, p_reloc=s.p_reloc, p_guide=s.p_guide, want_stats=True)
     rp.rp_best(ctx, outs["layout"], outs["score_fx"], outs["score_f64"])
     if stages is not None:
+        stages["chain_kernel"] = rp.rp_debug_chain_kernel(ctx)      # (compressed rows: known once they have been annealed)
         for k, v in rp.rp_debug_stage_times(ctx).items():
             if v is not None:
                 stages[k] = stages.get(k, 0.0) + v
@@ -334,6 +333,13 @@ def measure(rp, torch, args, name, steps, min_seconds, dist, dev, local, cpu_sec
                 "launch_ms": per_launch_s * 1e3, "launches_per_step": nl / steps,
                 "levels_per_launch": s.n_levels * steps / nl, "share_of_step": res["chain_ms"] / res["ms"]}
     prof = profiled_traffic(chain_kernel, s.name)
+    if chain_kernel == "k_anneal_row":
+        # Its move bytes are the rows that feasible moves name; most moves are rejected without reading them, so they are
+        # no traffic: the fraction is that of the captured DRAM bytes, null where there is no capture.
+        roofline["named_gbs"] = achieved
+        roofline["bound"] = "instruction issue and latency of a chain's rounds"
+        roofline["achieved"] = roofline["frac"] = None
+        roofline["served_by"] = "cell statistics on chip; L2+HBM for the moves that are scored (see dram)"
     if prof:
         scale = s.pop_size / float(prof["population"])
         dram = prof["dram_bytes_per_launch"] * scale
@@ -343,6 +349,9 @@ def measure(rp, torch, args, name, steps, min_seconds, dist, dev, local, cpu_sec
                             "hbm_frac": dram / per_launch_s / 1e9 / peak,
                             "l2_bytes_per_launch": prof.get("lts_bytes_per_launch", 0) * scale or None,
                             "captured_dram_gbs": prof.get("dram_gbs"), "captured_l2_gbs": prof.get("lts_gbs")}
+        if chain_kernel == "k_anneal_row":
+            roofline["achieved"] = dram / per_launch_s / 1e9
+            roofline["frac"] = roofline["achieved"] / peak
     n_le = s.n_samples * s.n_layers * s.n_experts * 4
     n_lp = s.n_samples * s.n_layers * s.ep_width * 4
     front = {}
@@ -516,7 +525,7 @@ def eval_stage(rp, torch, name, dev, l2_gbs, reps=10):
     gathered = s.pop_size * q_bytes
     hbm_min = s.pop_size * s.n_samples * 4 + q_bytes          # int32 layouts in, demand rows once
     return {"workload": name, "layouts": s.pop_size, "ms": ms, "layouts_per_s": s.pop_size / ms * 1e3,
-            "roofline": {"bound": "l2", "kernel": "k_eval", "achieved": gathered / ms / 1e6, "peak": l2_gbs, "unit": "GB/s",
+            "roofline": {"bound": "l2", "kernel": "k_eval_group, k_eval_sum, k_eval_score", "achieved": gathered / ms / 1e6, "peak": l2_gbs, "unit": "GB/s",
                          "frac": gathered / ms / 1e6 / l2_gbs, "peak_source": "read rate of a 32 MiB L2-resident buffer measured in this run (rp_debug_l2_read_rate)",
                          "gathered_bytes_per_launch": gathered, "hbm_bytes_per_launch_min": hbm_min,
                          "hbm_min_gbs": hbm_min / ms / 1e6, "hbm_min_frac": hbm_min / ms / 1e6 / peak}}

@@ -26,11 +26,11 @@
 //    row-shards nearly all satisfy it (checked on the device, see rp_launch_rows): 16 bytes per layer
 //    instead of 4*P: an eighth of the traffic at 32 ranks.
 //  * No staging area, so 12 to 16 chains per SM instead of 5 to 10.
-// What bounds it now: with 16 chains per SM (heavy) the instructions of a round, about 5600 cycles with four
-// warps per scheduler; with 7 (large) their latency, about 4900 cycles; launched once for all levels (medium)
-// about 2900 cycles a round and 25 us a level for the barrier and the states.  A level's time before (the
-// warp-per-chain kernel; medium: warp per candidate) and now: heavy 15.0 -> 4.8 ms, wide 1.2 -> 0.55 ms,
-// large 0.21 -> 0.16 ms, medium 50 -> 38 us (plans of perf/cases.py: 301 -> 98, 24.0 -> 12.3, 4.8 -> 3.8, 1.12 -> 0.98 ms).
+// What bounds it now: with 14 to 16 chains per SM (heavy) the instructions of a round, about 4900 cycles with four
+// warps per scheduler; with 7 (large) their latency, about 3900 cycles; launched once for all levels (medium)
+// about 2700 cycles a round and 20 us a level for the slowest chain, the barrier and the states.  A level's time before (the
+// warp-per-chain kernel; medium: warp per candidate) and now: heavy 15.0 -> 3.9 ms, wide 1.2 -> 0.41 ms,
+// large 0.21 -> 0.13 ms, medium 50 -> 36 us (plans: 301 -> 78, 24.0 -> 8.3, 4.8 -> 2.8, 1.12 -> 0.87 ms).
 // Step for step this is the sequential chain: proposals are evaluated against the current state,
 // feasible ones are decided in step order, and the speculation is redone after an acceptance.
 //
