@@ -181,6 +181,8 @@ k_level_turn(const AnnealArgs A, const TurnArgs T)
 // for one another would make them wait for its SMs, so the parts then stay launches of their own, as beyond the table on chip.
 bool rp_row_turns(const rp_ctx *c) { return c->knob_level_launches != 1 && c->Ppop <= TURN_MAX_MEMBERS; }
 
+int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A);
+
 // Between level A.level of an rp_anneal call and the next one.
 int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A0)
 {
@@ -208,7 +210,12 @@ int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A0)
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    RP_CUDA(cudaLaunchKernelEx(&cfg, k_level_turn, A, T));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_level_turn, A, T);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {        // a part of a GPU: the launches one by one, at every level
+        cudaGetLastError();
+        return rp_launch_level_end(c, A0);
+    }
+    RP_CUDA(e);
     ++g_rp_launches;
     c->slices_listed = 1;
     return RP_OK;
