@@ -253,7 +253,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
     const int L = dm.L, cpl = CPL == 1 ? 1 : X.cpl, rc = L * cpl;        // 16-byte chunks per layer and per row
     const int rot = (CPL > 1 && (cpl & (cpl - 1)) == 0) ? cpl - 1 : 0;   // lanes start at different chunks: fewer bank conflicts
     const bool ident = dm.own_shard;
-    const bool sum32 = (i64)L * dm.k * dm.C * ((dm.D + dm.G - 1) / dm.G) < (1ll << 31);
+    const bool sum32 = dm.sum32;
     const i64 aC = dm.asum * dm.C, bS = dm.bsum;
     const float aCf = (float)aC, bSf = (float)bS, ECf = (float)dm.EC;
     const int4 *qr = (const int4 *)X.qr;

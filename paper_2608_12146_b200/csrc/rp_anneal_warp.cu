@@ -197,7 +197,7 @@ k_anneal_warp(const AnnealArgs A, const RpWarpLayout wl)
     if (__ldcg(&A.status[RP_SW_TIMEOUT])) return;                  // the call has failed already: nothing to do
     const int src = min(max(A.anc[j], 0), A.Ppop - 1);
     const int LP = dm.LP, nchunks = LP >> 2, cpl = dm.P >> 2;      // 16-byte chunks per slice and per layer
-    const bool sum32 = (i64)dm.L * dm.k * dm.C * ((dm.D + dm.G - 1) / dm.G) < (1ll << 31);
+    const bool sum32 = dm.sum32;
     // The chain's assignment: the 16-bit array of its blob, read and written through L2.
     unsigned short *cells = (unsigned short *)(A.blob_dst + (size_t)j * A.bl.bytes + A.bl.off_cell);
     u32 phase = 0;

@@ -145,7 +145,7 @@ k_anneal_wpc(const AnnealArgs A)
     // A rank load is at most k*C tokens per cell of the row-shard (conservation of the demand
     // rows, token cap), so the sum over layers of the busiest ranks usually fits 32 bits and
     // the warp can add it up with one reduction instruction.
-    const bool sum32 = (i64)dm.L * dm.k * dm.C * ((dm.D + dm.G - 1) / dm.G) < (1ll << 31);
+    const bool sum32 = dm.sum32;
 
     const int P = A.Ppop;
     const int n_levels = PERSIST ? A.n_levels : 1;

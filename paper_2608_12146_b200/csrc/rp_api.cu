@@ -346,9 +346,14 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
     memcpy(c->pack_out, c->h_pin + 10, sizeof(int) * 4);
 
     // fixed-point range of the score: s1 <= (2^8*C*L*k + (asum+bsum)*C) * sum t  must stay below 2^62
-    const double total = (double)c->h_pin[8];
+    c->tokens = c->h_pin[8];
+    const double total = (double)c->tokens;
     double bound = ((double)dm.EC * L * dm.k + (double)(dm.asum + dm.bsum) * dm.C) * total;
     if (bound >= 4.0e18) return RP_ERR_RANGE;
+    // A row-shard holds at most C tokens in each of its shard's slots, and shards need not be of one size: the largest
+    // decides.  (Scoring also takes layouts whose cells are too full, see eval_launch.)
+    const double shard_tokens = (double)dm.C * maxshard;
+    dm.sum32 = (double)L * dm.k * (shard_tokens < total ? shard_tokens : total) < 2147483648.0;
     return RP_OK;
 }
 

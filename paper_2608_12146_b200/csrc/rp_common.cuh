@@ -42,6 +42,7 @@ struct RpDims {
     int R, K, RG, LP;                   // rows, cells R*D, row-shards R*G, L*P (set after packing)
     int slices;                         // rank loads kept as shared slices (set after packing; see AnnealArgs)
     int own_shard;                      // DP slot d is shard d: a cell and its row-shard have the same index
+    int sum32;                          // the busiest loads of all layers of a feasible row-shard add up to less than 2^31
     i64 ahat[RP_MAX_STAGES], bhat[RP_MAX_STAGES];
     i64 asum, bsum;                     // sums over stages (attention key of a cell)
     i64 SC;                             // 2^8 * C^2
@@ -122,6 +123,7 @@ struct rp_ctx {
     int *d_seed_layout;        // [N]
     int *d_order;              // [N] samples sorted by (-t, i)
     int Rstar, certified;
+    i64 tokens;                // sum of the lengths
     i64 seed_score[3];
     // population
     RpPopBuf buf[2];

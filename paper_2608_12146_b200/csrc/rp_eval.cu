@@ -228,14 +228,13 @@ k_eval_group(const EvalArgs A)
 // one strip, at a time took 127 to 175 us for 256 layouts (46 instructions per sample and strip; 20 per sample and three strips here).
 template <int NS, int U>
 __global__ void __launch_bounds__(EVAL_THREADS, NS == 1 ? 4 : (NS == 2 ? 3 : 2))
-k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt)
+k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt, bool sum32)
 {
     const RpDims &dm = A.dm;
     const int lane = threadIdx.x & 31, RG = dm.RG, rc = dm.LP >> 2;
     const bool vec = eval_vec(dm);
     const int groups = (RG + rpt - 1) / rpt, per = groups * sgroups;
     const int cpl = dm.P >> 2, used = vec ? (32 / cpl) * cpl : 32;
-    const bool sum32 = (i64)dm.L * dm.k * dm.C * ((dm.D + dm.G - 1) / dm.G) < (1ll << 31);
     for (unsigned task = blockIdx.x * (EVAL_THREADS / 32) + (threadIdx.x >> 5); task < (unsigned)n * (unsigned)per; task += gridDim.x * (EVAL_THREADS / 32)) {
         const int lay = (int)(task / (unsigned)per), r = (int)(task - (unsigned)lay * per), sg = r % sgroups, rg0 = r / sgroups * rpt, nr = min(rpt, RG - rg0);
         const int *go = A.off + (size_t)lay * (RG + 1) + rg0;
@@ -271,18 +270,19 @@ k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt)
         int x = 0, end = __shfl_sync(0xffffffffu, ends, 0);
         auto close = [&]() {                // row-shard rg0 + x is complete
             const size_t at = (size_t)lay * RG + rg0 + x;
-            int own = 0;
+            u32 own = 0, high = 0;          // sum of this lane's layers (see eval_launch); where it may pass 32 bits, its 16-bit halves
 #pragma unroll
             for (int z = 0; z < NS; ++z) {
                 const bool o = (on >> z) & 1u;
                 if (A.W_out && o) ((int4 *)(A.W_out + at * dm.LP))[(sg * NS + z) * used + lane] = a[z];
                 const int m = eval_layer_max(o ? max(max(a[z].x, a[z].y), max(a[z].z, a[z].w)) : 0, lane, cpl);
-                own += o && lane % cpl == 0 ? m : 0;          // (a layer's busiest load fits 31 bits, three of them 32)
+                const u32 v = o && lane % cpl == 0 ? (u32)m : 0u;
+                if (sum32) own += v;
+                else { own += v & 0xffffu; high += v >> 16; }
                 a[z] = make_int4(0, 0, 0, 0);
             }
-            i64 es;
-            if (sum32) es = (i64)__reduce_add_sync(0xffffffffu, (unsigned)own);
-            else { es = (i64)(unsigned)own; for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o); }
+            i64 es = (i64)__reduce_add_sync(0xffffffffu, own);
+            if (!sum32) es += (i64)__reduce_add_sync(0xffffffffu, high) << 16;
             if (lane == 0) {
                 if (sgroups > 1) atomicAdd((u64 *)(A.Esum + at), (u64)es);
                 else A.Esum[at] = es;
@@ -434,6 +434,9 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
         if (fm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_score, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
         const int cpl = dm.P >> 2, used = eval_vec(dm) ? 32 / cpl * cpl : 32, strips = eval_vec(dm) ? ((dm.LP >> 2) + used - 1) / used : 1;
         const int ns = std::min(3, strips), sgroups = (strips + ns - 1) / ns, warps = ns == 1 ? 32 : (ns == 2 ? 24 : 16);     // per SM
+        // What a warp adds up for a row-shard: the busiest loads of its layers, each at most k times the tokens of the window
+        // (a layout handed in may put them all into one cell).
+        const bool sum32 = eval_vec(dm) && (double)std::min(dm.L, ns * used / cpl) * dm.k * (double)c->tokens < 4294967296.0;
         for (int first = 0; first < n; first += 16384) {                 // (bounds the task numbers of a launch)
             EvalArgs B = A;
             const int m = std::min(16384, n - first);
@@ -448,9 +451,9 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
             const long long want = ((long long)m * ((dm.RG + rpt - 1) / rpt) * sgroups + 7) / 8;
             const int grid = (int)std::min<long long>(want, 148 * warps / 8);
             k_eval_group<<<m, GROUP_THREADS, gm, c->stream>>>(B);
-            if (ns == 1) k_eval_sum<1, 8><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt);
-            else if (ns == 2) k_eval_sum<2, 4><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt);
-            else k_eval_sum<3, 4><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt);
+            if (ns == 1) k_eval_sum<1, 8><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt, sum32);
+            else if (ns == 2) k_eval_sum<2, 4><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt, sum32);
+            else k_eval_sum<3, 4><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt, sum32);
             k_eval_score<<<m, EVAL_THREADS, fm, c->stream>>>(B);
             g_rp_launches += 2;
         }

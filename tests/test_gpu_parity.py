@@ -11,7 +11,7 @@ import pytest
 
 import oracle
 import paper_2608_12146_b200.binding as rp
-from paper_2608_12146_b200.windows import custom_spec, make_window
+from paper_2608_12146_b200.windows import Window, custom_spec, make_window
 
 pytestmark = pytest.mark.gpu
 F64_RTOL = 1e-9
@@ -1230,3 +1230,64 @@ def test_between_two_levels_at_the_edges(N, D, min_rows, edp, pop, levels):
         if knob == 0:
             assert stats.kernel_launches == 2 * levels + 2
         rp.rp_destroy(ctx)
+
+
+def one_heavy_expert(name, t, L, E, k, C, D, P, pop, share, **kw):
+    """A window of given lengths whose first expert takes `share` of every sample's routing."""
+    s = custom_spec(name, len(t), L, E, k, C, D, P, pop, 0, **kw)
+    a = np.zeros((len(t), L, E), np.int64)
+    rng = np.random.default_rng(len(t) + L)
+    total = k * t.astype(np.int64)
+    a[:, :, 0] = (share * total).astype(np.int64)[:, None]
+    rest = (total - a[:, 0, 0])[:, None, None] // (E + 3) + rng.integers(0, 50, (len(t), L, E - 1))
+    a[:, :, 1:] = rest
+    a[:, :, E - 1] += total[:, None] - a.sum(axis=2)
+    assert (a >= 0).all() and (a.sum(axis=2) == total[:, None]).all()
+    return Window(s, t.astype(np.int32), np.ascontiguousarray(a.astype(np.int32)))
+
+
+UNEVEN = [0] * 17 + list(range(1, 16))
+
+
+@pytest.mark.parametrize("n", [5, 1300])
+@pytest.mark.parametrize("case", ["uneven_shards", "overfull_cells"])
+def test_busiest_loads_that_add_up_beyond_32_bits(case, n):
+    """A row-shard's busiest loads over all layers pass 32 bits: a shard with 17 of 32 slots where the even share is two,
+    and layouts that put everything into one cell; both scoring forms."""
+    rng = np.random.default_rng(n)
+    if case == "uneven_shards":
+        w = one_heavy_expert(case, rng.integers(300_000, 340_000, 40), 120, 4, 8, 1 << 20, 32, 4, 2, 0.55)
+        edp, slots = UNEVEN, 17
+    else:
+        w = one_heavy_expert(case, rng.integers(300_000, 500_000, 64), 100, 8, 2, 1 << 20, 4, 4, 2, 0.9)
+        edp, slots = None, 1
+    s = w.spec
+    ref = oracle_front(w, edp)
+    ctx = load(w, pop=2, edp=edp)
+    check_front(w, ctx, ref)
+    K = ref["R"] * s.dp_width
+    lays = rng.integers(0, K, (n, s.n_samples)).astype(np.int32)
+    lays[1::2] = rng.integers(0, slots, (n // 2, s.n_samples))       # all of it in the first shard of the first row
+    fx, _ = rp.rp_eval_population(ctx, lays)
+    some = np.r_[0:5, n - 3:n]
+    ev = oracle.eval_layouts(w.lengths, ref["q"], lays[some], ref["R"], s.token_cap, s.dp_width, edp, s.alpha, s.beta)
+    assert ev["W"].max(axis=-1).sum(axis=-1, dtype=np.int64).max() >= 1 << 32
+    assert (fx[some] == ev["score"]).all()
+    rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("kernel", [0, 1, 2])
+def test_annealing_of_a_shard_with_most_of_the_slots(kernel):
+    """The same map under annealing: rank loads and slacks of the large shard beyond 2^31 on every chain kernel."""
+    rng = np.random.default_rng(3)
+    w = one_heavy_expert("uneven_anneal", rng.integers(250_000, 420_000, 40), 120, 4, 8, 1 << 20, 32, 4, 12, 0.9)
+    s = w.spec
+    ref = oracle_front(w, UNEVEN)
+    ev = oracle.eval_layouts(w.lengths, ref["q"], ref["seed"], ref["R"], s.token_cap, s.dp_width, UNEVEN, s.alpha, s.beta)
+    assert ev["W"].max(axis=-1).sum(axis=-1, dtype=np.int64).max() >= 1 << 32
+    ctx = load(w, pop=12, edp=UNEVEN)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", kernel)
+    check_front(w, ctx, ref)
+    _, stats = check_anneal(w, ctx, ref, UNEVEN, 12, 4, 60, t_ratio=0.6)
+    assert stats.accepted > 0
+    rp.rp_destroy(ctx)
