@@ -644,7 +644,7 @@ int rp_launch_anneal_level(rp_ctx *c, int level, int n_levels, const rp_anneal_p
 #define COOP_LAUNCH(MINB_, SL_, ID_)                                                                                 \
     do {                                                                                                     \
         if (smem > 32 * 1024)                                                                                \
-            RP_CUDA(cudaFuncSetAttribute(k_anneal_level<128, MINB_, SL_, ID_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+            RP_CUDA(cudaFuncSetAttribute(k_anneal_level<128, MINB_, SL_, ID_>, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT)); \
         k_anneal_level<128, MINB_, SL_, ID_><<<c->Ppop, 128, smem, c->stream>>>(A);                          \
     } while (0)
     const int minb = rp_coop_chains_per_sm(c->dm);

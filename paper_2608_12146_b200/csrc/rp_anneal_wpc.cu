@@ -721,7 +721,7 @@ static int launch_wpc(rp_ctx *c, const AnnealArgs &A, int ws, size_t smem, int c
 #define LAUNCH(WS_, CH_)                                                                              \
     do {                                                                                              \
         if (smem > 32 * 1024)                                                                         \
-            RP_CUDA(cudaFuncSetAttribute(k_anneal_wpc<NW, WS_, CH_, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+            RP_CUDA(cudaFuncSetAttribute(k_anneal_wpc<NW, WS_, CH_, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT)); \
         cudaLaunchConfig_t cfg;                                                                       \
         memset(&cfg, 0, sizeof cfg);                                                                  \
         cfg.gridDim = dim3(c->Ppop); cfg.blockDim = dim3(NW * 32);                                    \
@@ -764,7 +764,7 @@ template <int NW, int CH>
 static int launch_wpc_all(rp_ctx *c, const AnnealArgs &A, size_t smem, int *done)
 {
     auto kern = k_anneal_wpc<NW, true, CH, true>;
-    if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT));
     int per_sm = 0, sms = 0;
     RP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem));
     RP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));

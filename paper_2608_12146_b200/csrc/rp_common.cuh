@@ -10,6 +10,10 @@
 #define RP_FBITS 8              // fraction bits of the attention coefficients
 #define RP_MAX_EDP 1024         // G upper bound
 #define RP_MAX_EP 1024          // P upper bound
+// Dynamic shared memory a kernel is opted in to, above anything its launches ask for (227 KB per CTA on sm_100a, less static
+// arrays).  The limit belongs to the function and not to the launch: contexts that plan different windows at once on different
+// host threads would lower each other's if it followed the window at hand.
+#define RP_SMEM_LIMIT (220 * 1024)
 
 typedef unsigned long long u64;
 typedef long long i64;

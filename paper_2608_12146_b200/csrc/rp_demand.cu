@@ -571,7 +571,7 @@ int rp_launch_project(rp_ctx *c)
     size_t smem = (size_t)K3_WARPS * dm.E * sizeof(int);
     if ((size_t)(K3_WARPS + dm.L) * dm.E * sizeof(int) <= 96 * 1024) smem += (size_t)dm.L * dm.E * sizeof(int);
     if (smem > 32 * 1024)
-        RP_CUDA(cudaFuncSetAttribute(k_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        RP_CUDA(cudaFuncSetAttribute(k_project, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT));
     long long rows = (long long)dm.N * dm.L;
     long long want = (rows + K3_WARPS - 1) / K3_WARPS;
     int grid = (int)(want < 148 * 8 ? want : 148 * 8);

@@ -261,7 +261,7 @@ int rp_launch_pack_on(rp_ctx *c, cudaStream_t stream)
     int *fill_g = nullptr;
     if (smem > 160 * 1024) { keys_g = c->d_sort_keys; fill_g = (int *)(c->d_sort_keys + n_pow2); smem = 0; }
     if (smem > 32 * 1024)
-        RP_CUDA(cudaFuncSetAttribute(k_pack_ffd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        RP_CUDA(cudaFuncSetAttribute(k_pack_ffd, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT));
     // small windows: fewer warps make the block-wide barriers of the sort cheaper
     const int threads = n_pow2 >= PACK_THREADS ? PACK_THREADS : (n_pow2 < 256 ? 256 : n_pow2);
     // The order by counting on the whole GPU from 513 samples (below, the sort in the packing kernel is cheaper than a

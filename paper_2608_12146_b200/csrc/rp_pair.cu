@@ -265,7 +265,7 @@ int rp_launch_edp_pair(rp_ctx *c, const int *lay_in, int *lay_out, int *prof, in
     const size_t smem = rp_pair_smem_bytes(dm);
     if (smem > 200 * 1024) return RP_ERR_RANGE;
     if (smem > 32 * 1024)
-        RP_CUDA(cudaFuncSetAttribute(k_edp_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        RP_CUDA(cudaFuncSetAttribute(k_edp_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT));
     const unsigned short *rg_of = (const unsigned short *)(c->d_static + c->sl.off_rg);
     k_edp_pair<<<count, PAIR_THREADS, smem, c->stream>>>(dm, c->d_q, rg_of, lay_in, lay_out, prof, c->d_W, first, width,
                                                          (u32)c->cfg.seed, (u32)(c->cfg.seed >> 32));

@@ -150,7 +150,7 @@ int rp_launch_seed_trials(rp_ctx *c, int width, int *layouts, int *ok)
     while ((32 << lb) < dm.K) ++lb;
     const size_t smem = lb > 4 ? sizeof(u64) * (size_t)SEED_WARPS * ((32 << lb) + 32) : 0;
     if (smem > 200 * 1024) return RP_ERR_RANGE;
-    if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_seed_trials<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_seed_trials<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT));
     auto fn = lb > 4 ? k_seed_trials<0> : lb == 4 ? k_seed_trials<16> : lb == 3 ? k_seed_trials<8> : lb == 2 ? k_seed_trials<4> : k_seed_trials<2>;
     const int grid = (c->Ppop + SEED_WARPS - 1) / SEED_WARPS;
     fn<<<grid, SEED_WARPS * 32, smem, c->stream>>>(c->d_t, c->d_order, c->d_seed_layout, dm, width, lb,

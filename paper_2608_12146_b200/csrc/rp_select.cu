@@ -495,7 +495,7 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
     if (st == RP_OK && smem > 200 * 1024) st = RP_ERR_RANGE;
     cudaError_t e = cudaSuccess;
     if (st == RP_OK) {
-        if (smem > 32 * 1024) e = cudaFuncSetAttribute(k_sel_prepare, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (smem > 32 * 1024) e = cudaFuncSetAttribute(k_sel_prepare, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT);
         if (e == cudaSuccess) {
             k_sel_signs<<<(F * n_proj + 255) / 256, 256, 0, c->stream>>>(F, n_proj, (u32)c->cfg.seed, (u32)(c->cfg.seed >> 32), sgn);
             k_sel_prepare<<<(int)P, SEL_THREADS, smem, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_anc, c->d_W, c->d_wloc,
@@ -509,7 +509,7 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
             const size_t rtab = std::min<size_t>(sizeof(int) * (size_t)dm.R * dm.R, std::max<size_t>(8 * 1024, sizeof(int) * (size_t)dm.R));
             const size_t ctab = std::min<size_t>(sizeof(int) * (size_t)dm.K * dm.K, std::max<size_t>((72 * 1024 - rtab) / 4 * 4, sizeof(int) * (size_t)dm.K));
             const void *fn = dm.N <= 65535 ? (const void *)k_sel_dist<u32> : (const void *)k_sel_dist<u64>;
-            if (ctab + rtab > 32 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(ctab + rtab));
+            if (ctab + rtab > 32 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT);
             if (e == cudaSuccess) {
                 const size_t items = P * ((P + SEL_CHUNK - 1) / SEL_CHUNK);
                 const int grid = (int)std::min<size_t>(items, (size_t)148 * 3);

@@ -1291,3 +1291,50 @@ def test_annealing_of_a_shard_with_most_of_the_slots(kernel):
     _, stats = check_anneal(w, ctx, ref, UNEVEN, 12, 4, 60, t_ratio=0.6)
     assert stats.accepted > 0
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("stage", ["selection", "packing"])
+def test_kernels_with_window_sized_shared_memory_on_two_threads(stage):
+    """Two host threads, each with a window of its own size, the same stage over and over: the shared-memory limit of a
+    kernel that asks for as much as its window needs must not follow the other thread's window."""
+    import threading
+    import torch
+
+    def call(ctx):
+        if stage == "packing":
+            return np.array(rp.rp_pack_rows(ctx))
+        nd, order = rp.rp_select_population(ctx)
+        return np.r_[nd, order]
+
+    jobs = []
+    for N, D, min_rows in ((500, 16, 15), (220, 10, 10)) if stage == "selection" else ((5000, 8, 0), (3000, 8, 0)):
+        w = make_window(custom_spec("two_threads", N, 2, 8, 2, 4096, D, 4, 6, 0, data_seed=N))
+        s = w.spec
+        pair = []
+        for _ in range(2):                       # one for the reference run, one for the thread
+            ctx = rp.rp_window_load(torch.from_numpy(w.lengths).cuda(), torch.from_numpy(w.demand).cuda(), top_k=s.top_k,
+                                    token_cap=s.token_cap, dp_width=D, ep_width=4, pop_size=6, min_rows=min_rows, seed=3,
+                                    stream=torch.cuda.Stream())
+            rp.rp_place_experts(ctx)
+            rp.rp_pack_rows(ctx)
+            if stage == "selection":
+                rp.rp_seed_population(ctx, 4)
+            pair.append(ctx)
+        jobs.append((pair[1], [call(pair[0]) for _ in range(5)]))
+    errors = []
+
+    def worker(ctx, want):
+        try:
+            for n in range(3000):
+                got = call(ctx)
+                if n < len(want):
+                    assert (got == want[n]).all()
+        except Exception as e:          # reported by the main thread
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=worker, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
