@@ -413,7 +413,7 @@ void rp_decide_layouts(rp_ctx *c)
     c->row_mode = 0;
     if (c->knob_chain_kernel == 0 && c->knob_slices == 0) {
         if (c->knob_level_launches != 1 && rp_row_fits_chip(c, c->bl, c->sl)) c->row_mode = 1;
-        else if (rp_row_kind(dm) && (dm.slices || c->knob_level_launches != 1)) { c->row_mode = 2; dm.slices = 1; }
+        else if (rp_row_kind(dm) && (dm.slices || c->knob_level_launches != 1) && rp_row_fits_level(c, c->bl, c->sl)) { c->row_mode = 2; dm.slices = 1; }
     }
     if (dm.slices) rp_make_layouts(dm, &c->bl, &c->sl);
 }

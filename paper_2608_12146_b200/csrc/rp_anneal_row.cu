@@ -1046,6 +1046,23 @@ int rp_row_kind(const RpDims &dm)
     return 0;
 }
 
+// Whether the form that launches once per level is taken by the shared memory of a chain (a warp to itself).  Where DP slot d is
+// shard d, as far as it fits: it is the fastest kernel even with one chain per SM (L = 24, P = 16, 1024 members, three levels of
+// 200 steps: 63 KB 1.39 ms and 1.71 for the next best kernel, 117 KB 3.8 and 4.8, 140 KB 4.1 and 4.9; L = P = 32, 2048 members,
+// three of 100: 94 KB 2.2 and 3.0, 136 KB 6.0 and 8.1).  Else the attention of a shard's slots is looked up
+// (8*K + 18*R*G*S bytes more, S stages a move) and four-warp CTAs overtake it: with up to two stages where an SM holds fewer than
+// two chains (107 KB 2.3 ms and 2.9, 133 KB 3.7 and 3.2, 166 KB 4.9 and 4.3), with more where it holds fewer than three (four
+// stages 72 KB 1.82 and 1.83, 107 KB 2.61 and 2.52; eight stages 54 KB 1.94 and 1.85, 81 KB 2.6 and 2.2, 161 KB 5.4 and 3.1).
+bool rp_row_fits_level(const rp_ctx *c, const RpBlob &bl, const RpStatic &sl)
+{
+    RowArgs X;
+    memset(&X, 0, sizeof X);
+    X.comp = rp_row_kind(c->dm) == 2;
+    chain_layout(c->dm, bl, sl, X, false, 1, c->Ppop, 0);
+    const int limit = c->dm.own_shard ? ROW_SMEM_MAX : 227 * 1024 / (c->dm.S <= 2 ? 2 : 3) - 1024;
+    return X.smem_bytes <= limit;
+}
+
 // Whether rows are kept apart from the rank loads that scoring writes: padded or compressed.
 bool rp_row_separate(const rp_ctx *c)
 {

@@ -292,6 +292,7 @@ bool rp_may_use_row(const rp_ctx *c);
 bool rp_uses_row(const rp_ctx *c);
 bool rp_row_compressed(const rp_ctx *c);
 bool rp_row_fits_chip(const rp_ctx *c, const RpBlob &bl, const RpStatic &sl);
+bool rp_row_fits_level(const rp_ctx *c, const RpBlob &bl, const RpStatic &sl);
 int rp_row_kind(const RpDims &dm);
 bool rp_row_separate(const rp_ctx *c);
 size_t rp_row_ints(const rp_ctx *c);

@@ -1338,3 +1338,26 @@ def test_kernels_with_window_sized_shared_memory_on_two_threads(stage):
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+SHARD31 = list(range(31)) + [0]
+PERM32 = [(d + 1) % 32 for d in range(32)]
+
+
+@pytest.mark.parametrize("N,L,P,min_rows,edp,S,row", [
+    (2400, 24, 32, 72, SHARD31, 2, False),      # 235 KB a chain with one layer per lane: more than an SM has
+    (1300, 24, 16, 36, PERM32, 8, False),       # 241 KB
+    (1300, 24, 16, 32, PERM32, 2, True), (1300, 24, 16, 36, PERM32, 2, False),      # two chains to an SM, and no longer two
+    (700, 24, 16, 16, PERM32, 4, True), (700, 24, 16, 17, PERM32, 4, False)])       # three
+def test_windows_whose_chains_do_not_fit_one_layer_per_lane(N, L, P, min_rows, edp, S, row):
+    """Many cells under a shard map that is not the identity: the one-layer-per-lane kernel is chosen by the shared memory
+    of its chain, and what it does not take is annealed by the kernels for such windows."""
+    w = make_window(custom_spec("big_maps", N, L, P, 2, 8192, 32, P, 5, 0, data_seed=N + S, alpha=(1.0,) * S,
+                                beta=tuple(x / S for x in range(S))))
+    ref = oracle_front(w, edp, min_rows)
+    ctx = load(w, edp=edp, min_rows=min_rows)
+    check_front(w, ctx, ref)
+    assert (rp.rp_debug_chain_kernel(ctx) == "k_anneal_row") == row
+    _, stats = check_anneal(w, ctx, ref, edp, 5, 3, 50, t_ratio=0.6, check_members=1)
+    assert stats.accepted > 0
+    rp.rp_destroy(ctx)
