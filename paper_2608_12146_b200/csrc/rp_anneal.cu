@@ -604,7 +604,7 @@ int rp_upload_levels(rp_ctx *c, int n_levels)
     }
     const cudaError_t e = cudaMemcpyAsync(c->d_levels, h, bytes, cudaMemcpyHostToDevice, c->stream);
     if (bytes > RP_MAIL_BYTES / 2) free(h);            // pageable source: staged before the call returned
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     return RP_OK;
 }
 

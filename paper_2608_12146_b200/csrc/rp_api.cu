@@ -260,13 +260,13 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
         if (rp_is_device_ptr(lengths)) c->d_t = lengths;
         else {
             if ((st = dev_alloc(c, &c->own_t, N)) != RP_OK) break;
-            if (cudaMemcpyAsync(c->own_t, lengths, sizeof(int) * N, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) { st = RP_ERR_CUDA; break; }
+            if (const cudaError_t e = cudaMemcpyAsync(c->own_t, lengths, sizeof(int) * N, cudaMemcpyHostToDevice, c->stream)) { st = rp_fail(e); break; }
             c->d_t = c->own_t;
         }
         if (rp_is_device_ptr(demand)) c->d_a = demand;
         else {
             if ((st = dev_alloc(c, &c->own_a, n_a)) != RP_OK) break;
-            if (cudaMemcpyAsync(c->own_a, demand, sizeof(int) * n_a, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) { st = RP_ERR_CUDA; break; }
+            if (const cudaError_t e = cudaMemcpyAsync(c->own_a, demand, sizeof(int) * n_a, cudaMemcpyHostToDevice, c->stream)) { st = rp_fail(e); break; }
             c->d_a = c->own_a;
         }
         // everything sized by the window alone comes out of one allocation
@@ -300,7 +300,7 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
         c->d_dp_off = c->d_dp_list + D;
         // input checks + aggregate expert load + token total in one pass over the demand tensor,
         // put in flight before the rest of the set-up
-        if (cudaMemsetAsync(c->d_load_slab, 0, n_zero, c->stream) != cudaSuccess) { st = RP_ERR_CUDA; break; }
+        if (const cudaError_t e = cudaMemsetAsync(c->d_load_slab, 0, n_zero, c->stream)) { st = rp_fail(e); break; }
         stage_mark(c, RP_EV_K1_0, c->stream);
         if ((st = rp_launch_check_reduce(c)) != RP_OK) break;
         stage_mark(c, RP_EV_K1_1, c->stream);
@@ -311,7 +311,7 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
         memcpy(tab + 2 * D, off, sizeof(int) * (G + 1));
         const cudaError_t e = cudaMemcpyAsync(c->d_edp, tab, sizeof(int) * n_tab, cudaMemcpyHostToDevice, c->stream);
         if (n_tab * sizeof(int) > RP_MAIL_BYTES / 2) free(tab);            // pageable source: staged before the call returns
-        if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; st = RP_ERR_CUDA; break; }
+        if (e != cudaSuccess) { st = rp_fail(e); break; }
     } while (0);
     free(edp); free(off); free(list);
     RP_TRY(st);
@@ -603,7 +603,7 @@ extern "C" int rp_eval_population(rp_ctx *c, const int32_t *layouts, int32_t n, 
     if (layouts && !rp_is_device_ptr(layouts)) {
         RP_TRY(dev_alloc(c, &tmp, (size_t)n * dm.N));
         cudaError_t e = cudaMemcpyAsync(tmp, layouts, sizeof(int) * (size_t)n * dm.N, cudaMemcpyHostToDevice, c->stream);
-        if (e != cudaSuccess) { dev_free(c, tmp); g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+        if (e != cudaSuccess) { dev_free(c, tmp); return rp_fail(e); }
         dl = tmp;
     }
     // Results straight to where they are wanted: device outputs, or the second half of the pinned mail area.
@@ -669,7 +669,7 @@ static int install_population(rp_ctx *c, const int *lay, int n_distinct = 0)
     cudaError_t e = cudaSuccess;
     if (st == RP_OK) e = cudaMemcpyAsync(c->d_seed_score, best, sizeof(i64) * 3, cudaMemcpyDeviceToDevice, c->stream);
     dev_free(c, best);
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     return st;
 }
 
@@ -696,7 +696,7 @@ extern "C" int rp_seed_population(rp_ctx *c, int32_t choice_width, int32_t *n_ow
     if (st == RP_OK && e == cudaSuccess) for (size_t j = 0; j < P; ++j) own += h_ok[j];
     free(h_ok);
     dev_free(c, lay); dev_free(c, ok);
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     RP_TRY(st);
     if (n_own) *n_own = own;
     return RP_OK;
@@ -750,7 +750,7 @@ extern "C" int rp_pair_population(rp_ctx *c, int32_t choice_width, int32_t *n_ch
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     }
     dev_free(c, lay); dev_free(c, out); dev_free(c, prof); dev_free(c, cnt);
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     RP_TRY(st);
     if (n_changed) *n_changed = h_cnt;
     return RP_OK;
@@ -794,7 +794,7 @@ extern "C" int rp_select_population(rp_ctx *c, int32_t n_proj, int64_t eta_q16, 
     free(h);
     dev_free(c, lay); dev_free(c, out); dev_free(c, d_order); dev_free(c, d_nd);
     if (!c->trace_on) { dev_free(c, c->d_sel_dist); c->d_sel_dist = nullptr; }      // kept for inspection only
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     return st;
 }
 
@@ -894,7 +894,7 @@ extern "C" int rp_init_population(rp_ctx *c, int32_t n_candidates, int32_t choic
         const int st2 = build_population(c, false, true);
         if (st == RP_OK && e == cudaSuccess) st = st2;
     }
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     return st;
 }
 
@@ -942,6 +942,7 @@ static int rebuild_rank_loads(rp_ctx *c)
     k_iota<<<(int)((P + 255) / 256), 256, 0, c->stream>>>(c->d_anc, (int)P, 0);
     g_rp_launches += 3;
     RP_CUDA(cudaGetLastError());
+    c->full_stale = 0; c->rows_current = 0; c->row_members = c->Ppop;
     return RP_OK;
 }
 
@@ -1010,15 +1011,24 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     const bool row = rp_uses_row(c);
     if (!row) st = need_rank_loads(c, 2 * P, true);
     if (st == RP_OK && !row && c->full_stale) st = rebuild_rank_loads(c);
-    if (!row) c->rows_current = 0;
-    c->row_members = c->Ppop;                  // after a level every member has a state of its own
-    c->full_stale = row && rp_row_separate(c);
+    // What the context says about the population changes with the levels that have run, and with nothing that was refused
+    // before them: a call that fails here can be followed by one that does not.
+    auto levels_ran = [&]() {
+        if (!row) c->rows_current = 0;
+        c->row_members = c->Ppop;              // after a level every member has a state of its own
+        c->full_stale = row && rp_row_separate(c);
+    };
     if (st == RP_OK && (rp_uses_wpc(c->dm) || (row && c->row_mode == 1)) && c->knob_level_launches != 1) st = rp_upload_levels(c, NL);
     if (stats) cudaEventRecord(ev[0], c->stream);
     if (st == RP_OK) st = rp_launch_anneal_all(c, NL, p, rho_q32, guide_q32, &all_in_one);
-    if (all_in_one) c->cur = (c->cur + NL) & 1;       // the kernel has left both ancestor tables and both cell tables current
+    if (all_in_one) { c->cur = (c->cur + NL) & 1; levels_ran(); }       // the kernel has left both ancestor tables and both cell tables current
     for (int n = 0; n < NL && st == RP_OK && !all_in_one; ++n) {
         st = rp_launch_anneal_level(c, n, NL, p, rho_q32, guide_q32);
+        if (st != RP_OK) {
+            if (n > 0 || st == RP_ERR_CUDA) c->stage = 2;      // part of a level may have been queued: only rp_pack_rows makes sense now
+            break;
+        }
+        levels_ran();
         c->cur = 1 - c->cur;          // the terminal states are the next level's sources
         { int *sw = c->d_anc; c->d_anc = c->d_anc_next; c->d_anc_next = sw; }
         { int *sw = c->d_wloc; c->d_wloc = c->d_wloc_next; c->d_wloc_next = sw; }
@@ -1036,7 +1046,7 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
         if (e == cudaSuccess) cudaEventElapsedTime(&ms_chains, ev[0], ev[1]);
         if (!side) for (int x = 0; x < 2; ++x) cudaEventDestroy(ev[x]);
     }
-    if (st == RP_OK && e != cudaSuccess) { g_rp_last_cuda_error = (int)e; st = RP_ERR_CUDA; }
+    if (st == RP_OK && e != cudaSuccess) st = rp_fail(e);
     RP_TRY(st);
     if (sw[RP_SW_POOL]) { c->stage = 2; c->best_ready = 0; return RP_ERR_STATE; }     // slice pool exhausted: an internal invariant broke
     if (sw[RP_SW_TIMEOUT]) {
@@ -1276,7 +1286,7 @@ extern "C" int rp_debug_dump(rp_ctx *c, int what, int32_t index, void *buf, int6
     if (need) e = cudaMemcpyAsync(buf, src, need, cudaMemcpyDefault, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dev_free(c, tmp);
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     return RP_OK;
 }
 
@@ -1347,7 +1357,7 @@ extern "C" int rp_debug_l2_read_rate(int64_t bytes, int32_t reps, double *gb_per
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaFree(buf); cudaFree(sink);
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     *gb_per_s = (double)bytes * reps / (ms * 1e-3) / 1e9;
     return RP_OK;
 }
@@ -1364,7 +1374,7 @@ static int dbg_map(const TI *in, size_t in_per, TO *out, size_t out_per, int64_t
     if (e == cudaSuccess) { launch(din, dout); ++g_rp_launches; e = cudaGetLastError(); }
     if (e == cudaSuccess) e = cudaMemcpy(out, dout, sizeof(TO) * n * out_per, cudaMemcpyDefault);
     cudaFree(din); cudaFree(dout);
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     return RP_OK;
 }
 

@@ -24,13 +24,18 @@ typedef unsigned int u32;
 // ---------------------------------------------------------------------------------------
 extern thread_local int g_rp_last_cuda_error;
 extern long long g_rp_launches;
+// An error is handed over once: left with the runtime, the next launch check of this thread (the library's or its caller's)
+// would report it again.
+static inline int rp_fail(cudaError_t e)
+{
+    cudaGetLastError();
+    g_rp_last_cuda_error = (int)e;
+    return RP_ERR_CUDA;
+}
 #define RP_CUDA(call)                                                    \
     do {                                                                 \
         cudaError_t e_ = (call);                                         \
-        if (e_ != cudaSuccess) {                                         \
-            g_rp_last_cuda_error = (int)e_;                              \
-            return RP_ERR_CUDA;                                          \
-        }                                                                \
+        if (e_ != cudaSuccess) return rp_fail(e_);                       \
     } while (0)
 #define RP_TRY(call)                                                     \
     do {                                                                 \

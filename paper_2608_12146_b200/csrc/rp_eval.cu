@@ -730,7 +730,7 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
         out->joint = (double)h.s0 / (double)dm.SC;
     } while (0);
     cudaFreeAsync(buf, c->stream);
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     return st;
 }
 

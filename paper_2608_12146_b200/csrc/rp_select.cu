@@ -529,6 +529,6 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
     dev_free(c, B.canon); dev_free(c, B.hash); dev_free(c, B.clist); dev_free(c, B.cstart); dev_free(c, B.rlist);
     dev_free(c, B.rstart); dev_free(c, B.pc); dev_free(c, B.pr); dev_free(c, B.phi); dev_free(c, sgn); dev_free(c, rep);
     dev_free(c, mind); dev_free(c, pen); dev_free(c, B.lab); dev_free(c, B.big);
-    if (e != cudaSuccess) { g_rp_last_cuda_error = (int)e; return RP_ERR_CUDA; }
+    if (e != cudaSuccess) return rp_fail(e);
     return st;
 }

@@ -1361,3 +1361,40 @@ def test_windows_whose_chains_do_not_fit_one_layer_per_lane(N, L, P, min_rows, e
     _, stats = check_anneal(w, ctx, ref, edp, 5, 3, 50, t_ratio=0.6, check_members=1)
     assert stats.accepted > 0
     rp.rp_destroy(ctx)
+
+
+def test_a_call_that_fails_for_memory_leaves_the_population_as_it_is():
+    """51000 members whose rank loads fit the GPU as compressed rows (6 GB) and not in full form (200 GB): a kernel that
+    needs the full form is refused, before any level has run and after some, and the next call goes on from where the
+    population stands, as in a context that was never asked for more."""
+    import torch
+    N, L, P, D, R, pop = 200, 32, 128, 8, 15, 51000
+    rng = np.random.default_rng(8)
+    t = rng.integers(20, 200, N).astype(np.int32)
+    p = np.full((L, P), 0.35 / (P - 3))
+    for l in range(L):
+        p[l, rng.choice(P, 3, replace=False)] = (0.3, 0.2, 0.15)
+    a = rng.multinomial((20 * t.astype(np.int64))[:, None], p).astype(np.int32)
+    runs = []
+    for refused in (True, False):
+        ctx = rp.rp_window_load(t, a, top_k=20, token_cap=2048, dp_width=D, ep_width=P, pop_size=pop, min_rows=R, seed=4)
+        rp.rp_place_experts(ctx)
+        assert rp.rp_pack_rows(ctx)[0] == R
+        out = []
+        for levels in (2, 3):
+            if refused:
+                rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 1)
+                with pytest.raises(rp.RpError) as err:
+                    rp.rp_anneal(ctx, n_levels=2, steps_per_level=5, t0=1e-3, t_ratio=0.5, p_reloc=0.2, p_guide=0.8)
+                assert err.value.status == -6
+                rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 0)
+                torch.zeros(1, device="cuda").add_(1)            # the failure does not turn up in the caller's next launch
+            st = rp.rp_anneal(ctx, n_levels=levels, steps_per_level=8, t0=1e-3, t_ratio=0.5, p_reloc=0.2, p_guide=0.8)
+            assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and st.accepted > 0
+            out += [np.array([st.proposed, st.feasible, st.accepted, st.improved]), rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32),
+                    *rp.rp_best(ctx)]
+        runs.append(out)
+        rp.rp_destroy(ctx)
+        rp.rp_release_cached_memory()
+    for x, y in zip(*runs):
+        assert (x == y).all()
