@@ -305,7 +305,7 @@ def rp_debug_stage_times(ctx: Context) -> dict:
 
 
 KNOB = dict(BARRIER_WORKSPACE=1, WAIT_POLLS=2, STALL_ONE_CHAIN=3, RANK_LOAD_SLICES=4, LAUNCH_PER_LEVEL=5,
-            CHAIN_KERNEL=6)
+            CHAIN_KERNEL=6, RESIDENT_SMS=7)
 
 
 def rp_debug_set_knob(ctx: Context, knob: str, value: int):

@@ -485,7 +485,7 @@ int rp_launch_slice_gc(rp_ctx *c)
     k_slice_holders<<<c->Ppop, 128, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, c->dm.RG, c->Ppop, ns, c->d_wcount,
                                                     c->d_wfree_head, c->d_status);
     k_slice_free_list<<<nb, SLICE_BLOCK, 0, c->stream>>>(c->d_wcount, c->d_wref, ns, c->d_wfree, c->d_wfree_head, c->d_status);
-    g_rp_launches += 2;
+    g_rp_launches += 2; c->n_queued += 2;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
 }
@@ -621,8 +621,7 @@ int rp_launch_anneal_all(rp_ctx *c, int n_levels, const rp_anneal_params *prm, u
     fill_args(c, 0, n_levels, prm, rho_q32, guide_q32, A);
     if (rp_uses_row(c)) {
         if (c->row_mode != 1) return RP_OK;
-        RP_TRY(rp_launch_anneal_row_all(c, A, done));
-        return *done ? RP_OK : RP_ERR_STATE;
+        return rp_launch_anneal_row_all(c, A, done);
     }
     if (!use_wpc(c->dm)) return RP_OK;
     return rp_launch_anneal_wpc_all(c, A, done);
@@ -657,7 +656,7 @@ int rp_launch_anneal_level(rp_ctx *c, int level, int n_levels, const rp_anneal_p
     else { if (alias) { COOP_PICK(false, true) } else { COOP_PICK(false, false) } }
 #undef COOP_PICK
 #undef COOP_LAUNCH
-    ++g_rp_launches;
+    ++g_rp_launches; ++c->n_queued;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
 }

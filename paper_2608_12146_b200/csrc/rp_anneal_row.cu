@@ -984,7 +984,7 @@ static int row_chunks(const RpDims &dm, int cpl)
     return l * c;
 }
 
-static int row_chains_per_cta(int pop) { return pop <= 148 ? 1 : (pop <= 296 ? 2 : (pop <= 592 ? 4 : 8)); }
+static int row_chains_per_cta(int pop, int sms) { return pop <= sms ? 1 : (pop <= 2 * sms ? 2 : (pop <= 4 * sms ? 4 : 8)); }
 
 static void chain_layout(const RpDims &dm, const RpBlob &bl, const RpStatic &sl, RowArgs &X, bool chip, int cw, int pop, int steps)
 {
@@ -1025,15 +1025,15 @@ static void full_rows(const RpDims &dm, RowArgs &X)
 
 // One launch for all levels, the chains' rank loads on chip: at most eight chunks per lane, every chain resident at once.
 #define ROW_SMEM_MAX (220 * 1024)
-bool rp_row_fits_chip(const rp_ctx *c, const RpBlob &bl, const RpStatic &sl)
+bool rp_row_fits_chip(rp_ctx *c, const RpBlob &bl, const RpStatic &sl)
 {
     RowArgs X;
     memset(&X, 0, sizeof X);
     full_rows(c->dm, X);
-    const int nch = row_chunks(c->dm, X.cpl);
-    if (nch < 1 || nch > 8 || c->Ppop > 148 * ROW_MAX_WARPS || c->dm.N > 16384) return false;
-    const int cw = row_chains_per_cta(c->Ppop);
-    chain_layout(c->dm, bl, sl, X, true, cw, c->Ppop, 0);
+    const int nch = row_chunks(c->dm, X.cpl), sms = rp_sms(c);          // (a CTA to an SM)
+    if (nch < 1 || nch > 8 || c->Ppop > sms * ROW_MAX_WARPS || c->dm.N > 16384) return false;
+    c->row_cw = row_chains_per_cta(c->Ppop, sms);
+    chain_layout(c->dm, bl, sl, X, true, c->row_cw, c->Ppop, 0);
     return X.smem_bytes <= ROW_SMEM_MAX;
 }
 
@@ -1136,6 +1136,8 @@ static int launch_row_t(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int gr
     RP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_SMEM_MAX));
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
+    *done = 0;
+    if (CHIP && grid > rp_sms(c)) return RP_OK;
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = X.smem_bytes; cfg.stream = c->stream;
     cudaLaunchAttribute at[1];
@@ -1145,21 +1147,21 @@ static int launch_row_t(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int gr
         cfg.attrs = at; cfg.numAttrs = 1;
     }
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, A, X);
-    if (CHIP && e == cudaErrorCooperativeLaunchTooLarge) { cudaGetLastError(); *done = 0; return RP_OK; }
+    if (CHIP && e == cudaErrorCooperativeLaunchTooLarge) { cudaGetLastError(); return RP_OK; }
     RP_CUDA(e);
-    ++g_rp_launches;
+    ++g_rp_launches; ++c->n_queued;
     *done = 1;
     return RP_OK;
 }
 
-// One launch for all levels; *done = 0 when the chains cannot all be resident (an invariant of the choice
-// made when the population was built: the caller reports it).
+// One launch for all levels; *done = 0 when the chains cannot all be resident: fewer SMs are free than the device reported when
+// the population was built (a part of a GPU).  The caller then takes another kernel.
 int rp_launch_anneal_row_all(rp_ctx *c, const AnnealArgs &A0, int *done)
 {
     AnnealArgs A = A0;
     RowArgs X;
     row_args(c, X);
-    const int cw = row_chains_per_cta(c->Ppop);
+    const int cw = c->row_cw;
     // step records ahead of time as far as shared memory goes
     for (int steps = std::min(A.steps, 256);; steps /= 2) {
         chain_layout(c->dm, c->bl, c->sl, X, true, cw, c->Ppop, steps);

@@ -521,7 +521,7 @@ int rp_launch_anneal_warp(rp_ctx *c, AnnealArgs &A)
     A.smem_bytes = (unsigned)wl.bytes;
     if (identity) RP_TRY(launch_warp<true>(c, A, wl));
     else RP_TRY(launch_warp<false>(c, A, wl));
-    ++g_rp_launches;
+    ++g_rp_launches; ++c->n_queued;
     return rp_launch_level_end(c, A);
 }
 
@@ -535,7 +535,7 @@ int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A)
     B.smem_bytes = (unsigned)ws;
     RP_CUDA(cudaFuncSetAttribute(k_level_end, cudaFuncAttributeMaxDynamicSharedMemorySize, WARP_SMEM_OPTIN));
     k_level_end<<<1, LEVEL_END_THREADS, ws, c->stream>>>(B);
-    ++g_rp_launches;
+    ++g_rp_launches; ++c->n_queued;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
 }

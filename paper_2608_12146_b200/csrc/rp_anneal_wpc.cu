@@ -735,7 +735,7 @@ static int launch_wpc(rp_ctx *c, const AnnealArgs &A, int ws, size_t smem, int c
     if (ws) { if (chunks <= 1) LAUNCH(true, 1); else if (chunks <= 2) LAUNCH(true, 2); else LAUNCH(true, 4); }
     else { if (chunks <= 1) LAUNCH(false, 1); else if (chunks <= 2) LAUNCH(false, 2); else LAUNCH(false, 4); }
 #undef LAUNCH
-    ++g_rp_launches;
+    ++g_rp_launches; ++c->n_queued;
     RP_CUDA(cudaGetLastError());
     return RP_OK;
 }
@@ -765,10 +765,9 @@ static int launch_wpc_all(rp_ctx *c, const AnnealArgs &A, size_t smem, int *done
 {
     auto kern = k_anneal_wpc<NW, true, CH, true>;
     if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT));
-    int per_sm = 0, sms = 0;
+    int per_sm = 0;
     RP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem));
-    RP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
-    if ((long long)per_sm * sms < c->Ppop) return RP_OK;
+    if ((long long)per_sm * rp_sms(c) < c->Ppop) return RP_OK;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3(c->Ppop); cfg.blockDim = dim3(NW * 32);
@@ -780,7 +779,7 @@ static int launch_wpc_all(rp_ctx *c, const AnnealArgs &A, size_t smem, int *done
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, A);
     if (e == cudaErrorCooperativeLaunchTooLarge) { cudaGetLastError(); return RP_OK; }
     RP_CUDA(e);
-    ++g_rp_launches;
+    ++g_rp_launches; ++c->n_queued;
     *done = 1;
     return RP_OK;
 }

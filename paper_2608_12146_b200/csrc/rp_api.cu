@@ -376,7 +376,10 @@ extern "C" int rp_window_load(rp_ctx **out, const rp_config *cfg, const int32_t 
 
     rp_ctx *c = (rp_ctx *)calloc(1, sizeof(rp_ctx));
     if (!c) return RP_ERR_ARG;
-    if (cudaGetDevice(&c->device) != cudaSuccess) { free(c); return RP_ERR_CUDA; }
+    if (cudaGetDevice(&c->device) != cudaSuccess || cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
+        free(c);
+        return RP_ERR_CUDA;
+    }
     c->stream = (cudaStream_t)cuda_stream;
     c->cfg = *cfg;
     c->cfg.edp_of_dp = nullptr; c->cfg.alpha = nullptr; c->cfg.beta = nullptr;
@@ -961,12 +964,6 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     make_schedule(p, c->h_levels);
     const u64 rho_q32 = (u64)floor(p->p_reloc * 4294967296.0);
     const u64 guide_q32 = (u64)floor(p->p_guide * 4294967296.0);
-    // accepted-move log (not kept by the launch that runs all levels with one layer per lane)
-    if (c->log_cap < p->steps_per_level && !(rp_may_use_row(c) && c->row_mode == 1)) {
-        dev_free(c, c->d_log); c->d_log = nullptr; c->log_cap = 0;
-        RP_TRY(dev_alloc(c, &c->d_log, P * (size_t)p->steps_per_level));
-        c->log_cap = p->steps_per_level;
-    }
     // per-level trace (only when the inspection hook asked for it)
     free_trace(c);
     if (c->trace_on) {
@@ -996,21 +993,38 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     int st = RP_OK;
     // One launch for all levels where every chain can be resident at once, else one launch per level.
     int all_in_one = 0;
-    // Which kernel: the one-layer-per-lane kernel where the window allows it; compressed rows must decide nearly
-    // every row-shard of the members as they were scored.
-    if (rp_may_use_row(c)) {
-        if (!c->rows_made) { RP_TRY(rp_launch_make_rows(c)); c->rows_made = 1; }
-        if (!c->rows_current) { RP_TRY(rp_launch_member_rows(c, c->row_members)); c->rows_current = 1; }
-        if (rp_row_compressed(c) && c->row_undecided < 0) {
-            int *u = (int *)(c->h_pin + 60);
-            RP_CUDA(cudaMemcpyAsync(u, c->d_undecided, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-            RP_CUDA(cudaStreamSynchronize(c->stream));
-            c->row_undecided = *u;
+    bool row = false;
+    c->n_queued = 0;
+    for (bool again = true; again && st == RP_OK;) {
+        again = false;
+        // Which kernel: the one-layer-per-lane kernel where the window allows it; compressed rows must decide nearly
+        // every row-shard of the members as they were scored.
+        if (rp_may_use_row(c)) {
+            if (!c->rows_made) { RP_TRY(rp_launch_make_rows(c)); c->rows_made = 1; }
+            if (!c->rows_current) { RP_TRY(rp_launch_member_rows(c, c->row_members)); c->rows_current = 1; }
+            if (rp_row_compressed(c) && c->row_undecided < 0) {
+                int *u = (int *)(c->h_pin + 60);
+                RP_CUDA(cudaMemcpyAsync(u, c->d_undecided, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+                RP_CUDA(cudaStreamSynchronize(c->stream));
+                c->row_undecided = *u;
+            }
         }
+        row = rp_uses_row(c);
+        // accepted-move log (not kept by the launch that runs all levels with one layer per lane)
+        if (c->log_cap < p->steps_per_level && !(row && c->row_mode == 1)) {
+            dev_free(c, c->d_log); c->d_log = nullptr; c->log_cap = 0;
+            RP_TRY(dev_alloc(c, &c->d_log, P * (size_t)p->steps_per_level));
+            c->log_cap = p->steps_per_level;
+        }
+        if (!row) st = need_rank_loads(c, 2 * P, true);
+        if (st == RP_OK && !row && c->full_stale) st = rebuild_rank_loads(c);
+        if (st == RP_OK && (rp_uses_wpc(c->dm) || (row && c->row_mode == 1)) && c->knob_level_launches != 1) st = rp_upload_levels(c, NL);
+        if (stats) cudaEventRecord(ev[0], c->stream);
+        if (st == RP_OK) st = rp_launch_anneal_all(c, NL, p, rho_q32, guide_q32, &all_in_one);
+        // Not all chains of that kernel can be resident at once (fewer free SMs than the device reports): the other kernels, which
+        // launch once per level, until the population is built anew.
+        if (st == RP_OK && row && c->row_mode == 1 && !all_in_one) { c->row_mode = 0; again = true; }
     }
-    const bool row = rp_uses_row(c);
-    if (!row) st = need_rank_loads(c, 2 * P, true);
-    if (st == RP_OK && !row && c->full_stale) st = rebuild_rank_loads(c);
     // What the context says about the population changes with the levels that have run, and with nothing that was refused
     // before them: a call that fails here can be followed by one that does not.
     auto levels_ran = [&]() {
@@ -1018,9 +1032,6 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
         c->row_members = c->Ppop;              // after a level every member has a state of its own
         c->full_stale = row && rp_row_separate(c);
     };
-    if (st == RP_OK && (rp_uses_wpc(c->dm) || (row && c->row_mode == 1)) && c->knob_level_launches != 1) st = rp_upload_levels(c, NL);
-    if (stats) cudaEventRecord(ev[0], c->stream);
-    if (st == RP_OK) st = rp_launch_anneal_all(c, NL, p, rho_q32, guide_q32, &all_in_one);
     if (all_in_one) { c->cur = (c->cur + NL) & 1; levels_ran(); }       // the kernel has left both ancestor tables and both cell tables current
     for (int n = 0; n < NL && st == RP_OK && !all_in_one; ++n) {
         st = rp_launch_anneal_level(c, n, NL, p, rho_q32, guide_q32);
@@ -1060,8 +1071,7 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     if (stats) {
         stats->proposed = cn[0]; stats->feasible = cn[1]; stats->accepted = cn[2]; stats->improved = cn[3];
         stats->move_bytes = cn[4]; stats->gather_bytes = cn[5]; stats->staging_bytes = cn[6];
-        stats->kernel_launches = all_in_one ? 1 : row && rp_row_turns(c) ? 2 * (int64_t)NL + 2
-                               : (int64_t)NL * ((rp_uses_slices(c->dm) ? 3 : 1) + (row || rp_uses_warp_chains(c) ? 1 : 0));
+        stats->kernel_launches = c->n_queued;
         stats->ms_chains = ms_chains;
     }
     c->best_verdict = best_verdict(c, sw);
@@ -1178,6 +1188,9 @@ extern "C" int rp_debug_set_knob(rp_ctx *c, int knob, int64_t value)
         case RP_KNOB_CHAIN_KERNEL:
             if (value > 2) return RP_ERR_ARG;
             c->knob_chain_kernel = (int)value; return RP_OK;
+        case RP_KNOB_RESIDENT_SMS:
+            if (value > (1 << 16)) return RP_ERR_ARG;
+            c->knob_sms = (int)value; return RP_OK;
         default: return RP_ERR_ARG;
     }
 }

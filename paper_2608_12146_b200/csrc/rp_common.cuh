@@ -146,6 +146,8 @@ struct rp_ctx {
     int *d_wfree;              // [2*P_pop*RG] slices nobody holds, handed out in this order during the level
     int *d_wfree_head;         // [2] next free-list entry to hand out, entries in the list
     // One-layer-per-lane chain kernel (rp_anneal_row.cu)
+    int sms;                   // SMs that may hold the CTAs of a launch which wait for one another
+    int row_cw;                // chains per CTA of the launch that runs all levels
     int row_mode;              // 0 = not for this window, 1 = one launch for all levels (rank loads on chip), 2 = one launch per level
     int rows_current;          // the row-shard sums (and rows kept apart) describe the population
     int full_stale;            // that kernel ran on rows kept apart: d_W no longer describes the population
@@ -198,6 +200,8 @@ struct rp_ctx {
     int knob_chain_kernel;     // 1 = 128 threads per chain, 2 = one warp per chain, wherever the window allows both
     int knob_slices;           // inspection hook: 0 = automatic, 1 = slices wherever L*P > 512, 2 = never
     int knob_le_ws_cap, knob_wait_polls, knob_stall;   // inspection hooks (rp_debug_set_knob); 0 = off
+    int knob_sms;              // inspection hook: at most this many SMs hold CTAs that wait for one another
+    int n_queued;              // kernels rp_anneal has launched for its levels
     cudaEvent_t ev_stage[RP_STAGE_EVENTS];             // stage timing (rp_debug_set_stage_timing); null when off
     unsigned ev_recorded;                              // bit x: ev_stage[x] has been recorded
     i64 *d_tr_term, *d_tr_best, *d_tr_inc;
@@ -227,6 +231,8 @@ struct rp_ctx {
 };
 
 #define RP_MAIL_BYTES (256 * 1024)
+// SMs a launch whose CTAs wait for one another can count on: what the device reports; less may be free (then the launch is refused).
+static inline int rp_sms(const rp_ctx *c) { return c->knob_sms > 0 && c->knob_sms < c->sms ? c->knob_sms : c->sms; }
 static inline int *rp_pin_bad(rp_ctx *c) { return (int *)(c->h_pin + 30); }
 static inline char *rp_mail(rp_ctx *c) { return (char *)(c->h_pin + 64); }
 static inline size_t rp_mail_place(const RpDims &dm) { return ((size_t)4 * dm.L * dm.E + 7) / 8 * 8 + (size_t)8 * dm.L * dm.P; }
@@ -296,7 +302,7 @@ bool rp_uses_warp_chains(const rp_ctx *c);
 bool rp_may_use_row(const rp_ctx *c);
 bool rp_uses_row(const rp_ctx *c);
 bool rp_row_compressed(const rp_ctx *c);
-bool rp_row_fits_chip(const rp_ctx *c, const RpBlob &bl, const RpStatic &sl);
+bool rp_row_fits_chip(rp_ctx *c, const RpBlob &bl, const RpStatic &sl);
 bool rp_row_fits_level(const rp_ctx *c, const RpBlob &bl, const RpStatic &sl);
 int rp_row_kind(const RpDims &dm);
 bool rp_row_separate(const rp_ctx *c);

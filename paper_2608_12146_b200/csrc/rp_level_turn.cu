@@ -194,7 +194,7 @@ int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A0)
     T.ns = ns;
     A.sync = c->d_sync;
     // Workers: as many as have something to do (a meeting costs the more the more there are); every one resident.
-    const int workers = std::max(4, std::min(147, std::max((P + 15) / 16, (ns + 4095) / 4096)));
+    const int workers = std::max(4, std::min(rp_sms(c) - 1, std::max((P + 15) / 16, (ns + 4095) / 4096)));
     T.base = A.level * 2 * workers;                  // (the count is zero when the call starts)
     int lu = 0;
     while ((TURN_THREADS << lu) < P) ++lu;
@@ -210,13 +210,13 @@ int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A0)
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_level_turn, A, T);
+    const cudaError_t e = workers + 1 > rp_sms(c) ? cudaErrorCooperativeLaunchTooLarge : cudaLaunchKernelEx(&cfg, k_level_turn, A, T);
     if (e == cudaErrorCooperativeLaunchTooLarge) {        // a part of a GPU: the launches one by one, at every level
         cudaGetLastError();
         return rp_launch_level_end(c, A0);
     }
     RP_CUDA(e);
-    ++g_rp_launches;
+    ++g_rp_launches; ++c->n_queued;
     c->slices_listed = 1;
     return RP_OK;
 }

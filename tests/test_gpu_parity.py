@@ -1398,3 +1398,41 @@ def test_a_call_that_fails_for_memory_leaves_the_population_as_it_is():
         rp.rp_release_cached_memory()
     for x, y in zip(*runs):
         assert (x == y).all()
+
+
+@pytest.mark.parametrize("spec,when", [(ROW_CASES[0], "before"), (ROW_CASES[3], "before"), (ROW_CASES[0], "after"), (ROW_CASES[3], "after"),
+                                       (ROW_CASES[4], "after"), (ROW_CASES[5], "resumed"), (ROW_CASES[4], "resumed"),
+                                       (ROW_CASES[6], "after"), (ROW_CASES[7], "resumed")])
+def test_launches_that_need_more_sms_than_are_free(spec, when):
+    """Launches whose CTAs wait for one another where only three SMs can hold them: known when the population is built
+    (more chains per CTA, or another form), found out at the launch, and found out by a later call."""
+    name, N, L, E, k, C, D, P, edp, min_rows, pop = spec
+    w = make_window(custom_spec(name, N, L, E, k, C, D, P, pop, 400, data_seed=len(name) * 29 + N))
+    s = w.spec
+    ref = oracle_front(w, edp, min_rows)
+    ctx = load(w, pop=pop, edp=edp, min_rows=min_rows)
+    if when == "before":
+        rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 3)
+    check_front(w, ctx, ref)
+    if when == "after":
+        rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 3)
+    want, stats = check_anneal(w, ctx, ref, edp, pop, 4, 40, t_ratio=0.5, check_members=2)
+    assert stats.accepted > 0
+    if when == "before":
+        assert (stats.kernel_launches == 1) == (pop <= 24)
+    elif when == "after":
+        assert stats.kernel_launches >= 4
+    rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 3)
+    want = oracle.anneal(w.lengths, ref["q"], want["final_pop"], ref["R"], s.token_cap, D, n_levels=3, steps=33, t0=1e-4,
+                         t_ratio=0.5, p_reloc=0.5, p_guide=0.3, seed=s.anneal_seed, edp_of_dp=edp, alpha=s.alpha,
+                         beta=s.beta, n_threads=8)
+    stats = rp.rp_anneal(ctx, n_levels=3, steps_per_level=33, t0=1e-4, t_ratio=0.5, p_reloc=0.5, p_guide=0.3)
+    assert stats.kernel_launches >= 3 or pop <= 24
+    assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (3, pop, 3), np.int64) == want["term"]).all()
+    assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == want["final_pop"]).all()
+    G = 1 + (max(edp) if edp is not None else D - 1)
+    ev = oracle.eval_layouts(w.lengths, ref["q"], want["final_pop"][pop - 1], ref["R"], s.token_cap, D, edp, s.alpha, s.beta)
+    assert (rp.rp_debug_dump(ctx, "W", (ref["R"], G, L, P), np.int32, index=pop - 1) == ev["W"][0]).all()
+    layout, fx, _ = rp.rp_best(ctx)
+    assert (layout == want["best_layout"]).all() and (fx == want["best_score"]).all()
+    rp.rp_destroy(ctx)
