@@ -27,6 +27,7 @@ struct EvalArgs {
     const char *blobs;
     const int *src;
     const int *t, *q, *edp, *dp_list, *dp_off;
+    int first;                                    // layouts of the call before this launch's
     int *W_out;                                   // [n][RG][LP], nullable
     char *blob_out;                               // [n] chain-state blobs (see RpBlob), nullable
     i64 *score_out, *score_out2;                  // [n][3], nullable
@@ -141,8 +142,8 @@ __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const Ev
         ((i64 *)(b + A.bl.off_Esum))[rg] = f.Esum[rg];
         ((i64 *)(b + A.bl.off_Afx))[rg] = f.Afx[rg];
         ((i64 *)(b + A.bl.off_Jfx))[rg] = f.Afx[rg] + dm.EC * f.Esum[rg];
-        if (A.bl.off_wtab >= 0)        // W_out holds layout `lay` as RG consecutive slices of the pool
-            ((int *)(b + A.bl.off_wtab))[rg] = lay * dm.RG + rg;
+        if (A.bl.off_wtab >= 0)        // the pool holds the call's layouts as RG consecutive slices each
+            ((int *)(b + A.bl.off_wtab))[rg] = (A.first + lay) * dm.RG + rg;
     }
     for (int g = tid; g < dm.G; g += EVAL_THREADS) ((i64 *)(b + A.bl.off_U))[g] = f.U[g];
     for (int i = tid; i < dm.N; i += EVAL_THREADS) ((unsigned short *)(b + A.bl.off_cell))[i] = f.cell_of[i];
@@ -440,6 +441,7 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
         for (int first = 0; first < n; first += 16384) {                 // (bounds the task numbers of a launch)
             EvalArgs B = A;
             const int m = std::min(16384, n - first);
+            B.first = first;
             if (B.lay32) B.lay32 += (size_t)first * dm.N; else B.src += first;
             if (B.W_out) B.W_out += (size_t)first * dm.RG * dm.LP;
             if (B.blob_out) B.blob_out += (size_t)first * c->bl.bytes;

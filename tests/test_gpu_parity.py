@@ -1436,3 +1436,23 @@ def test_launches_that_need_more_sms_than_are_free(spec, when):
     layout, fx, _ = rp.rp_best(ctx)
     assert (layout == want["best_layout"]).all() and (fx == want["best_score"]).all()
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("P,kernel", [(3, 0), (3, 1), (16, 2)])
+def test_more_members_than_one_scoring_launch_takes(P, kernel):
+    """17000 members with seeds of their own, more than a launch of the scoring kernels takes: every member's rank loads
+    are its own, and annealing goes on from them."""
+    pop, N, L, D, min_rows = 17000, 24, 40, 2, 3
+    w = make_window(custom_spec("many_members", N, L, P, 1, 2048, D, P, pop, 0, data_seed=P))
+    s = w.spec
+    ref = oracle_front(w, None, min_rows)
+    ctx = load(w, min_rows=min_rows)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", kernel)
+    check_front(w, ctx, ref)
+    lays, ok = oracle.seed_trials(w.lengths, ref["seed"], ref["R"], s.token_cap, D, pop, 5, s.anneal_seed)
+    assert rp.rp_seed_population(ctx, 5) == int(ok.sum())
+    for j in (0, 16383, 16384, pop - 1):
+        ev = oracle.eval_layouts(w.lengths, ref["q"], lays[j], ref["R"], s.token_cap, D, None, s.alpha, s.beta)
+        assert (rp.rp_debug_dump(ctx, "W", (ref["R"], D, L, P), np.int32, index=j) == ev["W"][0]).all()
+    check_anneal(w, ctx, ref, None, pop, 2, 12, t_ratio=0.6, init=lays)
+    rp.rp_destroy(ctx)
