@@ -195,7 +195,7 @@ int rp_init_population(rp_ctx *ctx, int32_t n_candidates, int32_t choice_width, 
  * stage-aware-attention, row-expert-load, row-expert-cost, lexicographic-score).
  *   layouts [n][N] int32 cell ids, or NULL to score the current population (n = pop_size).
  *   score_fx [n][3] int64 out, nullable; score_f64 [n][3] double out, nullable.
- * Layouts with a cell id outside [0, R*D) give RP_ERR_ARG. */
+ * Layouts with a cell id outside [0, R*D) give RP_ERR_ARG, and no score is written. */
 int rp_eval_population(rp_ctx *ctx, const int32_t *layouts, int32_t n, int64_t *score_fx,
                        double *score_f64);
 

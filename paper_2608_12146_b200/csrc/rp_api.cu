@@ -434,7 +434,7 @@ static int ensure_eval_scratch(rp_ctx *c, size_t n, bool want_W)
         for (int pass = 0; pass < 2; ++pass) {
             slab.off = 0;
             slab.take(&c->d_eval_Esum, n * dm.RG);            // (these two start at zero)
-            slab.take(&c->d_eval_tickets, n);
+            slab.take(&c->d_eval_tickets, n + 1);             // (and a counter of finished layouts)
             if (pass == 0) n_zero = slab.off;
             slab.take(&c->d_eval_score, n * 3);
             slab.take(&c->d_eval_f64, n * 3);
@@ -609,25 +609,29 @@ extern "C" int rp_eval_population(rp_ctx *c, const int32_t *layouts, int32_t n, 
         if (e != cudaSuccess) { dev_free(c, tmp); return rp_fail(e); }
         dl = tmp;
     }
-    // Results straight to where they are wanted: device outputs, or the second half of the pinned mail area.
+    // Results straight to where they are wanted: device outputs, or the second half of the pinned mail area.  None is written
+    // when a layout is refused.
     const size_t nf = sizeof(i64) * 3 * (size_t)n;
     const bool mail = 2 * nf <= RP_MAIL_BYTES / 2;
     char *half = rp_mail(c) + RP_MAIL_BYTES / 2;
     const bool fx_dev = score_fx && rp_is_device_ptr(score_fx), f64_dev = score_f64 && rp_is_device_ptr(score_f64);
-    i64 *fx = fx_dev ? (i64 *)score_fx : mail ? (i64 *)half : c->d_eval_score;
-    double *fd = f64_dev ? score_f64 : mail ? (double *)(half + nf) : c->d_eval_f64;
+    i64 *fx = mail && !fx_dev ? (i64 *)half : c->d_eval_score;
+    double *fd = mail && !f64_dev ? (double *)(half + nf) : c->d_eval_f64;
     int *bad = rp_pin_bad(c);
     *bad = 0;
     if (mail) c->best_ready = 0;               // (the incumbent's layout was there)
-    int st = rp_launch_eval(c, dl, layouts ? nullptr : c->d_anc, n, keepW ? c->d_eval_W : nullptr, nullptr, fx, fd);
-    if (st == RP_OK && score_fx && !fx_dev && !mail) st = copy_out(c, score_fx, fx, nf);
-    if (st == RP_OK && score_f64 && !f64_dev && !mail) st = copy_out(c, score_f64, fd, nf);
+    const int st = rp_launch_eval(c, dl, layouts ? nullptr : c->d_anc, n, keepW ? c->d_eval_W : nullptr, nullptr, fx, fd,
+                                  fx_dev ? (i64 *)score_fx : nullptr, f64_dev ? score_f64 : nullptr);
     dev_free(c, tmp);
     RP_TRY(st);
     RP_CUDA(cudaStreamSynchronize(c->stream));
-    if (*bad) return RP_ERR_ARG;
-    if (score_fx && !fx_dev && mail) memcpy(score_fx, fx, nf);
-    if (score_f64 && !f64_dev && mail) memcpy(score_f64, fd, nf);
+    if (*bad) {
+        RP_CUDA(cudaMemsetAsync(c->d_status + RP_SW_BAD_LAYOUT, 0, sizeof(int), c->stream));
+        return RP_ERR_ARG;
+    }
+    if (score_fx && !fx_dev) { if (mail) memcpy(score_fx, fx, nf); else RP_TRY(copy_out(c, score_fx, fx, nf)); }
+    if (score_f64 && !f64_dev) { if (mail) memcpy(score_f64, fd, nf); else RP_TRY(copy_out(c, score_f64, fd, nf)); }
+    if (!mail && ((score_fx && !fx_dev) || (score_f64 && !f64_dev))) RP_CUDA(cudaStreamSynchronize(c->stream));
     return RP_OK;
 }
 

@@ -250,7 +250,8 @@ int rp_launch_check_reduce(rp_ctx *c);
 int rp_launch_lpt(rp_ctx *c);
 int rp_launch_project(rp_ctx *c);
 int rp_launch_pack(rp_ctx *c, int Rlb_hint);
-int rp_launch_eval(rp_ctx *c, const int *lay, const int *src, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out);
+int rp_launch_eval(rp_ctx *c, const int *lay, const int *src, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out,
+                   i64 *score_final = nullptr, double *f64_final = nullptr);
 int rp_launch_eval_seed(rp_ctx *c);
 int rp_launch_eval_incumbent(rp_ctx *c);
 size_t rp_eval_list_len(const RpDims &dm, int n);

@@ -33,6 +33,13 @@ struct EvalArgs {
     i64 *score_out, *score_out2;                  // [n][3], nullable
     double *f64_out;                              // [n][3], nullable
     int *bad;                                     // raised when a layout names a cell outside [0, K) (host memory; such a sample counts as cell 0)
+    // Scores for a caller's device memory, which stays as it is if any layout of the call is bad: `bad_dev` is raised with `bad`
+    // and zero before.  Many layouts: all are looked at before the first is scored.  Few: the CTA that finishes the last layout
+    // (counter behind the tickets) copies them from score_out / f64_out.
+    int *bad_dev;
+    i64 *score_final;
+    double *f64_final;
+    int n;
     i64 *Esum;                                    // [n][RG] row-shard sums handed to the finishing CTA; zero between launches
     int *tickets;                                 // [n] arrival counters; zero between launches
     unsigned short *list;                         // [n][N] samples grouped by row-shard (k_eval_group)
@@ -60,6 +67,7 @@ __device__ __forceinline__ int eval_cell(const EvalArgs &A, const EvalCells &e, 
     const int c = __ldg(e.a + i);
     if ((unsigned)c < (unsigned)A.dm.K) return c;
     *A.bad = 1;
+    if (A.bad_dev) *A.bad_dev = 1;
     return 0;
 }
 
@@ -83,6 +91,7 @@ __device__ __forceinline__ EvalFinish eval_finish_views(const RpDims &dm, unsign
 }
 
 // Scores layout `lay` once its row-shard sums are complete.  All threads of one CTA call; cell_of is in place.
+template <bool FEW>
 __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const EvalFinish &f, int tid)
 {
     const RpDims &dm = A.dm;
@@ -114,6 +123,7 @@ __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const Ev
         if (A.layout_host) for (int i = tid; i < dm.N; i += EVAL_THREADS) A.layout_host[i] = __ldg(A.lay32 + i);
     }
     if (tid < 32) {
+        const bool refused = !FEW && A.bad_dev && __ldcg(A.bad_dev);
         i64 s0 = 0, s1 = 0, s2 = 0;
         for (int g = lane; g < dm.G; g += 32) { const i64 u = f.U[g]; s1 += u; s0 = u > s0 ? u : s0; }
         for (int rg = lane; rg < dm.RG; rg += 32) { const i64 J = f.Afx[rg] + dm.EC * f.Esum[rg]; s2 = J > s2 ? J : s2; }
@@ -125,6 +135,7 @@ __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const Ev
         if (lane == 0) {
             const i64 sc[3] = { s0, s1, s2 };
             for (int x = 0; x < 3; ++x) {
+                if (refused) continue;
                 if (A.score_out) A.score_out[(size_t)lay * 3 + x] = sc[x];
                 if (A.score_out2) A.score_out2[(size_t)lay * 3 + x] = sc[x];
                 if (A.f64_out) A.f64_out[(size_t)lay * 3 + x] = (double)sc[x] / (double)dm.SC;
@@ -323,7 +334,7 @@ k_eval_score(const EvalArgs A)
     extern __shared__ __align__(16) unsigned char smraw[];
     const EvalFinish f = eval_finish_views(A.dm, smraw);
     eval_load_cells(A, blockIdx.x, f.cell_of, threadIdx.x, EVAL_THREADS);
-    eval_finish(A, blockIdx.x, f, threadIdx.x);
+    eval_finish<false>(A, blockIdx.x, f, threadIdx.x);
 }
 
 // grid = (MS, row-shards, layouts), clusters of MS CTAs along x: CTA x of a row-shard takes the samples of
@@ -389,7 +400,23 @@ k_eval_few(const EvalArgs A)
     __threadfence();
     const EvalFinish f = eval_finish_views(dm, smraw);
     eval_load_cells(A, lay, f.cell_of, tid, EVAL_THREADS);
-    eval_finish(A, lay, f, tid);
+    eval_finish<true>(A, lay, f, tid);
+    if (!A.score_final && !A.f64_final) return;
+    if (tid < 32) __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        last_s = (atomicAdd(&A.tickets[A.n], 1) == A.n - 1);
+        if (last_s) A.tickets[A.n] = 0;
+    }
+    __syncthreads();
+    if (!last_s) return;
+    __threadfence();
+    if (__ldcg(A.bad_dev)) return;
+#pragma unroll 4
+    for (int x = tid; x < 3 * A.n; x += EVAL_THREADS) {
+        if (A.score_final) A.score_final[x] = __ldcg(A.score_out + x);
+        if (A.f64_final) A.f64_final[x] = __ldcg(A.f64_out + x);
+    }
 }
 
 static size_t eval_smem_bytes(const RpDims &dm)
@@ -414,6 +441,7 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
     const RpDims &dm = c->dm;
     if (eval_smem_bytes(dm) > EVAL_SMEM_MAX) return RP_ERR_RANGE;
     A.dm = dm; A.bl = c->bl; A.t = c->d_t; A.q = c->d_q; A.edp = c->d_edp; A.dp_list = c->d_dp_list; A.dp_off = c->d_dp_off;
+    A.n = n;
     if (eval_is_few(dm, n)) {
         int MS = 1;
         while (MS < 8 && (long long)n * dm.RG * MS < 148 * 4 && dm.N >= 64 * MS) MS *= 2;
@@ -438,9 +466,10 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
         // What a warp adds up for a row-shard: the busiest loads of its layers, each at most k times the tokens of the window
         // (a layout handed in may put them all into one cell).
         const bool sum32 = eval_vec(dm) && (double)std::min(dm.L, ns * used / cpl) * dm.k * (double)c->tokens < 4294967296.0;
-        for (int first = 0; first < n; first += 16384) {                 // (bounds the task numbers of a launch)
+        if (A.score_final) A.score_out = A.score_final;
+        if (A.f64_final) A.f64_out = A.f64_final;
+        auto part = [&](int first) {                       // (16384 layouts: bounds the task numbers of a launch)
             EvalArgs B = A;
-            const int m = std::min(16384, n - first);
             B.first = first;
             if (B.lay32) B.lay32 += (size_t)first * dm.N; else B.src += first;
             if (B.W_out) B.W_out += (size_t)first * dm.RG * dm.LP;
@@ -448,17 +477,26 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
             if (B.score_out) B.score_out += 3 * (size_t)first;
             if (B.f64_out) B.f64_out += 3 * (size_t)first;
             B.Esum += (size_t)first * dm.RG; B.tickets += first; B.list += (size_t)first * dm.N; B.off += (size_t)first * (dm.RG + 1);
+            return B;
+        };
+        for (int first = 0; first < n; first += 16384) {
+            k_eval_group<<<std::min(16384, n - first), GROUP_THREADS, gm, c->stream>>>(part(first));
+            ++g_rp_launches;
+        }
+        for (int first = 0; first < n; first += 16384) {
+            const EvalArgs B = part(first);
+            const int m = std::min(16384, n - first);
             // several tasks for each warp the SMs hold, of at most 31 row-shards
             const int rpt = (int)std::max<long long>(1, std::min<long long>(31, (long long)m * dm.RG * sgroups / (148 * warps * 6)));
             const long long want = ((long long)m * ((dm.RG + rpt - 1) / rpt) * sgroups + 7) / 8;
             const int grid = (int)std::min<long long>(want, 148 * warps / 8);
-            k_eval_group<<<m, GROUP_THREADS, gm, c->stream>>>(B);
             if (ns == 1) k_eval_sum<1, 8><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt, sum32);
             else if (ns == 2) k_eval_sum<2, 4><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt, sum32);
             else k_eval_sum<3, 4><<<grid, EVAL_THREADS, 0, c->stream>>>(B, m, sgroups, rpt, sum32);
             k_eval_score<<<m, EVAL_THREADS, fm, c->stream>>>(B);
             g_rp_launches += 2;
         }
+        --g_rp_launches;                                   // (one is counted below)
     }
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
@@ -466,12 +504,15 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
 }
 
 // n layouts lay [n][N] (null: the assignments of the current buffer's blobs that src names) with the context's scratch.
-int rp_launch_eval(rp_ctx *c, const int *lay, const int *src, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out)
+// score_final, f64_final: see EvalArgs; score_out / f64_out are then scratch.
+int rp_launch_eval(rp_ctx *c, const int *lay, const int *src, int n, int *W_out, char *blob_out, i64 *score_out, double *f64_out,
+                   i64 *score_final, double *f64_final)
 {
     EvalArgs A = {};
     A.lay32 = lay; A.blobs = c->buf[c->cur].blob; A.src = src;
     A.W_out = W_out; A.blob_out = blob_out; A.score_out = score_out; A.f64_out = f64_out;
     A.bad = rp_pin_bad(c);
+    if (score_final || f64_final) { A.score_final = score_final; A.f64_final = f64_final; A.bad_dev = c->d_status + RP_SW_BAD_LAYOUT; }
     A.Esum = c->d_eval_Esum; A.tickets = c->d_eval_tickets; A.list = c->d_eval_list; A.off = c->d_eval_off;
     return eval_launch(c, A, n);
 }

@@ -1456,3 +1456,34 @@ def test_more_members_than_one_scoring_launch_takes(P, kernel):
         assert (rp.rp_debug_dump(ctx, "W", (ref["R"], D, L, P), np.int32, index=j) == ev["W"][0]).all()
     check_anneal(w, ctx, ref, None, pop, 2, 12, t_ratio=0.6, init=lays)
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [1, 3, 150, 2500, 4000, 16400])
+def test_a_refused_layout_leaves_the_outputs_alone(n):
+    """One bad cell id among n layouts: RP_ERR_ARG, and neither device nor host outputs are written; good layouts are
+    scored by the next call (few and many layouts, more than the pinned block and more than one launch holds)."""
+    import torch
+    w = make_window(custom_spec("refused", 40, 3, 8, 2, 4096, 4, 4, 2, 0, data_seed=n))
+    s = w.spec
+    ref = oracle_front(w, None, 2)
+    ctx = load(w, min_rows=2)
+    check_front(w, ctx, ref)
+    rng = np.random.default_rng(n)
+    good = rng.integers(0, ref["R"] * 4, (n, 40)).astype(np.int32)
+    want = oracle.eval_layouts(w.lengths, ref["q"], good[-2:], ref["R"], s.token_cap, 4, None, s.alpha, s.beta)["score"]
+    for value in (-1, ref["R"] * 4):
+        lays = good.copy()
+        lays[rng.integers(0, n), rng.integers(0, 40)] = value
+        for dev in (True, False):
+            fx, f64 = torch.full((n, 3), -7, dtype=torch.int64), torch.full((n, 3), -7.0, dtype=torch.float64)
+            if dev:
+                fx, f64 = fx.cuda(), f64.cuda()
+            for out64 in (f64, None, np.full((n, 3), -7.0)):
+                with pytest.raises(rp.RpError) as e:
+                    rp._check(rp.lib().rp_eval_population(ctx.handle, rp._ptr(lays), n, rp._ptr(fx), rp._ptr(out64)), "eval")
+                assert e.value.status == -1
+                assert bool((fx == -7).all()) and (out64 is None or bool((out64 == -7).all()))
+            rp.rp_eval_population(ctx, good, fx, f64)
+            assert (fx[-2:].cpu().numpy() == want).all()
+            np.testing.assert_allclose(f64[-2:].cpu().numpy(), want / (256.0 * s.token_cap ** 2), rtol=F64_RTOL)
+    rp.rp_destroy(ctx)
