@@ -148,6 +148,14 @@ bool rp_is_device_ptr(const void *p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Memory that kernels of this context can use where it is: another GPU's is only copied from and to.
+bool rp_is_local_ptr(const rp_ctx *c, const void *p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == c->device);
+}
+
 static int copy_out(rp_ctx *c, void *dst, const void *src, size_t bytes)
 {
     if (!dst || !bytes) return RP_OK;
@@ -603,23 +611,24 @@ extern "C" int rp_eval_population(rp_ctx *c, const int32_t *layouts, int32_t n, 
     RP_TRY(ensure_eval_scratch(c, (size_t)n, keepW));
     const int *dl = layouts;
     int *tmp = nullptr;
-    if (layouts && !rp_is_device_ptr(layouts)) {
+    if (layouts && !rp_is_local_ptr(c, layouts)) {
         RP_TRY(dev_alloc(c, &tmp, (size_t)n * dm.N));
-        cudaError_t e = cudaMemcpyAsync(tmp, layouts, sizeof(int) * (size_t)n * dm.N, cudaMemcpyHostToDevice, c->stream);
+        cudaError_t e = cudaMemcpyAsync(tmp, layouts, sizeof(int) * (size_t)n * dm.N, cudaMemcpyDefault, c->stream);
         if (e != cudaSuccess) { dev_free(c, tmp); return rp_fail(e); }
         dl = tmp;
     }
-    // Results straight to where they are wanted: device outputs, or the second half of the pinned mail area.  None is written
-    // when a layout is refused.
+    // Results straight to where they are wanted: this GPU's memory, or the second half of the pinned mail area for the host; copied
+    // there where they do not fit, and to other GPUs.  None is written when a layout is refused.
     const size_t nf = sizeof(i64) * 3 * (size_t)n;
     const bool mail = 2 * nf <= RP_MAIL_BYTES / 2;
     char *half = rp_mail(c) + RP_MAIL_BYTES / 2;
-    const bool fx_dev = score_fx && rp_is_device_ptr(score_fx), f64_dev = score_f64 && rp_is_device_ptr(score_f64);
-    i64 *fx = mail && !fx_dev ? (i64 *)half : c->d_eval_score;
-    double *fd = mail && !f64_dev ? (double *)(half + nf) : c->d_eval_f64;
+    const bool fx_dev = score_fx && rp_is_local_ptr(c, score_fx), f64_dev = score_f64 && rp_is_local_ptr(c, score_f64);
+    const bool fx_mail = mail && score_fx && !rp_is_device_ptr(score_fx), f64_mail = mail && score_f64 && !rp_is_device_ptr(score_f64);
+    i64 *fx = fx_mail ? (i64 *)half : c->d_eval_score;
+    double *fd = f64_mail ? (double *)(half + nf) : c->d_eval_f64;
     int *bad = rp_pin_bad(c);
     *bad = 0;
-    if (mail) c->best_ready = 0;               // (the incumbent's layout was there)
+    if (fx_mail || f64_mail) c->best_ready = 0;               // (the incumbent's layout was there)
     const int st = rp_launch_eval(c, dl, layouts ? nullptr : c->d_anc, n, keepW ? c->d_eval_W : nullptr, nullptr, fx, fd,
                                   fx_dev ? (i64 *)score_fx : nullptr, f64_dev ? score_f64 : nullptr);
     dev_free(c, tmp);
@@ -629,9 +638,12 @@ extern "C" int rp_eval_population(rp_ctx *c, const int32_t *layouts, int32_t n, 
         RP_CUDA(cudaMemsetAsync(c->d_status + RP_SW_BAD_LAYOUT, 0, sizeof(int), c->stream));
         return RP_ERR_ARG;
     }
-    if (score_fx && !fx_dev) { if (mail) memcpy(score_fx, fx, nf); else RP_TRY(copy_out(c, score_fx, fx, nf)); }
-    if (score_f64 && !f64_dev) { if (mail) memcpy(score_f64, fd, nf); else RP_TRY(copy_out(c, score_f64, fd, nf)); }
-    if (!mail && ((score_fx && !fx_dev) || (score_f64 && !f64_dev))) RP_CUDA(cudaStreamSynchronize(c->stream));
+    if (fx_mail) memcpy(score_fx, fx, nf);
+    if (f64_mail) memcpy(score_f64, fd, nf);
+    const bool fx_copy = score_fx && !fx_dev && !fx_mail, f64_copy = score_f64 && !f64_dev && !f64_mail;
+    if (fx_copy) RP_TRY(copy_out(c, score_fx, fx, nf));
+    if (f64_copy) RP_TRY(copy_out(c, score_f64, fd, nf));
+    if (fx_copy || f64_copy) RP_CUDA(cudaStreamSynchronize(c->stream));
     return RP_OK;
 }
 

@@ -728,7 +728,7 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
     if (dm.L > 1024) return RP_ERR_RANGE;
     cudaMemPool_t pool;
     RP_TRY(rp_get_pool(c->device, &pool));
-    // scratch: a copy of a host layout, W, one blob
+    // scratch: a copy of a layout that is not in this GPU's memory, W, one blob
     const size_t wn = (size_t)dm.RG * dm.LP;
     const size_t off_W = ((size_t)dm.N * 4 + 255) & ~(size_t)255, off_blob = off_W + ((wn * 4 + 255) & ~(size_t)255);
     const size_t off_res = off_blob + (((size_t)c->bl.bytes + 255) & ~(size_t)255);
@@ -739,7 +739,7 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
     cudaError_t e = cudaSuccess;
     do {
         const int *dl = layout ? layout : c->d_inc_layout;
-        if (layout && !rp_is_device_ptr(layout)) {
+        if (layout && !rp_is_local_ptr(c, layout)) {
             e = cudaMemcpyAsync(buf, layout, sizeof(int) * dm.N, cudaMemcpyDefault, c->stream);
             if (e != cudaSuccess) break;
             dl = (const int *)buf;
