@@ -310,7 +310,7 @@ k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt, bool sum32)
                 int4 v[U][NS];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {               // (past the end: sample 0, not counted)
-                    const int at = __shfl_sync(0xffffffffu, id, y + u) * rc;          // N*L*P/4 fits 31 bits
+                    const size_t at = (size_t)(u32)__shfl_sync(0xffffffffu, id, y + u) * (u32)rc;
 #pragma unroll
                     for (int z = 0; z < NS; ++z) v[u][z] = __ldg(col[z] + at);
                 }
