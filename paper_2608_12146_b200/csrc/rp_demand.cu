@@ -296,7 +296,9 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
     int *cnt = order + dm.E;                  // [P]
     const int l = blockIdx.x;
     const i64 *Le = Lagg + (size_t)l * dm.E;
-    for (int e = threadIdx.x; e < dm.E; e += blockDim.x) load[e] = Le[e];
+    // (queued behind the checks before their verdict: a window with negative counts is refused, but is placed until then, and
+    // the projection follows its slots; the searches below take loads for non-negative)
+    for (int e = threadIdx.x; e < dm.E; e += blockDim.x) load[e] = Le[e] > 0 ? Le[e] : 0;
     for (int p = threadIdx.x; p < dm.P; p += blockDim.x) { G[p] = 0; cnt[p] = 0; }
     __syncthreads();
     for (int e = threadIdx.x; e < dm.E; e += blockDim.x) {

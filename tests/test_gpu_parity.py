@@ -1487,3 +1487,24 @@ def test_a_refused_layout_leaves_the_outputs_alone(n):
             assert (fx[-2:].cpu().numpy() == want).all()
             np.testing.assert_allclose(f64[-2:].cpu().numpy(), want / (256.0 * s.token_cap ** 2), rtol=F64_RTOL)
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,L,E,P", [(1, 3, 8, 4), (7, 2, 8, 8), (5, 4, 64, 32), (300, 2, 128, 16), (9, 2, 128, 128), (4, 1, 512, 256), (6, 3, 1024, 8)])
+def test_windows_with_negative_counts_are_refused(N, L, E, P):
+    """Placement and projection are queued before the verdict on the counts: aggregate loads below zero must not upset them,
+    and a good window behind is planned as ever."""
+    t = np.full(N, 3, np.int32)
+    good = np.zeros((N, L, E), np.int32)
+    good[:, :, 0] = 6
+    kw = dict(top_k=2, token_cap=64, dp_width=1, ep_width=P, pop_size=2)
+    for value in (-1, -(1 << 31), -3):
+        for bad in (np.full((N, L, E), value, np.int32), np.where(np.arange(E) % 3 == 0, 1 << 20, value).astype(np.int32) + 0 * good):
+            with pytest.raises(rp.RpError) as e:
+                rp.rp_window_load(t, bad, **kw)
+            assert e.value.status == -3
+        ctx = rp.rp_window_load(t, good, **kw)
+        pi, load_ = rp.rp_place_experts(ctx)
+        want, G = oracle.lpt(oracle.aggregate(good), P)
+        assert (pi == want).all() and (load_ == G).all()
+        assert (rp.rp_debug_dump(ctx, "Q", (N, L, P), np.int32) == oracle.project(good, pi, P)).all()
+        rp.rp_destroy(ctx)
