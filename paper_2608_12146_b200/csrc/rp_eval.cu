@@ -641,7 +641,7 @@ k_diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, RpDim
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) { sums->s_ep = 0; sums->t_ep = 0; sums->n_ep = 0; sums->tickets = 0; }      // for the kernel behind this one
     double *G = cvs + 2 * dm.L + (size_t)warp * dm.P;
-    for (int x = warp; x < 2 * dm.L; x += DIAG_THREADS / 32) {
+    for (int x = warp; x < 2 * dm.L; x += (int)blockDim.x / 32) {
         const int l = x >> 1, which = x & 1;
         for (int p = lane; p < dm.P; p += 32) {
             i64 g = 0;
@@ -732,7 +732,9 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
     const size_t wn = (size_t)dm.RG * dm.LP;
     const size_t off_W = ((size_t)dm.N * 4 + 255) & ~(size_t)255, off_blob = off_W + ((wn * 4 + 255) & ~(size_t)255);
     const size_t off_res = off_blob + (((size_t)c->bl.bytes + 255) & ~(size_t)255);
-    const size_t cv_smem = sizeof(double) * (2 * (size_t)dm.L + (DIAG_THREADS / 32) * (size_t)dm.P);
+    // (a row of P rank loads per warp: beyond 900 ranks fewer warps than the kernel is made for)
+    const int cv_warps = (int)std::min<size_t>(DIAG_THREADS / 32, (EVAL_SMEM_MAX / sizeof(double) - 2 * (size_t)dm.L) / dm.P);
+    const size_t cv_smem = sizeof(double) * (2 * (size_t)dm.L + cv_warps * (size_t)dm.P);
     char *buf = nullptr;
     RP_CUDA(cudaMallocFromPoolAsync((void **)&buf, off_res + 256, pool, c->stream));
     int st = RP_OK;
@@ -757,7 +759,7 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
             e = cudaFuncSetAttribute(k_diag_cv, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX);
             if (e != cudaSuccess) break;
         }
-        k_diag_cv<<<1, DIAG_THREADS, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, dm, res, host);
+        k_diag_cv<<<1, 32 * cv_warps, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, dm, res, host);
         ++g_rp_launches;
         k_diag_peaks<<<148, 256, 0, c->stream>>>((const int *)(buf + off_W), buf + off_blob, c->bl, dm, res, host);
         ++g_rp_launches;

@@ -1508,3 +1508,20 @@ def test_windows_with_negative_counts_are_refused(N, L, E, P):
         assert (pi == want).all() and (load_ == G).all()
         assert (rp.rp_debug_dump(ctx, "Q", (N, L, P), np.int32) == oracle.project(good, pi, P)).all()
         rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("P,L", [(864, 5), (1000, 2), (1024, 16)])
+def test_diagnostics_of_many_ranks(P, L):
+    """Rows of rank loads that do not fit shared memory for 32 warps at once."""
+    w = make_window(custom_spec("many_ranks", 24, L, P, 2, 2048, 2, P, 3, 0, data_seed=P))
+    s = w.spec
+    ref = oracle_front(w, None, 2)
+    ctx = load(w, min_rows=2)
+    check_front(w, ctx, ref)
+    want = oracle.diagnostics(w.lengths, ref["q"], ref["Lagg"], ref["pi"], ref["seed"], ref["R"], s.token_cap, 2, None, s.alpha, s.beta)
+    got = rp.rp_diagnostics(ctx)
+    for key in ("s_ep", "t_ep", "n_ep"):
+        assert got[key] == want[key], key
+    for key in ("cv_identity", "cv_placed", "eta_ep", "attention", "joint"):
+        assert abs(got[key] - want[key]) <= F64_RTOL * abs(want[key]), key
+    rp.rp_destroy(ctx)
