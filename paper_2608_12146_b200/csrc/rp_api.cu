@@ -148,12 +148,13 @@ bool rp_is_device_ptr(const void *p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// Memory that kernels of this context can use where it is: another GPU's is only copied from and to.
-bool rp_is_local_ptr(const rp_ctx *c, const void *p)
+// 0 = host memory, 1 = another GPU's (only copied from and to), 2 = memory that kernels of this context can use where it is.
+int rp_ptr_kind(const rp_ctx *c, const void *p)
 {
     cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
-    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == c->device);
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (at.type == cudaMemoryTypeDevice) return at.device == c->device ? 2 : 1;
+    return at.type == cudaMemoryTypeManaged ? 2 : 0;
 }
 
 static int copy_out(rp_ctx *c, void *dst, const void *src, size_t bytes)
@@ -611,7 +612,7 @@ extern "C" int rp_eval_population(rp_ctx *c, const int32_t *layouts, int32_t n, 
     RP_TRY(ensure_eval_scratch(c, (size_t)n, keepW));
     const int *dl = layouts;
     int *tmp = nullptr;
-    if (layouts && !rp_is_local_ptr(c, layouts)) {
+    if (layouts && rp_ptr_kind(c, layouts) != 2) {
         RP_TRY(dev_alloc(c, &tmp, (size_t)n * dm.N));
         cudaError_t e = cudaMemcpyAsync(tmp, layouts, sizeof(int) * (size_t)n * dm.N, cudaMemcpyDefault, c->stream);
         if (e != cudaSuccess) { dev_free(c, tmp); return rp_fail(e); }
@@ -622,8 +623,8 @@ extern "C" int rp_eval_population(rp_ctx *c, const int32_t *layouts, int32_t n, 
     const size_t nf = sizeof(i64) * 3 * (size_t)n;
     const bool mail = 2 * nf <= RP_MAIL_BYTES / 2;
     char *half = rp_mail(c) + RP_MAIL_BYTES / 2;
-    const bool fx_dev = score_fx && rp_is_local_ptr(c, score_fx), f64_dev = score_f64 && rp_is_local_ptr(c, score_f64);
-    const bool fx_mail = mail && score_fx && !rp_is_device_ptr(score_fx), f64_mail = mail && score_f64 && !rp_is_device_ptr(score_f64);
+    const int fx_kind = score_fx ? rp_ptr_kind(c, score_fx) : -1, f64_kind = score_f64 ? rp_ptr_kind(c, score_f64) : -1;
+    const bool fx_dev = fx_kind == 2, f64_dev = f64_kind == 2, fx_mail = mail && fx_kind == 0, f64_mail = mail && f64_kind == 0;
     i64 *fx = fx_mail ? (i64 *)half : c->d_eval_score;
     double *fd = f64_mail ? (double *)(half + nf) : c->d_eval_f64;
     int *bad = rp_pin_bad(c);

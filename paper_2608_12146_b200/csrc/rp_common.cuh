@@ -258,7 +258,7 @@ size_t rp_eval_list_len(const RpDims &dm, int n);
 size_t rp_eval_off_len(const RpDims &dm, int n);
 int rp_launch_setup_population(rp_ctx *c);
 bool rp_is_device_ptr(const void *p);
-bool rp_is_local_ptr(const rp_ctx *c, const void *p);
+int rp_ptr_kind(const rp_ctx *c, const void *p);
 int rp_launch_seed_trials(rp_ctx *c, int width, int *layouts, int *ok);
 int rp_launch_edp_pair(rp_ctx *c, const int *lay_in, int *lay_out, int *prof, int first, int count, int width);
 int rp_launch_pack_on(rp_ctx *c, cudaStream_t stream);

@@ -3,7 +3,7 @@
 //
 // The work is the sum of the q rows of every row-shard's samples: N*L*P*4 bytes per layout, served by L2
 // (q is shared by all layouts).  Two forms:
-//  * few layouts (k_eval_few: the seed, the incumbent, diagnostics, small batches), bound by latency: a cluster of
+//  * few layouts of rows in whole 16-byte chunks (k_eval_few: the seed, the incumbent, diagnostics, small batches), bound by latency: a cluster of
 //    CTAs per row-shard, each over its share of the samples, sixteen 16-byte loads in flight per lane; the CTAs'
 //    sums meet through distributed shared memory;
 //  * many layouts (k_eval_group, k_eval_sum, k_eval_score), bound by L2: the samples of a layout are grouped by row-shard once, then
@@ -339,6 +339,7 @@ k_eval_score(const EvalArgs A)
 
 // grid = (MS, row-shards, layouts), clusters of MS CTAs along x: CTA x of a row-shard takes the samples of
 // range x, then the layers of range x of the summed row.
+template <bool WIDE>            // more than 32 chunks in a layer
 __global__ void __launch_bounds__(EVAL_THREADS)
 k_eval_few(const EvalArgs A)
 {
@@ -369,9 +370,25 @@ k_eval_few(const EvalArgs A)
         if (c < rc) ((int4 *)part)[c] = a;
     }
     cl.sync();
-    const int l0 = dm.L * ms / MS, l1 = dm.L * (ms + 1) / MS, lps = 32 / cpl, used = lps * cpl;
+    const int l0 = dm.L * ms / MS, l1 = dm.L * (ms + 1) / MS, lps = WIDE ? 1 : 32 / cpl, used = WIDE ? 32 : lps * cpl;
     int4 *wout = A.W_out ? (int4 *)(A.W_out + ((size_t)lay * dm.RG + rg) * dm.LP) : nullptr;
     i64 es = 0;
+    if (WIDE) {                                           // a layer per warp
+        for (int l = l0 + warp; l < l1; l += nwarps) {
+            int m = 0;
+            for (int c = l * cpl + lane; c < (l + 1) * cpl; c += 32) {
+                int4 a = make_int4(0, 0, 0, 0);
+                for (int x = 0; x < MS; ++x) {
+                    const int4 v = ((const int4 *)cl.map_shared_rank(part, x))[c];
+                    a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+                }
+                if (wout) wout[c] = a;
+                m = max(m, max(max(a.x, a.y), max(a.z, a.w)));
+            }
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) es += m;
+        }
+    } else
     for (int c0 = l0 * cpl + warp * used; c0 < l1 * cpl; c0 += nwarps * used) {
         const int c = c0 + lane;
         const bool on = lane < used && c < l1 * cpl;
@@ -404,13 +421,15 @@ k_eval_few(const EvalArgs A)
     if (!A.score_final && !A.f64_final) return;
     if (tid < 32) __threadfence();
     __syncthreads();
-    if (tid == 0) {
-        last_s = (atomicAdd(&A.tickets[A.n], 1) == A.n - 1);
-        if (last_s) A.tickets[A.n] = 0;
+    if (A.n > 1) {
+        if (tid == 0) {
+            last_s = (atomicAdd(&A.tickets[A.n], 1) == A.n - 1);
+            if (last_s) A.tickets[A.n] = 0;
+        }
+        __syncthreads();
+        if (!last_s) return;
+        __threadfence();
     }
-    __syncthreads();
-    if (!last_s) return;
-    __threadfence();
     if (__ldcg(A.bad_dev)) return;
 #pragma unroll 4
     for (int x = tid; x < 3 * A.n; x += EVAL_THREADS) {
@@ -426,11 +445,19 @@ static size_t eval_smem_bytes(const RpDims &dm)
 
 #define EVAL_SMEM_MAX (220 * 1024)
 
-// Whether n layouts take the few-layouts form: a cluster per row-shard scans the assignment once per row-shard, the other
-// form groups it once per layout; the first up to about sixteen waves of its CTAs.
+// Whether n layouts take the few-layouts form.  It has a cluster per row-shard and layout, which scans the whole assignment: per CTA
+// about 6 ns and a nanosecond for 300 samples, with the rows served less evenly (0.3 ns for 1000 counts).  The other form groups
+// an assignment once, but in one CTA, and streams through a row-shard with one warp: 9 us more for its launches, and the longer
+// a row-shard, the more, up to 30 us.  In us, few and many: 512 samples in 32 row-shards, 16 layers of 8 ranks, n = 8 30 and 28,
+// 64 40 and 30, 512 157 and 45; 2048 in 240, 24 of 16, n = 3 33 and 35, 8 47 and 35, 64 193 and 58; 4000 in 6, 16 of 8, n = 64
+// 100 and 135, 512 258 and 166; 30000 in 160, n = 1 110 and 146, 8 504 and 150.  One layout: 8192 in 448 56 and 57, 4000 in 2000
+// 76 and 44.
 static bool eval_is_few(const RpDims &dm, int n)
 {
-    return eval_vec(dm) && (long long)n * dm.RG <= 16 * 148 * 8 && n < 65536 && dm.RG < 65536 && dm.LP <= 16384;
+    if ((dm.P & 3) || n >= 65536 || dm.RG >= 65536 || dm.LP > 16384) return false;
+    const double N = dm.N, RG = dm.RG;
+    if (n == 1) return RG * N <= 5e6;
+    return n * (RG * (6.0 + N / 300.0) + 3e-4 * N * dm.LP) <= 9e3 + std::min(150.0 * N / RG, 30e3);
 }
 size_t rp_eval_list_len(const RpDims &dm, int n) { return eval_is_few(dm, n) ? 0 : (size_t)n * dm.N; }
 size_t rp_eval_off_len(const RpDims &dm, int n) { return eval_is_few(dm, n) ? 0 : (size_t)n * (dm.RG + 1); }
@@ -447,7 +474,8 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
         while (MS < 8 && (long long)n * dm.RG * MS < 148 * 4 && dm.N >= 64 * MS) MS *= 2;
         const size_t sm = std::max(eval_finish_bytes(dm), sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2));
         if (sm > EVAL_SMEM_MAX) return RP_ERR_RANGE;
-        if (sm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_few, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
+        auto few = eval_vec(dm) ? k_eval_few<false> : k_eval_few<true>;
+        if (sm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(few, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(MS, dm.RG, n); cfg.blockDim = dim3(EVAL_THREADS);
         cfg.dynamicSmemBytes = sm; cfg.stream = c->stream;
@@ -455,7 +483,7 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = MS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
         cfg.attrs = at; cfg.numAttrs = 1;
-        RP_CUDA(cudaLaunchKernelEx(&cfg, k_eval_few, A));
+        RP_CUDA(cudaLaunchKernelEx(&cfg, few, A));
     } else {
         const size_t gm = sizeof(int) * (size_t)dm.RG + 2 * ((size_t)dm.K + dm.N), fm = eval_finish_bytes(dm);
         if (gm > EVAL_SMEM_MAX || dm.N > 65535) return RP_ERR_RANGE;
@@ -741,7 +769,7 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
     cudaError_t e = cudaSuccess;
     do {
         const int *dl = layout ? layout : c->d_inc_layout;
-        if (layout && !rp_is_local_ptr(c, layout)) {
+        if (layout && rp_ptr_kind(c, layout) != 2) {
             e = cudaMemcpyAsync(buf, layout, sizeof(int) * dm.N, cudaMemcpyDefault, c->stream);
             if (e != cudaSuccess) break;
             dl = (const int *)buf;

@@ -1525,3 +1525,27 @@ def test_diagnostics_of_many_ranks(P, L):
     for key in ("cv_identity", "cv_placed", "eta_ep", "attention", "joint"):
         assert abs(got[key] - want[key]) <= F64_RTOL * abs(want[key]), key
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,L,P,D,R,edp,ns", [
+    (40, 3, 132, 2, 2, None, (1, 2, 400)),              # layers of 33 chunks: more than a warp has lanes
+    (60, 5, 256, 3, 2, [0, 1, 1], (1, 7, 300)), (30, 9, 1020, 2, 2, None, (1, 2, 90)),
+    (64, 4, 4, 2, 3, None, (256, 270, 290)),            # both sides of the line between few and many layouts
+    (2048, 6, 16, 16, 15, None, (1, 2, 3, 4)), (3000, 3, 8, 2, 3, [0, 0], (1, 150, 240)),
+    (4096, 2, 4, 32, 40, None, (1, 2))])                # 1280 row-shards of 4096 samples: many from the first layout on
+def test_scoring_at_the_edges_of_its_forms(N, L, P, D, R, edp, ns):
+    w = make_window(custom_spec("forms", N, L, P, 2, 4096, D, P, 2, 0, data_seed=N + P))
+    ref = oracle_front(w, edp, R)
+    ctx = load(w, edp=edp, min_rows=R)
+    check_front(w, ctx, ref)
+    check_eval(w, ctx, ref, edp, n=3)
+    s = w.spec
+    rng = np.random.default_rng(P)
+    for n in ns:
+        lays = rng.integers(0, ref["R"] * D, (n, N)).astype(np.int32)
+        some = sorted({0, n // 2, n - 1})
+        want = oracle.eval_layouts(w.lengths, ref["q"], lays[some], ref["R"], s.token_cap, D, edp, s.alpha, s.beta)["score"]
+        for _ in range(2):                              # the scratch is clear again after a call
+            fx, _f64 = rp.rp_eval_population(ctx, lays)
+            assert (fx[some] == want).all()
+    rp.rp_destroy(ctx)
