@@ -346,7 +346,7 @@ int rp_debug_l2_read_rate(int64_t bytes, int32_t reps, double *gb_per_s);
 /* Which chain kernel rp_anneal runs for this context (valid after rp_pack_rows; inspection only):
  * 0 = warp per candidate (k_anneal_wpc), 1 = 128 threads per chain (k_anneal_level), 2 = warp per
  * chain (k_anneal_warp), 3 = one layer per lane (k_anneal_row; windows whose rows it would compress decide
- * between 2 and 3 in the first rp_anneal call). */
+ * between 2 and 3, some windows of few layers between 0 and 3, in the first rp_anneal call that is long enough). */
 int rp_debug_chain_kernel(rp_ctx *ctx, int32_t *which);
 /* Number of kernels this library has launched in this process so far. */
 int64_t rp_debug_launch_count(void);

@@ -936,10 +936,11 @@ k_make_rows(RpDims dm, const int *__restrict__ t, const int *__restrict__ q, con
 
 // Member m = blockIdx.x, row-shard rg = blockIdx.y: the slack (sum of the busiest loads less the samples' f), and (Wr != null) the row-shard's
 // slice in row form, in the place its table names (windows without a table: cell m of the pool).
-// Compressed rows also count the row-shards with a layer whose three columns do not decide the maximum.
+// Compressed rows also count the row-shards with a layer whose three columns do not decide the maximum; `loose`: counts those
+// whose busiest loads exceed their samples' f by more than a sixteenth.
 __global__ void __launch_bounds__(256)
 k_member_rows(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *__restrict__ static_blk, RpStatic sl, const int2 *__restrict__ tf,
-              const int *__restrict__ qr, int rlp, int comp, i64 *__restrict__ Fo, int *__restrict__ Wr, const int *__restrict__ wloc, int *__restrict__ undecided)
+              const int *__restrict__ qr, int rlp, int comp, i64 *__restrict__ Fo, int *__restrict__ Wr, const int *__restrict__ wloc, int *__restrict__ undecided, int loose)
 {
     extern __shared__ int list[];                       // [N] samples of the row-shard
     __shared__ int n_s, bad_s;
@@ -955,7 +956,11 @@ k_member_rows(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *
         if (__ldg(rg_of + cells[i]) == rg) { f += __ldg(&tf[i].y); if (Wr) list[atomicAdd(&n_s, 1)] = i; }
     if (f) atomicAdd(&f_s, (u64)f);
     __syncthreads();
-    if (tid == 0) Fo[(size_t)m * dm.RG + rg] = ((const i64 *)(blob + bl.off_Esum))[rg] - (i64)f_s;
+    if (tid == 0) {
+        const i64 es = ((const i64 *)(blob + bl.off_Esum))[rg], slack = es - (i64)f_s;
+        Fo[(size_t)m * dm.RG + rg] = slack;
+        if (loose && slack * 16 > es) atomicAdd(undecided, 1);
+    }
     if (!Wr) return;
     const int n = n_s;
     const size_t slice = bl.off_wtab >= 0 ? (size_t)((const int *)(blob + bl.off_wtab))[rg] : (size_t)wloc[m] * dm.RG + rg;
@@ -1120,7 +1125,7 @@ int rp_launch_member_rows(rp_ctx *c, int n)
     RP_CUDA(cudaMemsetAsync(c->d_undecided, 0, sizeof(int), c->stream));
     k_member_rows<<<dim3(n, dm.RG), 256, smem, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_static, c->sl, (const int2 *)c->d_tf, X.qr,
                                                             X.rlp, X.comp, c->d_rowF + (size_t)c->cur * c->Ppop * dm.RG,
-                                                            sep ? c->d_Wr : nullptr, c->d_wloc, c->d_undecided);
+                                                            sep ? c->d_Wr : nullptr, c->d_wloc, c->d_undecided, c->row_check);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     c->row_counted = n;

@@ -756,6 +756,16 @@ int rp_launch_anneal_wpc(rp_ctx *c, const AnnealArgs &A0)
     return launch_wpc<4>(c, A, ws, smem, chunks);
 }
 
+// Whether the launch below is possible for this window, its chains two to an SM.
+bool rp_wpc_one_launch(const rp_ctx *c)
+{
+    const RpDims &dm = c->dm;
+    int ws = 0;
+    if (!rp_uses_wpc(dm) || rp_wpc_warps(c->Ppop) != 8 || c->Ppop > 256 || c->Ppop > 2 * rp_sms(c)) return false;
+    const size_t smem = rp_wpc_smem_bytes(dm, c->bl, c->sl, 8, &ws);
+    return ws && smem + 16 + (size_t)c->Ppop * 12 <= 220 * 1024;
+}
+
 // One launch for all levels.  Possible when the rank loads live on chip, the population is at most
 // one member per thread (the level barrier is worked out by every CTA for itself) and every chain
 // can be resident at once (cooperative launch, checked with the occupancy calculator).  *done = 0

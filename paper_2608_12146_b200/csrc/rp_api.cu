@@ -1019,11 +1019,16 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
         if (rp_may_use_row(c)) {
             if (!c->rows_made) { RP_TRY(rp_launch_make_rows(c)); c->rows_made = 1; }
             if (!c->rows_current) { RP_TRY(rp_launch_member_rows(c, c->row_members)); c->rows_current = 1; }
-            if (rp_row_compressed(c) && c->row_undecided < 0) {
+            const bool check = c->row_check && (long long)NL * p->steps_per_level >= 1000;
+            if ((rp_row_compressed(c) || check) && c->row_undecided < 0) {
                 int *u = (int *)(c->h_pin + 60);
                 RP_CUDA(cudaMemcpyAsync(u, c->d_undecided, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
                 RP_CUDA(cudaStreamSynchronize(c->stream));
                 c->row_undecided = *u;
+            }
+            if (check) {                       // decided until the population is built anew
+                if ((long long)c->row_undecided * 4 > (long long)c->row_counted * c->dm.RG) c->row_mode = 0;
+                c->row_check = 0;
             }
         }
         row = rp_uses_row(c);

@@ -149,6 +149,7 @@ struct rp_ctx {
     int sms;                   // SMs that may hold the CTAs of a launch which wait for one another
     int row_cw;                // chains per CTA of the launch that runs all levels
     int row_mode;              // 0 = not for this window, 1 = one launch for all levels (rank loads on chip), 2 = one launch per level
+    int row_check;             // row_mode 1, if few row-shards are loose (see rp_decide_layouts): looked at by the first rp_anneal call
     int rows_current;          // the row-shard sums (and rows kept apart) describe the population
     int full_stale;            // that kernel ran on rows kept apart: d_W no longer describes the population
     int row_undecided;         // compressed rows: row-shards of the evaluated members that they do not decide, -1 = not read back yet
@@ -300,6 +301,7 @@ struct RpSlab {
 int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj, i64 eta_q16, int *order,
                      int *n_distinct, i64 *dist);
 bool rp_uses_wpc(const RpDims &dm);
+bool rp_wpc_one_launch(const rp_ctx *c);
 bool rp_uses_warp_chains(const rp_ctx *c);
 bool rp_may_use_row(const rp_ctx *c);
 bool rp_uses_row(const rp_ctx *c);

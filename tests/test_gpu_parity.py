@@ -1549,3 +1549,30 @@ def test_scoring_at_the_edges_of_its_forms(N, L, P, D, R, edp, ns):
             fx, _f64 = rp.rp_eval_population(ctx, lays)
             assert (fx[some] == want).all()
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("L,P,D,edp,pop,mixes,kernel", [
+    (32, 4, 4, [1, 2, 3, 0], 9, 4, "k_anneal_wpc"), (8, 8, 3, [2, 0, 1], 256, 4, "k_anneal_wpc"),
+    (8, 8, 3, [2, 0, 1], 257, 4, "k_anneal_row"), (5, 12, 3, [2, 0, 1], 20, 4, "k_anneal_row"),
+    (6, 16, 4, None, 30, 4, "k_anneal_wpc"), (3, 32, 2, None, 60, 4, "k_anneal_wpc"), (7, 16, 4, None, 30, 4, "k_anneal_row"),
+    (12, 4, 2, None, 20, 4, "k_anneal_wpc"), (13, 4, 2, None, 20, 4, "k_anneal_row"), (12, 4, 2, None, 20, 1, "k_anneal_row"),
+    (6, 16, 4, None, 30, 1, "k_anneal_row"), (3, 32, 2, None, 200, 1, "k_anneal_row"), (4, 32, 4, [0, 0, 1, 1], 12, 4, "k_anneal_row")])
+def test_windows_that_stay_with_the_warp_per_candidate_kernel(L, P, D, edp, pop, mixes, kernel):
+    """Permuted one-slot shards, and few layers of many ranks whose row-shards differ in their busiest ranks: both sides of the
+    rules, first call and a second one that goes on."""
+    if mixes == 1:
+        w = one_heavy_expert("stay", np.random.default_rng(L).integers(20_000, 60_000, 70), L, 2 * P, 2, 1 << 19, D, P, pop, 0.4)
+    else:
+        w = make_window(custom_spec("stay", 70, L, 2 * P, 2, 4096, D, P, pop, 0, data_seed=L * P))
+    s = w.spec
+    ref = oracle_front(w, edp, 4)
+    ctx = load(w, pop=pop, edp=edp, min_rows=4)
+    check_front(w, ctx, ref)
+    want, stats = check_anneal(w, ctx, ref, edp, pop, 3, 340, t_ratio=0.6, check_members=2)
+    assert rp.rp_debug_chain_kernel(ctx) == kernel and stats.accepted > 0
+    want = oracle.anneal(w.lengths, ref["q"], want["final_pop"], ref["R"], s.token_cap, D, n_levels=2, steps=33, t0=1e-4,
+                         t_ratio=0.5, p_reloc=0.5, p_guide=0.3, seed=s.anneal_seed, edp_of_dp=edp, alpha=s.alpha, beta=s.beta)
+    rp.rp_anneal(ctx, n_levels=2, steps_per_level=33, t0=1e-4, t_ratio=0.5, p_reloc=0.5, p_guide=0.3)
+    assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (2, pop, 3), np.int64) == want["term"]).all()
+    assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, 70), np.int32) == want["final_pop"]).all()
+    rp.rp_destroy(ctx)
