@@ -300,7 +300,8 @@ typedef enum {
  *     gives up after that many microseconds (default 2 s + 50 us per step of a level).
  *   RP_KNOB_STALL_ONE_CHAIN: chain 0 waits once more, after its copies have landed, on a barrier
  *     phase that nothing completes: the wait runs out and rp_anneal returns RP_ERR_TIMEOUT.
- *   RP_KNOB_LAUNCH_PER_LEVEL (set before rp_pack_rows): how rp_anneal launches windows whose chains can
+ *   RP_KNOB_LAUNCH_PER_LEVEL (any time before the first rp_anneal; between two calls it changes only how the
+ *     population's present form is launched): how rp_anneal launches windows whose chains can
  *     all be resident at once with their rank loads on chip.  0 or 2 = one launch for all levels (lowest
  *     latency of a single plan); 1 = one launch per level (two windows planned at once on two
  *     streams then share the GPU, which two launches of the first kind cannot).

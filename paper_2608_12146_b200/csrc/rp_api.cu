@@ -1189,6 +1189,29 @@ extern "C" int rp_debug_stage_times(rp_ctx *c, double *ms)
     return RP_OK;
 }
 
+// The population laid out as the knobs now want it, where that is another way than it was built in (rp_pack_rows decides; before
+// rp_anneal the members are the first row_members ones in turn, so these are all there is to keep).
+static int relayout_population(rp_ctx *c)
+{
+    if (c->stage != 3) return RP_OK;
+    const RpDims dm = c->dm;
+    const RpBlob bl = c->bl;
+    const int row_mode = c->row_mode, row_check = c->row_check;
+    rp_decide_layouts(c);
+    if (c->row_mode == row_mode && c->dm.slices == dm.slices) return RP_OK;
+    c->dm = dm; c->bl = bl; c->row_mode = row_mode; c->row_check = row_check;
+    int *lay = nullptr;
+    const int n = c->row_members;
+    RP_TRY(dev_alloc(c, &lay, (size_t)n * dm.N));
+    k_gather_cells<<<n, 256, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, dm.N, lay);
+    ++g_rp_launches;
+    int st = build_population(c);
+    if (st == RP_OK) st = install_population(c, lay, n);
+    dev_free(c, lay);
+    if (st != RP_OK) c->stage = 2;             // no population any more: rp_pack_rows builds one
+    return st;
+}
+
 extern "C" int rp_debug_set_knob(rp_ctx *c, int knob, int64_t value)
 {
     if (!c || value < 0) return RP_ERR_ARG;
@@ -1203,7 +1226,8 @@ extern "C" int rp_debug_set_knob(rp_ctx *c, int knob, int64_t value)
             c->knob_stall = value ? 1 : 0; return RP_OK;
         case RP_KNOB_LAUNCH_PER_LEVEL:
             if (value > 2) return RP_ERR_ARG;
-            c->knob_level_launches = (int)value; return RP_OK;
+            c->knob_level_launches = (int)value;
+            return relayout_population(c);
         case RP_KNOB_RANK_LOAD_SLICES:
             if (value > 2) return RP_ERR_ARG;
             c->knob_slices = (int)value; return RP_OK;

@@ -1576,3 +1576,32 @@ def test_windows_that_stay_with_the_warp_per_candidate_kernel(L, P, D, edp, pop,
     assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (2, pop, 3), np.int64) == want["term"]).all()
     assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, 70), np.int32) == want["final_pop"]).all()
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,L,P,D,R,edp,pop", [(70, 32, 4, 3, 3, None, 21), (900, 24, 2, 8, 31, None, 200), (90, 20, 32, 4, 3, [0, 1, 1, 0], 160)])
+@pytest.mark.parametrize("seeds", ["length_only", "trials", "two_plans"])
+def test_launch_form_asked_for_after_packing(N, L, P, D, R, edp, pop, seeds):
+    """RP_KNOB_LAUNCH_PER_LEVEL set when the population has been built, or even seeded: the same kernel and launches as set before,
+    and the population is what it was."""
+    w = make_window(custom_spec("late_knob", N, L, 2 * P, 2, 4096, D, P, pop, 0, data_seed=N))
+    s = w.spec
+    ref = oracle_front(w, edp, R)
+    forms = []
+    for early in (True, False):
+        ctx = load(w, pop=pop, edp=edp, min_rows=R)
+        if early:
+            rp.rp_debug_set_knob(ctx, "LAUNCH_PER_LEVEL", 1)
+        check_front(w, ctx, ref)
+        if seeds == "trials":
+            rp.rp_seed_population(ctx, 4)
+        elif seeds == "two_plans":
+            rp.rp_init_population(ctx, 2)
+        if not early:
+            before = rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32)
+            rp.rp_debug_set_knob(ctx, "LAUNCH_PER_LEVEL", 1)
+            assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == before).all()
+        init = rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32)
+        _, stats = check_anneal(w, ctx, ref, edp, pop, 3, 30, t_ratio=0.6, check_members=2, init=init)
+        forms.append((rp.rp_debug_chain_kernel(ctx), stats.kernel_launches))
+        rp.rp_destroy(ctx)
+    assert forms[0] == forms[1]
