@@ -311,7 +311,8 @@ typedef enum {
  *   RP_KNOB_CHAIN_KERNEL: which chain kernel runs the levels.  0 = chosen by the window (one layer of the rank
  *     loads per lane wherever a row fits a warp's registers, whole or compressed; else one warp per chain, or
  *     several warps per chain); 1 = always several warps per chain; 2 = one warp per chain with whole
- *     rows staged in shared memory, where the rank loads live in the slice pool.
+ *     rows staged in shared memory, where the rank loads live in the slice pool; 3 (set before rp_pack_rows) =
+ *     one layer per lane wherever it fits, however many row-shards compressed rows leave undecided.
  *   RP_KNOB_RESIDENT_SMS: at most this many SMs are taken to hold the CTAs of a launch that wait for
  *     one another (0 = all the device reports), as where a context owns only a part of a GPU. */
 typedef enum { RP_KNOB_BARRIER_WORKSPACE = 1, RP_KNOB_WAIT_POLLS = 2, RP_KNOB_STALL_ONE_CHAIN = 3,

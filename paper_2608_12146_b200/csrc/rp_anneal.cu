@@ -411,7 +411,8 @@ void rp_decide_layouts(rp_ctx *c)
     // chain's rank loads fit on chip at once, else with the rank loads as slices.  (With one launch per level asked
     // for, windows whose rank loads the warp-per-candidate kernel keeps on chip stay with that kernel.)
     c->row_mode = 0; c->row_check = 0;
-    if (c->knob_chain_kernel == 0 && c->knob_slices == 0) {
+    const bool any = c->knob_chain_kernel == 3;                // (inspection hook: wherever it fits)
+    if ((c->knob_chain_kernel == 0 || any) && c->knob_slices == 0) {
         // Two kinds of window stay with the warp-per-candidate kernel where that runs all levels in one launch too:
         //  * one slot per row-shard, but slot d is not shard d, at most a layer per lane (20 levels of 100 steps: L = 24, P = 4,
         //    40 cells, 148 members 1.29 ms and 1.94 with one layer per lane; L = 6, P = 8, 24 cells 1.50 and 2.12; on average
@@ -422,7 +423,7 @@ void rp_decide_layouts(rp_ctx *c)
         //    shards, L = 8, P = 4, 24 cells 1.10 and 1.35; L = 3, P = 8 1.07 and 1.34; two or more shards of more layers even or
         //    the other way).  Where all samples follow one routing mix no row-shard is loose, and one layer per lane takes 0.74
         //    to 0.93 of the time; with four mixes 25 to 100 % are.  Finding out costs 10 us: for calls of 1000 steps and more.
-        const bool pow2 = dm.P >= 4 && (dm.P & (dm.P - 1)) == 0, wpc = c->knob_level_launches != 1 && pow2 && rp_wpc_one_launch(c);
+        const bool pow2 = dm.P >= 4 && (dm.P & (dm.P - 1)) == 0, wpc = !any && c->knob_level_launches != 1 && pow2 && rp_wpc_one_launch(c);
         if (wpc && dm.G == dm.D && !dm.own_shard && dm.L <= 32) return;
         c->row_check = wpc && dm.own_shard && ((dm.L <= 6 && dm.P >= 16) || (dm.L <= 12 && dm.G <= 2));
         if (c->knob_level_launches != 1 && rp_row_fits_chip(c, c->bl, c->sl)) c->row_mode = 1;
@@ -438,9 +439,9 @@ bool rp_row_compressed(const rp_ctx *c) { return c->row_mode == 2 && rp_row_kind
 // this runs the warp-per-chain kernel on whole rows).
 bool rp_may_use_row(const rp_ctx *c)
 {
-    if (!c->row_mode || c->knob_chain_kernel != 0) return false;
+    if (!c->row_mode || (c->knob_chain_kernel != 0 && c->knob_chain_kernel != 3)) return false;
     if (c->row_mode == 1) return c->knob_level_launches != 1;
-    return !rp_row_compressed(c) || c->row_undecided < 0 || (long long)c->row_undecided * 64 <= (long long)c->row_counted * c->dm.RG;
+    return !rp_row_compressed(c) || c->knob_chain_kernel == 3 || c->row_undecided < 0 || (long long)c->row_undecided * 64 <= (long long)c->row_counted * c->dm.RG;
 }
 bool rp_uses_row(const rp_ctx *c) { return rp_may_use_row(c) && !(rp_row_compressed(c) && c->row_undecided < 0); }
 

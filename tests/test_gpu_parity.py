@@ -1605,3 +1605,51 @@ def test_launch_form_asked_for_after_packing(N, L, P, D, R, edp, pop, seeds):
         forms.append((rp.rp_debug_chain_kernel(ctx), stats.kernel_launches))
         rp.rp_destroy(ctx)
     assert forms[0] == forms[1]
+
+
+COMPRESSED_CASES = [
+    # name, N, L, E, P, D, edp, min_rows, pop: rows of three ranks and a bound per layer, whatever they leave undecided
+    ("comp_33_layers", 90, 33, 64, 32, 3, None, 3, 20),            # two layers per lane
+    ("comp_65_layers", 60, 65, 32, 32, 2, None, 4, 9),             # four
+    ("comp_128_layers", 40, 128, 32, 32, 2, [1, 0], 3, 5),         # a permuted shard map
+    ("comp_48_ranks", 70, 12, 96, 48, 3, [0, 1, 1], 3, 30),        # ranks in two passes, shards of two slots
+    ("comp_128_ranks", 50, 5, 128, 128, 4, None, 2, 40),
+    ("comp_20_ranks", 64, 40, 40, 20, 4, [0, 0, 1, 1], 2, 16),
+    ("comp_long", 1500, 6, 48, 48, 2, None, 1, 6),                 # 700 samples a row-shard: collected a piece at a time
+    ("comp_one_shard", 900, 9, 40, 40, 3, [0, 0, 0], 1, 1200)]
+
+
+def compressed_window(spec):
+    name, N, L, E, P, D, edp, min_rows, pop = spec
+    w = make_window(custom_spec(name, N, L, E, 2, 4096 if N < 1000 else 1 << 18, D, P, pop, 0, data_seed=len(name) + N))
+    if N >= 900:                                    # short samples: all of a row-shard's in a few cells
+        rng = np.random.default_rng(N)
+        w.lengths[:] = rng.integers(1, 3 if N < 1000 else 150, N)
+        mixes = rng.dirichlet(np.full(E, 0.3), size=(4, L))
+        w.demand[:] = rng.multinomial((2 * w.lengths.astype(np.int64))[:, None], mixes[rng.integers(0, 4, N)])
+    return w
+
+
+@pytest.mark.parametrize("spec", COMPRESSED_CASES, ids=[e[0] for e in COMPRESSED_CASES])
+def test_compressed_rows_with_open_layers(spec):
+    """Compressed rows on windows of four routing mixes, where many layers are left open and added up from the samples; whole
+    trajectories, then on by another kernel and back."""
+    name, N, L, E, P, D, edp, min_rows, pop = spec
+    w = compressed_window(spec)
+    s = w.spec
+    ref = oracle_front(w, edp, min_rows)
+    ctx = load(w, pop=pop, edp=edp, min_rows=min_rows)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 3)
+    check_front(w, ctx, ref)
+    steps = 60 if pop < 1000 else 12
+    want, stats = check_anneal(w, ctx, ref, edp, pop, 3, steps, t_ratio=0.6, check_members=2, t0=1e-2)
+    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.accepted > 0
+    for knob in (1, 3):
+        rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", knob)
+        want = oracle.anneal(w.lengths, ref["q"], want["final_pop"], ref["R"], s.token_cap, D, n_levels=2, steps=steps, t0=1e-4,
+                             t_ratio=0.5, p_reloc=0.5, p_guide=0.3, seed=s.anneal_seed, edp_of_dp=edp, alpha=s.alpha, beta=s.beta,
+                             n_threads=8)
+        rp.rp_anneal(ctx, n_levels=2, steps_per_level=steps, t0=1e-4, t_ratio=0.5, p_reloc=0.5, p_guide=0.3)
+        assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (2, pop, 3), np.int64) == want["term"]).all()
+        assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == want["final_pop"]).all()
+    rp.rp_destroy(ctx)
