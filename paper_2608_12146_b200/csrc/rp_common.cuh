@@ -358,8 +358,8 @@ static __device__ __noinline__ u32 rp_nl2_fraction(u64 m)
 // The same from the logarithm in double precision: m in [1, 2) has 32 bits at most, log2(m) is within 2^-53 (one ulp), and the
 // truncations of the definition, 2^-63 of m halved from square to square, lower the logarithm by less than 2^-61.  So the
 // first 24 fraction bits are the definition's unless the rest is within 2^-26 of 0 or 1 (one word in 2^25, and m = 1):
-// then the definition decides.  (Compared for all 2^32 words.)  24 squarings are a chain of 1000 cycles and 350 instructions for
-// every 32 steps of a chain: large 3.01 -> 2.91 ms, wide 11.8 -> 11.6, heavy 78.9 -> 77.8.
+// then the definition decides.  (The words next to a boundary are listed and compared in a test.)  24 squarings are a chain
+// of 1000 cycles and 350 instructions for every 32 steps of a chain: large 3.01 -> 2.91 ms, wide 11.8 -> 11.6, heavy 78.9 -> 77.8.
 __device__ __forceinline__ u64 rp_nl2(u32 x)
 {
     const i64 v = __double_as_longlong((double)x + 1.0);

@@ -46,7 +46,6 @@ __device__ __forceinline__ bool first_fit_runs(const RpDims &dm, const u64 *keys
             else {
                 const int4 q = ((const int4 *)rem)[w * 32 + lane];
                 v[0] = q.x; v[E > 1 ? 1 : 0] = q.y; v[E > 2 ? 2 : 0] = q.z; v[E > 3 ? 3 : 0] = q.w;
-                if (E == 1) v[0] = q.x;
             }
             int big = v[0];
 #pragma unroll

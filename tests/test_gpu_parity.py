@@ -125,6 +125,21 @@ def check_anneal(w, ctx, ref, edp, pop, levels, steps, threads=8, t_ratio=None, 
 
 
 # ---------------------------------------------------------------------------------------------
+def log_boundary_words():
+    """Words whose (x+1)'s base-2 logarithm lies within 2^-26 of a 24-bit fraction boundary, powers of two aside: where the
+    device leaves the double-precision logarithm for the definition."""
+    k = np.arange(1, 1 << 24, dtype=np.float64)
+    root = np.exp2(k / (1 << 24))
+    found = []
+    for e in range(25, 32):
+        exact = root * float(1 << e)
+        near = np.abs(np.rint(exact) - exact) < 2.0 ** -17          # (a superset: one part in 2^49 of up to 2^32)
+        v, kk = np.rint(exact[near]).astype(np.uint64), k[near].astype(np.longdouble)
+        y = (np.log2(v.astype(np.longdouble)) - e) * (1 << 24)
+        found.append(v[np.abs(y - kk) < np.longdouble(2.0) ** -26])
+    return (np.unique(np.concatenate(found)) - 1).astype(np.uint32)
+
+
 def test_device_integer_functions_bit_exact():
     rng = np.random.default_rng(0)
     ctr = rng.integers(0, 2 ** 32, (4096, 4), dtype=np.uint64).astype(np.uint32)
@@ -137,6 +152,9 @@ def test_device_integer_functions_bit_exact():
     x = np.concatenate([rng.integers(0, 2 ** 32, 20000, dtype=np.uint64).astype(np.uint32),
                         np.array([0, 1, 2, 3, 2 ** 31 - 1, 2 ** 31, 2 ** 32 - 2, 2 ** 32 - 1], np.uint32),
                         (2 ** np.arange(1, 32, dtype=np.uint64) - 1).astype(np.uint32)])
+    near = log_boundary_words()
+    assert near.size > 100                 # one word in 2^25 is expected to lie there
+    x = np.concatenate([x, near, near - 1, near + 1])
     got = rp.rp_debug_nl2(x)
     assert got.tolist() == [oracle.nl2(int(v)) for v in x]
     z = np.concatenate([rng.integers(0, 34 << 32, 20000, dtype=np.uint64),
@@ -307,6 +325,7 @@ def test_large_windows_full_population(name, pop, levels, steps, t0, threads=16)
     ctx = load(w, pop=pop, device_inputs=True)
     check_front(w, ctx, ref)
     want, stats = check_anneal(w, ctx, ref, None, pop, levels, steps, threads=threads, check_members=2, t0=t0)
+    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row"
     assert stats.accepted > pop            # the levels did move
     if levels > 1:                          # resampling really replaced members and kept others
         anc = want["anc"][0]
@@ -852,16 +871,17 @@ def test_fuzz_warp_per_chain_kernel():
 
 
 def test_windows_planned_at_once_on_separate_streams():
-    """Three different windows (a warp-per-chain one with more than 32 KB of shared memory per
-    chain, a second warp-per-chain one, and one whose rank loads live on chip) planned at the same
-    time by three host threads, each on its own stream and context, several plans each: every
+    """Four different windows (two with more layers or ranks than stay on chip, one that does, one of
+    240 cells) planned, and their candidate stages run, at the same
+    time by four host threads, each on its own stream and context, several plans each: every
     plan equals the oracle's, so nothing process-wide (shared-memory limits of the kernels, memory
     pools, launch counters) is upset by another context."""
     import threading
     import torch
     cases = [("conc_a", 90, 40, 32, 2, 4096, 4, 32, None, 3, 37),        # L*P = 1280
              ("conc_b", 120, 20, 32, 2, 4096, 4, 32, [0, 1, 1, 0], 3, 25),
-             ("conc_c", 96, 5, 16, 2, 4096, 4, 4, None, 3, 40)]
+             ("conc_c", 96, 5, 16, 2, 4096, 4, 4, None, 3, 40),
+             ("conc_d", 300, 6, 16, 2, 4096, 16, 4, None, 15, 20)]        # 240 cells: larger candidate stages than the others'
     jobs = []
     for name, N, L, E, k, C, D, P, edp, min_rows, pop in cases:
         w = make_window(custom_spec(name, N, L, E, k, C, D, P, pop, 400, data_seed=len(name) * 19 + N))
@@ -870,12 +890,13 @@ def test_windows_planned_at_once_on_separate_streams():
         want = oracle.anneal(w.lengths, ref["q"], np.tile(ref["seed"], (pop, 1)), ref["R"], s.token_cap, D, n_levels=6, steps=40,
                              t0=s.t0, t_ratio=0.6, p_reloc=s.p_reloc, p_guide=s.p_guide, seed=s.anneal_seed, edp_of_dp=edp,
                              alpha=s.alpha, beta=s.beta)
-        jobs.append((w, edp, min_rows, pop, want))
+        cand = oracle_init_population(w, ref, edp, 12, pop, 4, 8, 1 << 16)
+        jobs.append((w, edp, min_rows, pop, want, cand))
     errors = []
 
     def worker(job):
         try:
-            w, edp, min_rows, pop, want = job
+            w, edp, min_rows, pop, want, cand = job
             s = w.spec
             stream = torch.cuda.Stream()
             for _ in range(6):
@@ -889,6 +910,10 @@ def test_windows_planned_at_once_on_separate_streams():
                 assert [st.proposed, st.feasible, st.accepted, st.improved] == want["counters"].tolist()
                 assert (layout == want["best_layout"]).all() and (fx == want["best_score"]).all()
                 assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, s.n_samples), np.int32) == want["final_pop"]).all()
+                rp.rp_pack_rows(ctx)                     # and the candidate stages
+                nd, picked = rp.rp_init_population(ctx, 12, 4, 8, 1 << 16)
+                assert nd == cand[0] and (picked == cand[1]).all()
+                assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, s.n_samples), np.int32) == cand[2]).all()
                 rp.rp_destroy(ctx)
         except Exception as e:          # reported by the main thread
             errors.append(repr(e))
