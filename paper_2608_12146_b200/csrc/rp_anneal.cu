@@ -434,9 +434,12 @@ void rp_decide_layouts(rp_ctx *c)
 
 bool rp_row_compressed(const rp_ctx *c) { return c->row_mode == 2 && rp_row_kind(c->dm) == 2; }
 
-// Compressed rows: at most one row-shard in 64 of the members counted may need its loads added up anew (a
-// scored candidate names two, and adding one up costs about what ten candidates cost; a window that fails
-// this runs the warp-per-chain kernel on whole rows).
+// Compressed rows: at most one row-shard in 64 of the members counted may need its loads added up anew; a window
+// that fails this runs the warp-per-chain kernel on whole rows.  What an open row-shard costs depends on why it is open.  Where all
+// samples follow one routing mix and the counts' noise opens a few, the row form is ahead well beyond (wide windows: none of 288
+// open 7.9 ms and 28 for whole rows, two 14 and 30, three 10 and 16).  Samples of another mix open whatever row-shard they visit:
+// 2048 members, L = P = 32, 192 row-shards, 1 % of the samples 3.3 ms and 1.2 (three open), 3 % 4.8 and 1.3 (seven); L = 48, 288
+// row-shards, 1 % 2.5 and 1.6 (six).  The line keeps the first kind and refuses most of the second.
 bool rp_may_use_row(const rp_ctx *c)
 {
     if (!c->row_mode || (c->knob_chain_kernel != 0 && c->knob_chain_kernel != 3)) return false;

@@ -30,7 +30,8 @@
 // warps per scheduler; with 7 (large) their latency, about 3900 cycles; launched once for all levels (medium)
 // about 2700 cycles a round and 20 us a level for the slowest chain, the barrier and the states.  A level's time before (the
 // warp-per-chain kernel; medium: warp per candidate) and now: heavy 15.0 -> 3.9 ms, wide 1.2 -> 0.41 ms,
-// large 0.21 -> 0.13 ms, medium 50 -> 36 us (plans: 301 -> 78, 24.0 -> 8.3, 4.8 -> 2.8, 1.12 -> 0.87 ms).
+// large 0.21 -> 0.13 ms, medium 50 -> 36 us (plans: 301 -> 78, 24.0 -> 8.1 to 10.8 over windows of the kind, 4.8 -> 2.8,
+// 1.12 -> 0.87 ms).
 // Step for step this is the sequential chain: proposals are evaluated against the current state,
 // feasible ones are decided in step order, and the speculation is redone after an acceptance.
 //
