@@ -23,7 +23,7 @@
 //    other rank's load: the sum over the samples of each one's largest count among those ranks.
 //    While the bound does not exceed the three, their maximum is the layer's maximum; where it
 //    does, the layer's loads are added up from the samples of the row-shard.  Used when the seed's
-//    row-shards nearly all satisfy it (checked on the device, see rp_launch_rows): 16 bytes per layer
+//    row-shards nearly all satisfy it (checked on the device, see k_member_rows): 16 bytes per layer
 //    instead of 4*P: an eighth of the traffic at 32 ranks.
 //  * No staging area, so 12 to 16 chains per SM instead of 5 to 10.
 // What bounds it now: with 14 to 16 chains per SM (heavy) the instructions of a round, about 4900 cycles with four
