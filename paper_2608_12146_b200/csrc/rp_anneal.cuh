@@ -87,12 +87,12 @@ struct MoveS { int reloc, i, i2, c1, c2; };
 // Purposes: 0 = proposal words A, 1 = proposal words B, 2 = accept word.
 // The uniform branch is stored as a tournament between a candidate and itself, so that the
 // proposal rule below needs no branch on it.
-__device__ __forceinline__ StepRec rp_make_step_rec(const AnnealArgs &A, int level, u64 tau, u32 k, u32 j)
+// In two parts, so that a caller can fetch what the candidates name ahead of the accept threshold's arithmetic.
+__device__ __forceinline__ StepRec rp_step_picks(const AnnealArgs &A, int level, u32 k, u32 j)
 {
     const RpDims &dm = A.dm;
     const uint4 a = rp_philox(k, (u32)level, j, 0u, A.key0, A.key1);
     const uint4 b = rp_philox(k, (u32)level, j, 1u, A.key0, A.key1);
-    const uint4 xw = rp_philox(k, (u32)level, j, 2u, A.key0, A.key1);
     const bool reloc = (u64)a.x < A.rho_q32, guided = (u64)a.y < A.guide_q32;
     StepRec r;
     r.i0 = rp_pick(a.z, dm.N);
@@ -106,11 +106,22 @@ __device__ __forceinline__ StepRec rp_make_step_rec(const AnnealArgs &A, int lev
         r.i3 = reloc ? rp_pick(b.y, dm.K) : rp_pick(b.y, dm.N);
     }
     r.bz = b.z;
+    r.thr = 0;
+    r.flags = (reloc ? 1u : 0u) | (guided ? 2u : 0u);
+    return r;
+}
+__device__ __forceinline__ void rp_step_threshold(const AnnealArgs &A, int level, u64 tau, u32 k, u32 j, StepRec &r)
+{
+    const uint4 xw = rp_philox(k, (u32)level, j, 2u, A.key0, A.key1);
     const u64 nl = rp_nl2(xw.x);
     const u64 hi = __umul64hi(tau, nl), lo = tau * nl;
-    const bool sat = (hi >> 30) != 0;
     r.thr = (hi << 32) | (lo >> 32);
-    r.flags = (reloc ? 1u : 0u) | (guided ? 2u : 0u) | (sat ? 4u : 0u);
+    if (hi >> 30) r.flags |= 4u;
+}
+__device__ __forceinline__ StepRec rp_make_step_rec(const AnnealArgs &A, int level, u64 tau, u32 k, u32 j)
+{
+    StepRec r = rp_step_picks(A, level, k, j);
+    rp_step_threshold(A, level, tau, k, j, r);
     return r;
 }
 

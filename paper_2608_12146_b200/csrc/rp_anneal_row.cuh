@@ -4,6 +4,8 @@
 
 #define ROW_MAX_WARPS 8          // chains of a CTA in the launch that runs all levels, at most
 #define ROW_THREADS 256          // its threads
+#define ROW_SMEM_MAX (220 * 1024)
+#define ROW_LIST 256             // samples of a row-shard collected at a time where its loads are added up anew
 
 struct RowArgs {
     const int *qr;               // [N][rlp] demand rows: cpl 16-byte chunks per layer
@@ -12,10 +14,14 @@ struct RowArgs {
     const i64 *F_src;            // [P_pop][RG] slack of a row-shard: sum of its busiest loads less sum of its samples' tf.y; the level's start, its end, both buffers
     i64 *F_dst, *F_buf;
     int rlp, cpl, comp;
-    int off_tab, off_leF, off_chain;                                       // shared memory of the CTA
-    int off_F, off_book, off_wtab, off_spare, off_top, off_cell, off_snap, off_recs, off_list, off_W;   // of one chain
+    int off_tab, off_leF, off_chain, off_tf;                                       // shared memory of the CTA
+    int off_E, off_Q, off_TC, off_U, off_S, cs_bytes;                      // of one chain: records handed on from level to level,
+    int off_F, off_mbar, off_ws, off_top, off_cell, off_snap, off_recs, off_list, off_W;   // the rest
     int chain_bytes, smem_bytes, cw, recs;
 };
+
+__device__ __forceinline__ int4 sub4(const int4 &a, const int4 &b) { return make_int4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+__device__ __forceinline__ int4 add4(const int4 &a, const int4 &b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
 // Bounded wait of one thread until a counter that the other CTAs of the launch add to has reached
 // `target`; false when the time allowed ran out or another chain has raised the time-out word.
@@ -35,3 +41,6 @@ __device__ __forceinline__ bool rp_wait_count(const int *ctr, int target, const 
         }
     }
 }
+
+int rp_launch_row_chip(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int l, int k, int grid, int *done);
+int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int l, int k, int grid);
