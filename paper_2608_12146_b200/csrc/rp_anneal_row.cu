@@ -120,13 +120,12 @@ k_member_rows(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *
 // ---------------------------------------------------------------------------------------------
 // Which windows, which form.
 // ---------------------------------------------------------------------------------------------
-static int lanes_of(int L) { return L <= 32 ? 1 : (L <= 64 ? 2 : (L <= 128 ? 4 : 0)); }      // layers per lane (template values)
 static int chunks_of(int cpl) { return cpl <= 1 ? 1 : (cpl <= 2 ? 2 : (cpl <= 4 ? 4 : (cpl <= 8 ? 8 : 0))); }
 
-// Chunks a lane holds per row, as the kernel is instantiated; 0 = not at all.
+// Chunks a lane that takes whole layers would hold per row, rounded up to powers of two; 0 = too many.
 static int row_chunks(const RpDims &dm, int cpl)
 {
-    const int l = lanes_of(dm.L), c = chunks_of(cpl);
+    const int l = rp_row_layers(dm), c = chunks_of(cpl);
     return l * c;
 }
 
@@ -190,7 +189,7 @@ int rp_row_kind(const RpDims &dm)
 {
     const int cpl = (dm.P + 3) / 4, nch = row_chunks(dm, cpl);
     if (nch >= 1 && nch <= 4) return 1;
-    if (dm.P >= 8 && dm.P <= 128 && lanes_of(dm.L)) return 2;      // (128: ranks the placement kernel orders)
+    if (dm.P >= 8 && dm.P <= 128 && rp_row_layers(dm)) return 2;      // (128: ranks the placement kernel orders)
     return 0;
 }
 
@@ -294,7 +293,7 @@ int rp_launch_anneal_row_all(rp_ctx *c, const AnnealArgs &A0, int *done)
     A.slices = c->dm.slices;
     A.smem_bytes = (unsigned)X.smem_bytes;
     A.lo.cand_layout = c->d_cand_layout;
-    return rp_launch_row_chip(c, A, X, lanes_of(c->dm.L), chunks_of(X.cpl), (c->Ppop + cw - 1) / cw, done);
+    return rp_launch_row_chip(c, A, X, (c->Ppop + cw - 1) / cw, done);
 }
 
 int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A);
@@ -309,7 +308,7 @@ int rp_launch_anneal_row(rp_ctx *c, AnnealArgs &A)
     A.smem_bytes = (unsigned)X.smem_bytes;
     A.slices = 1;
     A.lo.cand_layout = nullptr;
-    RP_TRY(rp_launch_row_level(c, A, X, lanes_of(c->dm.L), chunks_of(X.cpl), c->Ppop));
+    RP_TRY(rp_launch_row_level(c, A, X));
     if (!A.last && rp_row_turns(c)) return rp_launch_level_turn(c, A);
     return rp_launch_level_end(c, A);
 }

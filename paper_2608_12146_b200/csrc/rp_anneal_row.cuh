@@ -42,5 +42,8 @@ __device__ __forceinline__ bool rp_wait_count(const int *ctr, int target, const 
     }
 }
 
-int rp_launch_row_chip(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int l, int k, int grid, int *done);
-int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int l, int k, int grid);
+// Layers per lane where a lane takes whole layers (0: too many layers); whether a row's chunks are dealt out to the lanes instead.
+static inline int rp_row_layers(const RpDims &dm) { return dm.L <= 32 ? 1 : (dm.L <= 64 ? 2 : (dm.L <= 128 ? 4 : 0)); }
+static inline bool rp_row_split(int cpl) { return cpl == 2 || cpl == 4; }
+int rp_launch_row_chip(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int grid, int *done);
+int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);

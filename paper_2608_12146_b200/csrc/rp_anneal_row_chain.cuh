@@ -276,17 +276,21 @@ __device__ __forceinline__ void row_barrier_warp(const AnnealArgs &A, int P, con
     }
 }
 
-// Warps per SM the register budget is set for.  Heavy (one chunk per lane) at 12 / 14 / 16 / 19 / 24 chains: 96 / 87.5 /
-// 90 / 100 / 112 ms a plan (spills from 19 on); wide (two) at 12 / 14 / 16 / 19: 10.8 / 11.9 / 11.9 / 16.0 ms; four chunks need the
-// registers of 12.  (Figures of the form before the records.)
-#define ROW_WARPS_PER_SM(GL, LPL, CPL) ((GL) == 32 && (LPL) * (CPL) == 1 ? 14 : 12)
+// Warps per SM the register budget is set for: heavy, a chain to a warp and one chunk per lane, at 12 / 13 / 14: 66.1 / 66.0 / 66.7 ms,
+// but 14 take windows of up to 2072 members at once; two chains to a warp 10 / 12 / 14: 57.0 / 57.8 / 55.8; more chunks, or shards of
+// several slots, need the registers of 12.
+#define ROW_WARPS_PER_SM(GL, LPL, CPL, IDENT) ((GL) == 16 || ((LPL) * (CPL) == 1 && (IDENT)) ? 14 : 12)
 
-// LPL layers per lane, CPL 16-byte chunks per layer (X.cpl <= CPL of them in use); GL lanes run a chain.  IDENT: slot d is shard d.
-template <int GL, int LPL, int CPL, bool CHIP, bool COMP, bool IDENT>
-__global__ void __launch_bounds__(CHIP ? ROW_THREADS : 32, CHIP ? 1 : ROW_WARPS_PER_SM(GL, LPL, CPL))
+// GL lanes run a chain, LPL layers per lane, CPL 16-byte chunks per layer (X.cpl <= CPL of them in use).  IDENT: slot d is shard d.
+// SPLIT (X.cpl = 2 or 4): the row's chunks are dealt out to the lanes in turn instead, CPL of them to a lane, and a layer's maximum
+// meets in shuffles: a load touches consecutive bytes, and no lane is idle for want of layers.  Whole layers of four chunks put the
+// lanes of a load 64 bytes apart, twelve lines for 24 layers, eight stores 440 cycles (large 2563 -> 2396 us, with candidates 3377 ->
+// 3303).  With the rank loads on chip only the demand rows would gain, and the shuffles cost as much (two shards 1190 and 1225 us).
+template <int GL, int LPL, int CPL, bool SPLIT, bool CHIP, bool COMP, bool IDENT>
+__global__ void __launch_bounds__(CHIP ? ROW_THREADS : 32, CHIP ? 1 : ROW_WARPS_PER_SM(GL, LPL, CPL, IDENT))
 k_anneal_row(const AnnealArgs A, const RowArgs X)
 {
-    constexpr int NCH = LPL * CPL;
+    constexpr int NCH = SPLIT ? CPL : LPL * CPL;
     constexpr bool ONE = GL == 32;                                       // a warp runs one chain: its branches are the warp's
     using G = Lanes<GL>;
     const RpDims &dm = A.dm;
@@ -310,10 +314,11 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
     const unsigned short *rowbase = (const unsigned short *)(sm_tab + A.sl.off_row);
 
     if (!CHIP && __ldcg(&A.status[RP_SW_TIMEOUT])) return;               // the call has failed already: nothing to do
-    const int L = dm.L, cpl = CPL == 1 ? 1 : X.cpl, rc = L * cpl;        // 16-byte chunks per layer and per row
-    const int rot = (CPL > 1 && (cpl & (cpl - 1)) == 0) ? cpl - 1 : 0;   // lanes start at different chunks: fewer bank conflicts
+    const int L = dm.L, cpl = CPL == 1 && !SPLIT ? 1 : X.cpl, rc = L * cpl;        // 16-byte chunks per layer and per row
+    const int rot = CHIP && CPL > 1 && (cpl & (cpl - 1)) == 0 ? cpl - 1 : 0;     // lanes start at different chunks: fewer bank conflicts
     // 16-byte chunk u of this lane
     auto chunk = [&](int u, bool &on) {
+        if (SPLIT) { const int c = lane + 32 * u; on = c < rc; return c; }
         const int ly = lg + GL * (u / CPL), k = u % CPL;
         on = ly < L && (CPL == 1 || k < cpl);
         return ly * cpl + (rot ? ((k + lane) & rot) : k);
@@ -634,7 +639,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                     // with one launch per level, whose chains share the SM's load path (ahead or here: wide 10.6 ms, heavy 79 ms; behind 8.5 and 64).
                     if (CHIP) look();
                     unsigned over = 0;                      // COMP: layers of this lane whose other ranks may be the busiest
-                    constexpr int NM = LPL, PER = NCH / NM;
+                    constexpr int NM = SPLIT ? CPL : LPL, PER = NCH / NM;
                     int mx[NM][2];
 #pragma unroll
                     for (int y = 0; y < NM; ++y) {
@@ -651,6 +656,20 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                             } else { m1 = max(m1, max4(a)); m2 = max(m2, max4(b)); }
                         }
                         mx[y][0] = m1; mx[y][1] = m2;
+                    }
+                    if (SPLIT) {
+#pragma unroll
+                        for (int o = 1; o < 8; o <<= 1) {
+                            if (o >= cpl) break;
+#pragma unroll
+                            for (int y = 0; y < NM; ++y) {
+                                mx[y][0] = max(mx[y][0], __shfl_xor_sync(G::FULL, mx[y][0], o));
+                                mx[y][1] = max(mx[y][1], __shfl_xor_sync(G::FULL, mx[y][1], o));
+                            }
+                        }
+                        if (lane & (cpl - 1))                              // one lane of a layer has its share of the sum
+#pragma unroll
+                            for (int y = 0; y < NM; ++y) mx[y][0] = mx[y][1] = 0;
                     }
                     if (COMP && __any_sync(G::FULL, over != 0)) {
 #pragma unroll
@@ -1013,10 +1032,10 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
     }
 }
 
-template <int GL, int LPL, int CPL, bool CHIP, bool COMP, bool IDENT>
+template <int GL, int LPL, int CPL, bool SPLIT, bool CHIP, bool COMP, bool IDENT>
 static int launch_row_t(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int grid, int *done)
 {
-    auto kern = k_anneal_row<GL, LPL, CPL, CHIP, COMP, IDENT>;
+    auto kern = k_anneal_row<GL, LPL, CPL, SPLIT, CHIP, COMP, IDENT>;
     // (always the same value, above anything a launch asks for: contexts that plan different
     // windows at once on different host threads then never lower each other's limit)
     RP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_SMEM_MAX));

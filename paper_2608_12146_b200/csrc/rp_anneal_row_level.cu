@@ -2,17 +2,23 @@
 #include "rp_anneal_row_chain.cuh"
 
 template <bool IDENT>
-static int launch(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int l, int k, int grid)
+static int launch(rp_ctx *c, const AnnealArgs &A, const RowArgs &X)
 {
+    const int l = rp_row_layers(c->dm), n = (c->dm.L * X.cpl + 31) / 32;
     int done;
-#define ROW_CASE(L_, K_, C_) if (l == L_ && k == K_ && X.comp == C_) return launch_row_t<32, L_, K_, false, C_, IDENT>(c, A, X, grid, &done)
-    ROW_CASE(1, 1, 1); ROW_CASE(2, 1, 1); ROW_CASE(4, 1, 1);
-    ROW_CASE(1, 1, 0); ROW_CASE(1, 2, 0); ROW_CASE(1, 4, 0); ROW_CASE(2, 1, 0); ROW_CASE(2, 2, 0); ROW_CASE(4, 1, 0);
+#define ROW_CASE(WHEN, L_, K_, SPLIT_, COMP_) if (WHEN) return launch_row_t<32, L_, K_, SPLIT_, false, COMP_, IDENT>(c, A, X, c->Ppop, &done)
+    if (X.comp) { ROW_CASE(l == 1, 1, 1, false, true); ROW_CASE(l == 2, 2, 1, false, true); ROW_CASE(l == 4, 4, 1, false, true); }
+    else if (rp_row_split(X.cpl)) {
+        ROW_CASE(n <= 1, 1, 1, true, false); ROW_CASE(n <= 2, 1, 2, true, false); ROW_CASE(n <= 3, 1, 3, true, false); ROW_CASE(n <= 4, 1, 4, true, false);
+    } else {
+        ROW_CASE(l == 1 && X.cpl == 1, 1, 1, false, false); ROW_CASE(l == 2 && X.cpl == 1, 2, 1, false, false);
+        ROW_CASE(l == 4 && X.cpl == 1, 4, 1, false, false); ROW_CASE(l == 1 && X.cpl == 3, 1, 3, false, false);
+    }
 #undef ROW_CASE
     return RP_ERR_STATE;
 }
 
-int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int l, int k, int grid)
+int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X)
 {
-    return c->dm.own_shard ? launch<true>(c, A, X, l, k, grid) : launch<false>(c, A, X, l, k, grid);
+    return c->dm.own_shard ? launch<true>(c, A, X) : launch<false>(c, A, X);
 }

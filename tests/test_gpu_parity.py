@@ -1678,3 +1678,18 @@ def test_compressed_rows_with_open_layers(spec):
         assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (2, pop, 3), np.int64) == want["term"]).all()
         assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == want["final_pop"]).all()
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,L,P,D,edp", [(40, 16, 8, 2, None), (40, 9, 16, 3, [0, 0, 1]), (44, 17, 16, 2, None), (36, 40, 8, 3, [1, 0, 1]),
+                                         (36, 31, 16, 2, [1, 0]), (30, 64, 8, 2, None), (48, 7, 12, 2, None), (48, 32, 12, 3, [0, 0, 1])])
+def test_rows_dealt_out_to_the_lanes(N, L, P, D, edp):
+    """One launch per level with whole rows: 16-byte chunks dealt out to the lanes in turn, one to four of them to a lane, the last
+    ones of some lanes missing; and the three chunks of twelve ranks, whole layers to a lane."""
+    pop = 1190
+    w = make_window(custom_spec("dealt", N, L, 2 * P, 2, 4096, D, P, pop, 400, data_seed=N + L))
+    ref = oracle_front(w, edp, 3)
+    ctx = load(w, pop=pop, edp=edp, min_rows=3)
+    check_front(w, ctx, ref)
+    _, stats = check_anneal(w, ctx, ref, edp, pop, 3, 21, t_ratio=0.5, check_members=2)
+    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.accepted > 0
+    rp.rp_destroy(ctx)
