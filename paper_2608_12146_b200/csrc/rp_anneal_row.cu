@@ -154,7 +154,7 @@ static void chain_layout(const RpDims &dm, const RpBlob &bl, const RpStatic &sl,
     X.off_cell = (int)c;  c += chip ? lay : 0;
     X.off_snap = (int)c;  c += chip ? lay : 0;
     // (records of 256 steps at most, twice)
-    X.recs = chip && cw < ROW_THREADS / 32 ? std::min(steps, 256) : 0;
+    X.recs = chip && cw < ROW_THREADS / 32 ? std::min(steps, 256) : (!chip && cw == 2 ? 16 : 0);       // (two chains a warp: 32 steps, once)
     X.off_recs = (int)c;  c += (size_t)2 * X.recs * sizeof(StepRec);
     c = (c + 15) & ~(size_t)15;
     X.off_list = (int)c;  c += X.comp ? (size_t)4 * (ROW_LIST + 1) : 0;
@@ -296,6 +296,24 @@ int rp_launch_anneal_row_all(rp_ctx *c, const AnnealArgs &A0, int *done)
     return rp_launch_row_chip(c, A, X, (c->Ppop + cw - 1) / cw, done);
 }
 
+// Whether two chains share a warp: compressed rows of up to 32 layers where slot d is shard d, if there are more members than chains
+// resident with a warp each, and shared memory keeps at least half as many again when they share.  A round takes longer then (heavy
+// 5900 cycles for two, 4300 for one) and half the warps do it: eight levels of 200 steps on heavy, one chain to a warp and two, 2072
+// members (all resident either way) 2.41 and 2.57 ms, 2600 3.43 and 2.87, 4096 4.27 and 3.43, 6000 5.94 and 5.52, 8192 7.66 and 6.33; on
+// its first 16 layers 2.32 and 2.20, 3.30 and 2.45, 4.20 and 2.99, 5.69 and 4.62, 7.36 and 5.36.  Of 48 layers a lane would have
+// three, and wide's 288 row-shards leave shared memory for six warps: 8.5 and 12.7 ms.
+static bool row_pairs(const rp_ctx *c, const RowArgs &X0)
+{
+    if (!X0.comp || !c->dm.own_shard || c->dm.L > 32) return false;
+    RowArgs X = X0;
+    const int room = 227 * 1024;
+    chain_layout(c->dm, c->bl, c->sl, X, false, 1, c->Ppop, 0);
+    const int one = std::min(14, room / (X.smem_bytes + 1024));
+    chain_layout(c->dm, c->bl, c->sl, X, false, 2, c->Ppop, 0);
+    const int two = 2 * std::min(14, room / (X.smem_bytes + 1024));
+    return c->Ppop > one * rp_sms(c) && 2 * two >= 3 * one;
+}
+
 int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A);
 int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A);
 
@@ -303,12 +321,13 @@ int rp_launch_anneal_row(rp_ctx *c, AnnealArgs &A)
 {
     RowArgs X;
     row_args(c, X);
-    chain_layout(c->dm, c->bl, c->sl, X, false, 1, c->Ppop, 0);
+    const bool pair = row_pairs(c, X);
+    chain_layout(c->dm, c->bl, c->sl, X, false, pair ? 2 : 1, c->Ppop, 0);
     if (X.smem_bytes > ROW_SMEM_MAX) return RP_ERR_RANGE;
     A.smem_bytes = (unsigned)X.smem_bytes;
     A.slices = 1;
     A.lo.cand_layout = nullptr;
-    RP_TRY(rp_launch_row_level(c, A, X));
+    RP_TRY(pair ? rp_launch_row_pair(c, A, X) : rp_launch_row_level(c, A, X));
     if (!A.last && rp_row_turns(c)) return rp_launch_level_turn(c, A);
     return rp_launch_level_end(c, A);
 }

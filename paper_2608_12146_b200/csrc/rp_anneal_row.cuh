@@ -47,3 +47,4 @@ static inline int rp_row_layers(const RpDims &dm) { return dm.L <= 32 ? 1 : (dm.
 static inline bool rp_row_split(int cpl) { return cpl == 2 || cpl == 4; }
 int rp_launch_row_chip(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int grid, int *done);
 int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);
+int rp_launch_row_pair(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);

@@ -1693,3 +1693,37 @@ def test_rows_dealt_out_to_the_lanes(N, L, P, D, edp):
     _, stats = check_anneal(w, ctx, ref, edp, pop, 3, 21, t_ratio=0.5, check_members=2)
     assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.accepted > 0
     rp.rp_destroy(ctx)
+
+
+PAIR_CASES = [
+    # as COMPRESSED_CASES, and the steps of a level: sixteen lanes to a chain, one or two layers to a lane
+    (("pair_16_layers", 80, 16, 64, 32, 3, None, 3, 45), 50),
+    (("pair_17_layers", 80, 17, 64, 32, 3, None, 3, 100), 33),
+    (("pair_32_layers", 60, 32, 48, 24, 2, None, 4, 64), 16),
+    (("pair_1_layer", 70, 1, 96, 96, 4, None, 2, 57), 7),
+    (("pair_long", 1500, 6, 48, 48, 2, None, 1, 43), 64)]
+
+
+@pytest.mark.parametrize("spec,steps", PAIR_CASES, ids=[e[0][0] for e in PAIR_CASES])
+def test_two_chains_to_a_warp(spec, steps):
+    """Compressed rows with more members than three SMs hold with a warp each, an odd one left over, windows of steps that end before
+    the sixteenth, whole or with open layers; then on with a warp to a chain and back."""
+    name, N, L, E, P, D, edp, min_rows, pop = spec
+    w = compressed_window(spec)
+    s = w.spec
+    ref = oracle_front(w, edp, min_rows)
+    ctx = load(w, pop=pop, edp=edp, min_rows=min_rows)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 3)
+    rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 3)
+    check_front(w, ctx, ref)
+    want, stats = check_anneal(w, ctx, ref, edp, pop, 3, steps, t_ratio=0.6, check_members=2, t0=1e-2)
+    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.accepted > 0
+    for sms in (0, 3):
+        rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", sms)
+        want = oracle.anneal(w.lengths, ref["q"], want["final_pop"], ref["R"], s.token_cap, D, n_levels=2, steps=steps, t0=1e-4,
+                             t_ratio=0.5, p_reloc=0.5, p_guide=0.3, seed=s.anneal_seed, edp_of_dp=edp, alpha=s.alpha, beta=s.beta,
+                             n_threads=8)
+        rp.rp_anneal(ctx, n_levels=2, steps_per_level=steps, t0=1e-4, t_ratio=0.5, p_reloc=0.5, p_guide=0.3)
+        assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (2, pop, 3), np.int64) == want["term"]).all()
+        assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == want["final_pop"]).all()
+    rp.rp_destroy(ctx)
