@@ -555,7 +555,7 @@ static int build_population(rp_ctx *c, bool candidates, bool same_rows)
             slab.take(&c->d_inc_slot, 1);
             slab.take(&c->d_undecided, 1);
             slab.take(&c->d_static, (size_t)c->sl.bytes);
-            slab.take(&c->d_one_Esum, (size_t)dm.RG);
+            slab.take(&c->d_one_Esum, (size_t)dm.RG + 3);
             slab.take(&c->d_one_ticket, 1);
             slab.take(&c->d_one_list, rp_eval_list_len(dm, 1));
             slab.take(&c->d_one_off, rp_eval_off_len(dm, 1));

@@ -8,7 +8,7 @@
 //    sums meet through distributed shared memory;
 //  * many layouts (k_eval_group, k_eval_sum, k_eval_score), bound by L2: the samples of a layout are grouped by row-shard once, then
 //    a warp per row-shard sums its rows, sixteen bytes per lane and eight to twelve loads in flight.
-// In the first the CTA that finishes a layout last (atomic ticket) scores it.
+// In the first the cluster that finishes a layout last (atomic ticket) scores it.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -18,6 +18,7 @@
 namespace cg = cooperative_groups;
 
 #define EVAL_THREADS 256
+#define EVAL_SMEM_MAX (220 * 1024)
 
 // What a launch scores and where its results go.
 struct EvalArgs {
@@ -40,7 +41,7 @@ struct EvalArgs {
     i64 *score_final;
     double *f64_final;
     int n;
-    i64 *Esum;                                    // [n][RG] row-shard sums handed to the finishing CTA; zero between launches
+    i64 *Esum;                                    // [n][RG] row-shard sums (few layouts: costs) handed to the finishing CTA; zero between launches
     int *tickets;                                 // [n] arrival counters; zero between launches
     unsigned short *list;                         // [n][N] samples grouped by row-shard (k_eval_group)
     int *off;                                     // [n][RG+1]
@@ -91,7 +92,6 @@ __device__ __forceinline__ EvalFinish eval_finish_views(const RpDims &dm, unsign
 }
 
 // Scores layout `lay` once its row-shard sums are complete.  All threads of one CTA call; cell_of is in place.
-template <bool FEW>
 __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const EvalFinish &f, int tid)
 {
     const RpDims &dm = A.dm;
@@ -123,7 +123,7 @@ __device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const Ev
         if (A.layout_host) for (int i = tid; i < dm.N; i += EVAL_THREADS) A.layout_host[i] = __ldg(A.lay32 + i);
     }
     if (tid < 32) {
-        const bool refused = !FEW && A.bad_dev && __ldcg(A.bad_dev);
+        const bool refused = A.bad_dev && __ldcg(A.bad_dev);
         i64 s0 = 0, s1 = 0, s2 = 0;
         for (int g = lane; g < dm.G; g += 32) { const i64 u = f.U[g]; s1 += u; s0 = u > s0 ? u : s0; }
         for (int rg = lane; rg < dm.RG; rg += 32) { const i64 J = f.Afx[rg] + dm.EC * f.Esum[rg]; s2 = J > s2 ? J : s2; }
@@ -334,11 +334,25 @@ k_eval_score(const EvalArgs A)
     extern __shared__ __align__(16) unsigned char smraw[];
     const EvalFinish f = eval_finish_views(A.dm, smraw);
     eval_load_cells(A, blockIdx.x, f.cell_of, threadIdx.x, EVAL_THREADS);
-    eval_finish<false>(A, blockIdx.x, f, threadIdx.x);
+    eval_finish(A, blockIdx.x, f, threadIdx.x);
+}
+
+__device__ __forceinline__ i64 few_warp_max(i64 v)
+{
+    for (int o = 16; o; o >>= 1) { const i64 w = __shfl_xor_sync(0xffffffffu, v, o); v = w > v ? w : v; }
+    return v;
 }
 
 // grid = (MS, row-shards, layouts), clusters of MS CTAs along x: CTA x of a row-shard takes the samples of
-// range x, then the layers of range x of the summed row.
+// range x, then the layers of range x of the summed row.  The row-shard's cell statistics and cost are worked out by its own
+// cluster beside the sums, so that what is left for the CTA that finishes a layout is a sum over its row-shards (with the statistics of
+// all samples added up there, one CTA took two thirds of the time on heavy's 8192; with the one launch of the metrics behind it a call
+// of rp_diagnostics on heavy 90 -> 47 us).
+static inline size_t eval_few_smem(const RpDims &dm, int MS)
+{
+    const size_t part = (sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2) + 7) & ~(size_t)7;
+    return std::max(part + (size_t)16 * dm.D, (size_t)8 * dm.G);
+}
 template <bool WIDE>            // more than 32 chunks in a layer
 __global__ void __launch_bounds__(EVAL_THREADS)
 k_eval_few(const EvalArgs A)
@@ -350,18 +364,28 @@ k_eval_few(const EvalArgs A)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = EVAL_THREADS / 32;
     int *part = (int *)smraw;                                           // [LP] this CTA's share of the sum
     int *list = part + dm.LP;                                           // [N / MS + 1] its samples
-    __shared__ int n_s, last_s;
-    __shared__ u64 es_s;
+    u64 *Q = (u64 *)(smraw + ((sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2) + 7) & ~(size_t)7));      // [D] statistics of the row's cells on
+    int *T = (int *)(Q + dm.D), *cnt = T + dm.D;                        // this shard, by slot
+    __shared__ int n_s, last_s, wrong_s;
+    __shared__ u64 es_s, es_of[8];
+    __shared__ i64 s0_s, s1_s, s2_s;
     const EvalCells cells = eval_cells(A, lay);
-    if (tid == 0) { n_s = 0; es_s = 0; }
+    char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
+    if (tid == 0) { n_s = 0; es_s = 0; wrong_s = 0; s0_s = 0; s1_s = 0; s2_s = 0; }
+    for (int d = tid; d < dm.D; d += EVAL_THREADS) { Q[d] = 0; T[d] = 0; cnt[d] = 0; }
     __syncthreads();
-    const int row = rg / dm.G, g = rg % dm.G;
+    const int row = rg / dm.G, g = rg % dm.G, first = row * dm.D;
     const int i0 = (int)((long long)dm.N * ms / MS), i1 = (int)((long long)dm.N * (ms + 1) / MS);
 #pragma unroll 8
     for (int i = i0 + tid; i < i1; i += EVAL_THREADS) {
-        const int c = eval_cell(A, cells, i);
-        if (c / dm.D == row && __ldg(A.edp + c % dm.D) == g) list[atomicAdd(&n_s, 1)] = i;
+        const int c = eval_cell(A, cells, i), d = c - first;
+        if ((unsigned)d >= (unsigned)dm.D || __ldg(A.edp + d) != g) continue;
+        const int ti = __ldg(A.t + i);
+        list[atomicAdd(&n_s, 1)] = i;
+        atomicAdd(&T[d], ti); atomicAdd(&cnt[d], 1); atomicAdd(&Q[d], (u64)ti * (u64)ti);
+        if (b) ((unsigned short *)(b + A.bl.off_cell))[i] = (unsigned short)c;
     }
+    if (A.layout_host && rg == 0) for (int i = i0 + tid; i < i1; i += EVAL_THREADS) A.layout_host[i] = __ldg(A.lay32 + i);
     __syncthreads();
     const int cpl = dm.P >> 2, rc = dm.LP >> 2, n = n_s;
     for (int c0 = 32 * warp; c0 < rc; c0 += 32 * nwarps) {
@@ -394,6 +418,7 @@ k_eval_few(const EvalArgs A)
         const bool on = lane < used && c < l1 * cpl;
         int4 a = make_int4(0, 0, 0, 0);
         if (on)
+#pragma unroll 4
             for (int x = 0; x < MS; ++x) {
                 const int4 v = ((const int4 *)cl.map_shared_rank(part, x))[c];
                 a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
@@ -404,20 +429,94 @@ k_eval_few(const EvalArgs A)
     }
     for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
     if (lane == 0 && es) atomicAdd(&es_s, (u64)es);
+    // statistics of all of the cluster's samples, by its first CTA (the others leave theirs as they are)
+    if (ms == 0)
+        for (int d = tid; d < dm.D; d += EVAL_THREADS) {
+            if (__ldg(A.edp + d) != g) continue;
+            int t = T[d], m = cnt[d];
+            u64 q = Q[d];
+#pragma unroll 4
+            for (int x = 1; x < MS; ++x) { t += cl.map_shared_rank(T, x)[d]; m += cl.map_shared_rank(cnt, x)[d]; q += cl.map_shared_rank(Q, x)[d]; }
+            T[d] = t; cnt[d] = m; Q[d] = q;
+            if (m < 1 || t > dm.C) wrong_s = 1;
+            if (b) {
+                ((u64 *)(b + A.bl.off_Q))[first + d] = q;
+                ((int *)(b + A.bl.off_T))[first + d] = t;
+                ((int *)(b + A.bl.off_cnt))[first + d] = m;
+            }
+        }
+    __syncthreads();
+    if (tid == 0) cl.map_shared_rank(es_of, 0)[ms] = es_s;
     cl.sync();                                            // nobody reads another CTA's shared memory from here on
-    if (tid == 0) {
-        if (es_s) atomicAdd((u64 *)(A.Esum + (size_t)lay * dm.RG + rg), es_s);
-        __threadfence();
-        last_s = (atomicAdd(&A.tickets[lay], 1) == (int)(gridDim.x * gridDim.y) - 1);
-        if (last_s) A.tickets[lay] = 0;
+    if (ms) return;
+    if (warp == 0) {
+        i64 Af = 0, E = 0;
+        for (int x = 0; x < MS; ++x) E += (i64)es_of[x];
+        const int d0 = __ldg(A.dp_off + g), d1 = __ldg(A.dp_off + g + 1);
+        for (int s = 0; s < dm.S; ++s) {
+            const i64 ca = dm.ahat[s] * dm.C, cb = dm.bhat[s];
+            i64 v = 0;
+            for (int x = d0 + lane; x < d1; x += 32) { const int d = __ldg(A.dp_list + x); const i64 w = ca * T[d] + cb * (i64)Q[d]; v = w > v ? w : v; }
+            for (int o = 16; o; o >>= 1) { const i64 w = __shfl_xor_sync(0xffffffffu, v, o); v = w > v ? w : v; }
+            Af += v;
+        }
+        if (lane == 0) {
+            const i64 J = Af + dm.EC * E;
+            if (b) {
+                ((i64 *)(b + A.bl.off_Esum))[rg] = E; ((i64 *)(b + A.bl.off_Afx))[rg] = Af; ((i64 *)(b + A.bl.off_Jfx))[rg] = J;
+                if (A.bl.off_wtab >= 0) ((int *)(b + A.bl.off_wtab))[rg] = (A.first + lay) * dm.RG + rg;      // the pool holds the call's layouts as RG slices each
+            }
+            A.Esum[(size_t)lay * dm.RG + rg] = J;
+            __threadfence();
+            // arrivals in the lower half, row-shards with an empty or overfull cell in the upper one
+            const unsigned before = atomicAdd((unsigned *)&A.tickets[lay], 1u | (wrong_s ? 1u << 16 : 0u));
+            last_s = (before & 0xffffu) == (unsigned)dm.RG - 1;
+            if (last_s) { wrong_s |= (before >> 16) ? 1 : 0; A.tickets[lay] = 0; }
+        }
     }
-    if (wout) __threadfence();
     __syncthreads();
     if (!last_s) return;
     __threadfence();
-    const EvalFinish f = eval_finish_views(dm, smraw);
-    eval_load_cells(A, lay, f.cell_of, tid, EVAL_THREADS);
-    eval_finish<true>(A, lay, f, tid);
+    i64 *U = (i64 *)smraw;
+    for (int x = tid; x < dm.G; x += EVAL_THREADS) U[x] = 0;
+    __syncthreads();
+    {
+        i64 *eg = A.Esum + (size_t)lay * dm.RG, top = 0;
+#pragma unroll 4
+        for (int x = tid; x < dm.RG; x += EVAL_THREADS) {
+            const i64 J = __ldcg(eg + x);
+            eg[x] = 0;
+            top = J > top ? J : top;
+            atomicAdd((u64 *)&U[x % dm.G], (u64)J);
+        }
+        top = few_warp_max(top);
+        if (lane == 0) atomicMax(&s2_s, top);
+    }
+    __syncthreads();
+    {
+        i64 sum = 0, top = 0;
+        for (int x = tid; x < dm.G; x += EVAL_THREADS) {
+            const i64 u = U[x];
+            sum += u; top = u > top ? u : top;
+            if (b) ((i64 *)(b + A.bl.off_U))[x] = u;
+        }
+        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        top = few_warp_max(top);
+        if (lane == 0) { atomicMax(&s0_s, top); atomicAdd((u64 *)&s1_s, (u64)sum); }
+    }
+    __syncthreads();
+    if (A.host) {          // coverage is checked by the caller's `bad` flag: every sample sits in one cell by construction
+        if (tid < 8) A.host[tid] = A.counters[tid];
+        if (tid < 3) { A.host[16 + tid] = A.inc_score[tid]; A.host[22 + tid] = A.seed_score[tid]; }
+        if (tid < RP_SW_COUNT) ((int *)(A.host + 56))[tid] = A.status[tid] | (tid == RP_SW_VALIDATE && wrong_s ? 1 : 0);
+    }
+    if (tid < 3) {
+        const i64 sc = tid == 0 ? s0_s : (tid == 1 ? s1_s : s2_s);
+        if (A.score_out) A.score_out[(size_t)lay * 3 + tid] = sc;
+        if (A.score_out2) A.score_out2[(size_t)lay * 3 + tid] = sc;
+        if (A.f64_out) A.f64_out[(size_t)lay * 3 + tid] = (double)sc / (double)dm.SC;
+        if (b) { i64 *S = (i64 *)(b + A.bl.off_S); S[tid] = sc; if (tid == 0) S[3] = rp_energy(s0_s, s1_s, s2_s); }
+    }
     if (!A.score_final && !A.f64_final) return;
     if (tid < 32) __threadfence();
     __syncthreads();
@@ -443,8 +542,6 @@ static size_t eval_smem_bytes(const RpDims &dm)
     return (eval_finish_bytes(dm) + sizeof(int) * (2 * (size_t)dm.RG + 1 + dm.N) + 15) & ~(size_t)15;
 }
 
-#define EVAL_SMEM_MAX (220 * 1024)
-
 // Whether n layouts take the few-layouts form.  It has a cluster per row-shard and layout, which scans the whole assignment: per CTA
 // about 6 ns and a nanosecond for 300 samples, with the rows served less evenly (0.3 ns for 1000 counts).  The other form groups
 // an assignment once, but in one CTA, and streams through a row-shard with one warp: 9 us more for its launches, and the longer
@@ -454,7 +551,7 @@ static size_t eval_smem_bytes(const RpDims &dm)
 // 76 and 44.
 static bool eval_is_few(const RpDims &dm, int n)
 {
-    if ((dm.P & 3) || n >= 65536 || dm.RG >= 65536 || dm.LP > 16384) return false;
+    if ((dm.P & 3) || n >= 65536 || dm.RG >= 65536 || dm.LP > 16384 || eval_few_smem(dm, 8) > EVAL_SMEM_MAX) return false;
     const double N = dm.N, RG = dm.RG;
     if (n == 1) return RG * N <= 5e6;
     return n * (RG * (6.0 + N / 300.0) + 3e-4 * N * dm.LP) <= 9e3 + std::min(150.0 * N / RG, 30e3);
@@ -472,8 +569,8 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
     if (eval_is_few(dm, n)) {
         int MS = 1;
         while (MS < 8 && (long long)n * dm.RG * MS < 148 * 4 && dm.N >= 64 * MS) MS *= 2;
-        const size_t sm = std::max(eval_finish_bytes(dm), sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2));
-        if (sm > EVAL_SMEM_MAX) return RP_ERR_RANGE;
+        while (MS < 8 && eval_few_smem(dm, MS) > EVAL_SMEM_MAX) MS *= 2;
+        const size_t sm = eval_few_smem(dm, MS);
         auto few = eval_vec(dm) ? k_eval_few<false> : k_eval_few<true>;
         if (sm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(few, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
         cudaLaunchConfig_t cfg = {};
@@ -628,7 +725,7 @@ k_setup_population(const SetupArgs A)
     }
     for (int m = tid; m < A.P; m += nt) { A.anc[m] = 0; A.wloc[m] = 0; A.wloc_next[m] = A.P + m; }
     for (int i = tid; i < dm.N; i += nt) A.inc_layout[i] = A.seed_layout[i];
-    for (int x = tid; x < dm.RG; x += nt) A.one_Esum[x] = 0;
+    for (int x = tid; x < dm.RG + 3; x += nt) A.one_Esum[x] = 0;      // (three sums of the diagnostics behind them)
     for (int x = tid; x <= A.P; x += nt) A.sync[x] = 0;
     if (A.wcount) for (size_t x = tid; x < 2 * (size_t)A.P * dm.RG; x += nt) A.wcount[x] = 0;
     if (tid < 7) A.counters[tid] = 0;                      // (the eighth is the window's token total)
@@ -657,19 +754,20 @@ int rp_launch_setup_population(rp_ctx *c)
 // Load-balance diagnostics (evaluation section of the paper): coefficient of variation of the
 // aggregate rank loads, EP peak sum, tail peak, EP balance efficiency, attention and joint proxies.
 // ---------------------------------------------------------------------------------------------
-struct RpDiagDev { double cv_identity, cv_placed; i64 s_ep, t_ep, n_ep; i64 afx_sum, s0; int tickets, pad; };
+struct RpDiagDev { double cv_identity, cv_placed; i64 s_ep, t_ep, n_ep; i64 afx_sum, s0; };
 
-// One warp per layer: the lanes fetch the rank loads, one lane adds them up with plain sequential IEEE sums (no fused
+// One launch: the last CTA works out the coefficients of variation, the others the peaks (the two have nothing to do with one
+// another; as launches of their own, and with 64-bit shuffles for the peaks, they took 27 us behind the scoring).
+#define DIAG_THREADS 512
+#define DIAG_PEAK_CTAS 148
+// Coefficients: one warp per layer; the lanes fetch the rank loads, one lane adds them up with plain sequential IEEE sums (no fused
 // multiply-add); then thread 0 averages the layers in order.
-#define DIAG_THREADS 1024
-__global__ void __launch_bounds__(DIAG_THREADS)
-k_diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, RpDims dm, RpDiagDev *__restrict__ sums, RpDiagDev *__restrict__ out)
+__device__ __forceinline__ void diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, const RpDims &dm, int warps,
+                                        double *cvs, RpDiagDev *__restrict__ out)
 {
-    extern __shared__ double cvs[];          // [2][L], then one row of rank loads per warp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) { sums->s_ep = 0; sums->t_ep = 0; sums->n_ep = 0; sums->tickets = 0; }      // for the kernel behind this one
     double *G = cvs + 2 * dm.L + (size_t)warp * dm.P;
-    for (int x = warp; x < 2 * dm.L; x += (int)blockDim.x / 32) {
+    for (int x = warp; x < 2 * dm.L && warp < warps; x += warps) {
         const int l = x >> 1, which = x & 1;
         for (int p = lane; p < dm.P; p += 32) {
             i64 g = 0;
@@ -703,35 +801,48 @@ k_diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, RpDim
     }
 }
 
-// One warp per (row, layer): lanes over ranks, loop over shards; integer results by atomics.
-__global__ void k_diag_peaks(const int *__restrict__ W, const char *__restrict__ blob, RpBlob bl, RpDims dm,
-                             RpDiagDev *__restrict__ sums, RpDiagDev *__restrict__ out)
+// Peaks: one warp per (row, layer): lanes over ranks, loop over shards; integer results by atomics on `sums` (s_ep, n_ep, t_ep; zero
+// between launches, as the ticket is).
+__global__ void __launch_bounds__(DIAG_THREADS)
+k_diagnose(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, int cv_warps, const int *__restrict__ W, const char *__restrict__ blob,
+           RpBlob bl, RpDims dm, i64 *__restrict__ sums, int *__restrict__ ticket, RpDiagDev *__restrict__ out)
 {
+    extern __shared__ double cvs[];          // [2][L], then one row of rank loads per warp
+    if (blockIdx.x == DIAG_PEAK_CTAS) { diag_cv(Lagg, rank_load, dm, cv_warps, cvs, out); return; }
     const int lane = threadIdx.x & 31;
-    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    const int wid = (int)(threadIdx.x >> 5) * DIAG_PEAK_CTAS + (int)blockIdx.x, nw = DIAG_PEAK_CTAS * DIAG_THREADS / 32;
     i64 s_ep = 0, n_ep = 0, t_ep = 0;
     for (int rl = wid; rl < dm.R * dm.L; rl += nw) {
         const int r = rl / dm.L, l = rl % dm.L;
-        i64 peak = 0, best_sum = 0;
-#pragma unroll 4
-        for (int g = 0; g < dm.G; ++g) {
-            const int *w = W + (((size_t)r * dm.G + g) * dm.L + l) * dm.P;
-            i64 sum = 0, mx = 0;
-            for (int p = lane; p < dm.P; p += 32) { const i64 v = w[p]; sum += v; mx = v > mx ? v : mx; }
-            for (int o = 16; o; o >>= 1) {
-                sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                const i64 x = __shfl_xor_sync(0xffffffffu, mx, o);
-                mx = x > mx ? x : mx;
+        const int *w0 = W + ((size_t)r * dm.G * dm.L + l) * dm.P;
+        int peak = 0;
+        i64 best_sum = 0;
+        for (int g0 = 0; g0 < dm.G; g0 += 4) {
+            int mx[4] = { 0, 0, 0, 0 };
+            i64 sum[4] = { 0, 0, 0, 0 };
+            for (int p = lane; p < dm.P; p += 32)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int v = g0 + u < dm.G ? __ldg(w0 + (size_t)(g0 + u) * dm.LP + p) : 0;
+                    sum[u] += v; mx[u] = max(mx[u], v);
+                }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                // (32 lanes' sums of 21 bits at a time)
+                const u64 lo = __reduce_add_sync(0xffffffffu, (u32)sum[u] & 0x1fffffu), mid = __reduce_add_sync(0xffffffffu, (u32)(sum[u] >> 21) & 0x1fffffu),
+                          hi = __reduce_add_sync(0xffffffffu, (u32)(sum[u] >> 42));
+                const i64 all = (i64)(lo + (mid << 21) + (hi << 42));
+                peak = max(peak, (int)__reduce_max_sync(0xffffffffu, mx[u]));
+                best_sum = all > best_sum ? all : best_sum;
             }
-            peak = mx > peak ? mx : peak;
-            best_sum = sum > best_sum ? sum : best_sum;
         }
         s_ep += peak; n_ep += best_sum; t_ep = peak > t_ep ? peak : t_ep;
     }
     if (lane == 0) {
-        if (s_ep) atomicAdd((u64 *)&sums->s_ep, (u64)s_ep);
-        if (n_ep) atomicAdd((u64 *)&sums->n_ep, (u64)n_ep);
-        if (t_ep) atomicMax((i64 *)&sums->t_ep, t_ep);
+        if (s_ep) atomicAdd((u64 *)&sums[0], (u64)s_ep);
+        if (n_ep) atomicAdd((u64 *)&sums[1], (u64)n_ep);
+        if (t_ep) atomicMax(&sums[2], t_ep);
+        __threadfence();
     }
     if (blockIdx.x == 0 && threadIdx.x < 32) {      // attention total and joint from the layout's blob
         const i64 *Afx = (const i64 *)(blob + bl.off_Afx);
@@ -740,11 +851,11 @@ __global__ void k_diag_peaks(const int *__restrict__ W, const char *__restrict__
         for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
         if (lane == 0) { out->afx_sum = a; out->s0 = ((const i64 *)(blob + bl.off_S))[0]; }
     }
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&sums->tickets, 1) == (int)gridDim.x - 1) {
+    if (threadIdx.x == 0 && atomicAdd(ticket, 1) == DIAG_PEAK_CTAS - 1) {
         __threadfence();
-        out->s_ep = __ldcg(&sums->s_ep); out->n_ep = __ldcg(&sums->n_ep); out->t_ep = __ldcg(&sums->t_ep);
+        out->s_ep = __ldcg(sums); out->n_ep = __ldcg(sums + 1); out->t_ep = __ldcg(sums + 2);
+        sums[0] = 0; sums[1] = 0; sums[2] = 0; *ticket = 0;
     }
 }
 
@@ -759,12 +870,11 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
     // scratch: a copy of a layout that is not in this GPU's memory, W, one blob
     const size_t wn = (size_t)dm.RG * dm.LP;
     const size_t off_W = ((size_t)dm.N * 4 + 255) & ~(size_t)255, off_blob = off_W + ((wn * 4 + 255) & ~(size_t)255);
-    const size_t off_res = off_blob + (((size_t)c->bl.bytes + 255) & ~(size_t)255);
-    // (a row of P rank loads per warp: beyond 900 ranks fewer warps than the kernel is made for)
+    // (a row of P rank loads per warp: beyond 1700 ranks fewer warps than the kernel is made for)
     const int cv_warps = (int)std::min<size_t>(DIAG_THREADS / 32, (EVAL_SMEM_MAX / sizeof(double) - 2 * (size_t)dm.L) / dm.P);
     const size_t cv_smem = sizeof(double) * (2 * (size_t)dm.L + cv_warps * (size_t)dm.P);
     char *buf = nullptr;
-    RP_CUDA(cudaMallocFromPoolAsync((void **)&buf, off_res + 256, pool, c->stream));
+    RP_CUDA(cudaMallocFromPoolAsync((void **)&buf, off_blob + (size_t)c->bl.bytes + 256, pool, c->stream));
     int st = RP_OK;
     cudaError_t e = cudaSuccess;
     do {
@@ -782,14 +892,13 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
         st = eval_launch(c, A, 1);
         if (st != RP_OK) break;
         // the record goes to the pinned block: its sums by the last CTA of the peaks, the rest by the first
-        RpDiagDev *res = (RpDiagDev *)(buf + off_res), *host = (RpDiagDev *)(c->h_pin + 32);
+        RpDiagDev *host = (RpDiagDev *)(c->h_pin + 32);
         if (cv_smem > 32 * 1024) {
-            e = cudaFuncSetAttribute(k_diag_cv, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX);
+            e = cudaFuncSetAttribute(k_diagnose, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX);
             if (e != cudaSuccess) break;
         }
-        k_diag_cv<<<1, 32 * cv_warps, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, dm, res, host);
-        ++g_rp_launches;
-        k_diag_peaks<<<148, 256, 0, c->stream>>>((const int *)(buf + off_W), buf + off_blob, c->bl, dm, res, host);
+        k_diagnose<<<DIAG_PEAK_CTAS + 1, DIAG_THREADS, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, cv_warps, (const int *)(buf + off_W),
+                                                                            buf + off_blob, c->bl, dm, c->d_one_Esum + dm.RG, c->d_one_ticket, host);
         ++g_rp_launches;
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
