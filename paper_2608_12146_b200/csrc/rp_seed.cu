@@ -9,7 +9,7 @@
 // A trial is a chain of N steps, so its latency is what counts.  The warp keeps the keys of the cells sorted: the cells a
 // sample fits in are the keys from (length, 0, 0) on, the r-th of them is taken out, and its smaller new key goes in front of
 // those it passes, which move up by one.  Up to 512 cells a lane holds E consecutive keys in registers (a position is one
-// warp-wide sum of compares, the move one shuffle: 600 cycles a sample at 240 cells); beyond, the keys lie in shared memory
+// warp-wide sum of compares, the move one shuffle and a compare a key: 520 cycles a sample at 240 cells, 600 with a second sum); beyond, the keys lie in shared memory
 // (two searches of two ballots: 1100 cycles).  Ranking by r + 1 passes over all cells took 4400.  What does not depend on the
 // fit runs 32 samples at a time: a lane draws the random words of its sample, then the shuffle emits the 32 samples.
 #include "rp_common.cuh"
@@ -85,7 +85,7 @@ k_seed_trials(const int *__restrict__ t, const int *__restrict__ order, const in
                 } else {
                     int n = 0;
 #pragma unroll
-                    for (int e = 0; e < E; ++e) n += v[e] < ts;
+                    for (int e = 0; e < E; ++e) n += (u32)(v[e] >> 32) < (u32)(ts >> 32);      // (the lower word of ts is zero)
                     const int p0 = __reduce_add_sync(0xffffffffu, n), nc = dm.K - p0;        // feasible cells
                     if (nc == 0) { good = false; break; }
                     from = p0 + rp_pick(x, nc < width ? nc : width);
@@ -98,17 +98,17 @@ k_seed_trials(const int *__restrict__ t, const int *__restrict__ order, const in
                         for (int e = 0; e < half; ++e) m[e] = (from & half) ? m[e + half] : m[e];
                     key = __shfl_sync(0xffffffffu, m[0], from / (E ? E : 1)) - ts + (1ull << 20);
                 }
-                int n = 0;
-#pragma unroll
-                for (int e = 0; e < E; ++e) n += v[e] < key;
-                const int to = __reduce_add_sync(0xffffffffu, n) - lane * E, top = from - lane * E;
-                // keys to .. from-1 move up by one
+                // Keys that are not below the new one move up by one as far as place `from`; where a key moves from one that is
+                // below it, the new key comes in.
+                const int top = from - lane * E;
                 const u64 below = __shfl_up_sync(0xffffffffu, v[E ? E - 1 : 0], 1);
+                bool lt[E ? E + 1 : 1];                      // key of the place before; of place e at e + 1
+                lt[0] = lane == 0 || below < key;
 #pragma unroll
-                for (int e = E - 1; e >= 0; --e) {
-                    if (e > to && e <= top) v[e] = e ? v[e ? e - 1 : 0] : below;
-                    if (e == to) v[e] = key;
-                }
+                for (int e = 0; e < E; ++e) lt[e + 1] = v[e] < key;
+#pragma unroll
+                for (int e = E - 1; e >= 0; --e)
+                    if (!lt[e + 1] && e <= top) v[e] = lt[e] ? key : (e ? v[e ? e - 1 : 0] : below);
             } else {
                 const u64 top = keys[last];
                 if (h0 + u < dm.K) {
