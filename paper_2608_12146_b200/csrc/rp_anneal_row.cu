@@ -75,7 +75,7 @@ k_make_rows(RpDims dm, const int *__restrict__ t, const int *__restrict__ q, con
     }
 }
 
-// Member m = blockIdx.x, row-shard rg = blockIdx.y: the slack (sum of the busiest loads less the samples' f), and (Wr != null) the row-shard's
+// Member m = blockIdx.x, row-shard rg = blockIdx.y: the slack (sum of the busiest loads less the samples' f), and the row-shard's
 // slice in row form, in the place its table names (windows without a table: cell m of the pool).
 // Compressed rows also count the row-shards with a layer whose three columns do not decide the maximum; `loose`: counts those
 // whose busiest loads exceed their samples' f by more than a sixteenth.
@@ -94,7 +94,7 @@ k_member_rows(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *
     __syncthreads();
     i64 f = 0;
     for (int i = tid; i < dm.N; i += 256)
-        if (__ldg(rg_of + cells[i]) == rg) { f += __ldg(&tf[i].y); if (Wr) list[atomicAdd(&n_s, 1)] = i; }
+        if (__ldg(rg_of + cells[i]) == rg) { f += __ldg(&tf[i].y); list[atomicAdd(&n_s, 1)] = i; }
     if (f) atomicAdd(&f_s, (u64)f);
     __syncthreads();
     if (tid == 0) {
@@ -102,7 +102,6 @@ k_member_rows(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *
         Fo[(size_t)m * dm.RG + rg] = slack;
         if (loose && slack * 16 > es) atomicAdd(undecided, 1);
     }
-    if (!Wr) return;
     const int n = n_s;
     const size_t slice = bl.off_wtab >= 0 ? (size_t)((const int *)(blob + bl.off_wtab))[rg] : (size_t)wloc[m] * dm.RG + rg;
     int4 *out = (int4 *)(Wr + slice * rlp);
@@ -115,6 +114,31 @@ k_member_rows(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *
     }
     __syncthreads();
     if (comp && tid == 0 && bad_s) atomicAdd(undecided, 1);
+}
+
+// The slacks alone, one CTA per member: a scan of the assignment with 64-bit additions in shared memory (a CTA per row-shard scans it
+// once for each: 256 members of 2048 samples in 240 row-shards took 134 us, a plan with candidates 3.24 ms).
+__global__ void __launch_bounds__(256)
+k_member_slack(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *__restrict__ static_blk, RpStatic sl, const int2 *__restrict__ tf,
+               i64 *__restrict__ Fo, int *__restrict__ undecided, int loose)
+{
+    extern __shared__ u64 sum[];                        // [RG]
+    const int m = blockIdx.x, tid = threadIdx.x;
+    const char *blob = blobs + (size_t)m * bl.bytes;
+    const unsigned short *cells = (const unsigned short *)(blob + bl.off_cell);
+    const unsigned short *rg_of = (const unsigned short *)(static_blk + sl.off_rg);
+    for (int rg = tid; rg < dm.RG; rg += 256) sum[rg] = 0;
+    __syncthreads();
+#pragma unroll 8
+    for (int i = tid; i < dm.N; i += 256) atomicAdd(&sum[__ldg(rg_of + cells[i])], (u64)(i64)__ldg(&tf[i].y));
+    __syncthreads();
+    int n = 0;
+    for (int rg = tid; rg < dm.RG; rg += 256) {
+        const i64 es = ((const i64 *)(blob + bl.off_Esum))[rg], slack = es - (i64)sum[rg];
+        Fo[(size_t)m * dm.RG + rg] = slack;
+        n += loose && slack * 16 > es;
+    }
+    if (n) atomicAdd(undecided, n);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -265,9 +289,13 @@ int rp_launch_member_rows(rp_ctx *c, int n)
     if (smem > 200 * 1024) return RP_ERR_RANGE;
     if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_member_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024)));
     RP_CUDA(cudaMemsetAsync(c->d_undecided, 0, sizeof(int), c->stream));
-    k_member_rows<<<dim3(n, dm.RG), 256, smem, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_static, c->sl, (const int2 *)c->d_tf, X.qr,
-                                                            X.rlp, X.comp, c->d_rowF + (size_t)c->cur * c->Ppop * dm.RG,
-                                                            sep ? c->d_Wr : nullptr, c->d_wloc, c->d_undecided, c->row_check);
+    i64 *Fo = c->d_rowF + (size_t)c->cur * c->Ppop * dm.RG;
+    if (!sep)                       // (a chain keeps 40 bytes of a row-shard in shared memory: no more than 5632)
+        k_member_slack<<<n, 256, sizeof(u64) * (size_t)dm.RG, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_static, c->sl, (const int2 *)c->d_tf, Fo,
+                                                                          c->d_undecided, c->row_check);
+    else
+        k_member_rows<<<dim3(n, dm.RG), 256, smem, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_static, c->sl, (const int2 *)c->d_tf, X.qr, X.rlp,
+                                                                X.comp, Fo, c->d_Wr, c->d_wloc, c->d_undecided, c->row_check);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());
     c->row_counted = n;
