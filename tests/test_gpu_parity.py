@@ -1727,3 +1727,21 @@ def test_two_chains_to_a_warp(spec, steps):
         assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (2, pop, 3), np.int64) == want["term"]).all()
         assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == want["final_pop"]).all()
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("pop", [2, 303, 304])
+def test_selection_with_its_distances_on_chip_and_not(pop):
+    """The greedy order where all distances of the candidates just fit on chip, and with one candidate more."""
+    w = make_window(custom_spec("greedy", 60, 5, 16, 2, 4096, 3, 4, pop, 0, data_seed=3))
+    s = w.spec
+    ref = oracle_front(w, None, 3)
+    ctx = load(w, pop=pop, min_rows=3)
+    check_front(w, ctx, ref)
+    lays, ok = oracle.seed_trials(w.lengths, ref["seed"], ref["R"], s.token_cap, 3, pop, 5, s.anneal_seed)
+    assert rp.rp_seed_population(ctx, 5) == int(ok.sum())
+    sc = oracle.eval_layouts(w.lengths, ref["q"], lays, ref["R"], s.token_cap, 3, None, s.alpha, s.beta)["score"]
+    want = oracle.select_population(w.lengths, ref["q"], lays, sc, ref["R"], s.token_cap, 3, s.top_k, 4, 1 << 16, s.anneal_seed, None,
+                                    want_dist=True)
+    nd, order = rp.rp_select_population(ctx, 4, 1 << 16)
+    assert nd == want["n_distinct"] and (order == want["order"]).all()
+    rp.rp_destroy(ctx)
