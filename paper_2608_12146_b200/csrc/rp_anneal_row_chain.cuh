@@ -908,9 +908,65 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
             if (warp == 0) row_barrier_warp(A, P, eL, bestL, last, lv.cq, lv.resample_x, m0, m1, inc_s, &win_s, le_anc, lane);
             __syncthreads();
             if (win_s >= 0) inc_slot = win_s;
+        } else if (P <= NT) {
+            // A member a thread: energies meet once, warps' weights once, and an ancestor is a count over the threads (five more
+            // meetings of the CTA and a search of eight dependent steps before: medium 810 us, now 789; two shards 1188 and 1175).
+            const u64 r = tid < P ? __ldcg(eL + tid) : ~0ull >> 1;
+            i64 e[1] = { (i64)(r & ~(1ull << 63)) };
+            i64 b0 = 0, b1 = 0, b2 = 0;
+            int bj = 0x7fffffff;
+            if (r >> 63) {                               // its trajectory best beats the incumbent
+                b0 = __ldcg(bestL + 3 * tid); b1 = __ldcg(bestL + 3 * tid + 1); b2 = __ldcg(bestL + 3 * tid + 2);
+                bj = tid;
+            }
+            const u32 hi = (u32)((u64)e[0] >> 32), mh = __reduce_min_sync(0xffffffffu, hi), ml = __reduce_min_sync(0xffffffffu, hi == mh ? (u32)e[0] : 0xffffffffu);
+            if (lane == 0) { rmin[warp] = (i64)(((u64)mh << 32) | ml); rj[warp] = 0x7fffffff; }
+            if (__any_sync(0xffffffffu, bj != 0x7fffffff)) {
+                const int at = le_lexmin_lane(b0, b1, b2, bj);
+                __syncwarp();
+                if (lane == at) { r0[warp] = b0; r1s[warp] = b1; r2s[warp] = b2; rj[warp] = bj; }
+            }
+            if (tid == 0) win_s = -1;
+            __syncthreads();
+            i64 emin = rmin[0];
+#pragma unroll
+            for (int w = 1; w < NT / 32; ++w) emin = rmin[w] < emin ? rmin[w] : emin;
+            if (warp == NT / 32 - 1) {                   // (the last warp: others may have fewer members to weigh, none has more)
+                const int j0 = lane < NT / 32 ? rj[lane] : 0x7fffffff;
+                if (__any_sync(0xffffffffu, j0 != 0x7fffffff)) {
+                    const bool has = j0 != 0x7fffffff;
+                    const i64 c0 = has ? r0[lane] : 0, c1 = has ? r1s[lane] : 0, c2 = has ? r2s[lane] : 0;
+                    const int at = le_lexmin_lane(c0, c1, c2, j0);
+                    // (all of them beat the incumbent)
+                    if (lane == at) { inc_s[0] = c0; inc_s[1] = c1; inc_s[2] = c2; win_s = j0; }
+                }
+            }
+            if (last) __syncthreads();
+            else {
+                const u64 M = (u64)(emin > dm.SC ? emin : dm.SC);
+                u64 w[1] = { 0 };
+                if (tid < P) le_weights<1>(e, emin, M, lv.cq, w);
+                u64 F = w[0];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) { const u64 x = __shfl_up_sync(0xffffffffu, F, o); if (lane >= o) F += x; }
+                if (lane == 31) rsum[warp] = F;
+                __syncthreads();
+                u64 Ftot = 0;
+#pragma unroll
+                for (int x = 0; x < NT / 32; ++x) { const u64 y = rsum[x]; if (x < warp) F += y; Ftot += y; }
+                const u64 u0 = (u64)(((unsigned __int128)lv.resample_x * Ftot) >> 32);
+                const unsigned __int128 PF = (unsigned __int128)P * F;
+                for (int m = m0; m < m1; ++m) {
+                    // slots with P * F <= at
+                    const int n = __syncthreads_count(tid < P && PF <= (unsigned __int128)u0 + (unsigned __int128)m * Ftot);
+                    if (tid == 0) le_anc[m] = n;
+                }
+                __syncthreads();
+            }
+            if (win_s >= 0) inc_slot = win_s;
         } else {
         // incumbent: the lowest slot among the lexicographically best trajectory-best scores, if it beats it
-        i64 b0 = inc_s[0], b1 = inc_s[1], b2 = inc_s[2], emin = 0x7fffffffffffffffll, e_mine = emin;
+        i64 b0 = inc_s[0], b1 = inc_s[1], b2 = inc_s[2], emin = 0x7fffffffffffffffll;
         int bj = 0x7fffffff;
         for (int m = tid; m < P; m += NT) {
             const u64 r = __ldcg(eL + m);
@@ -920,7 +976,6 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                 if (rp_lex_less(s0, s1, s2, b0, b1, b2)) { b0 = s0; b1 = s1; b2 = s2; bj = m; }
             }
             emin = e < emin ? e : emin;
-            e_mine = e;
         }
         {
             const u32 hi = (u32)((u64)emin >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
@@ -954,8 +1009,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
         if (!last) {
             const u64 M = (u64)(emin > dm.SC ? emin : dm.SC);
             auto en_of = [&](int m) { return (i64)(__ldcg(eL + m) & ~(1ull << 63)); };
-            if (P <= NT) le_prefix_weights_of<1>(P, [&](int) { return e_mine; }, lv.cq, tid, NT, emin, M, le_F, rsum, &carry_s);
-            else if (P <= 2 * NT) le_prefix_weights_of<2>(P, en_of, lv.cq, tid, NT, emin, M, le_F, rsum, &carry_s);
+            if (P <= 2 * NT) le_prefix_weights_of<2>(P, en_of, lv.cq, tid, NT, emin, M, le_F, rsum, &carry_s);
             else le_prefix_weights_of<4>(P, en_of, lv.cq, tid, NT, emin, M, le_F, rsum, &carry_s);
             const u64 Ftot = le_F[P - 1];
             const u64 u0 = (u64)(((unsigned __int128)lv.resample_x * Ftot) >> 32);
