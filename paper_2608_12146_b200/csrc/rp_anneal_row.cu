@@ -25,13 +25,12 @@
 //    does, the layer's loads are added up from the samples of the row-shard.  Used when the seed's
 //    row-shards nearly all satisfy it (checked on the device, see k_member_rows): 16 bytes per layer
 //    instead of 4*P: an eighth of the traffic at 32 ranks.
-//  * No staging area, so 12 to 16 chains per SM instead of 5 to 10.
-// What bounds it now: with 14 to 16 chains per SM (heavy) the instructions of a round, about 4900 cycles with four
-// warps per scheduler; with 7 (large) their latency, about 3900 cycles; launched once for all levels (medium)
-// about 2700 cycles a round and 20 us a level for the slowest chain, the barrier and the states.  A level's time before (the
-// warp-per-chain kernel; medium: warp per candidate) and now: heavy 15.0 -> 3.9 ms, wide 1.2 -> 0.41 ms,
-// large 0.21 -> 0.13 ms, medium 50 -> 36 us (plans: 301 -> 78, 24.0 -> 8.1 to 10.8 over windows of the kind, 4.8 -> 2.8,
-// 1.12 -> 0.87 ms).
+//  * Two chains to a warp (sixteen lanes each, see row_pairs) where there are more members than a warp each keeps resident.
+//  * No staging area, so 12 to 14 warps per SM instead of 5 to 10.
+// What bounds it now: the latency of a round, about 2200 cycles alone on an SM (medium), 3300 with 7 warps (large), 3800 with 11 (wide)
+// and 5900 for two chains with 14 (heavy), where the warps' instructions share the issue slots; launched once for all levels the
+// slowest chain of a level takes twice the mean, three quarters of the level's time.  A level's time with the warp-per-chain kernel
+// (medium: warp per candidate) and now: heavy 15.0 -> 2.7 ms, wide 1.2 -> 0.40 ms, large 0.21 -> 0.10 ms, medium 50 -> 29 us.
 // Step for step this is the sequential chain: proposals are evaluated against the current state,
 // feasible ones are decided in step order, and the speculation is redone after an acceptance.
 //

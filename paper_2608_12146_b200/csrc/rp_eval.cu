@@ -372,14 +372,15 @@ k_eval_few(const EvalArgs A)
     const EvalCells cells = eval_cells(A, lay);
     char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
     if (tid == 0) { n_s = 0; es_s = 0; wrong_s = 0; s0_s = 0; s1_s = 0; s2_s = 0; }
-    for (int d = tid; d < dm.D; d += EVAL_THREADS) { Q[d] = 0; T[d] = 0; cnt[d] = 0; }
-    __syncthreads();
     const int row = rg / dm.G, g = rg % dm.G, first = row * dm.D;
+    // (a slot of another shard has a negative count: which slots are the row-shard's is looked up in global memory only here)
+    for (int d = tid; d < dm.D; d += EVAL_THREADS) { Q[d] = 0; T[d] = 0; cnt[d] = __ldg(A.edp + d) == g ? 0 : (int)0x80000000; }
+    __syncthreads();
     const int i0 = (int)((long long)dm.N * ms / MS), i1 = (int)((long long)dm.N * (ms + 1) / MS);
 #pragma unroll 8
     for (int i = i0 + tid; i < i1; i += EVAL_THREADS) {
         const int c = eval_cell(A, cells, i), d = c - first;
-        if ((unsigned)d >= (unsigned)dm.D || __ldg(A.edp + d) != g) continue;
+        if ((unsigned)d >= (unsigned)dm.D || cnt[d] < 0) continue;
         const int ti = __ldg(A.t + i);
         list[atomicAdd(&n_s, 1)] = i;
         atomicAdd(&T[d], ti); atomicAdd(&cnt[d], 1); atomicAdd(&Q[d], (u64)ti * (u64)ti);
@@ -432,8 +433,8 @@ k_eval_few(const EvalArgs A)
     // statistics of all of the cluster's samples, by its first CTA (the others leave theirs as they are)
     if (ms == 0)
         for (int d = tid; d < dm.D; d += EVAL_THREADS) {
-            if (__ldg(A.edp + d) != g) continue;
             int t = T[d], m = cnt[d];
+            if (m < 0) continue;
             u64 q = Q[d];
 #pragma unroll 4
             for (int x = 1; x < MS; ++x) { t += cl.map_shared_rank(T, x)[d]; m += cl.map_shared_rank(cnt, x)[d]; q += cl.map_shared_rank(Q, x)[d]; }
@@ -452,11 +453,10 @@ k_eval_few(const EvalArgs A)
     if (warp == 0) {
         i64 Af = 0, E = 0;
         for (int x = 0; x < MS; ++x) E += (i64)es_of[x];
-        const int d0 = __ldg(A.dp_off + g), d1 = __ldg(A.dp_off + g + 1);
         for (int s = 0; s < dm.S; ++s) {
             const i64 ca = dm.ahat[s] * dm.C, cb = dm.bhat[s];
             i64 v = 0;
-            for (int x = d0 + lane; x < d1; x += 32) { const int d = __ldg(A.dp_list + x); const i64 w = ca * T[d] + cb * (i64)Q[d]; v = w > v ? w : v; }
+            for (int d = lane; d < dm.D; d += 32) { const i64 w = cnt[d] < 0 ? 0 : ca * T[d] + cb * (i64)Q[d]; v = w > v ? w : v; }
             for (int o = 16; o; o >>= 1) { const i64 w = __shfl_xor_sync(0xffffffffu, v, o); v = w > v ? w : v; }
             Af += v;
         }
