@@ -337,6 +337,7 @@ static bool row_pairs(const rp_ctx *c, const RowArgs &X0)
     chain_layout(c->dm, c->bl, c->sl, X, false, 1, c->Ppop, 0);
     const int one = std::min(14, room / (X.smem_bytes + 1024));
     chain_layout(c->dm, c->bl, c->sl, X, false, 2, c->Ppop, 0);
+    if (X.smem_bytes > ROW_SMEM_MAX) return false;         // (what a launch may ask for is a little less than an SM has)
     const int two = 2 * std::min(14, room / (X.smem_bytes + 1024));
     return c->Ppop > one * rp_sms(c) && 2 * two >= 3 * one;
 }

@@ -1729,6 +1729,22 @@ def test_two_chains_to_a_warp(spec, steps):
     rp.rp_destroy(ctx)
 
 
+@pytest.mark.parametrize("D,R", [(32, 59), (16, 118), (8, 237)])
+def test_two_chains_that_take_more_than_half_an_sm_each(D, R):
+    """One chain to a warp where the shared memory of two lies between what a launch may ask for (220 KB) and what an SM has (227):
+    112 to 116 KB a chain and one resident, so that two to a warp would be half as many again."""
+    spec = ("pair_smem", D * R + 12, 2, 40, 20, D, None, R, 5)
+    w = compressed_window(spec)
+    ref = oracle_front(w, None, R)
+    ctx = load(w, pop=5, min_rows=R)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 3)
+    rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 3)
+    check_front(w, ctx, ref)
+    _, stats = check_anneal(w, ctx, ref, None, 5, 3, 40, t_ratio=0.6, check_members=2, t0=1e-2)
+    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.accepted > 0
+    rp.rp_destroy(ctx)
+
+
 @pytest.mark.parametrize("pop", [2, 303, 304])
 def test_selection_with_its_distances_on_chip_and_not(pop):
     """The greedy order where all distances of the candidates just fit on chip, and with one candidate more."""
