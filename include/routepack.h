@@ -350,6 +350,10 @@ int rp_debug_l2_read_rate(int64_t bytes, int32_t reps, double *gb_per_s);
  * chain (k_anneal_warp), 3 = one layer per lane (k_anneal_row; windows whose rows it would compress decide
  * between 2 and 3, some windows of few layers between 0 and 3, in the first rp_anneal call that is long enough). */
 int rp_debug_chain_kernel(rp_ctx *ctx, int32_t *which);
+/* Form of the one-layer-per-lane kernel that the last rp_anneal call ran (valid after rp_pack_rows; inspection only): 0 = none
+ * (another kernel, or no call yet), 1 = one launch for all levels; one launch per level: 2 = whole layers to a lane, 3 = a row's
+ * chunks dealt out to the lanes, 4 = compressed rows, 5 = compressed rows, two chains to a warp. */
+int rp_debug_chain_form(rp_ctx *ctx, int32_t *form);
 /* Number of kernels this library has launched in this process so far. */
 int64_t rp_debug_launch_count(void);
 

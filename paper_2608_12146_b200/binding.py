@@ -26,7 +26,7 @@ EXPORTS = ("rp_window_load", "rp_place_experts", "rp_pack_rows", "rp_seed_popula
            "rp_best", "rp_destroy", "rp_release_cached_memory", "rp_strerror", "rp_last_cuda_error", "rp_debug_dump",
            "rp_debug_set_trace", "rp_debug_set_knob", "rp_debug_set_stage_timing", "rp_debug_stage_times",
            "rp_debug_nl2", "rp_debug_exp2neg", "rp_debug_philox", "rp_debug_launch_count", "rp_debug_l2_read_rate",
-           "rp_debug_chain_kernel")
+           "rp_debug_chain_kernel", "rp_debug_chain_form")
 
 
 class RpError(RuntimeError):
@@ -102,6 +102,7 @@ def lib():
         L.rp_debug_launch_count.restype = C.c_int64
         L.rp_debug_l2_read_rate.argtypes = [C.c_int64, C.c_int32, C.POINTER(C.c_double)]
         L.rp_debug_chain_kernel.argtypes = [C.c_void_p, C.POINTER(C.c_int32)]
+        L.rp_debug_chain_form.argtypes = [C.c_void_p, C.POINTER(C.c_int32)]
         _lib = L
     return _lib
 
@@ -347,6 +348,16 @@ def rp_debug_chain_kernel(ctx: Context) -> str:
     out = C.c_int32(-1)
     _check(lib().rp_debug_chain_kernel(ctx.handle, C.byref(out)), "rp_debug_chain_kernel")
     return CHAIN_KERNELS[out.value]
+
+
+CHAIN_FORMS = ("none", "all levels", "whole layers", "dealt out", "compressed", "two to a warp")
+
+
+def rp_debug_chain_form(ctx: Context) -> str:
+    """Form of the one-layer-per-lane kernel that the last rp_anneal call ran."""
+    out = C.c_int32(-1)
+    _check(lib().rp_debug_chain_form(ctx.handle, C.byref(out)), "rp_debug_chain_form")
+    return CHAIN_FORMS[out.value]
 
 
 def rp_debug_launch_count() -> int:

@@ -320,26 +320,33 @@ int rp_launch_anneal_row_all(rp_ctx *c, const AnnealArgs &A0, int *done)
     A.slices = c->dm.slices;
     A.smem_bytes = (unsigned)X.smem_bytes;
     A.lo.cand_layout = c->d_cand_layout;
-    return rp_launch_row_chip(c, A, X, (c->Ppop + cw - 1) / cw, done);
+    RP_TRY(rp_launch_row_chip(c, A, X, (c->Ppop + cw - 1) / cw, done));
+    if (*done) c->row_form = 1;
+    return RP_OK;
 }
 
 // Whether two chains share a warp: compressed rows of up to 32 layers where slot d is shard d, if there are more members than chains
-// resident with a warp each, and shared memory keeps at least half as many again when they share.  A round takes longer then (heavy
-// 5900 cycles for two, 4300 for one) and half the warps do it: eight levels of 200 steps on heavy, one chain to a warp and two, 2072
-// members (all resident either way) 2.41 and 2.57 ms, 2600 3.43 and 2.87, 4096 4.27 and 3.43, 6000 5.94 and 5.52, 8192 7.66 and 6.33; on
-// its first 16 layers 2.32 and 2.20, 3.30 and 2.45, 4.20 and 2.99, 5.69 and 4.62, 7.36 and 5.36.  Of 48 layers a lane would have
-// three, and wide's 288 row-shards leave shared memory for six warps: 8.5 and 12.7 ms.
-static bool row_pairs(const rp_ctx *c, const RowArgs &X0)
+// resident with a warp each, and an SM keeps at least half as many again when they share.  A round takes longer then (heavy
+// 5900 cycles for two, 4300 for one) and half the warps do it.  How many warps are resident is asked for: 16 by the registers of
+// today's instances (128 a thread), fewer by the shared memory of windows with many row-shards.  20 levels of 100 steps, one chain to
+// a warp and two, in ms, with 2368 (16 on each of 148 SMs), 2400 and 3000 members: 16 layers of 32 ranks, 4000 samples 2.77 and 2.82,
+// 3.18 and 2.87, 3.60 and 2.97; 32 layers, 1000 samples 1.90 and 2.16, 2.04 and 2.18, 2.35 and 2.27; heavy 4.23 and 4.47, 5.31 and
+// 4.66, (3500) 6.46 and 5.21.  (14 were counted before, so that 2073 to 2368 members shared warps: 2200 members of the second 1.87
+// ms, 2.15.)  Of 48 layers a lane would have three, and wide's 288 row-shards leave shared memory for six warps: 8.5 and 12.7 ms.
+static int row_pairs(const rp_ctx *c, const RowArgs &X0, bool *pair)
 {
-    if (!X0.comp || !c->dm.own_shard || c->dm.L > 32) return false;
+    *pair = false;
+    if (!X0.comp || !c->dm.own_shard || c->dm.L > 32) return RP_OK;
     RowArgs X = X0;
-    const int room = 227 * 1024;
+    int one = 0, two = 0;
     chain_layout(c->dm, c->bl, c->sl, X, false, 1, c->Ppop, 0);
-    const int one = std::min(14, room / (X.smem_bytes + 1024));
+    RP_TRY(rp_row_level_resident(c, X, &one));
+    if (c->Ppop <= one * rp_sms(c)) return RP_OK;
     chain_layout(c->dm, c->bl, c->sl, X, false, 2, c->Ppop, 0);
-    if (X.smem_bytes > ROW_SMEM_MAX) return false;         // (what a launch may ask for is a little less than an SM has)
-    const int two = 2 * std::min(14, room / (X.smem_bytes + 1024));
-    return c->Ppop > one * rp_sms(c) && 2 * two >= 3 * one;
+    if (X.smem_bytes > ROW_SMEM_MAX) return RP_OK;         // (what a launch may ask for is a little less than an SM has)
+    RP_TRY(rp_row_pair_resident(c, X, &two));
+    *pair = 2 * 2 * two >= 3 * one;
+    return RP_OK;
 }
 
 int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A);
@@ -349,13 +356,15 @@ int rp_launch_anneal_row(rp_ctx *c, AnnealArgs &A)
 {
     RowArgs X;
     row_args(c, X);
-    const bool pair = row_pairs(c, X);
+    if (A.level == 0) RP_TRY(row_pairs(c, X, &c->row_pair));
+    const bool pair = c->row_pair;
     chain_layout(c->dm, c->bl, c->sl, X, false, pair ? 2 : 1, c->Ppop, 0);
     if (X.smem_bytes > ROW_SMEM_MAX) return RP_ERR_RANGE;
     A.smem_bytes = (unsigned)X.smem_bytes;
     A.slices = 1;
     A.lo.cand_layout = nullptr;
     RP_TRY(pair ? rp_launch_row_pair(c, A, X) : rp_launch_row_level(c, A, X));
+    c->row_form = pair ? 5 : X.comp ? 4 : rp_row_split(X.cpl) ? 3 : 2;
     if (!A.last && rp_row_turns(c)) return rp_launch_level_turn(c, A);
     return rp_launch_level_end(c, A);
 }

@@ -48,3 +48,6 @@ static inline bool rp_row_split(int cpl) { return cpl == 2 || cpl == 4; }
 int rp_launch_row_chip(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int grid, int *done);
 int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);
 int rp_launch_row_pair(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);
+// Warps of the instance that the launch would take which an SM keeps resident.
+int rp_row_level_resident(const rp_ctx *c, const RowArgs &X, int *warps);
+int rp_row_pair_resident(const rp_ctx *c, const RowArgs &X, int *warps);

@@ -276,9 +276,12 @@ __device__ __forceinline__ void row_barrier_warp(const AnnealArgs &A, int P, con
     }
 }
 
-// Warps per SM the register budget is set for: heavy, a chain to a warp and one chunk per lane, at 12 / 13 / 14: 66.1 / 66.0 / 66.7 ms,
-// but 14 take windows of up to 2072 members at once; two chains to a warp 10 / 12 / 14: 57.0 / 57.8 / 55.8; more chunks, or shards of
-// several slots, need the registers of 12.
+// Warps per SM the register budget is set for.  Registers come in quarters of an SM: 12 leaves 168 a thread and keeps 12 warps
+// resident, 13 to 16 leave 128 and keep 16.  Which is better depends on how many chains there are; at 12 / 14 / 16, plans in ms: heavy
+// (8192 members, two to a warp) 61.6 / 59.4 / 59.5, 4096 members of 16 layers of 32 ranks (two to a warp) 4.15 / 3.41 / 3.44; where 12 a
+// SM hold them all, 1776 members with a warp each, heavy's window at 20 levels of 200 steps 5.95 / 6.55 / 6.82.  (Asked for 16 the compiler
+// orders the code another way and spills less, 24 bytes for 40, to no gain.)  More chunks, or shards of several slots, need the
+// registers of 12.
 #define ROW_WARPS_PER_SM(GL, LPL, CPL, IDENT) ((GL) == 16 || ((LPL) * (CPL) == 1 && (IDENT)) ? 14 : 12)
 
 // GL lanes run a chain, LPL layers per lane, CPL 16-byte chunks per layer (X.cpl <= CPL of them in use).  IDENT: slot d is shard d.
@@ -1110,5 +1113,14 @@ static int launch_row_t(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int gr
     RP_CUDA(e);
     ++g_rp_launches; ++c->n_queued;
     *done = 1;
+    return RP_OK;
+}
+
+template <int GL, int LPL, int CPL, bool SPLIT, bool COMP, bool IDENT>
+static int row_resident_t(const RowArgs &X, int *warps)
+{
+    auto kern = k_anneal_row<GL, LPL, CPL, SPLIT, false, COMP, IDENT>;
+    RP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_SMEM_MAX));
+    RP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(warps, kern, 32, (size_t)X.smem_bytes));
     return RP_OK;
 }

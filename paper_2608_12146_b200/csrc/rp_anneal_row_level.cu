@@ -22,3 +22,9 @@ int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X)
 {
     return c->dm.own_shard ? launch<true>(c, A, X) : launch<false>(c, A, X);
 }
+
+// (asked for compressed rows of up to 32 layers where slot d is shard d)
+int rp_row_level_resident(const rp_ctx *, const RowArgs &X, int *warps)
+{
+    return row_resident_t<32, 1, 1, false, true, true>(X, warps);
+}

@@ -10,3 +10,8 @@ int rp_launch_row_pair(rp_ctx *c, const AnnealArgs &A, const RowArgs &X)
     if (c->dm.L <= 32) return launch_row_t<16, 2, 1, false, false, true, true>(c, A, X, grid, &done);
     return RP_ERR_STATE;
 }
+
+int rp_row_pair_resident(const rp_ctx *c, const RowArgs &X, int *warps)
+{
+    return c->dm.L <= 16 ? row_resident_t<16, 1, 1, false, true, true>(X, warps) : row_resident_t<16, 2, 1, false, true, true>(X, warps);
+}

@@ -1002,6 +1002,7 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     }
     c->log_clean = 0;
     c->slices_listed = 0;
+    c->row_form = 0;
 
     RpSide *side = (RpSide *)c->side;
     cudaEvent_t ev[2] = { side ? side->t0 : nullptr, side ? side->t1 : nullptr };
@@ -1388,6 +1389,14 @@ extern "C" int rp_debug_chain_kernel(rp_ctx *c, int32_t *which)
     if (c->stage < 3) return RP_ERR_STATE;
     // (compressed rows: decided by the first rp_anneal call)
     *which = rp_uses_row(c) ? 3 : rp_uses_warp_chains(c) ? 2 : (rp_uses_wpc(c->dm) ? 0 : 1);
+    return RP_OK;
+}
+
+extern "C" int rp_debug_chain_form(rp_ctx *c, int32_t *form)
+{
+    if (!c || !form) return RP_ERR_ARG;
+    if (c->stage < 3) return RP_ERR_STATE;
+    *form = c->row_form;
     return RP_OK;
 }
 

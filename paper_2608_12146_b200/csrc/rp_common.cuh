@@ -155,6 +155,8 @@ struct rp_ctx {
     int row_undecided;         // compressed rows: row-shards of the evaluated members that they do not decide, -1 = not read back yet
     int row_members;           // members with a scored state of their own (0 .. n-1 of the current buffer)
     int row_counted;           // members row_undecided was counted over
+    bool row_pair;             // two chains share a warp (decided at a call's first level)
+    int row_form;              // form the last rp_anneal call launched (see rp_debug_chain_form)
     int rows_made;             // d_tf and d_qr are filled
     int *d_top;                // [L][3] ranks of each layer by decreasing aggregate load
     int *d_tf;                 // [N][2] length, demand on the fixed ranks

@@ -1691,7 +1691,7 @@ def test_rows_dealt_out_to_the_lanes(N, L, P, D, edp):
     ctx = load(w, pop=pop, edp=edp, min_rows=3)
     check_front(w, ctx, ref)
     _, stats = check_anneal(w, ctx, ref, edp, pop, 3, 21, t_ratio=0.5, check_members=2)
-    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.accepted > 0
+    assert rp.rp_debug_chain_form(ctx) == ("whole layers" if P == 12 else "dealt out") and stats.accepted > 0
     rp.rp_destroy(ctx)
 
 
@@ -1706,7 +1706,7 @@ PAIR_CASES = [
 
 @pytest.mark.parametrize("spec,steps", PAIR_CASES, ids=[e[0][0] for e in PAIR_CASES])
 def test_two_chains_to_a_warp(spec, steps):
-    """Compressed rows with more members than three SMs hold with a warp each, an odd one left over, windows of steps that end before
+    """Compressed rows with more members than two SMs hold with a warp each, an odd one left over, windows of steps that end before
     the sixteenth, whole or with open layers; then on with a warp to a chain and back."""
     name, N, L, E, P, D, edp, min_rows, pop = spec
     w = compressed_window(spec)
@@ -1714,18 +1714,35 @@ def test_two_chains_to_a_warp(spec, steps):
     ref = oracle_front(w, edp, min_rows)
     ctx = load(w, pop=pop, edp=edp, min_rows=min_rows)
     rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 3)
-    rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 3)
+    rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 2)
     check_front(w, ctx, ref)
     want, stats = check_anneal(w, ctx, ref, edp, pop, 3, steps, t_ratio=0.6, check_members=2, t0=1e-2)
-    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.accepted > 0
-    for sms in (0, 3):
+    assert rp.rp_debug_chain_form(ctx) == "two to a warp" and stats.accepted > 0
+    for sms, form in ((0, "compressed"), (2, "two to a warp")):
         rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", sms)
         want = oracle.anneal(w.lengths, ref["q"], want["final_pop"], ref["R"], s.token_cap, D, n_levels=2, steps=steps, t0=1e-4,
                              t_ratio=0.5, p_reloc=0.5, p_guide=0.3, seed=s.anneal_seed, edp_of_dp=edp, alpha=s.alpha, beta=s.beta,
                              n_threads=8)
         rp.rp_anneal(ctx, n_levels=2, steps_per_level=steps, t0=1e-4, t_ratio=0.5, p_reloc=0.5, p_guide=0.3)
+        assert rp.rp_debug_chain_form(ctx) == form
         assert (rp.rp_debug_dump(ctx, "TRACE_TERM", (2, pop, 3), np.int64) == want["term"]).all()
         assert (rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32) == want["final_pop"]).all()
+    rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("L", [16, 17])
+@pytest.mark.parametrize("pop,form", [(32, "compressed"), (33, "two to a warp")])
+def test_as_many_members_as_are_resident_keep_a_warp_each(L, pop, form):
+    """Sixteen warps of 128 registers fill an SM: two SMs keep 32 chains with a warp each, and share warps from the 33rd on."""
+    spec = ("resident", 80, L, 64, 32, 3, None, 3, pop)
+    w = compressed_window(spec)
+    ref = oracle_front(w, None, 3)
+    ctx = load(w, pop=pop, min_rows=3)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 3)
+    rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 2)
+    check_front(w, ctx, ref)
+    _, stats = check_anneal(w, ctx, ref, None, pop, 2, 20, t_ratio=0.6, check_members=2, t0=1e-2)
+    assert rp.rp_debug_chain_form(ctx) == form and stats.accepted > 0
     rp.rp_destroy(ctx)
 
 
@@ -1741,7 +1758,7 @@ def test_two_chains_that_take_more_than_half_an_sm_each(D, R):
     rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 3)
     check_front(w, ctx, ref)
     _, stats = check_anneal(w, ctx, ref, None, 5, 3, 40, t_ratio=0.6, check_members=2, t0=1e-2)
-    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.accepted > 0
+    assert rp.rp_debug_chain_form(ctx) == "compressed" and stats.accepted > 0
     rp.rp_destroy(ctx)
 
 
