@@ -287,6 +287,8 @@ typedef enum {
     RP_DUMP_TRACE_INCUMBENT = 15, /* int64 [n_levels][3]                                   */
     RP_DUMP_SELECT_DIST = 17, /* int64 [P_pop][P_pop] plan distances between the representatives
                                  of the last rp_select_population (0 elsewhere); inspection hook on */
+    RP_DUMP_SLACK = 18,      /* int64 [R][G] of member `index`, one-layer-per-lane kernel: sum_l max_p W less what the
+                                row-shard's samples put on each layer's busiest rank of the window (after rp_anneal) */
     RP_DUMP_EVAL_W = 16      /* int32 [R][G][L][P] of layout `index` of the last
                                 rp_eval_population call with explicit layouts (n <= 64)    */
 } rp_dump_what;

@@ -284,7 +284,7 @@ def rp_release_cached_memory():
 # ---- inspection hooks -------------------------------------------------------------------
 DUMP = dict(LAGG=1, Q=2, SEED_LAYOUT=3, POPULATION=4, W=5, CELL_T=6, CELL_Q=7, CELL_CNT=8, ESUM=9,
             TRACE_TERM=10, TRACE_BEST=11, TRACE_BEST_STEP=12, TRACE_DIGEST=13, TRACE_ANC=14,
-            TRACE_INCUMBENT=15, EVAL_W=16, SELECT_DIST=17)
+            TRACE_INCUMBENT=15, EVAL_W=16, SELECT_DIST=17, SLACK=18)
 
 
 def rp_debug_set_trace(ctx: Context, on: bool = True):

@@ -115,25 +115,33 @@ k_member_rows(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *
     if (comp && tid == 0 && bad_s) atomicAdd(undecided, 1);
 }
 
-// The slacks alone, one CTA per member: a scan of the assignment with 64-bit additions in shared memory (a CTA per row-shard scans it
-// once for each: 256 members of 2048 samples in 240 row-shards took 134 us, a plan with candidates 3.24 ms).
+// The slacks alone, one CTA per member: one scan of the assignment (a CTA per row-shard scans it once for each: 256 members of 2048
+// samples in 240 row-shards 134 us, 5.4 here).  Sums in shared memory by the lower and upper 16 bits of each f apart (below 65536
+// samples neither passes 32 bits): a 64-bit addition there is a loop, and where many samples of a row-shard meet it took 180 us for 8192
+// samples in four row-shards, 10 here, and 24 in a CTA per row-shard.
 __global__ void __launch_bounds__(256)
 k_member_slack(RpDims dm, RpBlob bl, const char *__restrict__ blobs, const char *__restrict__ static_blk, RpStatic sl, const int2 *__restrict__ tf,
                i64 *__restrict__ Fo, int *__restrict__ undecided, int loose)
 {
-    extern __shared__ u64 sum[];                        // [RG]
+    extern __shared__ uint2 sum[];                      // [RG]
     const int m = blockIdx.x, tid = threadIdx.x;
     const char *blob = blobs + (size_t)m * bl.bytes;
     const unsigned short *cells = (const unsigned short *)(blob + bl.off_cell);
     const unsigned short *rg_of = (const unsigned short *)(static_blk + sl.off_rg);
-    for (int rg = tid; rg < dm.RG; rg += 256) sum[rg] = 0;
+    for (int rg = tid; rg < dm.RG; rg += 256) sum[rg] = make_uint2(0, 0);
     __syncthreads();
 #pragma unroll 8
-    for (int i = tid; i < dm.N; i += 256) atomicAdd(&sum[__ldg(rg_of + cells[i])], (u64)(i64)__ldg(&tf[i].y));
+    for (int i = tid; i < dm.N; i += 256) {
+        uint2 *s = sum + __ldg(rg_of + cells[i]);
+        const u32 f = (u32)__ldg(&tf[i].y);
+        atomicAdd(&s->x, f & 0xffffu);
+        if (f >> 16) atomicAdd(&s->y, f >> 16);
+    }
     __syncthreads();
     int n = 0;
     for (int rg = tid; rg < dm.RG; rg += 256) {
-        const i64 es = ((const i64 *)(blob + bl.off_Esum))[rg], slack = es - (i64)sum[rg];
+        const uint2 s = sum[rg];
+        const i64 es = ((const i64 *)(blob + bl.off_Esum))[rg], slack = es - ((i64)s.x + ((i64)s.y << 16));
         Fo[(size_t)m * dm.RG + rg] = slack;
         n += loose && slack * 16 > es;
     }
@@ -290,7 +298,7 @@ int rp_launch_member_rows(rp_ctx *c, int n)
     RP_CUDA(cudaMemsetAsync(c->d_undecided, 0, sizeof(int), c->stream));
     i64 *Fo = c->d_rowF + (size_t)c->cur * c->Ppop * dm.RG;
     if (!sep)                       // (a chain keeps 40 bytes of a row-shard in shared memory: no more than 5632)
-        k_member_slack<<<n, 256, sizeof(u64) * (size_t)dm.RG, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_static, c->sl, (const int2 *)c->d_tf, Fo,
+        k_member_slack<<<n, 256, sizeof(uint2) * (size_t)dm.RG, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_static, c->sl, (const int2 *)c->d_tf, Fo,
                                                                           c->d_undecided, c->row_check);
     else
         k_member_rows<<<dim3(n, dm.RG), 256, smem, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_static, c->sl, (const int2 *)c->d_tf, X.qr, X.rlp,

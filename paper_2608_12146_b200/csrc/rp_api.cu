@@ -1266,7 +1266,7 @@ extern "C" int rp_debug_dump(rp_ctx *c, int what, int32_t index, void *buf, int6
     void *tmp = nullptr;
     int st = RP_OK;
     int member = -1;
-    if (what >= RP_DUMP_POPULATION && what <= RP_DUMP_ESUM) {
+    if ((what >= RP_DUMP_POPULATION && what <= RP_DUMP_ESUM) || what == RP_DUMP_SLACK) {
         if (c->stage < 3) return RP_ERR_STATE;
         if (what != RP_DUMP_POPULATION) {
             if (index < 0 || index >= c->Ppop) return RP_ERR_ARG;
@@ -1313,6 +1313,9 @@ extern "C" int rp_debug_dump(rp_ctx *c, int what, int32_t index, void *buf, int6
             src = c->d_W + (size_t)cell * dm.RG * dm.LP; need = sizeof(int) * (size_t)dm.RG * dm.LP; break;
             }
         case RP_DUMP_ESUM: src = c->buf[c->cur].blob + (size_t)member * c->bl.bytes + c->bl.off_Esum; need = sizeof(i64) * dm.RG; break;
+        case RP_DUMP_SLACK:
+            if (!c->row_mode || !c->rows_current) return RP_ERR_STATE;
+            src = c->d_rowF + ((size_t)c->cur * P + member) * dm.RG; need = sizeof(i64) * dm.RG; break;
         case RP_DUMP_CELL_T: case RP_DUMP_CELL_Q: case RP_DUMP_CELL_CNT: {
             size_t K = dm.K;
             if ((st = dev_alloc(c, (i64 **)&tmp, 3 * K)) != RP_OK) return st;

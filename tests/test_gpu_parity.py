@@ -1695,6 +1695,46 @@ def test_rows_dealt_out_to_the_lanes(N, L, P, D, edp):
     rp.rp_destroy(ctx)
 
 
+@pytest.mark.parametrize("case", ["small", "beyond_16_bits", "beyond_32_bits"])
+def test_slacks_of_few_row_shards(case):
+    """Hundreds of samples to a row-shard: sums of 16-bit halves, whose lower or upper one alone is used, or both up to a sum
+    beyond 32 bits; as scored, and as the moves leave them."""
+    rng = np.random.default_rng(len(case))
+    edp = None
+    if case == "small":
+        w = make_window(custom_spec(case, 700, 3, 16, 2, 1 << 17, 2, 8, 6, 0, data_seed=5))
+        w.lengths[:] = rng.integers(1, 120, 700)
+        w.demand[:] = rng.multinomial((2 * w.lengths.astype(np.int64))[:, None], rng.dirichlet(np.full(16, 0.3), size=3))
+    elif case == "beyond_16_bits":
+        w = one_heavy_expert(case, rng.integers(20_000, 60_000, 2000), 4, 8, 4, 1 << 23, 2, 8, 6, 0.7)
+    else:
+        w = one_heavy_expert(case, rng.integers(250_000, 420_000, 40), 120, 4, 8, 1 << 20, 32, 4, 6, 0.9)
+        edp = UNEVEN
+    s = w.spec
+    ref = oracle_front(w, edp)
+    ctx = load(w, pop=6, edp=edp)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 3)
+    check_front(w, ctx, ref)
+    G = 1 + (max(edp) if edp is not None else s.dp_width - 1)
+    of = np.asarray(edp if edp is not None else range(s.dp_width))
+    fixed = ref["G"].argmax(axis=1)                                  # (of equal ones the lowest)
+    f = ref["q"].astype(np.int64)[:, np.arange(s.n_layers), fixed].sum(axis=1)
+    for init, steps in ((None, 1), ("now", 25)):
+        init = rp.rp_debug_dump(ctx, "POPULATION", (6, s.n_samples), np.int32) if init else None
+        check_anneal(w, ctx, ref, edp, 6, 2, steps, t_ratio=0.6, check_members=1, init=init, t0=1e-2)
+        assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row"
+        layouts = rp.rp_debug_dump(ctx, "POPULATION", (6, s.n_samples), np.int32)
+        for j in range(6):
+            rg = layouts[j] // s.dp_width * G + of[layouts[j] % s.dp_width]
+            sums = np.zeros(ref["R"] * G, np.int64)
+            np.add.at(sums, rg, f)
+            want = rp.rp_debug_dump(ctx, "ESUM", (ref["R"] * G,), np.int64, index=j) - sums
+            assert (rp.rp_debug_dump(ctx, "SLACK", (ref["R"] * G,), np.int64, index=j) == want).all()
+    assert f.max() < 1 << 16 if case == "small" else f.max() >= 1 << 16
+    assert (sums.max() >= 1 << 32) == (case == "beyond_32_bits")
+    rp.rp_destroy(ctx)
+
+
 PAIR_CASES = [
     # as COMPRESSED_CASES, and the steps of a level: sixteen lanes to a chain, one or two layers to a lane
     (("pair_16_layers", 80, 16, 64, 32, 3, None, 3, 45), 50),
