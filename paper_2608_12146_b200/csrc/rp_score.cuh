@@ -76,7 +76,6 @@ __device__ __forceinline__ i64 rp_warp_layer_max_sum(const RpDims &dm, int lane,
 __device__ __forceinline__ void rp_accumulate_cells(const RpDims &dm, const RpSmemState &st,
                                                     const int *__restrict__ t, int tid, int nt)
 {
-#pragma unroll 8
     for (int i = tid; i < dm.N; i += nt) {
         int c = st.cell_of[i];
         int ti = t[i];
