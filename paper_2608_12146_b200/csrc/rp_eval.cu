@@ -41,6 +41,7 @@ struct EvalArgs {
     i64 *score_final;
     double *f64_final;
     int n;
+    bool q_halves;                                // (few layouts) no cell's squared lengths add up to 2^48, whatever the layout
     i64 *Esum;                                    // [n][RG] row-shard sums (few layouts: costs) handed to the finishing CTA; zero between launches
     int *tickets;                                 // [n] arrival counters; zero between launches
     unsigned short *list;                         // [n][N] samples grouped by row-shard (k_eval_group)
@@ -343,11 +344,23 @@ __device__ __forceinline__ i64 few_warp_max(i64 v)
     return v;
 }
 
+// Sums of squared lengths in shared memory: 64 bits, or (halves: no sum reaches 2^48) the lower 16 bits of each square and what lies
+// above them added up in 32 bits each.  A 64-bit addition there is a loop, and the samples of a row-shard of few slots meet in it: 4000
+// samples in six row-shards of one slot, 128 layouts 206 us and 147 in halves, one layout 48 and 41.
+__device__ __forceinline__ void few_add(u64 *q, u32 low, u32 high, bool halves)
+{
+    if (halves) { atomicAdd((u32 *)q, low); atomicAdd((u32 *)q + 1, high); }
+    else atomicAdd(q, ((u64)high << 32) | low);
+}
+__device__ __forceinline__ u64 few_square(u64 v, bool halves) { return halves ? ((v >> 32) << 16) + (u32)v : v; }
+
 // grid = (MS, row-shards, layouts), clusters of MS CTAs along x: CTA x of a row-shard takes the samples of
 // range x, then the layers of range x of the summed row.  The row-shard's cell statistics and cost are worked out by its own
 // cluster beside the sums, so that what is left for the CTA that finishes a layout is a sum over its row-shards (with the statistics of
 // all samples added up there, one CTA took two thirds of the time on heavy's 8192; with the one launch of the metrics behind it a call
-// of rp_diagnostics on heavy 90 -> 47 us).
+// of rp_diagnostics on heavy 90 -> 47 us).  Where there are more CTAs than the SMs hold it matters how many those are: 48 registers
+// and five to an SM (the loop over the cluster's sums unrolled twice; 62 and four when it and the statistics were unrolled four times: two
+// layouts of 2048 samples in 240 row-shards 38.4 and 32.4 us, 69 of 401 in ten 53.4 and 48.3).
 static inline size_t eval_few_smem(const RpDims &dm, int MS)
 {
     const size_t part = (sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2) + 7) & ~(size_t)7;
@@ -371,7 +384,7 @@ k_eval_few(const EvalArgs A)
     __shared__ i64 s0_s, s1_s, s2_s;
     const EvalCells cells = eval_cells(A, lay);
     char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
-    if (tid == 0) { n_s = 0; es_s = 0; wrong_s = 0; s0_s = 0; s1_s = 0; s2_s = 0; }
+    if (tid == 0) { n_s = 0; es_s = 0; s0_s = 0; s1_s = 0; s2_s = 0; }
     const int row = rg / dm.G, g = rg % dm.G, first = row * dm.D;
     // (a slot of another shard has a negative count: which slots are the row-shard's is looked up in global memory only here)
     for (int d = tid; d < dm.D; d += EVAL_THREADS) { Q[d] = 0; T[d] = 0; cnt[d] = __ldg(A.edp + d) == g ? 0 : (int)0x80000000; }
@@ -383,7 +396,10 @@ k_eval_few(const EvalArgs A)
         if ((unsigned)d >= (unsigned)dm.D || cnt[d] < 0) continue;
         const int ti = __ldg(A.t + i);
         list[atomicAdd(&n_s, 1)] = i;
-        atomicAdd(&T[d], ti); atomicAdd(&cnt[d], 1); atomicAdd(&Q[d], (u64)ti * (u64)ti);
+        atomicAdd(&T[d], ti); atomicAdd(&cnt[d], 1);
+        const u64 sq = (u64)ti * (u64)ti;
+        if (A.q_halves) few_add(&Q[d], (u32)sq & 0xffffu, (u32)(sq >> 16), true);
+        else few_add(&Q[d], (u32)sq, (u32)(sq >> 32), false);
         if (b) ((unsigned short *)(b + A.bl.off_cell))[i] = (unsigned short)c;
     }
     if (A.layout_host && rg == 0) for (int i = i0 + tid; i < i1; i += EVAL_THREADS) A.layout_host[i] = __ldg(A.lay32 + i);
@@ -419,7 +435,7 @@ k_eval_few(const EvalArgs A)
         const bool on = lane < used && c < l1 * cpl;
         int4 a = make_int4(0, 0, 0, 0);
         if (on)
-#pragma unroll 4
+#pragma unroll 2
             for (int x = 0; x < MS; ++x) {
                 const int4 v = ((const int4 *)cl.map_shared_rank(part, x))[c];
                 a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
@@ -430,33 +446,47 @@ k_eval_few(const EvalArgs A)
     }
     for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
     if (lane == 0 && es) atomicAdd(&es_s, (u64)es);
-    // statistics of all of the cluster's samples, by its first CTA (the others leave theirs as they are)
-    if (ms == 0)
-        for (int d = tid; d < dm.D; d += EVAL_THREADS) {
-            int t = T[d], m = cnt[d];
-            if (m < 0) continue;
-            u64 q = Q[d];
-#pragma unroll 4
-            for (int x = 1; x < MS; ++x) { t += cl.map_shared_rank(T, x)[d]; m += cl.map_shared_rank(cnt, x)[d]; q += cl.map_shared_rank(Q, x)[d]; }
-            T[d] = t; cnt[d] = m; Q[d] = q;
-            if (m < 1 || t > dm.C) wrong_s = 1;
-            if (b) {
-                ((u64 *)(b + A.bl.off_Q))[first + d] = q;
-                ((int *)(b + A.bl.off_T))[first + d] = t;
-                ((int *)(b + A.bl.off_cnt))[first + d] = m;
+    // Statistics of all of the cluster's samples meet in its first CTA: a lane there for every CTA of a slot, which fetches; more slots
+    // than it has lanes for are added to it from afar (diagnostics of 6000 samples in four row-shards of 64 slots 56 us fetched).
+    if (dm.D * MS <= EVAL_THREADS) {
+        if (ms == 0 && MS > 1) {
+            const int d = tid / MS, x = tid & (MS - 1);
+            const bool on = d < dm.D && cnt[d < dm.D ? d : 0] >= 0;
+            int t = 0, m = 0;
+            u64 q = 0;
+            if (on) { t = cl.map_shared_rank(T, x)[d]; m = cl.map_shared_rank(cnt, x)[d]; q = cl.map_shared_rank(Q, x)[d]; }
+            for (int o = 1; o < MS; o <<= 1) {
+                t += __shfl_xor_sync(0xffffffffu, t, o); m += __shfl_xor_sync(0xffffffffu, m, o); q += __shfl_xor_sync(0xffffffffu, q, o);
             }
+            if (on && x == 0) { T[d] = t; cnt[d] = m; Q[d] = q; }
         }
+    } else if (ms) {
+        int *T0 = cl.map_shared_rank(T, 0), *cnt0 = cl.map_shared_rank(cnt, 0);
+        u64 *Q0 = cl.map_shared_rank(Q, 0);
+        for (int d = tid; d < dm.D; d += EVAL_THREADS)
+            if (cnt[d] > 0) { atomicAdd(T0 + d, T[d]); atomicAdd(cnt0 + d, cnt[d]); few_add(Q0 + d, (u32)Q[d], (u32)(Q[d] >> 32), A.q_halves); }
+    }
     __syncthreads();
     if (tid == 0) cl.map_shared_rank(es_of, 0)[ms] = es_s;
     cl.sync();                                            // nobody reads another CTA's shared memory from here on
     if (ms) return;
+    if (b)
+        for (int d = tid; d < dm.D; d += EVAL_THREADS) {
+            if (cnt[d] < 0) continue;
+            ((u64 *)(b + A.bl.off_Q))[first + d] = few_square(Q[d], A.q_halves);
+            ((int *)(b + A.bl.off_T))[first + d] = T[d];
+            ((int *)(b + A.bl.off_cnt))[first + d] = cnt[d];
+        }
     if (warp == 0) {
         i64 Af = 0, E = 0;
         for (int x = 0; x < MS; ++x) E += (i64)es_of[x];
+        bool wrong = false;
+        for (int d = lane; d < dm.D; d += 32) wrong |= cnt[d] == 0 || (cnt[d] > 0 && T[d] > dm.C);
+        wrong = __any_sync(0xffffffffu, wrong);
         for (int s = 0; s < dm.S; ++s) {
             const i64 ca = dm.ahat[s] * dm.C, cb = dm.bhat[s];
             i64 v = 0;
-            for (int d = lane; d < dm.D; d += 32) { const i64 w = cnt[d] < 0 ? 0 : ca * T[d] + cb * (i64)Q[d]; v = w > v ? w : v; }
+            for (int d = lane; d < dm.D; d += 32) { const i64 w = cnt[d] < 0 ? 0 : ca * T[d] + cb * (i64)few_square(Q[d], A.q_halves); v = w > v ? w : v; }
             for (int o = 16; o; o >>= 1) { const i64 w = __shfl_xor_sync(0xffffffffu, v, o); v = w > v ? w : v; }
             Af += v;
         }
@@ -469,9 +499,9 @@ k_eval_few(const EvalArgs A)
             A.Esum[(size_t)lay * dm.RG + rg] = J;
             __threadfence();
             // arrivals in the lower half, row-shards with an empty or overfull cell in the upper one
-            const unsigned before = atomicAdd((unsigned *)&A.tickets[lay], 1u | (wrong_s ? 1u << 16 : 0u));
+            const unsigned before = atomicAdd((unsigned *)&A.tickets[lay], 1u | (wrong ? 1u << 16 : 0u));
             last_s = (before & 0xffffu) == (unsigned)dm.RG - 1;
-            if (last_s) { wrong_s |= (before >> 16) ? 1 : 0; A.tickets[lay] = 0; }
+            if (last_s) { wrong_s = wrong || before >> 16; A.tickets[lay] = 0; }
         }
     }
     __syncthreads();
@@ -566,6 +596,7 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
     if (eval_smem_bytes(dm) > EVAL_SMEM_MAX) return RP_ERR_RANGE;
     A.dm = dm; A.bl = c->bl; A.t = c->d_t; A.q = c->d_q; A.edp = c->d_edp; A.dp_list = c->d_dp_list; A.dp_off = c->d_dp_off;
     A.n = n;
+    A.q_halves = (double)dm.C * (double)c->tokens < 281474976710656.0;         // (and N < 65536: see eval_smem_bytes)
     if (eval_is_few(dm, n)) {
         int MS = 1;
         while (MS < 8 && (long long)n * dm.RG * MS < 148 * 4 && dm.N >= 64 * MS) MS *= 2;

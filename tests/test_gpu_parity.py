@@ -1576,6 +1576,41 @@ def test_scoring_at_the_edges_of_its_forms(N, L, P, D, R, edp, ns):
     rp.rp_destroy(ctx)
 
 
+@pytest.mark.parametrize("N,D,edp", [(600, 32, [0] * 32), (600, 33, [0] * 33), (600, 64, None), (700, 80, [0, 1] * 40)])
+def test_cell_statistics_that_meet_in_a_cluster(N, D, edp):
+    """Scoring by clusters of eight: 32 slots, a lane for every CTA of a slot, and more; the scores, and the statistics a search
+    starts from."""
+    w = make_window(custom_spec("statistics", N, 3, 8, 2, 2048, D, 8, 3, 0, data_seed=D))
+    ref = oracle_front(w, edp, 2)
+    ctx = load(w, pop=3, edp=edp, min_rows=2)
+    check_front(w, ctx, ref)
+    check_eval(w, ctx, ref, edp, n=1)
+    check_anneal(w, ctx, ref, edp, 3, 2, 20, t_ratio=0.6)
+    rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,D", [(255, 5), (256, 4)])
+def test_squared_lengths_that_reach_48_bits(N, D):
+    """Cap times tokens just below 2^48, where squares are added up in two halves (all samples in one cell: the upper half just fits
+    32 bits), and at it, where they are not."""
+    t = np.full(N, 1 << 20)
+    if N == 255:
+        t[3::7] -= 3
+    w = one_heavy_expert("squares", t, 2, 4, 2, 1 << 20, D, 4, 2, 0.4)
+    s = w.spec
+    assert (s.token_cap * int(w.lengths.sum()) < 1 << 48) == (N == 255)
+    ref = oracle_front(w, None)
+    ctx = load(w, pop=2)
+    check_front(w, ctx, ref)
+    lays = np.random.default_rng(N).integers(0, ref["R"] * D, (2, N)).astype(np.int32)
+    lays[1] = ref["R"] * D - 1
+    fx, _ = rp.rp_eval_population(ctx, lays)
+    want = oracle.eval_layouts(w.lengths, ref["q"], lays, ref["R"], s.token_cap, D, None, s.alpha, s.beta)["score"]
+    assert (fx == want).all()
+    check_eval(w, ctx, ref, None, n=3)
+    rp.rp_destroy(ctx)
+
+
 @pytest.mark.parametrize("L,P,D,edp,pop,mixes,kernel", [
     (32, 4, 4, [1, 2, 3, 0], 9, 4, "k_anneal_wpc"), (8, 8, 3, [2, 0, 1], 256, 4, "k_anneal_wpc"),
     (8, 8, 3, [2, 0, 1], 257, 4, "k_anneal_row"), (5, 12, 3, [2, 0, 1], 20, 4, "k_anneal_row"),
