@@ -356,13 +356,14 @@ k_sel_dist(RpDims dm, int Ppop, int n_proj, const int *__restrict__ rep, SelBuf 
 }
 
 // ---- greedy selection (one CTA) -------------------------------------------------------------------
-// One selection after the other: a step is the load of one row of distances (L2), three warp-wide minima, one barrier and the
-// same minima over the warps' results, which every warp works out for itself (256 candidates 164 us; a shuffle tree over
-// triples, a serial pass of one thread and two barriers over 32 warps took 920).
+// One selection after the other: a step is the load of one row of distances, three warp-wide minima, one barrier and the
+// same minima over the warps' results, which every warp works out for itself (256 candidates, distances in L2, 220 us; a shuffle tree
+// over triples, a serial pass of one thread and two barriers over 32 warps took 920).
 #define GREEDY_THREADS 1024
 #define GREEDY_SMEM (160 * 1024)        // nearest distances and penalties of the candidates on chip up to this
-// The distances themselves on chip, 32 bits each and each pair once, where they fit (up to 303 candidates): a step then does not wait
-// for L2 (256 candidates 220 -> 196 us).
+// The distances themselves on chip, each pair once, where they fit (up to 307 candidates): a step then does not wait for L2 (256
+// candidates 220 -> 196 us).  In 32 bits: the two co-assignments are at most 2^20 each, and the sketch at most 2^21, since every row
+// feature of a plan within the cap is at most 2^16.
 #define GREEDY_DIST_MAX (184 * 1024)
 static inline size_t greedy_tri(size_t P) { return P * (P - 1) / 2; }
 struct SelPick { i64 v0, v1, v2; int j; };
@@ -425,19 +426,16 @@ k_sel_greedy(int Ppop, const int *__restrict__ rep, const i64 *__restrict__ scor
         mind[j] = rep[j] ? 0x7fffffffffffffffll : -1;      // -1 = not a candidate (or already selected)
     }
     __syncthreads();
-    // pair (i, j), i > j, at i (i - 1) / 2 + j (as long as every distance fits 32 bits)
+    // pair (i, j), i > j, at i (i - 1) / 2 + j
     u32 *near = (u32 *)(greedy_smem + 2 * (size_t)Ppop);
     if (tri) {
-        int over = 0;
         for (int i = warp; i < Ppop; i += nw)
 #pragma unroll 4
             for (int j = lane; j < i; j += 32) {
                 if (mind[i] < 0 || mind[j] < 0) continue;            // (no distance to a plan that stands for no class)
-                const i64 d = __ldg(dist + (size_t)i * Ppop + j);
-                over |= (u64)d >> 32 ? 1 : 0;
-                near[i * (i - 1) / 2 + j] = (u32)d;
+                near[i * (i - 1) / 2 + j] = (u32)__ldg(dist + (size_t)i * Ppop + j);
             }
-        tri = !__syncthreads_or(over);
+        __syncthreads();
     }
     for (int n = 0; n < nd; ++n) {
         if (tid == 0) order[n] = last;
