@@ -793,12 +793,12 @@ struct RpDiagDev { double cv_identity, cv_placed; i64 s_ep, t_ep, n_ep; i64 afx_
 #define DIAG_PEAK_CTAS 148
 // Coefficients: one warp per layer; the lanes fetch the rank loads, one lane adds them up with plain sequential IEEE sums (no fused
 // multiply-add); then thread 0 averages the layers in order.
-__device__ __forceinline__ void diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, const RpDims &dm, int warps,
+__device__ __forceinline__ void diag_cv(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, const RpDims &dm,
                                         double *cvs, RpDiagDev *__restrict__ out)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double *G = cvs + 2 * dm.L + (size_t)warp * dm.P;
-    for (int x = warp; x < 2 * dm.L && warp < warps; x += warps) {
+    for (int x = warp; x < 2 * dm.L; x += DIAG_THREADS / 32) {
         const int l = x >> 1, which = x & 1;
         for (int p = lane; p < dm.P; p += 32) {
             i64 g = 0;
@@ -835,11 +835,11 @@ __device__ __forceinline__ void diag_cv(const i64 *__restrict__ Lagg, const i64 
 // Peaks: one warp per (row, layer): lanes over ranks, loop over shards; integer results by atomics on `sums` (s_ep, n_ep, t_ep; zero
 // between launches, as the ticket is).
 __global__ void __launch_bounds__(DIAG_THREADS)
-k_diagnose(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, int cv_warps, const int *__restrict__ W, const char *__restrict__ blob,
+k_diagnose(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, const int *__restrict__ W, const char *__restrict__ blob,
            RpBlob bl, RpDims dm, i64 *__restrict__ sums, int *__restrict__ ticket, RpDiagDev *__restrict__ out)
 {
     extern __shared__ double cvs[];          // [2][L], then one row of rank loads per warp
-    if (blockIdx.x == DIAG_PEAK_CTAS) { diag_cv(Lagg, rank_load, dm, cv_warps, cvs, out); return; }
+    if (blockIdx.x == DIAG_PEAK_CTAS) { diag_cv(Lagg, rank_load, dm, cvs, out); return; }
     const int lane = threadIdx.x & 31;
     const int wid = (int)(threadIdx.x >> 5) * DIAG_PEAK_CTAS + (int)blockIdx.x, nw = DIAG_PEAK_CTAS * DIAG_THREADS / 32;
     i64 s_ep = 0, n_ep = 0, t_ep = 0;
@@ -901,9 +901,8 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
     // scratch: a copy of a layout that is not in this GPU's memory, W, one blob
     const size_t wn = (size_t)dm.RG * dm.LP;
     const size_t off_W = ((size_t)dm.N * 4 + 255) & ~(size_t)255, off_blob = off_W + ((wn * 4 + 255) & ~(size_t)255);
-    // (a row of P rank loads per warp: beyond 1700 ranks fewer warps than the kernel is made for)
-    const int cv_warps = (int)std::min<size_t>(DIAG_THREADS / 32, (EVAL_SMEM_MAX / sizeof(double) - 2 * (size_t)dm.L) / dm.P);
-    const size_t cv_smem = sizeof(double) * (2 * (size_t)dm.L + cv_warps * (size_t)dm.P);
+    // (a row of P rank loads per warp: 144 KB with 1024 layers of 1024 ranks, the most there are)
+    const size_t cv_smem = sizeof(double) * (2 * (size_t)dm.L + DIAG_THREADS / 32 * (size_t)dm.P);
     char *buf = nullptr;
     RP_CUDA(cudaMallocFromPoolAsync((void **)&buf, off_blob + (size_t)c->bl.bytes + 256, pool, c->stream));
     int st = RP_OK;
@@ -928,7 +927,7 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
             e = cudaFuncSetAttribute(k_diagnose, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX);
             if (e != cudaSuccess) break;
         }
-        k_diagnose<<<DIAG_PEAK_CTAS + 1, DIAG_THREADS, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, cv_warps, (const int *)(buf + off_W),
+        k_diagnose<<<DIAG_PEAK_CTAS + 1, DIAG_THREADS, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, (const int *)(buf + off_W),
                                                                             buf + off_blob, c->bl, dm, c->d_one_Esum + dm.RG, c->d_one_ticket, host);
         ++g_rp_launches;
         e = cudaGetLastError();

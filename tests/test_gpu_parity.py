@@ -1537,7 +1537,7 @@ def test_windows_with_negative_counts_are_refused(N, L, E, P):
 
 @pytest.mark.parametrize("P,L", [(864, 5), (1000, 2), (1024, 16)])
 def test_diagnostics_of_many_ranks(P, L):
-    """Rows of rank loads that do not fit shared memory for 32 warps at once."""
+    """Rows of rank loads of up to the most ranks there are, one per warp in shared memory."""
     w = make_window(custom_spec("many_ranks", 24, L, P, 2, 2048, 2, P, 3, 0, data_seed=P))
     s = w.spec
     ref = oracle_front(w, None, 2)
