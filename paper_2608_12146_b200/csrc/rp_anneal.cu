@@ -413,16 +413,17 @@ void rp_decide_layouts(rp_ctx *c)
     c->row_mode = 0; c->row_check = 0;
     const bool any = c->knob_chain_kernel == 3;                // (inspection hook: wherever it fits)
     if ((c->knob_chain_kernel == 0 || any) && c->knob_slices == 0) {
-        // Two kinds of window stay with the warp-per-candidate kernel where that runs all levels in one launch too:
-        //  * one slot per row-shard, but slot d is not shard d, at most a layer per lane (20 levels of 100 steps: L = 24, P = 4,
-        //    40 cells, 148 members 1.29 ms and 1.94 with one layer per lane; L = 6, P = 8, 24 cells 1.50 and 2.12; on average
-        //    a fifth.  Shards of several slots: a fifth to a half the other way);
+        // Two kinds of window stay with the warp-per-candidate kernel where that runs all levels in one launch too (20 levels of 100
+        // steps, 148 members, warp per candidate and one layer per lane, in ms, windows of four routing mixes):
+        //  * one slot per row-shard, but slot d is not shard d, at most a layer per lane (L = 24, P = 4, 56 cells 1.11 and 1.21; L = 6,
+        //    P = 8, 39 cells 0.72 and 0.80; L = P = 16, 52 cells 0.85 and 0.89; with one mix 0.85 and 0.80, 0.64 and 0.61, 0.73 and 0.68.
+        //    Shards of several slots: the other way);
         //  * few layers of many ranks (six lanes at most have a layer each, of four or eight chunks), or two shards and few layers, if
         //    the fixed ranks decide few rejections: more than a quarter of the row-shards are loose, their busiest loads a
-        //    sixteenth above the fixed ranks' (L = 3, P = 32, 24 cells 1.01 ms and 1.45; L = 2, 32 cells 2.03 and 2.53; two
-        //    shards, L = 8, P = 4, 24 cells 1.10 and 1.35; L = 3, P = 8 1.07 and 1.34; two or more shards of more layers even or
-        //    the other way).  Where all samples follow one routing mix no row-shard is loose, and one layer per lane takes 0.74
-        //    to 0.93 of the time; with four mixes 25 to 100 % are.  Finding out costs 10 us: for calls of 1000 steps and more.
+        //    sixteenth above the fixed ranks' (L = 3, P = 32, 40 cells 0.95 and 1.04; L = 2 0.76 and 0.81; but L = 6, P = 16 0.96 and 0.82; two
+        //    shards, L = 8, P = 4, 42 cells 0.65 and 0.56; L = 3, P = 8 0.79 and 0.61: the rule was drawn by an earlier form of the kernel,
+        //    which was behind on all of these).  Where all samples follow one routing mix no row-shard is loose, and one layer per lane
+        //    is ahead; with four mixes 25 to 100 % are.  Finding out costs 10 us: for calls of 1000 steps and more.
         const bool pow2 = dm.P >= 4 && (dm.P & (dm.P - 1)) == 0, wpc = !any && c->knob_level_launches != 1 && pow2 && rp_wpc_one_launch(c);
         if (wpc && dm.G == dm.D && !dm.own_shard && dm.L <= 32) return;
         c->row_check = wpc && dm.own_shard && ((dm.L <= 6 && dm.P >= 16) || (dm.L <= 12 && dm.G <= 2));

@@ -1,5 +1,5 @@
 // Chain kernel of the population annealing for windows whose rank-load rows are short enough to be
-// scored from registers: "one warp per chain, one layer per lane".
+// scored from registers: a warp per chain (or half a warp), one layer per lane.
 //
 // A chain of Algorithm 3 is a sequence of dependent rounds; what bounds a level is the latency of a
 // round times the rounds of a chain, over the chains an SM keeps in flight.  The kernel shortens and
@@ -8,7 +8,7 @@
 //    fixed rank per layer (the busiest of the window as a whole) and f_i = sum_l q[i][l][p_l], the new
 //    expert cost of the row-shard that gives sample i and takes i2 is at least F - f_i + f_i2, F the sum of
 //    f over its samples (kept as the slack Esum - F).  Score and energy are monotone in it, so the lane that proposes a step can
-//    reject it by itself from cell statistics, F and two scalars: 32 steps at a time, no rank load read.
+//    reject it by itself from cell statistics, F and two scalars: 32 steps at a time (16 where two chains share a warp), no rank load read.
 //    Windows whose samples follow one routing mix have the same busiest rank nearly everywhere, and
 //    then every rejection is decided this way and what is scored is accepted (large, wide, heavy, medium of
 //    the named windows: all but 1e-4 of the rejections); with four routing mixes an eighth to a third
@@ -16,7 +16,8 @@
 //    allowance for its roundings: in 64-bit integers it was a third of a round's instructions (with the decision shared by two
 //    lanes: heavy 89.2 -> 81.4 ms, wide 8.22 -> 8.04, medium 0.87 -> 0.84).
 //  * Rows in registers.  A lane holds whole layers (layer = lane, lane + 32, ...) of the two slices and the two
-//    demand rows: 16-byte loads, one trip, no shuffles, no staging; the new slices are stored from the
+//    demand rows, or, one launch per level with rows of two or four chunks a layer, the chunks are dealt out to the lanes in turn and
+//    a layer's maximum meets in shuffles: 16-byte loads, one trip, no staging; the new slices are stored from the
 //    same registers.
 //  * Compressed rows (COMP: rank counts of 8 and more whose full rows do not fit the registers).  A row keeps, per
 //    layer, the loads of the three ranks that are busiest in the window and an upper bound of every
@@ -26,9 +27,9 @@
 //    row-shards nearly all satisfy it (checked on the device, see k_member_rows): 16 bytes per layer
 //    instead of 4*P: an eighth of the traffic at 32 ranks.
 //  * Two chains to a warp (sixteen lanes each, see row_pairs) where there are more members than a warp each keeps resident.
-//  * No staging area, so 12 to 14 warps per SM instead of 5 to 10.
+//  * No staging area, so 12 or 16 warps per SM instead of 5 to 10.
 // What bounds it now: the latency of a round, about 2200 cycles alone on an SM (medium), 3300 with 7 warps (large), 3800 with 11 (wide)
-// and 5900 for two chains with 14 (heavy), where the warps' instructions share the issue slots; launched once for all levels the
+// and 5900 for two chains with 16 (heavy), where the warps' instructions share the issue slots; launched once for all levels the
 // slowest chain of a level takes twice the mean, three quarters of the level's time.  A level's time with the warp-per-chain kernel
 // (medium: warp per candidate) and now: heavy 15.0 -> 2.7 ms, wide 1.2 -> 0.40 ms, large 0.21 -> 0.10 ms, medium 50 -> 29 us.
 // Step for step this is the sequential chain: proposals are evaluated against the current state,
@@ -226,11 +227,12 @@ int rp_row_kind(const RpDims &dm)
 
 // Whether the form that launches once per level is taken by the shared memory of a chain (a warp to itself).  Where DP slot d is
 // shard d, as far as it fits: it is the fastest kernel even with one chain per SM (L = 24, P = 16, 1024 members, three levels of
-// 200 steps: 63 KB 1.39 ms and 1.71 for the next best kernel, 117 KB 3.8 and 4.8, 140 KB 4.1 and 4.9; L = P = 32, 2048 members,
-// three of 100: 94 KB 2.2 and 3.0, 136 KB 6.0 and 8.1).  Else the attention of a shard's slots is looked up
-// (8*K + 18*R*G*S bytes more, S stages a move) and four-warp CTAs overtake it: with up to two stages where an SM holds fewer than
-// two chains (107 KB 2.3 ms and 2.9, 133 KB 3.7 and 3.2, 166 KB 4.9 and 4.3), with more where it holds fewer than three (four
-// stages 72 KB 1.82 and 1.83, 107 KB 2.61 and 2.52; eight stages 54 KB 1.94 and 1.85, 81 KB 2.6 and 2.2, 161 KB 5.4 and 3.1).
+// 200 steps: 63 KB 3.4 ms and 4.2 for the next best kernel, 93 KB 4.0 and 5.4, 118 KB 8.4 and 23).  Else the attention of a shard's slots
+// is looked up (8*K + 18*R*G*S bytes more, S stages a move) and a chain's rounds are longer: with up to two stages where an SM holds two
+// chains, with more where it holds three.  The same search with shards of two slots, below the line and beyond it: two stages 61 KB
+// 4.0 and 4.9, 109 KB 5.9 and 19, beyond 130 KB 11.8 and 24; four stages 43 KB 1.3 and 2.2, 66 KB 3.0 and 3.4, beyond 86 KB 6.6 and 5.8,
+// 107 KB 6.7 and 7.8; eight stages 54 KB 1.5 and 2.8, beyond 79 KB 2.64 and 2.68, 108 KB 7.7 and 7.2.  (The line was drawn by an
+// earlier form of the kernel, which fell behind there; today's is about even for some way beyond.)
 bool rp_row_fits_level(const rp_ctx *c, const RpBlob &bl, const RpStatic &sl)
 {
     RowArgs X;

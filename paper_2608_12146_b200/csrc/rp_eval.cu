@@ -572,13 +572,14 @@ static size_t eval_smem_bytes(const RpDims &dm)
     return (eval_finish_bytes(dm) + sizeof(int) * (2 * (size_t)dm.RG + 1 + dm.N) + 15) & ~(size_t)15;
 }
 
-// Whether n layouts take the few-layouts form.  It has a cluster per row-shard and layout, which scans the whole assignment: per CTA
-// about 6 ns and a nanosecond for 300 samples, with the rows served less evenly (0.3 ns for 1000 counts).  The other form groups
-// an assignment once, but in one CTA, and streams through a row-shard with one warp: 9 us more for its launches, and the longer
-// a row-shard, the more, up to 30 us.  In us, few and many: 512 samples in 32 row-shards, 16 layers of 8 ranks, n = 8 30 and 28,
-// 64 40 and 30, 512 157 and 45; 2048 in 240, 24 of 16, n = 3 33 and 35, 8 47 and 35, 64 193 and 58; 4000 in 6, 16 of 8, n = 64
-// 100 and 135, 512 258 and 166; 30000 in 160, n = 1 110 and 146, 8 504 and 150.  One layout: 8192 in 448 56 and 57, 4000 in 2000
-// 76 and 44.
+// Whether n layouts take the few-layouts form.  It has a cluster per row-shard and layout, which scans the whole assignment; the other
+// form groups an assignment once, but in one CTA, and streams through a row-shard with one warp: more launches, and slow where
+// row-shards are long.  Calls in us, few and many: 512 samples in 32 row-shards, 16 layers of 8 ranks, n = 8 36.8 and 41.8, 40 41.3 and
+// 42.4, 64 49.0 and 42.4, 512 204 and 64; 2048 in 240, 24 of 16, n = 4 37.6 and 51.1, 8 46.8 and 51.2, 64 171 and 77; 4000 in 6, 16 of
+// 8, n = 128 147 and 276, 512 307 and 336; 30000 in 160, n = 1 79 and 363, 8 516 and 373.  One layout: 8192 in 448 47.6 and 94, 4000 in
+// 2000 44.5 and 50.7, 8000 in 1920 51.6 and 69.3.  The line was drawn for an earlier few-layouts kernel (per CTA 6 ns and a nanosecond for 300
+// samples, rows served less evenly, 0.3 ns for 1000 counts, against 9 us of launches and up to 30 us of a long row-shard); today's is still
+// ahead somewhat above it (2048 samples, n = 6 44.8 and 51.1; 4000 in 6, n = 300 220 and 301; 30000, n = 3 141 and 376).
 static bool eval_is_few(const RpDims &dm, int n)
 {
     if ((dm.P & 3) || n >= 65536 || dm.RG >= 65536 || dm.LP > 16384 || eval_few_smem(dm, 8) > EVAL_SMEM_MAX) return false;
