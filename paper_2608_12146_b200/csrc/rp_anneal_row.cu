@@ -14,7 +14,7 @@
 //    the named windows: all but 1e-4 of the rejections); with four routing mixes an eighth to a third
 //    is.  A candidate that is not rejected by its bound is scored exactly.  The bound is worked out in single precision with an
 //    allowance for its roundings: in 64-bit integers it was a third of a round's instructions (with the decision shared by two
-//    lanes: heavy 89.2 -> 81.4 ms, wide 8.22 -> 8.04, medium 0.87 -> 0.84).
+//    lanes, heavy 1.10 times as fast, wide 1.02, medium 1.04).
 //  * Rows in registers.  A lane holds whole layers (layer = lane, lane + 32, ...) of the two slices and the two
 //    demand rows, or, one launch per level with rows of two or four chunks a layer, the chunks are dealt out to the lanes in turn and
 //    a layer's maximum meets in shuffles: 16-byte loads, one trip, no staging; the new slices are stored from the

@@ -5,8 +5,9 @@
 // samples of a cell in 8), its score, energy and trajectory best in registers; both sides of a move look at their entries once, for
 // the decision and the commit; a slice table entry carries where the next rewrite goes; what leaves a best layout behind copies it,
 // not what finds it; windows whose slot d is shard d have instances of their own.  In cycles, alone on an SM (medium): proposals 874 ->
-// 503, scoring 934 -> 740, decision 467 -> 378, commit 902 -> 566; plans 1.12 times as fast (medium 835 -> 719 us, large 2.86 -> 2.47
-// ms, wide 8.9 -> 7.6, heavy 76.0 -> 65.4, two shards 1144 -> 1023 us, ragged 1622 -> 1551).
+// 503, scoring 934 -> 740, decision 467 -> 378, commit 902 -> 566; plans 1.12 times as fast.  With the barrier, the dealt-out rows and
+// the shared warps below: medium 972 -> 807 us, large 3169 -> 2499, two shards 916 -> 816, ragged 1781 -> 1570, wide 10.9 -> 9.8 ms, heavy
+// 83.4 -> 59.3 (windows of perf/cases.py, seed 5, one GPU; times below without a window's sizes are of these).
 #pragma once
 #include <string.h>
 
@@ -239,8 +240,8 @@ __device__ __forceinline__ i64 row_energy(i64 s0, i64 s1, i64 s2)       // rp_en
 }
 
 // The level barrier of up to 32 members by one warp, a member a lane: incumbent (inc, *win = its slot or -1), then, unless this
-// was the last level, ancestors of members m0 .. m1-1.  No CTA-wide barrier between its parts (tiny 333 -> 308 us a plan); with
-// eight members a lane one warp takes longer than eight do with their barriers (medium 913 -> 978 us).
+// was the last level, ancestors of members m0 .. m1-1.  No CTA-wide barrier between its parts (8 % of a tiny plan); with
+// eight members a lane one warp takes longer than eight do with their barriers (7 % of medium's).
 __device__ __forceinline__ void row_barrier_warp(const AnnealArgs &A, int P, const u64 *eL, const i64 *bestL, bool last, u64 cq, u32 resample_x,
                                                  int m0, int m1, i64 *inc, int *win, int *anc, int lane)
 {
@@ -287,8 +288,8 @@ __device__ __forceinline__ void row_barrier_warp(const AnnealArgs &A, int P, con
 // GL lanes run a chain, LPL layers per lane, CPL 16-byte chunks per layer (X.cpl <= CPL of them in use).  IDENT: slot d is shard d.
 // SPLIT (X.cpl = 2 or 4): the row's chunks are dealt out to the lanes in turn instead, CPL of them to a lane, and a layer's maximum
 // meets in shuffles: a load touches consecutive bytes, and no lane is idle for want of layers.  Whole layers of four chunks put the
-// lanes of a load 64 bytes apart, twelve lines for 24 layers, eight stores 440 cycles (large 2563 -> 2396 us, with candidates 3377 ->
-// 3303).  With the rank loads on chip only the demand rows would gain, and the shuffles cost as much (two shards 1190 and 1225 us).
+// lanes of a load 64 bytes apart, twelve lines for 24 layers, eight stores 440 cycles (large 2662 us, dealt out 2499; with candidates
+// 3023 and 2999).  With the rank loads on chip only the demand rows would gain, and the shuffles cost more (3 % of two shards).
 template <int GL, int LPL, int CPL, bool SPLIT, bool CHIP, bool COMP, bool IDENT>
 __global__ void __launch_bounds__(CHIP ? ROW_THREADS : 32, CHIP ? 1 : ROW_WARPS_PER_SM(GL, LPL, CPL, IDENT))
 k_anneal_row(const AnnealArgs A, const RowArgs X)
@@ -638,8 +639,9 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                             w1[u] = W1[c]; w2[u] = W2[c];
                         }
                     }
-                    // Under the rows' loads where all levels run in one launch (medium 822 us ahead of them, 802 here); behind the sums
-                    // with one launch per level, whose chains share the SM's load path (ahead or here: wide 10.6 ms, heavy 79 ms; behind 8.5 and 64).
+                    // Under the rows' loads where all levels run in one launch (medium 818 us ahead of them, 807 here; two shards 828 and
+                    // 816); behind the sums with one launch per level, whose chains share the SM's load path (wide and heavy a quarter slower
+                    // ahead of the loads or here).
                     if (CHIP) look();
                     unsigned over = 0;                      // COMP: layers of this lane whose other ranks may be the busiest
                     constexpr int NM = SPLIT ? CPL : LPL, PER = NCH / NM;
@@ -913,7 +915,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
             if (win_s >= 0) inc_slot = win_s;
         } else if (P <= NT) {
             // A member a thread: energies meet once, warps' weights once, and an ancestor is a count over the threads (five more
-            // meetings of the CTA and a search of eight dependent steps before: medium 810 us, now 789; two shards 1188 and 1175).
+            // meetings of the CTA and a search of eight dependent steps as below: medium 849 us, here 807; two shards 859 and 816).
             const u64 r = tid < P ? __ldcg(eL + tid) : ~0ull >> 1;
             i64 e[1] = { (i64)(r & ~(1ull << 63)) };
             i64 b0 = 0, b1 = 0, b2 = 0;
