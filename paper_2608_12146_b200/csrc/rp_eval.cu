@@ -447,7 +447,7 @@ k_eval_few(const EvalArgs A)
     for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
     if (lane == 0 && es) atomicAdd(&es_s, (u64)es);
     // Statistics of all of the cluster's samples meet in its first CTA: a lane there for every CTA of a slot, which fetches; more slots
-    // than it has lanes for are added to it from afar (diagnostics of 6000 samples in four row-shards of 64 slots 56 us fetched).
+    // than it has lanes for are added to it from afar (diagnostics of 6000 samples in four row-shards of 256 slots 56.5 us fetched, 55 so).
     if (dm.D * MS <= EVAL_THREADS) {
         if (ms == 0 && MS > 1) {
             const int d = tid / MS, x = tid & (MS - 1);

@@ -1837,7 +1837,7 @@ def test_two_chains_that_take_more_than_half_an_sm_each(D, R):
     rp.rp_destroy(ctx)
 
 
-@pytest.mark.parametrize("pop", [2, 307, 308])
+@pytest.mark.parametrize("pop", [2, 303, 304, 307, 308])
 def test_selection_with_its_distances_on_chip_and_not(pop):
     """The greedy order where all distances of the candidates just fit on chip, and with one candidate more."""
     w = make_window(custom_spec("greedy", 60, 5, 16, 2, 4096, 3, 4, pop, 0, data_seed=3))
