@@ -4,106 +4,81 @@
 // The samples are sorted by (-t_i, i) (by counting on the whole GPU, small and very large windows with a bitonic sort
 // on 64-bit keys in the packing CTA), then for
 // R = R_lb, R_lb+1, ... first-fit-decreasing is tried into K = R*D cells: the K longest
-// samples open the cells, each later sample goes to the lowest-numbered cell it still fits
-// in.  The fit search is done by one warp, 32 cells per ballot.
+// samples open the cells, each later sample goes to the lowest-numbered cell it still fits in (first_fit_flow).
 #include "rp_common.cuh"
 
 #define PACK_THREADS 1024
-#define FFD_MAX_CELLS 4096
+#define FLOW_PHASE 8                  // cells between two meetings of the warps
+#define FLOW_LAG (32 / FLOW_PHASE + 1)
+#define FLOW_GONE 0x40000000u         // a sample that has found its cell, with the cell below (no cell has as much left)
+#define FLOW_FEW 5120                 // samples up to which a lane holds eight of them, not sixteen
+#define FLOW_PAD 48                   // zeros behind the capacities: the cells a warp's lanes see behind the last one
 
-// First fit of the samples keys[K..N) into K <= 1024*E cells by one warp, a run of samples at a time.
+// First fit of 32*G samples a warp, in decreasing order over the lanes and warps, into K cells of `rest` (what is left of each; FLOW_PAD
+// zeros behind them), the lowest cell first.
 //
-// Lane w keeps the largest remaining capacity of block w (32*E consecutive cells): a ballot finds the block, a second one
-// the cell c that takes the next sample.  M, the largest remaining capacity below c, is what rejected it.  The samples
-// behind it are no longer than it; they go to c as well as long as they are longer than M (no lower cell takes them) and
-// fit after the ones before (prefix sums of the lengths, worked out once per 32 samples): one ballot gives the length of
-// the run, and only then does a cell change.  Bound by the chain of warp-wide operations: about 440 cycles a run (38 runs
-// for the 42 samples behind the first of a 64-sample window, 619 for 1808 at 2048, 349 for 8144 at 8192) instead of 170 to
-// 250 a sample: 2048 samples in 270 k cycles, 4096 in 374 k (639 k with a tree of maxima searched by 32 samples at once,
-// which placed 7 to 28 samples in 1800 cycles; 487 k and 393 k at 2048 and 8192, now 270 k and 228 k).
-template <int E>
-__device__ __forceinline__ bool first_fit_runs(const RpDims &dm, const u64 *keys, int *rem, int *cell_of, int K, int lane)
+// Which samples a cell takes depends on nothing but the samples that no lower cell has taken, so the samples are a pipeline that the
+// cells run through: a lane holds G consecutive samples, the capacity of a cell moves from lane to lane with one shuffle a step, and
+// a sample that is taken keeps the cell's number in place of its length.  Between warps a cell goes through `rest` itself: warp w starts
+// FLOW_LAG phases behind warp w-1, whose last lane has written a cell 31 steps after the first has read it.  About 100 cycles a step
+// with eight samples a lane and 180 with sixteen (their chain of subtractions and minima, the shuffle), for N/G + K steps and the
+// lags, whatever the lengths are; in cycles, 8 and 16 samples a lane: 512 samples in 72 cells 12 k and 15 k, 2048 in 240 56 k
+// and 56 k, 4096 in 288 100 k and 112 k, 8192 in 48 120 k and 100 k.  (Samples that move through lanes of cells need a shuffle for every
+// sample: 32 k, 97 k, 206 k and 261 k.  One warp that placed a run of samples at a time, before: 440 cycles a run, 270 k, 374 k and 228 k
+// for the last three.)
+template <int G>
+__device__ __forceinline__ void first_fit_flow(u32 (&x)[G], u32 *rest, int K, int warp, int n_warps, int lane)
 {
-    // rem[32*32*E]: remaining capacities, -1 past the last cell
-    int bm = -1;
-    for (int x = 0; x < 32 * E; ++x) bm = max(bm, rem[lane * 32 * E + x]);
-    for (int x0 = K; x0 < dm.N; x0 += 32) {
-        const int nb = min(32, dm.N - x0);
-        const u64 key = lane < nb ? keys[x0 + lane] : 0;
-        const int len = lane < nb ? dm.C - (int)(key >> 32) : 0, id = (int)(u32)key;
-        u32 pre = (u32)len;                         // at most 32*C, C <= 2^24
+    const int phases = (K + 31 + FLOW_PHASE - 1) / FLOW_PHASE, all = phases + FLOW_LAG * (n_warps - 1);
+    u32 r = 0;
+    for (int ph = 0; ph < all; ++ph) {
+        const int p = ph - FLOW_LAG * warp;
+        if (p >= 0 && p < phases) {
+            u32 in[FLOW_PHASE];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const u32 y = __shfl_up_sync(0xffffffffu, pre, o); if (lane >= o) pre += y; }
-        int p = 0;
-        while (p < nb) {
-            const int ts = __shfl_sync(0xffffffffu, len, p);
-            const u32 base = __shfl_sync(0xffffffffu, pre, p) - (u32)ts;
-            const unsigned m = __ballot_sync(0xffffffffu, bm >= ts);
-            if (!m) return true;                    // the sample fits nowhere
-            const int w = __ffs(m) - 1;
-            int v[E];
-            if (E == 1) v[0] = rem[w * 32 + lane];
-            else {
-                const int4 q = ((const int4 *)rem)[w * 32 + lane];
-                v[0] = q.x; v[E > 1 ? 1 : 0] = q.y; v[E > 2 ? 2 : 0] = q.z; v[E > 3 ? 3 : 0] = q.w;
+            for (int u = 0; u < FLOW_PHASE; u += 4) {
+                const uint4 v = *(const uint4 *)(rest + p * FLOW_PHASE + u);
+                in[u] = v.x; in[u + 1] = v.y; in[u + 2] = v.z; in[u + 3] = v.w;
             }
-            int big = v[0];
 #pragma unroll
-            for (int e = 1; e < E; ++e) big = max(big, v[e]);
-            const int i = __ffs(__ballot_sync(0xffffffffu, big >= ts)) - 1;
-            // first cell of lane i that takes it, what is left there, and the largest before it
-            int f = E - 1, rc = 0, low = 0;
+            for (int u = 0; u < FLOW_PHASE; ++u) {
+                const int c = p * FLOW_PHASE + u;                       // lane 0 has cell c, the others the cells before it
+                const u32 y = __shfl_up_sync(0xffffffffu, r, 1), tag = FLOW_GONE + (u32)(c - lane);
+                r = lane ? y : in[u];
 #pragma unroll
-            for (int e = E - 1; e >= 0; --e) if (v[e] >= ts) f = e;
-#pragma unroll
-            for (int e = 0; e < E; ++e) { if (e == f) rc = v[e]; if (e < f) low = max(low, v[e]); }
-            rc = __shfl_sync(0xffffffffu, rc, i);
-            const unsigned below = (unsigned)max(lane < w ? bm : 0, lane < i ? max(big, 0) : (lane == i ? low : 0));
-            const int M = (int)__reduce_max_sync(0xffffffffu, below);
-            const bool in = lane < nb && len > M && pre - base <= (u32)rc;
-            const unsigned out = __ballot_sync(0xffffffffu, lane > p && !in);      // p itself is always placed
-            const int e1 = out ? __ffs(out) - 1 : 32;           // the run is p .. e1-1
-            const int used = (int)(__shfl_sync(0xffffffffu, pre, e1 - 1) - base);
-            const int ff = E == 1 ? 0 : __shfl_sync(0xffffffffu, f, i);
-            if (lane >= p && lane < e1) cell_of[id] = (w * 32 + i) * E + ff;
-            if (lane == i) {
-#pragma unroll
-                for (int e = 0; e < E; ++e) if (e == f) { v[e] = rc - used; rem[(w * 32 + i) * E + e] = v[e]; }
+                for (int k = 0; k < G; ++k) {
+                    const u32 left = r - x[k];                          // (more than r where it does not fit)
+                    x[k] = x[k] <= r ? tag : x[k];
+                    r = min(r, left);
+                }
+                if (lane == 31 && c >= 31 && c - 31 < K) rest[c - 31] = r;
             }
-            big = v[0];
-#pragma unroll
-            for (int e = 1; e < E; ++e) big = max(big, v[e]);
-            const int nm = __reduce_max_sync(0xffffffffu, big);
-            if (lane == w) bm = nm;
-            __syncwarp();
-            p = e1;
         }
+        if (n_warps > 1) asm volatile("bar.sync 1, %0;" ::"r"(32 * n_warps) : "memory");
     }
-    return false;
 }
 
-__device__ __forceinline__ bool first_fit_smem(const RpDims &dm, const u64 *keys, int *fill, int *cell_of, int K, int B, int tid)
+// The samples behind the K longest, as many at a time as the CTA's lanes hold; whether one of this thread's has found no cell.
+template <int G>
+__device__ __forceinline__ bool first_fit(const RpDims &dm, const u64 *keys, u32 *rest, int *cell_of, int K, int tid, int nt)
 {
-    const int b0 = tid * B, b1 = min(K, b0 + B);
-    int blockmax = -1;
-    for (int b = b0; b < b1; ++b) blockmax = max(blockmax, dm.C - fill[b]);
-    for (int x = K; x < dm.N; ++x) {
-        const u64 key = keys[x];
-        const int ts = dm.C - (int)(key >> 32);
-        const unsigned m = __ballot_sync(0xffffffffu, blockmax >= ts);
-        if (!m) return true;
-        if (tid == __ffs(m) - 1) {
-            int found = -1, nm = -1;
-            for (int b = b0; b < b1; ++b) {
-                int rem = dm.C - fill[b];
-                if (found < 0 && rem >= ts) { found = b; rem -= ts; fill[b] += ts; }
-                nm = max(nm, rem);
+    bool left = false;
+    for (int b = K; b < dm.N; b += nt * G) {
+        const int n_warps = (min(dm.N - b, nt * G) + 32 * G - 1) / (32 * G), first = b + tid * G;
+        if (b > K) __syncthreads();                                     // the cells as the samples before have left them
+        if (tid >> 5 >= n_warps) continue;
+        u32 x[G];
+#pragma unroll
+        for (int k = 0; k < G; ++k) x[k] = first + k < dm.N ? max(1u, (u32)dm.C - (u32)(keys[first + k] >> 32)) : FLOW_GONE;
+        first_fit_flow<G>(x, rest, K, tid >> 5, n_warps, tid & 31);
+#pragma unroll
+        for (int k = 0; k < G; ++k)
+            if (first + k < dm.N) {
+                left |= x[k] < FLOW_GONE;
+                cell_of[(u32)keys[first + k]] = (int)(x[k] - FLOW_GONE);
             }
-            blockmax = nm;
-            cell_of[(u32)key] = found;
-        }
     }
-    return false;
+    return left;
 }
 
 // Packing runs beside the checks of the window: lengths outside [1, C] are still possible (the window is then refused).
@@ -138,13 +113,13 @@ k_pack_rank(RpDims dm, const int *__restrict__ t, u64 *__restrict__ keys, int *_
 }
 
 __global__ void __launch_bounds__(PACK_THREADS)
-k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *keys_g, int n_pow2,
-           int *__restrict__ fill_g, int *__restrict__ cell_of, int *__restrict__ out, int *__restrict__ order_out, const u64 *sorted)
+k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *keys_g, int n_pow2, u32 *rest_g,
+           int *__restrict__ cell_of, int *__restrict__ out, int *__restrict__ order_out, const u64 *sorted)
 {
     extern __shared__ __align__(16) u64 keys_s[];
-    u64 *keys = keys_g ? keys_g : keys_s;
-    int *fill = fill_g ? fill_g : (int *)(keys_s + (keys_g ? 0 : n_pow2));
-    int *rem = fill;                               // remaining capacities (cells of the run-at-a-time form), else fills
+    u64 *sort = keys_g ? keys_g : keys_s;
+    const u64 *keys = sorted ? sorted : sort;
+    u32 *rest = rest_g ? rest_g : (u32 *)(keys_s + (sorted ? 0 : n_pow2));           // what is left of the cells
     __shared__ i64 total_s;
     __shared__ int fail_s;
     const int tid = threadIdx.x, nt = (int)blockDim.x;
@@ -153,11 +128,11 @@ k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *keys_g, int 
     i64 part = 0;
     for (int i = tid; i < n_pow2; i += nt) {
         if (i < dm.N) {
-            part += t[i];
-            const int ti = pack_len(dm, t[i]);
-            keys[i] = sorted ? sorted[i] : ((u64)(u32)(dm.C - ti) << 32) | (u32)i;     // ascending = longest first, then id
-        } else {
-            keys[i] = ~0ull;
+            const int ti = t[i];
+            part += ti;
+            if (!sorted) sort[i] = ((u64)(u32)(dm.C - pack_len(dm, ti)) << 32) | (u32)i;     // ascending = longest first, then id
+        } else if (!sorted) {
+            sort[i] = ~0ull;
         }
     }
     for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
@@ -174,9 +149,9 @@ k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *keys_g, int 
             for (int i = tid; i < n_pow2; i += nt) {
                 int ixj = i ^ j;
                 if (ixj > i) {
-                    u64 a = keys[i], b = keys[ixj];
+                    u64 a = sort[i], b = sort[ixj];
                     bool up = ((i & k) == 0);
-                    if ((a > b) == up) { keys[i] = b; keys[ixj] = a; }
+                    if ((a > b) == up) { sort[i] = b; sort[ixj] = a; }
                 }
             }
             __syncthreads();
@@ -185,7 +160,7 @@ k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *keys_g, int 
             // all remaining distances of this k (and, while k <= 32, of the following k as well)
             u64 r[SORT_E];
 #pragma unroll
-            for (int m = 0; m < SORT_E; ++m) { const int i = m * nt + tid; r[m] = i < n_pow2 ? keys[i] : ~0ull; }
+            for (int m = 0; m < SORT_E; ++m) { const int i = m * nt + tid; r[m] = i < n_pow2 ? sort[i] : ~0ull; }
             int kk = k;
             for (;;) {
                 for (int jj = min(kk >> 1, 16); jj > 0; jj >>= 1) {
@@ -204,7 +179,7 @@ k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *keys_g, int 
             }
             k = kk;
 #pragma unroll
-            for (int m = 0; m < SORT_E; ++m) { const int i = m * nt + tid; if (i < n_pow2) keys[i] = r[m]; }
+            for (int m = 0; m < SORT_E; ++m) { const int i = m * nt + tid; if (i < n_pow2) sort[i] = r[m]; }
             __syncthreads();
         }
     }
@@ -218,21 +193,13 @@ k_pack_ffd(RpDims dm, const int *__restrict__ t, int min_rows, u64 *keys_g, int 
         const int K = (int)(R * dm.D);
         if (tid == 0) fail_s = 0;
         // the K longest samples open the cells
-        for (int x = tid; x < K; x += nt) {
-            const u64 key = keys[x];
-            if (K > FFD_MAX_CELLS) fill[x] = dm.C - (int)(key >> 32);
-            else rem[x] = (int)(key >> 32);                          // what is left of the cell
-            cell_of[(u32)key] = x;
+        for (int x = tid; x < K + FLOW_PAD; x += nt) {
+            const u64 key = x < K ? keys[x] : 0;
+            rest[x] = (u32)(key >> 32);
+            if (x < K) cell_of[(u32)key] = x;
         }
-        if (K <= FFD_MAX_CELLS) for (int x = K + tid; x < (K <= 1024 ? 1024 : FFD_MAX_CELLS); x += nt) rem[x] = -1;
         __syncthreads();
-        if (tid < 32) {
-            // First fit = the lowest cell whose remaining capacity takes the sample.
-            const bool failed = K > FFD_MAX_CELLS ? first_fit_smem(dm, keys, fill, cell_of, K, (K + 31) / 32, tid)
-                              : K <= 1024 ? first_fit_runs<1>(dm, keys, rem, cell_of, K, tid)
-                                          : first_fit_runs<4>(dm, keys, rem, cell_of, K, tid);
-            if (failed && tid == 0) fail_s = 1;
-        }
+        if (dm.N - K <= FLOW_FEW ? first_fit<8>(dm, keys, rest, cell_of, K, tid, nt) : first_fit<16>(dm, keys, rest, cell_of, K, tid, nt)) fail_s = 1;
         __syncthreads();
         if (!fail_s) Rstar = (int)R;
         __syncthreads();
@@ -252,15 +219,6 @@ int rp_launch_pack_on(rp_ctx *c, cudaStream_t stream)
     const RpDims &dm = c->dm;
     int n_pow2 = 1;
     while (n_pow2 < dm.N) n_pow2 <<= 1;
-    // sort keys (8 bytes each) and cell fills (4 bytes per cell: at most N cells, or the padded blocks of the run-at-a-time
-    // form) on chip when they fit
-    const size_t fills = dm.N > (dm.N <= 1024 ? 1024 : FFD_MAX_CELLS) ? dm.N : (dm.N <= 1024 ? 1024 : FFD_MAX_CELLS);
-    size_t smem = (size_t)n_pow2 * sizeof(u64) + fills * sizeof(int);
-    u64 *keys_g = nullptr;
-    int *fill_g = nullptr;
-    if (smem > 160 * 1024) { keys_g = c->d_sort_keys; fill_g = (int *)(c->d_sort_keys + n_pow2); smem = 0; }
-    if (smem > 32 * 1024)
-        RP_CUDA(cudaFuncSetAttribute(k_pack_ffd, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT));
     // small windows: fewer warps make the block-wide barriers of the sort cheaper
     const int threads = n_pow2 >= PACK_THREADS ? PACK_THREADS : (n_pow2 < 256 ? 256 : n_pow2);
     // The order by counting on the whole GPU from 513 samples (below, the sort in the packing kernel is cheaper than a
@@ -273,7 +231,15 @@ int rp_launch_pack_on(rp_ctx *c, cudaStream_t stream)
         ++g_rp_launches;
         sorted = c->d_sort_keys;
     }
-    k_pack_ffd<<<1, threads, smem, stream>>>(dm, c->d_t, c->cfg.min_rows, keys_g, n_pow2, fill_g,
+    // On chip where they fit: the keys to sort (8 bytes each) and what is left of the cells (4; at most as many as samples).  Beyond,
+    // in the two halves of the scratch.
+    size_t smem = (sorted ? 0 : (size_t)n_pow2 * sizeof(u64)) + sizeof(u32) * ((size_t)dm.N + FLOW_PAD);
+    u64 *keys_g = nullptr;
+    u32 *rest_g = nullptr;
+    if (smem > 160 * 1024) { keys_g = c->d_sort_keys; rest_g = (u32 *)(c->d_sort_keys + n_pow2); smem = 0; }
+    if (smem > 32 * 1024)
+        RP_CUDA(cudaFuncSetAttribute(k_pack_ffd, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT));
+    k_pack_ffd<<<1, threads, smem, stream>>>(dm, c->d_t, c->cfg.min_rows, keys_g, n_pow2, rest_g,
                                                     c->d_seed_layout, (int *)(c->h_pin + 10), c->d_order, sorted);
     ++g_rp_launches;
     RP_CUDA(cudaGetLastError());

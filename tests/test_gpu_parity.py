@@ -1855,3 +1855,23 @@ def test_selection_with_its_distances_on_chip_and_not(pop):
     dist = rp.rp_debug_dump(ctx, "SELECT_DIST", (pop, pop), np.int64)
     assert dist.min() >= 0 and dist.max() <= 1 << 22             # (kept in 32 bits on chip)
     rp.rp_destroy(ctx)
+
+
+# Samples behind the first of each cell: none, one warp of eight a lane filled and one more, both sides of where a lane holds sixteen
+# (5120), a CTA of sixteen a lane filled (16384) and one more; cells on both sides of eight to a phase, and of 31 behind the last; more
+# cells than samples behind them; five and ten attempts before a row count that fits.
+@pytest.mark.parametrize("N,D,min_rows,cap,longest", [
+    (12, 4, 3, 50, 50), (257, 1, 0, 1 << 20, 1000), (264, 8, 1, 4096, 60), (265, 8, 0, 4096, 60), (5160, 8, 5, 1 << 16, 300),
+    (5161, 8, 5, 1 << 16, 300), (16424, 8, 5, 1 << 20, 500), (16425, 8, 5, 1 << 20, 500), (36000, 3, 0, 1 << 20, 900),
+    (900, 31, 0, 700, 400), (1500, 33, 40, 700, 30), (700, 3, 0, 100, 67), (333, 2, 0, 1000, 520), (2600, 1100, 0, 90, 61)])
+def test_first_fit_at_the_edges_of_its_warps(N, D, min_rows, cap, longest):
+    rng = np.random.default_rng(N + D)
+    t = rng.integers(longest // 2 if longest in (67, 61, 520) else 1, longest + 1, N).astype(np.int32)
+    a = np.zeros((N, 1, 2), np.int32)
+    a[np.arange(N), 0, rng.integers(0, 2, N)] = t
+    R, cert, seed = oracle.pack_ffd(t, cap, D, min_rows)
+    ctx = rp.rp_window_load(t, a, top_k=1, token_cap=cap, dp_width=D, ep_width=2, pop_size=2, min_rows=min_rows)
+    rp.rp_place_experts(ctx)
+    assert rp.rp_pack_rows(ctx) == (R, cert)
+    assert (rp.rp_debug_dump(ctx, "SEED_LAYOUT", (N,), np.int32) == seed).all()
+    rp.rp_destroy(ctx)
