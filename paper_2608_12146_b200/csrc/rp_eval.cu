@@ -6,8 +6,9 @@
 //  * few layouts of rows in whole 16-byte chunks (k_eval_few: the seed, the incumbent, diagnostics, small batches), bound by latency: a cluster of
 //    CTAs per row-shard, each over its share of the samples, sixteen 16-byte loads in flight per lane; the CTAs'
 //    sums meet through distributed shared memory;
-//  * many layouts (k_eval_group, k_eval_sum, k_eval_score), bound by L2: the samples of a layout are grouped by row-shard once, then
-//    a warp per row-shard sums its rows, sixteen bytes per lane and eight to twelve loads in flight.
+//  * many layouts (k_eval_group, k_eval_slice or k_eval_sum, k_eval_score): the samples of a layout are grouped by row-shard once; then a
+//    CTA keeps a slice of all samples' rows on chip and adds up the row-shards of many layouts from there (bound by shared memory), or,
+//    where such a slice does not fit, warps stream through the rows in L2.
 // In the first the cluster that finishes a layout last (atomic ticket) scores it.
 #include <cooperative_groups.h>
 
@@ -42,10 +43,10 @@ struct EvalArgs {
     double *f64_final;
     int n;
     bool q_halves;                                // (few layouts) no cell's squared lengths add up to 2^48, whatever the layout
-    i64 *Esum;                                    // [n][RG] row-shard sums (few layouts: costs) handed to the finishing CTA; zero between launches
-    int *tickets;                                 // [n] arrival counters; zero between launches
+    i64 *cost;                                    // [n][RG] row-shard costs handed to the finishing CTA; zero between launches
+    int *tickets;                                 // [n] arrival counters (many layouts: whether a cell is empty or overfull); zero between launches
     unsigned short *list;                         // [n][N] samples grouped by row-shard (k_eval_group)
-    int *off;                                     // [n][RG+1]
+    u32 *off;                                     // [n][RG+1] where a row-shard's samples start, and in the upper half which row-shard it is
     // Validation of the incumbent: with `host` set (pinned), the finishing CTA leaves the search's counters, the status
     // words, the incumbent's cached score, its full score, the best seed's and its layout there.
     i64 *host;
@@ -73,101 +74,6 @@ __device__ __forceinline__ int eval_cell(const EvalArgs &A, const EvalCells &e, 
     return 0;
 }
 
-// Shared memory of the finishing CTA.
-struct EvalFinish { u64 *Q; i64 *Esum, *Afx, *U; int *T, *cnt; unsigned short *cell_of; };
-__host__ __device__ static inline size_t eval_finish_bytes(const RpDims &dm)
-{
-    return (sizeof(u64) * dm.K + sizeof(i64) * (2 * (size_t)dm.RG + dm.G) + sizeof(int) * 2 * (size_t)dm.K + 2 * (size_t)dm.N + 15) & ~(size_t)15;
-}
-__device__ __forceinline__ EvalFinish eval_finish_views(const RpDims &dm, unsigned char *sm)
-{
-    EvalFinish f;
-    f.Q = (u64 *)sm;
-    f.Esum = (i64 *)(f.Q + dm.K);
-    f.Afx = f.Esum + dm.RG;
-    f.U = f.Afx + dm.RG;
-    f.T = (int *)(f.U + dm.G);
-    f.cnt = f.T + dm.K;
-    f.cell_of = (unsigned short *)(f.cnt + dm.K);
-    return f;
-}
-
-// Scores layout `lay` once its row-shard sums are complete.  All threads of one CTA call; cell_of is in place.
-__device__ __forceinline__ void eval_finish(const EvalArgs &A, int lay, const EvalFinish &f, int tid)
-{
-    const RpDims &dm = A.dm;
-    const int lane = tid & 31;
-    i64 *eg = A.Esum + (size_t)lay * dm.RG;
-    for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS) { f.Esum[rg] = __ldcg(eg + rg); eg[rg] = 0; }
-    for (int c = tid; c < dm.K; c += EVAL_THREADS) { f.T[c] = 0; f.Q[c] = 0; f.cnt[c] = 0; }
-    __syncthreads();
-    RpSmemState st = { f.cell_of, f.T, f.Q, f.cnt, f.Esum, f.Afx, f.U };
-    rp_accumulate_cells(dm, st, A.t, tid, EVAL_THREADS);
-    __syncthreads();
-    for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS)
-        f.Afx[rg] = rp_attention(dm, st, A.dp_list, A.dp_off, rg / dm.G, rg % dm.G, -1, 0, 0, -1, 0, 0);
-    __syncthreads();
-    for (int g = tid; g < dm.G; g += EVAL_THREADS) {
-        i64 u = 0;
-        for (int r = 0; r < dm.R; ++r) u += f.Afx[r * dm.G + g] + dm.EC * f.Esum[r * dm.G + g];
-        f.U[g] = u;
-    }
-    __syncthreads();
-    char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
-    if (A.host) {          // coverage is checked by the caller's `bad` flag: every sample sits in one cell by construction
-        int wrong = 0;
-        for (int c = tid; c < dm.K; c += EVAL_THREADS) wrong |= (f.cnt[c] < 1 ? 2 : 0) | (f.T[c] > dm.C ? 4 : 0);
-        wrong = __syncthreads_or(wrong);
-        if (tid < 8) A.host[tid] = A.counters[tid];
-        if (tid < 3) { A.host[16 + tid] = A.inc_score[tid]; A.host[22 + tid] = A.seed_score[tid]; }
-        if (tid < RP_SW_COUNT) ((int *)(A.host + 56))[tid] = A.status[tid] | (tid == RP_SW_VALIDATE && wrong ? 1 : 0);
-        if (A.layout_host) for (int i = tid; i < dm.N; i += EVAL_THREADS) A.layout_host[i] = __ldg(A.lay32 + i);
-    }
-    if (tid < 32) {
-        const bool refused = A.bad_dev && __ldcg(A.bad_dev);
-        i64 s0 = 0, s1 = 0, s2 = 0;
-        for (int g = lane; g < dm.G; g += 32) { const i64 u = f.U[g]; s1 += u; s0 = u > s0 ? u : s0; }
-        for (int rg = lane; rg < dm.RG; rg += 32) { const i64 J = f.Afx[rg] + dm.EC * f.Esum[rg]; s2 = J > s2 ? J : s2; }
-        for (int o = 16; o; o >>= 1) {
-            const i64 a = __shfl_xor_sync(0xffffffffu, s0, o), c = __shfl_xor_sync(0xffffffffu, s2, o);
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            s0 = a > s0 ? a : s0; s2 = c > s2 ? c : s2;
-        }
-        if (lane == 0) {
-            const i64 sc[3] = { s0, s1, s2 };
-            for (int x = 0; x < 3; ++x) {
-                if (refused) continue;
-                if (A.score_out) A.score_out[(size_t)lay * 3 + x] = sc[x];
-                if (A.score_out2) A.score_out2[(size_t)lay * 3 + x] = sc[x];
-                if (A.f64_out) A.f64_out[(size_t)lay * 3 + x] = (double)sc[x] / (double)dm.SC;
-            }
-            if (b) { i64 *S = (i64 *)(b + A.bl.off_S); S[0] = s0; S[1] = s1; S[2] = s2; S[3] = rp_energy(s0, s1, s2); }
-        }
-    }
-    if (!b) return;
-    for (int c = tid; c < dm.K; c += EVAL_THREADS) {
-        ((u64 *)(b + A.bl.off_Q))[c] = f.Q[c];
-        ((int *)(b + A.bl.off_T))[c] = f.T[c];
-        ((int *)(b + A.bl.off_cnt))[c] = f.cnt[c];
-    }
-    for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS) {
-        ((i64 *)(b + A.bl.off_Esum))[rg] = f.Esum[rg];
-        ((i64 *)(b + A.bl.off_Afx))[rg] = f.Afx[rg];
-        ((i64 *)(b + A.bl.off_Jfx))[rg] = f.Afx[rg] + dm.EC * f.Esum[rg];
-        if (A.bl.off_wtab >= 0)        // the pool holds the call's layouts as RG consecutive slices each
-            ((int *)(b + A.bl.off_wtab))[rg] = (A.first + lay) * dm.RG + rg;
-    }
-    for (int g = tid; g < dm.G; g += EVAL_THREADS) ((i64 *)(b + A.bl.off_U))[g] = f.U[g];
-    for (int i = tid; i < dm.N; i += EVAL_THREADS) ((unsigned short *)(b + A.bl.off_cell))[i] = f.cell_of[i];
-}
-
-__device__ __forceinline__ void eval_load_cells(const EvalArgs &A, int lay, unsigned short *cell_of, int tid, int nt)
-{
-    const EvalCells e = eval_cells(A, lay);
-#pragma unroll 4
-    for (int i = tid; i < A.dm.N; i += nt) cell_of[i] = (unsigned short)eval_cell(A, e, i);
-}
-
 // Sum of one 16-byte column of the listed samples' rows, U loads in flight.
 template <int U>
 __device__ __forceinline__ int4 eval_sum_column(const int4 *__restrict__ col, size_t row4, const int *list, int m0, int m1)
@@ -192,49 +98,268 @@ __device__ __forceinline__ int eval_layer_max(int m, int lane, int cpl)      // 
     return m;
 }
 
-// Many layouts, first kernel: the samples of each layout grouped by row-shard (one CTA per layout).
+// Sums of squared lengths in shared memory: 64 bits, or (halves: no sum reaches 2^48) the lower 16 bits of each square and what lies
+// above them added up in 32 bits each.  A 64-bit addition there is a loop, and the samples of a row-shard of few slots meet in it: 4000
+// samples in six row-shards of one slot, 128 layouts 206 us and 147 in halves, one layout 48 and 41.
+__device__ __forceinline__ void few_add(u64 *q, u32 low, u32 high, bool halves)
+{
+    if (halves) { atomicAdd((u32 *)q, low); atomicAdd((u32 *)q + 1, high); }
+    else atomicAdd(q, ((u64)high << 32) | low);
+}
+__device__ __forceinline__ u64 few_square(u64 v, bool halves) { return halves ? ((v >> 32) << 16) + (u32)v : v; }
+__device__ __forceinline__ void few_add_square(u64 *q, int t, bool halves)
+{
+    const u64 sq = (u64)t * (u64)t;
+    if (halves) few_add(q, (u32)sq & 0xffffu, (u32)(sq >> 16), true);
+    else few_add(q, (u32)sq, (u32)(sq >> 32), false);
+}
+
+// Many layouts, first kernel (one CTA per layout): its samples grouped by row-shard, the cells' statistics and from them the
+// attention part of every row-shard's cost.  by_length: the row-shards in order of decreasing sample counts (equal from
+// GROUP_BINS - 1 on), so that those summed side by side are of nearly the same length.
 #define GROUP_THREADS 512
+#define GROUP_BINS GROUP_THREADS
+static inline size_t eval_group_bytes(const RpDims &dm)
+{
+    return (sizeof(u64) * (size_t)dm.K + sizeof(int) * 2 * ((size_t)dm.RG + (size_t)dm.K) + 2 * ((size_t)dm.K + dm.N) + 15) & ~(size_t)15;
+}
 __global__ void __launch_bounds__(GROUP_THREADS)
-k_eval_group(const EvalArgs A)
+k_eval_group(const EvalArgs A, bool by_length)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     const RpDims &dm = A.dm;
-    int *off = (int *)smraw;                                            // [RG] counts, then fill pointers
-    unsigned short *rg_of = (unsigned short *)(off + dm.RG);            // [K]
+    u64 *Q = (u64 *)smraw;                                              // [K] statistics
+    int *T = (int *)(Q + dm.K), *cnt = T + dm.K;
+    int *off = cnt + dm.K;                                              // [RG] counts, then fill pointers
+    int *end = off + dm.RG;                                             // [RG] the same from the other end
+    unsigned short *rg_of = (unsigned short *)(end + dm.RG);            // [K]
     unsigned short *rgs = rg_of + dm.K;                                 // [N]
-    __shared__ int wsum[GROUP_THREADS / 32];
+    __shared__ int wsum[GROUP_THREADS / 32], bins[GROUP_BINS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lay = blockIdx.x;
     for (int x = tid; x < dm.RG; x += GROUP_THREADS) off[x] = 0;
-    for (int c = tid; c < dm.K; c += GROUP_THREADS) rg_of[c] = (unsigned short)rp_rowshard(dm, A.edp, c);
+    for (int c = tid; c < dm.K; c += GROUP_THREADS) { rg_of[c] = (unsigned short)rp_rowshard(dm, A.edp, c); Q[c] = 0; T[c] = 0; cnt[c] = 0; }
+    bins[tid] = 0;
     __syncthreads();
     const EvalCells e = eval_cells(A, lay);
+    char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
 #pragma unroll 4
     for (int i = tid; i < dm.N; i += GROUP_THREADS) {
-        const int rg = rg_of[eval_cell(A, e, i)];
+        const int c = eval_cell(A, e, i), rg = rg_of[c], t = __ldg(A.t + i);
         rgs[i] = (unsigned short)rg;
         atomicAdd(&off[rg], 1);
+        atomicAdd(&T[c], t); atomicAdd(&cnt[c], 1);
+        few_add_square(&Q[c], t, A.q_halves);
+        if (b) ((unsigned short *)(b + A.bl.off_cell))[i] = (unsigned short)c;
     }
     __syncthreads();
-    {   // exclusive prefix sums: a thread takes consecutive row-shards
-        const int chunk = (dm.RG + GROUP_THREADS - 1) / GROUP_THREADS, x0 = min(dm.RG, tid * chunk), x1 = min(dm.RG, x0 + chunk);
-        int sum = 0;
-        for (int x = x0; x < x1; ++x) sum += off[x];
-        int v = sum;
+    u32 *go = A.off + (size_t)lay * (dm.RG + 1);
+    // exclusive sums over the CTA of one number per thread
+    auto before = [&](int own) {
+        int v = own;
         for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += y; }
         if (lane == 31) wsum[warp] = v;
         __syncthreads();
-        int run = v - sum;
+        int run = v - own;
         for (int w = 0; w < warp; ++w) run += wsum[w];
-        int *go = A.off + (size_t)lay * (dm.RG + 1);
-        for (int x = x0; x < x1; ++x) { const int c = off[x]; off[x] = run; go[x] = run; run += c; }
-        if (tid == 0) go[dm.RG] = dm.N;
+        return run;
+    };
+    if (by_length) {
+        // the row-shards of one length lie together, the lengths in decreasing order: where the samples and the row-shards
+        // of a length start (a thread per length)
+        for (int x = tid; x < dm.RG; x += GROUP_THREADS) atomicAdd(&bins[min(off[x], GROUP_BINS - 1)], 1);
+        __syncthreads();
+        const int len = GROUP_BINS - 1 - tid, first = before(bins[len]);
+        __syncthreads();
+        bins[len] = first;
+        __syncthreads();
+        // (a row-shard's place is handed to the prefix sums through the list of places)
+        for (int x = tid; x < dm.RG; x += GROUP_THREADS) go[atomicAdd(&bins[min(off[x], GROUP_BINS - 1)], 1)] = (u32)x << 16;
+        __syncthreads();
+    }
+    {   // exclusive prefix sums: a thread takes consecutive places
+        const int chunk = (dm.RG + GROUP_THREADS - 1) / GROUP_THREADS, x0 = min(dm.RG, tid * chunk), x1 = min(dm.RG, x0 + chunk);
+        int sum = 0;
+        for (int x = x0; x < x1; ++x) sum += off[by_length ? go[x] >> 16 : x];
+        int run = before(sum);
+        for (int x = x0; x < x1; ++x) {
+            const int rg = by_length ? go[x] >> 16 : x, c = off[rg];
+            off[rg] = run; go[x] = (u32)run | (u32)rg << 16; run += c;
+            end[rg] = run;
+        }
+        if (tid == 0) go[dm.RG] = (u32)dm.N;
     }
     __syncthreads();
     unsigned short *list = A.list + (size_t)lay * dm.N;
-    for (int i = tid; i < dm.N; i += GROUP_THREADS) list[atomicAdd(&off[rgs[i]], 1)] = (unsigned short)i;
+    for (int i = tid; i < dm.N; i += GROUP_THREADS) {
+        if (!by_length || !(i & 1)) list[atomicAdd(&off[rgs[i]], 1)] = (unsigned short)i;
+        else list[atomicSub(&end[rgs[i]], 1) - 1] = (unsigned short)i;                 // odd ones from the end (see k_eval_slice)
+    }
+    for (int rg = tid; rg < dm.RG; rg += GROUP_THREADS) {
+        const int r = rg / dm.G, g = rg % dm.G, d0 = __ldg(A.dp_off + g), d1 = __ldg(A.dp_off + g + 1);
+        i64 Af = 0;
+        for (int s = 0; s < dm.S; ++s) {
+            const i64 ca = dm.ahat[s] * dm.C, cb = dm.bhat[s];
+            i64 worst = 0;
+            for (int x = d0; x < d1; ++x) {
+                const int c = r * dm.D + __ldg(A.dp_list + x);
+                const i64 v = ca * T[c] + cb * (i64)few_square(Q[c], A.q_halves);
+                worst = v > worst ? v : worst;
+            }
+            Af += worst;
+        }
+        A.cost[(size_t)lay * dm.RG + rg] = Af;                          // the sums add the expert part
+        if (b) {
+            ((i64 *)(b + A.bl.off_Afx))[rg] = Af;
+            if (A.bl.off_wtab >= 0)        // the pool holds the call's layouts as RG consecutive slices each
+                ((int *)(b + A.bl.off_wtab))[rg] = (A.first + lay) * dm.RG + rg;
+        }
+    }
+    int wrong = 0;
+    for (int c = tid; c < dm.K; c += GROUP_THREADS) {
+        wrong |= cnt[c] < 1 || T[c] > dm.C;
+        if (b) { ((u64 *)(b + A.bl.off_Q))[c] = few_square(Q[c], A.q_halves); ((int *)(b + A.bl.off_T))[c] = T[c]; ((int *)(b + A.bl.off_cnt))[c] = cnt[c]; }
+    }
+    wrong = __syncthreads_or(wrong);
+    if (tid == 0) A.tickets[lay] = wrong;
 }
 
-// Many layouts, second kernel.  A task is NS strips of 32 chunks (whole layers) of `rpt` consecutive row-shards of one
+// Many layouts, second kernel where N rows of at least one 16-byte chunk fit on chip.  A CTA holds `w` consecutive chunks of every
+// sample's row, `lps` whole layers or one of `parts` pieces of a layer, and adds up the row-shards of a share of the layouts
+// from there: teams of TW lanes, a row-shard each and a chunk a lane, read their samples' ids sixteen bits at a time and then the
+// rows from shared memory; a team that has finished reads the row of zeros behind the last sample.  Every sample's row crosses
+// L2 once a CTA instead of once a layout; bound by its instructions and by shared memory alike (a quarter warp reads 128 bytes at a
+// time, two rows of 64 bytes collide where both are even or odd): 256 layouts of 2048 samples in 240 row-shards, 24 layers of 16 ranks, 136 us
+// with the streaming sums, 80 with a division and a multiplication per row-shard and sample left in, 67.
+#define SLICE_THREADS 1024
+#define SLICE_MAX (1 << 12)           // row-shards whose busiest loads are kept between the pieces of a layer
+struct SlicePlan { int tw, w, parts, lps, slices, groups, batch; size_t smem; };
+template <int TW>
+__global__ void __launch_bounds__(SLICE_THREADS)
+k_eval_slice(const EvalArgs A, const SlicePlan S, int n)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const RpDims &dm = A.dm;
+    constexpr int TPW = 32 / TW, IDS = TW < 4 ? 4 : TW, PER = IDS / TW;          // teams of a warp; samples a round, ids of a lane
+    int4 *rows = (int4 *)smraw;                                                 // [N + 1][w]
+    const int N = dm.N, RG = dm.RG, cpl = dm.P >> 2, rc = dm.LP >> 2, w = S.w;
+    int *top = (int *)(rows + (size_t)(N + 1) * w);                             // parts > 1: [batch * RG] busiest loads so far
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, team = lane / TW, k = lane & (TW - 1);
+    const int slice = blockIdx.x % S.slices, group = blockIdx.x / S.slices, layer = slice * S.lps;
+    const bool first_of_layer = k % cpl == 0;
+    const int nl = min(S.lps, dm.L - layer), used = S.parts > 1 ? w : nl * cpl;        // chunks that exist
+    const int last = (int)((long long)n * (group + 1) / S.groups);
+    for (int lay0 = (int)((long long)n * group / S.groups); lay0 < last; lay0 += S.batch) {
+        const u32 nrg = min(S.batch, last - lay0) * RG;                         // row-shards of this batch of layouts
+        for (int part = 0; part < S.parts; ++part) {
+            const int first = layer * cpl + part * w;                           // first chunk
+            if (part || S.parts > 1 || lay0 == (int)((long long)n * group / S.groups)) {
+                __syncthreads();
+                const int4 *q4 = (const int4 *)A.q + first;
+                for (int x = tid; x < N * w; x += SLICE_THREADS) {
+                    const int i = x / w, c = x - i * w;
+                    if (c < used) {
+                        const unsigned dst = (unsigned)__cvta_generic_to_shared(rows + x);
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(q4 + (size_t)i * rc + c) : "memory");
+                    } else rows[x] = make_int4(0, 0, 0, 0);
+                }
+                if (tid < w) rows[(size_t)N * w + tid] = make_int4(0, 0, 0, 0);
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncthreads();
+            }
+            const int4 *col = rows + min(k, w - 1);
+            constexpr int STRIDE = SLICE_THREADS / TW;
+            const int dl = STRIDE / RG, dy = STRIDE % RG;
+            u32 f = warp * TPW + team, lay = lay0 + f / RG, y = f % RG;         // this team's row-shard of the batch: place y of layout lay
+            u32 o0 = 0, o1 = 0;
+            if (f < nrg) { const u32 *go = A.off + lay * (RG + 1u) + y; o0 = __ldg(go); o1 = __ldg(go + 1); }
+            while (f - team < nrg) {
+                const bool on = f < nrg;
+                const int p = (int)(o0 & 0xffffu), len = (int)(o1 & 0xffffu) - p;
+                const u32 at = lay * (u32)RG + (o0 >> 16), here = f;
+                // Odd teams walk their list from its end: a list holds its even samples first, and rows of 64 bytes that a
+                // quarter warp reads together collide where both are even or both odd.
+                const unsigned short *list = A.list + lay * (u32)N + ((team & 1) ? p + len - 1 : p);
+                const int step = (team & 1) ? -1 : 1;
+                f += STRIDE; lay += dl; y += dy;                                // the next one's offsets under this one's sums
+                if (y >= (u32)RG) { y -= RG; ++lay; }
+                o0 = o1 = 0;
+                if (f < nrg) { const u32 *go = A.off + lay * (RG + 1u) + y; o0 = __ldg(go); o1 = __ldg(go + 1); }
+                const int most = (int)__reduce_max_sync(0xffffffffu, len);
+                int4 a = make_int4(0, 0, 0, 0);
+                int id[PER];
+#pragma unroll
+                for (int m = 0; m < PER; ++m) { const int e = m * TW + k; id[m] = w * (e < len ? (int)__ldg(list + e * step) : N); }
+                for (int done = 0; done < most; done += IDS) {
+                    int now[PER];
+#pragma unroll
+                    for (int m = 0; m < PER; ++m) { const int e = done + IDS + m * TW + k; now[m] = id[m]; id[m] = w * (e < len ? (int)__ldg(list + e * step) : N); }
+#pragma unroll
+                    for (int u = 0; u < IDS; u += 2) {
+                        if (done + u >= most) break;
+                        const int i0 = TW == 1 ? now[u] : __shfl_sync(0xffffffffu, now[u / TW], u % TW, TW),
+                                  i1 = TW == 1 ? now[u + 1] : __shfl_sync(0xffffffffu, now[(u + 1) / TW], (u + 1) % TW, TW);
+                        const int4 v = col[i0], z = col[i1];
+                        a.x += v.x + z.x; a.y += v.y + z.y; a.z += v.z + z.z; a.w += v.w + z.w;
+                    }
+                }
+                const bool mine = on && k < used;
+                if (A.W_out && mine) ((int4 *)(A.W_out + (size_t)at * dm.LP))[first + k] = a;
+                int m = mine ? max(max(a.x, a.y), max(a.z, a.w)) : 0;
+                i64 es;
+                if (S.lps == 1) {                                               // (a piece of) one layer
+#pragma unroll
+                    for (int o = 1; o < TW; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+                    if (S.parts > 1 && on && k == 0) {
+                        if (part) m = max(m, top[here]);
+                        top[here] = m;
+                    }
+                    es = m;
+                } else {                                                        // whole layers: maximum over cpl lanes, sum over the layers
+                    const int own = m;
+                    for (int o = 1; o < cpl; ++o) m = max(m, __shfl_down_sync(0xffffffffu, own, o, TW));
+                    es = mine && first_of_layer ? (i64)m : 0;
+#pragma unroll
+                    for (int o = 1; o < TW; o <<= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
+                }
+                if (on && k == 0 && part + 1 == S.parts) atomicAdd((u64 *)A.cost + at, (u64)(dm.EC * es));
+            }
+        }
+    }
+}
+
+// How k_eval_slice divides the rows (tw = 0: not at all).  As many chunks of a row as fit, up to eight, a CTA to an SM; the SMs
+// are shared out so that their busiest has the least to do.  A layer in pieces is read a piece at a time, over again for every batch of layouts,
+// and pieces of one or two chunks are slower than the streaming sums.  Calls in us, streaming and from slices: whole layers, 2048 samples in 240
+// row-shards, 24 layers of 16 ranks, n = 256 159 and 102; 13000 in 96, 8 of 4, n = 16 181 and 142; 700 in 48, 48 of 24, n = 256 163 and 121;
+// pieces of four chunks, 3000 in 192, 24 of 32, n = 4 62 and 60, 64 128 and 93, 256 274 and 234; of two, 6000 in 96, 48 of 32, n = 4 146
+// and 192, 256 855 and 1726; of one, 8192 in 448, 24 of 16, n = 4 84 and 117, 256 344 and 1033.
+static SlicePlan eval_slice_plan(const RpDims &dm, int n)
+{
+    SlicePlan S = {};
+    const int cpl = dm.P >> 2;
+    if ((dm.P & 3) || dm.N > 65534) return S;
+    auto fits = [&](int w, int parts) { return 16 * (size_t)w * (dm.N + 1) + (parts > 1 ? 4 * (size_t)SLICE_MAX : 0) <= EVAL_SMEM_MAX; };
+    S.parts = 1;
+    while (S.parts <= cpl && !(cpl % S.parts == 0 && cpl / S.parts <= 8 && fits(cpl / S.parts, S.parts))) ++S.parts;
+    if (S.parts > cpl || (S.parts > 1 && (cpl / S.parts < 3 || dm.RG > SLICE_MAX))) return SlicePlan{};
+    S.lps = 1;
+    if (S.parts == 1) while (S.lps < dm.L && cpl * (S.lps + 1) <= 8 && fits(cpl * (S.lps + 1), 1)) ++S.lps;
+    S.w = cpl * S.lps / S.parts;
+    S.tw = 1;
+    while (S.tw < S.w) S.tw *= 2;
+    S.slices = (dm.L + S.lps - 1) / S.lps;
+    double best = 1e300;
+    for (int g = 1; g <= std::min(n, 32); ++g) {
+        // per CTA: loading its slice, then its layouts, in units of a layout's samples (64 bytes a cycle and SM from L2, 90 from shared memory)
+        const double cost = std::ceil((double)S.slices * g / 148) * (1.5 + (double)((n + g - 1) / g));
+        if (cost < best) { best = cost; S.groups = g; }
+    }
+    S.batch = S.parts > 1 ? std::max(1, SLICE_MAX / dm.RG) : n;
+    S.smem = 16 * (size_t)S.w * (dm.N + 1) + (S.parts > 1 ? 4 * (size_t)SLICE_MAX : 0);
+    return S;
+}
+
+// Many layouts, second kernel elsewhere.  A task is NS strips of 32 chunks (whole layers) of `rpt` consecutive row-shards of one
 // layout: a warp streams through their samples, which lie one after the other in the list, with U*NS loads in flight
 // whatever row-shard they belong to, and closes a row-shard when its last sample has been added.  Bound by its
 // instructions before it is by L2: row-shards hold 8.5 samples on average on large, and loops over one row-shard, or
@@ -250,9 +375,9 @@ k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt, bool sum32)
     const int cpl = dm.P >> 2, used = vec ? (32 / cpl) * cpl : 32;
     for (unsigned task = blockIdx.x * (EVAL_THREADS / 32) + (threadIdx.x >> 5); task < (unsigned)n * (unsigned)per; task += gridDim.x * (EVAL_THREADS / 32)) {
         const int lay = (int)(task / (unsigned)per), r = (int)(task - (unsigned)lay * per), sg = r % sgroups, rg0 = r / sgroups * rpt, nr = min(rpt, RG - rg0);
-        const int *go = A.off + (size_t)lay * (RG + 1) + rg0;
+        const u32 *go = A.off + (size_t)lay * (RG + 1) + rg0;
         const unsigned short *list = A.list + (size_t)lay * dm.N;
-        const int ends = __ldg(go + min(lane + 1, nr)), s0 = __ldg(go);           // lane x: where row-shard rg0 + x ends
+        const int ends = (int)(__ldg(go + min(lane + 1, nr)) & 0xffffu), s0 = (int)(__ldg(go) & 0xffffu);        // lane x: where row-shard rg0 + x ends
         if (!vec) {
             int m0 = s0;
             for (int x = 0; x < nr; ++x) {
@@ -264,7 +389,7 @@ k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt, bool sum32)
                     if (wout) wout[e] = sum;
                     return sum;
                 });
-                if (lane == 0) A.Esum[(size_t)lay * RG + rg0 + x] = es;
+                if (lane == 0) A.cost[(size_t)lay * RG + rg0 + x] += dm.EC * es;
                 m0 = m1;
             }
             continue;
@@ -296,10 +421,7 @@ k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt, bool sum32)
             }
             i64 es = (i64)__reduce_add_sync(0xffffffffu, own);
             if (!sum32) es += (i64)__reduce_add_sync(0xffffffffu, high) << 16;
-            if (lane == 0) {
-                if (sgroups > 1) atomicAdd((u64 *)(A.Esum + at), (u64)es);
-                else A.Esum[at] = es;
-            }
+            if (lane == 0) atomicAdd((u64 *)A.cost + at, (u64)(dm.EC * es));
             ++x;
             end = __shfl_sync(0xffffffffu, ends, x);
         };
@@ -329,30 +451,65 @@ k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt, bool sum32)
     }
 }
 
-__global__ void __launch_bounds__(EVAL_THREADS)
-k_eval_score(const EvalArgs A)
-{
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const EvalFinish f = eval_finish_views(A.dm, smraw);
-    eval_load_cells(A, blockIdx.x, f.cell_of, threadIdx.x, EVAL_THREADS);
-    eval_finish(A, blockIdx.x, f, threadIdx.x);
-}
-
 __device__ __forceinline__ i64 few_warp_max(i64 v)
 {
     for (int o = 16; o; o >>= 1) { const i64 w = __shfl_xor_sync(0xffffffffu, v, o); v = w > v ? w : v; }
     return v;
 }
 
-// Sums of squared lengths in shared memory: 64 bits, or (halves: no sum reaches 2^48) the lower 16 bits of each square and what lies
-// above them added up in 32 bits each.  A 64-bit addition there is a loop, and the samples of a row-shard of few slots meet in it: 4000
-// samples in six row-shards of one slot, 128 layouts 206 us and 147 in halves, one layout 48 and 41.
-__device__ __forceinline__ void few_add(u64 *q, u32 low, u32 high, bool halves)
+// Many layouts, last kernel: the scores from the row-shards' costs, and what is left of the blob.
+__global__ void __launch_bounds__(EVAL_THREADS)
+k_eval_score(const EvalArgs A)
 {
-    if (halves) { atomicAdd((u32 *)q, low); atomicAdd((u32 *)q + 1, high); }
-    else atomicAdd(q, ((u64)high << 32) | low);
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const RpDims &dm = A.dm;
+    i64 *U = (i64 *)smraw;                                               // [G]
+    __shared__ i64 top_s[EVAL_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, lay = blockIdx.x;
+    i64 *cost = A.cost + (size_t)lay * dm.RG;
+    char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
+    for (int g = tid; g < dm.G; g += EVAL_THREADS) U[g] = 0;
+    __syncthreads();
+    i64 top = 0;
+    for (int rg = tid; rg < dm.RG; rg += EVAL_THREADS) {
+        const i64 J = __ldcg(cost + rg);
+        cost[rg] = 0;
+        top = J > top ? J : top;
+        atomicAdd((u64 *)&U[rg % dm.G], (u64)J);
+        if (b) {
+            ((i64 *)(b + A.bl.off_Jfx))[rg] = J;
+            ((i64 *)(b + A.bl.off_Esum))[rg] = (J - ((const i64 *)(b + A.bl.off_Afx))[rg]) / dm.EC;
+        }
+    }
+    top = few_warp_max(top);
+    if (lane == 0) top_s[tid >> 5] = top;
+    const int wrong = A.tickets[lay];
+    __syncthreads();
+    if (tid == 0) A.tickets[lay] = 0;
+    if (A.host) {          // coverage is checked by the caller's `bad` flag: every sample sits in one cell by construction
+        if (tid < 8) A.host[tid] = A.counters[tid];
+        if (tid < 3) { A.host[16 + tid] = A.inc_score[tid]; A.host[22 + tid] = A.seed_score[tid]; }
+        if (tid < RP_SW_COUNT) ((int *)(A.host + 56))[tid] = A.status[tid] | (tid == RP_SW_VALIDATE && wrong ? 1 : 0);
+        if (A.layout_host) for (int i = tid; i < dm.N; i += EVAL_THREADS) A.layout_host[i] = __ldg(A.lay32 + i);
+    }
+    if (b) for (int g = tid; g < dm.G; g += EVAL_THREADS) ((i64 *)(b + A.bl.off_U))[g] = U[g];
+    if (tid >= 32) return;
+    const bool refused = A.bad_dev && __ldcg(A.bad_dev);
+    i64 s0 = 0, s1 = 0, s2 = lane < EVAL_THREADS / 32 ? top_s[lane] : 0;
+    for (int g = lane; g < dm.G; g += 32) { const i64 u = U[g]; s1 += u; s0 = u > s0 ? u : s0; }
+    for (int o = 16; o; o >>= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    s0 = few_warp_max(s0); s2 = few_warp_max(s2);
+    if (lane == 0) {
+        const i64 sc[3] = { s0, s1, s2 };
+        for (int x = 0; x < 3; ++x) {
+            if (refused) continue;
+            if (A.score_out) A.score_out[(size_t)lay * 3 + x] = sc[x];
+            if (A.score_out2) A.score_out2[(size_t)lay * 3 + x] = sc[x];
+            if (A.f64_out) A.f64_out[(size_t)lay * 3 + x] = (double)sc[x] / (double)dm.SC;
+        }
+        if (b) { i64 *S = (i64 *)(b + A.bl.off_S); S[0] = s0; S[1] = s1; S[2] = s2; S[3] = rp_energy(s0, s1, s2); }
+    }
 }
-__device__ __forceinline__ u64 few_square(u64 v, bool halves) { return halves ? ((v >> 32) << 16) + (u32)v : v; }
 
 // grid = (MS, row-shards, layouts), clusters of MS CTAs along x: CTA x of a row-shard takes the samples of
 // range x, then the layers of range x of the summed row.  The row-shard's cell statistics and cost are worked out by its own
@@ -397,9 +554,7 @@ k_eval_few(const EvalArgs A)
         const int ti = __ldg(A.t + i);
         list[atomicAdd(&n_s, 1)] = i;
         atomicAdd(&T[d], ti); atomicAdd(&cnt[d], 1);
-        const u64 sq = (u64)ti * (u64)ti;
-        if (A.q_halves) few_add(&Q[d], (u32)sq & 0xffffu, (u32)(sq >> 16), true);
-        else few_add(&Q[d], (u32)sq, (u32)(sq >> 32), false);
+        few_add_square(&Q[d], ti, A.q_halves);
         if (b) ((unsigned short *)(b + A.bl.off_cell))[i] = (unsigned short)c;
     }
     if (A.layout_host && rg == 0) for (int i = i0 + tid; i < i1; i += EVAL_THREADS) A.layout_host[i] = __ldg(A.lay32 + i);
@@ -496,7 +651,7 @@ k_eval_few(const EvalArgs A)
                 ((i64 *)(b + A.bl.off_Esum))[rg] = E; ((i64 *)(b + A.bl.off_Afx))[rg] = Af; ((i64 *)(b + A.bl.off_Jfx))[rg] = J;
                 if (A.bl.off_wtab >= 0) ((int *)(b + A.bl.off_wtab))[rg] = (A.first + lay) * dm.RG + rg;      // the pool holds the call's layouts as RG slices each
             }
-            A.Esum[(size_t)lay * dm.RG + rg] = J;
+            A.cost[(size_t)lay * dm.RG + rg] = J;
             __threadfence();
             // arrivals in the lower half, row-shards with an empty or overfull cell in the upper one
             const unsigned before = atomicAdd((unsigned *)&A.tickets[lay], 1u | (wrong ? 1u << 16 : 0u));
@@ -511,7 +666,7 @@ k_eval_few(const EvalArgs A)
     for (int x = tid; x < dm.G; x += EVAL_THREADS) U[x] = 0;
     __syncthreads();
     {
-        i64 *eg = A.Esum + (size_t)lay * dm.RG, top = 0;
+        i64 *eg = A.cost + (size_t)lay * dm.RG, top = 0;
 #pragma unroll 4
         for (int x = tid; x < dm.RG; x += EVAL_THREADS) {
             const i64 J = __ldcg(eg + x);
@@ -567,25 +722,26 @@ k_eval_few(const EvalArgs A)
     }
 }
 
+// Windows are taken up to this measure of their size (no kernel here needs as much shared memory).
 static size_t eval_smem_bytes(const RpDims &dm)
 {
-    return (eval_finish_bytes(dm) + sizeof(int) * (2 * (size_t)dm.RG + 1 + dm.N) + 15) & ~(size_t)15;
+    const size_t cells = (sizeof(u64) * dm.K + sizeof(i64) * (2 * (size_t)dm.RG + dm.G) + sizeof(int) * 2 * (size_t)dm.K + 2 * (size_t)dm.N + 15) & ~(size_t)15;
+    return (cells + sizeof(int) * (2 * (size_t)dm.RG + 1 + dm.N) + 15) & ~(size_t)15;
 }
 
 // Whether n layouts take the few-layouts form.  It has a cluster per row-shard and layout, which scans the whole assignment; the other
-// form groups an assignment once, but in one CTA, and streams through a row-shard with one warp: more launches, and slow where
-// row-shards are long.  Calls in us, few and many: 512 samples in 32 row-shards, 16 layers of 8 ranks, n = 8 36.8 and 41.8, 40 41.3 and
-// 42.4, 64 49.0 and 42.4, 512 204 and 64; 2048 in 240, 24 of 16, n = 4 37.6 and 51.1, 8 46.8 and 51.2, 64 171 and 77; 4000 in 6, 16 of
-// 8, n = 128 147 and 276, 512 307 and 336; 30000 in 160, n = 1 79 and 363, 8 516 and 373.  One layout: 8192 in 448 47.6 and 94, 4000 in
-// 2000 44.5 and 50.7, 8000 in 1920 51.6 and 69.3.  The line was drawn for an earlier few-layouts kernel (per CTA 6 ns and a nanosecond for 300
-// samples, rows served less evenly, 0.3 ns for 1000 counts, against 9 us of launches and up to 30 us of a long row-shard); today's is still
-// ahead somewhat above it (2048 samples, n = 6 44.8 and 51.1; 4000 in 6, n = 300 220 and 301; 30000, n = 3 141 and 376).
+// form groups an assignment once, but in one CTA, and has three launches where this has one.  Calls in us, few and many: 512 samples in
+// 32 row-shards, 16 layers of 8 ranks, n = 8 37.0 and 36.6, 16 38.8 and 36.9, 64 49 and 37, 512 204 and 54; 2048 in 240, 24 of 16, n = 4 36.9
+// and 41.5, 6 44.7 and 42.5, 64 172 and 54; 1000 in 128, 8 of 8, n = 8 37.8 and 37.4, 12 42.1 and 38.5; 4000 in 6, 16 of 8, n = 64 96 and
+// 138, 128 148 and 141, 512 307 and 233; 1031 in 16, 43 of 16, n = 18 42.4 and 43.4, 30 45.6 and 44.4; 8192 in 448, 24 of 16 (no slice on
+// chip), n = 2 63 and 95; 30000 in 160, n = 3 142 and 270, 4 335 and 267.  One layout: 8192 in 448 47.6 and 94, 4000 in 2000 44.8 and 46.3,
+// 8000 in 1920 51.8 and 71.
 static bool eval_is_few(const RpDims &dm, int n)
 {
     if ((dm.P & 3) || n >= 65536 || dm.RG >= 65536 || dm.LP > 16384 || eval_few_smem(dm, 8) > EVAL_SMEM_MAX) return false;
     const double N = dm.N, RG = dm.RG;
     if (n == 1) return RG * N <= 5e6;
-    return n * (RG * (6.0 + N / 300.0) + 3e-4 * N * dm.LP) <= 9e3 + std::min(150.0 * N / RG, 30e3);
+    return n * (RG * (6.0 + N / 300.0) + 3e-4 * N * dm.LP) <= 4e3 + 5.0 * std::min(N, 1e4);
 }
 size_t rp_eval_list_len(const RpDims &dm, int n) { return eval_is_few(dm, n) ? 0 : (size_t)n * dm.N; }
 size_t rp_eval_off_len(const RpDims &dm, int n) { return eval_is_few(dm, n) ? 0 : (size_t)n * (dm.RG + 1); }
@@ -614,7 +770,7 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
         cfg.attrs = at; cfg.numAttrs = 1;
         RP_CUDA(cudaLaunchKernelEx(&cfg, few, A));
     } else {
-        const size_t gm = sizeof(int) * (size_t)dm.RG + 2 * ((size_t)dm.K + dm.N), fm = eval_finish_bytes(dm);
+        const size_t gm = eval_group_bytes(dm), fm = sizeof(i64) * (size_t)dm.G;
         if (gm > EVAL_SMEM_MAX || dm.N > 65535) return RP_ERR_RANGE;
         if (gm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_group, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
         if (fm > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_eval_score, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
@@ -633,16 +789,27 @@ static int eval_launch(rp_ctx *c, EvalArgs &A, int n)
             if (B.blob_out) B.blob_out += (size_t)first * c->bl.bytes;
             if (B.score_out) B.score_out += 3 * (size_t)first;
             if (B.f64_out) B.f64_out += 3 * (size_t)first;
-            B.Esum += (size_t)first * dm.RG; B.tickets += first; B.list += (size_t)first * dm.N; B.off += (size_t)first * (dm.RG + 1);
+            B.cost += (size_t)first * dm.RG; B.tickets += first; B.list += (size_t)first * dm.N; B.off += (size_t)first * (dm.RG + 1);
             return B;
         };
+        const SlicePlan S = eval_slice_plan(dm, std::min(n, 16384));
+        auto slice = S.tw == 1 ? k_eval_slice<1> : S.tw == 2 ? k_eval_slice<2> : S.tw == 4 ? k_eval_slice<4> : k_eval_slice<8>;
+        if (S.tw) RP_CUDA(cudaFuncSetAttribute(slice, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX));
         for (int first = 0; first < n; first += 16384) {
-            k_eval_group<<<std::min(16384, n - first), GROUP_THREADS, gm, c->stream>>>(part(first));
+            k_eval_group<<<std::min(16384, n - first), GROUP_THREADS, gm, c->stream>>>(part(first), S.tw != 0);
             ++g_rp_launches;
         }
         for (int first = 0; first < n; first += 16384) {
             const EvalArgs B = part(first);
             const int m = std::min(16384, n - first);
+            if (S.tw) {
+                SlicePlan P = S;
+                P.groups = std::min(P.groups, m);
+                slice<<<P.slices * P.groups, SLICE_THREADS, P.smem, c->stream>>>(B, P, m);
+                k_eval_score<<<m, EVAL_THREADS, fm, c->stream>>>(B);
+                g_rp_launches += 2;
+                continue;
+            }
             // several tasks for each warp the SMs hold, of at most 31 row-shards
             const int rpt = (int)std::max<long long>(1, std::min<long long>(31, (long long)m * dm.RG * sgroups / (148 * warps * 6)));
             const long long want = ((long long)m * ((dm.RG + rpt - 1) / rpt) * sgroups + 7) / 8;
@@ -670,7 +837,7 @@ int rp_launch_eval(rp_ctx *c, const int *lay, const int *src, int n, int *W_out,
     A.W_out = W_out; A.blob_out = blob_out; A.score_out = score_out; A.f64_out = f64_out;
     A.bad = rp_pin_bad(c);
     if (score_final || f64_final) { A.score_final = score_final; A.f64_final = f64_final; A.bad_dev = c->d_status + RP_SW_BAD_LAYOUT; }
-    A.Esum = c->d_eval_Esum; A.tickets = c->d_eval_tickets; A.list = c->d_eval_list; A.off = c->d_eval_off;
+    A.cost = c->d_eval_Esum; A.tickets = c->d_eval_tickets; A.list = c->d_eval_list; A.off = (u32 *)c->d_eval_off;
     return eval_launch(c, A, n);
 }
 
@@ -678,7 +845,7 @@ int rp_launch_eval(rp_ctx *c, const int *lay, const int *src, int n, int *W_out,
 static void eval_one(rp_ctx *c, EvalArgs &A)
 {
     A.bad = rp_pin_bad(c);
-    A.Esum = c->d_one_Esum; A.tickets = c->d_one_ticket; A.list = c->d_one_list; A.off = c->d_one_off;
+    A.cost = c->d_one_Esum; A.tickets = c->d_one_ticket; A.list = c->d_one_list; A.off = (u32 *)c->d_one_off;
 }
 int rp_launch_eval_seed(rp_ctx *c)
 {
@@ -1003,7 +1170,7 @@ extern "C" int rp_eval_layouts_noalloc(rp_ctx *c, const int32_t *layouts, int32_
     *bad = 0;
     EvalArgs A = {};
     A.lay32 = layouts; A.score_out = (i64 *)score_fx; A.f64_out = score_f64; A.bad = bad;
-    A.Esum = sc->esum; A.tickets = sc->tickets; A.list = sc->list; A.off = sc->off;
+    A.cost = sc->esum; A.tickets = sc->tickets; A.list = sc->list; A.off = (u32 *)sc->off;
     RP_TRY(eval_launch(c, A, n));
     RP_CUDA(cudaStreamSynchronize(c->stream));
     return *bad ? RP_ERR_ARG : RP_OK;

@@ -1875,3 +1875,42 @@ def test_first_fit_at_the_edges_of_its_warps(N, D, min_rows, cap, longest):
     assert rp.rp_pack_rows(ctx) == (R, cert)
     assert (rp.rp_debug_dump(ctx, "SEED_LAYOUT", (N,), np.int32) == seed).all()
     rp.rp_destroy(ctx)
+
+
+# Scoring from a slice of all rows on chip: chunks of a layer one, three and six (several layers to a slice, the last slice with fewer),
+# eight, in two pieces and eleven; as many samples as one chunk a row holds and more (no slice); pieces of a layer with a few layouts
+# to a batch; row-shards of more samples than are told apart by their number, and of none; odd batches.
+@pytest.mark.parametrize("N,L,P,D,R,edp,n", [
+    (300, 11, 4, 4, 3, None, 700), (301, 5, 12, 4, 3, None, 500), (120, 3, 24, 2, 9, [0, 0], 900), (1900, 3, 32, 16, 8, None, 40),
+    (900, 2, 64, 16, 6, None, 67), (60, 3, 132, 2, 2, None, 400), (14079, 2, 4, 4, 2, None, 100), (14080, 2, 4, 4, 2, None, 100),
+    (2600, 2, 64, 32, 40, None, 5), (3000, 3, 16, 2, 2, [0, 0], 700)])
+def test_scoring_from_slices_on_chip(N, L, P, D, R, edp, n):
+    w = make_window(custom_spec("slices", N, L, P, 2, 4096, D, P, 2, 0, data_seed=N + P))
+    ref = oracle_front(w, edp, R)
+    ctx = load(w, edp=edp, min_rows=R)
+    check_front(w, ctx, ref)
+    s = w.spec
+    rng = np.random.default_rng(P + N)
+    lays = rng.integers(0, ref["R"] * D, (n, N)).astype(np.int32)
+    lays[n // 2] = rng.integers(0, 2, N)                # nearly all row-shards empty
+    want = oracle.eval_layouts(w.lengths, ref["q"], lays, ref["R"], s.token_cap, D, edp, s.alpha, s.beta)["score"]
+    for _ in range(2):                                  # the scratch is clear again after a call
+        fx, _f64 = rp.rp_eval_population(ctx, lays)
+        assert (fx == want).all()
+    if n <= 64:
+        check_eval(w, ctx, ref, edp, n=n)               # rank loads too
+    rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,L,P,D,pop", [(200, 5, 12, 6, 220), (900, 3, 64, 4, 200)])
+def test_rank_loads_of_members_scored_from_slices(N, L, P, D, pop):
+    """The rank loads and statistics that scoring leaves for a population are what a search starts from."""
+    w = make_window(custom_spec("slice_loads", N, L, P, 2, 4096, D, P, pop, 0, data_seed=P))
+    s = w.spec
+    ref = oracle_front(w, None, 4)
+    ctx = load(w, pop=pop, min_rows=4)
+    check_front(w, ctx, ref)
+    rp.rp_seed_population(ctx, 4)
+    init, _ok = oracle.seed_trials(w.lengths, ref["seed"], ref["R"], s.token_cap, D, pop, 4, s.anneal_seed)
+    check_anneal(w, ctx, ref, None, pop, 2, 20, t_ratio=0.6, init=init)
+    rp.rp_destroy(ctx)
