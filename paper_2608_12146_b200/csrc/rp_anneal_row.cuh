@@ -23,6 +23,12 @@ struct RowArgs {
 __device__ __forceinline__ int4 sub4(const int4 &a, const int4 &b) { return make_int4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
 __device__ __forceinline__ int4 add4(const int4 &a, const int4 &b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
+// The chains of a level may be launched before the launch between two levels (rp_level_turn.cu) has ended: once each of its CTAs has called
+// rp_let_next_launch_start or has ended.  What it leaves behind, or reads still, they touch behind rp_wait_for_launch_before, which
+// waits for its end.  Launched without the attribute that allows it, both do nothing.
+__device__ __forceinline__ void rp_let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void rp_wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Bounded wait of one thread until a counter that the other CTAs of the launch add to has reached
 // `target`; false when the time allowed ran out or another chain has raised the time-out word.
 __device__ __forceinline__ bool rp_wait_count(const int *ctr, int target, const AnnealArgs &A)
@@ -45,6 +51,10 @@ __device__ __forceinline__ bool rp_wait_count(const int *ctr, int target, const 
 // Layers per lane where a lane takes whole layers (0: too many layers); whether a row's chunks are dealt out to the lanes instead.
 static inline int rp_row_layers(const RpDims &dm) { return dm.L <= 32 ? 1 : (dm.L <= 64 ? 2 : (dm.L <= 128 ? 4 : 0)); }
 static inline bool rp_row_split(int cpl) { return cpl == 2 || cpl == 4; }
+// Whether they may start right away, up to four to an SM: their first step records and tables are then ready when the launch before ends
+// (300 members of 17 layers 1469 us at its end, 1401 right away; 512 of 24 2730 and 2715).  With more, the SM is full and what its
+// rows have left of the L1 cache counts (1024 members 2377 and 2390).
+static inline bool rp_row_starts_early(const rp_ctx *c) { return c->Ppop <= 4 * rp_sms(c); }
 int rp_launch_row_chip(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int grid, int *done);
 int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);
 int rp_launch_row_pair(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);

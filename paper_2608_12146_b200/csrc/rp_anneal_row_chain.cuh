@@ -9,6 +9,7 @@
 // the shared warps below: medium 972 -> 807 us, large 3169 -> 2499, two shards 916 -> 816, ragged 1781 -> 1570, wide 10.9 -> 9.8 ms, heavy
 // 83.4 -> 59.3 (windows of perf/cases.py, seed 5, one GPU; times below without a window's sizes are of these).
 #pragma once
+#include <algorithm>
 #include <string.h>
 
 #include "rp_level_end.cuh"
@@ -317,7 +318,11 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
     const unsigned short *g_of = (const unsigned short *)(sm_tab + A.sl.off_g);
     const unsigned short *rowbase = (const unsigned short *)(sm_tab + A.sl.off_row);
 
-    if (!CHIP && __ldcg(&A.status[RP_SW_TIMEOUT])) return;               // the call has failed already: nothing to do
+    constexpr bool AHEAD = ONE && !CHIP;
+    if (!CHIP && !AHEAD) {
+        rp_wait_for_launch_before();
+        if (__ldcg(&A.status[RP_SW_TIMEOUT])) return;                    // the call has failed already: nothing to do
+    }
     const int L = dm.L, cpl = CPL == 1 && !SPLIT ? 1 : X.cpl, rc = L * cpl;        // 16-byte chunks per layer and per row
     const int rot = CHIP && CPL > 1 && (cpl & (cpl - 1)) == 0 ? cpl - 1 : 0;     // lanes start at different chunks: fewer bank conflicts
     // 16-byte chunk u of this lane
@@ -335,13 +340,29 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
     const int n4 = dm.N >> 2;
     const StepRec *recs = (const StepRec *)(ch.base + X.off_recs);
 
-    // ---- prologue: the static tables and the ancestor's terminal state ---------------------------
+    // ---- prologue: the static tables, the first steps (a launch per level: they depend on nothing the launch before leaves behind) and the
+    // ancestor's terminal state -----------------------------------------------------------------
+    StepX ahead;
     {
         const int nd = A.sl.off_t >> 2, nc = (A.sl.bytes - A.sl.off_rg) >> 2;
         for (int x = tid; x < nd; x += NT) ((int *)sm_cta)[x] = __ldg((const int *)A.static_blk + x);
         for (int x = tid; x < nc; x += NT) ((int *)(sm_cta + X.off_tab))[x] = __ldg((const int *)(A.static_blk + A.sl.off_rg) + x);
     }
     if (CHIP && X.off_tf) for (int x = tid; x < dm.N; x += NT) ((int2 *)(sm_cta + X.off_tf))[x] = __ldg(X.tf + x);
+    if (AHEAD) {
+        const StepRec r = rp_make_step_rec(A, A.level, A.tau, (u32)lane, (u32)j);
+        const bool rl = r.flags & 1u;
+        ahead.i[0] = r.i0; ahead.i[1] = r.i1; ahead.i[2] = rl ? (int)(r.i2 | 0x80000000u) : r.i2; ahead.i[3] = rl ? (int)(r.i3 | 0x80000000u) : r.i3;
+        ahead.bz = r.bz; ahead.thr = r.flags & 4u ? 1ull << 63 : r.thr;
+        ahead.thrf = r.flags & 4u ? __int_as_float(0x7f800000) : (float)r.thr * (0x1p-32f * (1.f + 0x1p-20f));
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const int2 v = x < 2 || !rl ? __ldg(X.tf + ahead.i[x]) : make_int2(0, 0);
+            ahead.t[x] = v.x; ahead.f[x] = v.y;
+        }
+        rp_wait_for_launch_before();
+        if (__ldcg(&A.status[RP_SW_TIMEOUT])) return;                    // the call has failed already: nothing to do
+    }
     int half_w = 0, inc_slot = -1;
     __shared__ i64 inc_s[3];
     __shared__ int failed_s;
@@ -454,9 +475,15 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
         bool done = !live, need = false;
         unsigned pmask = 0;
         StepX sr;
-        sr.bz = 0; sr.thr = 0; sr.thrf = 0.f;
+        if (AHEAD) {
+            sr = ahead;
 #pragma unroll
-        for (int x = 0; x < 4; ++x) { sr.i[x] = 0; sr.c[x] = 0; sr.t[x] = 0; sr.f[x] = 0; }
+            for (int x = 0; x < 4; ++x) sr.c[x] = 0;
+        } else {
+            sr.bz = 0; sr.thr = 0; sr.thrf = 0.f;
+#pragma unroll
+            for (int x = 0; x < 4; ++x) { sr.i[x] = 0; sr.c[x] = 0; sr.t[x] = 0; sr.f[x] = 0; }
+        }
         bool ok = false;
         int mi = 0, mi2 = -1, ti = 0, t2 = 0, df = 0;
         u32 p1 = 0, p2 = 0;
@@ -485,6 +512,10 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                 if (fresh) {
                     nb = min(GL, A.steps - kb); pos = 0;
                     if (lg < nb) {
+                        if (AHEAD && kb == 0) {                         // (all but the cells is known)
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) sr.c[x] = x < 2 || sr.i[x] >= 0 ? (u32)__ldcg(cells + sr.i[x]) : (u32)sr.i[x] & 0x7fffffffu;
+                        } else {
                         StepRec r;
                         const bool kept = !ONE || (CHIP && kb + lane < X.recs);
                         if (kept) r = recs[ONE ? (ln & 1) * X.recs + kb + lane : (kb & 16) + lg];
@@ -505,6 +536,7 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                         sr.bz = r.bz; sr.thr = r.flags & 4u ? 1ull << 63 : r.thr;
                         sr.thrf = r.flags & 4u ? __int_as_float(0x7f800000) : (float)r.thr * (0x1p-32f * (1.f + 0x1p-20f));
                         if (rl) { sr.i[2] = (int)0x80000000; sr.i[3] = (int)0x80000000; }
+                        }
 #pragma unroll
                         for (int x = 0; x < 4; ++x) sr.c[x] |= (u32)(IDENT ? g_of[sr.c[x]] : rg_of[sr.c[x]]) << 16;
                     }
@@ -1104,10 +1136,20 @@ static int launch_row_t(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int gr
     if (CHIP && grid > rp_sms(c)) return RP_OK;
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(CHIP ? ROW_THREADS : 32);
     cfg.dynamicSmemBytes = X.smem_bytes; cfg.stream = c->stream;
+    // Chains that start beside the launch before them (see rp_row_starts_early) go where there is room first: as much shared memory a CTA that
+    // an SM takes its share of them and no more.
+    if (!CHIP && rp_row_starts_early(c)) {
+        const size_t share = (grid + rp_sms(c) - 1) / rp_sms(c);
+        cfg.dynamicSmemBytes = std::max(cfg.dynamicSmemBytes, (size_t)228 * 1024 / (share + 1) - 1024 + 256);
+    }
     cudaLaunchAttribute at[1];
     if (CHIP) {
         at[0].id = cudaLaunchAttributeCooperative;
         at[0].val.cooperative = 1;
+        cfg.attrs = at; cfg.numAttrs = 1;
+    } else if (A.level > 0) {                       // behind the launch between two levels, see rp_level_turn.cu
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at; cfg.numAttrs = 1;
     }
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, A, X);
