@@ -279,11 +279,11 @@ __device__ __forceinline__ void row_barrier_warp(const AnnealArgs &A, int P, con
 }
 
 // Warps per SM the register budget is set for.  Registers come in quarters of an SM: 12 leaves 168 a thread and keeps 12 warps
-// resident, 13 to 16 leave 128 and keep 16.  Which is better depends on how many chains there are; at 12 / 14 / 16, plans in ms: heavy
+// resident, 13 to 16 leave 128 and keep 16.  Which is better depends on how many warps there are; at 12 / 14 / 16, plans in ms: heavy
 // (8192 members, two to a warp) 61.6 / 59.4 / 59.5, 4096 members of 16 layers of 32 ranks (two to a warp) 4.15 / 3.41 / 3.44; where 12 a
-// SM hold them all, 1776 members with a warp each, heavy's window at 20 levels of 200 steps 5.95 / 6.55 / 6.82.  (Asked for 16 the compiler
-// orders the code another way and spills less, 24 bytes for 40, to no gain.)  More chunks, or shards of several slots, need the
-// registers of 12.
+// SM hold them all (ROOMY), 1776 members with a warp each, heavy's window at 20 levels of 200 steps 5.95 / 6.55 / 6.82, 1184 5.28 / 5.99,
+// 3000 members of 16 layers, two to a warp, 2.83 / 3.00.  (Asked for 16 the compiler orders the code another way and spills less, 24
+// bytes for 40, to no gain.)  More chunks, or shards of several slots, need the registers of 12.
 #define ROW_WARPS_PER_SM(GL, LPL, CPL, IDENT) ((GL) == 16 || ((LPL) * (CPL) == 1 && (IDENT)) ? 14 : 12)
 
 // GL lanes run a chain, LPL layers per lane, CPL 16-byte chunks per layer (X.cpl <= CPL of them in use).  IDENT: slot d is shard d.
@@ -291,8 +291,8 @@ __device__ __forceinline__ void row_barrier_warp(const AnnealArgs &A, int P, con
 // meets in shuffles: a load touches consecutive bytes, and no lane is idle for want of layers.  Whole layers of four chunks put the
 // lanes of a load 64 bytes apart, twelve lines for 24 layers, eight stores 440 cycles (large 2662 us, dealt out 2499; with candidates
 // 3023 and 2999).  With the rank loads on chip only the demand rows would gain, and the shuffles cost more (3 % of two shards).
-template <int GL, int LPL, int CPL, bool SPLIT, bool CHIP, bool COMP, bool IDENT>
-__global__ void __launch_bounds__(CHIP ? ROW_THREADS : 32, CHIP ? 1 : ROW_WARPS_PER_SM(GL, LPL, CPL, IDENT))
+template <int GL, int LPL, int CPL, bool SPLIT, bool CHIP, bool COMP, bool IDENT, bool ROOMY>
+__global__ void __launch_bounds__(CHIP ? ROW_THREADS : 32, CHIP ? 1 : ROOMY ? 12 : ROW_WARPS_PER_SM(GL, LPL, CPL, IDENT))
 k_anneal_row(const AnnealArgs A, const RowArgs X)
 {
     constexpr int NCH = SPLIT ? CPL : LPL * CPL;
@@ -1126,7 +1126,10 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
 template <int GL, int LPL, int CPL, bool SPLIT, bool CHIP, bool COMP, bool IDENT>
 static int launch_row_t(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int grid, int *done)
 {
-    auto kern = k_anneal_row<GL, LPL, CPL, SPLIT, CHIP, COMP, IDENT>;
+    constexpr bool TIGHT = !CHIP && ROW_WARPS_PER_SM(GL, LPL, CPL, IDENT) > 12;
+    auto kern = k_anneal_row<GL, LPL, CPL, SPLIT, CHIP, COMP, IDENT, false>;
+    // (or shared memory keeps no more than twelve resident anyway)
+    if (TIGHT && (grid <= 12 * rp_sms(c) || 228 * 1024 / (X.smem_bytes + 1024) <= 12)) kern = k_anneal_row<GL, LPL, CPL, SPLIT, CHIP, COMP, IDENT, TIGHT>;
     // (always the same value, above anything a launch asks for: contexts that plan different
     // windows at once on different host threads then never lower each other's limit)
     RP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_SMEM_MAX));
@@ -1163,7 +1166,7 @@ static int launch_row_t(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int gr
 template <int GL, int LPL, int CPL, bool SPLIT, bool COMP, bool IDENT>
 static int row_resident_t(const RowArgs &X, int *warps)
 {
-    auto kern = k_anneal_row<GL, LPL, CPL, SPLIT, false, COMP, IDENT>;
+    auto kern = k_anneal_row<GL, LPL, CPL, SPLIT, false, COMP, IDENT, false>;
     RP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_SMEM_MAX));
     RP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(warps, kern, 32, (size_t)X.smem_bytes));
     return RP_OK;

@@ -1914,3 +1914,20 @@ def test_rank_loads_of_members_scored_from_slices(N, L, P, D, pop):
     init, _ok = oracle.seed_trials(w.lengths, ref["seed"], ref["R"], s.token_cap, D, pop, 4, s.anneal_seed)
     check_anneal(w, ctx, ref, None, pop, 2, 20, t_ratio=0.6, init=init)
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("L", [16, 17])
+@pytest.mark.parametrize("pop", [8, 9, 24, 25, 48, 49])
+def test_instances_by_the_members_of_an_sm(L, pop):
+    """On two SMs: chains that start beside the launch before them, four to an SM, and more; twelve warps of 168 registers to an SM,
+    with a chain each or with two, and more of 128."""
+    spec = ("instances", 80, L, 64, 32, 3, None, 3, pop)
+    w = compressed_window(spec)
+    ref = oracle_front(w, None, 3)
+    ctx = load(w, pop=pop, min_rows=3)
+    rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 3)
+    rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 2)
+    check_front(w, ctx, ref)
+    _, stats = check_anneal(w, ctx, ref, None, pop, 4, 70, t_ratio=0.6, check_members=2, t0=1e-2)
+    assert rp.rp_debug_chain_form(ctx) == ("two to a warp" if pop > 32 else "compressed") and stats.accepted > 0
+    rp.rp_destroy(ctx)
