@@ -1921,10 +1921,11 @@ def test_rank_loads_of_members_scored_from_slices(N, L, P, D, pop):
 def test_instances_by_the_members_of_an_sm(L, pop):
     """On two SMs: chains that start beside the launch before them, four to an SM, and more; twelve warps of 168 registers to an SM,
     with a chain each or with two, and more of 128."""
-    spec = ("instances", 80, L, 64, 32, 3, None, 3, pop)
+    R = 3 if pop > 16 else 40                   # (few members: rank loads that do not fit on chip)
+    spec = ("instances", 80 if R == 3 else 200, L, 64, 32, 3, None, R, pop)
     w = compressed_window(spec)
-    ref = oracle_front(w, None, 3)
-    ctx = load(w, pop=pop, min_rows=3)
+    ref = oracle_front(w, None, R)
+    ctx = load(w, pop=pop, min_rows=R)
     rp.rp_debug_set_knob(ctx, "CHAIN_KERNEL", 3)
     rp.rp_debug_set_knob(ctx, "RESIDENT_SMS", 2)
     check_front(w, ctx, ref)
