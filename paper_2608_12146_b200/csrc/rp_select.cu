@@ -358,7 +358,7 @@ k_sel_dist(RpDims dm, int Ppop, int n_proj, const int *__restrict__ rep, SelBuf 
 // ---- greedy selection (one CTA) -------------------------------------------------------------------
 // One selection after the other: a step is the load of one row of distances, three warp-wide minima, one barrier and the
 // same minima over the warps' results, which every warp works out for itself (256 candidates, distances in L2, 220 us; a shuffle tree
-// over triples, a serial pass of one thread and two barriers over 32 warps took 920).
+// over triples, a serial pass of one thread and two barriers over 32 warps took 920); by a single warp where the distances are on chip.
 #define GREEDY_THREADS 1024
 #define GREEDY_SMEM (160 * 1024)        // nearest distances and penalties of the candidates on chip up to this
 // The distances themselves on chip, each pair once, where they fit (up to 307 candidates): a step then does not wait for L2 (256
@@ -367,6 +367,42 @@ k_sel_dist(RpDims dm, int Ppop, int n_proj, const int *__restrict__ rep, SelBuf 
 #define GREEDY_DIST_MAX (184 * 1024)
 static inline size_t greedy_tri(size_t P) { return P * (P - 1) / 2; }
 struct SelPick { i64 v0, v1, v2; int j; };
+
+// The steps by one warp, E candidates a lane: distances to the nearest selected one and penalties in registers, pairs in `near`; penalties
+// below 2^30.  A step is a load, a minimum and a compare a candidate and two warp-wide minima, and no barrier (256 candidates 196 -> 70 us; 253
+// where a branch around each load made one wait for the other).
+template <int E>
+__device__ __forceinline__ void greedy_by_warp(int Ppop, int nd, int last, const u32 *near, const i64 *mind, const i64 *pen, int *__restrict__ order, int lane)
+{
+    u32 m[E], p[E], left = 0;                                    // left: candidates not selected yet
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int j = lane + 32 * e;
+        const bool on = j < Ppop && mind[min(j, Ppop - 1)] >= 0;
+        m[e] = 0xffffffffu; p[e] = on ? (u32)pen[j] : 0;
+        left |= on ? 1u << e : 0;
+    }
+    for (int n = 0; n < nd; ++n) {
+        if (lane == 0) order[n] = last;
+        if (lane == (last & 31)) left &= ~(1u << (last >> 5));
+        const int row = last * (last - 1) / 2;
+        u32 best = 0xffffffffu, who = 0xffffffffu, d[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {                            // (all at once: an entry that is not used is read, at 0)
+            const int j = lane + 32 * e, at = j > last ? j * (j - 1) / 2 + last : row + j;
+            d[e] = near[(left >> e) & 1u ? at : 0];
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            m[e] = min(m[e], d[e]);
+            const u32 key = (left >> e) & 1u ? p[e] - m[e] + 0x80000000u : 0xffffffffu;
+            who = key < best ? (u32)(lane + 32 * e) : who;       // (ties: the lower index)
+            best = min(best, key);
+        }
+        const u32 top = __reduce_min_sync(0xffffffffu, best);
+        last = (int)__reduce_min_sync(0xffffffffu, best == top ? who : 0xffffffffu);
+    }
+}
 
 __global__ void __launch_bounds__(GREEDY_THREADS)
 k_sel_greedy(int Ppop, const int *__restrict__ rep, const i64 *__restrict__ score, const i64 *__restrict__ dist,
@@ -416,6 +452,7 @@ k_sel_greedy(int Ppop, const int *__restrict__ rep, const i64 *__restrict__ scor
     const int nd = nd_s;
     const i64 s0 = pick_s.v0;
     int last = pick_s.j;
+    bool large = false;                                    // a penalty that 30 bits do not hold
     for (int j = tid; j < Ppop; j += nt) {
         i64 p = 0;
         if (rep[j] && s0 > 0) {
@@ -423,20 +460,27 @@ k_sel_greedy(int Ppop, const int *__restrict__ rep, const i64 *__restrict__ scor
             p = (i64)((gap * (unsigned __int128)(u64)eta_q16) >> 16);
         }
         pen[j] = p;
+        large |= (u64)p >> 30;
         mind[j] = rep[j] ? 0x7fffffffffffffffll : -1;      // -1 = not a candidate (or already selected)
     }
     __syncthreads();
     // pair (i, j), i > j, at i (i - 1) / 2 + j
     u32 *near = (u32 *)(greedy_smem + 2 * (size_t)Ppop);
     if (tri) {
-        for (int i = warp; i < Ppop; i += nw)
-#pragma unroll 4
-            for (int j = lane; j < i; j += 32) {
-                if (mind[i] < 0 || mind[j] < 0) continue;            // (no distance to a plan that stands for no class)
-                near[i * (i - 1) / 2 + j] = (u32)__ldg(dist + (size_t)i * Ppop + j);
-            }
-        __syncthreads();
+        for (int i = warp; i < Ppop; i += nw)                        // (no distance is used to a plan that stands for no class)
+#pragma unroll 8
+            for (int j = lane; j < i; j += 32) near[i * (i - 1) / 2 + j] = (u32)__ldg(dist + (size_t)i * Ppop + j);
     }
+    large = __syncthreads_or(large);
+    if (tri && !large) {
+        if (warp == 0) {
+            if (Ppop <= 64) greedy_by_warp<2>(Ppop, nd, last, near, mind, pen, order, lane);
+            else if (Ppop <= 128) greedy_by_warp<4>(Ppop, nd, last, near, mind, pen, order, lane);
+            else if (Ppop <= 256) greedy_by_warp<8>(Ppop, nd, last, near, mind, pen, order, lane);
+            else greedy_by_warp<10>(Ppop, nd, last, near, mind, pen, order, lane);
+        }
+        __syncthreads();
+    } else
     for (int n = 0; n < nd; ++n) {
         if (tid == 0) order[n] = last;
         // negated objective, as an unsigned number, so that the minimum applies: maximise distance - penalty, lowest index
@@ -533,9 +577,9 @@ int rp_launch_select(rp_ctx *c, int *lay, int *out, const i64 *score, int n_proj
                 if (dm.N <= 65535) k_sel_dist<u32><<<grid, SEL_THREADS, ctab + rtab, c->stream>>>(dm, (int)P, n_proj, rep, B, dist, (int)ctab, (int)rtab);
                 else k_sel_dist<u64><<<grid, SEL_THREADS, ctab + rtab, c->stream>>>(dm, (int)P, n_proj, rep, B, dist, (int)ctab, (int)rtab);
             }
-            const int gt = (int)std::min<size_t>(GREEDY_THREADS, (P + 31) / 32 * 32);
             const int tri = greedy_smem && sizeof(u32) * greedy_tri(P) <= GREEDY_DIST_MAX;
-            const size_t gm = greedy_smem ? 2 * sizeof(i64) * P + (tri ? sizeof(u32) * greedy_tri(P) : 0) : 0;
+            const int gt = tri ? GREEDY_THREADS : (int)std::min<size_t>(GREEDY_THREADS, (P + 31) / 32 * 32);
+            const size_t gm = greedy_smem ? 2 * sizeof(i64) * P + (tri ? sizeof(u32) * greedy_tri(P) + 16 : 0) : 0;        // (one pair at least)
             if (e == cudaSuccess && gm > 32 * 1024) e = cudaFuncSetAttribute(k_sel_greedy, cudaFuncAttributeMaxDynamicSharedMemorySize, RP_SMEM_LIMIT);
             if (e == cudaSuccess)
                 k_sel_greedy<<<1, gt, gm, c->stream>>>((int)P, rep, score, dist, eta_q16, mind, pen, order, n_distinct, tri);

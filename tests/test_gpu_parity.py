@@ -1932,3 +1932,20 @@ def test_instances_by_the_members_of_an_sm(L, pop):
     _, stats = check_anneal(w, ctx, ref, None, pop, 4, 70, t_ratio=0.6, check_members=2, t0=1e-2)
     assert rp.rp_debug_chain_form(ctx) == ("two to a warp" if pop > 32 else "compressed") and stats.accepted > 0
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("pop,eta", [(64, 0), (65, 1 << 16), (128, 1 << 20), (129, 1 << 16), (256, 1 << 16), (257, 1 << 18), (40, 1 << 40), (307, 1 << 40)])
+def test_greedy_order_by_one_warp(pop, eta):
+    """Two, four, eight and ten candidates a lane, filled and one more; penalties that 30 bits do not hold."""
+    w = make_window(custom_spec("greedy_warp", 60, 5, 16, 2, 4096, 3, 4, pop, 0, data_seed=4))
+    s = w.spec
+    ref = oracle_front(w, None, 3)
+    ctx = load(w, pop=pop, min_rows=3)
+    check_front(w, ctx, ref)
+    lays, ok = oracle.seed_trials(w.lengths, ref["seed"], ref["R"], s.token_cap, 3, pop, 5, s.anneal_seed)
+    assert rp.rp_seed_population(ctx, 5) == int(ok.sum())
+    sc = oracle.eval_layouts(w.lengths, ref["q"], lays, ref["R"], s.token_cap, 3, None, s.alpha, s.beta)["score"]
+    want = oracle.select_population(w.lengths, ref["q"], lays, sc, ref["R"], s.token_cap, 3, s.top_k, 4, eta, s.anneal_seed)
+    nd, order = rp.rp_select_population(ctx, 4, eta)
+    assert nd == want["n_distinct"] and (order == want["order"]).all()
+    rp.rp_destroy(ctx)
