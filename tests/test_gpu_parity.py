@@ -1949,3 +1949,25 @@ def test_greedy_order_by_one_warp(pop, eta):
     nd, order = rp.rp_select_population(ctx, 4, eta)
     assert nd == want["n_distinct"] and (order == want["order"]).all()
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,longest,width", [(700, 1, 1), (700, 3, 4), (767, 2, 1), (768, 1, 1)])
+def test_trials_whose_cells_outgrow_short_keys(N, longest, width):
+    """Six cells of 2^20 tokens: keys of 32 bits count 511 samples of a cell (up to 767 samples in the window); with one cell to
+    choose from the fullest takes all of the short samples, more than that."""
+    rng = np.random.default_rng(N + width)
+    t = rng.integers(1, longest + 1, N)
+    t[rng.permutation(N)[:6]] = rng.integers(800_000, 1_000_000, 6)
+    s = custom_spec("short_keys", N, 2, 4, 2, 1 << 20, 6, 4, 5, 0)
+    a = np.zeros((N, 2, 4), np.int32)
+    for l in range(2):
+        a[np.arange(N), l, rng.integers(0, 4, N)] = 2 * t
+    w = Window(s, t.astype(np.int32), a)
+    ref = oracle_front(w, None)
+    ctx = load(w, pop=5)
+    check_front(w, ctx, ref)
+    lays, ok = oracle.seed_trials(w.lengths, ref["seed"], ref["R"], s.token_cap, 6, 5, width, s.anneal_seed)
+    assert rp.rp_seed_population(ctx, width) == int(ok.sum())
+    assert (rp.rp_debug_dump(ctx, "POPULATION", (5, N), np.int32) == lays).all()
+    assert ref["R"] == 1 and (max(np.bincount(x).max() for x in lays[1:]) > 511) == (width == 1)
+    rp.rp_destroy(ctx)
