@@ -459,7 +459,7 @@ bool rp_uses_row(const rp_ctx *c) { return rp_may_use_row(c) && !(rp_row_compres
 // everything as it is (the chains of the remaining levels do nothing either).  Indices are
 // checked before they are used, so that a broken table can only raise the status word.
 __global__ void k_slice_holders(const char *__restrict__ blobs, RpBlob bl, const int *__restrict__ anc, int RG, int P, int ns,
-                                int *__restrict__ ref, int *__restrict__ head, int *__restrict__ status)
+                                int *__restrict__ ref, int *__restrict__ head, int *__restrict__ status, int members)
 {
     if (__ldcg(&status[RP_SW_TIMEOUT])) return;
     const int a = anc[blockIdx.x];
@@ -467,7 +467,7 @@ __global__ void k_slice_holders(const char *__restrict__ blobs, RpBlob bl, const
     const int *tab = (const int *)(blobs + (size_t)a * bl.bytes + bl.off_wtab);
     for (int rg = threadIdx.x; rg < RG; rg += blockDim.x) {
         const int s = tab[rg];
-        if ((unsigned)s < (unsigned)ns) atomicAdd(&ref[s], 1);
+        if ((unsigned)s < (unsigned)ns) atomicAdd(&ref[s], members);
         else atomicExch(&status[RP_SW_POOL], 1);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) { head[0] = 0; head[1] = 0; }
@@ -500,8 +500,11 @@ k_slice_free_list(int *__restrict__ ref, int *__restrict__ holders, int n, int *
 int rp_launch_slice_gc(rp_ctx *c)
 {
     const int ns = 2 * c->Ppop * c->dm.RG, nb = (ns + SLICE_BLOCK - 1) / SLICE_BLOCK;
-    k_slice_holders<<<c->Ppop, 128, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, c->dm.RG, c->Ppop, ns, c->d_wcount,
-                                                    c->d_wfree_head, c->d_status);
+    // (a population just set up descends from its first member as a whole: 1024 additions to each of 240 addresses took 10 us)
+    const int one = c->one_ancestor;
+    c->one_ancestor = 0;
+    k_slice_holders<<<one ? 1 : c->Ppop, 128, 0, c->stream>>>(c->buf[c->cur].blob, c->bl, c->d_anc, c->dm.RG, c->Ppop, ns, c->d_wcount,
+                                                             c->d_wfree_head, c->d_status, one ? c->Ppop : 1);
     k_slice_free_list<<<nb, SLICE_BLOCK, 0, c->stream>>>(c->d_wcount, c->d_wref, ns, c->d_wfree, c->d_wfree_head, c->d_status);
     g_rp_launches += 2; c->n_queued += 2;
     RP_CUDA(cudaGetLastError());

@@ -297,7 +297,8 @@ int rp_launch_member_rows(rp_ctx *c, int n)
     const size_t smem = sep ? sizeof(int) * (size_t)dm.N : 0;
     if (smem > 200 * 1024) return RP_ERR_RANGE;
     if (smem > 32 * 1024) RP_CUDA(cudaFuncSetAttribute(k_member_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024)));
-    RP_CUDA(cudaMemsetAsync(c->d_undecided, 0, sizeof(int), c->stream));
+    if (!c->undecided_clear) RP_CUDA(cudaMemsetAsync(c->d_undecided, 0, sizeof(int), c->stream));
+    c->undecided_clear = 0;
     i64 *Fo = c->d_rowF + (size_t)c->cur * c->Ppop * dm.RG;
     if (!sep)                       // (a chain keeps 40 bytes of a row-shard in shared memory: no more than 5632)
         k_member_slack<<<n, 256, sizeof(uint2) * (size_t)dm.RG, c->stream>>>(dm, c->bl, c->buf[c->cur].blob, c->d_static, c->sl, (const int2 *)c->d_tf, Fo,

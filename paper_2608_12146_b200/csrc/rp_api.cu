@@ -601,6 +601,7 @@ static int build_population(rp_ctx *c, bool candidates, bool same_rows)
     stage_mark(c, RP_EV_SEED_0, c->stream);
     RP_TRY(rp_launch_setup_population(c));
     c->log_clean = 1;
+    c->one_ancestor = 1; c->undecided_clear = 1;
     RP_TRY(rp_launch_eval_seed(c));
     c->rows_made = 0;
     forget_rows(c, 1);
@@ -683,6 +684,7 @@ static int install_population(rp_ctx *c, const int *lay, int n_distinct = 0)
     const size_t P = (size_t)c->Ppop;
     const size_t ne = (n_distinct > 0 && (size_t)n_distinct < P) ? (size_t)n_distinct : P;
     c->best_ready = 0;
+    c->one_ancestor = 0;
     i64 *best = nullptr;
     RP_TRY(dev_alloc(c, &best, 3));
     int st = ensure_eval_scratch(c, ne, false);
@@ -1065,6 +1067,7 @@ extern "C" int rp_anneal(rp_ctx *c, const rp_anneal_params *p, rp_anneal_stats *
     // What the context says about the population changes with the levels that have run, and with nothing that was refused
     // before them: a call that fails here can be followed by one that does not.
     auto levels_ran = [&]() {
+        c->one_ancestor = 0;
         if (!row) c->rows_current = 0;
         c->row_members = c->Ppop;              // after a level every member has a state of its own
         c->full_stale = row && rp_row_separate(c);

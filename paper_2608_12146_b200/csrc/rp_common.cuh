@@ -184,6 +184,8 @@ struct rp_ctx {
     int log_cap;
     u64 *d_F;                  // [P_pop] cumulative weights; the one-layer-per-lane kernel: [2*P_pop] energies and weights, then the smallest energy
     int slices_listed;         // the level before has left holders and free slices for the next one
+    int one_ancestor;          // all members descend from the first, no level has run since
+    int undecided_clear;       // d_undecided is zero
     i64 *d_counters;           // [4]
     // incumbent
     int *d_inc_layout;         // [N]
