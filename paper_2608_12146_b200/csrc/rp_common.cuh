@@ -389,21 +389,35 @@ __device__ __constant__ const u64 RP_EXP2_Q63[24] = {
     0x7FFFFE9D1BD1FC58ULL, 0x7FFFFF4E8DE8832DULL, 0x7FFFFFA746F422D6ULL,
 };
 
-// 2^(-z), z unsigned Q32 -> Q32 (2^32 = 1.0); 24 fraction bits of z are used.
-__device__ __forceinline__ u64 rp_exp2neg(u64 z)
+// 2^(-f / 2^24) in Q32 by its definition: the constants of f's bits multiplied up in Q63, each product cut off.
+static __device__ __noinline__ u64 rp_exp2neg_product(u32 f)
 {
-    u64 ip = z >> 32;
-    if (ip >= 32) return 0;
     u64 acc = 1ull << 63;
 #pragma unroll 1
     for (int i = 1; i <= 24; ++i) {
-        if ((z >> (32 - i)) & 1ull) {
-            u64 c = RP_EXP2_Q63[i - 1];
+        if ((f >> (24 - i)) & 1u) {
+            const u64 c = RP_EXP2_Q63[i - 1];
             // (acc * c) >> 63 with a 128-bit product
             acc = (__umul64hi(acc, c) << 1) | ((acc * c) >> 63);
         }
     }
-    return (acc >> 31) >> ip;
+    return acc >> 31;
+}
+
+// 2^(-z), z unsigned Q32 -> Q32 (2^32 = 1.0); 24 fraction bits of z are used.  In double precision: exp2 is within 2^-20 of 2^32 * 2^(-f / 2^24)
+// (one unit in the last place), and so are the product's 24 roundings together (2^-26), so that both have the same integer part wherever that of the first
+// is 2^-16 and more from the next integer below and above; elsewhere (one fraction in 32768) the product itself.  (The product alone, 24
+// dependent 64-bit multiplications and their selections, took 3 to 4 k of a level barrier's cycles with a member a thread.)
+__device__ __forceinline__ u64 rp_exp2neg(u64 z)
+{
+    const u32 f = (u32)z >> 8;
+    const double x = exp2(32.0 - (double)f * 0x1p-24);
+    u64 q = __double2ull_rz(x);
+    const double r = x - __ull2double_rn(q);
+    if (f == 0) q = 1ull << 32;
+    else if (!(r > 0x1p-16 && r < 1.0 - 0x1p-16)) q = rp_exp2neg_product(f);
+    const u64 ip = z >> 32;
+    return ip >= 32 ? 0 : q >> ip;
 }
 
 __device__ __forceinline__ bool rp_lex_less(i64 a0, i64 a1, i64 a2, i64 b0, i64 b1, i64 b2)

@@ -44,39 +44,13 @@ __device__ __forceinline__ u64 le_scaled_quotient(u64 Dd, u64 M, double rM)
 template <int U>
 __device__ __forceinline__ void le_weights(const i64 (&e)[U], i64 emin, u64 M, u64 cq, u64 (&w)[U])
 {
-    u64 z[U], acc[U];
     const double rM = 4294967296.0 / (double)M;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const u64 eq = le_scaled_quotient((u64)(e[u] - emin), M, rM);
         const u64 zh = __umul64hi(eq, cq), zl = eq * cq;
-        u64 zz = (zh >> 16) ? (1ull << 40) : ((zh << 48) | (zl >> 16));
-        z[u] = zz > (1ull << 40) ? (1ull << 40) : zz;
-        acc[u] = 1ull << 63;
-    }
-    // the fraction bits in the order of rp_exp2neg; a clear bit multiplies by one (2^63 in Q63), which is exact
-    // (acc * cc) >> 63 = high word of (2*acc) * cc; acc = 2^63 (nothing applied yet) gives cc itself
-    if constexpr (U == 1) {          // one member per thread: a single dependent chain, unrolled (constants inline)
-#pragma unroll
-        for (int i = 1; i <= 24; ++i) {
-            const u64 cc = ((z[0] >> (32 - i)) & 1ull) ? RP_EXP2_Q63[i - 1] : (1ull << 63);
-            acc[0] = (acc[0] >> 63) ? cc : __umul64hi(acc[0] << 1, cc);
-        }
-    } else {
-#pragma unroll 1
-        for (int i = 1; i <= 24; ++i) {
-            const u64 c = RP_EXP2_Q63[i - 1];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const u64 cc = ((z[u] >> (32 - i)) & 1ull) ? c : (1ull << 63);
-                acc[u] = (acc[u] >> 63) ? cc : __umul64hi(acc[u] << 1, cc);
-            }
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const u64 ip = z[u] >> 32;
-        w[u] = ip >= 32 ? 0 : (acc[u] >> 31) >> ip;
+        const u64 z = (zh >> 16) ? (1ull << 40) : ((zh << 48) | (zl >> 16));
+        w[u] = rp_exp2neg(z > (1ull << 40) ? (1ull << 40) : z);
     }
 }
 

@@ -1971,3 +1971,16 @@ def test_trials_whose_cells_outgrow_short_keys(N, longest, width):
     assert (rp.rp_debug_dump(ctx, "POPULATION", (5, N), np.int32) == lays).all()
     assert ref["R"] == 1 and (max(np.bincount(x).max() for x in lays[1:]) > 511) == (width == 1)
     rp.rp_destroy(ctx)
+
+
+def test_weights_next_to_an_integer():
+    """Fractions whose power lies so close to an integer that double precision does not decide it, all of them, their neighbours, and
+    whole exponents with and without a fraction."""
+    f = np.arange(1 << 24, dtype=np.uint64)
+    y = np.exp2(32.0 - f * 2.0 ** -24)
+    r = y - np.floor(y)
+    near = f[(r < 2.0 ** -15) | (r > 1 - 2.0 ** -15)]
+    assert 500 < near.size < 2000 and near[0] == 0
+    z = np.concatenate([near, near[1:] - 1, near[:-1] + 1, np.random.default_rng(1).integers(0, 1 << 24, 4000, dtype=np.uint64)]) << np.uint64(8)
+    z = np.concatenate([z, z + np.uint64(255), z + (np.uint64(3) << np.uint64(32)), z + (np.uint64(31) << np.uint64(32))])
+    assert rp.rp_debug_exp2neg(z).tolist() == [oracle.exp2neg(int(v)) for v in z]
