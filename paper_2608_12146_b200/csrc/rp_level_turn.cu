@@ -5,21 +5,22 @@
 // other: what bounds them is latency, 34 us a level at 1024 members of 240 row-shards with the gaps.  Here the worker CTAs
 // share the members out, meet once or twice and otherwise never wait; the last CTA looks after the incumbent (whose move log is
 // replayed by a warp) beside them.  The chains leave their energies and the smallest of them behind.
-//   1. weights, and all cumulative weights (every worker for itself).  Up to 512 members every worker weighs them all, a member a thread
-//      (5.7 k cycles, without a meeting; shared out, a meeting and the sums behind it 8.5 k); more are shared out (two members a
-//      thread weighed by every worker: 10.9 k cycles at 1024)
+//   1. weights, and all cumulative weights (every worker for itself).  Up to 1024 members every worker weighs them all, one or two a thread, and
+//      there is no meeting (1024 members 2345 and 2324 us; four a thread at 1500 and 2048 gave nothing); more are shared out
 //   2. ancestors of its members by 32 probes a step, the holders of the slices of each one that occurs
 //   3. its piece of the slice table: free slices to the list, the counts of the level before back to zero (two tables taken in turn)
 // In us a launch, 300 members of 100 row-shards 10.0 before, 9.0 here, 512 of 240 11.0 and 9.9, 1024 of 240 14, 4096 of 288 28 and 23.  What is left is
 // trips to L2: two loads, a meeting of 2.5 k cycles and what the additions before it take to arrive, two loads and an addition.
 #include <algorithm>
 #include <string.h>
+#include <type_traits>
 
 #include "rp_level_end.cuh"
 #include "rp_anneal_row.cuh"
 
 #define TURN_THREADS 512
 #define TURN_WARPS (TURN_THREADS / 32)
+#define TURN_OWN 2                       // members a thread whose weights every worker works out for itself
 #define TURN_ROWS 32
 #define TURN_MAX_MEMBERS 16384           // cumulative weights on chip (with their padding, 136 KB)
 
@@ -52,7 +53,7 @@ k_level_turn(const AnnealArgs A, const TurnArgs T)
     __shared__ LeShared S;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int workers = (int)gridDim.x - 1, P = A.Ppop, RG = A.dm.RG;
-    const bool own_weights = P <= TURN_THREADS;
+    const bool own_weights = P <= TURN_OWN * TURN_THREADS;
     if (T.early) rp_let_next_launch_start();
     if ((int)blockIdx.x == workers) {
         if (__ldcg(&A.status[RP_SW_TIMEOUT])) return;
@@ -68,27 +69,36 @@ k_level_turn(const AnnealArgs A, const TurnArgs T)
     int lu = 0;
     const int late = __ldcg(&A.status[RP_SW_TIMEOUT]);
     const i64 emin = (i64)__ldcg(T.emin);
-    const int mine = own_weights ? tid : m0 + tid, end = own_weights ? P : m1;
-    const i64 e[1] = { mine < end ? (i64)__ldcg(T.E + mine) : emin };
-    if (late) return;
     const u64 M = (u64)(emin > A.dm.SC ? emin : A.dm.SC);
-    u64 own = 0, v;
-    if (mine < end) { u64 w[1]; le_weights<1>(e, emin, M, A.cq, w); own = w[0]; }
-    if (!own_weights) {
-        if (mine < end) T.weight[mine] = own;
-        for (int m = mine + TURN_THREADS; m < end; m += TURN_THREADS) {        // (few SMs: more than a member a thread)
-            const i64 f[1] = { (i64)__ldcg(T.E + m) };
+    while ((TURN_THREADS << lu) < P) ++lu;
+    const int j0 = tid << lu, j1 = min(P, j0 + (1 << lu));
+    u64 own = 0;
+    auto weigh = [&](auto count) {                               // its own members, worked out here
+        constexpr int U = decltype(count)::value;
+        i64 e[U];
+        u64 w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) e[u] = j0 + u < P ? (i64)__ldcg(T.E + j0 + u) : emin;
+        le_weights<U>(e, emin, M, A.cq, w);
+#pragma unroll
+        for (int u = 0; u < U; ++u) if (j0 + u < P) { own += w[u]; F[j0 + u + (j0 + u) / U] = own; }
+    };
+    if (own_weights) {
+        if (late) return;
+        if (lu == 0) weigh(std::integral_constant<int, 1>());
+        else weigh(std::integral_constant<int, TURN_OWN>());
+    } else {
+        if (late) return;
+        for (int m = m0 + tid; m < m1; m += TURN_THREADS) {
+            const i64 e[1] = { (i64)__ldcg(T.E + m) };
             u64 w[1];
-            le_weights<1>(f, emin, M, A.cq, w);
+            le_weights<1>(e, emin, M, A.cq, w);
             T.weight[m] = w[0];
         }
         if (!turn_meet(A, T.base + workers)) { if (tid == 0) atomicExch(&A.status[RP_SW_TIMEOUT], 1); return; }
-        while ((TURN_THREADS << lu) < P) ++lu;
-        own = 0;
+        for (int j = j0; j < j1; ++j) { own += __ldcg(T.weight + j); F[j + (j >> lu)] = own; }
     }
-    const int j0 = tid << lu, j1 = min(P, j0 + (1 << lu));
-    if (!own_weights) for (int j = j0; j < j1; ++j) { own += __ldcg(T.weight + j); F[j + (j >> lu)] = own; }
-    v = own;
+    u64 v = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) { const u64 x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
     if (lane == 31) S.rsum[warp] = v;
@@ -96,8 +106,7 @@ k_level_turn(const AnnealArgs A, const TurnArgs T)
     u64 before = v - own;
 #pragma unroll
     for (int x = 0; x < TURN_WARPS; ++x) { const u64 y = S.rsum[x]; if (x < warp) before += y; }
-    if (own_weights) { if (tid < P) F[2 * tid] = before + own; }
-    else for (int j = j0; j < j1; ++j) F[j + (j >> lu)] += before;
+    for (int j = j0; j < j1; ++j) F[j + (j >> lu)] += before;
     __syncthreads();
     if (blockIdx.x == 0 && tid == 0) { T.head[0] = 0; T.head[1] = 0; }
 
@@ -235,7 +244,7 @@ int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A0)
     A.sync = c->d_sync;
     // Workers: as many as have something to do (a meeting costs the more the more there are); every one resident.
     const int workers = std::max(4, std::min(rp_sms(c) - 1, std::max((P + 15) / 16, (ns + 4095) / 4096)));
-    T.base = A.level * (P <= TURN_THREADS ? 1 : 2) * workers;                  // (the count is zero when the call starts)
+    T.base = A.level * (P <= TURN_OWN * TURN_THREADS ? 1 : 2) * workers;                  // (the count is zero when the call starts)
     int lu = 0;
     while ((TURN_THREADS << lu) < P) ++lu;
     const size_t ws_workers = sizeof(u64) * ((size_t)P + (P >> lu) + 1) + sizeof(int) * 3 * ((size_t)P / workers + 3);

@@ -1984,3 +1984,15 @@ def test_weights_next_to_an_integer():
     z = np.concatenate([near, near[1:] - 1, near[:-1] + 1, np.random.default_rng(1).integers(0, 1 << 24, 4000, dtype=np.uint64)]) << np.uint64(8)
     z = np.concatenate([z, z + np.uint64(255), z + (np.uint64(3) << np.uint64(32)), z + (np.uint64(31) << np.uint64(32))])
     assert rp.rp_debug_exp2neg(z).tolist() == [oracle.exp2neg(int(v)) for v in z]
+
+
+@pytest.mark.parametrize("pop", [511, 512, 513, 1024, 1025])
+def test_between_two_levels_by_members_a_thread(pop):
+    """One member a thread weighed by every worker, two, and more, shared out; full and not."""
+    w = make_window(custom_spec("members", 600, 3, 8, 2, 2048, 4, 4, pop, 0, data_seed=140))
+    ref = oracle_front(w, None, 140)
+    ctx = load(w, pop=pop, min_rows=140)
+    check_front(w, ctx, ref)
+    _, stats = check_anneal(w, ctx, ref, None, pop, 4, 24, t_ratio=0.4, check_members=2, t0=3e-3)
+    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.kernel_launches == 2 * 4 + 2
+    rp.rp_destroy(ctx)
