@@ -253,12 +253,9 @@ __device__ __forceinline__ void row_barrier_warp(const AnnealArgs &A, int P, con
 {
     const u64 r = lane < P ? __ldcg(eL + lane) : 0x7fffffffffffffffull;
     const i64 e[1] = { (i64)(r & ~(1ull << 63)) };
-    i64 b0 = inc[0], b1 = inc[1], b2 = inc[2];
-    int bj = 0x7fffffff;
-    if (r >> 63) {                               // its trajectory best beats the incumbent
-        b0 = __ldcg(bestL + 3 * lane); b1 = __ldcg(bestL + 3 * lane + 1); b2 = __ldcg(bestL + 3 * lane + 2);
-        bj = lane;
-    }
+    // (fetched beside the energy, whether its trajectory best beats the incumbent or not)
+    const i64 b0 = lane < P ? __ldcg(bestL + 3 * lane) : 0, b1 = lane < P ? __ldcg(bestL + 3 * lane + 1) : 0, b2 = lane < P ? __ldcg(bestL + 3 * lane + 2) : 0;
+    const int bj = r >> 63 ? lane : 0x7fffffff;
     const u32 hi = (u32)((u64)e[0] >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
     const i64 emin = (i64)(((u64)mh << 32) | __reduce_min_sync(0xffffffffu, hi == mh ? (u32)e[0] : 0xffffffffu));
     int slot = -1;
@@ -955,12 +952,9 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
             // meetings of the CTA and a search of eight dependent steps as below: medium 849 us, here 807; two shards 859 and 816).
             const u64 r = tid < P ? __ldcg(eL + tid) : ~0ull >> 1;
             i64 e[1] = { (i64)(r & ~(1ull << 63)) };
-            i64 b0 = 0, b1 = 0, b2 = 0;
-            int bj = 0x7fffffff;
-            if (r >> 63) {                               // its trajectory best beats the incumbent
-                b0 = __ldcg(bestL + 3 * tid); b1 = __ldcg(bestL + 3 * tid + 1); b2 = __ldcg(bestL + 3 * tid + 2);
-                bj = tid;
-            }
+            // (fetched beside the energy, whether its trajectory best beats the incumbent or not)
+            const i64 b0 = tid < P ? __ldcg(bestL + 3 * tid) : 0, b1 = tid < P ? __ldcg(bestL + 3 * tid + 1) : 0, b2 = tid < P ? __ldcg(bestL + 3 * tid + 2) : 0;
+            const int bj = r >> 63 ? tid : 0x7fffffff;
             const u32 hi = (u32)((u64)e[0] >> 32), mh = __reduce_min_sync(0xffffffffu, hi), ml = __reduce_min_sync(0xffffffffu, hi == mh ? (u32)e[0] : 0xffffffffu);
             if (lane == 0) { rmin[warp] = (i64)(((u64)mh << 32) | ml); rj[warp] = 0x7fffffff; }
             if (__any_sync(0xffffffffu, bj != 0x7fffffff)) {
