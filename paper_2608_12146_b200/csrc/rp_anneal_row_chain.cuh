@@ -891,10 +891,10 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
         return;
     } else {
         // Meet the other chains: the reports are all they wait for, so arrive as soon as they are out.
-        __threadfence();
         __syncthreads();
         if (tid == 0) {
-            atomicAdd(A.sync, 1);
+            // (one thread's release covers what the CTA's threads wrote before they met)
+            asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(A.sync) : "memory");
             // (the pool may be written once every chain has read its start state)
             failed_s = (ln == 0 && !rp_wait_count(A.lo.done, (int)gridDim.x, A)) ? 1 : 0;
         }
@@ -923,7 +923,6 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
                 for (int rg = ht; rg < dm.RG; rg += hn) td[rg] = (half_w * P + jj) * dm.RG + rg;
             }
         }
-        __threadfence();
         __syncthreads();
         if (tid < cw && blockIdx.x * cw + tid < P)
             asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(A.sync + 1 + blockIdx.x * cw + tid), "r"(ln + 1) : "memory");
