@@ -5,6 +5,8 @@
 // K1 and K3 stream the demand tensor a[N][L][E] once each and are bound by HBM bandwidth:
 // algorithmic bytes are N*L*E*4 read (+ N*L*P*4 written by K3).  K2 is a few microseconds
 // of integer work per layer.
+#include <algorithm>
+
 #include "rp_common.cuh"
 
 #define K1_WARPS 8
@@ -282,11 +284,12 @@ int rp_launch_check_reduce(rp_ctx *c)
 }
 
 // Algorithm 1 for one layer per CTA.  Experts are ranked by (-load, id) by counting how
-// many experts precede each one; then one warp assigns them in that order to the rank
+// many experts precede each one, four threads an expert; then one warp assigns them in that order to the rank
 // with the smallest (load, id) among ranks holding fewer than H experts.
+#define LPT_PARTS 4
 __global__ void __launch_bounds__(1024)
-k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
-      i64 *rank_load, int *__restrict__ top, const int *__restrict__ status, const i64 *__restrict__ t_sum,
+k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *__restrict__ pi, int *__restrict__ inv,
+      i64 *__restrict__ rank_load, int *__restrict__ top, const int *__restrict__ status, const i64 *__restrict__ t_sum,
       i64 *__restrict__ h_pin, int *__restrict__ h_pi, i64 *__restrict__ h_load)
 {
     extern __shared__ unsigned char smraw[];
@@ -294,6 +297,8 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
     i64 *G = load + dm.E;                     // [P]
     int *order = (int *)(G + dm.P);           // [E]
     int *cnt = order + dm.E;                  // [P]
+    u32 *sorted = (u32 *)(cnt + dm.P);        // [E] loads in that order (where 32 bits hold them)
+    int *place = (int *)(sorted + dm.E);      // [E] slots
     const int l = blockIdx.x;
     const i64 *Le = Lagg + (size_t)l * dm.E;
     // (queued behind the checks before their verdict: a window with negative counts is refused, but is placed until then, and
@@ -301,15 +306,18 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
     for (int e = threadIdx.x; e < dm.E; e += blockDim.x) load[e] = Le[e] > 0 ? Le[e] : 0;
     for (int p = threadIdx.x; p < dm.P; p += blockDim.x) { G[p] = 0; cnt[p] = 0; }
     __syncthreads();
-    for (int e = threadIdx.x; e < dm.E; e += blockDim.x) {
-        i64 mine = load[e];
+    for (int e0 = 0; e0 < dm.E; e0 += blockDim.x / LPT_PARTS) {
+        const int e = e0 + (int)threadIdx.x / LPT_PARTS;
+        const i64 mine = e < dm.E ? load[e] : 0;
         int before = 0;
 #pragma unroll 8
-        for (int f = 0; f < dm.E; ++f) {
+        for (int f = (int)threadIdx.x % LPT_PARTS; f < dm.E; f += LPT_PARTS) {
             const i64 o = load[f];
             before += (o > mine) || (o == mine && f < e);
         }
-        order[before] = e;
+#pragma unroll
+        for (int o = 1; o < LPT_PARTS; o <<= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        if (threadIdx.x % LPT_PARTS == 0 && e < dm.E) { order[before] = e; sorted[before] = (u32)mine; }
     }
     __syncthreads();
     if (threadIdx.x < 32 && dm.P <= 128) {
@@ -325,24 +333,28 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
         const bool narrow = dm.P <= 32 && total < 0xffffffffll;
         if (narrow) {
             // Every rank load fits 32 bits and there is a rank per lane: one reduction and a ballot find the least-loaded free
-            // rank (lowest id first), the next expert and its load are fetched a step ahead.  (350 -> 100 cycles an expert.)
-            u32 G0 = lane < dm.P ? 0u : 0xffffffffu;
-            int c0 = 0, e = order[0];
-            u32 le = (u32)load[e];
+            // rank (lowest id first), and nothing else is waited for: loads come in their order, a step ahead, and the slot takes the load's
+            // place until all are known (48 layers of 256 experts 38 us with two global stores and two dependent loads an expert, 28
+            // with a search for the lowest bit and a shuffle, 23 here; 24 of 128 21 and 13, 16 of 64 13.8 and 10.2).
+            u32 G0 = lane < dm.P ? 0u : 0xffffffffu, le = sorted[0];
+            const unsigned lower = (1u << lane) - 1;
+            int slot = lane * dm.H;                      // the rank's next one
+            const int end = slot + dm.H;
+#pragma unroll 4
             for (int x = 0; x < dm.E; ++x) {
-                const int e1 = order[x + 1 < dm.E ? x + 1 : x];
-                const u32 key = c0 < dm.H ? G0 : 0xffffffffu;
+                const u32 next = sorted[min(x + 1, dm.E - 1)];
+                const u32 key = slot < end ? G0 : 0xffffffffu;
                 const u32 least = __reduce_min_sync(0xffffffffu, key);
-                const int mp = __ffs(__ballot_sync(0xffffffffu, key == least)) - 1;
-                const u32 le1 = (u32)load[e1];
-                if (lane == mp) {
-                    const int slot = mp * dm.H + c0;
-                    pi[(size_t)l * dm.E + e] = slot;
-                    inv[(size_t)l * dm.E + slot] = e;
-                    G0 += le;
-                    c0 += 1;
-                }
-                e = e1; le = le1;
+                const bool in = key == least;
+                const unsigned who = __ballot_sync(0xffffffffu, in);
+                if (in && !(who & lower)) { sorted[x] = (u32)slot; G0 += le; ++slot; }
+                le = next;
+            }
+            __syncwarp();
+            for (int x = lane; x < dm.E; x += 32) {
+                const int e = order[x], s = (int)sorted[x];
+                place[e] = s;
+                inv[(size_t)l * dm.E + s] = e;
             }
             Gr[0] = lane < dm.P ? (i64)G0 : 0;
         }
@@ -367,7 +379,7 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
                 for (int u = 0; u < 4; ++u) {
                     if (u == (mp >> 5)) {
                         const int slot = mp * dm.H + cr[u];
-                        pi[(size_t)l * dm.E + e] = slot;
+                        place[e] = slot;
                         inv[(size_t)l * dm.E + slot] = e;
                         Gr[u] += le;
                         cr[u] += 1;
@@ -376,7 +388,7 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) { const int p = lane + 32 * u; if (p < dm.P) rank_load[(size_t)l * dm.P + p] = Gr[u]; else Gr[u] = -1; }
+        for (int u = 0; u < 4; ++u) { const int p = lane + 32 * u; if (p < dm.P) G[p] = Gr[u]; else Gr[u] = -1; }
         // the three busiest ranks (ties: lower rank), for the chain kernel's fixed ranks and compressed rows
         for (int x = 0; x < 3; ++x) {
             i64 best = -1;
@@ -407,30 +419,33 @@ k_lpt(const i64 *__restrict__ Lagg, RpDims dm, int *pi, int *__restrict__ inv,
             }
             if (lane == 0) {
                 int slot = bestP * dm.H + cnt[bestP];
-                pi[(size_t)l * dm.E + e] = slot;
+                place[e] = slot;
                 inv[(size_t)l * dm.E + slot] = e;
                 G[bestP] += load[e];
                 cnt[bestP] += 1;
             }
             __syncwarp();
         }
-        for (int p = lane; p < dm.P; p += 32) rank_load[(size_t)l * dm.P + p] = G[p];
     }
     // what the host is waiting for, straight into its memory: the verdict of the checks, the token total, the placement
     if (l == 0 && threadIdx.x < RP_SW_COUNT) ((int *)(h_pin + 56))[threadIdx.x] = status[threadIdx.x];
     if (l == 0 && threadIdx.x == 0) h_pin[8] = *t_sum;
-    if (h_pi) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < dm.E; e += blockDim.x) h_pi[(size_t)l * dm.E + e] = pi[(size_t)l * dm.E + e];
-        for (int p = threadIdx.x; p < dm.P; p += blockDim.x) h_load[(size_t)l * dm.P + p] = rank_load[(size_t)l * dm.P + p];
+    __syncthreads();
+    for (int e = threadIdx.x; e < dm.E; e += blockDim.x) {
+        pi[(size_t)l * dm.E + e] = place[e];
+        if (h_pi) h_pi[(size_t)l * dm.E + e] = place[e];
+    }
+    for (int p = threadIdx.x; p < dm.P; p += blockDim.x) {
+        rank_load[(size_t)l * dm.P + p] = G[p];
+        if (h_pi) h_load[(size_t)l * dm.P + p] = G[p];
     }
 }
 
 int rp_launch_lpt(rp_ctx *c)
 {
     const RpDims &dm = c->dm;
-    size_t smem = sizeof(i64) * (dm.E + dm.P) + sizeof(int) * (dm.E + dm.P);
-    int threads = dm.E < 32 ? 32 : (dm.E > 1024 ? 1024 : ((dm.E + 31) / 32) * 32);
+    size_t smem = sizeof(i64) * (dm.E + dm.P) + sizeof(int) * (3 * dm.E + dm.P);
+    int threads = dm.E < 32 ? 32 : std::min(1024, (LPT_PARTS * dm.E + 31) / 32 * 32);
     k_lpt<<<dm.L, threads, smem, c->stream>>>(c->d_Lagg, dm, c->d_pi, c->d_inv, c->d_rank_load, c->d_top, c->d_status,
                                                 c->d_counters + 7, c->h_pin, rp_mail_pi(c), rp_mail_rank_load(c));
     ++g_rp_launches;
