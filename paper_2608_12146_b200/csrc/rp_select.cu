@@ -232,12 +232,14 @@ k_sel_map(int N, int Ppop, const int *__restrict__ canon, const u64 *__restrict_
 // Pairs together in a group of both plans = sum over (group of a, group of b) of C(count, 2).  Every sample adds one to the
 // count of its pair of groups in shared memory; what the atomic returns is the number of samples before it there, and these
 // sum up to C(count, 2): no pass over the table.  Clearing stores a zero at the same places.  Bound by the shared-memory
-// atomics, two a sample (cells and rows): 32640 pairs of plans of 2048 samples in 240 cells 0.27 ms; looking every pair of a
+// atomics, two a sample (cells and rows): 32640 pairs of plans of 2048 samples in 240 cells 0.23 ms (0.28 with eight warps' 64-bit
+// additions to one address and groups fetched twice; the next plan's groups fetched ahead gave nothing); looking every pair of a
 // cell's samples up in the other plan took 4.15 ms.
 //
 // Counts are as narrow as the largest group of a allows when the whole table fits only so (8 bits up to 255 samples); where
 // no width fits, the groups of a are taken in blocks, whose samples are contiguous in a's grouped list.
 #define SEL_CHUNK 8             // plans b per work item
+#define SEL_HELD 8              // samples a thread keeps in registers
 struct SelTab { u32 *tab; int n, lbits, block; };      // n groups; counts of 2^lbits bits; groups of a per pass
 
 __device__ __forceinline__ SelTab sel_table(u32 *tab, size_t bytes, int n, int big)
@@ -280,30 +282,52 @@ __device__ __forceinline__ SUM sel_blocks(const SelTab &t, const int *list, cons
 
 // SUM: 32 bits hold the pairs of up to 65535 samples.
 template <typename SUM>
-__global__ void __launch_bounds__(SEL_THREADS)
+__global__ void __launch_bounds__(SEL_THREADS, 3)
 k_sel_dist(RpDims dm, int Ppop, int n_proj, const int *__restrict__ rep, SelBuf B, i64 *__restrict__ dist, int ctab_bytes, int rtab_bytes)
 {
     extern __shared__ __align__(16) u32 sel_tabs[];
-    __shared__ u64 acc[SEL_CHUNK][3];
-    const int tid = threadIdx.x, lane = tid & 31;
+    __shared__ u64 acc[SEL_CHUNK][3][SEL_WARPS];         // (a place a warp: 64-bit additions of eight warps to one address queue up)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = dm.N, K = dm.K, R = dm.R, F = 2 + dm.G * dm.L;
+    const bool held = N <= SEL_HELD * SEL_THREADS;       // a thread's samples fit its registers
     for (int x = tid; x < (ctab_bytes + rtab_bytes) / 4; x += SEL_THREADS) sel_tabs[x] = 0;
     const int chunks = (Ppop + SEL_CHUNK - 1) / SEL_CHUNK;
     for (size_t item = blockIdx.x; item < (size_t)chunks * Ppop; item += gridDim.x) {
         const int a = (int)(item % Ppop), b0 = (int)(item / Ppop) * SEL_CHUNK;
         if (b0 + SEL_CHUNK - 1 <= a || !rep[a]) continue;
-        if (tid < 3 * SEL_CHUNK) acc[tid / 3][tid % 3] = 0;
         __syncthreads();
         const SelTab ct = sel_table(sel_tabs, ctab_bytes, K, B.big[2 * a]), rt = sel_table(sel_tabs + ctab_bytes / 4, rtab_bytes, R, B.big[2 * a + 1]);
         const bool whole = ct.block == K && rt.block == R;
         const u32 *la = B.lab + (size_t)a * N;
         const i64 *pa = B.phi + (size_t)a * n_proj * R;
+        int ca[SEL_HELD], ra[SEL_HELD];                          // where the samples' groups of a start in the tables
+        if (held)
+#pragma unroll
+            for (int x = 0; x < SEL_HELD; ++x) {
+                const int i = tid + x * SEL_THREADS;
+                const u32 ga = i < N ? la[i] : 0;
+                ca[x] = (int)(ga & 0xffffu) * K; ra[x] = (int)(ga >> 16) * R;
+            }
         for (int u = 0; u < SEL_CHUNK; ++u) {
             const int b = b0 + u;
             if (b <= a || b >= Ppop || !rep[b]) continue;
             const u32 *lb = B.lab + (size_t)b * N;
             SUM bc = 0, br = 0;
-            if (whole) {
+            if (whole && held) {
+                u32 gb[SEL_HELD];
+#pragma unroll
+                for (int x = 0; x < SEL_HELD; ++x) gb[x] = tid + x * SEL_THREADS < N ? __ldg(lb + tid + x * SEL_THREADS) : 0;
+#pragma unroll
+                for (int x = 0; x < SEL_HELD; ++x)
+                    if (tid + x * SEL_THREADS < N) {
+                        bc += sel_add(ct, ca[x] + (int)(gb[x] & 0xffffu));
+                        br += sel_add(rt, ra[x] + (int)(gb[x] >> 16));
+                    }
+                __syncthreads();
+#pragma unroll
+                for (int x = 0; x < SEL_HELD; ++x)
+                    if (tid + x * SEL_THREADS < N) { sel_clear(ct, ca[x] + (int)(gb[x] & 0xffffu)); sel_clear(rt, ra[x] + (int)(gb[x] >> 16)); }
+            } else if (whole) {
 #pragma unroll 4
                 for (int i = tid; i < N; i += SEL_THREADS) {
                     const u32 ga = la[i], gb = lb[i];
@@ -322,32 +346,28 @@ k_sel_dist(RpDims dm, int Ppop, int n_proj, const int *__restrict__ rep, SelBuf 
                 br = sel_blocks<SUM, 16>(rt, B.rlist + (size_t)a * N, B.rstart + (size_t)a * (R + 1), la, lb, tid);
             }
             const i64 *pb = B.phi + (size_t)b * n_proj * R;
-            if (tid - lane < n_proj * R) {                       // sketch: the warps that have part of it
-                i64 sw = 0;
-                for (int x = tid; x < n_proj * R; x += SEL_THREADS) { const i64 d = pa[x] - pb[x]; sw += d < 0 ? -d : d; }
-                for (int o = 16; o; o >>= 1) sw += __shfl_xor_sync(0xffffffffu, sw, o);
-                if (lane == 0) atomicAdd((unsigned long long *)&acc[u][2], (unsigned long long)sw);
-            }
+            i64 sw = 0;                                          // sketch
+            for (int x = tid; x < n_proj * R; x += SEL_THREADS) { const i64 d = pa[x] - pb[x]; sw += d < 0 ? -d : d; }
+            if (tid - lane < n_proj * R) for (int o = 16; o; o >>= 1) sw += __shfl_xor_sync(0xffffffffu, sw, o);
             if (sizeof(SUM) == 4) {
                 const u32 sc = __reduce_add_sync(0xffffffffu, (u32)bc), sr = __reduce_add_sync(0xffffffffu, (u32)br);
                 bc = sc; br = sr;
             } else {
                 for (int o = 16; o; o >>= 1) { bc += __shfl_xor_sync(0xffffffffu, bc, o); br += __shfl_xor_sync(0xffffffffu, br, o); }
             }
-            if (lane == 0) {
-                atomicAdd((unsigned long long *)&acc[u][0], (unsigned long long)bc);
-                atomicAdd((unsigned long long *)&acc[u][1], (unsigned long long)br);
-            }
+            if (lane == 0) { acc[u][0][warp] = (u64)bc; acc[u][1][warp] = (u64)br; acc[u][2][warp] = (u64)sw; }
             __syncthreads();                                     // tables are clear again
         }
         const int b = b0 + tid;
         if (tid < SEL_CHUNK && b > a && b < Ppop && rep[b]) {
-            const i64 bc = (i64)acc[tid][0], br = (i64)acc[tid][1];
+            i64 bc = 0, br = 0, sw = 0;
+#pragma unroll
+            for (int w = 0; w < SEL_WARPS; ++w) { bc += (i64)acc[tid][0][w]; br += (i64)acc[tid][1][w]; sw += (i64)acc[tid][2][w]; }
             const i64 uc = B.pc[a] + B.pc[b] - bc, ur = B.pr[a] + B.pr[b] - br;
             i64 d = 0;
             if (uc) d += ((i64)1 << 20) - (bc << 20) / uc;
             if (ur) d += ((i64)1 << 20) - (br << 20) / ur;
-            d += ((i64)acc[tid][2] * 16) / ((i64)n_proj * R * F);
+            d += (sw * 16) / ((i64)n_proj * R * F);
             dist[(size_t)a * Ppop + b] = d;
             dist[(size_t)b * Ppop + a] = d;
         }
