@@ -451,10 +451,17 @@ k_eval_sum(const EvalArgs A, int n, int sgroups, int rpt, bool sum32)
     }
 }
 
+// Of 32 lanes' non-negative numbers: the largest, by its upper and its lower word; the sum (below 2^63), 21 bits of each at a time.
 __device__ __forceinline__ i64 few_warp_max(i64 v)
 {
-    for (int o = 16; o; o >>= 1) { const i64 w = __shfl_xor_sync(0xffffffffu, v, o); v = w > v ? w : v; }
-    return v;
+    const u32 hi = (u32)((u64)v >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+    return (i64)(((u64)mh << 32) | __reduce_max_sync(0xffffffffu, hi == mh ? (u32)v : 0u));
+}
+__device__ __forceinline__ i64 few_warp_sum(i64 v)
+{
+    const u64 lo = __reduce_add_sync(0xffffffffu, (u32)v & 0x1fffffu), mid = __reduce_add_sync(0xffffffffu, (u32)(v >> 21) & 0x1fffffu),
+              hi = __reduce_add_sync(0xffffffffu, (u32)(v >> 42));
+    return (i64)(lo + (mid << 21) + (hi << 42));
 }
 
 // Many layouts, last kernel: the scores from the row-shards' costs, and what is left of the blob.
@@ -521,7 +528,7 @@ k_eval_score(const EvalArgs A)
 static inline size_t eval_few_smem(const RpDims &dm, int MS)
 {
     const size_t part = (sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2) + 7) & ~(size_t)7;
-    return std::max(part + (size_t)16 * dm.D, (size_t)8 * dm.G);
+    return std::max(part + (size_t)16 * dm.D, (size_t)8 * dm.RG);
 }
 template <bool WIDE>            // more than 32 chunks in a layer
 __global__ void __launch_bounds__(EVAL_THREADS)
@@ -537,11 +544,10 @@ k_eval_few(const EvalArgs A)
     u64 *Q = (u64 *)(smraw + ((sizeof(int) * ((size_t)dm.LP + dm.N / MS + 2) + 7) & ~(size_t)7));      // [D] statistics of the row's cells on
     int *T = (int *)(Q + dm.D), *cnt = T + dm.D;                        // this shard, by slot
     __shared__ int n_s, last_s, wrong_s;
-    __shared__ u64 es_s, es_of[8];
-    __shared__ i64 s0_s, s1_s, s2_s;
+    __shared__ i64 of_warp[3][EVAL_THREADS / 32], es_of[8];                      // (a place a warp: 64-bit additions to one address queue up)
     const EvalCells cells = eval_cells(A, lay);
     char *b = A.blob_out ? A.blob_out + (size_t)lay * A.bl.bytes : nullptr;
-    if (tid == 0) { n_s = 0; es_s = 0; s0_s = 0; s1_s = 0; s2_s = 0; }
+    if (tid == 0) n_s = 0;
     const int row = rg / dm.G, g = rg % dm.G, first = row * dm.D;
     // (a slot of another shard has a negative count: which slots are the row-shard's is looked up in global memory only here)
     for (int d = tid; d < dm.D; d += EVAL_THREADS) { Q[d] = 0; T[d] = 0; cnt[d] = __ldg(A.edp + d) == g ? 0 : (int)0x80000000; }
@@ -599,8 +605,8 @@ k_eval_few(const EvalArgs A)
         const int m = eval_layer_max(on ? max(max(a.x, a.y), max(a.z, a.w)) : 0, lane, cpl);
         if (on && lane % cpl == 0) es += m;
     }
-    for (int o = 16; o; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
-    if (lane == 0 && es) atomicAdd(&es_s, (u64)es);
+    es = few_warp_sum(es);
+    if (lane == 0) of_warp[0][warp] = es;
     // Statistics of all of the cluster's samples meet in its first CTA: a lane there for every CTA of a slot, which fetches; more slots
     // than it has lanes for are added to it from afar (diagnostics of 6000 samples in four row-shards of 256 slots 56.5 us fetched, 55 so).
     if (dm.D * MS <= EVAL_THREADS) {
@@ -622,7 +628,12 @@ k_eval_few(const EvalArgs A)
             if (cnt[d] > 0) { atomicAdd(T0 + d, T[d]); atomicAdd(cnt0 + d, cnt[d]); few_add(Q0 + d, (u32)Q[d], (u32)(Q[d] >> 32), A.q_halves); }
     }
     __syncthreads();
-    if (tid == 0) cl.map_shared_rank(es_of, 0)[ms] = es_s;
+    if (tid == 0) {
+        i64 sum = 0;
+#pragma unroll
+        for (int w = 0; w < EVAL_THREADS / 32; ++w) sum += of_warp[0][w];
+        cl.map_shared_rank(es_of, 0)[ms] = sum;
+    }
     cl.sync();                                            // nobody reads another CTA's shared memory from here on
     if (ms) return;
     if (b)
@@ -634,7 +645,7 @@ k_eval_few(const EvalArgs A)
         }
     if (warp == 0) {
         i64 Af = 0, E = 0;
-        for (int x = 0; x < MS; ++x) E += (i64)es_of[x];
+        for (int x = 0; x < MS; ++x) E += es_of[x];
         bool wrong = false;
         for (int d = lane; d < dm.D; d += 32) wrong |= cnt[d] == 0 || (cnt[d] > 0 && T[d] > dm.C);
         wrong = __any_sync(0xffffffffu, wrong);
@@ -642,8 +653,7 @@ k_eval_few(const EvalArgs A)
             const i64 ca = dm.ahat[s] * dm.C, cb = dm.bhat[s];
             i64 v = 0;
             for (int d = lane; d < dm.D; d += 32) { const i64 w = cnt[d] < 0 ? 0 : ca * T[d] + cb * (i64)few_square(Q[d], A.q_halves); v = w > v ? w : v; }
-            for (int o = 16; o; o >>= 1) { const i64 w = __shfl_xor_sync(0xffffffffu, v, o); v = w > v ? w : v; }
-            Af += v;
+            Af += few_warp_max(v);
         }
         if (lane == 0) {
             const i64 J = Af + dm.EC * E;
@@ -662,45 +672,47 @@ k_eval_few(const EvalArgs A)
     __syncthreads();
     if (!last_s) return;
     __threadfence();
-    i64 *U = (i64 *)smraw;
-    for (int x = tid; x < dm.G; x += EVAL_THREADS) U[x] = 0;
-    __syncthreads();
+    // costs of the row-shards on chip, one trip; a thread adds up a shard's rows
+    i64 *Js = (i64 *)smraw;                                              // [RG]
+    i64 top = 0, sum = 0, most = 0;
     {
-        i64 *eg = A.cost + (size_t)lay * dm.RG, top = 0;
+        i64 *eg = A.cost + (size_t)lay * dm.RG;
 #pragma unroll 4
         for (int x = tid; x < dm.RG; x += EVAL_THREADS) {
             const i64 J = __ldcg(eg + x);
             eg[x] = 0;
+            Js[x] = J;
             top = J > top ? J : top;
-            atomicAdd((u64 *)&U[x % dm.G], (u64)J);
         }
-        top = few_warp_max(top);
-        if (lane == 0) atomicMax(&s2_s, top);
     }
     __syncthreads();
-    {
-        i64 sum = 0, top = 0;
-        for (int x = tid; x < dm.G; x += EVAL_THREADS) {
-            const i64 u = U[x];
-            sum += u; top = u > top ? u : top;
-            if (b) ((i64 *)(b + A.bl.off_U))[x] = u;
-        }
-        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        top = few_warp_max(top);
-        if (lane == 0) { atomicMax(&s0_s, top); atomicAdd((u64 *)&s1_s, (u64)sum); }
+    for (int x = tid; x < dm.G; x += EVAL_THREADS) {
+        i64 u = 0;
+#pragma unroll 4
+        for (int r = 0; r < dm.R; ++r) u += Js[r * dm.G + x];
+        sum += u; most = u > most ? u : most;
+        if (b) ((i64 *)(b + A.bl.off_U))[x] = u;
     }
+    top = few_warp_max(top); most = few_warp_max(most); sum = few_warp_sum(sum);
+    if (lane == 0) { of_warp[0][warp] = most; of_warp[1][warp] = sum; of_warp[2][warp] = top; }
     __syncthreads();
+    i64 sc[3] = { 0, 0, 0 };
+#pragma unroll
+    for (int w = 0; w < EVAL_THREADS / 32; ++w) {
+        const i64 m = of_warp[0][w], n = of_warp[2][w];
+        sc[0] = m > sc[0] ? m : sc[0]; sc[1] += of_warp[1][w]; sc[2] = n > sc[2] ? n : sc[2];
+    }
     if (A.host) {          // coverage is checked by the caller's `bad` flag: every sample sits in one cell by construction
         if (tid < 8) A.host[tid] = A.counters[tid];
         if (tid < 3) { A.host[16 + tid] = A.inc_score[tid]; A.host[22 + tid] = A.seed_score[tid]; }
         if (tid < RP_SW_COUNT) ((int *)(A.host + 56))[tid] = A.status[tid] | (tid == RP_SW_VALIDATE && wrong_s ? 1 : 0);
     }
     if (tid < 3) {
-        const i64 sc = tid == 0 ? s0_s : (tid == 1 ? s1_s : s2_s);
-        if (A.score_out) A.score_out[(size_t)lay * 3 + tid] = sc;
-        if (A.score_out2) A.score_out2[(size_t)lay * 3 + tid] = sc;
-        if (A.f64_out) A.f64_out[(size_t)lay * 3 + tid] = (double)sc / (double)dm.SC;
-        if (b) { i64 *S = (i64 *)(b + A.bl.off_S); S[tid] = sc; if (tid == 0) S[3] = rp_energy(s0_s, s1_s, s2_s); }
+        const i64 v = tid == 0 ? sc[0] : (tid == 1 ? sc[1] : sc[2]);
+        if (A.score_out) A.score_out[(size_t)lay * 3 + tid] = v;
+        if (A.score_out2) A.score_out2[(size_t)lay * 3 + tid] = v;
+        if (A.f64_out) A.f64_out[(size_t)lay * 3 + tid] = (double)v / (double)dm.SC;
+        if (b) { i64 *S = (i64 *)(b + A.bl.off_S); S[tid] = v; if (tid == 0) S[3] = rp_energy(sc[0], sc[1], sc[2]); }
     }
     if (!A.score_final && !A.f64_final) return;
     if (tid < 32) __threadfence();

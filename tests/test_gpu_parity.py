@@ -1996,3 +1996,22 @@ def test_between_two_levels_by_members_a_thread(pop):
     _, stats = check_anneal(w, ctx, ref, None, pop, 4, 24, t_ratio=0.4, check_members=2, t0=3e-3)
     assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row" and stats.kernel_launches == 2 * 4 + 2
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("N", [2047, 2048, 2049])
+def test_distances_of_as_many_samples_as_registers_hold(N):
+    """Eight samples a thread, and one more."""
+    w = make_window(custom_spec("held", N, 2, 8, 2, 1 << 16, 4, 4, 9, 0, data_seed=N))
+    s = w.spec
+    ref = oracle_front(w, None, 3)
+    ctx = load(w, pop=9, min_rows=3)
+    check_front(w, ctx, ref)
+    lays, ok = oracle.seed_trials(w.lengths, ref["seed"], ref["R"], s.token_cap, 4, 9, 5, s.anneal_seed)
+    assert rp.rp_seed_population(ctx, 5) == int(ok.sum())
+    sc = oracle.eval_layouts(w.lengths, ref["q"], lays, ref["R"], s.token_cap, 4, None, s.alpha, s.beta)["score"]
+    want = oracle.select_population(w.lengths, ref["q"], lays, sc, ref["R"], s.token_cap, 4, s.top_k, 4, 1 << 16, s.anneal_seed, None,
+                                    want_dist=True)
+    nd, order = rp.rp_select_population(ctx, 4, 1 << 16)
+    assert nd == want["n_distinct"] and (order == want["order"]).all()
+    assert (rp.rp_debug_dump(ctx, "SELECT_DIST", (9, 9), np.int64) == want["dist"]).all()
+    rp.rp_destroy(ctx)
