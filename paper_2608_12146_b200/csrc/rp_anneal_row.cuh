@@ -25,9 +25,7 @@ __device__ __forceinline__ int4 add4(const int4 &a, const int4 &b) { return make
 
 // The chains of a level may be launched before the launch between two levels (rp_level_turn.cu) has ended: once each of its CTAs has called
 // rp_let_next_launch_start or has ended.  What it leaves behind, or reads still, they touch behind rp_wait_for_launch_before, which
-// waits for its end.  Launched without the attribute that allows it, both do nothing.
-__device__ __forceinline__ void rp_let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void rp_wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// waits for its end.
 
 // Bounded wait of one thread until a counter that the other CTAs of the launch add to has reached
 // `target`; false when the time allowed ran out or another chain has raised the time-out word.

@@ -420,6 +420,11 @@ __device__ __forceinline__ u64 rp_exp2neg(u64 z)
     return ip >= 32 ? 0 : q >> ip;
 }
 
+// Programmatic dependent launches: the next launch may start once every CTA of this one has called the first or has ended; the second
+// waits for the end of the launch before.  Where the next launch does not ask for it, both do nothing.
+__device__ __forceinline__ void rp_let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void rp_wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ bool rp_lex_less(i64 a0, i64 a1, i64 a2, i64 b0, i64 b1, i64 b2)
 {
     if (a0 != b0) return a0 < b0;

@@ -535,6 +535,7 @@ __global__ void __launch_bounds__(EVAL_THREADS)
 k_eval_few(const EvalArgs A)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
+    rp_let_next_launch_start();                                          // (the diagnostics' coefficients need nothing of this)
     const RpDims &dm = A.dm;
     const cg::cluster_group cl = cg::this_cluster();
     const int MS = gridDim.x, ms = blockIdx.x, rg = blockIdx.y, lay = blockIdx.z;
@@ -1020,6 +1021,7 @@ k_diagnose(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, cons
 {
     extern __shared__ double cvs[];          // [2][L], then one row of rank loads per warp
     if (blockIdx.x == DIAG_PEAK_CTAS) { diag_cv(Lagg, rank_load, dm, cvs, out); return; }
+    rp_wait_for_launch_before();
     const int lane = threadIdx.x & 31;
     const int wid = (int)(threadIdx.x >> 5) * DIAG_PEAK_CTAS + (int)blockIdx.x, nw = DIAG_PEAK_CTAS * DIAG_THREADS / 32;
     i64 s_ep = 0, n_ep = 0, t_ep = 0;
@@ -1107,8 +1109,16 @@ extern "C" int rp_diagnostics(rp_ctx *c, const int32_t *layout, rp_diag *out)
             e = cudaFuncSetAttribute(k_diagnose, cudaFuncAttributeMaxDynamicSharedMemorySize, EVAL_SMEM_MAX);
             if (e != cudaSuccess) break;
         }
-        k_diagnose<<<DIAG_PEAK_CTAS + 1, DIAG_THREADS, cv_smem, c->stream>>>(c->d_Lagg, c->d_rank_load, (const int *)(buf + off_W),
-                                                                            buf + off_blob, c->bl, dm, c->d_one_Esum + dm.RG, c->d_one_ticket, host);
+        // (started beside the scoring: what the peaks read of it they wait for, the coefficients are of the placement alone)
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(DIAG_PEAK_CTAS + 1); cfg.blockDim = dim3(DIAG_THREADS); cfg.dynamicSmemBytes = cv_smem; cfg.stream = c->stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at; cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, k_diagnose, (const i64 *)c->d_Lagg, (const i64 *)c->d_rank_load, (const int *)(buf + off_W), (const char *)(buf + off_blob),
+                               c->bl, dm, c->d_one_Esum + dm.RG, c->d_one_ticket, host);
+        if (e != cudaSuccess) break;
         ++g_rp_launches;
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
