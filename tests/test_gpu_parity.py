@@ -1184,8 +1184,8 @@ def test_smallest_window_and_empty_moves():
     rp.rp_destroy(ctx)
 
 
-# Both orders (sort in the packing CTA up to 512 samples and above 32768, counting on the whole GPU between), cells held one
-# and four a lane, keys in shared and global memory, one-token samples that fill a cell by the run.
+# Both orders (sort in the packing CTA up to 512 samples and above 32768, counting on the whole GPU between), up to 1024 cells and
+# more, keys in shared and global memory, one-token samples that fill a cell by the run.
 @pytest.mark.parametrize("N,D,min_rows,cap,longest", [
     (33, 1, 0, 40, 40), (512, 4, 0, 64, 64), (513, 4, 0, 64, 20), (700, 7, 0, 4096, 1), (2100, 4, 256, 64, 40),
     (2100, 5, 205, 64, 40), (2049, 2, 1024, 100, 100), (8193, 8, 120, 64, 4),
