@@ -13,6 +13,8 @@
 // of 32 bits, which pass by a minimum and a maximum: a warp alone pays two to three cycles an instruction); beyond, the keys lie in shared memory
 // (two searches of two ballots: 1100 cycles).  Ranking by r + 1 passes over all cells took 4400.  What does not depend on the
 // fit runs 32 samples at a time: a lane draws the random words of its sample, then the shuffle emits the 32 samples.
+#include <algorithm>
+
 #include "rp_common.cuh"
 
 #define SEED_WARPS 4
@@ -52,6 +54,9 @@ __device__ __forceinline__ void seed_emit(const int *__restrict__ order, const R
 }
 
 // Widths of the fields of a key: remaining capacity on top, samples, index + 1.
+// The capacity's field holds what an open cell can have left, one less than the cap at most.  A length can be the cap itself: where that is a power
+// of two as large as the field, the length shifted there is 2^32 (2^64), which is zero.  A cell that such a sample opens has nothing left, as the
+// subtraction says anyway; behind the opening samples it fits nowhere, which every comparison with a shifted length has to say.
 struct SeedKey { int rem, index; };              // (shifts of the capacity and of the samples)
 
 // A key that passes `from` places on its way down: keys that are not below it move up by one as far as place `from`.
@@ -105,11 +110,13 @@ __device__ __forceinline__ int seed_trial(const int *__restrict__ t, const int *
                 key = (Key)((u64)(u32)dm.C << sk.rem) - ts;
                 key |= one | (Key)(u32)(from + 1);
             } else {
+                // keys below ts, which has nothing in the lower word of 64 bits; of a length that is zero up there, all (unused places too)
+                const u32 under = (u32)(sizeof(Key) == 4 ? (u64)ts : (u64)ts >> 32) - 1u;
                 int n = 0;
 #pragma unroll
-                for (int e = 0; e < E; ++e) n += sizeof(Key) == 4 ? (u32)v[e] < (u32)ts : (u32)((u64)v[e] >> 32) < (u32)((u64)ts >> 32);   // (the lower word of ts is zero)
+                for (int e = 0; e < E; ++e) n += (u32)(sizeof(Key) == 4 ? (u64)v[e] : (u64)v[e] >> 32) <= under;
                 const int p0 = __reduce_add_sync(0xffffffffu, n), nc = dm.K - p0;        // feasible cells
-                if (nc == 0) return over ? -1 : 0;
+                if (nc <= 0) return over ? -1 : 0;
                 from = p0 + rp_pick(x, nc < width ? nc : width);
                 Key m[E];                            // key number from % E of every lane by halving
 #pragma unroll
@@ -178,7 +185,7 @@ k_seed_trials(const int *__restrict__ t, const int *__restrict__ order, const in
                     from = h0 + u;
                     key = (((u64)(u32)dm.C << 40) - ts) | (1ull << 20) | (u64)(u32)(from + 1);
                 } else {
-                    const int p0 = seed_below(keys, lb, top, ts, lane), nc = dm.K - p0;
+                    const int p0 = ts ? seed_below(keys, lb, top, ts, lane) : dm.K, nc = dm.K - p0;        // (ts = 0: see SeedKey)
                     if (nc == 0) { good = false; break; }
                     from = p0 + rp_pick(x, nc < width ? nc : width);
                     key = keys[seed_at(from, lb)] - ts + (1ull << 20);
@@ -219,7 +226,7 @@ int rp_launch_seed_trials(rp_ctx *c, int width, int *layouts, int *ok)
     auto bits = [](u32 x) { int n = 0; while (x >> n) ++n; return n; };
     SeedKey sk;
     sk.index = bits((u32)dm.K);
-    const int cb = 32 - bits((u32)dm.C - 1) - sk.index;
+    const int cb = 32 - std::max(1, bits((u32)dm.C - 1)) - sk.index;
     sk.rem = sk.index + cb;
     const bool narrow = lb <= 4 && cb > 0 && 4ll * dm.N / dm.K < (1ll << cb);
 #define SEED_FN(E_) (narrow ? k_seed_trials<E_, true> : k_seed_trials<E_, false>)

@@ -2015,3 +2015,42 @@ def test_distances_of_as_many_samples_as_registers_hold(N):
     assert nd == want["n_distinct"] and (order == want["order"]).all()
     assert (rp.rp_debug_dump(ctx, "SELECT_DIST", (9, 9), np.int64) == want["dist"]).all()
     rp.rp_destroy(ctx)
+
+
+# Samples exactly as long as the cap: one, two, eight, and all cells but one; caps of a power of two, one less and one more; cells on both
+# sides of 64, 128, 256 and 512 (two to sixteen keys a lane, and keys in shared memory); the largest cap, where a length fills 64 bits too.
+@pytest.mark.parametrize("C,D,R,n_cap,n_short,width", [
+    (4096, 2, 4, 1, 56, 4), (4096, 8, 3, 8, 60, 32), (4096, 8, 8, 63, 70, 4), (4097, 8, 8, 63, 70, 4), (4095, 8, 8, 63, 70, 4),
+    (8192, 8, 1, 2, 62, 1), (8192, 8, 1, 2, 62, 4), (8192, 8, 1, 2, 62, 8), (8191, 8, 1, 2, 62, 8), (8193, 8, 1, 2, 62, 8), (8192, 8, 1, 7, 250, 32),
+    (131072, 8, 9, 70, 90, 8), (131072, 8, 16, 126, 60, 32), (131072, 8, 17, 133, 60, 8), (131072, 8, 32, 254, 60, 32), (131072, 8, 33, 262, 60, 8),
+    (65536, 8, 64, 510, 80, 32), (65536, 8, 65, 518, 80, 32), (1, 4, 3, 12, 0, 4), (2, 4, 3, 8, 8, 4), (1 << 24, 8, 1, 7, 20, 4), (1 << 24, 8, 1, 7, 200, 8)])
+def test_trials_with_samples_as_long_as_the_cap(C, D, R, n_cap, n_short, width):
+    N, K, pop = n_cap + n_short, D * R, 60
+    rng = np.random.default_rng(C + N + width)
+    t = np.full(N, C)
+    free = K - n_cap                                             # cells that no sample of the cap's length takes
+    t[:n_short] = rng.integers(1, max(1, min(C - 1, 2 * free * C // (3 * max(1, n_short)))) + 1, n_short)
+    t = t[rng.permutation(N)].astype(np.int32)
+    s = custom_spec("capped", N, 1, 4, 1, C, D, 4, pop, 0)
+    a = np.zeros((N, 1, 4), np.int32)
+    a[np.arange(N), 0, rng.integers(0, 4, N)] = t
+    w = Window(s, t, a)
+    ref = oracle_front(w, None, R)
+    assert ref["R"] == R
+    lays, ok = oracle.seed_trials(w.lengths, ref["seed"], R, C, D, pop, width, s.anneal_seed)
+    ctx = load(w, pop=pop, min_rows=R)
+    check_front(w, ctx, ref)
+    own = rp.rp_seed_population(ctx, width)
+    got = rp.rp_debug_dump(ctx, "POPULATION", (pop, N), np.int32)
+    assert max(np.bincount(x, weights=t).max() for x in got) <= C
+    assert own == int(ok.sum()) and (got == lays).all()
+    rp.rp_destroy(ctx)
+    if C > 1 << 20:                                              # (selection refuses so large a cap)
+        return
+    ctx = load(w, pop=8, min_rows=R)
+    check_front(w, ctx, ref)
+    nd_want, picked_want, lays_want = oracle_init_population(w, ref, None, pop, 8, width, 4, 1 << 16)
+    nd, picked = rp.rp_init_population(ctx, pop, width, 4, 1 << 16)
+    assert nd == nd_want and (picked == picked_want).all()
+    assert (rp.rp_debug_dump(ctx, "POPULATION", (8, N), np.int32) == lays_want).all()
+    rp.rp_destroy(ctx)
