@@ -2054,3 +2054,49 @@ def test_trials_with_samples_as_long_as_the_cap(C, D, R, n_cap, n_short, width):
     assert nd == nd_want and (picked == picked_want).all()
     assert (rp.rp_debug_dump(ctx, "POPULATION", (8, N), np.int32) == lays_want).all()
     rp.rp_destroy(ctx)
+
+
+def pack_only(t, cap, D, min_rows=0):
+    """(rows, certified) and the seed of a window of these lengths (None where it does not fit), and the packing's device time in ms."""
+    N = len(t)
+    a = np.zeros((N, 1, 2), np.int32)
+    a[np.arange(N), 0, np.arange(N) % 2] = t
+    rp.rp_debug_set_stage_timing(True)
+    ctx = rp.rp_window_load(t, a, top_k=1, token_cap=cap, dp_width=D, ep_width=2, pop_size=2, min_rows=min_rows)
+    rp.rp_debug_set_stage_timing(False)
+    rp.rp_place_experts(ctx)
+    try:
+        rows, seed = rp.rp_pack_rows(ctx), rp.rp_debug_dump(ctx, "SEED_LAYOUT", (N,), np.int32)
+    except rp.RpError as e:
+        assert e.status == -4
+        rows, seed = None, None
+    ms = rp.rp_debug_stage_times(ctx)["pack_rows"]
+    rp.rp_destroy(ctx)
+    return rows, seed, ms
+
+
+# Samples of more than half the cap (no row count but the last will do, or none), of half and one more, a third and one more and less, of both
+# sides of both; a few long ones among short ones; attempts that fail in the first and in a later warp, and samples in two parts (more than
+# 16384 behind the cells).
+@pytest.mark.parametrize("N,D,cap,lo,hi,short", [
+    (600, 4, 1000, 501, 900, 0), (601, 4, 1000, 501, 900, 0), (600, 4, 1000, 500, 500, 0), (600, 4, 1000, 400, 600, 0), (602, 7, 999, 334, 499, 0),
+    (600, 4, 999, 333, 333, 0), (602, 7, 999, 332, 400, 0), (900, 8, 1000, 200, 600, 0), (40, 3, 100, 40, 70, 0), (300, 4, 1000, 501, 900, 300),
+    (500, 2, 1 << 16, 22000, 40000, 700), (5000, 8, 1000, 250, 334, 100), (2500, 8, 400, 101, 200, 100), (900, 4, 100000, 30000, 60000, 17500)])
+def test_packing_of_long_samples(N, D, cap, lo, hi, short):
+    rng = np.random.default_rng(N + cap)
+    t = np.concatenate([rng.integers(lo, hi + 1, N), rng.integers(1, max(2, lo // 20), short)])[rng.permutation(N + short)].astype(np.int32)
+    R, cert, seed = oracle.pack_ffd(t, cap, D, 0)
+    rows, got, _ms = pack_only(t, cap, D)
+    if R == 0:
+        assert rows is None
+    else:
+        assert rows == (R, cert) and (got == seed).all()
+
+
+@pytest.mark.parametrize("cap,lo,hi", [(32768, 17000, 30000), (32768, 12000, 30000)])
+def test_packing_does_not_try_every_row_count(cap, lo, hi):
+    """Row counts that the long samples rule out take no pass over the samples each: less time than ten windows of as many short samples."""
+    rng = np.random.default_rng(5)
+    hard, easy = rng.integers(lo, hi + 1, 2000).astype(np.int32), rng.integers(lo // 8, hi // 8, 2000).astype(np.int32)
+    times = [sorted(pack_only(t, cap, 8)[2] for _ in range(5))[2] for t in (hard, easy)]
+    assert times[0] < 10 * times[1]

@@ -1077,3 +1077,33 @@ def test_canonical_map_and_quality_diversity_selection():
     # a large eta turns the order into the score order (by primary score)
     prim = [int(sc[j][0]) for j in order[:nd]]
     assert prim == sorted(prim)
+
+
+def rows_too_few(t, cap, D, R):
+    """The rule by which packing passes over row counts: among the samples longer than a third of the cap, the K longest open the cells, a cell
+    takes one more, and the i-th behind them needs i + 1 openers it fits beside."""
+    u = np.sort(t)[::-1].astype(np.int64)
+    K = R * D
+    n = int((3 * u > cap).sum())
+    i = np.arange(max(0, min(n - K, K)))
+    return bool((u[K + i] + u[K - 1 - i] > cap).any()) or n > 2 * K
+
+
+@pytest.mark.parametrize("seed", range(40))
+def test_rows_ruled_out_by_long_samples(seed):
+    """No row count is passed over that first fit would take; none is left that the long samples alone rule out; more rows are never worse."""
+    rng = np.random.default_rng(seed)
+    cap, D = int(rng.integers(3, 400)), int(rng.integers(1, 6))
+    N = int(rng.integers(D, 120))
+    lo = int(rng.integers(1, cap + 1))
+    t = rng.integers(lo, int(rng.integers(lo, cap + 1)) + 1, N).astype(np.int32)
+    if seed % 3 == 0:
+        t[rng.random(N) < 0.5] = rng.integers(1, max(2, cap // 6))
+    few = [rows_too_few(t, cap, D, R) for R in range(1, N // D + 1)]
+    assert all(a >= b for a, b in zip(few, few[1:]))
+    long_ = t[3 * t.astype(np.int64) > cap]
+    for R in range(1, N // D + 1):
+        takes = oracle.pack_ffd(t, cap, D, R)[0] == R
+        assert not (few[R - 1] and takes)
+        if len(long_) >= R * D and len(long_) >= D and not few[R - 1] and -(-int(long_.sum()) // (cap * D)) <= R:
+            assert oracle.pack_ffd(long_, cap, D, R)[0] == R
