@@ -421,7 +421,9 @@ __device__ __forceinline__ u64 rp_exp2neg(u64 z)
 }
 
 // Programmatic dependent launches: the next launch may start once every CTA of this one has called the first or has ended; the second
-// waits for the end of the launch before.  Where the next launch does not ask for it, both do nothing.
+// waits for the end of the launch before.  Where the next launch does not ask for it, both do nothing.  What the launch before writes is not
+// read-only while the next one lives: there it is read by plain loads or __ldcg, never by __ldg or through a const __restrict__ pointer, which
+// promise that (and which the compiler may move in front of the wait).
 __device__ __forceinline__ void rp_let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void rp_wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

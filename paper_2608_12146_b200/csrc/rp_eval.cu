@@ -1014,9 +1014,9 @@ __device__ __forceinline__ void diag_cv(const i64 *__restrict__ Lagg, const i64 
 }
 
 // Peaks: one warp per (row, layer): lanes over ranks, loop over shards; integer results by atomics on `sums` (s_ep, n_ep, t_ep; zero
-// between launches, as the ticket is).
+// between launches, as the ticket is).  W and blob are written by the scoring, beside which this launch starts: neither __ldg nor __restrict__.
 __global__ void __launch_bounds__(DIAG_THREADS)
-k_diagnose(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, const int *__restrict__ W, const char *__restrict__ blob,
+k_diagnose(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, const int *W, const char *blob,
            RpBlob bl, RpDims dm, i64 *__restrict__ sums, int *__restrict__ ticket, RpDiagDev *__restrict__ out)
 {
     extern __shared__ double cvs[];          // [2][L], then one row of rank loads per warp
@@ -1036,7 +1036,7 @@ k_diagnose(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, cons
             for (int p = lane; p < dm.P; p += 32)
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int v = g0 + u < dm.G ? __ldg(w0 + (size_t)(g0 + u) * dm.LP + p) : 0;
+                    const int v = g0 + u < dm.G ? __ldcg(w0 + (size_t)(g0 + u) * dm.LP + p) : 0;
                     sum[u] += v; mx[u] = max(mx[u], v);
                 }
 #pragma unroll

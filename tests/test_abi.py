@@ -44,3 +44,19 @@ def test_null_arguments_are_rejected_without_a_device():
     assert lib.rp_best(None, None, None, None) == -1
     assert lib.rp_eval_population(None, None, 0, None, None) == -1
     lib.rp_destroy(None)
+
+
+def test_what_the_launch_before_may_still_write_is_not_read_as_read_only():
+    """Kernels that start beside the launch before them: nothing it writes is read by __ldg, or through a pointer that promises no writer."""
+    csrc = os.path.join(ROOT, "paper_2608_12146_b200", "csrc")
+    chain = open(os.path.join(csrc, "rp_anneal_row_chain.cuh")).read()
+    turn = open(os.path.join(csrc, "rp_level_turn.cu")).read()
+    assert all(x in turn for x in ("A.lo.anc_out[m] =", "T.list[at", "&T.ref["))                # what it writes, as the chains know it:
+    for name in ("wfree", "wref", "wfree_head", "anc"):
+        assert re.search(r"A\.%s\b" % name, chain) and not re.search(r"__ldg\(\s*&?A\.%s\b" % name, chain), name
+    text = open(os.path.join(csrc, "rp_eval.cu")).read()
+    start = text.index("\nk_diagnose(")
+    body = text[start:text.index("\n}\n", start)]
+    head, behind = body.split("rp_wait_for_launch_before();")
+    assert not re.search(r"__restrict__ (W|blob)\b", head)
+    assert "__ldg(" not in behind
