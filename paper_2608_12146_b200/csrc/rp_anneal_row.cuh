@@ -51,8 +51,8 @@ static inline int rp_row_layers(const RpDims &dm) { return dm.L <= 32 ? 1 : (dm.
 static inline bool rp_row_split(int cpl) { return cpl == 2 || cpl == 4; }
 // Whether they may start right away, up to four to an SM: their first step records and tables are then ready when the launch before ends
 // (300 members of 17 layers 1469 us at its end, 1401 right away; 512 of 24 2730 and 2715).  With more, the SM is full and what its
-// rows have left of the L1 cache counts (1024 members 2377 and 2390).
-static inline bool rp_row_starts_early(const rp_ctx *c) { return c->Ppop <= 4 * rp_sms(c); }
+// rows have left of the L1 cache counts (1024 members 2377 and 2390).  Only where there is a launch between two levels to start beside.
+static inline bool rp_row_starts_early(const rp_ctx *c) { return rp_row_turns(c) && c->Ppop <= 4 * rp_sms(c); }
 int rp_launch_row_chip(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int grid, int *done);
 int rp_launch_row_level(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);
 int rp_launch_row_pair(rp_ctx *c, const AnnealArgs &A, const RowArgs &X);

@@ -1140,8 +1140,9 @@ static int launch_row_t(rp_ctx *c, const AnnealArgs &A, const RowArgs &X, int gr
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(CHIP ? ROW_THREADS : 32);
     cfg.dynamicSmemBytes = X.smem_bytes; cfg.stream = c->stream;
     // Chains that start beside the launch before them (see rp_row_starts_early) go where there is room first: as much shared memory a CTA that
-    // an SM takes its share of them and no more.
-    if (!CHIP && rp_row_starts_early(c)) {
+    // an SM takes its share of them and no more.  Nowhere else: other windows' chains have the room then (one launch per level each, 300 members
+    // of 17 layers, two windows at once 896 -> 861 us a plan, four 513 -> 491; 512 of 24, four 548 -> 520).
+    if (!CHIP && A.level > 0 && rp_row_starts_early(c)) {
         const size_t share = (grid + rp_sms(c) - 1) / rp_sms(c);
         cfg.dynamicSmemBytes = std::max(cfg.dynamicSmemBytes, (size_t)228 * 1024 / (share + 1) - 1024 + 256);
     }

@@ -226,9 +226,17 @@ k_level_turn(const AnnealArgs A, const TurnArgs T)
     }
 }
 
+// Workers: as many as have something to do (a meeting costs the more the more there are); every one resident.
+static int turn_workers(const rp_ctx *c)
+{
+    const int P = c->Ppop, ns = 2 * P * c->dm.RG;
+    return std::max(4, std::min(rp_sms(c) - 1, std::max((P + 15) / 16, (ns + 4095) / 4096)));
+}
+
 // One launch per level asked for means that a caller plans several windows at once on separate streams: a launch whose CTAs wait
-// for one another would make them wait for its SMs, so the parts then stay launches of their own, as beyond the table on chip.
-bool rp_row_turns(const rp_ctx *c) { return c->knob_level_launches != 1 && c->Ppop <= TURN_MAX_MEMBERS; }
+// for one another would make them wait for its SMs, so the parts then stay launches of their own, as beyond the table on chip and where a
+// part of a GPU does not hold the workers and the CTA for the incumbent.
+bool rp_row_turns(const rp_ctx *c) { return c->knob_level_launches != 1 && c->Ppop <= TURN_MAX_MEMBERS && turn_workers(c) < rp_sms(c); }
 
 int rp_launch_level_end(rp_ctx *c, const AnnealArgs &A);
 
@@ -242,8 +250,7 @@ int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A0)
     T.ref = c->d_wcount; T.before = c->d_wref; T.list = c->d_wfree; T.head = c->d_wfree_head;
     T.ns = ns; T.early = rp_row_starts_early(c);
     A.sync = c->d_sync;
-    // Workers: as many as have something to do (a meeting costs the more the more there are); every one resident.
-    const int workers = std::max(4, std::min(rp_sms(c) - 1, std::max((P + 15) / 16, (ns + 4095) / 4096)));
+    const int workers = turn_workers(c);
     T.base = A.level * (P <= TURN_OWN * TURN_THREADS ? 1 : 2) * workers;                  // (the count is zero when the call starts)
     int lu = 0;
     while ((TURN_THREADS << lu) < P) ++lu;
@@ -259,7 +266,7 @@ int rp_launch_level_turn(rp_ctx *c, const AnnealArgs &A0)
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    const cudaError_t e = workers + 1 > rp_sms(c) ? cudaErrorCooperativeLaunchTooLarge : cudaLaunchKernelEx(&cfg, k_level_turn, A, T);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_level_turn, A, T);
     if (e == cudaErrorCooperativeLaunchTooLarge) {        // a part of a GPU: the launches one by one, at every level
         cudaGetLastError();
         return rp_launch_level_end(c, A0);

@@ -2100,3 +2100,21 @@ def test_packing_does_not_try_every_row_count(cap, lo, hi):
     hard, easy = rng.integers(lo, hi + 1, 2000).astype(np.int32), rng.integers(lo // 8, hi // 8, 2000).astype(np.int32)
     times = [sorted(pack_only(t, cap, 8)[2] for _ in range(5))[2] for t in (hard, easy)]
     assert times[0] < 10 * times[1]
+
+
+@pytest.mark.parametrize("extra", [0, 1])
+@pytest.mark.parametrize("L,per_level", [(17, 0), (24, 0), (17, 1)])
+def test_chains_that_start_beside_the_launch_between_two_levels(L, per_level, extra):
+    """Four chains to an SM start beside the launch between two levels, one chain more and they start at its end; with one launch per level that
+    launch is not there.  (The number of launches says which of the two ran.)"""
+    import torch
+    pop = 4 * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    w = make_window(custom_spec("beside", 400, L, 32, 2, 4096, 4, 16, pop, 0, data_seed=L))
+    ref = oracle_front(w, None, 90)
+    ctx = load(w, pop=pop, min_rows=90)
+    rp.rp_debug_set_knob(ctx, "LAUNCH_PER_LEVEL", per_level)
+    check_front(w, ctx, ref)
+    _, stats = check_anneal(w, ctx, ref, None, pop, 5, 40, t_ratio=0.4, check_members=2, t0=3e-3)
+    assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row"
+    assert stats.kernel_launches == 2 * 5 + 2 if per_level == 0 else stats.kernel_launches > 2 * 5 + 2
+    rp.rp_destroy(ctx)
