@@ -381,15 +381,16 @@ k_anneal_row(const AnnealArgs A, const RowArgs X)
         // A slice that only this member holds when the level starts is rewritten in place; a shared
         // one is left at its first rewrite for this chain's spare slice of that row-shard (entry
         // j*RG + rg of the free list, which holds at least RG slices per member).  (List and holders, like the ancestors, may be written while
-        // this launch is there already: no __ldg.  The states are of the launch before that one.)
+        // this launch is there already: no __ldg, but plain loads, which stay behind the wait; __ldcg took 2 % of large.  The states are of the
+        // launch before that one.)
         const int n_free = A.wfree_head[1];
 #pragma unroll 4
         for (int rg = lg; rg < dm.RG; rg += GL) {
             ch.slack[rg] = __ldg(fs + rg);
             const int s = __ldg(ts + rg);
             const size_t at = (size_t)j * dm.RG + rg;
-            const int sp = at < (size_t)n_free ? __ldcg(A.wfree + at) : -2;
-            ch.ws[rg] = make_int2(s, __ldcg(A.wref + s) == 1 ? s : sp);
+            const int sp = at < (size_t)n_free ? A.wfree[at] : -2;
+            ch.ws[rg] = make_int2(s, A.wref[s] == 1 ? s : sp);
         }
         const unsigned short *cs = (const unsigned short *)(bsrc + A.bl.off_cell);        // 8-byte aligned
 #pragma unroll 8

@@ -1036,7 +1036,7 @@ k_diagnose(const i64 *__restrict__ Lagg, const i64 *__restrict__ rank_load, cons
             for (int p = lane; p < dm.P; p += 32)
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int v = g0 + u < dm.G ? __ldcg(w0 + (size_t)(g0 + u) * dm.LP + p) : 0;
+                    const int v = g0 + u < dm.G ? w0[(size_t)(g0 + u) * dm.LP + p] : 0;
                     sum[u] += v; mx[u] = max(mx[u], v);
                 }
 #pragma unroll
