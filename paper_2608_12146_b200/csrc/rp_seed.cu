@@ -98,10 +98,13 @@ __device__ __forceinline__ int seed_trial(const int *__restrict__ t, const int *
         u32 xf;
         seed_emit(order, dm, width, key0, key1, j, h0, nb, lane, win, em, xf);
         const int len = lane < nb ? t[em] : 0;
+        // the length as a capacity of a key (its upper word; there is nothing in the lower one of 64 bits), less one: zero less one is all ones
+        const u32 lim = (sizeof(Key) == 4 ? (u32)len << sk.rem : (u32)len << (sk.rem - 32)) - 1u;
         int place = 0;
         bool over = false;
         for (int u = 0; u < nb; ++u) {
-            const Key ts = (Key)(u32)__shfl_sync(0xffffffffu, len, u) << sk.rem;
+            const u32 under = __shfl_sync(0xffffffffu, lim, u);
+            const Key ts = sizeof(Key) == 4 ? (Key)(under + 1u) : (Key)((u64)(under + 1u) << 32);
             const u32 x = __shfl_sync(0xffffffffu, xf, u);
             Key key;
             int from;                                // place the new key comes from
@@ -110,9 +113,7 @@ __device__ __forceinline__ int seed_trial(const int *__restrict__ t, const int *
                 key = (Key)((u64)(u32)dm.C << sk.rem) - ts;
                 key |= one | (Key)(u32)(from + 1);
             } else {
-                // keys below ts, which has nothing in the lower word of 64 bits; of a length that is zero up there, all (unused places too)
-                const u32 under = (u32)(sizeof(Key) == 4 ? (u64)ts : (u64)ts >> 32) - 1u;
-                int n = 0;
+                int n = 0;                           // keys below ts: all of them, unused places too, where ts is zero
 #pragma unroll
                 for (int e = 0; e < E; ++e) n += (u32)(sizeof(Key) == 4 ? (u64)v[e] : (u64)v[e] >> 32) <= under;
                 const int p0 = __reduce_add_sync(0xffffffffu, n), nc = dm.K - p0;        // feasible cells
