@@ -219,11 +219,6 @@ static int reset_status(rp_ctx *c)
     return RP_OK;
 }
 
-static int build_population(rp_ctx *c, bool candidates = false, bool same_rows = false);
-
-// Rows, cells and row-shards of a window packed into R rows.
-static void set_rows(rp_ctx *c, int R) { RpDims &dm = c->dm; dm.R = R; dm.K = R * dm.D; dm.RG = R * dm.G; }
-
 static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *lengths, const int32_t *demand)
 {
     RpDims &dm = c->dm;
@@ -368,13 +363,6 @@ static int window_load_impl(rp_ctx *c, const rp_config *cfg, const int32_t *leng
     // decides.  (Scoring also takes layouts whose cells are too full, see eval_launch.)
     const double shard_tokens = (double)dm.C * maxshard;
     dm.sum32 = (double)L * dm.k * (shard_tokens < total ? shard_tokens : total) < 2147483648.0;
-    // The population of the seed as well: rp_pack_rows finds it built, unless something has been asked for since that decides how.  What
-    // fails here is left to fail there.
-    if (c->eager_pack && !c->pack_out[3] && c->pack_out[0] > 0 && (long long)c->pack_out[0] * dm.D <= 65535) {
-        set_rows(c, c->pack_out[0]);
-        c->eager_pop = build_population(c) == RP_OK;
-        if (!c->eager_pop) { free_population(c); cudaGetLastError(); }
-    }
     return RP_OK;
 }
 
@@ -428,7 +416,6 @@ extern "C" int rp_place_experts(rp_ctx *c, int32_t *pi, int64_t *rank_load)
         RP_TRY(rp_launch_project(c));
     }
     const bool waited = c->eager_place;       // rp_window_load has waited for the kernels
-    if (!waited) c->eager_pop = 0;            // (the seed was scored with the placement before)
     c->eager_place = 0;               // a repeated call recomputes
     // Outputs are complete when the call returns (nothing to wait for when none was asked for): the placement is in the
     // pinned block, or copied when it is wanted on the device or does not fit there.
@@ -483,6 +470,8 @@ __global__ void k_iota(int *out, int n, int first)
     if (x < n) out[x] = first + x;
 }
 
+static int build_population(rp_ctx *c, bool candidates = false, bool same_rows = false);
+
 // Rank-load cells in full form, at least `cells` of them (keep: with what the present ones hold).  A population that
 // is annealed on rows kept apart (padded or compressed) needs only as many as it is scored with: one for the seed
 // instead of two per member (wide: 14.5 GB).
@@ -510,16 +499,13 @@ extern "C" int rp_pack_rows(rp_ctx *c, int32_t *n_rows, int32_t *certified)
         RP_TRY(rp_launch_pack(c, 0));
         RP_CUDA(cudaStreamSynchronize(c->stream));
         memcpy(c->pack_out, c->h_pin + 10, sizeof(int) * 4);
-        c->eager_pop = 0;
     }
     c->eager_pack = 0;                // a repeated call recomputes
     if (po[3] || po[0] <= 0) return RP_ERR_INFEASIBLE;
     c->Rstar = po[0]; c->certified = po[1];
-    const bool built = c->eager_pop;
-    c->eager_pop = 0;
-    set_rows(c, po[0]);
+    dm.R = po[0]; dm.K = dm.R * dm.D; dm.RG = dm.R * dm.G;
     if (dm.K > 65535) return RP_ERR_RANGE;
-    if (!built) RP_TRY(build_population(c));
+    RP_TRY(build_population(c));
     if (n_rows) *n_rows = c->Rstar;
     if (certified) *certified = c->certified;
     c->stage = 3;
@@ -1233,7 +1219,6 @@ static int relayout_population(rp_ctx *c)
 extern "C" int rp_debug_set_knob(rp_ctx *c, int knob, int64_t value)
 {
     if (!c || value < 0) return RP_ERR_ARG;
-    c->eager_pop = 0;
     switch (knob) {
         case RP_KNOB_BARRIER_WORKSPACE:
             if (value > (1 << 20) || (value & 15) || (value && value < 64)) return RP_ERR_ARG;

@@ -195,7 +195,6 @@ struct rp_ctx {
     i64 *d_inc_score;          // [3]
     void *side;                // side stream + two events borrowed for the call that packs beside the placement (see RpSide)
     int eager_place, eager_pack;   // rp_window_load already queued the placement / packing kernels behind its checks
-    int eager_pop;                 // and has built the seed's population as rp_pack_rows would
     int pack_out[4];           // R*, certified, R_lb, failure flag as read back with the load's verdict
     int best_ready;            // the incumbent has been validated and rescored since it last changed
     int best_verdict;          // RP_OK or RP_ERR_INVALID_PLAN of that validation

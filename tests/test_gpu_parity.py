@@ -2118,3 +2118,20 @@ def test_chains_that_start_beside_the_launch_between_two_levels(L, per_level, ex
     assert rp.rp_debug_chain_kernel(ctx) == "k_anneal_row"
     assert stats.kernel_launches == 2 * 5 + 2 if per_level == 0 else stats.kernel_launches > 2 * 5 + 2
     rp.rp_destroy(ctx)
+
+
+@pytest.mark.parametrize("name", ["tiny", "medium"])
+def test_loading_and_placing_builds_no_population(name):
+    """A caller that only places pays for no population: it is rp_pack_rows that launches its set-up and the seed's scoring."""
+    w = make_window(name)
+    ref = oracle_front(w)
+    counts = [rp.rp_debug_launch_count()]
+    ctx = load(w)
+    pi, _ = rp.rp_place_experts(ctx)
+    counts.append(rp.rp_debug_launch_count())
+    assert (pi == ref["pi"]).all()
+    assert rp.rp_pack_rows(ctx) == (ref["R"], ref["cert"])
+    counts.append(rp.rp_debug_launch_count())
+    # checks, placement, projection, packing (with the order of 513 and more samples by a launch of its own); set-up, scoring
+    assert counts[1] - counts[0] <= 4 + (w.spec.n_samples > 512) and counts[2] - counts[1] >= 2
+    rp.rp_destroy(ctx)
