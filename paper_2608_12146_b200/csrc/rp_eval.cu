@@ -42,7 +42,7 @@ struct EvalArgs {
     i64 *score_final;
     double *f64_final;
     int n;
-    bool q_halves;                                // (few layouts) no cell's squared lengths add up to 2^48, whatever the layout
+    bool q_halves;                                // no cell's squared lengths add up to 2^48, whatever the layout
     i64 *cost;                                    // [n][RG] row-shard costs handed to the finishing CTA; zero between launches
     int *tickets;                                 // [n] arrival counters (many layouts: whether a cell is empty or overfull); zero between launches
     unsigned short *list;                         // [n][N] samples grouped by row-shard (k_eval_group)
@@ -735,7 +735,8 @@ k_eval_few(const EvalArgs A)
     }
 }
 
-// Windows are taken up to this measure of their size (no kernel here needs as much shared memory).
+// Windows are scored up to this measure of their size.  It is the shared memory of a scoring kernel that is gone, no kernel here needs as much,
+// and stays as what callers have been told: what was refused with RP_ERR_RANGE is refused.
 static size_t eval_smem_bytes(const RpDims &dm)
 {
     const size_t cells = (sizeof(u64) * dm.K + sizeof(i64) * (2 * (size_t)dm.RG + dm.G) + sizeof(int) * 2 * (size_t)dm.K + 2 * (size_t)dm.N + 15) & ~(size_t)15;

@@ -63,8 +63,8 @@ k_level_turn(const AnnealArgs A, const TurnArgs T)
     }
     const int m0 = (int)((long long)P * blockIdx.x / workers), m1 = (int)((long long)P * (blockIdx.x + 1) / workers);
 
-    // ---- 1: cumulative weights.  Up to a member a thread every worker weighs all members itself; more are shared out, and the workers
-    // meet.  A thread adds up 2^lu consecutive members, place j of the table is j + (j >> lu) (no bank conflicts) ------------
+    // ---- 1: cumulative weights.  Up to TURN_OWN members a thread every worker weighs all members itself; more are shared out, and the
+    // workers meet.  A thread adds up 2^lu consecutive members, place j of the table is j + (j >> lu) (no bank conflicts) ------------
     u64 *F = (u64 *)turn_smem;
     int lu = 0;
     const int late = __ldcg(&A.status[RP_SW_TIMEOUT]);

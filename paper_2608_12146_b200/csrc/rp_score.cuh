@@ -1,4 +1,4 @@
-// Device routines shared by the full-evaluation kernel and the annealing kernel: the
+// Device routines shared by the full-evaluation kernels and the annealing kernels: the
 // EDP-shard-aware objective of Sections 3.4-3.5 in integer units (score scale 2^8*C^2).
 #pragma once
 #include "rp_common.cuh"
@@ -69,18 +69,4 @@ __device__ __forceinline__ i64 rp_warp_layer_max_sum(const RpDims &dm, int lane,
     }
     for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     return sum;
-}
-
-// Cell statistics from the assignment (Eq. cell-token-statistics), with shared-memory atomics
-// (integer sums: order does not matter).  Arrays must be zeroed and the block synchronised.
-__device__ __forceinline__ void rp_accumulate_cells(const RpDims &dm, const RpSmemState &st,
-                                                    const int *__restrict__ t, int tid, int nt)
-{
-    for (int i = tid; i < dm.N; i += nt) {
-        int c = st.cell_of[i];
-        int ti = t[i];
-        atomicAdd(&st.T[c], ti);
-        atomicAdd(&st.Q[c], (u64)ti * (u64)ti);
-        atomicAdd(&st.cnt[c], 1);
-    }
 }
