@@ -268,22 +268,29 @@ k_eval_slice(const EvalArgs A, const SlicePlan S, int n)
             }
             const int4 *col = rows + min(k, w - 1);
             constexpr int STRIDE = SLICE_THREADS / TW;
-            const int dl = STRIDE / RG, dy = STRIDE % RG;
-            u32 f = warp * TPW + team, lay = lay0 + f / RG, y = f % RG;         // this team's row-shard of the batch: place y of layout lay
+            // This team's row-shard of the batch: place `hi` of layout `lo` of the batch (across), or place `lo` of layout `hi`.  Across, the
+            // teams of a warp have row-shards of one place, which are of nearly the same length in all layouts, and the longest come first:
+            // few long row-shards of a layout differ much (3300 samples in 32, 47 layers of 16 ranks, 500 layouts 1152 us one layout after the other, 310
+            // across; in 208, 383 and 379).  With one or two lanes a team a warp's ids then lie in 32 or 16 lists at a time, which only pays
+            // where there are several rounds (6900 in 24, 11 of 8, 64 layouts 140 and 160, 500 405 and 259), with one lane hardly ever (13000 in
+            // 240, 24 of 4, 500 layouts 692 and 990).
+            const bool across = TW > 2 || (TW == 2 && nrg >= (u32)STRIDE);
+            const u32 inner = across ? nrg / RG : RG, dh = STRIDE / inner, dl = STRIDE % inner;
+            u32 f = warp * TPW + team, hi = f / inner, lo = f - hi * inner;
             u32 o0 = 0, o1 = 0;
-            if (f < nrg) { const u32 *go = A.off + lay * (RG + 1u) + y; o0 = __ldg(go); o1 = __ldg(go + 1); }
+            if (f < nrg) { const u32 *go = A.off + (lay0 + (across ? lo : hi)) * (RG + 1u) + (across ? hi : lo); o0 = __ldg(go); o1 = __ldg(go + 1); }
             while (f - team < nrg) {
                 const bool on = f < nrg;
                 const int p = (int)(o0 & 0xffffu), len = (int)(o1 & 0xffffu) - p;
-                const u32 at = lay * (u32)RG + (o0 >> 16), here = f;
+                const u32 lay = lay0 + (across ? lo : hi), at = lay * (u32)RG + (o0 >> 16), here = f;
                 // Odd teams walk their list from its end: a list holds its even samples first, and rows of 64 bytes that a
                 // quarter warp reads together collide where both are even or both odd.
                 const unsigned short *list = A.list + lay * (u32)N + ((team & 1) ? p + len - 1 : p);
                 const int step = (team & 1) ? -1 : 1;
-                f += STRIDE; lay += dl; y += dy;                                // the next one's offsets under this one's sums
-                if (y >= (u32)RG) { y -= RG; ++lay; }
+                f += STRIDE; hi += dh; lo += dl;                                // the next one's offsets under this one's sums
+                if (lo >= inner) { lo -= inner; ++hi; }
                 o0 = o1 = 0;
-                if (f < nrg) { const u32 *go = A.off + lay * (RG + 1u) + y; o0 = __ldg(go); o1 = __ldg(go + 1); }
+                if (f < nrg) { const u32 *go = A.off + (lay0 + (across ? lo : hi)) * (RG + 1u) + (across ? hi : lo); o0 = __ldg(go); o1 = __ldg(go + 1); }
                 const int most = (int)__reduce_max_sync(0xffffffffu, len);
                 int4 a = make_int4(0, 0, 0, 0);
                 int id[PER];

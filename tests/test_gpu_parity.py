@@ -2135,3 +2135,32 @@ def test_loading_and_placing_builds_no_population(name):
     # checks, placement, projection, packing (with the order of 513 and more samples by a launch of its own); set-up, scoring
     assert counts[1] - counts[0] <= 4 + (w.spec.n_samples > 512) and counts[2] - counts[1] >= 2
     rp.rp_destroy(ctx)
+
+
+def test_scoring_of_few_long_row_shards_keeps_its_time():
+    """Few row-shards of very different lengths, as first fit leaves them, take no more than 1.6 times as long as as many of one length (they took
+    more than twice as long)."""
+    import torch
+    N, L, P, dp, R, n = 3300, 47, 16, 8, 4, 500
+    rng = np.random.default_rng(N)
+    t = np.clip(rng.lognormal(np.log(0.93 * 65536 * R * dp / N / 1.9), 1.2, N), 16, 16384).astype(np.int32)
+    a = torch.zeros((N, L, P), dtype=torch.int32, device="cuda")
+    a[torch.arange(N)[:, None], torch.arange(L)[None, :], torch.from_numpy(rng.integers(0, P, (N, L)))] = torch.from_numpy(t).cuda()[:, None]
+    ctx = rp.rp_window_load(torch.from_numpy(t).cuda(), a, top_k=1, token_cap=65536, dp_width=dp, ep_width=P, pop_size=2, min_rows=R)
+    rp.rp_place_experts(ctx)
+    assert rp.rp_pack_rows(ctx)[0] == R
+    fx, f64 = torch.empty((n, 3), dtype=torch.int64, device="cuda"), torch.empty((n, 3), dtype=torch.float64, device="cuda")
+    times = []
+    for seed in (rp.rp_best(ctx)[0], np.arange(N) % (R * dp)):
+        lays = torch.from_numpy(np.stack([rng.permutation(R * dp)[seed] for _ in range(n)]).astype(np.int32)).cuda()
+        ms = []
+        for _ in range(9):
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            ev[0].record()
+            rp.rp_eval_population(ctx, lays, fx, f64)
+            ev[1].record()
+            torch.cuda.synchronize()
+            ms.append(ev[0].elapsed_time(ev[1]))
+        times.append(sorted(ms)[4])
+    rp.rp_destroy(ctx)
+    assert times[0] < 1.6 * times[1]
