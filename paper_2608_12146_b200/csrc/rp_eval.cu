@@ -361,6 +361,16 @@ static SlicePlan eval_slice_plan(const RpDims &dm, int n)
         const double cost = std::ceil((double)S.slices * g / 148) * (1.5 + (double)((n + g - 1) / g));
         if (cost < best) { best = cost; S.groups = g; }
     }
+    // Narrow slices collide in shared memory (rows of 16 or 32 bytes) and pay a trip through the lists per layer, in ps a sample and layer 4.0 and
+    // 3.6; rows that stream fill a warp's strips whatever a layer has, 80, 104 and 140 ps a sample for one to three of them.  With enough layouts
+    // for both rates: 13000 samples in 240 row-shards, 47 layers of 4 ranks, 500 layouts 1182 us from slices and 697 streaming, 24 layers
+    // 692 and 531, 11 394 and 526; 6900 in 240, 47 of 8, 622 and 568, 24 357 and 427.  Few long row-shards stream badly (6900 in 24, 47 of 8,
+    // 1008 and, across, 713).
+    if (S.tw <= 2 && (long long)n * S.slices >= 6000) {
+        const int used = 32 / cpl * cpl, strips = ((dm.LP >> 2) + used - 1) / used, ns = std::min(3, strips);
+        const double row = S.slices * (S.tw == 1 ? 4.0 : 3.6), streamed = (strips + ns - 1) / ns * (ns == 1 ? 80.0 : ns == 2 ? 104.0 : 140.0);
+        if (row > streamed && (S.tw == 1 || dm.N <= 128ll * dm.RG)) return SlicePlan{};
+    }
     S.batch = S.parts > 1 ? std::max(1, SLICE_MAX / dm.RG) : n;
     S.smem = 16 * (size_t)S.w * (dm.N + 1) + (S.parts > 1 ? 4 * (size_t)SLICE_MAX : 0);
     return S;

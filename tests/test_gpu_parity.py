@@ -2137,6 +2137,30 @@ def test_loading_and_placing_builds_no_population(name):
     rp.rp_destroy(ctx)
 
 
+# Narrow slices: one chunk with more layers than are worth it (streamed), and fewer; two chunks of many layers, short row-shards (streamed), long
+# ones, and few layers with less and more row-shards to a batch than teams.
+@pytest.mark.parametrize("N,L,P,D,R,n", [(7100, 30, 4, 4, 3, 210), (7100, 12, 4, 4, 3, 510), (5000, 40, 8, 4, 12, 160), (5000, 40, 8, 2, 2, 160),
+                                         (5000, 3, 8, 8, 30, 40), (5000, 3, 8, 8, 30, 400)])
+def test_scoring_from_narrow_slices(N, L, P, D, R, n):
+    rng = np.random.default_rng(L)
+    s = custom_spec("narrow", N, L, P, 1, 1 << 20, D, P, 2, 0)
+    t = rng.integers(1, 400, N).astype(np.int32)
+    a = np.zeros((N, L, P), np.int32)
+    np.put_along_axis(a, rng.integers(0, P, (N, L, 1)), np.broadcast_to(t[:, None, None], (N, L, 1)), 2)
+    w = Window(s, t, a)
+    ref = oracle_front(w, None, R)
+    assert ref["R"] == R
+    ctx = load(w, min_rows=R)
+    check_front(w, ctx, ref)
+    K = R * D
+    lays = np.minimum(rng.integers(0, K, (n, N)), rng.integers(0, K, (n, N))).astype(np.int32)      # (row-shards of different lengths)
+    lays[-1] = K - 1
+    want = oracle.eval_layouts(w.lengths, ref["q"], lays, ref["R"], s.token_cap, D, None, s.alpha, s.beta)["score"]
+    fx, _f64 = rp.rp_eval_population(ctx, lays)
+    assert (fx == want).all()
+    rp.rp_destroy(ctx)
+
+
 def test_scoring_of_few_long_row_shards_keeps_its_time():
     """Few row-shards of very different lengths, as first fit leaves them, take no more than 1.6 times as long as as many of one length (they took
     more than twice as long)."""
