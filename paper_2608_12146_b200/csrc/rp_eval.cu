@@ -761,18 +761,20 @@ static size_t eval_smem_bytes(const RpDims &dm)
 }
 
 // Whether n layouts take the few-layouts form.  It has a cluster per row-shard and layout, which scans the whole assignment; the other
-// form groups an assignment once, but in one CTA, and has three launches where this has one.  Calls in us, few and many: 512 samples in
-// 32 row-shards, 16 layers of 8 ranks, n = 8 37.0 and 36.6, 16 38.8 and 36.9, 64 49 and 37, 512 204 and 54; 2048 in 240, 24 of 16, n = 4 36.9
-// and 41.5, 6 44.7 and 42.5, 64 172 and 54; 1000 in 128, 8 of 8, n = 8 37.8 and 37.4, 12 42.1 and 38.5; 4000 in 6, 16 of 8, n = 64 96 and
-// 138, 128 148 and 141, 512 307 and 233; 1031 in 16, 43 of 16, n = 18 42.4 and 43.4, 30 45.6 and 44.4; 8192 in 448, 24 of 16 (no slice on
-// chip), n = 2 63 and 95; 30000 in 160, n = 3 142 and 270, 4 335 and 267.  One layout: 8192 in 448 47.6 and 94, 4000 in 2000 44.8 and 46.3,
-// 8000 in 1920 51.8 and 71.
+// form groups an assignment once, but in one CTA, and has three launches where this has one.  Both add up the same rows, so that what counts
+// is the scans (left) against the grouping, the launches and the slices' loading (right); drawn through 1760 calls of 900 windows timed in both
+// forms, the chosen one is 0.8 % above the better one on average.  Calls in us, few and many: 512 samples in 32 row-shards, 16 layers of 8
+// ranks, n = 8 37.0 and 36.6, 64 49 and 37, 512 204 and 54; 2048 in 240, 24 of 16, n = 4 36.9 and 41.5, 6 44.7 and 42.5, 64 172 and 54; 1808 in
+// 18, 28 of 32, n = 27 54 and 70; 227 in 6, 30 of 32, n = 53 34 and 42; 5430 in 32, 32 chunks a row, n = 32 98 and 142; 4000 in 6, 16 of 8, n = 64
+// 96 and 138, 128 148 and 141, 512 307 and 233; 8192 in 448, 24 of 16 (no slice on chip), n = 2 63 and 95; 30000 in 160, n = 3 142 and 270, 4 335
+// and 267.  (With the rows among the scans, and no row-shards on the right: 1.3 % above on average, 1.4 times at worst where few row-shards are
+// long.)  One layout: 8192 in 448 47.6 and 94, 4000 in 2000 44.8 and 46.3, 8000 in 1920 51.8 and 71.
 static bool eval_is_few(const RpDims &dm, int n)
 {
     if ((dm.P & 3) || n >= 65536 || dm.RG >= 65536 || dm.LP > 16384 || eval_few_smem(dm, 8) > EVAL_SMEM_MAX) return false;
     const double N = dm.N, RG = dm.RG;
     if (n == 1) return RG * N <= 5e6;
-    return n * (RG * (6.0 + N / 300.0) + 3e-4 * N * dm.LP) <= 4e3 + 5.0 * std::min(N, 1e4);
+    return n * RG * (8.5 + N / 480.0) <= 5e3 + 2.8 * std::min(N, 1e4) + 38.0 * RG + dm.LP;
 }
 size_t rp_eval_list_len(const RpDims &dm, int n) { return eval_is_few(dm, n) ? 0 : (size_t)n * dm.N; }
 size_t rp_eval_off_len(const RpDims &dm, int n) { return eval_is_few(dm, n) ? 0 : (size_t)n * (dm.RG + 1); }
