@@ -525,7 +525,8 @@ def eval_stage(rp, torch, name, dev, l2_gbs, reps=10):
     gathered = s.pop_size * q_bytes
     hbm_min = s.pop_size * s.n_samples * 4 + q_bytes          # int32 layouts in, demand rows once
     return {"workload": name, "layouts": s.pop_size, "ms": ms, "layouts_per_s": s.pop_size / ms * 1e3,
-            "roofline": {"bound": "l2", "kernel": "k_eval_group, k_eval_sum, k_eval_score", "achieved": gathered / ms / 1e6, "peak": l2_gbs, "unit": "GB/s",
+            "roofline": {"bound": "l2 where the rows stream (k_eval_sum), shared memory where slices of them stay on chip (k_eval_slice)",
+                         "kernel": "k_eval_group, k_eval_slice or k_eval_sum, k_eval_score", "achieved": gathered / ms / 1e6, "peak": l2_gbs, "unit": "GB/s",
                          "frac": gathered / ms / 1e6 / l2_gbs, "peak_source": "read rate of a 32 MiB L2-resident buffer measured in this run (rp_debug_l2_read_rate)",
                          "gathered_bytes_per_launch": gathered, "hbm_bytes_per_launch_min": hbm_min,
                          "hbm_min_gbs": hbm_min / ms / 1e6, "hbm_min_frac": hbm_min / ms / 1e6 / peak}}
