@@ -229,7 +229,7 @@ k_eval_group(const EvalArgs A, bool by_length)
 // rows from shared memory; a team that has finished reads the row of zeros behind the last sample.  Every sample's row crosses
 // L2 once a CTA instead of once a layout; bound by its instructions and by shared memory alike (a quarter warp reads 128 bytes at a
 // time, two rows of 64 bytes collide where both are even or odd): 256 layouts of 2048 samples in 240 row-shards, 24 layers of 16 ranks, 136 us
-// with the streaming sums, 80 with a division and a multiplication per row-shard and sample left in, 67.
+// with the streaming sums, 80 with a division and a multiplication per row-shard and sample left in, 66 (a call 161, and 93 now).
 #define SLICE_THREADS 1024
 #define SLICE_MAX (1 << 12)           // row-shards whose busiest loads are kept between the pieces of a layer
 struct SlicePlan { int tw, w, parts, lps, slices, groups, batch; size_t smem; };
